@@ -231,3 +231,100 @@ def tolerance(case):
     if case["op"] == "hca":
         return {"rel": 1.2e-2, "max": 0.35}
     return {"rel": 2.4e-2 if case["op"] == "combined" else 1.2e-2, "max": 0.8, "differ": 2e-3}
+
+
+def exact(case, seed):
+    """What run() returns for these inputs, in float64 torch; None for token ids, counts and values that a variant leaves out."""
+    s = prepare(case, seed)
+    return _exact_hca(s) if case["op"] == "hca" else _exact_loss(case, s)
+
+
+def _exact_loss(case, s):
+    op, K, N = case["op"], case["K"], case["N"]
+    W = s["W"].double()
+    rows = max(1, min(N, (1 << 27) // W.shape[0]))
+    parts = []
+    for r in range(0, N, rows):
+        parts.append(_exact_rows(op, K, W, s, slice(r, min(N, r + rows))))
+    got = {k: None if parts[0][k] is None else torch.cat([p[k] for p in parts]) for k in parts[0]}
+    keys = {"fwd_bwd_draft": ("loss", "lse_d", "dH_d"), "combined": ("loss_ce", "loss", "topk_idx", "topk_q", "lse_t", "lse_d", "dH_d")}
+    plain = ("loss", "topk_idx", "topk_q", "lse_t", "lse_d", "dH_d")
+    variant = ("loss", "topk_idx", "topk_q", "topk_n", "lse_t", "lse_d", "dH_d")
+    return {k: got[k] for k in keys.get(op, variant if op in VARIANTS else plain)}
+
+
+def _exact_rows(op, K, W, s, rows):
+    out = dict.fromkeys(("loss_ce", "topk_idx", "topk_q", "topk_n", "lse_t"))
+    H_d = s["H_d"][rows].double()
+    z_d = H_d @ W.T
+    lse_d = z_d.logsumexp(1)
+    p = (z_d - lse_d[:, None]).exp()
+    g = s["grad"][rows].double()[:, None] if s["grad"] is not None else 1.0
+    if op == "fwd_bwd_draft":
+        idx, q = s["topk_idx"][rows].long(), s["topk_q"][rows].double()
+        q_all = None
+    else:
+        z_t = s["H_t"][rows].double() @ W.T
+        out["lse_t"] = z_t.logsumexp(1)
+        q_all = (z_t - out["lse_t"][:, None]).exp()
+        q, idx = q_all.topk(K, dim=1)
+        if op == "top_p":
+            q = torch.where(q.cumsum(1) - q > s["p"], 0.0, q)
+        if op == "bidir":
+            # the draft's K most probable tokens that the target's set does not hold, in descending p, then zeros
+            idx_d = p.topk(K, dim=1).indices
+            new = torch.ones_like(p, dtype=torch.bool).scatter_(1, idx, False).gather(1, idx_d)
+            order = (~new).int().argsort(dim=1, stable=True)
+            idx = torch.cat((idx, idx_d.gather(1, order)), 1)
+            q = torch.cat((q, torch.where(new, q_all.gather(1, idx_d), 0.0).gather(1, order)), 1)
+        out["topk_q"] = q
+    if op == "normed":
+        qn = q / q.sum(1, keepdim=True)
+        zk = z_d.gather(1, idx)
+        log_pn = zk.log_softmax(1)
+        dz = torch.zeros_like(p).scatter_(1, idx, g * (log_pn.exp() - qn))
+        return dict(out, loss=-(qn * log_pn).sum(1), lse_d=None, dH_d=dz @ W)
+    log_p = z_d.gather(1, idx) - lse_d[:, None]
+    if op == "combined":
+        out["loss_ce"] = lse_d - (q_all * z_d).sum(1)
+        dz = (1.0 + q.sum(1, keepdim=True)) * p - q_all
+    else:
+        dz = q.sum(1, keepdim=True) * p
+    # (tokens beyond a variant's set carry q = 0)
+    dz.scatter_add_(1, idx, -q)
+    return dict(out, loss=-(q * log_p).sum(1), lse_d=lse_d, dH_d=(g * dz) @ W)
+
+
+def _exact_hca(s):
+    B, T, H, D = s["Q"].shape
+    Hkv, m = s["K_t"].shape[2], min(len(s["K_d"]), T)
+    shape, kv = (B, T, H, D), (B, T, Hkv, D)
+    new = lambda sh: torch.zeros(sh, dtype=torch.float64, device=s["Q"].device)
+    O, lse = new(shape), new((B, H, T))
+    dQ, dK, dV = new(shape), [new(kv) for _ in range(1 + len(s["K_d"]))], [new(kv) for _ in range(1 + len(s["K_d"]))]
+    causal = torch.ones(T, T, dtype=torch.bool, device=O.device).triu_(1)
+    for b in range(B):
+        for h in range(H):
+            n = h // (H // Hkv)
+            leaf = lambda x, i: x[b, :, i].double().requires_grad_(s["bwd"])
+            Q, K, V = leaf(s["Q"], h), [leaf(x, n) for x in (s["K_t"], *s["K_d"])], [leaf(x, n) for x in (s["V_t"], *s["V_d"])]
+            S = Q @ K[0].T
+            for i in range(m):
+                S = S.diagonal_scatter((Q[i:] * K[1 + i][:T - i]).sum(1), -i)
+            S = (S * D ** -0.5).masked_fill(causal, -math.inf)
+            P = S.softmax(1)
+            near = torch.ones_like(causal).triu_(-(m - 1)) if m else torch.zeros_like(causal)
+            o = P.masked_fill(near, 0.0) @ V[0]
+            for i in range(m):
+                o = o + torch.nn.functional.pad(P.diagonal(-i)[:, None] * V[1 + i][:T - i], (0, 0, i, 0))
+            O[b, :, h], lse[b, h] = o.detach(), S.detach().logsumexp(1)
+            if s["bwd"]:
+                grads = torch.autograd.grad(o, [Q, *K, *V], s["dO"][b, :, h].double(), allow_unused=True)
+                dQ[b, :, h] = grads[0]
+                for x, gx in zip(dK + dV, grads[1:]):
+                    if gx is not None:
+                        x[b, :, n] += gx
+    out = {"O": O, "lse": lse}
+    if s["bwd"]:
+        out.update(dQ=dQ, dK_t=dK[0], dV_t=dV[0], dK_d=dK[1:], dV_d=dV[1:])
+    return out
