@@ -46,6 +46,11 @@ struct KernelTimer {
     }
 };
 
+// duration of a pair's step (256 x 256 outputs) over that of two single CTAs (128 x 256 outputs each); measured 0.89-0.92
+constexpr double kPairStepTime = 0.90;
+
+typedef void (*GemmFn)(GemmParams);
+
 // ---- device info ------------------------------------------------------------------------------
 struct DeviceInfo {
     int ok = 0;   // 0 unknown, 1 usable, <0 hass_status
@@ -71,14 +76,17 @@ static int device_info(DeviceInfo* out) {
             di.ok = HASS_ERR_ARCH;
         } else {
             di.sms = sms;
-            cudaError_t e0 = cudaFuncSetAttribute(gemm_kernel<MODE_STATS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-            cudaError_t e1 = cudaFuncSetAttribute(gemm_kernel<MODE_PROBS>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-            cudaError_t e2 = cudaFuncSetAttribute(gemm_kernel<MODE_OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-            cudaError_t e3 = cudaFuncSetAttribute(gemm_kernel<MODE_STATS, TOPK_REG>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-            if (e3 == cudaSuccess) e3 = cudaFuncSetAttribute(gemm_kernel<MODE_STATS, TOPK_NONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+            GemmFn const gemms[] = {gemm_kernel<MODE_STATS, TOPK_REG, 1>,  gemm_kernel<MODE_STATS, TOPK_REG, 2>,
+                                    gemm_kernel<MODE_STATS, TOPK_BUF, 1>,  gemm_kernel<MODE_STATS, TOPK_BUF, 2>,
+                                    gemm_kernel<MODE_STATS, TOPK_NONE, 1>, gemm_kernel<MODE_STATS, TOPK_NONE, 2>,
+                                    gemm_kernel<MODE_PROBS, TOPK_BUF, 1>,  gemm_kernel<MODE_PROBS, TOPK_BUF, 2>,
+                                    gemm_kernel<MODE_OUT, TOPK_BUF, 1>,    gemm_kernel<MODE_OUT, TOPK_BUF, 2>};
+            cudaError_t e3 = cudaSuccess;
+            for (GemmFn f : gemms)
+                if (e3 == cudaSuccess) e3 = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
             cudaError_t e4 = cudaFuncSetAttribute(hca2::hca_attention_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hca2::SMEM_BYTES);
             if (e4 == cudaSuccess) e4 = cudaFuncSetAttribute(hca_bwd::hca_bwd_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hca_bwd::F_SMEM_BYTES);
-            if (e0 != cudaSuccess || e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess || e4 != cudaSuccess) {
+            if (e3 != cudaSuccess || e4 != cudaSuccess) {
                 cudaGetLastError();
                 return HASS_ERR_CUDA;
             }
@@ -102,29 +110,33 @@ static int sm_count_or_default() {
 
 // ---- tile schedule ----------------------------------------------------------------------------
 // Splits RT row tiles into phases (G row tiles x S lanes, G * S <= sms) minimising the summed phase
-// durations ceil(CT / S), by dynamic programming over the number of row tiles already covered.
-static int plan_schedule(int RT, int CT, int sms, Schedule* out) {
-    if (RT < 1 || CT < 1 || sms < 1) return HASS_ERR_INVALID_ARG;
+// durations ceil(CT / S), by dynamic programming over the number of row tiles already covered. pair = 2: the
+// same in units of CTA pairs, each covering two row tiles (an odd RT counts as the next even number).
+// *cost = the summed durations, in column tiles. one_phase: all row tiles side by side (at most sms slots).
+static int plan_schedule(int RT, int CT, int sms, int pair, Schedule* out, int* cost = nullptr, bool one_phase = false) {
+    const int units = (RT + pair - 1) / pair, groups_max = sms / pair;
+    if (RT < 1 || CT < 1 || groups_max < 1) return HASS_ERR_INVALID_ARG;
+    if (one_phase && units > groups_max) return HASS_ERR_UNSUPPORTED;
     const int INF = 1 << 30;
-    std::vector<int> best(RT + 1, INF), nph(RT + 1, INF), choice(RT + 1, 0);
+    std::vector<int> best(units + 1, INF), nph(units + 1, INF), choice(units + 1, 0);
     best[0] = 0;
     nph[0] = 0;
-    for (int n = 1; n <= RT; ++n) {
-        for (int G = 1; G <= n && G <= sms; ++G) {
-            int S = sms / G;
+    for (int n = 1; n <= units; ++n) {
+        for (int G = one_phase ? n : 1; G <= n && G <= groups_max; ++G) {
+            int S = groups_max / G;
             if (S > CT) S = CT;
-            const int cost = best[n - G] + (CT + S - 1) / S;
+            const int c = best[n - G] + (CT + S - 1) / S;
             const int ph = nph[n - G] + 1;
-            if (cost < best[n] || (cost == best[n] && ph < nph[n])) {
-                best[n] = cost;
+            if (c < best[n] || (c == best[n] && ph < nph[n])) {
+                best[n] = c;
                 nph[n] = ph;
                 choice[n] = G;
             }
         }
     }
-    if (nph[RT] > MAX_PHASES) return HASS_ERR_UNSUPPORTED;
+    if (nph[units] > MAX_PHASES) return HASS_ERR_UNSUPPORTED;
     std::vector<int> groups;
-    for (int n = RT; n > 0; n -= choice[n]) groups.push_back(choice[n]);
+    for (int n = units; n > 0; n -= choice[n]) groups.push_back(choice[n]);
     std::memset(out, 0, sizeof(*out));
     int rt = 0, slot = 0, maxc = 0;
     // largest groups first: the widest phases start together
@@ -132,8 +144,8 @@ static int plan_schedule(int RT, int CT, int sms, Schedule* out) {
         for (size_t j = i + 1; j < groups.size(); ++j)
             if (groups[j] > groups[i]) std::swap(groups[i], groups[j]);
     for (size_t i = 0; i < groups.size(); ++i) {
-        const int G = groups[i];
-        int S = sms / G;
+        const int G = groups[i] * pair;
+        int S = groups_max / groups[i];
         if (S > CT) S = CT;
         out->ph[i] = Phase{rt, G, S, slot};
         rt += G;
@@ -143,8 +155,79 @@ static int plan_schedule(int RT, int CT, int sms, Schedule* out) {
     out->n_phases = static_cast<int>(groups.size());
     out->total_slots = slot;
     out->max_ctas = maxc;
+    out->pair = pair;
+    if (cost) *cost = best[units];
     return HASS_OK;
 }
+
+// The schedule that a launch over RT row tiles uses, of at most max_slots slots: the one of least expected time
+// among single CTAs and pairs, in as many phases as it takes or in one.
+static int plan_launch(int RT, int CT, int sms, int max_slots, Schedule* out) {
+    int rc = HASS_ERR_WORKSPACE;
+    double best = 0.;
+    for (int i = 0; i < 4; ++i) {
+        const int pair = i & 1 ? 2 : 1;
+        if (pair == 2 && (RT < 2 || sms < 2)) continue;
+        Schedule s;
+        int steps = 0;
+        const int r = plan_schedule(RT, CT, sms, pair, &s, &steps, i >= 2);
+        if (i == 0 && r != HASS_OK) return r;
+        const double time = steps * (pair == 2 ? kPairStepTime : 1.);
+        if (r == HASS_OK && s.total_slots <= max_slots && (rc != HASS_OK || time < best)) {
+            *out = s;
+            best = time;
+            rc = HASS_OK;
+        }
+    }
+    return rc;
+}
+
+// ---- division of the output tiles of MODE_OUT -----------------------------------------------------
+constexpr int kPartTilesMax = 296;      // partial tiles of one CTA each, at most (38.8 MB): two rounds of the grid
+
+// Over `rows` rows, CT column tiles and a contraction of `kb` blocks, with room for part_bytes of partial tiles. Expected
+// times in steps of one k block (about 0.5 us): cutting the rest of the last round costs a kernel of its own (14 steps),
+// the partial tiles' way to memory and back (4 TB/s) and one fill and drain of the pipeline (6 steps) per piece.
+// Measured (second GEMM alone): 61 rows x 4096 x 32000 179 -> 56 us (16 tiles in 16 x 8 pieces on 128 of the SMs), 517
+// rows x 4096 x 128256 822 -> 657 us, the 28-row-tile chunk of 8192 rows 4 rounds of 74 pairs -> 3 and a cut rest.
+static OutPlan plan_out(int rows, int CT, int kb, int sms, size_t part_bytes) {
+    const int RT = (rows + BM - 1) / BM;
+    const int part_rows = RT == 1 ? rows : BM;      // rows kept of a partial tile
+    const size_t tile_bytes = static_cast<size_t>(part_rows) * BN * 4;
+    OutPlan best = {};
+    double best_cost = 0.;
+    for (int pair = 1; pair <= 2; ++pair) {
+        if (pair == 2 && (RT < 2 || sms < 2)) break;
+        const int units = (RT + pair - 1) / pair, groups = sms / pair;
+        const long long tiles = static_cast<long long>(units) * CT;
+        const int rest = static_cast<int>(tiles % groups);
+        const int whole = static_cast<int>(tiles - rest);
+        const double step = pair == 2 ? kPairStepTime : 1.;
+        for (int cuts = 1; cuts == 1 || (rest > 0 && cuts <= kb / 4 && static_cast<long long>(rest) * cuts * pair <= kPartTilesMax &&
+                                         static_cast<size_t>(rest) * cuts * pair * tile_bytes <= part_bytes); ++cuts) {
+            double cost = step * (whole / groups) * (kb + 6.);
+            if (rest > 0) {
+                const int rounds = (rest * cuts + groups - 1) / groups;
+                cost += step * rounds * ((kb + cuts - 1) / cuts + 6.);
+                if (cuts > 1) cost += 14. + 2. * rest * cuts * pair * tile_bytes / 2e6;
+            }
+            if (best.groups == 0 || cost < best_cost) {
+                best_cost = cost;
+                best.pair = pair;
+                best.part_rows = part_rows;
+                best.row_units = units;
+                best.whole = cuts == 1 ? static_cast<int>(tiles) : whole;
+                best.rest = cuts == 1 ? 0 : rest;
+                best.cuts = cuts;
+                best.groups = static_cast<int>(tiles < groups && cuts == 1 ? tiles
+                                               : whole == 0 && static_cast<long long>(rest) * cuts < groups ? rest * cuts
+                                                                                                            : groups);
+            }
+        }
+    }
+    return best;
+}
+static size_t part_bytes_of(const OutPlan& o) { return o.rest ? static_cast<size_t>(o.rest) * o.cuts * o.pair * o.part_rows * BN * 4 : 0; }
 
 // ---- TMA descriptors --------------------------------------------------------------------------
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -206,30 +289,38 @@ struct Layout {
     int pref_chunk_tiles;
     int slot_cap;
     size_t total_pref;
+    size_t part_bytes;               // partial tiles of the second GEMM, behind the scratch; without them it is not cut
 };
 
 static int ceil_div(long long a, long long b) { return static_cast<int>((a + b - 1) / b); }
 
+// Row tiles per chunk when at most `most` fit: all RT, or an even number of them (pairs of CTAs work on two).
+static int even_chunk(int most, int RT) {
+    if (most >= RT) return RT;
+    return most > 1 ? most & ~1 : most;
+}
+
 // The forward schedule covers 2 * RT row tiles (target then draft).
-static int make_layout(long long N, long long d, long long V, int K, int sms, Layout* L, Schedule* fwd_sched) {
+static int make_layout(long long N, long long d, long long V, int K, int sms, Layout* L) {
     const int RT = ceil_div(N, BM), CT = ceil_div(V, BN);
     Schedule s;
-    int rc = plan_schedule(2 * RT, CT, sms, &s);
+    int rc = plan_schedule(2 * RT, CT, sms, 1, &s);
     if (rc != HASS_OK) return rc;
-    if (fwd_sched) *fwd_sched = s;
-    int pref = sms / 4;
+    int pref = even_chunk(sms / 4, RT);
     if (pref < 1) pref = 1;
-    if (pref > RT) pref = RT;
-    // partial-statistics slots: enough for the whole-batch forward and for the per-chunk forward
-    // sweeps of the fused path (target + draft tiles, or draft tiles only, of a full or last chunk)
+    // partial-statistics slots: enough for the whole-batch forward and for sweeps over chunks of about sms / 4 row tiles
+    // (target + draft tiles, or one of them, of a full or last chunk); plan_launch keeps to them
     int slot_cap = s.total_slots;
     {
-        const int rem = RT % pref;
-        const int cands[5] = {RT, 2 * pref, pref, 2 * rem, rem};
+        int most = sms / 4;
+        if (most < 1) most = 1;
+        if (most > RT) most = RT;
+        const int rem = RT % most;
+        const int cands[5] = {RT, 2 * most, most, 2 * rem, rem};
         for (int i = 0; i < 5; ++i) {
             if (cands[i] < 1) continue;
             Schedule t;
-            rc = plan_schedule(cands[i], CT, sms, &t);
+            rc = plan_schedule(cands[i], CT, sms, 1, &t);
             if (rc != HASS_OK) return rc;
             if (t.total_slots > slot_cap) slot_cap = t.total_slots;
         }
@@ -270,7 +361,17 @@ static int make_layout(long long N, long long d, long long V, int K, int sms, La
     L->p_pitch = static_cast<long long>(CT) * BN;
     L->scratch_row_tile_bytes = static_cast<size_t>(BM) * L->p_pitch * 2;
     L->pref_chunk_tiles = pref;
-    L->total_pref = off + L->scratch_row_tile_bytes * pref;
+    L->total_pref = align256(off + L->scratch_row_tile_bytes * pref);
+    L->part_bytes = 0;
+    // less than a row tile of scratch, so that a workspace's size still tells how many row tiles fit
+    const long long all = N < static_cast<long long>(pref) * BM ? N : static_cast<long long>(pref) * BM;
+    const long long chunks[2] = {all, N % (static_cast<long long>(pref) * BM)};
+    for (long long rows : chunks) {
+        if (rows < 1) continue;
+        const size_t need = part_bytes_of(plan_out(static_cast<int>(rows), ceil_div(d, BN), ceil_div(V, BK), sms,
+                                                   L->scratch_row_tile_bytes - 256));
+        if (need > L->part_bytes) L->part_bytes = need;
+    }
     return HASS_OK;
 }
 
@@ -301,12 +402,73 @@ static void log_schedule(const char* what, const Schedule& s) {
 template <int MODE>
 static int launch_gemm(const GemmParams& p, cudaStream_t st, int kind = -1) {
     KernelTimer timer(p.only_if_range ? KIND_CONDITIONAL : (kind >= 0 ? kind : MODE), st);
+    const bool pair = p.sched.pair == 2;
+    GemmFn fn;
     if (MODE == MODE_STATS && p.topk_row_tiles == 0 && p.cap_z != nullptr)
-        gemm_kernel<MODE_STATS, TOPK_NONE><<<p.sched.max_ctas, NUM_THREADS, SMEM_BYTES, st>>>(p);
+        fn = pair ? gemm_kernel<MODE_STATS, TOPK_NONE, 2> : gemm_kernel<MODE_STATS, TOPK_NONE, 1>;
     else if (MODE == MODE_STATS && p.K <= K_REG)
-        gemm_kernel<MODE_STATS, TOPK_REG><<<p.sched.max_ctas, NUM_THREADS, SMEM_BYTES, st>>>(p);
+        fn = pair ? gemm_kernel<MODE_STATS, TOPK_REG, 2> : gemm_kernel<MODE_STATS, TOPK_REG, 1>;
     else
-        gemm_kernel<MODE><<<p.sched.max_ctas, NUM_THREADS, SMEM_BYTES, st>>>(p);
+        fn = pair ? gemm_kernel<MODE, TOPK_BUF, 2> : gemm_kernel<MODE, TOPK_BUF, 1>;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(p.sched.max_ctas);
+    cfg.blockDim = dim3(NUM_THREADS);
+    cfg.dynamicSmemBytes = SMEM_BYTES;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    if (pair) {
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 2;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+    }
+    if (cudaLaunchKernelEx(&cfg, fn, p) != cudaSuccess) {
+        cudaGetLastError();
+        return HASS_ERR_CUDA;
+    }
+    g_launches.fetch_add(1);
+    return cudaGetLastError() == cudaSuccess ? HASS_OK : HASS_ERR_CUDA;
+}
+
+// Partial tiles' room of a call: behind the scratch of its row chunks, where the caller says, or (routes without an
+// Omega_hat term of their own) in the fp32 rows kept for that term, whichever is larger.
+struct PartRoom {
+    float* at = nullptr;
+    size_t bytes = 0;
+};
+static PartRoom part_room(uint8_t* ws, size_t workspace_bytes, const Layout& L, int chunk_tiles, const PartRoom* given,
+                          bool sparse_free) {
+    PartRoom r;
+    if (given) r = *given;
+    const size_t off = align256(L.fixed_end + L.scratch_row_tile_bytes * chunk_tiles);
+    if (!given && workspace_bytes > off) {
+        r.at = reinterpret_cast<float*>(ws + off);
+        r.bytes = workspace_bytes - off;
+    }
+    if (sparse_free && L.scratch - L.sparse > r.bytes) {
+        r.at = reinterpret_cast<float*>(ws + L.sparse);
+        r.bytes = L.scratch - L.sparse;
+    }
+    return r;
+}
+
+// The second GEMM (MODE_OUT) over p.row_tiles row tiles: plan, tiles, and the sum of the partial tiles.
+static int launch_out(GemmParams& p, const PartRoom& room, int sms, cudaStream_t st) {
+    const long long left = p.rows_valid - p.row_global_offset;
+    const int rows = static_cast<int>(left < static_cast<long long>(p.row_tiles) * BM ? left : p.row_tiles * BM);
+    p.plan = plan_out(rows, p.col_tiles, p.k_blocks, sms, room.bytes);
+    p.part = room.at;
+    p.sched.pair = p.plan.pair;
+    p.sched.max_ctas = p.plan.groups * p.plan.pair;
+    if (kLog)
+        std::fprintf(stderr, "[hass] out: pair %d, grid %d, %d whole tiles, %d rest tiles x %d cuts\n", p.plan.pair, p.sched.max_ctas,
+                     p.plan.whole, p.plan.rest, p.plan.cuts);
+    const int rc = launch_gemm<MODE_OUT>(p, st);
+    if (rc != HASS_OK || p.plan.rest == 0) return rc;
+    KernelTimer timer(p.only_if_range ? KIND_CONDITIONAL : KIND_OUT, st);
+    out_reduce_kernel<<<p.plan.rest * p.plan.pair * (BM * BN / 4 / 256), 256, 0, st>>>(p);
     g_launches.fetch_add(1);
     return cudaGetLastError() == cudaSuccess ? HASS_OK : HASS_ERR_CUDA;
 }
@@ -331,8 +493,7 @@ static int forward_impl(bool with_target, const void* H_t, const void* H_d, cons
     if (rc != HASS_OK) return rc;
 
     Layout L;
-    Schedule full;
-    rc = make_layout(N, d, V, K, di.sms, &L, &full);
+    rc = make_layout(N, d, V, K, di.sms, &L);
     if (rc != HASS_OK) return rc;
     if (workspace_bytes < L.fwd_end) return HASS_ERR_WORKSPACE;
     const int RT = ceil_div(N, BM), CT = ceil_div(V, BN);
@@ -345,22 +506,21 @@ static int forward_impl(bool with_target, const void* H_t, const void* H_d, cons
 
     GemmParams p;
     std::memset(&p, 0, sizeof(p));
+    p.row_tiles = with_target ? 2 * RT : RT;
+    rc = plan_launch(p.row_tiles, CT, di.sms, L.slot_cap, &p.sched);
+    if (rc != HASS_OK) return rc;
     if (with_target) {
-        p.sched = full;
         p.row_tiles0 = RT;
         p.topk_row_tiles = RT;
         rc = make_tmap(&p.tmA0, H_t, N, d, d, BK, BM);
         if (rc == HASS_OK) rc = make_tmap(&p.tmA1, H_d, N, d, d, BK, BM);
     } else {
-        rc = plan_schedule(RT, CT, di.sms, &p.sched);   // never needs more slots than the full schedule
-        if (rc != HASS_OK) return rc;
-        if (p.sched.total_slots > L.slot_cap) return HASS_ERR_WORKSPACE;
         p.row_tiles0 = RT;
         p.topk_row_tiles = 0;
         rc = make_tmap(&p.tmA0, H_d, N, d, d, BK, BM);
         if (rc == HASS_OK) rc = make_tmap(&p.tmA1, H_d, N, d, d, BK, BM);
     }
-    if (rc == HASS_OK) rc = make_tmap(&p.tmB, W, V, d, d, BK, BN);
+    if (rc == HASS_OK) rc = make_tmap(&p.tmB, W, V, d, d, BK, BN / p.sched.pair);
     if (rc != HASS_OK) return rc;
     log_schedule(with_target ? "fwd stats" : "fwd stats (draft)", p.sched);
     p.spill_begin = INT_MAX;
@@ -424,7 +584,7 @@ static int forward_impl(bool with_target, const void* H_t, const void* H_d, cons
 static int backward_impl(const void* H_d, const void* W, long long N, long long d, long long V, int K,
                          const int* topk_idx, const float* topk_q, const float* lse_d, const float* grad_loss,
                          void* dH_d, int dH_dtype, void* workspace, size_t workspace_bytes, cudaStream_t st,
-                         bool clear_status, const unsigned int* only_if_range = nullptr) {
+                         bool clear_status, const unsigned int* only_if_range = nullptr, const PartRoom* room = nullptr) {
     int rc = check_sizes(N, d, V, K);
     if (rc != HASS_OK) return rc;
     if (!H_d || !W || !topk_idx || !topk_q || !lse_d || !dH_d) return HASS_ERR_INVALID_ARG;
@@ -438,14 +598,15 @@ static int backward_impl(const void* H_d, const void* W, long long N, long long 
     if (rc != HASS_OK) return rc;
 
     Layout L;
-    rc = make_layout(N, d, V, K, di.sms, &L, nullptr);
+    rc = make_layout(N, d, V, K, di.sms, &L);
     if (rc != HASS_OK) return rc;
     if (workspace_bytes < L.fixed_end + L.scratch_row_tile_bytes) return HASS_ERR_WORKSPACE;
     const int RT = ceil_div(N, BM), CT = ceil_div(V, BN), DT = ceil_div(d, BN);
     long long fit = static_cast<long long>((workspace_bytes - L.fixed_end) / L.scratch_row_tile_bytes);
     int chunk_tiles = L.pref_chunk_tiles;
-    if (fit < chunk_tiles) chunk_tiles = static_cast<int>(fit);
+    if (fit < chunk_tiles) chunk_tiles = even_chunk(static_cast<int>(fit), RT);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
+    const PartRoom part = part_room(ws, workspace_bytes, L, chunk_tiles, room, true);
     int* sidx = reinterpret_cast<int*>(ws + L.sidx);
     float* sgq = reinterpret_cast<float*>(ws + L.sgq);
     float* coef = reinterpret_cast<float*>(ws + L.coef);
@@ -464,9 +625,8 @@ static int backward_impl(const void* H_d, const void* W, long long N, long long 
     g_launches.fetch_add(1);
     if (cudaGetLastError() != cudaSuccess) return HASS_ERR_CUDA;
 
-    CUtensorMap tmHd, tmWk, tmWn, tmP;
+    CUtensorMap tmHd, tmWn, tmP;
     rc = make_tmap(&tmHd, H_d, N, d, d, BK, BM);
-    if (rc == HASS_OK) rc = make_tmap(&tmWk, W, V, d, d, BK, BN);      // B of z_d = H_d W^T: K-major
     if (rc == HASS_OK) rc = make_tmap(&tmWn, W, V, d, d, 64, BK);      // B of dH_d = dz_d W: MN-major boxes
     if (rc == HASS_OK) rc = make_tmap(&tmP, P, static_cast<long long>(chunk_tiles) * BM, V, L.p_pitch, BK, BM);
     if (rc != HASS_OK) return rc;
@@ -476,12 +636,14 @@ static int backward_impl(const void* H_d, const void* W, long long N, long long 
         // (1) dz_d tiles of this chunk of rows -> scratch
         GemmParams p;
         std::memset(&p, 0, sizeof(p));
-        rc = plan_schedule(tiles, CT, di.sms, &p.sched);
+        rc = plan_launch(tiles, CT, di.sms, L.slot_cap, &p.sched);
         if (rc != HASS_OK) return rc;
         log_schedule("bwd dz_d", p.sched);
         p.tmA0 = tmHd;
         p.tmA1 = tmHd;
-        p.tmB = tmWk;
+        rc = make_tmap(&p.tmB, W, V, d, d, BK, BN / p.sched.pair);      // B of z = H W^T: K-major
+        if (rc != HASS_OK) return rc;
+        p.row_tiles = tiles;
         p.row_tiles0 = tiles;
         p.a_row_offset = t0 * BM;
         p.row_global_offset = t0 * BM;
@@ -503,12 +665,10 @@ static int backward_impl(const void* H_d, const void* W, long long N, long long 
         // (2) dH_d rows of this chunk = dz_d chunk x W
         GemmParams o;
         std::memset(&o, 0, sizeof(o));
-        rc = plan_schedule(tiles, DT, di.sms, &o.sched);
-        if (rc != HASS_OK) return rc;
-        log_schedule("bwd dH_d", o.sched);
         o.tmA0 = tmP;
         o.tmA1 = tmP;
         o.tmB = tmWn;
+        o.row_tiles = tiles;
         o.row_tiles0 = tiles;
         o.a_row_offset = 0;
         o.row_global_offset = t0 * BM;
@@ -523,7 +683,7 @@ static int backward_impl(const void* H_d, const void* W, long long N, long long 
         o.out_pitch = d;
         o.status = p.status;
         o.only_if_range = only_if_range;
-        rc = launch_gemm<MODE_OUT>(o, st);
+        rc = launch_out(o, part, di.sms, st);
         if (rc != HASS_OK) return rc;
     }
     return HASS_OK;
@@ -549,7 +709,7 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
                       long long V, int K, const float* grad_loss, const int* idx_in, const float* q_in, float* loss,
                       int* idx_out, float* q_out, float* lse_t, float* lse_d, void* dH_d, int dH_dtype,
                       void* workspace, size_t workspace_bytes, cudaStream_t st, const Combined* cmb = nullptr,
-                      int* topk_n = nullptr, bool bidir = false) {
+                      int* topk_n = nullptr, bool bidir = false, const PartRoom* room = nullptr) {
     int rc = check_sizes(N, d, V, K);
     if (rc != HASS_OK) return rc;
     if (!H_d || !W || !loss || !lse_d || !dH_d || !aligned16(H_d) || !aligned16(W) || !aligned16(dH_d))
@@ -565,14 +725,15 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
     rc = get_encode();
     if (rc != HASS_OK) return rc;
     Layout L;
-    rc = make_layout(N, d, V, K, di.sms, &L, nullptr);
+    rc = make_layout(N, d, V, K, di.sms, &L);
     if (rc != HASS_OK) return rc;
     if (workspace_bytes < L.fixed_end + L.scratch_row_tile_bytes) return HASS_ERR_WORKSPACE;
     const int RT = ceil_div(N, BM), CT = ceil_div(V, BN), DT = ceil_div(d, BN);
     long long fit = static_cast<long long>((workspace_bytes - L.fixed_end) / L.scratch_row_tile_bytes);
     int chunk_tiles = L.pref_chunk_tiles;
-    if (fit < chunk_tiles) chunk_tiles = static_cast<int>(fit);
+    if (fit < chunk_tiles) chunk_tiles = even_chunk(static_cast<int>(fit), RT);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
+    const PartRoom part = part_room(ws, workspace_bytes, L, chunk_tiles, room, false);
     float* gq = bidir ? nullptr : reinterpret_cast<float*>(ws + L.sgq);    // [N, K]: too small for the 2K-token union
     float* coef = reinterpret_cast<float*>(ws + L.coef);
     float* sparse = reinterpret_cast<float*>(ws + L.sparse);
@@ -582,10 +743,9 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
         cudaGetLastError();
         return HASS_ERR_CUDA;
     }
-    CUtensorMap tmHt, tmHd, tmWk, tmWn, tmP;
+    CUtensorMap tmHt, tmHd, tmWn, tmP;
     rc = make_tmap(&tmHd, H_d, N, d, d, BK, BM);
     if (rc == HASS_OK) rc = with_target ? make_tmap(&tmHt, H_t, N, d, d, BK, BM) : make_tmap(&tmHt, H_d, N, d, d, BK, BM);
-    if (rc == HASS_OK) rc = make_tmap(&tmWk, W, V, d, d, BK, BN);
     if (rc == HASS_OK) rc = make_tmap(&tmWn, W, V, d, d, 64, BK);
     if (rc == HASS_OK) rc = make_tmap(&tmP, P, static_cast<long long>(chunk_tiles) * BM, V, L.p_pitch, BK, BM);
     CUtensorMap tmPt;
@@ -610,13 +770,14 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
         // (1) logits sweep with statistics, candidates and spill
         GemmParams p;
         std::memset(&p, 0, sizeof(p));
-        rc = plan_schedule(with_target ? 2 * tiles : tiles, CT, di.sms, &p.sched);
+        rc = plan_launch(with_target ? 2 * tiles : tiles, CT, di.sms, L.slot_cap, &p.sched);
         if (rc != HASS_OK) return rc;
-        if (p.sched.total_slots > L.slot_cap) return HASS_ERR_WORKSPACE;
         log_schedule("fused stats", p.sched);
         p.tmA0 = tmHt;
         p.tmA1 = tmHd;
-        p.tmB = tmWk;
+        rc = make_tmap(&p.tmB, W, V, d, d, BK, BN / p.sched.pair);      // B of z = H W^T: K-major
+        if (rc != HASS_OK) return rc;
+        p.row_tiles = with_target ? 2 * tiles : tiles;
         p.row_tiles0 = tiles;
         p.topk_row_tiles = with_target ? (bidir ? 2 * tiles : tiles) : 0;
         p.spill_begin = with_target ? tiles : 0;
@@ -691,15 +852,13 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
         // (3) dH_d rows of the chunk
         GemmParams o;
         std::memset(&o, 0, sizeof(o));
-        rc = plan_schedule(tiles, DT, di.sms, &o.sched);
-        if (rc != HASS_OK) return rc;
-        log_schedule("fused dH_d", o.sched);
         if (cmb) {
             // (2b) q W of the chunk's rows from the target spill, then the cross-entropy and its gradient term
             GemmParams t = o;
             t.tmA0 = tmPt;
             t.tmA1 = tmPt;
             t.tmB = tmWn;
+            t.row_tiles = tiles;
             t.row_tiles0 = tiles;
             t.spill_begin = INT_MAX;
             t.row_global_offset = 0;
@@ -715,7 +874,7 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
             t.out_pitch = d;
             t.status = status;
             t.only_if_range = gate;
-            rc = launch_gemm<MODE_OUT>(t, st);
+            rc = launch_out(t, part, di.sms, st);
             if (rc != HASS_OK) return rc;
             {
                 KernelTimer timer(retry ? KIND_CONDITIONAL : KIND_FINALIZE, st);
@@ -729,6 +888,7 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
         o.tmA0 = tmP;
         o.tmA1 = tmP;
         o.tmB = tmWn;
+        o.row_tiles = tiles;
         o.row_tiles0 = tiles;
         o.spill_begin = INT_MAX;
         o.a_row_offset = 0;
@@ -746,7 +906,7 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
         o.out_pitch = d;
         o.status = status;
         o.only_if_range = gate;
-        rc = launch_gemm<MODE_OUT>(o, st);
+        rc = launch_out(o, part, di.sms, st);
         if (rc != HASS_OK) return rc;
     }
     return HASS_OK;
@@ -791,7 +951,7 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
                        long long V, int K, const float* grad_loss, const int* idx_in, const float* q_in, float* loss,
                        int* idx_out, float* q_out, float* lse_t, float* lse_d, void* dH_d, int dH_dtype,
                        void* workspace, size_t workspace_bytes, cudaStream_t st, float top_p = 0.f,
-                       int* topk_n = nullptr, ChunkPipe* pipe = nullptr) {
+                       int* topk_n = nullptr, ChunkPipe* pipe = nullptr, const PartRoom* room = nullptr) {
     int rc = check_sizes(N, d, V, K);
     if (rc != HASS_OK) return rc;
     if (!H_d || !W || !loss || !lse_d || !dH_d || !aligned16(H_d) || !aligned16(W) || !aligned16(dH_d))
@@ -806,14 +966,15 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
     rc = get_encode();
     if (rc != HASS_OK) return rc;
     Layout L;
-    rc = make_layout(N, d, V, K, di.sms, &L, nullptr);
+    rc = make_layout(N, d, V, K, di.sms, &L);
     if (rc != HASS_OK) return rc;
     if (workspace_bytes < L.fixed_end + L.scratch_row_tile_bytes) return HASS_ERR_WORKSPACE;
     const int RT = ceil_div(N, BM), CT = ceil_div(V, BN), DT = ceil_div(d, BN);
     long long fit = static_cast<long long>((workspace_bytes - L.fixed_end) / L.scratch_row_tile_bytes);
     int chunk_tiles = L.pref_chunk_tiles;
-    if (fit < chunk_tiles) chunk_tiles = static_cast<int>(fit);
+    if (fit < chunk_tiles) chunk_tiles = even_chunk(static_cast<int>(fit), RT);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
+    const PartRoom part = part_room(ws, workspace_bytes, L, chunk_tiles, room, true);
     int* sidx = reinterpret_cast<int*>(ws + L.sidx);
     float* sq = reinterpret_cast<float*>(ws + L.sgq);
     float* coef = reinterpret_cast<float*>(ws + L.coef);
@@ -824,10 +985,9 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
         cudaGetLastError();
         return HASS_ERR_CUDA;
     }
-    CUtensorMap tmHt, tmHd, tmWk, tmWn, tmP;
+    CUtensorMap tmHt, tmHd, tmWn, tmP;
     rc = make_tmap(&tmHd, H_d, N, d, d, BK, BM);
     if (rc == HASS_OK) rc = with_target ? make_tmap(&tmHt, H_t, N, d, d, BK, BM) : make_tmap(&tmHt, H_d, N, d, d, BK, BM);
-    if (rc == HASS_OK) rc = make_tmap(&tmWk, W, V, d, d, BK, BN);
     if (rc == HASS_OK) rc = make_tmap(&tmWn, W, V, d, d, 64, BK);
     if (rc == HASS_OK) rc = make_tmap(&tmP, P, static_cast<long long>(chunk_tiles) * BM, V, L.p_pitch, BK, BM);
     // the same buffer as the draft sweep's TMA stores see it: boxes of 64 columns x 32 rows, every column up to the pitch
@@ -843,11 +1003,12 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
         // both sweeps cover `tiles` row tiles and share one schedule
         GemmParams p;
         std::memset(&p, 0, sizeof(p));
-        rc = plan_schedule(tiles, CT, di.sms, &p.sched);
+        rc = plan_launch(tiles, CT, di.sms, L.slot_cap, &p.sched);
         if (rc != HASS_OK) return rc;
-        if (p.sched.total_slots > L.slot_cap) return HASS_ERR_WORKSPACE;
         log_schedule("fused sweep (target / draft)", p.sched);
-        p.tmB = tmWk;
+        rc = make_tmap(&p.tmB, W, V, d, d, BK, BN / p.sched.pair);      // B of z = H W^T: K-major
+        if (rc != HASS_OK) return rc;
+        p.row_tiles = tiles;
         p.row_tiles0 = tiles;
         p.a_row_offset = t0 * BM;
         p.row_global_offset = t0 * BM;
@@ -970,12 +1131,10 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
         // (5) dH_d rows of the chunk = row scale x (patched spill x W)
         GemmParams o;
         std::memset(&o, 0, sizeof(o));
-        rc = plan_schedule(tiles, DT, di.sms, &o.sched);
-        if (rc != HASS_OK) return rc;
-        log_schedule("fused dH_d", o.sched);
         o.tmA0 = tmP;
         o.tmA1 = tmP;
         o.tmB = tmWn;
+        o.row_tiles = tiles;
         o.row_tiles0 = tiles;
         o.spill_begin = INT_MAX;
         o.a_row_offset = 0;
@@ -991,7 +1150,7 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
         o.out_align32 = ((reinterpret_cast<uintptr_t>(dH_d) | static_cast<uintptr_t>(d * (dH_dtype == HASS_FP32 ? 4 : 2))) & 31u) == 0 ? 1 : 0;
         o.out_pitch = d;
         o.status = status;
-        rc = launch_gemm<MODE_OUT>(o, st);
+        rc = launch_out(o, part, di.sms, st);
         if (rc != HASS_OK) return rc;
         if (pipe) {
             // the chunk's dH_d rows on the outbound copy stream
@@ -1016,7 +1175,7 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
                           workspace, workspace_bytes, st, status, top_p, topk_n);
         if (rc != HASS_OK) return rc;
         rc = backward_impl(H_d, W, N, d, V, K, with_target ? idx_out : idx_in, with_target ? q_out : q_in, lse_d,
-                           grad_loss, dH_d, dH_dtype, workspace, workspace_bytes, st, false, status);
+                           grad_loss, dH_d, dH_dtype, workspace, workspace_bytes, st, false, status, room);
         if (rc != HASS_OK) return rc;
         {
             KernelTimer timer(KIND_CONDITIONAL, st);
@@ -1050,7 +1209,7 @@ static int forward2_impl(bool with_target, const void* H_t, const void* H_d, con
     rc = get_encode();
     if (rc != HASS_OK) return rc;
     Layout L;
-    rc = make_layout(N, d, V, K, di.sms, &L, nullptr);
+    rc = make_layout(N, d, V, K, di.sms, &L);
     if (rc != HASS_OK) return rc;
     if (workspace_bytes < L.sparse)
         return forward_impl(with_target, H_t, H_d, W, N, d, V, K, idx_in, q_in, loss, idx_out, q_out, lse_t, lse_d,
@@ -1063,12 +1222,12 @@ static int forward2_impl(bool with_target, const void* H_t, const void* H_d, con
     }
     GemmParams p;
     std::memset(&p, 0, sizeof(p));
-    rc = plan_schedule(RT, CT, di.sms, &p.sched);
+    rc = plan_launch(RT, CT, di.sms, L.slot_cap, &p.sched);
     if (rc != HASS_OK) return rc;
-    if (p.sched.total_slots > L.slot_cap) return HASS_ERR_WORKSPACE;
     log_schedule("fwd sweep (target / draft)", p.sched);
-    rc = make_tmap(&p.tmB, W, V, d, d, BK, BN);
+    rc = make_tmap(&p.tmB, W, V, d, d, BK, BN / p.sched.pair);
     if (rc != HASS_OK) return rc;
+    p.row_tiles = RT;
     p.row_tiles0 = RT;
     p.spill_begin = INT_MAX;
     p.rows_valid = static_cast<int>(N);
@@ -1175,7 +1334,7 @@ static int normed_impl(const void* H_t, const void* H_d, const void* W, long lon
     rc = get_encode();
     if (rc != HASS_OK) return rc;
     Layout L;
-    rc = make_layout(N, d, V, K, di.sms, &L, nullptr);
+    rc = make_layout(N, d, V, K, di.sms, &L);
     if (rc != HASS_OK) return rc;
     if (workspace_bytes < L.fwd_end) return HASS_ERR_WORKSPACE;
     const int RT = ceil_div(N, BM), CT = ceil_div(V, BN);
@@ -1186,14 +1345,14 @@ static int normed_impl(const void* H_t, const void* H_d, const void* W, long lon
     }
     GemmParams p;
     std::memset(&p, 0, sizeof(p));
-    rc = plan_schedule(RT, CT, di.sms, &p.sched);
+    rc = plan_launch(RT, CT, di.sms, L.slot_cap, &p.sched);
     if (rc != HASS_OK) return rc;
-    if (p.sched.total_slots > L.slot_cap) return HASS_ERR_WORKSPACE;
     log_schedule("normed stats (target)", p.sched);
     rc = make_tmap(&p.tmA0, H_t, N, d, d, BK, BM);
     if (rc == HASS_OK) rc = make_tmap(&p.tmA1, H_t, N, d, d, BK, BM);
-    if (rc == HASS_OK) rc = make_tmap(&p.tmB, W, V, d, d, BK, BN);
+    if (rc == HASS_OK) rc = make_tmap(&p.tmB, W, V, d, d, BK, BN / p.sched.pair);
     if (rc != HASS_OK) return rc;
+    p.row_tiles = RT;
     p.row_tiles0 = RT;
     p.topk_row_tiles = RT;
     p.spill_begin = INT_MAX;
@@ -1315,9 +1474,9 @@ int hass_topk_distill_workspace_bytes(int64_t N, int64_t d, int64_t V, int32_t K
     int rc = check_sizes(N, d, V, K);
     if (rc != HASS_OK) return rc;
     Layout L;
-    rc = make_layout(N, d, V, K, sm_count_or_default(), &L, nullptr);
+    rc = make_layout(N, d, V, K, sm_count_or_default(), &L);
     if (rc != HASS_OK) return rc;
-    *bytes = L.total_pref;
+    *bytes = L.total_pref + L.part_bytes;
     return HASS_OK;
 }
 
@@ -1385,13 +1544,15 @@ int hass_variant_distill_fwd_bwd(const void* H_t, const void* H_d, const void* W
 
 // Buffers appended to the normal workspace by the combined-objective entry.
 struct CombinedStage {
-    size_t coef_t, T, Pt, total;
+    size_t base, coef_t, T, Pt, total, part_bytes;      // base: the normal workspace without the partial tiles, which follow `total`
 };
-static int combined_stage(int64_t N, int64_t d, int64_t V, int32_t K, size_t base, CombinedStage* c) {
+static int combined_stage(int64_t N, int64_t d, int64_t V, int32_t K, CombinedStage* c) {
     Layout L;
-    int rc = make_layout(N, d, V, K, sm_count_or_default(), &L, nullptr);
+    int rc = make_layout(N, d, V, K, sm_count_or_default(), &L);
     if (rc != HASS_OK) return rc;
-    size_t off = align256(base);
+    c->base = L.total_pref;
+    c->part_bytes = L.part_bytes;
+    size_t off = align256(c->base);
     c->coef_t = off;
     off = align256(off + static_cast<size_t>(N) * 4);
     c->T = off;
@@ -1404,13 +1565,12 @@ static int combined_stage(int64_t N, int64_t d, int64_t V, int32_t K, size_t bas
 
 int hass_combined_distill_workspace_bytes(int64_t N, int64_t d, int64_t V, int32_t K, size_t* bytes) {
     if (!bytes) return HASS_ERR_INVALID_ARG;
-    size_t base = 0;
-    int rc = hass_topk_distill_workspace_bytes(N, d, V, K, &base);
+    int rc = check_sizes(N, d, V, K);
     if (rc != HASS_OK) return rc;
     CombinedStage c;
-    rc = combined_stage(N, d, V, K, base, &c);
+    rc = combined_stage(N, d, V, K, &c);
     if (rc != HASS_OK) return rc;
-    *bytes = c.total;
+    *bytes = c.total + c.part_bytes;
     return HASS_OK;
 }
 
@@ -1422,14 +1582,14 @@ int hass_combined_distill_fwd_bwd(const void* H_t, const void* H_d, const void* 
     if (rc != HASS_OK) return rc;
     if (!loss_ce || !(w_topk == w_topk)) return HASS_ERR_INVALID_ARG;
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u)) return HASS_ERR_WORKSPACE;
-    size_t base = 0;
-    rc = hass_topk_distill_workspace_bytes(N, d, V, K, &base);
-    if (rc != HASS_OK) return rc;
     CombinedStage c;
-    rc = combined_stage(N, d, V, K, base, &c);
+    rc = combined_stage(N, d, V, K, &c);
     if (rc != HASS_OK) return rc;
     if (workspace_bytes < c.total) return HASS_ERR_WORKSPACE;
     uint8_t* ws = static_cast<uint8_t*>(workspace);
+    PartRoom room;
+    room.at = reinterpret_cast<float*>(ws + c.total);
+    room.bytes = workspace_bytes - c.total;
     Combined cmb;
     cmb.w = w_topk;
     cmb.loss_ce = loss_ce;
@@ -1437,15 +1597,20 @@ int hass_combined_distill_fwd_bwd(const void* H_t, const void* H_d, const void* 
     cmb.T = reinterpret_cast<float*>(ws + c.T);
     cmb.Pt = reinterpret_cast<__nv_bfloat16*>(ws + c.Pt);
     return fused_impl(true, H_t, H_d, W, N, d, V, K, grad_loss, nullptr, nullptr, loss_topk, topk_idx, topk_q, lse_t,
-                      lse_d, dH_d, dH_dtype, workspace, base, static_cast<cudaStream_t>(cuda_stream), &cmb);
+                      lse_d, dH_d, dH_dtype, workspace, c.base, static_cast<cudaStream_t>(cuda_stream), &cmb, nullptr, false, &room);
 }
 
 // Device staging appended to the normal workspace by the *_host entry.
 struct HostStage {
-    size_t H_t, H_d, grad, loss, idx, q, lse_t, lse_d, dH, total;
+    size_t base, H_t, H_d, grad, loss, idx, q, lse_t, lse_d, dH, total, part_bytes;   // base, part_bytes: as in CombinedStage
 };
-static int host_stage(int64_t N, int64_t d, int64_t V, int32_t K, int dH_dtype, size_t base, HostStage* s) {
-    size_t off = align256(base);
+static int host_stage(int64_t N, int64_t d, int64_t V, int32_t K, int dH_dtype, HostStage* s) {
+    Layout L;
+    const int rc = make_layout(N, d, V, K, sm_count_or_default(), &L);
+    if (rc != HASS_OK) return rc;
+    s->base = L.total_pref;
+    s->part_bytes = L.part_bytes;
+    size_t off = align256(s->base);
     s->H_t = off;
     off = align256(off + static_cast<size_t>(N) * d * 2);
     s->H_d = off;
@@ -1465,18 +1630,17 @@ static int host_stage(int64_t N, int64_t d, int64_t V, int32_t K, int dH_dtype, 
     s->dH = off;
     off = align256(off + static_cast<size_t>(N) * d * (dH_dtype == HASS_FP32 ? 4 : 2));
     s->total = off;
-    (void)V;
     return HASS_OK;
 }
 
 int hass_topk_distill_host_workspace_bytes(int64_t N, int64_t d, int64_t V, int32_t K, int dH_dtype, size_t* bytes) {
     if (!bytes || (dH_dtype != HASS_BF16 && dH_dtype != HASS_FP32)) return HASS_ERR_INVALID_ARG;
-    size_t base = 0;
-    int rc = hass_topk_distill_workspace_bytes(N, d, V, K, &base);
+    int rc = check_sizes(N, d, V, K);
     if (rc != HASS_OK) return rc;
     HostStage s;
-    host_stage(N, d, V, K, dH_dtype, base, &s);
-    *bytes = s.total;
+    rc = host_stage(N, d, V, K, dH_dtype, &s);
+    if (rc != HASS_OK) return rc;
+    *bytes = s.total + s.part_bytes;
     return HASS_OK;
 }
 
@@ -1518,14 +1682,15 @@ int hass_topk_distill_fwd_bwd_host(const void* H_t_host, const void* H_d_host, c
     if (!H_t_host || !H_d_host || !W || !loss_host || !dH_d_host) return HASS_ERR_INVALID_ARG;
     if (dH_dtype != HASS_BF16 && dH_dtype != HASS_FP32) return HASS_ERR_INVALID_ARG;
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u)) return HASS_ERR_WORKSPACE;
-    size_t base = 0;
-    rc = hass_topk_distill_workspace_bytes(N, d, V, K, &base);
-    if (rc != HASS_OK) return rc;
     HostStage s;
-    host_stage(N, d, V, K, dH_dtype, base, &s);
+    rc = host_stage(N, d, V, K, dH_dtype, &s);
+    if (rc != HASS_OK) return rc;
     if (workspace_bytes < s.total) return HASS_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
+    PartRoom room;
+    room.at = reinterpret_cast<float*>(ws + s.total);
+    room.bytes = workspace_bytes - s.total;
     HostPipeResources* res = nullptr;
     rc = host_pipe_resources(&res);
     if (rc != HASS_OK) return rc;
@@ -1560,7 +1725,7 @@ int hass_topk_distill_fwd_bwd_host(const void* H_t_host, const void* H_d_host, c
     rc = fused2_impl(true, ws + s.H_t, ws + s.H_d, W, N, d, V, K, grad_dev, nullptr, nullptr,
                      reinterpret_cast<float*>(ws + s.loss), reinterpret_cast<int32_t*>(ws + s.idx),
                      reinterpret_cast<float*>(ws + s.q), reinterpret_cast<float*>(ws + s.lse_t),
-                     reinterpret_cast<float*>(ws + s.lse_d), ws + s.dH, dH_dtype, workspace, base, st, 0.f, nullptr, &pipe);
+                     reinterpret_cast<float*>(ws + s.lse_d), ws + s.dH, dH_dtype, workspace, s.base, st, 0.f, nullptr, &pipe, &room);
     if (rc == HASS_ERR_UNSUPPORTED) {
         // more row chunks than events (a very small workspace): one copy in, the call, one copy out
         const size_t hbytes = static_cast<size_t>(N) * d * 2;
@@ -1574,7 +1739,7 @@ int hass_topk_distill_fwd_bwd_host(const void* H_t_host, const void* H_d_host, c
         rc = fused2_impl(true, ws + s.H_t, ws + s.H_d, W, N, d, V, K, grad_dev, nullptr, nullptr,
                          reinterpret_cast<float*>(ws + s.loss), reinterpret_cast<int32_t*>(ws + s.idx),
                          reinterpret_cast<float*>(ws + s.q), reinterpret_cast<float*>(ws + s.lse_t),
-                         reinterpret_cast<float*>(ws + s.lse_d), ws + s.dH, dH_dtype, workspace, base, st);
+                         reinterpret_cast<float*>(ws + s.lse_d), ws + s.dH, dH_dtype, workspace, s.base, st, 0.f, nullptr, nullptr, &room);
         if (rc == HASS_OK && cudaMemcpyAsync(dH_d_host, ws + s.dH, static_cast<size_t>(N) * pipe.out_row_bytes,
                                              cudaMemcpyDeviceToHost, st) != cudaSuccess) {
             cudaGetLastError();
@@ -1634,7 +1799,7 @@ int hass_topk_distill_fwd_static_scratch_bytes(int64_t N, int64_t d, int64_t V, 
     if (rc != HASS_OK) return rc;
     // the forward needs the statistics / candidate part of the workspace layout only
     Layout L;
-    rc = make_layout(N, d, V, K, sm_count_or_default(), &L, nullptr);
+    rc = make_layout(N, d, V, K, sm_count_or_default(), &L);
     if (rc != HASS_OK) return rc;
     *bytes = L.fwd_end;
     return HASS_OK;

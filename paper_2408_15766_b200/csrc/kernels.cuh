@@ -30,16 +30,19 @@ constexpr int BM = 128;        // rows per tile (TMEM lanes)
 constexpr int BN = 256;        // columns per tile (one UMMA N)
 constexpr int BK = 64;         // contraction elements per pipeline stage (128 B of bf16: one swizzle row)
 constexpr int UMMA_K = 16;     // contraction elements per tcgen05.mma (bf16)
-constexpr int STAGES = 4;
 constexpr int A_STAGE_BYTES = BM * BK * 2;
-constexpr int B_STAGE_BYTES = BN * BK * 2;
+// CG = CTAs that work on one product (1, or a pair): each holds its own BM rows of A and BN / CG of the tile's columns
+__host__ __device__ constexpr int stages(int CG) { return CG == 2 ? 6 : 4; }
+__host__ __device__ constexpr int b_stage_bytes(int CG) { return BN / CG * BK * 2; }
+constexpr int OPERAND_BYTES = stages(1) * (A_STAGE_BYTES + b_stage_bytes(1));
+static_assert(OPERAND_BYTES == stages(2) * (A_STAGE_BYTES + b_stage_bytes(2)), "both forms use the same shared memory");
 constexpr int NUM_THREADS = 192;   // warp 0: TMA, warp 1: MMA + TMEM owner, warps 2-5: epilogue
 constexpr int TMEM_COLS = 512;     // two accumulator buffers of BN fp32 columns
 constexpr int MAX_PHASES = 48;
 constexpr int K_CAP = 256;         // == HASS_K_MAX
 constexpr int SPILL_STAGE_BYTES = 32 * 128;   // 32 rows x 64 bf16 of a spilled tile on their way to global memory
 constexpr int SPILL_STAGES = 2;               // per epilogue warp
-constexpr int SMEM_BYTES = STAGES * (A_STAGE_BYTES + B_STAGE_BYTES) + 4 * SPILL_STAGES * SPILL_STAGE_BYTES +
+constexpr int SMEM_BYTES = OPERAND_BYTES + 4 * SPILL_STAGES * SPILL_STAGE_BYTES +
                            1024 /*alignment slack*/ + 256 /*barriers*/;
 constexpr float LOG2E = 1.4426950408889634f;
 
@@ -49,6 +52,9 @@ enum { MODE_STATS = 0, MODE_PROBS = 1, MODE_OUT = 2 };
 // tiles l, l + S, l + 2S, ... CTA b < G * S works on row tile row_tile_begin + b / S, lane b % S, and
 // owns partial-result slot slot_base + b. All CTAs of a phase walk the column tiles in lockstep,
 // so a column tile of B is fetched from HBM once and then served from L2 to the G row tiles.
+// With CTA pairs (pair = 2) G is even and pair b < G / 2 * S works on row tiles row_tile_begin + 2 (b / S) + {0, 1}, lane
+// b % S; slots are numbered as before (row tile by row tile, S each). The last row tile of an odd number has a partner
+// beyond the matrix, whose CTA takes part in the products and writes nothing.
 struct Phase {
     int row_tile_begin, G, S, slot_base;
 };
@@ -56,15 +62,27 @@ struct Schedule {
     int n_phases;
     int total_slots;
     int max_ctas;          // largest G * S over the phases = grid size
-    int pad;
+    int pair;              // CTAs per product: 1 or 2
     Phase ph[MAX_PHASES];
 };
 
+// How MODE_OUT divides its output tiles (row tiles, or pairs of them, x column tiles of BN) over the `groups` CTAs or
+// pairs of the grid. Tile u = (row u % row_units, column tile u / row_units): the column tile's part of B is read by all
+// rows at about the same time. Tiles [0, whole) go out round by round, each contracted to its end; the last `rest`
+// tiles, which would leave most of a round idle, are cut into `cuts` equal pieces of the contraction that are dealt
+// out the same way (piece v = piece index v / rest of tile whole + v % rest: pieces at the same depth run together), stored as
+// fp32 partial tiles and added up by out_reduce_kernel. cuts = 1: whole = all tiles, rest = 0.
+struct OutPlan {
+    int pair, groups, row_units, whole, rest, cuts;
+    int part_rows;         // rows kept of a partial tile: BM, or all there are in a single row tile
+};
+
 struct GemmParams {
-    CUtensorMap tmA0, tmA1, tmB;
+    CUtensorMap tmA0, tmA1, tmB;   // boxes: 128 rows of A; of B the BN / pair columns that one CTA holds
     CUtensorMap tmSpill;   // MODE_STATS without Top-K lists (the draft sweep): the spill P as [chunk rows, p_pitch] bf16 with
                            // boxes of 64 columns x 32 rows, 128-byte swizzle, for TMA stores
     Schedule sched;
+    int row_tiles;         // row tiles of this launch; a pair's second tile may lie beyond
     int row_tiles0;        // row tiles [0, row_tiles0) read A0, the others A1 (tile index - row_tiles0)
     int topk_row_tiles;    // leading row tiles whose rows collect Top-K candidates (MODE_STATS)
     int a_row_offset;      // added to A0's row coordinate (chunked backward)
@@ -103,6 +121,8 @@ struct GemmParams {
     int out_align32;       // out base and row pitch are multiples of 32 bytes (256-bit stores allowed)
     long long out_pitch;   // elements
     unsigned int* status;
+    OutPlan plan;
+    float* part;           // [cuts][rest][pair][part_rows][BN] partial tiles
     const unsigned int* only_if_range;   // nullptr, or: run only if this status word reports a range overflow
     // The single-sweep route (spilling sweeps with Top-K lists): every spilling row leaves the ordered key of its
     // largest logit in row_zmax[row tile * 128 + row] (atomicMax over the lanes of the row tile; zeroed by the
@@ -243,7 +263,13 @@ __device__ __forceinline__ uint32_t compact_candidates(uint2* buf, int n, int K,
 enum { TOPK_REG = 0, TOPK_BUF = 1, TOPK_NONE = 2 };
 constexpr int K_REG = 16;
 
-template <int MODE, int TOPK = TOPK_BUF>
+// CG: CTAs per product. The kernel is bound by the tensor pipe and, in calls of many milliseconds, by the power cap. A pair
+// (tcgen05 cta_group::2, 256 x 256 tile) fetches 32 KB per CTA and k block instead of 48 (10 instead of 15 TB/s out of
+// L2) and reads half as much of B from shared memory; with the stages smaller there are six instead of four. A step of
+// a pair takes 0.89-0.91 of the time of the two single steps it replaces (sweep of 8192 rows x 4096 x 32000: 1.77 -> 1.45 ms
+// = 1480 TFLOP/s in short runs; 1.24 -> 1.30 PFLOP/s where the power cap holds). Single CTAs stay for one row tile, where
+// a partner would have nothing to do, and where an odd number of row tiles makes pairs slower (plan_launch, plan_out).
+template <int MODE, int TOPK, int CG>
 __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_constant__ GemmParams p) {
     constexpr bool B_MN_MAJOR = (MODE == MODE_OUT);
     // conditional launch (the exact route that follows a fused call): nothing to do unless the fused sweep
@@ -252,8 +278,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t smemA = smem_base;
+    constexpr int STAGES = stages(CG);
+    constexpr int B_STAGE_BYTES = b_stage_bytes(CG);
     const uint32_t smemB = smem_base + STAGES * A_STAGE_BYTES;
-    const uint32_t spill_stage = smemB + STAGES * B_STAGE_BYTES;      // [epilogue warp][SPILL_STAGES] x SPILL_STAGE_BYTES
+    const uint32_t spill_stage = smem_base + OPERAND_BYTES;      // [epilogue warp][SPILL_STAGES] x SPILL_STAGE_BYTES
     const uint32_t bar_base = spill_stage + 4 * SPILL_STAGES * SPILL_STAGE_BYTES;
     // barriers: full[STAGES], empty[STAGES], tmem_full[2], tmem_empty[2]; then tmem pointer, abort flag
     auto full_bar = [&](int s) { return bar_base + 8u * s; };
@@ -262,13 +290,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
     auto tempty_bar = [&](int b) { return bar_base + 8u * (2 * STAGES + 2 + b); };
     uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
     uint32_t* tmem_ptr_smem =
-        reinterpret_cast<uint32_t*>(smem_gen + STAGES * (A_STAGE_BYTES + B_STAGE_BYTES) + 4 * SPILL_STAGES * SPILL_STAGE_BYTES +
+        reinterpret_cast<uint32_t*>(smem_gen + OPERAND_BYTES + 4 * SPILL_STAGES * SPILL_STAGE_BYTES +
                                     8 * (2 * STAGES + 4));
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_ptr_smem + 1);
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    const int cta = blockIdx.x;
+    const int cta = CG == 2 ? blockIdx.x >> 1 : blockIdx.x;             // CTA or pair
+    const uint32_t rank = CG == 2 ? cluster_ctarank() : 0;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -277,7 +306,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(tfull_bar(b), 1);
-            mbar_init(tempty_bar(b), 4);
+            mbar_init(tempty_bar(b), 4 * CG);
         }
         *abort_flag = 0;
         fence_barrier_init();
@@ -287,23 +316,52 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
         if (MODE == MODE_STATS) prefetch_tensormap(&p.tmA1);
     }
     if (warp == 1) {
-        tmem_alloc(smem_u32(tmem_ptr_smem), TMEM_COLS);
-        tmem_relinquish();
+        if (CG == 2) {
+            tmem_alloc_pair(smem_u32(tmem_ptr_smem), TMEM_COLS);
+            tmem_relinquish_pair();
+        } else {
+            tmem_alloc(smem_u32(tmem_ptr_smem), TMEM_COLS);
+            tmem_relinquish();
+        }
     }
     tc_fence_before_sync();
     __syncthreads();
+    if (CG == 2) cluster_sync();      // the partner's barriers are initialised, its tensor memory is allocated
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_ptr_smem;
 
-    // Calls f(row_tile, lane, S, slot) for every item of this CTA; f returns false to stop.
+    // Calls f(row_tile, lane, S, slot, first k block, end of k blocks) for every item of this CTA; f returns false to
+    // stop. MODE_OUT: one column tile (= lane; S = all of them), slot = the partial tile it goes to or -1.
     auto for_each_item = [&](auto&& f) {
-        for (int ph = 0; ph < p.sched.n_phases; ++ph) {
-            const Phase P = p.sched.ph[ph];
-            if (cta < P.G * P.S) {
-                const int gi = cta / P.S;
-                if (!f(P.row_tile_begin + gi, cta - gi * P.S, P.S, P.slot_base + cta)) return;
+        if constexpr (MODE == MODE_OUT) {
+            const OutPlan& o = p.plan;
+            for (int u = cta; u < o.whole; u += o.groups)
+                if (!f(u % o.row_units * CG + static_cast<int>(rank), u / o.row_units, p.col_tiles, -1, 0, p.k_blocks)) return;
+            for (int v = cta; v < o.rest * o.cuts; v += o.groups) {
+                const int z = v / o.rest, u = o.whole + v - z * o.rest;
+                const int kb0 = static_cast<int>(static_cast<long long>(p.k_blocks) * z / o.cuts);
+                const int kb1 = static_cast<int>(static_cast<long long>(p.k_blocks) * (z + 1) / o.cuts);
+                if (!f(u % o.row_units * CG + static_cast<int>(rank), u / o.row_units, p.col_tiles,
+                       v * CG + static_cast<int>(rank), kb0, kb1))
+                    return;
+            }
+        } else {
+            for (int ph = 0; ph < p.sched.n_phases; ++ph) {
+                const Phase P = p.sched.ph[ph];
+                if (cta < P.G / CG * P.S) {
+                    const int gi = cta / P.S;
+                    const int ln = cta - gi * P.S;
+                    const int ri = gi * CG + static_cast<int>(rank);
+                    if (!f(P.row_tile_begin + ri, ln, P.S, P.slot_base + ri * P.S + ln, 0, p.k_blocks)) return;
+                }
             }
         }
+    };
+    // a lane that does not begin with column tile 0 computes it first where its rows spill (t = -1); a pair agrees
+    auto first_tile = [&](int rt, int ln) {
+        if (MODE != MODE_STATS || ln == 0) return 0;
+        const int rt0 = rt - static_cast<int>(rank);
+        return spills(p, rt0) || (CG == 2 && spills(p, rt0 + 1)) ? -1 : 0;
     };
 
     if (warp == 0) {
@@ -311,27 +369,35 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
         if (lane == 0) {
             int stage = 0;
             uint32_t phase = 0;
-            for_each_item([&](int rt, int ln, int S, int) {
+            for_each_item([&](int rt, int ln, int S, int, int kb0, int kb1) {
                 const bool second = (MODE == MODE_STATS) && rt >= p.row_tiles0;
                 const CUtensorMap* tmA = second ? &p.tmA1 : &p.tmA0;
                 const int row0 = p.a_row_offset + (second ? rt - p.row_tiles0 : rt) * BM;
-                const int t0 = (MODE == MODE_STATS && spills(p, rt) && ln != 0) ? -1 : 0;
+                const int t0 = first_tile(rt, ln);
                 const int nt = (p.col_tiles - ln + S - 1) / S;
                 for (int t = t0; t < nt; ++t) {
                     const int ct = t < 0 ? 0 : ln + t * S;   // t = -1: column tile 0, for the row references only
-                    for (int kb = 0; kb < p.k_blocks; ++kb) {
+                    for (int kb = kb0; kb < kb1; ++kb) {
                         if (!wait_barrier(empty_bar(stage), phase ^ 1u, abort_flag, p.status, 1)) return false;
-                        mbar_arrive_expect_tx(full_bar(stage), A_STAGE_BYTES + B_STAGE_BYTES);
-                        tma_load_2d(smemA + stage * A_STAGE_BYTES, tmA, full_bar(stage), kb * BK, row0);
+                        // a pair's bytes are all counted on the barrier of its first CTA, whose thread issues the products
+                        if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), CG * (A_STAGE_BYTES + B_STAGE_BYTES));
+                        const uint32_t bar = CG == 2 ? map_to_rank(full_bar(stage), 0) : full_bar(stage);
+                        auto load = [&](uint32_t dst, const CUtensorMap* tm, int x, int y) {
+                            if (CG == 2)
+                                tma_load_2d_pair(dst, tm, bar, x, y);
+                            else
+                                tma_load_2d(dst, tm, bar, x, y);
+                        };
+                        const int col0 = ct * BN + static_cast<int>(rank) * (BN / CG);
+                        load(smemA + stage * A_STAGE_BYTES, tmA, kb * BK, row0);
                         if (!B_MN_MAJOR) {
-                            tma_load_2d(smemB + stage * B_STAGE_BYTES, &p.tmB, full_bar(stage), kb * BK, ct * BN);
+                            load(smemB + stage * B_STAGE_BYTES, &p.tmB, kb * BK, col0);
                         } else {
-                            // B tile = BK contraction rows x BN contiguous columns, fetched as BN/64 boxes
+                            // B tile = BK contraction rows x BN / CG contiguous columns, fetched as boxes
                             // of 64 columns (one 128-byte swizzle row) x BK rows
 #pragma unroll
-                            for (int j = 0; j < BN / 64; ++j)
-                                tma_load_2d(smemB + stage * B_STAGE_BYTES + j * (BK * 128), &p.tmB, full_bar(stage),
-                                            ct * BN + j * 64, kb * BK);
+                            for (int j = 0; j < BN / CG / 64; ++j)
+                                load(smemB + stage * B_STAGE_BYTES + j * (BK * 128), &p.tmB, col0 + j * 64, kb * BK);
                         }
                         if (++stage == STAGES) {
                             stage = 0;
@@ -344,20 +410,20 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
         }
     } else if (warp == 1) {
         // ===================== MMA issuer =====================
-        if (lane == 0) {
-            constexpr uint32_t idesc = make_idesc_bf16(BM, BN, 0, B_MN_MAJOR ? 1 : 0);
+        if (lane == 0 && rank == 0) {
+            constexpr uint32_t idesc = make_idesc_bf16(CG * BM, BN, 0, B_MN_MAJOR ? 1 : 0);
             int stage = 0;
             uint32_t phase = 0;
             int ab = 0;
             uint32_t aphase = 0;
-            for_each_item([&](int rt, int ln, int S, int) {
-                const int t0 = (MODE == MODE_STATS && spills(p, rt) && ln != 0) ? -1 : 0;
+            for_each_item([&](int rt, int ln, int S, int, int kb0, int kb1) {
+                const int t0 = first_tile(rt, ln);
                 const int nt = (p.col_tiles - ln + S - 1) / S;
                 for (int t = t0; t < nt; ++t) {
                     if (!wait_barrier(tempty_bar(ab), aphase ^ 1u, abort_flag, p.status, 2)) return false;
                     tc_fence_after_sync();
                     const uint32_t d_tmem = tmem_base + ab * BN;
-                    for (int kb = 0; kb < p.k_blocks; ++kb) {
+                    for (int kb = kb0; kb < kb1; ++kb) {
                         if (!wait_barrier(full_bar(stage), phase, abort_flag, p.status, 3)) return false;
                         tc_fence_after_sync();
                         // A: K-major, 8-row groups 1024 B apart. B: K-major likewise, or MN-major with
@@ -372,15 +438,25 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                             const uint64_t a_adv = static_cast<uint64_t>((k * UMMA_K * 2) >> 4);
                             const uint64_t b_adv = B_MN_MAJOR ? static_cast<uint64_t>((k * UMMA_K * 128) >> 4)
                                                               : static_cast<uint64_t>((k * UMMA_K * 2) >> 4);
-                            umma_bf16(d_tmem, a_desc + a_adv, b_desc + b_adv, idesc, (kb | k) != 0 ? 1u : 0u);
+                            if (CG == 2)
+                                umma_bf16_pair(d_tmem, a_desc + a_adv, b_desc + b_adv, idesc, (kb - kb0 | k) != 0 ? 1u : 0u);
+                            else
+                                umma_bf16(d_tmem, a_desc + a_adv, b_desc + b_adv, idesc, (kb - kb0 | k) != 0 ? 1u : 0u);
                         }
-                        umma_commit(empty_bar(stage));   // frees the stage once these MMAs have read it
+                        // frees the stage (of both CTAs) once these MMAs have read it
+                        if (CG == 2)
+                            umma_commit_pair(empty_bar(stage));
+                        else
+                            umma_commit(empty_bar(stage));
                         if (++stage == STAGES) {
                             stage = 0;
                             phase ^= 1u;
                         }
                     }
-                    umma_commit(tfull_bar(ab));          // accumulator complete
+                    if (CG == 2)                         // accumulator complete
+                        umma_commit_pair(tfull_bar(ab));
+                    else
+                        umma_commit(tfull_bar(ab));
                     ab ^= 1;
                     if (ab == 0) aphase ^= 1u;
                 }
@@ -414,15 +490,16 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
         const uint32_t pend_i = pend_v + 32 * 128 * 4;
         constexpr int lo = 0;
 
-        for_each_item([&](int rt, int ln, int S, int slot) {
+        for_each_item([&](int rt, int ln, int S, int slot, int, int) {
             const int g_row = p.row_global_offset + rt * BM + r_local;
-            const bool row_ok = g_row < p.rows_valid;
+            const bool tile_ok = CG == 1 || rt < p.row_tiles;     // false: the partner of the last row tile, nothing to write
+            const bool row_ok = tile_ok && g_row < p.rows_valid;
             // ---- per-item state ----
             float m = -INFINITY, s = 0.f, thr = -INFINITY;        // MODE_STATS; thr = admission threshold in force
             float thr_own = -INFINITY;                            // K-th (K_REG-th) largest logit of this lane's own list
             float thr_sh = -INFINITY;                             // just below the best threshold published by the other lanes
             bool want_topk = false;
-            const bool spill = MODE == MODE_STATS && spills(p, rt);
+            const bool spill = MODE == MODE_STATS && tile_ok && spills(p, rt);
             const bool track_zmax = MODE == MODE_STATS && TOPK != TOPK_NONE && spill && p.row_zmax != nullptr;
             float zmax = -INFINITY;                               // the row's largest logit in this lane's column tiles
             float ref2 = 0.f;                                     // spill rows: exponent offset (log2 units)
@@ -431,7 +508,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
             const float* sg = nullptr;
             int cur = 0, nxt = INT_MAX;
             if (MODE == MODE_STATS) {
-                want_topk = HAS_TOPK && rt < p.topk_row_tiles;
+                want_topk = HAS_TOPK && tile_ok && rt < p.topk_row_tiles;
                 if (HAS_TOPK) cbuf = p.cand + (static_cast<long long>(slot) * BM + r_local) * p.cap;
                 cnt = 0;
                 if (USE_REG) {
@@ -457,7 +534,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                 cz = p.cap_z + static_cast<long long>(g_row) * p.K;
                 nxt = si[0];
             }
-            const int t0 = (spill && ln != 0) ? -1 : 0;
+            const int t0 = first_tile(rt, ln);
             const int nt = (p.col_tiles - ln + S - 1) / S;
             for (int t = t0; t < nt; ++t) {
                 const int ct = t < 0 ? 0 : ln + t * S;
@@ -467,7 +544,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                 tc_fence_after_sync();
                 const uint32_t t_row = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + ab * BN;
                 const int col_base = ct * BN;
-                bool skip_tile = false;
+                const bool skip_tile = t < 0 || !tile_ok;
                 if (MODE == MODE_STATS && spill && t == t0) {
                     // Reference exponent of this row: its largest logit in column tile 0. Every lane of
                     // the row tile computes tile 0 first and so derives the same value.
@@ -490,7 +567,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                     // 2^191 of headroom above the reference before bf16 / fp32 overflow
                     ref2 = fmaf(mx, LOG2E, 64.f);
                     m = ref2 * (1.0f / LOG2E);
-                    skip_tile = t < 0;
                 }
                 if (MODE == MODE_STATS && HAS_TOPK && !USE_REG && want_topk && t == 0 && p.n_cols - col_base >= BN) {
                     // First tile of the sweep, buffer empty, no threshold yet: admitting all 256 logits would fill
@@ -737,6 +813,15 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
 #pragma unroll
                         for (int j = 0; j < 32; ++j) o[j] = __uint_as_float(r[j]);
                         const bool full = col0 + 32 <= p.n_cols;
+                        if (slot >= 0) {
+                            // a piece of the contraction: the accumulator as it is
+                            float* dst = p.part + (static_cast<long long>(slot) * p.plan.part_rows + r_local) * BN + ch * 32;
+#pragma unroll
+                            for (int g8 = 0; g8 < 4; ++g8)
+                                st_global_v8(dst + 8 * g8, r[8 * g8], r[8 * g8 + 1], r[8 * g8 + 2], r[8 * g8 + 3], r[8 * g8 + 4],
+                                             r[8 * g8 + 5], r[8 * g8 + 6], r[8 * g8 + 7]);
+                            continue;
+                        }
                         if (p.sparse != nullptr) {
                             // dH_d = coef * (spilled tile x W) - sum_{x in Omega_hat} g q(x) W[x, :]
                             const float* sp = p.sparse + static_cast<long long>(rt * BM + r_local) * p.out_pitch + col0;
@@ -814,7 +899,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                 // accumulator drained: hand the buffer back to the MMA warp
                 tc_fence_before_sync();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(tempty_bar(ab));
+                if (lane == 0) {
+                    if (CG == 2)
+                        mbar_arrive_cluster(map_to_rank(tempty_bar(ab), 0));
+                    else
+                        mbar_arrive(tempty_bar(ab));
+                }
                 ab ^= 1;
                 if (ab == 0) aphase ^= 1u;
                 if (MODE == MODE_STATS && want_topk && p.thr_share != nullptr && S > 1) {
@@ -833,7 +923,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                     thr = fmaxf(thr, thr_sh);
                 }
             }
-            if (MODE == MODE_STATS) {
+            if (MODE == MODE_STATS && tile_ok) {
                 const long long so = static_cast<long long>(slot) * BM + r_local;
                 p.part_m[so] = m;
                 p.part_s[so] = s;
@@ -864,10 +954,50 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
         const unsigned long long t0 = globaltimer_ns();
         while (globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
     }
+    if (CG == 2) cluster_sync();      // the partner's products, loads and arrivals on this CTA's memory are done
     if (warp == 1) {
         tc_fence_after_sync();
-        tmem_dealloc(tmem_base, TMEM_COLS);
+        if (CG == 2)
+            tmem_dealloc_pair(tmem_base, TMEM_COLS);
+        else
+            tmem_dealloc(tmem_base, TMEM_COLS);
     }
+}
+
+// ---------------------------------------------------------------------------------------------
+// out_reduce_kernel: adds up the partial tiles of MODE_OUT in the order of the contraction and finishes them as its
+// epilogue does. One thread per four columns; memory-bound (reads cuts x, writes 1 x the rest tiles).
+__global__ void __launch_bounds__(256) out_reduce_kernel(const __grid_constant__ GemmParams p) {
+    if (p.only_if_range != nullptr && ((*p.only_if_range) & 0xffu) != 2u) return;
+    const OutPlan& o = p.plan;
+    const long long i = static_cast<long long>(blockIdx.x) * 256 + threadIdx.x;
+    const int c = static_cast<int>(i % (BN / 4)) * 4;
+    const int r_local = static_cast<int>(i / (BN / 4) % BM);
+    const int tile = static_cast<int>(i / (BN / 4 * BM));             // rest tile * pair + rank
+    const int u = o.whole + tile / o.pair;
+    const int rt = u % o.row_units * o.pair + tile % o.pair;
+    const int col = u / o.row_units * BN + c;
+    const int row = p.row_global_offset + rt * BM + r_local;
+    if (tile >= o.rest * o.pair || rt >= p.row_tiles || row >= p.rows_valid || col >= p.n_cols) return;
+    const float4* src = reinterpret_cast<const float4*>(p.part + (static_cast<long long>(tile) * o.part_rows + r_local) * BN + c);
+    const long long step = static_cast<long long>(o.rest) * o.pair * o.part_rows * (BN / 4);
+    float4 a = src[0];
+#pragma unroll 4
+    for (int z = 1; z < o.cuts; ++z) {
+        const float4 v = src[z * step];
+        a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
+    }
+    if (p.coef != nullptr) {
+        const float coef = p.coef[row];
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (p.sparse != nullptr) s = *reinterpret_cast<const float4*>(p.sparse + static_cast<long long>(rt * BM + r_local) * p.out_pitch + col);
+        a.x = fmaf(coef, a.x, -s.x); a.y = fmaf(coef, a.y, -s.y); a.z = fmaf(coef, a.z, -s.z); a.w = fmaf(coef, a.w, -s.w);
+    }
+    const long long at = static_cast<long long>(row) * p.out_pitch + col;
+    if (p.out_fp32)
+        *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + at) = a;
+    else
+        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + at) = make_uint2(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w));
 }
 
 // ---------------------------------------------------------------------------------------------
