@@ -138,26 +138,23 @@ int hass_topk_distill_bwd(const void* H_d, const void* W, int64_t N, int64_t d, 
  * target rows are swept first (statistics and Top-K candidates), Omega_hat is selected, then the
  * draft rows are swept: their statistics, their logits at the row's Omega_hat (copied out of the
  * fp32 accumulator for Eq. 1), and the tile itself, written to the workspace as bf16 values
- * 2^(z_d log2(e) - ref2), ref2 a per-row exponent fixed from the row's largest logit among the
- * first 256 tokens. With coef = g S_q 2^ref2 / sum_v e^{z_d},
+ * 2^(z_d log2(e) - ref2), ref2 a per-row exponent fixed from the row's draft logit at the most
+ * probable token of Omega_hat. With coef = g S_q 2^ref2 / sum_v e^{z_d},
  *     dz_d(v) = coef ( spill(v) - [v in Omega_hat] g q(v) / coef ),
  * so the K entries of a row at its Omega_hat tokens are lowered in place (in bf16) and
  * dH_d = coef (spill W) is formed by the second GEMM, whose epilogue applies the row scale.
  * Precision: every entry of dz_d, the Omega_hat entries included, reaches the tensor cores in bf16
  * (2^-9 relative); the loss uses fp32 logits throughout.
- * Range condition: the fixed exponent holds as long as no draft logit of a row exceeds that
- * row's largest logit among tokens 0..255 by more than about 130 (natural-log units; a probability
- * ratio of e^130). The sweep detects a violation; the call therefore also enqueues the separate
- * forward and the recomputing backward as conditional launches that return at once unless a
- * violation was detected, in which case they redo the whole call exactly. The result is correct
- * either way; the conditional launches cost about 0.3 % when they have nothing to do. The _draft
- * form and the Top-P variant work the same way.
- * hass_combined_distill_fwd_bwd and the Bi-directional variant handle a violation differently: their
- * sweep records every row's largest logit, and the whole sequence is enqueued a second time as
- * conditional launches that take each row's exponent from that record (no logit of the row can
- * exceed it); a violation therefore costs one more pass and the result is correct either way.
- * HASS_ERR_RANGE is what hass_check reports if a violation was detected and nothing redid the call
- * (none of the entry points of this version leaves it at that).
+ * Range condition: the fixed exponent holds as long as no draft logit of a row exceeds the one it
+ * was taken from by more than about 130 (natural-log units; a probability ratio of e^130). The sweep
+ * detects a violation and records every row's largest logit; the call therefore also enqueues the
+ * steps from the draft sweep on a second time, as conditional launches that return at once unless a
+ * violation was detected, in which case they redo the call with each row's exponent taken from that
+ * record (no logit of the row can exceed it). The result is correct either way. The _draft form and
+ * the Top-P variant work the same way, and so do hass_combined_distill_fwd_bwd and the Bi-directional
+ * variant, whose exponent comes from the row's largest logit among the first 256 tokens and whose
+ * second pass repeats the whole sequence.
+ * (HASS_ERR_RANGE is kept for callers that name it; no entry point of this version returns it.)
  */
 int hass_topk_distill_fwd_bwd(const void* H_t, const void* H_d, const void* W, int64_t N, int64_t d,
                               int64_t V, int32_t K, const float* grad_loss, float* loss,

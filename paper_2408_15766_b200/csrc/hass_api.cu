@@ -331,6 +331,8 @@ static int make_layout(long long N, long long d, long long V, int K, int sms, La
     L->status = off;
     off += 256;
     const size_t slots = static_cast<size_t>(slot_cap);
+    L->thr_share = off;                     // admission thresholds the lanes of a row tile publish to each other; behind the
+    off = align256(off + slots * BM * 4);   // status block, so that one memset clears both
     L->part_m = off;
     off = align256(off + slots * BM * 4);
     L->part_s = off;
@@ -338,8 +340,6 @@ static int make_layout(long long N, long long d, long long V, int K, int sms, La
     L->cand_v = off;                        // candidate buffers: (logit, token id) pairs, cand_cap(K) per (row, slot)
     off = align256(off + slots * BM * 8 * topk_cap(K));
     L->cand_i = off;                        // entries in use per (row, slot)
-    off = align256(off + slots * BM * 4);
-    L->thr_share = off;                     // admission thresholds the lanes of a row tile publish to each other
     off = align256(off + slots * BM * 4);
     L->fwd_end = off;                       // what the forward-only entry points use
     L->sidx = off;
@@ -401,7 +401,7 @@ static void log_schedule(const char* what, const Schedule& s) {
 
 template <int MODE>
 static int launch_gemm(const GemmParams& p, cudaStream_t st, int kind = -1) {
-    KernelTimer timer(p.only_if_range ? KIND_CONDITIONAL : (kind >= 0 ? kind : MODE), st);
+    KernelTimer timer(p.gate ? KIND_CONDITIONAL : (kind >= 0 ? kind : MODE), st);
     const bool pair = p.sched.pair == 2;
     GemmFn fn;
     if (MODE == MODE_STATS && p.topk_row_tiles == 0 && p.cap_z != nullptr)
@@ -427,6 +427,75 @@ static int launch_gemm(const GemmParams& p, cudaStream_t st, int kind = -1) {
     if (cudaLaunchKernelEx(&cfg, fn, p) != cudaSuccess) {
         cudaGetLastError();
         return HASS_ERR_CUDA;
+    }
+    g_launches.fetch_add(1);
+    return cudaGetLastError() == cudaSuccess ? HASS_OK : HASS_ERR_CUDA;
+}
+
+// Clears the status block (only_thresholds: not) and the published thresholds of `slots` slots.
+static int clear_status(uint8_t* ws, const Layout& L, int slots, cudaStream_t st, bool only_thresholds = false) {
+    const size_t from = only_thresholds ? L.thr_share : L.status;
+    if (only_thresholds && slots == 0) return HASS_OK;
+    if (cudaMemsetAsync(ws + from, 0, L.thr_share + static_cast<size_t>(slots) * BM * 4 - from, st) != cudaSuccess) {
+        cudaGetLastError();
+        return HASS_ERR_CUDA;
+    }
+    return HASS_OK;
+}
+
+// Four warps per row while that is at most four blocks per SM, one warp beyond. The lists of K <= 16 hold 16 entries each
+// and need the smaller window. Against one warp per row that walks the lists one after the other: 61 rows x 125 lists
+// 113 -> 15 us, 4096 rows x 4 lists 40 -> 9 us (22 with the dot product for the reference exponent, which saves the
+// draft sweep its extra tile: 25 us here, half of it at 61 rows), 4096 rows of K = 64 275 -> 130 us.
+static int launch_select(const SelectParams& sp, int sms, cudaStream_t st) {
+    {
+        KernelTimer timer(sp.gate ? KIND_CONDITIONAL : KIND_FINALIZE, st);
+        const bool reg = sp.cap == K_REG;
+        if (sp.rows <= 4 * sms) {
+            if (reg)
+                select_kernel<4, 512><<<sp.rows, SEL_WARPS * 32, 0, st>>>(sp);
+            else
+                select_kernel<4, 1024><<<sp.rows, SEL_WARPS * 32, 0, st>>>(sp);
+        } else {
+            if (reg)
+                select_kernel<1, 512><<<ceil_div(sp.rows, SEL_WARPS), SEL_WARPS * 32, 0, st>>>(sp);
+            else
+                select_kernel<1, 1024><<<ceil_div(sp.rows, SEL_WARPS), SEL_WARPS * 32, 0, st>>>(sp);
+        }
+    }
+    g_launches.fetch_add(1);
+    return cudaGetLastError() == cudaSuccess ? HASS_OK : HASS_ERR_CUDA;
+}
+
+// What select_kernel needs to pick the K best of the candidates that sweep `p` left on its row tiles from first_tile on
+static SelectParams select_params(const GemmParams& p, int first_tile, int row_begin, int rows, int* idx_out, float* q_out,
+                                  int out_pitch, float* lse) {
+    SelectParams sp;
+    std::memset(&sp, 0, sizeof(sp));
+    sp.sched = p.sched;
+    sp.first_tile = first_tile;
+    sp.K = p.K;
+    sp.cap = p.cap;
+    sp.row_begin = row_begin;
+    sp.rows = rows;
+    sp.from_sweep = 1;
+    sp.part_m = p.part_m;
+    sp.part_s = p.part_s;
+    sp.cand = p.cand;
+    sp.cand_n = p.cand_n;
+    sp.thr_share = p.thr_share;
+    sp.idx_out = idx_out;
+    sp.q_out = q_out;
+    sp.out_pitch = out_pitch;
+    sp.lse_t = lse;
+    sp.gate = p.gate;
+    return sp;
+}
+
+static int launch_finalize(const FinalizeParams& f, cudaStream_t st) {
+    {
+        KernelTimer timer(f.gate ? KIND_CONDITIONAL : KIND_FINALIZE, st);
+        finalize_kernel<<<f.rows, FIN_WARPS * 32, 0, st>>>(f);
     }
     g_launches.fetch_add(1);
     return cudaGetLastError() == cudaSuccess ? HASS_OK : HASS_ERR_CUDA;
@@ -467,7 +536,7 @@ static int launch_out(GemmParams& p, const PartRoom& room, int sms, cudaStream_t
                      p.plan.whole, p.plan.rest, p.plan.cuts);
     const int rc = launch_gemm<MODE_OUT>(p, st);
     if (rc != HASS_OK || p.plan.rest == 0) return rc;
-    KernelTimer timer(p.only_if_range ? KIND_CONDITIONAL : KIND_OUT, st);
+    KernelTimer timer(p.gate ? KIND_CONDITIONAL : KIND_OUT, st);
     out_reduce_kernel<<<p.plan.rest * p.plan.pair * (BM * BN / 4 / 256), 256, 0, st>>>(p);
     g_launches.fetch_add(1);
     return cudaGetLastError() == cudaSuccess ? HASS_OK : HASS_ERR_CUDA;
@@ -478,8 +547,7 @@ static int launch_out(GemmParams& p, const PartRoom& room, int sms, cudaStream_t
 static int forward_impl(bool with_target, const void* H_t, const void* H_d, const void* W, long long N, long long d,
                         long long V, int K, const int* idx_in, const float* q_in, float* loss, int* idx_out,
                         float* q_out, float* lse_t, float* lse_d, void* workspace, size_t workspace_bytes,
-                        cudaStream_t st, const unsigned int* only_if_range = nullptr, float top_p = 0.f,
-                        int* topk_n = nullptr) {
+                        cudaStream_t st) {
     int rc = check_sizes(N, d, V, K);
     if (rc != HASS_OK) return rc;
     if (!H_d || !W || !loss || !lse_d || !aligned16(H_d) || !aligned16(W)) return HASS_ERR_INVALID_ARG;
@@ -498,12 +566,6 @@ static int forward_impl(bool with_target, const void* H_t, const void* H_d, cons
     if (workspace_bytes < L.fwd_end) return HASS_ERR_WORKSPACE;
     const int RT = ceil_div(N, BM), CT = ceil_div(V, BN);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
-    // every public call starts with a clean status word (a conditional follow-up keeps the one it reads)
-    if (!only_if_range && cudaMemsetAsync(ws + L.status, 0, 256, st) != cudaSuccess) {
-        cudaGetLastError();
-        return HASS_ERR_CUDA;
-    }
-
     GemmParams p;
     std::memset(&p, 0, sizeof(p));
     p.row_tiles = with_target ? 2 * RT : RT;
@@ -537,14 +599,15 @@ static int forward_impl(bool with_target, const void* H_t, const void* H_d, cons
     p.cand = reinterpret_cast<uint2*>(ws + L.cand_v);
     p.cand_n = reinterpret_cast<int*>(ws + L.cand_i);
     p.status = reinterpret_cast<unsigned int*>(ws + L.status);
-    p.only_if_range = only_if_range;
-    p.thr_share = reinterpret_cast<float*>(ws + L.thr_share);
-    if (cudaMemsetAsync(p.thr_share, 0xff, static_cast<size_t>(p.sched.total_slots) * BM * 4, st) != cudaSuccess) {   // NaN
-        cudaGetLastError();
-        return HASS_ERR_CUDA;
-    }
+    p.thr_share = reinterpret_cast<unsigned int*>(ws + L.thr_share);
+    rc = clear_status(ws, L, p.sched.total_slots, st);
+    if (rc != HASS_OK) return rc;
     rc = launch_gemm<MODE_STATS>(p, st);
     if (rc != HASS_OK) return rc;
+    if (with_target) {
+        rc = launch_select(select_params(p, 0, 0, static_cast<int>(N), idx_out, q_out, K, lse_t), di.sms, st);
+        if (rc != HASS_OK) return rc;
+    }
 
     FinalizeParams f;
     std::memset(&f, 0, sizeof(f));
@@ -553,38 +616,24 @@ static int forward_impl(bool with_target, const void* H_t, const void* H_d, cons
     f.rows = static_cast<int>(N);
     f.d = static_cast<int>(d);
     f.K = K;
-    f.cap = topk_cap(K);
     f.row_tiles_t = with_target ? RT : 0;
     f.part_m = p.part_m;
     f.part_s = p.part_s;
-    f.cand = p.cand;
-    f.cand_n = p.cand_n;
     f.H_d = static_cast<const __nv_bfloat16*>(H_d);
     f.W = static_cast<const __nv_bfloat16*>(W);
-    f.idx_in = idx_in;
-    f.q_in = q_in;
+    f.idx = with_target ? idx_out : const_cast<int*>(idx_in);
+    f.q = with_target ? q_out : const_cast<float*>(q_in);
+    f.idx_pitch = K;
     f.loss = loss;
-    f.idx_out = idx_out;
-    f.q_out = q_out;
     f.lse_t = lse_t;
     f.lse_d = lse_d;
-    f.only_if_range = only_if_range;
-    f.top_p = top_p;
-    f.n_out = topk_n;
-    const int warps_per_block = 8;
-    {
-        KernelTimer timer(only_if_range ? KIND_CONDITIONAL : KIND_FINALIZE, st);
-        finalize_kernel<<<ceil_div(N, warps_per_block), warps_per_block * 32, 0, st>>>(f);
-    }
-    g_launches.fetch_add(1);
-    return cudaGetLastError() == cudaSuccess ? HASS_OK : HASS_ERR_CUDA;
+    return launch_finalize(f, st);
 }
 
 // ---- backward ---------------------------------------------------------------------------------
 static int backward_impl(const void* H_d, const void* W, long long N, long long d, long long V, int K,
                          const int* topk_idx, const float* topk_q, const float* lse_d, const float* grad_loss,
-                         void* dH_d, int dH_dtype, void* workspace, size_t workspace_bytes, cudaStream_t st,
-                         bool clear_status, const unsigned int* only_if_range = nullptr, const PartRoom* room = nullptr) {
+                         void* dH_d, int dH_dtype, void* workspace, size_t workspace_bytes, cudaStream_t st) {
     int rc = check_sizes(N, d, V, K);
     if (rc != HASS_OK) return rc;
     if (!H_d || !W || !topk_idx || !topk_q || !lse_d || !dH_d) return HASS_ERR_INVALID_ARG;
@@ -606,21 +655,21 @@ static int backward_impl(const void* H_d, const void* W, long long N, long long 
     int chunk_tiles = L.pref_chunk_tiles;
     if (fit < chunk_tiles) chunk_tiles = even_chunk(static_cast<int>(fit), RT);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
-    const PartRoom part = part_room(ws, workspace_bytes, L, chunk_tiles, room, true);
+    const PartRoom part = part_room(ws, workspace_bytes, L, chunk_tiles, nullptr, true);
     int* sidx = reinterpret_cast<int*>(ws + L.sidx);
     float* sgq = reinterpret_cast<float*>(ws + L.sgq);
     float* coef = reinterpret_cast<float*>(ws + L.coef);
     float* lse2 = reinterpret_cast<float*>(ws + L.lse2);
     __nv_bfloat16* P = reinterpret_cast<__nv_bfloat16*>(ws + L.scratch);
-    if (clear_status && cudaMemsetAsync(ws + L.status, 0, 256, st) != cudaSuccess) {
+    if (cudaMemsetAsync(ws + L.status, 0, 256, st) != cudaSuccess) {
         cudaGetLastError();
         return HASS_ERR_CUDA;
     }
 
     {
-        KernelTimer timer(only_if_range ? KIND_CONDITIONAL : KIND_PREP, st);
+        KernelTimer timer(KIND_PREP, st);
         bwd_prep_kernel<<<ceil_div(N, PREP_WARPS), PREP_WARPS * 32, 0, st>>>(static_cast<int>(N), K, topk_idx, topk_q, lse_d, grad_loss,
-                                                           sidx, sgq, coef, lse2, only_if_range);
+                                                           sidx, sgq, coef, lse2);
     }
     g_launches.fetch_add(1);
     if (cudaGetLastError() != cudaSuccess) return HASS_ERR_CUDA;
@@ -659,7 +708,6 @@ static int backward_impl(const void* H_d, const void* W, long long N, long long 
         p.P = P;
         p.p_pitch = L.p_pitch;
         p.status = reinterpret_cast<unsigned int*>(ws + L.status);
-        p.only_if_range = only_if_range;
         rc = launch_gemm<MODE_PROBS>(p, st);
         if (rc != HASS_OK) return rc;
         // (2) dH_d rows of this chunk = dz_d chunk x W
@@ -682,7 +730,6 @@ static int backward_impl(const void* H_d, const void* W, long long N, long long 
         o.out_align32 = ((reinterpret_cast<uintptr_t>(dH_d) | static_cast<uintptr_t>(d * (dH_dtype == HASS_FP32 ? 4 : 2))) & 31u) == 0 ? 1 : 0;
         o.out_pitch = d;
         o.status = p.status;
-        o.only_if_range = only_if_range;
         rc = launch_out(o, part, di.sms, st);
         if (rc != HASS_OK) return rc;
     }
@@ -734,15 +781,11 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
     if (fit < chunk_tiles) chunk_tiles = even_chunk(static_cast<int>(fit), RT);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     const PartRoom part = part_room(ws, workspace_bytes, L, chunk_tiles, room, false);
-    float* gq = bidir ? nullptr : reinterpret_cast<float*>(ws + L.sgq);    // [N, K]: too small for the 2K-token union
     float* coef = reinterpret_cast<float*>(ws + L.coef);
     float* sparse = reinterpret_cast<float*>(ws + L.sparse);
     __nv_bfloat16* P = reinterpret_cast<__nv_bfloat16*>(ws + L.scratch);
     unsigned int* status = reinterpret_cast<unsigned int*>(ws + L.status);
-    if (cudaMemsetAsync(status, 0, 256, st) != cudaSuccess) {
-        cudaGetLastError();
-        return HASS_ERR_CUDA;
-    }
+    int* idx_d = reinterpret_cast<int*>(ws + L.sidx);
     CUtensorMap tmHt, tmHd, tmWn, tmP;
     rc = make_tmap(&tmHd, H_d, N, d, d, BK, BM);
     if (rc == HASS_OK) rc = with_target ? make_tmap(&tmHt, H_t, N, d, d, BK, BM) : make_tmap(&tmHt, H_d, N, d, d, BK, BM);
@@ -761,7 +804,7 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
         return HASS_ERR_CUDA;
     }
     auto run = [&](bool retry) -> int {
-    const unsigned int* gate = retry ? status : nullptr;
+    const unsigned int* gate = retry ? status + 1 : nullptr;
     for (int t0 = 0; t0 < RT; t0 += chunk_tiles) {
         const int tiles = (RT - t0 < chunk_tiles) ? RT - t0 : chunk_tiles;
         const int rows = static_cast<int>((N - static_cast<long long>(t0) * BM < static_cast<long long>(tiles) * BM)
@@ -797,58 +840,59 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
         p.Pt = cmb ? cmb->Pt : nullptr;
         p.p_pitch = L.p_pitch;
         p.status = status;
-        p.thr_share = reinterpret_cast<float*>(ws + L.thr_share);
+        p.thr_share = reinterpret_cast<unsigned int*>(ws + L.thr_share);
         p.row_zmax = zmax + static_cast<size_t>(with_target ? 2 : 1) * t0 * BM;
         p.use_row_zmax = retry ? 1 : 0;
-        p.only_if_range = gate;
-    if (cudaMemsetAsync(p.thr_share, 0xff, static_cast<size_t>(p.sched.total_slots) * BM * 4, st) != cudaSuccess) {   // NaN
-        cudaGetLastError();
-        return HASS_ERR_CUDA;
-    }
-    rc = launch_gemm<MODE_STATS>(p, st);
+        p.gate = gate;
+        if (!retry || RT > chunk_tiles) {      // (a single chunk's thresholds hold for its second pass too)
+            rc = clear_status(ws, L, p.sched.total_slots, st, retry || t0 > 0);
+            if (rc != HASS_OK) return rc;
+        }
+        rc = launch_gemm<MODE_STATS>(p, st);
         if (rc != HASS_OK) return rc;
+        if (with_target) {
+            rc = launch_select(select_params(p, 0, t0 * BM, rows, idx_out, q_out, bidir ? 2 * K : K, lse_t), di.sms, st);
+            if (rc != HASS_OK) return rc;
+        }
+        if (bidir) {
+            // the draft's own K most probable tokens, in descending p
+            rc = launch_select(select_params(p, tiles, t0 * BM, rows, idx_d, reinterpret_cast<float*>(ws + L.sgq), K, nullptr),
+                               di.sms, st);
+            if (rc != HASS_OK) return rc;
+        }
         // (2) statistics -> loss, Omega_hat, per-row scale
         FinalizeParams f;
         std::memset(&f, 0, sizeof(f));
         f.sched = p.sched;
         f.d = static_cast<int>(d);
         f.K = K;
-        f.cap = topk_cap(K);
         f.row_begin = t0 * BM;
         f.rows = rows;
         f.row_tiles_t = with_target ? tiles : 0;
         f.part_m = p.part_m;
         f.part_s = p.part_s;
-        f.cand = p.cand;
-        f.cand_n = p.cand_n;
         f.H_d = static_cast<const __nv_bfloat16*>(H_d);
         f.W = static_cast<const __nv_bfloat16*>(W);
-        f.idx_in = idx_in;
-        f.q_in = q_in;
+        f.idx = with_target ? idx_out : const_cast<int*>(idx_in);
+        f.q = with_target ? q_out : const_cast<float*>(q_in);
+        f.idx_pitch = bidir ? 2 * K : K;
         f.loss = loss;
-        f.idx_out = idx_out;
-        f.q_out = q_out;
         f.lse_t = lse_t;
         f.lse_d = lse_d;
         f.grad_loss = grad_loss;
         f.coef_out = coef;
-        f.gq_out = gq;
         f.sparse_out = sparse;
         f.n_out = topk_n;
-        f.bidir = bidir ? 1 : 0;
+        f.idx_d = bidir ? idx_d : nullptr;
         f.H_t = static_cast<const __nv_bfloat16*>(H_t);
         f.w_topk = cmb ? cmb->w : 1.f;
         f.coef_t_out = cmb ? cmb->coef_t : nullptr;
         f.Pt = cmb ? cmb->Pt : nullptr;
         f.p_pitch = L.p_pitch;
         f.ce_corr_out = reinterpret_cast<float*>(ws + L.lse2);    // [N] floats, otherwise used by the split backward
-        f.only_if_range = gate;
-        {
-            KernelTimer timer(retry ? KIND_CONDITIONAL : KIND_FINALIZE, st);
-            finalize_kernel<<<ceil_div(rows, 8), 256, 0, st>>>(f);
-        }
-        g_launches.fetch_add(1);
-        if (cudaGetLastError() != cudaSuccess) return HASS_ERR_CUDA;
+        f.gate = gate;
+        rc = launch_finalize(f, st);
+        if (rc != HASS_OK) return rc;
         // (3) dH_d rows of the chunk
         GemmParams o;
         std::memset(&o, 0, sizeof(o));
@@ -873,7 +917,7 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
             t.out_align32 = 1;
             t.out_pitch = d;
             t.status = status;
-            t.only_if_range = gate;
+            t.gate = gate;
             rc = launch_out(t, part, di.sms, st);
             if (rc != HASS_OK) return rc;
             {
@@ -905,7 +949,7 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
         o.out_align32 = ((reinterpret_cast<uintptr_t>(dH_d) | static_cast<uintptr_t>(d * (dH_dtype == HASS_FP32 ? 4 : 2))) & 31u) == 0 ? 1 : 0;
         o.out_pitch = d;
         o.status = status;
-        o.only_if_range = gate;
+        o.gate = gate;
         rc = launch_out(o, part, di.sms, st);
         if (rc != HASS_OK) return rc;
     }
@@ -913,21 +957,13 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
     };
     rc = run(false);
     if (rc != HASS_OK) return rc;
-    rc = run(true);
-    if (rc != HASS_OK) return rc;
-    {
-        KernelTimer timer(KIND_CONDITIONAL, st);
-        range_handled_kernel<<<1, 1, 0, st>>>(status);
-    }
-    g_launches.fetch_add(1);
-    if (cudaGetLastError() != cudaSuccess) return HASS_ERR_CUDA;
-    return HASS_OK;
+    return run(true);
 }
 
 // ---- fused forward + backward, Omega_hat known before the draft rows are swept -------------------------
 // The route of hass_topk_distill_fwd_bwd, its _draft form and the Top-P variant. Per chunk of row tiles:
 // (1) sweep of the chunk's TARGET rows: statistics and Top-K candidates; (2) select_kernel: lse_t, Omega_hat,
-// and the same set sorted by token id; (3) sweep of the chunk's DRAFT rows: statistics, the bf16 spill of
+// the same set sorted by token id, and ref2; (3) sweep of the chunk's DRAFT rows: statistics, the bf16 spill of
 // 2^(z_d log2e - ref2), and z_d at the row's Omega_hat copied out of the accumulator as the sweep passes those
 // columns; (4) loss_patch_kernel: lse_d, Eq. 1, the per-row scale, and the Omega_hat term of dz_d subtracted
 // from the K spilled entries it concerns; (5) the second GEMM with the row scale in its epilogue. No logit
@@ -979,12 +1015,10 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
     float* sq = reinterpret_cast<float*>(ws + L.sgq);
     float* coef = reinterpret_cast<float*>(ws + L.coef);
     float* capz = reinterpret_cast<float*>(ws + L.capz);
+    float* ref2 = reinterpret_cast<float*>(ws + L.lse2);
     __nv_bfloat16* P = reinterpret_cast<__nv_bfloat16*>(ws + L.scratch);
     unsigned int* status = reinterpret_cast<unsigned int*>(ws + L.status);
-    if (cudaMemsetAsync(status, 0, 256, st) != cudaSuccess) {
-        cudaGetLastError();
-        return HASS_ERR_CUDA;
-    }
+    unsigned int* zmax = reinterpret_cast<unsigned int*>(ws + L.zmax);
     CUtensorMap tmHt, tmHd, tmWn, tmP;
     rc = make_tmap(&tmHd, H_d, N, d, d, BK, BM);
     if (rc == HASS_OK) rc = with_target ? make_tmap(&tmHt, H_t, N, d, d, BK, BM) : make_tmap(&tmHt, H_d, N, d, d, BK, BM);
@@ -995,196 +1029,183 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
     if (rc == HASS_OK) rc = make_tmap(&tmPst, P, static_cast<long long>(chunk_tiles) * BM, L.p_pitch, L.p_pitch, 64, 32);
     if (rc != HASS_OK) return rc;
 
-    for (int t0 = 0; t0 < RT; t0 += chunk_tiles) {
-        const int tiles = (RT - t0 < chunk_tiles) ? RT - t0 : chunk_tiles;
-        const int rows = static_cast<int>((N - static_cast<long long>(t0) * BM < static_cast<long long>(tiles) * BM)
-                                              ? N - static_cast<long long>(t0) * BM
-                                              : static_cast<long long>(tiles) * BM);
-        // both sweeps cover `tiles` row tiles and share one schedule
-        GemmParams p;
-        std::memset(&p, 0, sizeof(p));
-        rc = plan_launch(tiles, CT, di.sms, L.slot_cap, &p.sched);
-        if (rc != HASS_OK) return rc;
-        log_schedule("fused sweep (target / draft)", p.sched);
-        rc = make_tmap(&p.tmB, W, V, d, d, BK, BN / p.sched.pair);      // B of z = H W^T: K-major
-        if (rc != HASS_OK) return rc;
-        p.row_tiles = tiles;
-        p.row_tiles0 = tiles;
-        p.a_row_offset = t0 * BM;
-        p.row_global_offset = t0 * BM;
-        p.rows_valid = static_cast<int>(N);
-        p.n_cols = static_cast<int>(V);
-        p.col_tiles = CT;
-        p.k_blocks = ceil_div(d, BK);
-        p.K = K;
-        p.cap = topk_cap(K);
-        p.part_m = reinterpret_cast<float*>(ws + L.part_m);
-        p.part_s = reinterpret_cast<float*>(ws + L.part_s);
-        p.cand = reinterpret_cast<uint2*>(ws + L.cand_v);
-        p.cand_n = reinterpret_cast<int*>(ws + L.cand_i);
-        p.p_pitch = L.p_pitch;
-        p.status = status;
-        cudaEvent_t ev_d = nullptr;
-        if (pipe) {
-            // this chunk's rows of H_t, then of H_d, on the inbound copy stream; the sweeps wait for them
-            const size_t off = static_cast<size_t>(t0) * BM * pipe->in_row_bytes, bytes = static_cast<size_t>(rows) * pipe->in_row_bytes;
-            cudaEvent_t ev_t = pipe->next();
-            ev_d = pipe->next();
-            if (!ev_t || !ev_d) return HASS_ERR_UNSUPPORTED;
-            bool ok = cudaMemcpyAsync(const_cast<uint8_t*>(static_cast<const uint8_t*>(H_t)) + off, pipe->Ht_host + off, bytes,
-                                      cudaMemcpyHostToDevice, pipe->h2d) == cudaSuccess;
-            ok = ok && cudaEventRecord(ev_t, pipe->h2d) == cudaSuccess;
-            ok = ok && cudaMemcpyAsync(const_cast<uint8_t*>(static_cast<const uint8_t*>(H_d)) + off, pipe->Hd_host + off, bytes,
-                                       cudaMemcpyHostToDevice, pipe->h2d) == cudaSuccess;
-            ok = ok && cudaEventRecord(ev_d, pipe->h2d) == cudaSuccess;
-            ok = ok && cudaStreamWaitEvent(st, ev_t, 0) == cudaSuccess;
-            if (!ok) {
-                cudaGetLastError();
-                return HASS_ERR_CUDA;
-            }
-        }
-        if (with_target) {
-            // (1) target rows: statistics + candidates
-            GemmParams t = p;
-            t.tmA0 = tmHt;
-            t.tmA1 = tmHt;
-            t.topk_row_tiles = tiles;
-            t.spill_begin = INT_MAX;
-            t.thr_share = reinterpret_cast<float*>(ws + L.thr_share);
-            if (cudaMemsetAsync(t.thr_share, 0xff, static_cast<size_t>(t.sched.total_slots) * BM * 4, st) != cudaSuccess) {   // NaN
-                cudaGetLastError();
-                return HASS_ERR_CUDA;
-            }
-            rc = launch_gemm<MODE_STATS>(t, st);
+    // Every spilling row records its largest logit. If a draft sweep reports a row beyond the exponent range of its spill,
+    // the steps from the draft sweep on run a second time as conditional launches with each row's exponent taken from that
+    // record, which no logit of the row can exceed.
+    auto run = [&](bool retry) -> int {
+        const unsigned int* gate = retry ? status + 1 : nullptr;
+        for (int t0 = 0; t0 < RT; t0 += chunk_tiles) {
+            const int tiles = (RT - t0 < chunk_tiles) ? RT - t0 : chunk_tiles;
+            const int rows = static_cast<int>((N - static_cast<long long>(t0) * BM < static_cast<long long>(tiles) * BM)
+                                                  ? N - static_cast<long long>(t0) * BM
+                                                  : static_cast<long long>(tiles) * BM);
+            // both sweeps cover `tiles` row tiles and share one schedule
+            GemmParams p;
+            std::memset(&p, 0, sizeof(p));
+            rc = plan_launch(tiles, CT, di.sms, L.slot_cap, &p.sched);
             if (rc != HASS_OK) return rc;
-        }
-        // (2) Omega_hat of the chunk's rows
-        SelectParams sp;
-        std::memset(&sp, 0, sizeof(sp));
-        sp.sched = p.sched;
-        sp.K = K;
-        sp.cap = p.cap;
-        sp.row_begin = t0 * BM;
-        sp.rows = rows;
-        sp.from_sweep = with_target ? 1 : 0;
-        sp.part_m = p.part_m;
-        sp.part_s = p.part_s;
-        sp.cand = p.cand;
-        sp.cand_n = p.cand_n;
-        sp.idx_in = idx_in;
-        sp.q_in = q_in;
-        sp.idx_out = idx_out;
-        sp.q_out = q_out;
-        sp.lse_t = lse_t;
-        sp.n_out = topk_n;
-        sp.top_p = top_p;
-        sp.sidx = sidx;
-        sp.sq = sq;
-        {
-            KernelTimer timer(KIND_FINALIZE, st);
-            select_kernel<<<ceil_div(rows, SEL_WARPS), SEL_WARPS * 32, 0, st>>>(sp);
-        }
-        g_launches.fetch_add(1);
-        if (cudaGetLastError() != cudaSuccess) return HASS_ERR_CUDA;
-        // (3) draft rows: statistics, spill, z_d at Omega_hat
-        if (pipe && cudaStreamWaitEvent(st, ev_d, 0) != cudaSuccess) {
-            cudaGetLastError();
-            return HASS_ERR_CUDA;
-        }
-        {
-            GemmParams q = p;
-            q.tmA0 = tmHd;
-            q.tmA1 = tmHd;
-            q.topk_row_tiles = 0;
-            q.spill_begin = 0;
-            q.sidx = sidx;
-            q.cap_z = capz;
-            q.P = P;
-            q.tmSpill = tmPst;
-            rc = launch_gemm<MODE_STATS>(q, st, KIND_STATS_DRAFT);
+            log_schedule("fused sweep (target / draft)", p.sched);
+            rc = make_tmap(&p.tmB, W, V, d, d, BK, BN / p.sched.pair);      // B of z = H W^T: K-major
             if (rc != HASS_OK) return rc;
-        }
-        // (4) lse_d, loss, row scale, Omega_hat term into the spill
-        LossPatchParams lp;
-        std::memset(&lp, 0, sizeof(lp));
-        lp.sched = p.sched;
-        lp.K = K;
-        lp.row_begin = t0 * BM;
-        lp.rows = rows;
-        lp.part_m = p.part_m;
-        lp.part_s = p.part_s;
-        lp.sidx = sidx;
-        lp.sq = sq;
-        lp.cap_z = capz;
-        lp.grad_loss = grad_loss;
-        lp.loss = loss;
-        lp.lse_d = lse_d;
-        lp.coef_out = coef;
-        lp.P = P;
-        lp.p_pitch = L.p_pitch;
-        {
-            KernelTimer timer(KIND_FINALIZE, st);
-            loss_patch_kernel<<<ceil_div(rows, 8), 256, 0, st>>>(lp);
-        }
-        g_launches.fetch_add(1);
-        if (cudaGetLastError() != cudaSuccess) return HASS_ERR_CUDA;
-        // (5) dH_d rows of the chunk = row scale x (patched spill x W)
-        GemmParams o;
-        std::memset(&o, 0, sizeof(o));
-        o.tmA0 = tmP;
-        o.tmA1 = tmP;
-        o.tmB = tmWn;
-        o.row_tiles = tiles;
-        o.row_tiles0 = tiles;
-        o.spill_begin = INT_MAX;
-        o.a_row_offset = 0;
-        o.row_global_offset = t0 * BM;
-        o.rows_valid = static_cast<int>(N);
-        o.n_cols = static_cast<int>(d);
-        o.col_tiles = DT;
-        o.k_blocks = ceil_div(V, BK);
-        o.K = K;
-        o.coef = coef;
-        o.out = dH_d;
-        o.out_fp32 = dH_dtype == HASS_FP32 ? 1 : 0;
-        o.out_align32 = ((reinterpret_cast<uintptr_t>(dH_d) | static_cast<uintptr_t>(d * (dH_dtype == HASS_FP32 ? 4 : 2))) & 31u) == 0 ? 1 : 0;
-        o.out_pitch = d;
-        o.status = status;
-        rc = launch_out(o, part, di.sms, st);
-        if (rc != HASS_OK) return rc;
-        if (pipe) {
-            // the chunk's dH_d rows on the outbound copy stream
-            const size_t off = static_cast<size_t>(t0) * BM * pipe->out_row_bytes, bytes = static_cast<size_t>(rows) * pipe->out_row_bytes;
-            cudaEvent_t ev_o = pipe->next();
-            if (!ev_o) return HASS_ERR_UNSUPPORTED;
-            bool ok = cudaEventRecord(ev_o, st) == cudaSuccess;
-            ok = ok && cudaStreamWaitEvent(pipe->d2h, ev_o, 0) == cudaSuccess;
-            ok = ok && cudaMemcpyAsync(pipe->dH_host + off, static_cast<const uint8_t*>(dH_d) + off, bytes, cudaMemcpyDeviceToHost,
-                                       pipe->d2h) == cudaSuccess;
-            if (!ok) {
-                cudaGetLastError();
-                return HASS_ERR_CUDA;
+            p.row_tiles = tiles;
+            p.row_tiles0 = tiles;
+            p.a_row_offset = t0 * BM;
+            p.row_global_offset = t0 * BM;
+            p.rows_valid = static_cast<int>(N);
+            p.n_cols = static_cast<int>(V);
+            p.col_tiles = CT;
+            p.k_blocks = ceil_div(d, BK);
+            p.K = K;
+            p.cap = topk_cap(K);
+            p.part_m = reinterpret_cast<float*>(ws + L.part_m);
+            p.part_s = reinterpret_cast<float*>(ws + L.part_s);
+            p.cand = reinterpret_cast<uint2*>(ws + L.cand_v);
+            p.cand_n = reinterpret_cast<int*>(ws + L.cand_i);
+            p.thr_share = reinterpret_cast<unsigned int*>(ws + L.thr_share);
+            p.p_pitch = L.p_pitch;
+            p.status = status;
+            p.gate = gate;
+            if (!retry) {
+                cudaEvent_t ev_d = nullptr;
+                if (pipe) {
+                    // this chunk's rows of H_t, then of H_d, on the inbound copy stream; the sweeps wait for them
+                    const size_t off = static_cast<size_t>(t0) * BM * pipe->in_row_bytes, bytes = static_cast<size_t>(rows) * pipe->in_row_bytes;
+                    cudaEvent_t ev_t = pipe->next();
+                    ev_d = pipe->next();
+                    if (!ev_t || !ev_d) return HASS_ERR_UNSUPPORTED;
+                    bool ok = cudaMemcpyAsync(const_cast<uint8_t*>(static_cast<const uint8_t*>(H_t)) + off, pipe->Ht_host + off, bytes,
+                                              cudaMemcpyHostToDevice, pipe->h2d) == cudaSuccess;
+                    ok = ok && cudaEventRecord(ev_t, pipe->h2d) == cudaSuccess;
+                    ok = ok && cudaMemcpyAsync(const_cast<uint8_t*>(static_cast<const uint8_t*>(H_d)) + off, pipe->Hd_host + off, bytes,
+                                               cudaMemcpyHostToDevice, pipe->h2d) == cudaSuccess;
+                    ok = ok && cudaEventRecord(ev_d, pipe->h2d) == cudaSuccess;
+                    ok = ok && cudaStreamWaitEvent(st, ev_t, 0) == cudaSuccess;
+                    if (!ok) {
+                        cudaGetLastError();
+                        return HASS_ERR_CUDA;
+                    }
+                }
+                rc = clear_status(ws, L, with_target ? p.sched.total_slots : 0, st, t0 > 0);
+                if (rc != HASS_OK) return rc;
+                if (with_target) {
+                    // (1) target rows: statistics + candidates
+                    GemmParams t = p;
+                    t.tmA0 = tmHt;
+                    t.tmA1 = tmHt;
+                    t.topk_row_tiles = tiles;
+                    t.spill_begin = INT_MAX;
+                    rc = launch_gemm<MODE_STATS>(t, st);
+                    if (rc != HASS_OK) return rc;
+                }
+                // (2) Omega_hat of the chunk's rows, and the reference exponent of their spill (reads H_d)
+                if (pipe && cudaStreamWaitEvent(st, ev_d, 0) != cudaSuccess) {
+                    cudaGetLastError();
+                    return HASS_ERR_CUDA;
+                }
+                SelectParams sp = select_params(p, 0, t0 * BM, rows, idx_out, q_out, K, lse_t);
+                sp.from_sweep = with_target ? 1 : 0;
+                sp.idx_in = idx_in;
+                sp.q_in = q_in;
+                sp.n_out = topk_n;
+                sp.top_p = top_p;
+                sp.sidx = sidx;
+                sp.sq = sq;
+                sp.H_d = static_cast<const __nv_bfloat16*>(H_d);
+                sp.W = static_cast<const __nv_bfloat16*>(W);
+                sp.d = static_cast<int>(d);
+                sp.V = static_cast<int>(V);
+                sp.ref2 = ref2;
+                sp.zmax = zmax + static_cast<size_t>(t0) * BM;
+                rc = launch_select(sp, di.sms, st);
+                if (rc != HASS_OK) return rc;
+            }
+            // (3) draft rows: statistics, spill, z_d at Omega_hat
+            {
+                GemmParams q = p;
+                q.tmA0 = tmHd;
+                q.tmA1 = tmHd;
+                q.topk_row_tiles = 0;
+                q.spill_begin = 0;
+                q.sidx = sidx;
+                q.cap_z = capz;
+                q.row_ref2 = ref2;
+                q.row_zmax = zmax + static_cast<size_t>(t0) * BM;
+                q.use_row_zmax = retry ? 1 : 0;
+                q.P = P;
+                q.tmSpill = tmPst;
+                rc = launch_gemm<MODE_STATS>(q, st, KIND_STATS_DRAFT);
+                if (rc != HASS_OK) return rc;
+            }
+            // (4) lse_d, loss, row scale, Omega_hat term into the spill
+            LossPatchParams lp;
+            std::memset(&lp, 0, sizeof(lp));
+            lp.sched = p.sched;
+            lp.K = K;
+            lp.row_begin = t0 * BM;
+            lp.rows = rows;
+            lp.part_m = p.part_m;
+            lp.part_s = p.part_s;
+            lp.sidx = sidx;
+            lp.sq = sq;
+            lp.cap_z = capz;
+            lp.grad_loss = grad_loss;
+            lp.loss = loss;
+            lp.lse_d = lse_d;
+            lp.coef_out = coef;
+            lp.P = P;
+            lp.p_pitch = L.p_pitch;
+            lp.gate = gate;
+            {
+                KernelTimer timer(retry ? KIND_CONDITIONAL : KIND_FINALIZE, st);
+                loss_patch_kernel<<<ceil_div(rows, 8), 256, 0, st>>>(lp);
+            }
+            g_launches.fetch_add(1);
+            if (cudaGetLastError() != cudaSuccess) return HASS_ERR_CUDA;
+            // (5) dH_d rows of the chunk = row scale x (patched spill x W)
+            GemmParams o;
+            std::memset(&o, 0, sizeof(o));
+            o.tmA0 = tmP;
+            o.tmA1 = tmP;
+            o.tmB = tmWn;
+            o.row_tiles = tiles;
+            o.row_tiles0 = tiles;
+            o.spill_begin = INT_MAX;
+            o.a_row_offset = 0;
+            o.row_global_offset = t0 * BM;
+            o.rows_valid = static_cast<int>(N);
+            o.n_cols = static_cast<int>(d);
+            o.col_tiles = DT;
+            o.k_blocks = ceil_div(V, BK);
+            o.K = K;
+            o.coef = coef;
+            o.out = dH_d;
+            o.out_fp32 = dH_dtype == HASS_FP32 ? 1 : 0;
+            o.out_align32 = ((reinterpret_cast<uintptr_t>(dH_d) | static_cast<uintptr_t>(d * (dH_dtype == HASS_FP32 ? 4 : 2))) & 31u) == 0 ? 1 : 0;
+            o.out_pitch = d;
+            o.status = status;
+            o.gate = gate;
+            rc = launch_out(o, part, di.sms, st);
+            if (rc != HASS_OK) return rc;
+            if (pipe && !retry) {
+                // the chunk's dH_d rows on the outbound copy stream
+                const size_t off = static_cast<size_t>(t0) * BM * pipe->out_row_bytes, bytes = static_cast<size_t>(rows) * pipe->out_row_bytes;
+                cudaEvent_t ev_o = pipe->next();
+                if (!ev_o) return HASS_ERR_UNSUPPORTED;
+                bool ok = cudaEventRecord(ev_o, st) == cudaSuccess;
+                ok = ok && cudaStreamWaitEvent(pipe->d2h, ev_o, 0) == cudaSuccess;
+                ok = ok && cudaMemcpyAsync(pipe->dH_host + off, static_cast<const uint8_t*>(dH_d) + off, bytes, cudaMemcpyDeviceToHost,
+                                           pipe->d2h) == cudaSuccess;
+                if (!ok) {
+                    cudaGetLastError();
+                    return HASS_ERR_CUDA;
+                }
             }
         }
-    }
-    {
-        // Exact route, enqueued behind every call of this route: if a sweep reported a row beyond its exponent
-        // range, the separate forward and the recomputing backward (which have no such limit) redo the call
-        // and the report is withdrawn; otherwise each of these launches returns at once.
-        rc = forward_impl(with_target, H_t, H_d, W, N, d, V, K, idx_in, q_in, loss, idx_out, q_out, lse_t, lse_d,
-                          workspace, workspace_bytes, st, status, top_p, topk_n);
-        if (rc != HASS_OK) return rc;
-        rc = backward_impl(H_d, W, N, d, V, K, with_target ? idx_out : idx_in, with_target ? q_out : q_in, lse_d,
-                           grad_loss, dH_d, dH_dtype, workspace, workspace_bytes, st, false, status, room);
-        if (rc != HASS_OK) return rc;
-        {
-            KernelTimer timer(KIND_CONDITIONAL, st);
-            range_handled_kernel<<<1, 1, 0, st>>>(status);
-        }
-        g_launches.fetch_add(1);
-        if (cudaGetLastError() != cudaSuccess) return HASS_ERR_CUDA;
-    }
-    return HASS_OK;
+        return HASS_OK;
+    };
+    rc = run(false);
+    if (rc != HASS_OK) return rc;
+    return run(true);
 }
 
 // ---- forward alone, Omega_hat known before the draft rows are swept -----------------------------------
@@ -1216,10 +1237,6 @@ static int forward2_impl(bool with_target, const void* H_t, const void* H_d, con
                             workspace, workspace_bytes, st);
     const int RT = ceil_div(N, BM), CT = ceil_div(V, BN);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
-    if (cudaMemsetAsync(ws + L.status, 0, 256, st) != cudaSuccess) {
-        cudaGetLastError();
-        return HASS_ERR_CUDA;
-    }
     GemmParams p;
     std::memset(&p, 0, sizeof(p));
     rc = plan_launch(RT, CT, di.sms, L.slot_cap, &p.sched);
@@ -1244,45 +1261,26 @@ static int forward2_impl(bool with_target, const void* H_t, const void* H_d, con
     int* sidx = reinterpret_cast<int*>(ws + L.sidx);
     float* sq = reinterpret_cast<float*>(ws + L.sgq);
     float* capz = reinterpret_cast<float*>(ws + L.capz);
+    p.thr_share = reinterpret_cast<unsigned int*>(ws + L.thr_share);
+    rc = clear_status(ws, L, with_target ? p.sched.total_slots : 0, st);
+    if (rc != HASS_OK) return rc;
     if (with_target) {
         GemmParams t = p;
         rc = make_tmap(&t.tmA0, H_t, N, d, d, BK, BM);
         if (rc != HASS_OK) return rc;
         t.tmA1 = t.tmA0;
         t.topk_row_tiles = RT;
-        t.thr_share = reinterpret_cast<float*>(ws + L.thr_share);
-        if (cudaMemsetAsync(t.thr_share, 0xff, static_cast<size_t>(t.sched.total_slots) * BM * 4, st) != cudaSuccess) {   // NaN
-            cudaGetLastError();
-            return HASS_ERR_CUDA;
-        }
         rc = launch_gemm<MODE_STATS>(t, st);
         if (rc != HASS_OK) return rc;
     }
-    SelectParams sp;
-    std::memset(&sp, 0, sizeof(sp));
-    sp.sched = p.sched;
-    sp.K = K;
-    sp.cap = p.cap;
-    sp.row_begin = 0;
-    sp.rows = static_cast<int>(N);
+    SelectParams sp = select_params(p, 0, 0, static_cast<int>(N), idx_out, q_out, K, lse_t);
     sp.from_sweep = with_target ? 1 : 0;
-    sp.part_m = p.part_m;
-    sp.part_s = p.part_s;
-    sp.cand = p.cand;
-    sp.cand_n = p.cand_n;
     sp.idx_in = idx_in;
     sp.q_in = q_in;
-    sp.idx_out = idx_out;
-    sp.q_out = q_out;
-    sp.lse_t = lse_t;
     sp.sidx = sidx;
     sp.sq = sq;
-    {
-        KernelTimer timer(KIND_FINALIZE, st);
-        select_kernel<<<ceil_div(N, SEL_WARPS), SEL_WARPS * 32, 0, st>>>(sp);
-    }
-    g_launches.fetch_add(1);
-    if (cudaGetLastError() != cudaSuccess) return HASS_ERR_CUDA;
+    rc = launch_select(sp, di.sms, st);
+    if (rc != HASS_OK) return rc;
     {
         GemmParams q = p;
         rc = make_tmap(&q.tmA0, H_d, N, d, d, BK, BM);
@@ -1339,10 +1337,6 @@ static int normed_impl(const void* H_t, const void* H_d, const void* W, long lon
     if (workspace_bytes < L.fwd_end) return HASS_ERR_WORKSPACE;
     const int RT = ceil_div(N, BM), CT = ceil_div(V, BN);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
-    if (cudaMemsetAsync(ws + L.status, 0, 256, st) != cudaSuccess) {
-        cudaGetLastError();
-        return HASS_ERR_CUDA;
-    }
     GemmParams p;
     std::memset(&p, 0, sizeof(p));
     rc = plan_launch(RT, CT, di.sms, L.slot_cap, &p.sched);
@@ -1367,43 +1361,37 @@ static int normed_impl(const void* H_t, const void* H_d, const void* W, long lon
     p.cand = reinterpret_cast<uint2*>(ws + L.cand_v);
     p.cand_n = reinterpret_cast<int*>(ws + L.cand_i);
     p.status = reinterpret_cast<unsigned int*>(ws + L.status);
-    p.thr_share = reinterpret_cast<float*>(ws + L.thr_share);
-    if (cudaMemsetAsync(p.thr_share, 0xff, static_cast<size_t>(p.sched.total_slots) * BM * 4, st) != cudaSuccess) {   // NaN
-        cudaGetLastError();
-        return HASS_ERR_CUDA;
-    }
+    p.thr_share = reinterpret_cast<unsigned int*>(ws + L.thr_share);
+    rc = clear_status(ws, L, p.sched.total_slots, st);
+    if (rc != HASS_OK) return rc;
     rc = launch_gemm<MODE_STATS>(p, st);
+    if (rc != HASS_OK) return rc;
+    SelectParams sp = select_params(p, 0, 0, static_cast<int>(N), idx_out, q_out, K, lse_t);
+    sp.n_out = topk_n;
+    rc = launch_select(sp, di.sms, st);
     if (rc != HASS_OK) return rc;
     FinalizeParams f;
     std::memset(&f, 0, sizeof(f));
     f.sched = p.sched;
     f.d = static_cast<int>(d);
     f.K = K;
-    f.cap = p.cap;
     f.row_begin = 0;
     f.rows = static_cast<int>(N);
     f.row_tiles_t = RT;
     f.part_m = p.part_m;
     f.part_s = p.part_s;
-    f.cand = p.cand;
-    f.cand_n = p.cand_n;
     f.H_d = static_cast<const __nv_bfloat16*>(H_d);
     f.W = static_cast<const __nv_bfloat16*>(W);
     f.loss = loss;
-    f.idx_out = idx_out;
-    f.q_out = q_out;
+    f.idx = idx_out;
+    f.q = q_out;
+    f.idx_pitch = K;
     f.lse_t = lse_t;
     f.grad_loss = grad_loss;
-    f.n_out = topk_n;
     f.normed = 1;
     f.dH_out = dH_d;
     f.dH_fp32 = dH_dtype == HASS_FP32 ? 1 : 0;
-    {
-        KernelTimer timer(KIND_FINALIZE, st);
-        finalize_kernel<<<ceil_div(N, 8), 256, 0, st>>>(f);
-    }
-    g_launches.fetch_add(1);
-    return cudaGetLastError() == cudaSuccess ? HASS_OK : HASS_ERR_CUDA;
+    return launch_finalize(f, st);
 }
 
 }  // namespace hass
@@ -1498,7 +1486,7 @@ int hass_topk_distill_bwd(const void* H_d, const void* W, int64_t N, int64_t d, 
                           const int32_t* topk_idx, const float* topk_q, const float* lse_d, const float* grad_loss,
                           void* dH_d, int dH_dtype, void* workspace, size_t workspace_bytes, void* cuda_stream) {
     return backward_impl(H_d, W, N, d, V, K, topk_idx, topk_q, lse_d, grad_loss, dH_d, dH_dtype, workspace,
-                         workspace_bytes, static_cast<cudaStream_t>(cuda_stream), true);
+                         workspace_bytes, static_cast<cudaStream_t>(cuda_stream));
 }
 
 int hass_topk_distill_fwd_bwd(const void* H_t, const void* H_d, const void* W, int64_t N, int64_t d, int64_t V,
@@ -1767,9 +1755,9 @@ int hass_topk_distill_fwd_bwd_host(const void* H_t_host, const void* H_d_host, c
         cudaGetLastError();
         return HASS_ERR_CUDA;
     }
-    // word 2 of the status block: the exact route ran after the chunks' dH_d rows had left; fetch them again
+    // word 1 of the status block: the second pass ran after the chunks' dH_d rows had left; fetch them again
     unsigned int redo = 0;
-    ok = cudaMemcpyAsync(&redo, ws + 8, 4, cudaMemcpyDeviceToHost, st) == cudaSuccess;
+    ok = cudaMemcpyAsync(&redo, ws + 4, 4, cudaMemcpyDeviceToHost, st) == cudaSuccess;
     rc = hass_check(workspace, cuda_stream);
     cudaStreamSynchronize(pipe.d2h);
     if (rc != HASS_OK) return rc;
@@ -2082,7 +2070,7 @@ int hass_check(void* workspace, void* cuda_stream) {
     if (word != 0) {
         cudaMemset(workspace, 0, 4);
         if (kLog) std::fprintf(stderr, "[hass] device status word 0x%x\n", word);
-        return (word & 0xffu) == 2u ? HASS_ERR_RANGE : HASS_ERR_TIMEOUT;
+        return HASS_ERR_TIMEOUT;
     }
     return HASS_OK;
 }

@@ -9,12 +9,12 @@
 //               (the separate, recomputing backward)
 //   MODE_OUT    dH_d tile: coef * acc - Omega_hat row (fused), coef * acc (q W of the combined objective)
 //               or the accumulator as is (separate backward)
-// plus small kernels: select (between the sweep of the target rows and the sweep of the draft rows: lse_t,
-// Omega_hat, the set sorted by token id), loss_patch (after the draft sweep: lse_d, Eq. 1, row scale, the
-// Omega_hat term into the spill), finalize (the single-sweep route: merge partial statistics, pick Omega_hat,
-// Eq. 1 and its variants, the Omega_hat term of dH_d), ce_kernel (cross-entropy of the combined objective),
-// bwd_prep (index-sorted Top-K lists for MODE_PROBS) and range_handled_kernel.
-// Beside the four operand stages the kernel's shared memory holds 32 KB that the epilogue warps use: staging
+// plus small kernels: out_reduce (partial tiles of MODE_OUT), select (after a sweep with Top-K candidates: lse,
+// Omega_hat, the set sorted by token id, the reference exponent of the draft rows' spill), loss_patch (after the draft
+// sweep: lse_d, Eq. 1, row scale, the Omega_hat term into the spill), finalize (routes without a draft sweep that
+// knows Omega_hat: gathered draft logits, Eq. 1 and its variants, the Omega_hat term of dH_d), ce_kernel (cross-entropy
+// of the combined objective) and bwd_prep (index-sorted Top-K lists for MODE_PROBS).
+// Beside the operand stages the kernel's shared memory holds 32 KB that the epilogue warps use: staging
 // buffers for the TMA stores of the spill (draft sweep) or the logits waiting for admission to the register
 // Top-K lists (target sweep).
 #pragma once
@@ -95,13 +95,14 @@ struct GemmParams {
     int cap;               // capacity of a (row, slot) candidate buffer: cand_cap(K)
     int spill_begin;       // MODE_STATS: row tiles >= spill_begin also write the tile 2^(z log2e - ref2) in bf16 to
                            // P (row tile index - spill_begin); INT_MAX: none
+    const float* row_ref2; // MODE_STATS, spilling rows: [N] reference exponents, or nullptr: from column tile 0
     // MODE_STATS outputs (per slot)
     float* part_m;
     float* part_s;
     uint2* cand;           // [slot, row, cap] (logit bits, token id)
     int* cand_n;           // [slot, row] entries in use
-    float* thr_share;      // [slot, row] each lane's current threshold, read by the other lanes of its row tile
-                           // (initialised to NaN = "nothing published"; nullptr: no sharing)
+    unsigned int* thr_share;   // [slot, row] ordered key of each lane's current threshold, read by the other lanes of its row
+                           // tile (zeroed before the sweep: nothing published)
     // MODE_PROBS
     const float* lse2;     // [N] lse_d * log2(e)
     const float* coef;     // [N] g * S_q
@@ -123,11 +124,10 @@ struct GemmParams {
     unsigned int* status;
     OutPlan plan;
     float* part;           // [cuts][rest][pair][part_rows][BN] partial tiles
-    const unsigned int* only_if_range;   // nullptr, or: run only if this status word reports a range overflow
-    // The single-sweep route (spilling sweeps with Top-K lists): every spilling row leaves the ordered key of its
-    // largest logit in row_zmax[row tile * 128 + row] (atomicMax over the lanes of the row tile; zeroed by the
-    // host). A second sweep with use_row_zmax = 1 takes the row's fixed exponent from there instead of from
-    // column tile 0, so that no logit of the row can exceed it.
+    const unsigned int* gate;            // nullptr, or: run only if this word (the range report, status[1]) is not zero
+    // Every spilling row leaves the ordered key of its largest logit in row_zmax[row tile * 128 + row] (atomicMax over the
+    // lanes of the row tile; zeroed before the sweep). A second sweep with use_row_zmax = 1 takes the row's fixed exponent
+    // from there, so that no logit of the row can exceed it.
     unsigned int* row_zmax;              // nullable
     int use_row_zmax;
 };
@@ -255,6 +255,23 @@ __device__ __forceinline__ uint32_t compact_candidates(uint2* buf, int n, int K,
     return key_bits(T);
 }
 
+// Bitonic sorting network over 16 registers.
+__device__ __forceinline__ void sort16_descending(float (&v)[16]) {
+#pragma unroll
+    for (int k = 2; k <= 16; k *= 2)
+#pragma unroll
+        for (int j = k / 2; j > 0; j /= 2)
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const int l = i ^ j;
+                if (l > i) {
+                    const float hi = fmaxf(v[i], v[l]), lo = fminf(v[i], v[l]);
+                    v[i] = (i & k) == 0 ? hi : lo;
+                    v[l] = (i & k) == 0 ? lo : hi;
+                }
+            }
+}
+
 // TOPK selects how MODE_STATS keeps a row's Top-K candidates: TOPK_REG (K <= K_REG) a sorted list in
 // registers, all lanes inserting in parallel - best while most rows still admit logits; TOPK_BUF (any K)
 // append buffers with warp-cooperative compaction - cost nearly independent of K; TOPK_NONE: a sweep of draft
@@ -272,9 +289,9 @@ constexpr int K_REG = 16;
 template <int MODE, int TOPK, int CG>
 __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_constant__ GemmParams p) {
     constexpr bool B_MN_MAJOR = (MODE == MODE_OUT);
-    // conditional launch (the exact route that follows a fused call): nothing to do unless the fused sweep
-    // reported a row beyond its exponent range
-    if (p.only_if_range != nullptr && ((*p.only_if_range) & 0xffu) != 2u) return;
+    // conditional launch (the second pass that follows every spilling call): nothing to do unless the first reported a
+    // row beyond its exponent range
+    if (p.gate != nullptr && *p.gate == 0u) return;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t smemA = smem_base;
@@ -357,9 +374,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
             }
         }
     };
-    // a lane that does not begin with column tile 0 computes it first where its rows spill (t = -1); a pair agrees
+    // Where rows spill without a given reference exponent, a lane that does not begin with column tile 0 computes it first
+    // (t = -1); a pair agrees.
     auto first_tile = [&](int rt, int ln) {
-        if (MODE != MODE_STATS || ln == 0) return 0;
+        if (MODE != MODE_STATS || TOPK == TOPK_NONE || ln == 0) return 0;
         const int rt0 = rt - static_cast<int>(rank);
         return spills(p, rt0) || (CG == 2 && spills(p, rt0 + 1)) ? -1 : 0;
     };
@@ -500,7 +518,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
             float thr_sh = -INFINITY;                             // just below the best threshold published by the other lanes
             bool want_topk = false;
             const bool spill = MODE == MODE_STATS && tile_ok && spills(p, rt);
-            const bool track_zmax = MODE == MODE_STATS && TOPK != TOPK_NONE && spill && p.row_zmax != nullptr;
+            const bool track_zmax = MODE == MODE_STATS && spill && p.row_zmax != nullptr;
             float zmax = -INFINITY;                               // the row's largest logit in this lane's column tiles
             float ref2 = 0.f;                                     // spill rows: exponent offset (log2 units)
             float lse2 = 0.f, coef = 0.f;                         // MODE_PROBS / fused MODE_OUT
@@ -545,11 +563,16 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                 const uint32_t t_row = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + ab * BN;
                 const int col_base = ct * BN;
                 const bool skip_tile = t < 0 || !tile_ok;
-                if (MODE == MODE_STATS && spill && t == t0) {
+                if (CAPTURE && spill && t == 0) {
+                    ref2 = 0.f;
+                    if (row_ok) ref2 = p.use_row_zmax ? fmaf(__uint_as_float(key_bits(p.row_zmax[rt * BM + r_local])), LOG2E, 64.f) : p.row_ref2[g_row];
+                    m = ref2 * (1.0f / LOG2E);
+                }
+                if (MODE == MODE_STATS && TOPK != TOPK_NONE && spill && t == t0) {
                     // Reference exponent of this row: its largest logit in column tile 0. Every lane of
                     // the row tile computes tile 0 first and so derives the same value.
                     float mx = -INFINITY;
-                    if (TOPK != TOPK_NONE && p.use_row_zmax) {
+                    if (p.use_row_zmax) {
                         // second sweep after a range report: the row's largest logit is known
                         mx = __uint_as_float(key_bits(p.row_zmax[rt * BM + r_local]));
                     } else {
@@ -600,6 +623,33 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                         thr_own = below;
                         thr = fmaxf(thr_own, thr_sh);
                     }
+                }
+                if (USE_REG && want_topk && t == 0 && p.n_cols - col_base >= BN) {
+                    // First tile of the sweep, list empty: the K-th largest of the maxima of 16 groups of 16 logits is a
+                    // lower bound of the row's K-th largest that about 16 of the tile's 256 logits reach. Without it every
+                    // row inserts its first 32 logits and some 70 more one by one, the warp as often as its slowest row
+                    // (64 rows x 256 x 1024, four tiles on four CTAs: 28.0 -> 17.5 us).
+                    float gm[16];
+#pragma unroll
+                    for (int ch = 0; ch < BN / 32; ++ch) {
+                        uint32_t r[32];
+                        tmem_ld32(t_row + ch * 32, r);
+                        tmem_ld_wait(r);
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            float x = fmaxf(__uint_as_float(r[16 * h]), __uint_as_float(r[16 * h + 1]));
+#pragma unroll
+                            for (int j = 2; j < 16; j += 2) x = fmax3(x, __uint_as_float(r[16 * h + j]), __uint_as_float(r[16 * h + j + 1]));
+                            gm[2 * ch + h] = x;
+                        }
+                    }
+                    sort16_descending(gm);
+                    float kth = gm[0];
+#pragma unroll
+                    for (int i = 1; i < 16; ++i)
+                        if (i == p.K - 1) kth = gm[i];
+                    thr_sh = fmaxf(thr_sh, nextafterf(kth, -INFINITY));      // (a logit equal to the bound must be admitted)
+                    thr = fmaxf(thr, thr_sh);
                 }
                 if (CAPTURE && !skip_tile) {
                     while (nxt < col_base) {
@@ -907,18 +957,18 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                 }
                 ab ^= 1;
                 if (ab == 0) aphase ^= 1u;
-                if (MODE == MODE_STATS && want_topk && p.thr_share != nullptr && S > 1) {
+                if (MODE == MODE_STATS && want_topk && S > 1) {
                     // The K-th largest logit of ANY lane's part of the row is a lower bound of the row's K-th
                     // largest, so a lane may adopt the other lanes' thresholds: publish ours, read up to three
                     // neighbours. A logit equal to a foreign threshold must still be admitted (ties are settled
                     // by token id when the lists are merged), hence the step just below it. Stale or missing
-                    // (NaN) values only leave the threshold lower than it could be.
-                    volatile float* sh = p.thr_share + static_cast<long long>(slot - ln) * BM + r_local;
-                    sh[static_cast<long long>(ln) * BM] = thr_own;
+                    // (zero) values only leave the threshold lower than it could be.
+                    volatile unsigned int* sh = p.thr_share + static_cast<long long>(slot - ln) * BM + r_local;
+                    sh[static_cast<long long>(ln) * BM] = ordered_key(__float_as_uint(thr_own));      // (the first tile's bound is in thr_sh)
                     const int nn = S - 1 < 3 ? S - 1 : 3;
                     for (int q = 1; q <= nn; ++q) {
-                        const float v = sh[static_cast<long long>((ln + q) % S) * BM];
-                        thr_sh = fmaxf(thr_sh, nextafterf(v, -INFINITY));
+                        const unsigned int v = sh[static_cast<long long>((ln + q) % S) * BM];
+                        if (v != 0u) thr_sh = fmaxf(thr_sh, nextafterf(__uint_as_float(key_bits(v)), -INFINITY));
                     }
                     thr = fmaxf(thr, thr_sh);
                 }
@@ -929,7 +979,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                 p.part_s[so] = s;
                 // a spilled value reached the top of the fp32 range: the row's logits spread too far
                 // above its reference for the fixed-exponent spill
-                if (spill && !(s < 1e38f)) atomicCAS(p.status, 0u, (5u << 8) | 2u);
+                if (spill && !(s < 1e38f)) atomicExch(p.status + 1, 1u);
                 if (track_zmax && !p.use_row_zmax) atomicMax(p.row_zmax + rt * BM + r_local, ordered_key(__float_as_uint(zmax)));
                 if (USE_REG && want_topk) {
                     // the register list goes out as a full buffer of K_REG entries (unused ones carry id -1)
@@ -968,7 +1018,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
 // out_reduce_kernel: adds up the partial tiles of MODE_OUT in the order of the contraction and finishes them as its
 // epilogue does. One thread per four columns; memory-bound (reads cuts x, writes 1 x the rest tiles).
 __global__ void __launch_bounds__(256) out_reduce_kernel(const __grid_constant__ GemmParams p) {
-    if (p.only_if_range != nullptr && ((*p.only_if_range) & 0xffu) != 2u) return;
+    if (p.gate != nullptr && *p.gate == 0u) return;
     const OutPlan& o = p.plan;
     const long long i = static_cast<long long>(blockIdx.x) * 256 + threadIdx.x;
     const int c = static_cast<int>(i % (BN / 4)) * 4;
@@ -1001,32 +1051,26 @@ __global__ void __launch_bounds__(256) out_reduce_kernel(const __grid_constant__
 }
 
 // ---------------------------------------------------------------------------------------------
-// finalize: one warp per row. Merges the per-slot (max, sum-exp) pairs into lse_t / lse_d, selects
-// Omega_hat from the slots' candidates (or takes it as an input), gathers the draft logits at
-// Omega_hat with K dot products, and evaluates Eq. 1.
+// finalize: the routes that do not know Omega_hat before their sweep of the draft rows. Merges the draft's partial
+// statistics into lse_d, gathers the draft logits at Omega_hat with dot products, and evaluates Eq. 1.
 struct FinalizeParams {
     Schedule sched;
     int d, K;
-    int cap;               // capacity of a (row, slot) candidate buffer
     int row_begin, rows;   // global rows [row_begin, row_begin + rows) = local row tiles 0.. of the schedule
-    int row_tiles_t;       // row tiles of the target matrix in the schedule (0: Omega_hat is an input)
+    int row_tiles_t;       // row tiles of the target matrix in the schedule, before the draft's
     const float* part_m;
     const float* part_s;
-    const uint2* cand;
-    const int* cand_n;
     const __nv_bfloat16* H_d;
     const __nv_bfloat16* W;
-    const int* idx_in;     // [N,K] when row_tiles_t == 0
-    const float* q_in;
+    int* idx;              // [N, idx_pitch] Omega_hat in descending q, from select_kernel or the caller
+    float* q;              // (bidir: the joining tokens are added behind the K of the target)
+    int idx_pitch;
+    const float* lse_t;    // (read by the combined objective, Normed and Bi-directional Top-K)
     float* loss;
-    int* idx_out;
-    float* q_out;
-    float* lse_t;
     float* lse_d;
-    // fused backward (all nullable): per-row scale of the spilled tiles and g * q of Omega_hat
+    // fused backward (all nullable): per-row scale of the spilled tiles and the Omega_hat term
     const float* grad_loss;
     float* coef_out;       // [N]   g * S_q * exp(m_spill - lse_d), m_spill = the row's spill reference
-    float* gq_out;         // [N,K] g * q, in the order of topk_idx
     float* sparse_out;     // [rows, d] sum_{x in Omega_hat} g q(x) W[x, :], indexed by local row
     // combined objective CE(q, p) + w * Top-K (coef_t_out != nullptr): the target tiles were spilled as well
     float w_topk;          // weight w of the Top-K term
@@ -1036,16 +1080,15 @@ struct FinalizeParams {
     float* ce_corr_out;    // [N] sum_{x in Omega_hat} (q(x) - bf16 q(x)) z_d(x): the cross-entropy is formed from
                            // the bf16 spill; its largest terms are put back in fp32
     // loss variants of Section 4.3
-    float top_p;           // > 0: Omega_hat is cut to the shortest sorted prefix with cumulative q > top_p (Top-P)
-    int* n_out;            // [N] |Omega_hat| (nullable)
+    int* n_out;            // [N] |Omega_hat| (bidir, nullable)
     int normed;            // 1: Normed Top-K - q, p renormalised over Omega_hat; no draft sweep exists, and the
                            // gradient row sum_x g (pn(x) - qn(x)) W[x,:] goes straight to dH_out
     void* dH_out;          // [N, d] (normed only)
     int dH_fp32;
-    int bidir;             // 1: Bi-directional Top-K - Omega_hat also takes the draft's K most probable tokens (the draft
-                           // rows collected candidates too); idx_out / q_out then have 2K entries per row
+    const int* idx_d;      // bidir: [N, K] the draft's K most probable tokens in descending p; those outside the target's
+                           // set join Omega_hat (idx / q have 2K entries per row)
     const __nv_bfloat16* H_t;   // target features (bidir: target logits of the draft's tokens)
-    const unsigned int* only_if_range;   // as in GemmParams
+    const unsigned int* gate;            // as in GemmParams
 };
 
 __device__ __forceinline__ void find_slots(const Schedule& sc, int row_tile, int& slot0, int& S) {
@@ -1076,220 +1119,96 @@ __device__ __forceinline__ float warp_lse(const float* pm, const float* ps, int 
     return m + logf(s);
 }
 
-constexpr int FIN_GRP = 16;   // tokens of Omega_hat whose W rows finalize reads together
+constexpr int FIN_GRP = 16;       // tokens of Omega_hat whose W rows finalize reads together
+constexpr int FIN_WARPS = 4;      // warps that share a row
 
-__global__ void __launch_bounds__(256) finalize_kernel(const __grid_constant__ FinalizeParams p) {
-    if (p.only_if_range != nullptr && ((*p.only_if_range) & 0xffu) != 2u) return;
-    const int lane = threadIdx.x & 31;
-    const int local = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (local >= p.rows) return;
+__device__ __forceinline__ void unpack8(const uint4& v, float (&f)[8]) {
+    const __nv_bfloat162* p2 = reinterpret_cast<const __nv_bfloat162*>(&v);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        const float2 f2 = __bfloat1622float2(p2[t]);
+        f[2 * t] = f2.x;
+        f[2 * t + 1] = f2.y;
+    }
+}
+
+// One block per row (2048 rows, 20 tokens, d = 4096: 390 us with a warp per row and a serial selection -> 158 us, and 24 us
+// in select_kernel; 1024 rows, 10 tokens: 144 -> 55 us): bound by the latency of the gathered rows of W, so that a row's columns are spread over FIN_WARPS
+// warps (8 columns per thread and step) and FIN_GRP rows of W are in flight per thread.
+__global__ void __launch_bounds__(FIN_WARPS * 32) finalize_kernel(const __grid_constant__ FinalizeParams p) {
+    if (p.gate != nullptr && *p.gate == 0u) return;
+    __shared__ int sh_tok[K_CAP];         // Omega_hat of the row (the bi-directional set needs 2K <= K_CAP)
+    __shared__ float sh_q[K_CAP];
+    __shared__ float sh_dot[K_CAP];       // z_d at Omega_hat
+    __shared__ float sh_part[FIN_WARPS][FIN_GRP];
+    __shared__ int sh_n;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int local = blockIdx.x;
     const int row = p.row_begin + local;
     const int rt = local / BM, r = local % BM;
     const int K = p.K;
-    int slot0, S;
+    auto warp_sum = [](float v) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        return v;
+    };
 
     // draft statistics (the Normed Top-K variant has none: it needs the draft logits on Omega_hat only)
     float lse_d = 0.f, m_spill = 0.f;
-    int slot0_d = 0, S_d = 0;
+    int slot0, S;
     if (!p.normed) {
         find_slots(p.sched, p.row_tiles_t + rt, slot0, S);
-        slot0_d = slot0;
-        S_d = S;
         lse_d = warp_lse(p.part_m, p.part_s, slot0, S, r, lane);
-        if (lane == 0) p.lse_d[row] = lse_d;
         m_spill = p.part_m[static_cast<long long>(slot0) * BM + r];
     }
     const float g = p.grad_loss ? p.grad_loss[row] : 1.f;
-    float S_q = 0.f;
-
-    float lse_t = 0.f;
-    if (p.row_tiles_t > 0) {
-        find_slots(p.sched, rt, slot0, S);
-        lse_t = warp_lse(p.part_m, p.part_s, slot0, S, r, lane);
-        if (lane == 0) {
-            p.lse_t[row] = lse_t;
-            if (p.coef_t_out) p.coef_t_out[row] = expf(p.part_m[static_cast<long long>(slot0) * BM + r] - lse_t);
-        }
-    }
     const bool combined = p.coef_t_out != nullptr;
-    const float coef_t = combined ? expf(p.part_m[static_cast<long long>(slot0) * BM + r] - lse_t) : 0.f;
-    float ce_corr = 0.f;
+    float coef_t = 0.f;
+    if (combined) {
+        find_slots(p.sched, rt, slot0, S);
+        coef_t = expf(p.part_m[static_cast<long long>(slot0) * BM + r] - p.lse_t[row]);
+    }
     const float gw = combined ? g * p.w_topk : g;     // weight of the Omega_hat term q 1[Omega_hat] in dz_d
 
     const __nv_bfloat16* hrow = p.H_d + static_cast<long long>(row) * p.d;
-    float loss = 0.f;
-    float prev_v = INFINITY;
-    int prev_i = -1;
-    const int cap = p.cap;
-    __shared__ int sh_tok[8][K_CAP];      // Omega_hat of the warp's row (the bi-directional set needs 2K <= K_CAP)
-    __shared__ float sh_q[8][K_CAP];
-    __shared__ float sh_dot[8][K_CAP];
-    float cum_q = 0.f;
-    int n_sel = 0;
-    const int wib = threadIdx.x >> 5;
-    // next candidate of the slots [sl0, sl0 + nS) after (pv, pi) in the order: logit descending, then token id
-    // ascending (warp-collective; every lane gets the result)
-    auto select_next = [&](int sl0, int nS, float pv, int pi, float& bv, int& bi) {
-        bv = -INFINITY;
-        bi = INT_MAX;
-        for (int sl = 0; sl < nS; ++sl) {
-            const long long so = static_cast<long long>(sl0 + sl) * BM + r;
-            const int n = p.cand_n[so];
-            for (int e = lane; e < n; e += 32) {
-                const uint2 ce = p.cand[so * cap + e];
-                const float v = __uint_as_float(ce.x);
-                const int i = static_cast<int>(ce.y);
-                if (i < 0) continue;
-                const bool after_prev = (v < pv) || (v == pv && i > pi);
-                const bool better = (v > bv) || (v == bv && i < bi);
-                if (after_prev && better) {
-                    bv = v;
-                    bi = i;
-                }
-            }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-            if (ov > bv || (ov == bv && oi < bi)) {
-                bv = ov;
-                bi = oi;
-            }
-        }
-    };
-    const int ostride = p.bidir ? 2 * K : K;     // entries per row of idx_out / q_out
-    for (int j = 0; j < K; ++j) {
-        int tok;
-        float qv;
-        if (p.row_tiles_t > 0) {
-            float bv;
-            int bi;
-            select_next(slot0, S, prev_v, prev_i, bv, bi);
-            prev_v = bv;
-            prev_i = bi;
-            tok = bi == INT_MAX ? 0 : bi;     // cannot happen for K <= V; keeps the gather in range
-            qv = expf(bv - lse_t);
-            int tok_out = tok;
-            if (p.top_p > 0.f) {
-                // Top-P: a token belongs to Omega_hat while the probability of those before it is <= P
-                if (cum_q > p.top_p) {
-                    tok_out = -1;
-                    tok = 0;
-                    qv = 0.f;
-                } else {
-                    ++n_sel;
-                }
-                cum_q += qv;
-            } else {
-                ++n_sel;
-            }
-            if (lane == 0) {
-                p.idx_out[static_cast<long long>(row) * ostride + j] = tok_out;
-                p.q_out[static_cast<long long>(row) * ostride + j] = qv;
-            }
-        } else {
-            tok = p.idx_in[static_cast<long long>(row) * K + j];
-            qv = p.q_in[static_cast<long long>(row) * K + j];
-        }
-        S_q += qv;
-        if (lane == 0) {
-            if (p.gq_out) p.gq_out[static_cast<long long>(row) * K + j] = g * qv;
-            sh_tok[wib][j] = tok;
-            sh_q[wib][j] = qv;
-        }
+    const long long io = static_cast<long long>(row) * p.idx_pitch;
+    for (int j = tid; j < K; j += FIN_WARPS * 32) {
+        const int tok = p.idx[io + j];
+        sh_tok[j] = tok < 0 ? 0 : tok;                // (cut entries carry q = 0)
+        sh_q[j] = p.q[io + j];
     }
-    __syncwarp();
-    int Ku = K;                                   // |Omega_hat| slots in use (2K at most for the bi-directional set)
-    if (p.bidir) {
-        // the draft's own K most probable tokens, in descending p; those not in the target's set join Omega_hat
-        float pv = INFINITY;
-        int pi = -1;
-        for (int j = 0; j < K; ++j) {
-            float bv;
-            int bi;
-            select_next(slot0_d, S_d, pv, pi, bv, bi);
-            pv = bv;
-            pi = bi;
-            if (bi == INT_MAX) break;
-            bool dup = false;
-            for (int t = lane; t < K; t += 32) dup |= (sh_tok[wib][t] == bi);
-            if (__any_sync(0xffffffffu, dup)) continue;
-            // target probability of this token: q = exp(<H_t[row], W[tok]> - lse_t)
-            const __nv_bfloat16* trow = p.H_t + static_cast<long long>(row) * p.d;
-            const __nv_bfloat16* wrow = p.W + static_cast<long long>(bi) * p.d;
-            float acc = 0.f;
-            for (int k0 = lane * 8; k0 < p.d; k0 += 256) {
-                const uint4 hv = *reinterpret_cast<const uint4*>(trow + k0);
-                const uint4 wv = *reinterpret_cast<const uint4*>(wrow + k0);
-                const __nv_bfloat162* hp = reinterpret_cast<const __nv_bfloat162*>(&hv);
-                const __nv_bfloat162* wp = reinterpret_cast<const __nv_bfloat162*>(&wv);
-#pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    const float2 a2 = __bfloat1622float2(hp[t]);
-                    const float2 b2 = __bfloat1622float2(wp[t]);
-                    acc = fmaf(a2.x, b2.x, acc);
-                    acc = fmaf(a2.y, b2.y, acc);
-                }
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            const float qv = expf(acc - lse_t);
-            S_q += qv;
-            if (lane == 0) {
-                sh_tok[wib][Ku] = bi;
-                sh_q[wib][Ku] = qv;
-                p.idx_out[static_cast<long long>(row) * ostride + Ku] = bi;
-                p.q_out[static_cast<long long>(row) * ostride + Ku] = qv;
-            }
-            ++Ku;
-        }
-        for (int u = Ku + lane; u < 2 * K; u += 32) {
-            p.idx_out[static_cast<long long>(row) * ostride + u] = -1;
-            p.q_out[static_cast<long long>(row) * ostride + u] = 0.f;
-        }
-        n_sel = Ku;
-        __syncwarp();
-    }
-    // Draft logits at Omega_hat (K dot products with rows of W) and, for the fused backward, the row
-    // sum_{x in Omega_hat} g q(x) W[x, :]. The W rows are read once: FIN_GRP tokens at a time, 256 columns
-    // (8 per lane) per step; the fp32 row is accumulated across token groups.
-    float* so = (p.sparse_out && !p.normed) ? p.sparse_out + static_cast<long long>(local) * p.d : nullptr;
-    for (int g0 = 0; g0 < Ku; g0 += FIN_GRP) {
-        const int ng = Ku - g0 < FIN_GRP ? Ku - g0 : FIN_GRP;
+    __syncthreads();
+
+    // The dot products of `from`'s row with the W rows of tokens [b, b + n), n <= FIN_GRP, summed over the block into
+    // `to`; with `so` also the row sum of gw q(x) W[x, :], added to what is there when b > 0.
+    auto gather = [&](const __nv_bfloat16* from, int b, int n, float* to, float* so) {
         float dot[FIN_GRP];
 #pragma unroll
         for (int jj = 0; jj < FIN_GRP; ++jj) dot[jj] = 0.f;
-        for (int k0 = lane * 8; k0 < p.d; k0 += 256) {
-            const uint4 hv = *reinterpret_cast<const uint4*>(hrow + k0);
-            const __nv_bfloat162* hp = reinterpret_cast<const __nv_bfloat162*>(&hv);
+        for (int k0 = tid * 8; k0 < p.d; k0 += FIN_WARPS * 256) {
             float h[8];
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                const float2 f2 = __bfloat1622float2(hp[t]);
-                h[2 * t] = f2.x;
-                h[2 * t + 1] = f2.y;
-            }
+            unpack8(*reinterpret_cast<const uint4*>(from + k0), h);
             float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            if (so && g0 > 0) {
+            if (so && b > 0) {
                 const float4 a0 = *reinterpret_cast<const float4*>(so + k0);
                 const float4 a1 = *reinterpret_cast<const float4*>(so + k0 + 4);
                 a[0] = a0.x; a[1] = a0.y; a[2] = a0.z; a[3] = a0.w;
                 a[4] = a1.x; a[5] = a1.y; a[6] = a1.z; a[7] = a1.w;
             }
+            uint4 wv[FIN_GRP];
+#pragma unroll
+            for (int jj = 0; jj < FIN_GRP; ++jj)
+                if (jj < n) wv[jj] = *reinterpret_cast<const uint4*>(p.W + static_cast<long long>(sh_tok[b + jj]) * p.d + k0);
 #pragma unroll
             for (int jj = 0; jj < FIN_GRP; ++jj) {
-                if (jj < ng) {
-                    const float gq = gw * sh_q[wib][g0 + jj];
-                    const uint4 wv = *reinterpret_cast<const uint4*>(p.W + static_cast<long long>(sh_tok[wib][g0 + jj]) * p.d + k0);
-                    const __nv_bfloat162* wp = reinterpret_cast<const __nv_bfloat162*>(&wv);
+                if (jj < n) {
+                    float wf[8];
+                    unpack8(wv[jj], wf);
+                    const float gq = so ? gw * sh_q[b + jj] : 0.f;
 #pragma unroll
-                    for (int t = 0; t < 4; ++t) {
-                        const float2 b = __bfloat1622float2(wp[t]);
-                        dot[jj] = fmaf(h[2 * t], b.x, dot[jj]);
-                        dot[jj] = fmaf(h[2 * t + 1], b.y, dot[jj]);
-                        a[2 * t] = fmaf(gq, b.x, a[2 * t]);
-                        a[2 * t + 1] = fmaf(gq, b.y, a[2 * t + 1]);
+                    for (int t = 0; t < 8; ++t) {
+                        dot[jj] = fmaf(h[t], wf[t], dot[jj]);
+                        a[t] = fmaf(gq, wf[t], a[t]);
                     }
                 }
             }
@@ -1300,56 +1219,82 @@ __global__ void __launch_bounds__(256) finalize_kernel(const __grid_constant__ F
         }
 #pragma unroll
         for (int jj = 0; jj < FIN_GRP; ++jj) {
-            float acc = dot[jj];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (jj < ng) {
-                const float qv = sh_q[wib][g0 + jj];
-                if (lane == 0) sh_dot[wib][g0 + jj] = acc;
-                loss += qv * (lse_d - acc);     // -q log p,  log p = z_d - lse_d
-                if (combined) {
-                    const float q_spill = __bfloat162float(p.Pt[static_cast<long long>(local) * p.p_pitch + sh_tok[wib][g0 + jj]]) * coef_t;
-                    ce_corr += (qv - q_spill) * acc;
-                }
-            }
+            const float acc = warp_sum(dot[jj]);
+            if (lane == 0) sh_part[warp][jj] = acc;
         }
+        __syncthreads();
+        if (tid < n) {
+            float acc = 0.f;
+#pragma unroll
+            for (int w = 0; w < FIN_WARPS; ++w) acc += sh_part[w][tid];
+            to[b + tid] = acc;
+        }
+        __syncthreads();
+    };
+
+    int Ku = K;                                       // |Omega_hat| (2K at most for the bi-directional set)
+    if (p.idx_d != nullptr) {
+        // the draft's own K most probable tokens that are not in the target's set join Omega_hat, in their order
+        if (warp == 0) {
+            int n = K;
+            for (int j0 = 0; j0 < K; j0 += 32) {
+                const int j = j0 + lane;
+                const int tok = j < K ? p.idx_d[static_cast<long long>(row) * K + j] : -1;
+                bool joins = j < K;
+                for (int t = 0; t < K; ++t) joins = joins && sh_tok[t] != tok;
+                const uint32_t bm = __ballot_sync(0xffffffffu, joins);
+                if (joins) sh_tok[n + __popc(bm & ((1u << lane) - 1u))] = tok;
+                n += __popc(bm);
+            }
+            if (lane == 0) sh_n = n;
+        }
+        __syncthreads();
+        Ku = sh_n;
+        // their target probabilities: q = exp(<H_t[row], W[tok]> - lse_t)
+        const float lse_t = p.lse_t[row];
+        for (int b = K; b < Ku; b += FIN_GRP)
+            gather(p.H_t + static_cast<long long>(row) * p.d, b, Ku - b < FIN_GRP ? Ku - b : FIN_GRP, sh_q, nullptr);
+        for (int j = K + tid; j < 2 * K; j += FIN_WARPS * 32) {
+            const float qv = j < Ku ? expf(sh_q[j] - lse_t) : 0.f;
+            if (j < Ku) sh_q[j] = qv;
+            p.idx[io + j] = j < Ku ? sh_tok[j] : -1;
+            p.q[io + j] = qv;
+        }
+        if (tid == 0 && p.n_out) p.n_out[row] = Ku;
+        __syncthreads();
     }
-    if (lane == 0 && p.n_out) p.n_out[row] = (p.top_p > 0.f && !(cum_q > p.top_p)) ? -n_sel : n_sel;
+    // draft logits at Omega_hat and, for the fused backward, the row sum_{x in Omega_hat} g q(x) W[x, :]
+    float* so = (p.sparse_out && !p.normed) ? p.sparse_out + static_cast<long long>(local) * p.d : nullptr;
+    for (int b = 0; b < Ku; b += FIN_GRP) gather(hrow, b, Ku - b < FIN_GRP ? Ku - b : FIN_GRP, sh_dot, so);
+
+    float S_q = 0.f;
+    for (int j = lane; j < Ku; j += 32) S_q += sh_q[j];
+    S_q = warp_sum(S_q);
     if (p.normed) {
         // Normed Top-K: qn = q / S_q, pn = softmax of the draft logits restricted to Omega_hat
-        __syncwarp();
         float mx = -INFINITY;
-        for (int j = lane; j < K; j += 32) mx = fmaxf(mx, sh_dot[wib][j]);
+        for (int j = lane; j < K; j += 32) mx = fmaxf(mx, sh_dot[j]);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         float se = 0.f;
-        for (int j = lane; j < K; j += 32) se += expf(sh_dot[wib][j] - mx);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
-        const float lse_k = mx + logf(se);
+        for (int j = lane; j < K; j += 32) se += expf(sh_dot[j] - mx);
+        const float lse_k = mx + logf(warp_sum(se));
         float ln = 0.f;
-        for (int j = lane; j < K; j += 32) {
-            const float qn = sh_q[wib][j] / S_q;
-            const float zj = sh_dot[wib][j];
-            ln += qn * (lse_k - zj);
-            sh_dot[wib][j] = g * (expf(zj - lse_k) - qn);      // dL/dz_d on Omega_hat
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ln += __shfl_xor_sync(0xffffffffu, ln, o);
-        loss = ln;
-        __syncwarp();
-        for (int k0 = lane * 8; k0 < p.d; k0 += 256) {
+        for (int j = lane; j < K; j += 32) ln += sh_q[j] / S_q * (lse_k - sh_dot[j]);
+        ln = warp_sum(ln);
+        __syncthreads();
+        for (int j = tid; j < K; j += FIN_WARPS * 32)
+            sh_dot[j] = g * (expf(sh_dot[j] - lse_k) - sh_q[j] / S_q);      // dL/dz_d on Omega_hat
+        __syncthreads();
+        for (int k0 = tid * 8; k0 < p.d; k0 += FIN_WARPS * 256) {
             float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 8
             for (int j = 0; j < K; ++j) {
-                const float c = sh_dot[wib][j];
-                const uint4 wv = *reinterpret_cast<const uint4*>(p.W + static_cast<long long>(sh_tok[wib][j]) * p.d + k0);
-                const __nv_bfloat162* wp = reinterpret_cast<const __nv_bfloat162*>(&wv);
+                const float c = sh_dot[j];
+                float wf[8];
+                unpack8(*reinterpret_cast<const uint4*>(p.W + static_cast<long long>(sh_tok[j]) * p.d + k0), wf);
 #pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    const float2 b = __bfloat1622float2(wp[t]);
-                    a[2 * t] = fmaf(c, b.x, a[2 * t]);
-                    a[2 * t + 1] = fmaf(c, b.y, a[2 * t + 1]);
-                }
+                for (int t = 0; t < 8; ++t) a[t] = fmaf(c, wf[t], a[t]);
             }
             if (p.dH_fp32) {
                 float* o = reinterpret_cast<float*>(p.dH_out) + static_cast<long long>(row) * p.d + k0;
@@ -1364,212 +1309,333 @@ __global__ void __launch_bounds__(256) finalize_kernel(const __grid_constant__ F
                 *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.dH_out) + static_cast<long long>(row) * p.d + k0) = w;
             }
         }
+        if (tid == 0) p.loss[row] = ln;
+        return;
     }
-    if (lane == 0) {
-        if (combined) p.ce_corr_out[row] = ce_corr;
-        p.loss[row] = loss;
-        // dense part of dz_d: g S_q p (Top-K loss) or g (1 + w S_q) p (combined objective)
-        if (p.coef_out) p.coef_out[row] = (combined ? g * (1.f + p.w_topk * S_q) : g * S_q) * expf(m_spill - lse_d);
+    if (warp == 0) {
+        float loss = 0.f, ce_corr = 0.f;
+        for (int j = lane; j < Ku; j += 32) {
+            loss += sh_q[j] * (lse_d - sh_dot[j]);    // -q log p,  log p = z_d - lse_d
+            if (combined) {
+                const float q_spill = __bfloat162float(p.Pt[static_cast<long long>(local) * p.p_pitch + sh_tok[j]]) * coef_t;
+                ce_corr += (sh_q[j] - q_spill) * sh_dot[j];
+            }
+        }
+        loss = warp_sum(loss);
+        ce_corr = warp_sum(ce_corr);
+        if (lane == 0) {
+            p.loss[row] = loss;
+            p.lse_d[row] = lse_d;
+            if (combined) {
+                p.ce_corr_out[row] = ce_corr;
+                p.coef_t_out[row] = coef_t;
+            }
+            // dense part of dz_d: g S_q p (Top-K loss) or g (1 + w S_q) p (combined objective)
+            if (p.coef_out) p.coef_out[row] = (combined ? g * (1.f + p.w_topk * S_q) : g * S_q) * expf(m_spill - lse_d);
+        }
     }
 }
 
 // ---------------------------------------------------------------------------------------------
-// select_kernel: one warp per row, between the sweep of the target rows and the sweep of the draft rows of
-// the fused call. Merges the target's partial statistics into lse_t, picks Omega_hat from the sweep's
-// candidates (or takes it as an input), writes topk_idx / topk_q in descending q, and leaves the same set
-// sorted by token id (sidx, sq) for the draft sweep, which copies z_d at those tokens out of its accumulators.
-constexpr int SEL_WARPS = 4;          // warps (rows) per block
-constexpr int SEL_MAX = 768;          // candidates of one row that fit its shared-memory window (> K_CAP + 32)
+// select_kernel: between the sweep of the target rows and the sweep of the draft rows of the fused call. Merges the
+// target's partial statistics into lse_t, picks Omega_hat from the sweep's candidates (or takes it as an input), writes
+// topk_idx / topk_q in descending q, and leaves the same set sorted by token id (sidx, sq) for the draft sweep, which
+// copies z_d at those tokens out of its accumulators.
+// Bound by load latency: the lists of the row's lanes are read 256 entries at a time per warp (32 lanes x SEL_LOADS loads in
+// flight) and what lies below the best K-th logit of any list is dropped on the way. WARPS warps share a row: one where
+// there are rows enough to fill the GPU, four where few rows have lists of up to 148 lanes each.
+constexpr int SEL_WARPS = 4;          // warps per block
+constexpr int SEL_LOADS = 8;          // candidate loads a lane has in flight
+constexpr int SEL_FIRST = 5;          // lists per lane whose first entries set the floor (the first 160 of the row)
 
 struct SelectParams {
-    Schedule sched;        // schedule of the target sweep; its row tile t = rows [128 t, 128 t + 128) of the chunk
+    Schedule sched;        // schedule of the sweep; its row tile first_tile + t = rows [128 t, 128 t + 128) of the chunk
+    int first_tile;
     int K, cap;
     int row_begin, rows;   // global rows [row_begin, row_begin + rows)
     int from_sweep;        // 1: Omega_hat from the sweep's candidates; 0: idx_in / q_in are given
+    int out_pitch;         // entries per row of idx_out / q_out
     const float* part_m;
     const float* part_s;
     const uint2* cand;
     const int* cand_n;
+    const unsigned int* thr_share;    // [slot, row] key of the K-th largest logit of a lane's buffer at its last compaction, or 0
     const int* idx_in;     // [N, K]
     const float* q_in;
     int* idx_out;          // [N, K] (from_sweep)
     float* q_out;
-    float* lse_t;
+    float* lse_t;          // (nullable)
     int* n_out;            // [N] |Omega_hat| (nullable)
     float top_p;           // > 0: Omega_hat is cut to the shortest sorted prefix with cumulative q > top_p
-    int* sidx;             // [N, K] Omega_hat in increasing token id; unused entries INT_MAX
+    int* sidx;             // [N, K] Omega_hat in increasing token id; unused entries INT_MAX (nullable)
     float* sq;             // [N, K] q in the same order; unused entries 0
-    const unsigned int* only_if_range;
+    unsigned int* zmax;    // [chunk row] set to zero for the draft sweep (nullable)
+    const unsigned int* gate;
+    // Reference exponent of the row's spill (nullable ref2): z_d at the most probable token of Omega_hat, a logit that the
+    // draft sweep will meet, so that the row's largest is never below it
+    const __nv_bfloat16* H_d;
+    const __nv_bfloat16* W;
+    int d, V;
+    float* ref2;           // [N] z_d log2e + 64
 };
 
-// Warp-collective: the largest t such that at least `want` of the n keys satisfy key >= t (keys pass the
-// filter `use`); bit by bit from the top.
-template <typename KeyFn>
-__device__ __forceinline__ uint32_t kth_largest_key(int n, int want, int lane, KeyFn key_of) {
-    uint32_t T = 0u;
+// A candidate as one number: larger = larger logit, lower token id first among equal logits.
+__device__ __forceinline__ unsigned long long cand_rank(uint32_t key, uint32_t id) {
+    return (static_cast<unsigned long long>(key) << 32) | (~id);
+}
+
+// Warp-collective: keeps the K best of the n > K candidates in `pool` (distinct numbers), in place, and returns the
+// smallest one kept. The bound is searched bit by bit from the top until exactly K reach it.
+__device__ __forceinline__ unsigned long long cut_to_best(unsigned long long* pool, int n, int K, int lane) {
+    unsigned long long T = 0ull;
 #pragma unroll 1
-    for (int bit = 31; bit >= 0; --bit) {
-        const uint32_t c2 = T | (1u << bit);
+    for (int bit = 63; bit >= 0; --bit) {
+        const unsigned long long c2 = T | (1ull << bit);
         int c = 0;
-        for (int e = lane; e < n; e += 32) {
-            uint32_t k;
-            if (key_of(e, k)) c += (k >= c2) ? 1 : 0;
-        }
+        for (int e = lane; e < n; e += 32) c += pool[e] >= c2 ? 1 : 0;
         c = __reduce_add_sync(0xffffffffu, c);
-        if (c >= want) T = c2;
+        if (c >= K) T = c2;
+        if (c == K) break;
+    }
+    const uint32_t lt_mask = (1u << lane) - 1u;
+    int np = 0;
+    for (int e0 = 0; e0 < n; e0 += 32) {
+        const int e = e0 + lane;
+        const unsigned long long v = e < n ? pool[e] : 0ull;
+        const bool take = e < n && v >= T;
+        const uint32_t bm = __ballot_sync(0xffffffffu, take);
+        if (take) pool[np + __popc(bm & lt_mask)] = v;      // position <= e: in place
+        np += __popc(bm);
+        __syncwarp();
     }
     return T;
 }
 
+template <int WARPS, int WIN>
 __global__ void __launch_bounds__(SEL_WARPS * 32) select_kernel(const __grid_constant__ SelectParams p) {
-    if (p.only_if_range != nullptr && ((*p.only_if_range) & 0xffu) != 2u) return;
-    __shared__ uint32_t sh_key[SEL_WARPS][SEL_MAX];   // ordered keys of the row's candidates
-    __shared__ int sh_id[SEL_WARPS][SEL_MAX];
-    __shared__ int sel_tok[SEL_WARPS][K_CAP];         // Omega_hat in descending q
-    __shared__ float sel_q[SEL_WARPS][K_CAP];
+    static_assert(WIN >= K_CAP + 32 * SEL_LOADS, "a cut leaves room for one batch of loads");
+    constexpr int ROWS = SEL_WARPS / WARPS;                   // rows per block
+    __shared__ unsigned long long pools[SEL_WARPS][WIN];
+    __shared__ int pool_n[SEL_WARPS];
+    __shared__ int sel_tok[ROWS][K_CAP];                      // Omega_hat in descending q
+    __shared__ float sel_q[ROWS][K_CAP];
     const int lane = threadIdx.x & 31;
-    const int wib = threadIdx.x >> 5;
-    const int local = blockIdx.x * SEL_WARPS + wib;
-    if (local >= p.rows) return;
+    const int warp = threadIdx.x >> 5;
+    const int rib = warp / WARPS, w = warp % WARPS;           // row in the block, warp of the row
+    const int tid = w * 32 + lane;                            // thread of the row
+    const int local = blockIdx.x * ROWS + rib;
+    if (local >= p.rows || (p.gate != nullptr && *p.gate == 0u)) return;      // (WARPS > 1: the whole block)
+    auto sync_row = [&]() {
+        if (WARPS > 1)
+            __syncthreads();
+        else
+            __syncwarp();
+    };
     const int row = p.row_begin + local;
-    const int rt = local / BM, r = local % BM;
+    const int rt = p.first_tile + local / BM, r = local % BM;
     const int K = p.K;
     const long long ro = static_cast<long long>(row) * K;
+    if (p.zmax != nullptr && tid == 0) p.zmax[local] = 0u;
 
     if (p.from_sweep) {
         int slot0, S;
         find_slots(p.sched, rt, slot0, S);
-        const float lse_t = warp_lse(p.part_m, p.part_s, slot0, S, r, lane);
-        if (lane == 0) p.lse_t[row] = lse_t;
-        // Pool of candidates in shared memory. The slots' lists are appended 32 entries at a time; whenever the
-        // next 32 might not fit, the pool is cut to its K best (logit descending, lower token id first among
-        // equal logits) and the K-th logit becomes a floor below which later candidates are not even copied.
-        uint32_t* kk = sh_key[wib];
-        int* ii = sh_id[wib];
-        int n = 0;
+        const bool lists = p.cap == K_REG;      // sorted register lists of K_REG entries (unused ones: id -1)
+        // lse_t, and a floor below which no candidate can be among the K best: the best K-th largest logit of any list,
+        // or the K-th largest of the lists' first entries
+        float m = -INFINITY, sum = 0.f;
         uint32_t floor_key = 0u;
+        uint32_t first[SEL_FIRST];
+#pragma unroll
+        for (int q = 0; q < SEL_FIRST; ++q) first[q] = 0u;
+#pragma unroll
+        for (int q = 0; q < SEL_FIRST; ++q) {
+            const int j = lane + 32 * q;
+            if (lists && j < S) {
+                const uint2* list = p.cand + (static_cast<long long>(slot0 + j) * BM + r) * K_REG;
+                const uint2 best = list[0], kth = list[K - 1];
+                if (static_cast<int>(best.y) >= 0) first[q] = ordered_key(best.x);
+                if (static_cast<int>(kth.y) >= 0) floor_key = max(floor_key, ordered_key(kth.x));
+            }
+        }
+        for (int j = lane; j < S; j += 32) {
+            const long long so = static_cast<long long>(slot0 + j) * BM + r;
+            const float pm = p.part_m[so], ps = p.part_s[so];
+            if (!lists) floor_key = max(floor_key, p.thr_share[so]);
+            if (pm > m) {
+                sum *= exp2f((m - pm) * LOG2E);
+                m = pm;
+            }
+            sum += ps * exp2f((pm - m) * LOG2E);
+        }
+        float mx = m;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (m > -INFINITY) sum *= exp2f((m - mx) * LOG2E);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        floor_key = __reduce_max_sync(0xffffffffu, floor_key);
+        if (lists && S >= K) {
+            uint32_t T = 0u;
+#pragma unroll 1
+            for (int bit = 31; bit >= 0; --bit) {
+                const uint32_t c2 = T | (1u << bit);
+                int c = 0;
+#pragma unroll
+                for (int q = 0; q < SEL_FIRST; ++q) c += first[q] >= c2 ? 1 : 0;
+                if (static_cast<int>(__reduce_add_sync(0xffffffffu, c)) >= K) T = c2;
+            }
+            floor_key = max(floor_key, T);
+        }
+        const float lse_t = mx + logf(sum);
+        if (tid == 0 && p.lse_t) p.lse_t[row] = lse_t;
+
+        // this warp's share of the candidates: lanes of the row tile w, w + WARPS, ...
+        unsigned long long* pool = pools[warp];
+        int n = 0;
         const uint32_t lt_mask = (1u << lane) - 1u;
-        auto cut_to_k = [&]() {
-            // K-th largest logit, then (only if several candidates share it) the id bound among those
-            const uint32_t T = kth_largest_key(n, K, lane, [&](int e, uint32_t& k) { k = kk[e]; return true; });
-            int n_gt = 0, n_eq = 0;
-            for (int e = lane; e < n; e += 32) {
-                n_gt += kk[e] > T ? 1 : 0;
-                n_eq += kk[e] == T ? 1 : 0;
-            }
-            n_gt = __reduce_add_sync(0xffffffffu, n_gt);
-            n_eq = __reduce_add_sync(0xffffffffu, n_eq);
-            const int need_eq = K - n_gt;
-            uint32_t T2 = 0u;      // among the candidates equal to T: those with ~id >= T2 (the lowest ids) are kept
-            if (n_eq > need_eq)
-                T2 = kth_largest_key(n, need_eq, lane, [&](int e, uint32_t& k) { k = ~static_cast<uint32_t>(ii[e]); return kk[e] == T; });
-            int np = 0;
-            for (int e0 = 0; e0 < n; e0 += 32) {
-                const int e = e0 + lane;
-                uint32_t ke = 0u;
-                int ie = 0;
-                if (e < n) {
-                    ke = kk[e];
-                    ie = ii[e];
-                }
-                const bool take = e < n && (ke > T || (ke == T && ~static_cast<uint32_t>(ie) >= T2));
-                const uint32_t bm = __ballot_sync(0xffffffffu, take);
-                __syncwarp();
-                if (take) {
-                    const int at = np + __popc(bm & lt_mask);      // at <= e: in place
-                    kk[at] = ke;
-                    ii[at] = ie;
-                }
-                np += __popc(bm);
-                __syncwarp();
-            }
-            n = np;
-            floor_key = T;
-        };
-        for (int sl = 0; sl < S; ++sl) {
-            const long long so = static_cast<long long>(slot0 + sl) * BM + r;
-            const int cn = p.cand_n[so];
-            for (int e0 = 0; e0 < cn; e0 += 32) {
-                if (n + 32 > SEL_MAX) cut_to_k();      // n > K here: the window holds more than K_CAP + 32 entries
-                const int e = e0 + lane;
-                bool ok = false;
-                uint2 ce = make_uint2(0u, 0u);
-                uint32_t key = 0u;
-                if (e < cn) {
-                    ce = p.cand[so * p.cap + e];
-                    key = ordered_key(ce.x);
-                    // unused register-list entries carry id -1; anything below the floor cannot be among the K best
-                    ok = static_cast<int>(ce.y) >= 0 && key >= floor_key;
-                }
+        auto append = [&](const uint2 (&ce)[SEL_LOADS], const bool (&in)[SEL_LOADS]) {
+#pragma unroll
+            for (int q = 0; q < SEL_LOADS; ++q) {
+                const uint32_t key = ordered_key(ce[q].x);
+                const bool ok = in[q] && static_cast<int>(ce[q].y) >= 0 && key >= floor_key;
                 const uint32_t bm = __ballot_sync(0xffffffffu, ok);
-                if (ok) {
-                    const int at = n + __popc(bm & lt_mask);
-                    kk[at] = key;
-                    ii[at] = static_cast<int>(ce.y);
-                }
+                if (ok) pool[n + __popc(bm & lt_mask)] = cand_rank(key, ce[q].y);
                 n += __popc(bm);
             }
             __syncwarp();
-        }
-        if (n > K) cut_to_k();
-        __syncwarp();
-        // order the K picks: logit descending, token id ascending
-        for (int j = lane; j < K; j += 32) {
-            const uint32_t kj = j < n ? kk[j] : 0u;
-            const int ij = j < n ? ii[j] : 0;
-            int rank = 0;
-            for (int i = 0; i < K; ++i) {
-                const uint32_t ki = i < n ? kk[i] : 0u;
-                const int i2 = i < n ? ii[i] : 0;
-                rank += (ki > kj || (ki == kj && (i2 < ij || (i2 == ij && i < j)))) ? 1 : 0;
+            if (n + 32 * SEL_LOADS > WIN) {      // n > K here
+                floor_key = max(floor_key, static_cast<uint32_t>(cut_to_best(pool, n, K, lane) >> 32));
+                n = K;
             }
-            sel_tok[wib][rank] = ij;
-            sel_q[wib][rank] = j < n ? expf(__uint_as_float(key_bits(kj)) - lse_t) : 0.f;
+        };
+        if (lists) {
+            for (int e0 = w * 32 * SEL_LOADS; e0 < S * K_REG; e0 += WARPS * 32 * SEL_LOADS) {
+                uint2 ce[SEL_LOADS];
+                bool in[SEL_LOADS];
+#pragma unroll
+                for (int q = 0; q < SEL_LOADS; ++q) {
+                    const int e = e0 + q * 32 + lane;
+                    in[q] = e < S * K_REG;
+                    ce[q] = make_uint2(0u, 0u);
+                    if (in[q]) ce[q] = p.cand[(static_cast<long long>(slot0 + e / K_REG) * BM + r) * K_REG + e % K_REG];
+                }
+                append(ce, in);
+            }
+        } else {
+            for (int s0 = 0; s0 < S; s0 += 32 * WARPS) {
+                const int mine = s0 + lane * WARPS + w;
+                const int cn_mine = mine < S ? p.cand_n[static_cast<long long>(slot0 + mine) * BM + r] : 0;
+                for (int j = 0; j < 32 && s0 + j * WARPS + w < S; ++j) {
+                    const int cn = __shfl_sync(0xffffffffu, cn_mine, j);
+                    const uint2* list = p.cand + (static_cast<long long>(slot0 + s0 + j * WARPS + w) * BM + r) * p.cap;
+                    for (int e0 = 0; e0 < cn; e0 += 32 * SEL_LOADS) {
+                        uint2 ce[SEL_LOADS];
+                        bool in[SEL_LOADS];
+#pragma unroll
+                        for (int q = 0; q < SEL_LOADS; ++q) {
+                            const int e = e0 + q * 32 + lane;
+                            in[q] = e < cn;
+                            ce[q] = make_uint2(0u, 0u);
+                            if (in[q]) ce[q] = list[e];
+                        }
+                        append(ce, in);
+                    }
+                }
+            }
         }
-        __syncwarp();
+        // Rank what is left: every candidate counts those above it. Beyond 128 a pool is cut to K first.
+        if (n > K && n > 128) {
+            cut_to_best(pool, n, K, lane);
+            n = K;
+        }
+        if (lane == 0) pool_n[warp] = n;
+        for (int j = tid; j < K; j += WARPS * 32) {           // cannot stay for K <= V; keeps ids in range
+            sel_tok[rib][j] = 0;
+            sel_q[rib][j] = 0.f;
+        }
+        sync_row();
+        for (int e = lane; e < n; e += 32) {
+            const unsigned long long v = pool[e];
+            int rank = 0;
+            for (int w2 = 0; w2 < WARPS; ++w2) {
+                const unsigned long long* other = pools[rib * WARPS + w2];
+                const int n2 = pool_n[rib * WARPS + w2];
+                for (int i = 0; i < n2; ++i) rank += other[i] > v ? 1 : 0;
+            }
+            if (rank < K) {
+                sel_tok[rib][rank] = static_cast<int>(~static_cast<uint32_t>(v));
+                sel_q[rib][rank] = expf(__uint_as_float(key_bits(static_cast<uint32_t>(v >> 32))) - lse_t);
+            }
+        }
+        sync_row();
         int n_sel = K;
         if (p.top_p > 0.f) {
             // Top-P: a token belongs to Omega_hat while the probability of those before it is <= P
-            int n = 0;
-            if (lane == 0) {
+            if (tid == 0) {
+                int taken = 0;
                 float cum = 0.f;
                 for (int j = 0; j < K; ++j) {
                     if (cum > p.top_p) {
-                        sel_tok[wib][j] = -1;
-                        sel_q[wib][j] = 0.f;
+                        sel_tok[rib][j] = -1;
+                        sel_q[rib][j] = 0.f;
                     } else {
-                        ++n;
+                        ++taken;
                     }
-                    cum += sel_q[wib][j];
+                    cum += sel_q[rib][j];
                 }
-                if (!(cum > p.top_p)) n = -n;      // all K tokens taken and P still not exceeded: the cap cut the prefix
+                if (!(cum > p.top_p)) taken = -taken;      // all K tokens taken and P still not exceeded: the cap cut the prefix
+                n_sel = taken;
             }
-            __syncwarp();
-            n_sel = __shfl_sync(0xffffffffu, n, 0);
+            sync_row();
         }
-        for (int j = lane; j < K; j += 32) {
-            p.idx_out[ro + j] = sel_tok[wib][j];
-            p.q_out[ro + j] = sel_q[wib][j];
+        for (int j = tid; j < K; j += WARPS * 32) {
+            p.idx_out[static_cast<long long>(row) * p.out_pitch + j] = sel_tok[rib][j];
+            p.q_out[static_cast<long long>(row) * p.out_pitch + j] = sel_q[rib][j];
         }
-        if (lane == 0 && p.n_out) p.n_out[row] = n_sel;
+        if (tid == 0 && p.n_out) p.n_out[row] = n_sel;
     } else {
-        for (int j = lane; j < K; j += 32) {
-            sel_tok[wib][j] = p.idx_in[ro + j];
-            sel_q[wib][j] = p.q_in[ro + j];
+        for (int j = tid; j < K; j += WARPS * 32) {
+            sel_tok[rib][j] = p.idx_in[ro + j];
+            sel_q[rib][j] = p.q_in[ro + j];
         }
-        if (lane == 0 && p.n_out) p.n_out[row] = K;
+        if (tid == 0 && p.n_out) p.n_out[row] = K;
+        sync_row();
     }
-    __syncwarp();
+    if (p.ref2 != nullptr && w == WARPS - 1) {
+        const int tok = sel_tok[rib][0];
+        const __nv_bfloat16* hrow = p.H_d + static_cast<long long>(row) * p.d;
+        const __nv_bfloat16* wrow = p.W + static_cast<long long>(tok < 0 || tok >= p.V ? 0 : tok) * p.d;
+        float acc = 0.f;
+#pragma unroll 4
+        for (int k0 = lane * 8; k0 < p.d; k0 += 256) {
+            const uint4 hv = *reinterpret_cast<const uint4*>(hrow + k0);
+            const uint4 wv = *reinterpret_cast<const uint4*>(wrow + k0);
+            const __nv_bfloat162* hp = reinterpret_cast<const __nv_bfloat162*>(&hv);
+            const __nv_bfloat162* wp = reinterpret_cast<const __nv_bfloat162*>(&wv);
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const float2 a2 = __bfloat1622float2(hp[t]);
+                const float2 b2 = __bfloat1622float2(wp[t]);
+                acc = fmaf(a2.x, b2.x, acc);
+                acc = fmaf(a2.y, b2.y, acc);
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (lane == 0) p.ref2[row] = fmaf(acc, LOG2E, 64.f);
+    }
+    if (p.sidx == nullptr) return;
     // the same set in increasing token id (entries cut by Top-P go to the end as INT_MAX / 0)
-    for (int j = lane; j < K; j += 32) {
-        const int tj = sel_tok[wib][j] < 0 ? INT_MAX : sel_tok[wib][j];
+    for (int j = tid; j < K; j += WARPS * 32) {
+        const int tj = sel_tok[rib][j] < 0 ? INT_MAX : sel_tok[rib][j];
         int rank = 0;
         for (int i = 0; i < K; ++i) {
-            const int ti = sel_tok[wib][i] < 0 ? INT_MAX : sel_tok[wib][i];
+            const int ti = sel_tok[rib][i] < 0 ? INT_MAX : sel_tok[rib][i];
             rank += (ti < tj || (ti == tj && i < j)) ? 1 : 0;
         }
         p.sidx[ro + rank] = tj;
-        p.sq[ro + rank] = tj == INT_MAX ? 0.f : sel_q[wib][j];
+        p.sq[ro + rank] = tj == INT_MAX ? 0.f : sel_q[rib][j];
     }
 }
 
@@ -1595,9 +1661,11 @@ struct LossPatchParams {
     float* coef_out;       // [N] g S_q e^(m_spill - lse_d)
     __nv_bfloat16* P;      // spill of the chunk [rows, p_pitch]
     long long p_pitch;
+    const unsigned int* gate;
 };
 
 __global__ void __launch_bounds__(256) loss_patch_kernel(const __grid_constant__ LossPatchParams p) {
+    if (p.gate != nullptr && *p.gate == 0u) return;
     const int lane = threadIdx.x & 31;
     const int local = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (local >= p.rows) return;
@@ -1647,8 +1715,8 @@ __global__ void __launch_bounds__(256) ce_kernel(int rows, int row_begin, int d,
                                                  const float* __restrict__ T, const float* __restrict__ lse_d,
                                                  const float* __restrict__ grad_loss, const float* __restrict__ ce_corr,
                                                  float* __restrict__ loss_ce, float* __restrict__ sparse,
-                                                 const unsigned int* __restrict__ only_if_range) {
-    if (only_if_range != nullptr && ((*only_if_range) & 0xffu) != 2u) return;
+                                                 const unsigned int* __restrict__ gate) {
+    if (gate != nullptr && *gate == 0u) return;
     const int lane = threadIdx.x & 31;
     const int local = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (local >= rows) return;
@@ -1704,15 +1772,6 @@ __global__ void wait_expiry_selftest_kernel(unsigned int* status, unsigned long 
     }
 }
 
-// Ends the exact route after a fused call: the range report has been dealt with. Word 2 of the status block
-// records that the route ran (the host-buffer entry then copies dH_d to the host once more).
-__global__ void range_handled_kernel(unsigned int* status) {
-    if (((*status) & 0xffu) == 2u) {
-        *status = 0u;
-        status[2] = 1u;
-    }
-}
-
 // ---------------------------------------------------------------------------------------------
 // bwd_prep: one warp per row. Sorts Omega_hat by token id (the MODE_PROBS epilogue walks the vocabulary in
 // increasing order; entries cut by Top-P carry id -1 and come first) by ranking every entry against the
@@ -1723,9 +1782,7 @@ __global__ void __launch_bounds__(PREP_WARPS * 32) bwd_prep_kernel(int N, int K,
                                                                     const float* __restrict__ lse_d,
                                                                     const float* __restrict__ grad_loss,
                                                                     int* __restrict__ sidx, float* __restrict__ sgq,
-                                                                    float* __restrict__ coef, float* __restrict__ lse2,
-                                                                    const unsigned int* __restrict__ only_if_range) {
-    if (only_if_range != nullptr && ((*only_if_range) & 0xffu) != 2u) return;
+                                                                    float* __restrict__ coef, float* __restrict__ lse2) {
     __shared__ int s_tok[PREP_WARPS][K_CAP];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int row = blockIdx.x * PREP_WARPS + wib;

@@ -1,8 +1,9 @@
-"""The forms of the GEMM kernel at the sizes where they can go wrong: CTA pairs whose last row tile has no partner, output
-tiles cut along the contraction (alone, behind whole rounds, with few rows), against the oracle with the tolerances of
-the parity tests, every buffer between guard bands."""
+"""The forms of the GEMM and selection kernels at the sizes where they can go wrong: CTA pairs whose last row tile has no
+partner, output tiles cut along the contraction (alone, behind whole rounds, with few rows), selections of one and of
+four warps per row, against the oracle with the tolerances of the parity tests, every buffer between guard bands."""
 import numpy as np
 import pytest
+import torch
 
 import hass_inputs as hi
 from parity import compare
@@ -16,6 +17,9 @@ pytestmark = pytest.mark.gpu
     (1537, 200, 3000, 20, False),      # the same with one row in the last tile and a ragged last column tile
     (61, 520, 20000, 10, False),       # one row tile: cut output tiles that keep 61 rows
     (129, 264, 30001, 5, True),        # two row tiles, one row in the second, a ragged contraction
+    (700, 64, 9000, 200, True),        # selection of a large K with one warp per row, which cuts its pool
+    (40, 64, 33000, 40, True),         # the same with four warps per row and buffers of 129 lanes
+    (620, 64, 40000, 16, True),        # one warp per row, K lists whose first entries set the floor
     (1601, 2824, 12000, 10, False),    # whole rounds of output tiles, then a cut rest, d not a multiple of 256
 ])
 def test_pairs_and_cut_tiles(N, d, V, K, fp32):
@@ -25,3 +29,23 @@ def test_pairs_and_cut_tiles(N, d, V, K, fp32):
     fused, split = _guarded_fused(inp, K, grad, dH_fp32=fp32)
     print("fused", compare(inp.H_t, inp.H_d[0], inp.W, K, fused, grad_loss=grad, rows=rows))
     print("split", compare(inp.H_t, inp.H_d[0], inp.W, K, split, grad_loss=grad, rows=rows))
+
+
+@pytest.mark.parametrize("value", [3.0, 200.0])
+def test_reference_exponent_far_below_the_row(value):
+    """The target's first token has a low draft logit (-60): draft rows whose largest logit is 60 above it stay within the
+    spill's range, rows 260 above it are redone by the second pass; both match the oracle."""
+    N, d, V, K = 200, 64, 3000, 4
+    inp = hi.make_custom(N, d, V, K, seed=9, sigma_w=0.05)
+    W = inp.W.clone()
+    W[:, 0] = 0
+    W[5, 0] = 1.0                       # token 5: the target's favourite, and far down in the draft
+    W[2000, 1] = 0.5
+    H_t, H_d = inp.H_t.clone(), inp.H_d[0].clone()
+    H_t[:, 0] = 20.0
+    H_d[:, 0] = -60.0
+    H_d[::3, 1] = 2.0 * value           # token 2000 at +value on every third row
+    case = hi.Inputs(**{**inp.__dict__, "H_t": H_t, "H_d": [H_d], "W": W})
+    fused, split = _guarded_fused(case, K, None)
+    print("fused", compare(H_t, H_d, W, K, fused))
+    print("split", compare(H_t, H_d, W, K, split))
