@@ -586,6 +586,7 @@ static int forward_impl(bool with_target, const void* H_t, const void* H_d, cons
     if (rc != HASS_OK) return rc;
     log_schedule(with_target ? "fwd stats" : "fwd stats (draft)", p.sched);
     p.spill_begin = INT_MAX;
+    p.z_begin = INT_MAX;
     p.a_row_offset = 0;
     p.row_global_offset = 0;
     p.rows_valid = static_cast<int>(N);
@@ -824,6 +825,7 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
         p.row_tiles0 = tiles;
         p.topk_row_tiles = with_target ? (bidir ? 2 * tiles : tiles) : 0;
         p.spill_begin = with_target ? tiles : 0;
+        p.z_begin = INT_MAX;
         p.a_row_offset = t0 * BM;
         p.row_global_offset = t0 * BM;
         p.rows_valid = static_cast<int>(N);
@@ -983,6 +985,147 @@ struct ChunkPipe {
     cudaEvent_t next() { return used < n_events ? events[used++] : nullptr; }
 };
 
+// Rows [row, row + rows) of H_t, then of H_d, on the inbound copy stream; `st` waits for H_t's here and for H_d's here or,
+// with ev_d, where the caller makes it.
+static int pipe_in(ChunkPipe* pipe, const void* H_t, const void* H_d, size_t row, size_t rows, cudaStream_t st,
+                   cudaEvent_t* ev_d = nullptr) {
+    const size_t off = row * pipe->in_row_bytes, bytes = rows * pipe->in_row_bytes;
+    cudaEvent_t t = pipe->next(), d = pipe->next();
+    if (!t || !d) return HASS_ERR_UNSUPPORTED;
+    bool ok = cudaMemcpyAsync(const_cast<uint8_t*>(static_cast<const uint8_t*>(H_t)) + off, pipe->Ht_host + off, bytes,
+                              cudaMemcpyHostToDevice, pipe->h2d) == cudaSuccess;
+    ok = ok && cudaEventRecord(t, pipe->h2d) == cudaSuccess;
+    ok = ok && cudaMemcpyAsync(const_cast<uint8_t*>(static_cast<const uint8_t*>(H_d)) + off, pipe->Hd_host + off, bytes,
+                               cudaMemcpyHostToDevice, pipe->h2d) == cudaSuccess;
+    ok = ok && cudaEventRecord(d, pipe->h2d) == cudaSuccess;
+    ok = ok && cudaStreamWaitEvent(st, t, 0) == cudaSuccess;
+    if (ev_d)
+        *ev_d = d;
+    else
+        ok = ok && cudaStreamWaitEvent(st, d, 0) == cudaSuccess;
+    if (!ok) {
+        cudaGetLastError();
+        return HASS_ERR_CUDA;
+    }
+    return HASS_OK;
+}
+
+// Rows [row, row + rows) of dH_d, as `st` leaves them here, on the outbound copy stream.
+static int pipe_out(ChunkPipe* pipe, const void* dH_d, size_t row, size_t rows, cudaStream_t st) {
+    cudaEvent_t ev = pipe->next();
+    if (!ev) return HASS_ERR_UNSUPPORTED;
+    const size_t off = row * pipe->out_row_bytes;
+    bool ok = cudaEventRecord(ev, st) == cudaSuccess;
+    ok = ok && cudaStreamWaitEvent(pipe->d2h, ev, 0) == cudaSuccess;
+    ok = ok && cudaMemcpyAsync(pipe->dH_host + off, static_cast<const uint8_t*>(dH_d) + off, rows * pipe->out_row_bytes,
+                               cudaMemcpyDeviceToHost, pipe->d2h) == cudaSuccess;
+    if (!ok) {
+        cudaGetLastError();
+        return HASS_ERR_CUDA;
+    }
+    return HASS_OK;
+}
+
+// Rows of one call up to which the draft logits go through the workspace in fp32 (narrow_impl): two rows of 128-row bf16
+// scratch hold one of them. Up to here a call is bound by reading W, which this route does twice (both sweeps in one
+// launch, then the second GEMM) instead of three times, with no range condition and so no second pass: 61 rows x 4096 x
+// 32000 211 -> 147 us, 64 rows x 256 x 1024 67 -> 46 us. Beyond, the fp32 logits would not fit a workspace of one row tile.
+constexpr int kNarrowRows = BM / 2;
+
+static int narrow_impl(bool with_target, const void* H_t, const void* H_d, const void* W, int N, long long d, long long V,
+                       int K, const float* grad_loss, const int* idx_in, const float* q_in, float* loss, int* idx_out,
+                       float* q_out, float* lse_t, float* lse_d, void* dH_d, int dH_dtype, uint8_t* ws, const Layout& L,
+                       const PartRoom& part, int sms, cudaStream_t st, float top_p, int* topk_n) {
+    const int CT = ceil_div(V, BN), DT = ceil_div(d, BN);
+    unsigned int* status = reinterpret_cast<unsigned int*>(ws + L.status);
+    float* z = reinterpret_cast<float*>(ws + L.scratch);
+    // (1) target and draft rows in one sweep: statistics, candidates, the draft's logits
+    GemmParams p;
+    std::memset(&p, 0, sizeof(p));
+    p.row_tiles = with_target ? 2 : 1;
+    int rc = plan_launch(p.row_tiles, CT, sms, L.slot_cap, &p.sched);
+    if (rc != HASS_OK) return rc;
+    log_schedule("narrow sweep", p.sched);
+    rc = make_tmap(&p.tmA1, H_d, N, d, d, BK, BM);
+    if (rc == HASS_OK) rc = make_tmap(&p.tmA0, with_target ? H_t : H_d, N, d, d, BK, BM);
+    if (rc == HASS_OK) rc = make_tmap(&p.tmB, W, V, d, d, BK, BN / p.sched.pair);
+    if (rc != HASS_OK) return rc;
+    p.row_tiles0 = 1;
+    p.topk_row_tiles = with_target ? 1 : 0;
+    p.spill_begin = INT_MAX;
+    p.z_begin = p.row_tiles - 1;
+    p.z_rows = N;
+    p.z_out = z;
+    p.z_pitch = L.p_pitch;
+    p.rows_valid = N;
+    p.n_cols = static_cast<int>(V);
+    p.col_tiles = CT;
+    p.k_blocks = ceil_div(d, BK);
+    p.K = K;
+    p.cap = topk_cap(K);
+    p.part_m = reinterpret_cast<float*>(ws + L.part_m);
+    p.part_s = reinterpret_cast<float*>(ws + L.part_s);
+    p.cand = reinterpret_cast<uint2*>(ws + L.cand_v);
+    p.cand_n = reinterpret_cast<int*>(ws + L.cand_i);
+    p.thr_share = reinterpret_cast<unsigned int*>(ws + L.thr_share);
+    p.status = status;
+    rc = clear_status(ws, L, with_target ? p.sched.total_slots : 0, st);
+    if (rc != HASS_OK) return rc;
+    rc = launch_gemm<MODE_STATS>(p, st, with_target ? KIND_STATS : KIND_STATS_DRAFT);
+    if (rc != HASS_OK) return rc;
+    // (2) Omega_hat
+    if (with_target) {
+        SelectParams sp = select_params(p, 0, 0, N, idx_out, q_out, K, lse_t);
+        sp.n_out = topk_n;
+        sp.top_p = top_p;
+        rc = launch_select(sp, sms, st);
+        if (rc != HASS_OK) return rc;
+    }
+    // (3) lse_d, loss, dz_d
+    DzParams z_params;
+    std::memset(&z_params, 0, sizeof(z_params));
+    z_params.sched = p.sched;
+    z_params.first_tile = p.z_begin;
+    z_params.K = K;
+    z_params.V = static_cast<int>(V);
+    z_params.part_m = p.part_m;
+    z_params.part_s = p.part_s;
+    z_params.idx = with_target ? idx_out : idx_in;
+    z_params.q = with_target ? q_out : q_in;
+    z_params.grad_loss = grad_loss;
+    z_params.loss = loss;
+    z_params.lse_d = lse_d;
+    z_params.z = z;
+    z_params.pitch = L.p_pitch;
+    {
+        KernelTimer timer(KIND_FINALIZE, st);
+        dz_kernel<<<N, DZ_THREADS, 0, st>>>(z_params);
+    }
+    g_launches.fetch_add(1);
+    if (cudaGetLastError() != cudaSuccess) return HASS_ERR_CUDA;
+    // (4) dH_d = dz_d W
+    GemmParams o;
+    std::memset(&o, 0, sizeof(o));
+    rc = make_tmap(&o.tmA0, z, N, V, 2 * L.p_pitch, BK, BM);
+    if (rc == HASS_OK) rc = make_tmap(&o.tmB, W, V, d, d, 64, BK);
+    if (rc != HASS_OK) return rc;
+    o.tmA1 = o.tmA0;
+    o.row_tiles = 1;
+    o.row_tiles0 = 1;
+    o.spill_begin = INT_MAX;
+    o.rows_valid = N;
+    o.n_cols = static_cast<int>(d);
+    o.col_tiles = DT;
+    o.k_blocks = ceil_div(V, BK);
+    o.K = K;
+    o.out = dH_d;
+    o.out_fp32 = dH_dtype == HASS_FP32 ? 1 : 0;
+    o.out_align32 = ((reinterpret_cast<uintptr_t>(dH_d) | static_cast<uintptr_t>(d * (dH_dtype == HASS_FP32 ? 4 : 2))) & 31u) == 0 ? 1 : 0;
+    o.out_pitch = d;
+    o.status = status;
+    return launch_out(o, part, sms, st);
+}
+
 static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const void* W, long long N, long long d,
                        long long V, int K, const float* grad_loss, const int* idx_in, const float* q_in, float* loss,
                        int* idx_out, float* q_out, float* lse_t, float* lse_d, void* dH_d, int dH_dtype,
@@ -1016,6 +1159,16 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
     float* coef = reinterpret_cast<float*>(ws + L.coef);
     float* capz = reinterpret_cast<float*>(ws + L.capz);
     float* ref2 = reinterpret_cast<float*>(ws + L.lse2);
+    if (N <= kNarrowRows) {
+        if (pipe) {
+            rc = pipe_in(pipe, H_t, H_d, 0, static_cast<size_t>(N), st);
+            if (rc != HASS_OK) return rc;
+        }
+        rc = narrow_impl(with_target, H_t, H_d, W, static_cast<int>(N), d, V, K, grad_loss, idx_in, q_in, loss, idx_out, q_out,
+                         lse_t, lse_d, dH_d, dH_dtype, ws, L, part, di.sms, st, top_p, topk_n);
+        if (rc != HASS_OK || !pipe) return rc;
+        return pipe_out(pipe, dH_d, 0, static_cast<size_t>(N), st);
+    }
     __nv_bfloat16* P = reinterpret_cast<__nv_bfloat16*>(ws + L.scratch);
     unsigned int* status = reinterpret_cast<unsigned int*>(ws + L.status);
     unsigned int* zmax = reinterpret_cast<unsigned int*>(ws + L.zmax);
@@ -1068,22 +1221,8 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
             if (!retry) {
                 cudaEvent_t ev_d = nullptr;
                 if (pipe) {
-                    // this chunk's rows of H_t, then of H_d, on the inbound copy stream; the sweeps wait for them
-                    const size_t off = static_cast<size_t>(t0) * BM * pipe->in_row_bytes, bytes = static_cast<size_t>(rows) * pipe->in_row_bytes;
-                    cudaEvent_t ev_t = pipe->next();
-                    ev_d = pipe->next();
-                    if (!ev_t || !ev_d) return HASS_ERR_UNSUPPORTED;
-                    bool ok = cudaMemcpyAsync(const_cast<uint8_t*>(static_cast<const uint8_t*>(H_t)) + off, pipe->Ht_host + off, bytes,
-                                              cudaMemcpyHostToDevice, pipe->h2d) == cudaSuccess;
-                    ok = ok && cudaEventRecord(ev_t, pipe->h2d) == cudaSuccess;
-                    ok = ok && cudaMemcpyAsync(const_cast<uint8_t*>(static_cast<const uint8_t*>(H_d)) + off, pipe->Hd_host + off, bytes,
-                                               cudaMemcpyHostToDevice, pipe->h2d) == cudaSuccess;
-                    ok = ok && cudaEventRecord(ev_d, pipe->h2d) == cudaSuccess;
-                    ok = ok && cudaStreamWaitEvent(st, ev_t, 0) == cudaSuccess;
-                    if (!ok) {
-                        cudaGetLastError();
-                        return HASS_ERR_CUDA;
-                    }
+                    rc = pipe_in(pipe, H_t, H_d, static_cast<size_t>(t0) * BM, static_cast<size_t>(rows), st, &ev_d);
+                    if (rc != HASS_OK) return rc;
                 }
                 rc = clear_status(ws, L, with_target ? p.sched.total_slots : 0, st, t0 > 0);
                 if (rc != HASS_OK) return rc;
@@ -1094,6 +1233,7 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
                     t.tmA1 = tmHt;
                     t.topk_row_tiles = tiles;
                     t.spill_begin = INT_MAX;
+                    t.z_begin = INT_MAX;
                     rc = launch_gemm<MODE_STATS>(t, st);
                     if (rc != HASS_OK) return rc;
                 }
@@ -1187,18 +1327,8 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
             rc = launch_out(o, part, di.sms, st);
             if (rc != HASS_OK) return rc;
             if (pipe && !retry) {
-                // the chunk's dH_d rows on the outbound copy stream
-                const size_t off = static_cast<size_t>(t0) * BM * pipe->out_row_bytes, bytes = static_cast<size_t>(rows) * pipe->out_row_bytes;
-                cudaEvent_t ev_o = pipe->next();
-                if (!ev_o) return HASS_ERR_UNSUPPORTED;
-                bool ok = cudaEventRecord(ev_o, st) == cudaSuccess;
-                ok = ok && cudaStreamWaitEvent(pipe->d2h, ev_o, 0) == cudaSuccess;
-                ok = ok && cudaMemcpyAsync(pipe->dH_host + off, static_cast<const uint8_t*>(dH_d) + off, bytes, cudaMemcpyDeviceToHost,
-                                           pipe->d2h) == cudaSuccess;
-                if (!ok) {
-                    cudaGetLastError();
-                    return HASS_ERR_CUDA;
-                }
+                rc = pipe_out(pipe, dH_d, static_cast<size_t>(t0) * BM, static_cast<size_t>(rows), st);
+                if (rc != HASS_OK) return rc;
             }
         }
         return HASS_OK;
@@ -1247,6 +1377,7 @@ static int forward2_impl(bool with_target, const void* H_t, const void* H_d, con
     p.row_tiles = RT;
     p.row_tiles0 = RT;
     p.spill_begin = INT_MAX;
+    p.z_begin = INT_MAX;
     p.rows_valid = static_cast<int>(N);
     p.n_cols = static_cast<int>(V);
     p.col_tiles = CT;
@@ -1350,6 +1481,7 @@ static int normed_impl(const void* H_t, const void* H_d, const void* W, long lon
     p.row_tiles0 = RT;
     p.topk_row_tiles = RT;
     p.spill_begin = INT_MAX;
+    p.z_begin = INT_MAX;
     p.rows_valid = static_cast<int>(N);
     p.n_cols = static_cast<int>(V);
     p.col_tiles = CT;

@@ -113,6 +113,11 @@ struct GemmParams {
     __nv_bfloat16* P;      // [chunk rows, p_pitch]
     __nv_bfloat16* Pt;     // [chunk rows, p_pitch] spill of the target tiles, or nullptr
     long long p_pitch;
+    // MODE_STATS: row tiles from z_begin on write their logits in fp32 to z_out [rows of these tiles, z_pitch]; the last
+    // z_rows of them are valid (INT_MAX: none)
+    int z_begin, z_rows;
+    float* z_out;
+    long long z_pitch;
     // MODE_OUT. With sparse != nullptr the epilogue computes coef[row] * acc - sparse[local row, :] (row scale
     // and the Omega_hat term of dz_d W, precomputed by finalize); with coef alone coef[row] * acc; with neither
     // it stores the accumulator.
@@ -552,6 +557,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                 cz = p.cap_z + static_cast<long long>(g_row) * p.K;
                 nxt = si[0];
             }
+            float* zrow = nullptr;
+            if (HAS_TOPK && tile_ok && rt >= p.z_begin && (rt - p.z_begin) * BM + r_local < p.z_rows)
+                zrow = p.z_out + static_cast<long long>((rt - p.z_begin) * BM + r_local) * p.z_pitch;
             const int t0 = first_tile(rt, ln);
             const int nt = (p.col_tiles - ln + S - 1) / S;
             for (int t = t0; t < nt; ++t) {
@@ -690,6 +698,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
 #pragma unroll
                             for (int j = 0; j < 32; ++j)
                                 if (col0 + j >= p.n_cols) r[j] = __float_as_uint(-INFINITY);
+                        }
+                        if (HAS_TOPK && zrow != nullptr) {
+#pragma unroll
+                            for (int g8 = 0; g8 < 4; ++g8)
+                                st_global_v8(zrow + col0 + 8 * g8, r[8 * g8], r[8 * g8 + 1], r[8 * g8 + 2], r[8 * g8 + 3],
+                                             r[8 * g8 + 4], r[8 * g8 + 5], r[8 * g8 + 6], r[8 * g8 + 7]);
                         }
                         if (CAPTURE) {
                             // draft logits at the row's Omega_hat, straight from the fp32 accumulator
@@ -1705,6 +1719,97 @@ __global__ void __launch_bounds__(256) loss_patch_kernel(const __grid_constant__
             if (tok != INT_MAX) prow[tok] = __float2bfloat16_rn(__bfloat162float(prow[tok]) - p.sq[ro + j] * inv);
         }
     }
+}
+
+// ---------------------------------------------------------------------------------------------
+// dz_kernel: one block per row, after a sweep that left the draft logits of few rows in fp32. Merges the draft's partial
+// statistics into lse_d, evaluates Eq. 1 from the logits at Omega_hat, and turns the row into
+// dz_d(v) = g (S_q p(v) - q(v) [v in Omega_hat]) in bf16, in place: the bf16 row begins where the fp32 row did. Every step
+// reads a piece twice as long as the one it writes, and a piece is written after all threads have read theirs.
+// Bound by the latency of one pass over a row of 4 V bytes: DZ_THREADS threads with DZ_LOADS 16-byte loads each in flight.
+constexpr int DZ_THREADS = 1024;
+constexpr int DZ_LOADS = 4;
+
+struct DzParams {
+    Schedule sched;        // schedule of the sweep
+    int first_tile;        // its row tile of the draft rows
+    int K, V;
+    const float* part_m;
+    const float* part_s;
+    const int* idx;        // [N, K] Omega_hat; entries < 0 carry q = 0
+    const float* q;
+    const float* grad_loss;
+    float* loss;
+    float* lse_d;
+    float* z;              // [N, pitch] in: logits (columns up to the pitch readable); out: bf16 [N, 2 pitch]
+    long long pitch;       // a multiple of 256
+};
+
+__global__ void __launch_bounds__(DZ_THREADS) dz_kernel(const __grid_constant__ DzParams p) {
+    __shared__ int sh_tok[K_CAP];
+    __shared__ float sh_q[K_CAP];
+    __shared__ float sh_z[K_CAP];
+    __shared__ float sh_sum[2];           // lse_d, S_q
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int row = blockIdx.x;
+    const int K = p.K;
+    float* zrow = p.z + static_cast<long long>(row) * p.pitch;
+    __nv_bfloat16* drow = reinterpret_cast<__nv_bfloat16*>(zrow);
+    if (tid < K) {
+        const int tok = p.idx[static_cast<long long>(row) * K + tid];
+        sh_tok[tid] = tok < p.V ? tok : -1;
+        sh_q[tid] = p.q[static_cast<long long>(row) * K + tid];
+        sh_z[tid] = tok >= 0 && tok < p.V ? zrow[tok] : 0.f;
+    }
+    if (warp == DZ_THREADS / 32 - 1) {
+        int slot0, S;
+        find_slots(p.sched, p.first_tile, slot0, S);
+        const float lse = warp_lse(p.part_m, p.part_s, slot0, S, row, lane);
+        if (lane == 0) sh_sum[0] = lse;
+    }
+    __syncthreads();
+    const float g = p.grad_loss ? p.grad_loss[row] : 1.f;
+    const float lse_d = sh_sum[0];
+    if (warp == 0) {
+        float S_q = 0.f, loss = 0.f;
+        for (int j = lane; j < K; j += 32) {
+            if (sh_tok[j] < 0) continue;
+            S_q += sh_q[j];
+            loss += sh_q[j] * (lse_d - sh_z[j]);      // -q log p,  log p = z_d - lse_d
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            S_q += __shfl_xor_sync(0xffffffffu, S_q, o);
+            loss += __shfl_xor_sync(0xffffffffu, loss, o);
+        }
+        if (lane == 0) {
+            sh_sum[1] = S_q;
+            p.loss[row] = loss;
+            p.lse_d[row] = lse_d;
+        }
+    }
+    __syncthreads();
+    const float S_q = sh_sum[1], c = g * S_q, shift = -lse_d * LOG2E;
+    for (long long c0 = 0; c0 < p.pitch; c0 += DZ_LOADS * DZ_THREADS * 4) {
+        float4 v[DZ_LOADS];
+#pragma unroll
+        for (int u = 0; u < DZ_LOADS; ++u) {
+            const long long at = c0 + (u * DZ_THREADS + tid) * 4;
+            if (at < p.pitch) v[u] = *reinterpret_cast<const float4*>(zrow + at);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < DZ_LOADS; ++u) {
+            const long long at = c0 + (u * DZ_THREADS + tid) * 4;
+            if (at < p.pitch)
+                *reinterpret_cast<uint2*>(drow + at) =
+                    make_uint2(pack_bf16x2(c * ex2(fmaf(v[u].x, LOG2E, shift)), c * ex2(fmaf(v[u].y, LOG2E, shift))),
+                               pack_bf16x2(c * ex2(fmaf(v[u].z, LOG2E, shift)), c * ex2(fmaf(v[u].w, LOG2E, shift))));
+        }
+    }
+    __syncthreads();
+    if (tid < K && sh_tok[tid] >= 0)
+        drow[sh_tok[tid]] = __float2bfloat16_rn(c * ex2(fmaf(sh_z[tid], LOG2E, shift)) - g * sh_q[tid]);
 }
 
 // ---------------------------------------------------------------------------------------------
