@@ -163,6 +163,7 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
 constexpr int CAND_CAP_MAX = 800;                 // largest buffer: K = 256
 constexpr int CAND_REGS = CAND_CAP_MAX / 32;      // entries per lane during a compaction of the largest buffer
 constexpr int CAND_REGS_SMALL = 13;               // ... of a buffer of up to 416 entries (K <= 128)
+constexpr int CAND_REGS_TINY = 7;                 // ... of up to 224 entries (K <= 64)
 constexpr int CAND_SLACK = 32;                    // a compaction may leave up to K + CAND_SLACK entries
 
 // K entries kept + room for max(2K, 96) new ones between compactions (each compaction then multiplies the
@@ -178,46 +179,60 @@ __device__ __forceinline__ uint32_t key_bits(uint32_t key) {
     return (key & 0x80000000u) ? (key ^ 0x80000000u) : ~key;
 }
 
-// Warp-collective: compacts the buffer `buf` holding n >= K entries, in place, keeping their order, and
-// returns the bit pattern of the new admission threshold (only logits strictly above it can still belong to
-// the row's K best); n_out = entries left. The K-th largest key is searched bit by bit from the top. After
-// the upper 16 bits (bf16 resolution) the search stops if at most K + CAND_SLACK entries reach the prefix
-// found so far: all of them are kept and the threshold is the value just below the prefix. Otherwise the
-// search runs to the last bit, exactly K entries are kept (among logits equal to the K-th, the lowest token
-// ids) and the threshold is the K-th largest logit itself.
+// Warp-collective: the n entries of a buffer of `cap`, entry e = lane + 32 t in v[t].
 template <int REGS>
-__device__ __forceinline__ uint32_t compact_candidates(uint2* buf, int n, int K, int cap, int lane, int& n_out) {
-    constexpr int CAND_REGS = REGS;
-    uint32_t key[CAND_REGS];
-    int id[CAND_REGS];
+__device__ __forceinline__ void load_candidates(const uint2* buf, int n, int cap, int lane, uint2 (&v)[REGS]) {
     const int groups = cap >> 5;
 #pragma unroll
-    for (int t = 0; t < CAND_REGS; ++t) {
-        key[t] = 0u;
-        id[t] = -1;
+    for (int t = 0; t < REGS; ++t) {
         const int e = lane + 32 * t;
-        if (t < groups && e < n) {
-            const uint2 v = __ldcg(buf + e);
-            key[t] = ordered_key(v.x);
-            id[t] = static_cast<int>(v.y);
-        }
+        v[t] = make_uint2(0u, 0u);
+        if (t < groups && e < n) v[t] = __ldcg(buf + e);
     }
-    // largest T with at least K keys >= T, bit by bit; cT = number of keys >= T
-    uint32_t T = 0u;
-    int cT = n;
+}
+
+// Warp-collective: compacts the buffer `buf`, whose n > K + CAND_SLACK entries are in v, in place, keeping their order, and
+// returns the bit pattern of the new admission threshold (only logits strictly above it can still belong to
+// the row's K best); n_out = entries left. The bits of the K-th largest key are searched from the highest one in which the
+// keys differ, two per step (three counts, whose warp sums overlap), until at most K + CAND_SLACK entries reach the
+// prefix found so far: all of them are kept and the threshold is the value just below the prefix. If the search has to run
+// to the last bit (equal logits), exactly K entries are kept (among logits equal to the K-th, the lowest token
+// ids) and the threshold is the K-th largest logit itself.
+template <int REGS>
+__device__ __forceinline__ uint32_t compact_candidates(uint2* buf, const uint2 (&v)[REGS], int n, int K, int cap, int lane, int& n_out) {
+    uint32_t key[REGS];
+    const int groups = cap >> 5;
+    uint32_t hi = 0u, lo = 0xffffffffu;
+#pragma unroll
+    for (int t = 0; t < REGS; ++t) {
+        const bool used = t < groups && lane + 32 * t < n;
+        key[t] = used ? ordered_key(v[t].x) : 0u;
+        hi = max(hi, key[t]);
+        lo = used ? min(lo, key[t]) : lo;
+    }
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    // largest T with at least K keys >= T; the bits above `bit` are common to all keys
+    int bit = 32 - __clz(hi ^ lo);      // bits left to find
+    bit += bit & 1;
+    uint32_t T = bit < 32 ? (hi >> bit) << bit : 0u;
     bool exact = true;
 #pragma unroll 1
-    for (int bit = 31; bit >= 0; --bit) {
-        const uint32_t cand = T | (1u << bit);
-        int c = 0;
+    for (bit -= 2; bit >= 0; bit -= 2) {
+        const uint32_t T1 = T | (1u << bit), T2 = T | (2u << bit), T3 = T | (3u << bit);
+        int c1 = 0, c2 = 0, c3 = 0;
 #pragma unroll
-        for (int t = 0; t < CAND_REGS; ++t) c += (key[t] >= cand) ? 1 : 0;
-        c = __reduce_add_sync(0xffffffffu, c);
-        if (c >= K) {
-            T = cand;
-            cT = c;
+        for (int t = 0; t < REGS; ++t) {
+            c1 += (key[t] >= T1) ? 1 : 0;
+            c2 += (key[t] >= T2) ? 1 : 0;
+            c3 += (key[t] >= T3) ? 1 : 0;
         }
-        if (bit == 16 && cT <= K + CAND_SLACK) {
+        c1 = __reduce_add_sync(0xffffffffu, c1);
+        c2 = __reduce_add_sync(0xffffffffu, c2);
+        c3 = __reduce_add_sync(0xffffffffu, c3);
+        const int c = c3 >= K ? c3 : c2 >= K ? c2 : c1 >= K ? c1 : INT_MAX;
+        T = c3 >= K ? T3 : c2 >= K ? T2 : c1 >= K ? T1 : T;
+        if (c <= K + CAND_SLACK && bit > 0) {
             exact = false;
             break;
         }
@@ -225,39 +240,79 @@ __device__ __forceinline__ uint32_t compact_candidates(uint2* buf, int n, int K,
     const uint32_t lt_mask = (1u << lane) - 1u;
     int out = 0;
     if (!exact) {
-        // keep every entry that reaches the 16-bit prefix
+        // keep every entry that reaches the prefix
 #pragma unroll
-        for (int t = 0; t < CAND_REGS; ++t) {
+        for (int t = 0; t < REGS; ++t) {
             if (t < groups) {
                 const bool keep = key[t] >= T;
                 const uint32_t km = __ballot_sync(0xffffffffu, keep);
-                if (keep) buf[out + __popc(km & lt_mask)] = make_uint2(key_bits(key[t]), static_cast<uint32_t>(id[t]));
+                if (keep) buf[out + __popc(km & lt_mask)] = v[t];
                 out += __popc(km);
             }
         }
         n_out = out;
-        return key_bits(T - 1u);      // T >= 2^16 here: at least K keys reach it
+        return key_bits(T - 1u);      // T > 0: fewer than n keys reach it
     }
     int n_gt = 0;
 #pragma unroll
-    for (int t = 0; t < CAND_REGS; ++t) n_gt += (key[t] > T) ? 1 : 0;
+    for (int t = 0; t < REGS; ++t) n_gt += (key[t] > T) ? 1 : 0;
     n_gt = __reduce_add_sync(0xffffffffu, n_gt);
     const int need_eq = K - n_gt;             // >= 1: how many entries equal to the K-th are kept
     int run_eq = 0;
 #pragma unroll
-    for (int t = 0; t < CAND_REGS; ++t) {
+    for (int t = 0; t < REGS; ++t) {
         if (t < groups) {
             const bool eq = key[t] == T;
             const uint32_t em = __ballot_sync(0xffffffffu, eq);
             const bool keep = key[t] > T || (eq && run_eq + __popc(em & lt_mask) < need_eq);
             run_eq += __popc(em);
             const uint32_t km = __ballot_sync(0xffffffffu, keep);
-            if (keep) buf[out + __popc(km & lt_mask)] = make_uint2(key_bits(key[t]), static_cast<uint32_t>(id[t]));
+            if (keep) buf[out + __popc(km & lt_mask)] = v[t];
             out += __popc(km);
         }
     }
     n_out = out;
     return key_bits(T);
+}
+
+// Warp-collective: compacts the buffers of the lanes in `full` (cbuf, cnt: each lane's own) and raises their
+// thresholds. The next buffer's entries are requested before the current one is worked on.
+// A compaction is a chain of latencies (7 k cycles with one bit per step from the top and no load ahead), and while a new
+// row's threshold is still low the sweep waits for it: 2047 rows x 4096 x 32000, sweep with K = 64 546 -> 437 us, K = 100
+// 597 -> 503 us, K = 256 888 -> 728 us (K = 10: 328 us).
+template <int REGS>
+__device__ __forceinline__ void compact_rows(uint32_t full, uint2* cbuf, int& cnt, float& thr_own, int K, int cap, int lane) {
+    auto row = [&](int L, uint2*& buf, int& n) {
+        buf = reinterpret_cast<uint2*>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(cbuf), L));
+        n = __shfl_sync(0xffffffffu, cnt, L);
+    };
+    __syncwarp();
+    int L = __ffs(full) - 1, n;
+    uint2* buf;
+    row(L, buf, n);
+    uint2 v[REGS];
+    load_candidates<REGS>(buf, n, cap, lane, v);
+    while (full) {
+        full &= full - 1u;
+        const int L2 = full ? __ffs(full) - 1 : L;
+        int n2;
+        uint2* buf2;
+        row(L2, buf2, n2);
+        uint2 v2[REGS];
+        load_candidates<REGS>(buf2, full ? n2 : 0, cap, lane, v2);
+        int left = 0;
+        const uint32_t tb = compact_candidates<REGS>(buf, v, n, K, cap, lane, left);
+        if (lane == L) {
+            cnt = left;
+            thr_own = __uint_as_float(tb);
+        }
+        L = L2;
+        n = n2;
+        buf = buf2;
+#pragma unroll
+        for (int t = 0; t < REGS; ++t) v[t] = v2[t];
+    }
+    __syncwarp();
 }
 
 // Bitonic sorting network over 16 registers.
@@ -275,6 +330,28 @@ __device__ __forceinline__ void sort16_descending(float (&v)[16]) {
                     v[l] = (i & k) == 0 ? lo : hi;
                 }
             }
+}
+
+// Histogram of a thread's row in shared memory: bucket b of thread T at word b * 128 + T of `hist` (the thread's own
+// column, no conflicts, no synchronisation). The bucket of x is a non-decreasing function of x.
+constexpr int HIST_BUCKETS = 32;
+__device__ __forceinline__ int hist_bucket(float x, float lo, float inv) {
+    return min(max(__float2int_rz((x - lo) * inv), 0), HIST_BUCKETS - 1);
+}
+__device__ __forceinline__ void hist_clear(uint32_t hist) {
+#pragma unroll
+    for (int b = 0; b < HIST_BUCKETS; ++b) st_shared_b32(hist + b * 512, 0u);
+}
+// the highest bucket that together with those above it holds at least K entries; 0 if there is none
+__device__ __forceinline__ int hist_top(uint32_t hist, int K) {
+    int acc = 0, top = 0;
+#pragma unroll
+    for (int b = HIST_BUCKETS - 1; b > 0; --b) {
+        const int before = acc;
+        acc += static_cast<int>(ld_shared_b32(hist + b * 512));
+        if (before < K && acc >= K) top = b;
+    }
+    return top;
 }
 
 // TOPK selects how MODE_STATS keeps a row's Top-K candidates: TOPK_REG (K <= K_REG) a sorted list in
@@ -534,6 +611,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                 want_topk = HAS_TOPK && tile_ok && rt < p.topk_row_tiles;
                 if (HAS_TOPK) cbuf = p.cand + (static_cast<long long>(slot) * BM + r_local) * p.cap;
                 cnt = 0;
+                if (HAS_TOPK && p.row_global_offset + (rt < p.row_tiles0 ? rt : rt - p.row_tiles0) * BM + r_local >= p.rows_valid) {
+                    // A padding row collects nothing: its logits are all equal (zero), and 256 of them filled its buffer and
+                    // made the warp compact row after row (sweep of 64 rows x 256 x 1024, K = 64: 195 -> 30 us).
+                    thr_own = INFINITY;
+                    thr = INFINITY;
+                }
                 if (USE_REG) {
 #pragma unroll
                     for (int i = 0; i < (USE_REG ? K_REG : 1); ++i) {
@@ -600,35 +683,40 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                     m = ref2 * (1.0f / LOG2E);
                 }
                 if (MODE == MODE_STATS && HAS_TOPK && !USE_REG && want_topk && t == 0 && p.n_cols - col_base >= BN) {
-                    // First tile of the sweep, buffer empty, no threshold yet: admitting all 256 logits would fill
-                    // the buffer and force a compaction of every row of the warp at once (32 warp-wide compactions
-                    // in a row, during which the tensor core runs out of free accumulators). Instead each thread
-                    // searches, bit by bit, the largest 12-bit prefix (sign, exponent, three mantissa bits) that at
-                    // least K of its row's 256 logits reach - comparisons against the tile in tensor memory, the same
-                    // instructions for every row - and starts from the threshold just below it: a valid lower bound
-                    // of the row's K-th largest logit that admits little more than K of the tile's logits.
-                    uint32_t T = 0u;
+                    // First tile of the sweep, buffer empty, no threshold yet: admitting all 256 logits would fill the buffer
+                    // at once. Each thread takes a histogram of its row's 256 logits between the least and the largest and
+                    // starts from half a bucket below the bucket above which at least K of them lie: a valid lower bound of
+                    // the row's K-th largest logit that admits little more than K of the tile's.
+                    float lo = INFINITY, hi = -INFINITY;
 #pragma unroll 1
-                    for (int bit = 31; bit >= 20; --bit) {
-                        const uint32_t cand = T | (1u << bit);
-                        const float fc = __uint_as_float(key_bits(cand));      // keys order like the floats they stand for
-                        int c = 0;
-#pragma unroll 1
-                        for (int ch = 0; ch < BN / 32; ++ch) {
-                            uint32_t r[32];
-                            tmem_ld32(t_row + ch * 32, r);
-                            tmem_ld_wait(r);
+                    for (int ch = 0; ch < BN / 32; ++ch) {
+                        uint32_t r[32];
+                        tmem_ld32(t_row + ch * 32, r);
+                        tmem_ld_wait(r);
 #pragma unroll
-                            for (int j = 0; j < 32; ++j) c += (__uint_as_float(r[j]) >= fc) ? 1 : 0;
+                        for (int j = 0; j < 32; ++j) {
+                            lo = fminf(lo, __uint_as_float(r[j]));
+                            hi = fmaxf(hi, __uint_as_float(r[j]));
                         }
-                        if (c >= p.K) T = cand;
                     }
-                    if (T >= (1u << 20)) {
-                        // the float just below the prefix; at the prefix of +0 that is -0, which compares equal to
-                        // the zeros that were counted, so step down to a float that is really smaller
-                        float below = __uint_as_float(key_bits(T - 1u));
-                        if (below == 0.f) below = -1.17549435e-38f;
-                        thr_own = below;
+                    const float inv = HIST_BUCKETS / (hi - lo);
+                    hist_clear(pend_v);
+#pragma unroll 1
+                    for (int ch = 0; ch < BN / 32; ++ch) {
+                        uint32_t r[32];
+                        tmem_ld32(t_row + ch * 32, r);
+                        tmem_ld_wait(r);
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) {
+                            const uint32_t at = pend_v + hist_bucket(__uint_as_float(r[j]), lo, inv) * 512;
+                            st_shared_b32(at, ld_shared_b32(at) + 1u);
+                        }
+                    }
+                    const int top = hist_top(pend_v, p.K);
+                    const float bound = lo + (static_cast<float>(top) - 0.5f) / inv;
+                    // (half a bucket must exceed the rounding of these few operations; also false for infinities and NaN)
+                    if (top > 0 && 0.5f / inv > 1e-6f * fmaxf(fabsf(lo), fabsf(hi))) {
+                        thr_own = fmaxf(thr_own, bound);
                         thr = fmaxf(thr_own, thr_sh);
                     }
                 }
@@ -670,23 +758,15 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                     if (MODE == MODE_STATS && !USE_REG && want_topk) {
                         // make room for a whole chunk in every row's buffer (warp-uniform control flow), before the
                         // chunk's logits occupy registers
-                        uint32_t full = __ballot_sync(0xffffffffu, cnt > p.cap - 32);
-                        while (full) {
-                            const int L = __ffs(full) - 1;
-                            full &= full - 1u;
-                            __syncwarp();
-                            const unsigned long long bp = __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(cbuf), L);
-                            const int n = __shfl_sync(0xffffffffu, cnt, L);
-                            int left = 0;
-                            const uint32_t tb = p.cap <= 32 * CAND_REGS_SMALL
-                                                    ? compact_candidates<CAND_REGS_SMALL>(reinterpret_cast<uint2*>(bp), n, p.K, p.cap, lane, left)
-                                                    : compact_candidates<CAND_REGS>(reinterpret_cast<uint2*>(bp), n, p.K, p.cap, lane, left);
-                            __syncwarp();
-                            if (lane == L) {
-                                cnt = left;
-                                thr_own = __uint_as_float(tb);
-                                thr = fmaxf(thr_own, thr_sh);
-                            }
+                        const uint32_t full = __ballot_sync(0xffffffffu, cnt > p.cap - 32);
+                        if (full) {
+                            if (p.cap <= 32 * CAND_REGS_TINY)
+                                compact_rows<CAND_REGS_TINY>(full, cbuf, cnt, thr_own, p.K, p.cap, lane);
+                            else if (p.cap <= 32 * CAND_REGS_SMALL)
+                                compact_rows<CAND_REGS_SMALL>(full, cbuf, cnt, thr_own, p.K, p.cap, lane);
+                            else
+                                compact_rows<CAND_REGS>(full, cbuf, cnt, thr_own, p.K, p.cap, lane);
+                            thr = fmaxf(thr_own, thr_sh);
                         }
                     }
                     uint32_t r[32];
@@ -798,12 +878,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                         if (!USE_REG && want_topk && cm > thr) {
                             // predicated stores, no branches: as 32 conditional blocks this section took about 5000
                             // cycles whenever any row of the warp admitted a logit
+                            uint2* at = cbuf + cnt;
 #pragma unroll
-                            for (int j = 0; j < 32; ++j) {
-                                const bool in = __uint_as_float(r[j]) > thr;
-                                st_global_v2_if(cbuf + cnt, r[j], static_cast<uint32_t>(col0 + j), in);
-                                cnt += in ? 1 : 0;
-                            }
+                            for (int j = 0; j < 32; ++j) append_if_above(at, __uint_as_float(r[j]), static_cast<uint32_t>(col0 + j), thr);
+                            cnt = static_cast<int>(at - cbuf);
                         }
                         if (USE_REG && want_topk && cm > thr) {
                             // collect the chunk's candidates, then admit them one by one (the

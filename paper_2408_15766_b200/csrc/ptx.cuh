@@ -259,10 +259,14 @@ __device__ __forceinline__ void st_shared_b32_if(uint32_t addr, uint32_t v, bool
                  "r"(static_cast<uint32_t>(on))
                  : "memory");
 }
-__device__ __forceinline__ void st_global_v2_if(void* ptr, uint32_t a, uint32_t b, bool on) {
-    asm volatile("{\n.reg .pred q;\nsetp.ne.b32 q, %3, 0;\n@q st.global.v2.b32 [%0], {%1, %2};\n}" ::"l"(ptr), "r"(a), "r"(b),
-                 "r"(static_cast<uint32_t>(on))
+// *at++ = (x, id) where x > bound
+__device__ __forceinline__ void append_if_above(uint2*& at, float x, uint32_t id, float bound) {
+    unsigned long long p = reinterpret_cast<unsigned long long>(at);
+    asm volatile("{\n.reg .pred q;\nsetp.gt.f32 q, %1, %3;\n@q st.global.v2.b32 [%0], {%4, %2};\n@q add.s64 %0, %0, 8;\n}"
+                 : "+l"(p)
+                 : "f"(x), "r"(id), "f"(bound), "r"(__float_as_uint(x))
                  : "memory");
+    at = reinterpret_cast<uint2*>(p);
 }
 __device__ __forceinline__ uint32_t ld_shared_b32(uint32_t addr) {
     uint32_t v;

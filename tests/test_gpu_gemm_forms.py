@@ -19,6 +19,7 @@ pytestmark = pytest.mark.gpu
     (129, 264, 30001, 5, True),        # two row tiles, one row in the second, a ragged contraction
     (700, 64, 9000, 200, True),        # selection of a large K with one warp per row, which cuts its pool
     (40, 64, 33000, 40, True),         # the same with four warps per row and buffers of 129 lanes
+    (129, 64, 9000, 64, True),         # 127 padding rows in the second row tile, buffered candidates
     (64, 72, 33001, 256, False),       # the most rows whose draft logits go through the workspace in fp32, the largest K
     (65, 72, 33001, 256, False),       # one row more
     (620, 64, 40000, 16, True),        # one warp per row, K lists whose first entries set the floor
