@@ -84,6 +84,8 @@ static int device_info(DeviceInfo* out) {
             cudaError_t e3 = cudaSuccess;
             for (GemmFn f : gemms)
                 if (e3 == cudaSuccess) e3 = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+            if (e3 == cudaSuccess) e3 = cudaFuncSetAttribute(select_kernel<16, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * 512 * 8);
+            if (e3 == cudaSuccess) e3 = cudaFuncSetAttribute(select_kernel<16, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * 1024 * 8);
             cudaError_t e4 = cudaFuncSetAttribute(hca2::hca_attention_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hca2::SMEM_BYTES);
             if (e4 == cudaSuccess) e4 = cudaFuncSetAttribute(hca_bwd::hca_bwd_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hca_bwd::F_SMEM_BYTES);
             if (e3 != cudaSuccess || e4 != cudaSuccess) {
@@ -443,7 +445,16 @@ static int clear_status(uint8_t* ws, const Layout& L, int slots, cudaStream_t st
     return HASS_OK;
 }
 
-// Four warps per row while that is at most four blocks per SM, one warp beyond. The lists of K <= 16 hold 16 entries each
+template <int WARPS, int WIN>
+static constexpr size_t select_smem() { return static_cast<size_t>(sel_block_warps(WARPS)) * WIN * 8; }
+template <int WARPS, int WIN>
+static void select_as(const SelectParams& sp, cudaStream_t st) {
+    constexpr int bw = sel_block_warps(WARPS);
+    select_kernel<WARPS, WIN><<<ceil_div(sp.rows, bw / WARPS), bw * 32, select_smem<WARPS, WIN>(), st>>>(sp);
+}
+
+// Sixteen warps per row while every row has an SM of its own, four while that is at most four blocks per SM, one warp
+// beyond. The lists of K <= 16 hold 16 entries each
 // and need the smaller window. Against one warp per row that walks the lists one after the other: 61 rows x 125 lists
 // 113 -> 15 us, 4096 rows x 4 lists 40 -> 9 us (22 with the dot product for the reference exponent, which saves the
 // draft sweep its extra tile: 25 us here, half of it at 61 rows), 4096 rows of K = 64 275 -> 130 us.
@@ -451,17 +462,12 @@ static int launch_select(const SelectParams& sp, int sms, cudaStream_t st) {
     {
         KernelTimer timer(sp.gate ? KIND_CONDITIONAL : KIND_FINALIZE, st);
         const bool reg = sp.cap == K_REG;
-        if (sp.rows <= 4 * sms) {
-            if (reg)
-                select_kernel<4, 512><<<sp.rows, SEL_WARPS * 32, 0, st>>>(sp);
-            else
-                select_kernel<4, 1024><<<sp.rows, SEL_WARPS * 32, 0, st>>>(sp);
-        } else {
-            if (reg)
-                select_kernel<1, 512><<<ceil_div(sp.rows, SEL_WARPS), SEL_WARPS * 32, 0, st>>>(sp);
-            else
-                select_kernel<1, 1024><<<ceil_div(sp.rows, SEL_WARPS), SEL_WARPS * 32, 0, st>>>(sp);
-        }
+        if (sp.rows <= sms)
+            reg ? select_as<16, 512>(sp, st) : select_as<16, 1024>(sp, st);
+        else if (sp.rows <= 4 * sms)
+            reg ? select_as<4, 512>(sp, st) : select_as<4, 1024>(sp, st);
+        else
+            reg ? select_as<1, 512>(sp, st) : select_as<1, 1024>(sp, st);
     }
     g_launches.fetch_add(1);
     return cudaGetLastError() == cudaSuccess ? HASS_OK : HASS_ERR_CUDA;

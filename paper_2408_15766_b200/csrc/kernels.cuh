@@ -1435,8 +1435,9 @@ __global__ void __launch_bounds__(FIN_WARPS * 32) finalize_kernel(const __grid_c
 // copies z_d at those tokens out of its accumulators.
 // Bound by load latency: the lists of the row's lanes are read 256 entries at a time per warp (32 lanes x SEL_LOADS loads in
 // flight) and what lies below the best K-th logit of any list is dropped on the way. WARPS warps share a row: one where
-// there are rows enough to fill the GPU, four where few rows have lists of up to 148 lanes each.
-constexpr int SEL_WARPS = 4;          // warps per block
+// there are rows enough to fill the GPU, four or sixteen where few rows have lists of up to 148 lanes each. A block has
+// four warps, or the sixteen of its row.
+__host__ __device__ constexpr int sel_block_warps(int WARPS) { return WARPS > 4 ? WARPS : 4; }
 constexpr int SEL_LOADS = 8;          // candidate loads a lane has in flight
 constexpr int SEL_FIRST = 5;          // lists per lane whose first entries set the floor (the first 160 of the row)
 
@@ -1476,18 +1477,63 @@ __device__ __forceinline__ unsigned long long cand_rank(uint32_t key, uint32_t i
     return (static_cast<unsigned long long>(key) << 32) | (~id);
 }
 
-// Warp-collective: keeps the K best of the n > K candidates in `pool` (distinct numbers), in place, and returns the
-// smallest one kept. The bound is searched bit by bit from the top until exactly K reach it.
-__device__ __forceinline__ unsigned long long cut_to_best(unsigned long long* pool, int n, int K, int lane) {
-    unsigned long long T = 0ull;
+// Cuts the candidates (distinct numbers) in the pools of WARPS warps, n in this warp's `pool`, total > K of them, to the
+// K best and at most `slack` more, in place, and returns the bound that those kept reach. The bound is searched from the
+// highest bit in which the numbers differ, two bits per step. Collective over the WARPS warps; sh: CUT_WORDS words of
+// shared memory that the block uses for nothing else (WARPS > 1 only; the block is then these warps).
+constexpr int CUT_WORDS = 12;
+template <int WARPS>
+__device__ __forceinline__ unsigned long long cut_to_best(unsigned long long* pool, int& n, int K, int slack, int lane, uint32_t* sh) {
+    uint32_t hi = 0u, lo = 0xffffffffu;
+    for (int e = lane; e < n; e += 32) {
+        const uint32_t k = static_cast<uint32_t>(pool[e] >> 32);
+        hi = max(hi, k);
+        lo = min(lo, k);
+    }
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    if (WARPS > 1) {
+        if (threadIdx.x < CUT_WORDS) sh[threadIdx.x] = threadIdx.x == 10 ? 0xffffffffu : 0u;
+        __syncthreads();
+        if (lane == 0) {
+            atomicMax(sh + 9, hi);
+            atomicMin(sh + 10, lo);
+        }
+        __syncthreads();
+        hi = sh[9];
+        lo = sh[10];
+    }
+    int bit = 64 - __clz(hi ^ lo);      // (equal logits: the token ids' 32 bits are left)
+    bit += bit & 1;
+    unsigned long long T = bit < 64 ? (static_cast<unsigned long long>(hi) << 32 >> bit) << bit : 0ull;
+    int step = 0;                       // sums of step i in words 3 (i % 3) ..; those of the next step are cleared meanwhile
 #pragma unroll 1
-    for (int bit = 63; bit >= 0; --bit) {
-        const unsigned long long c2 = T | (1ull << bit);
-        int c = 0;
-        for (int e = lane; e < n; e += 32) c += pool[e] >= c2 ? 1 : 0;
-        c = __reduce_add_sync(0xffffffffu, c);
-        if (c >= K) T = c2;
-        if (c == K) break;
+    for (bit -= 2; bit >= 0; bit -= 2) {
+        const unsigned long long T1 = T | (1ull << bit), T2 = T | (2ull << bit), T3 = T | (3ull << bit);
+        int c1 = 0, c2 = 0, c3 = 0;
+#pragma unroll 4
+        for (int e = lane; e < n; e += 32) {
+            const unsigned long long v = pool[e];
+            c1 += v >= T1 ? 1 : 0;
+            c2 += v >= T2 ? 1 : 0;
+            c3 += v >= T3 ? 1 : 0;
+        }
+        c1 = __reduce_add_sync(0xffffffffu, c1);
+        c2 = __reduce_add_sync(0xffffffffu, c2);
+        c3 = __reduce_add_sync(0xffffffffu, c3);
+        if (WARPS > 1) {
+            uint32_t* sum = sh + 3 * step;
+            step = step == 2 ? 0 : step + 1;
+            if (lane < 3) atomicAdd(sum + lane, static_cast<uint32_t>(lane == 0 ? c1 : lane == 1 ? c2 : c3));
+            if (threadIdx.x < 3) sh[3 * step + threadIdx.x] = 0u;
+            __syncthreads();
+            c1 = static_cast<int>(sum[0]);
+            c2 = static_cast<int>(sum[1]);
+            c3 = static_cast<int>(sum[2]);
+        }
+        const int c = c3 >= K ? c3 : c2 >= K ? c2 : c1 >= K ? c1 : INT_MAX;
+        T = c3 >= K ? T3 : c2 >= K ? T2 : c1 >= K ? T1 : T;
+        if (c <= K + slack) break;
     }
     const uint32_t lt_mask = (1u << lane) - 1u;
     int np = 0;
@@ -1500,15 +1546,18 @@ __device__ __forceinline__ unsigned long long cut_to_best(unsigned long long* po
         np += __popc(bm);
         __syncwarp();
     }
+    n = np;
     return T;
 }
 
 template <int WARPS, int WIN>
-__global__ void __launch_bounds__(SEL_WARPS * 32) select_kernel(const __grid_constant__ SelectParams p) {
-    static_assert(WIN >= K_CAP + 32 * SEL_LOADS, "a cut leaves room for one batch of loads");
-    constexpr int ROWS = SEL_WARPS / WARPS;                   // rows per block
-    __shared__ unsigned long long pools[SEL_WARPS][WIN];
-    __shared__ int pool_n[SEL_WARPS];
+__global__ void __launch_bounds__(sel_block_warps(WARPS) * 32) select_kernel(const __grid_constant__ SelectParams p) {
+    static_assert(WIN >= (WIN > 512 ? K_CAP : K_REG) + 64 + 32 * SEL_LOADS, "a cut leaves room for one batch of loads");
+    constexpr int BLOCK_WARPS = sel_block_warps(WARPS);
+    constexpr int ROWS = BLOCK_WARPS / WARPS;                 // rows per block
+    extern __shared__ unsigned long long sel_pools[];         // [BLOCK_WARPS][WIN]
+    __shared__ int pool_n[BLOCK_WARPS];
+    __shared__ uint32_t cut_words[CUT_WORDS];
     __shared__ int sel_tok[ROWS][K_CAP];                      // Omega_hat in descending q
     __shared__ float sel_q[ROWS][K_CAP];
     const int lane = threadIdx.x & 31;
@@ -1583,7 +1632,7 @@ __global__ void __launch_bounds__(SEL_WARPS * 32) select_kernel(const __grid_con
         if (tid == 0 && p.lse_t) p.lse_t[row] = lse_t;
 
         // this warp's share of the candidates: lanes of the row tile w, w + WARPS, ...
-        unsigned long long* pool = pools[warp];
+        unsigned long long* pool = sel_pools + warp * WIN;
         int n = 0;
         const uint32_t lt_mask = (1u << lane) - 1u;
         auto append = [&](const uint2 (&ce)[SEL_LOADS], const bool (&in)[SEL_LOADS]) {
@@ -1596,10 +1645,8 @@ __global__ void __launch_bounds__(SEL_WARPS * 32) select_kernel(const __grid_con
                 n += __popc(bm);
             }
             __syncwarp();
-            if (n + 32 * SEL_LOADS > WIN) {      // n > K here
-                floor_key = max(floor_key, static_cast<uint32_t>(cut_to_best(pool, n, K, lane) >> 32));
-                n = K;
-            }
+            if (n + 32 * SEL_LOADS > WIN)        // n > K + 64 here
+                floor_key = max(floor_key, static_cast<uint32_t>(cut_to_best<1>(pool, n, K, 64, lane, nullptr) >> 32));
         };
         if (lists) {
             for (int e0 = w * 32 * SEL_LOADS; e0 < S * K_REG; e0 += WARPS * 32 * SEL_LOADS) {
@@ -1636,11 +1683,15 @@ __global__ void __launch_bounds__(SEL_WARPS * 32) select_kernel(const __grid_con
                 }
             }
         }
-        // Rank what is left: every candidate counts those above it. Beyond 128 a pool is cut to K first.
-        if (n > K && n > 128) {
-            cut_to_best(pool, n, K, lane);
-            n = K;
+        // Rank what is left: every candidate counts those above it. Beyond 128 they are cut to about K first.
+        int total = n;
+        if (WARPS > 1) {
+            if (lane == 0) pool_n[warp] = n;
+            __syncthreads();
+            total = __reduce_add_sync(0xffffffffu, lane < WARPS ? pool_n[lane] : 0);
         }
+        if (total > K && total > 128) cut_to_best<WARPS>(pool, n, K, 16, lane, cut_words);
+        if (WARPS > 1) __syncthreads();
         if (lane == 0) pool_n[warp] = n;
         for (int j = tid; j < K; j += WARPS * 32) {           // cannot stay for K <= V; keeps ids in range
             sel_tok[rib][j] = 0;
@@ -1651,7 +1702,7 @@ __global__ void __launch_bounds__(SEL_WARPS * 32) select_kernel(const __grid_con
             const unsigned long long v = pool[e];
             int rank = 0;
             for (int w2 = 0; w2 < WARPS; ++w2) {
-                const unsigned long long* other = pools[rib * WARPS + w2];
+                const unsigned long long* other = sel_pools + (rib * WARPS + w2) * WIN;
                 const int n2 = pool_n[rib * WARPS + w2];
                 for (int i = 0; i < n2; ++i) rank += other[i] > v ? 1 : 0;
             }
