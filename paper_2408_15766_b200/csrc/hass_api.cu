@@ -759,6 +759,118 @@ struct Combined {
     __nv_bfloat16* Pt;     // [chunk rows, p_pitch] scratch: spill of the target tiles
 };
 
+// Rows of one call up to which the draft logits go through the workspace in fp32 (narrow_impl): two rows of 128-row bf16
+// scratch hold one of them. Up to here a call is bound by reading W, which this route does twice (both sweeps in one
+// launch, then the second GEMM) instead of three times, with no range condition and so no second pass: 61 rows x 4096 x
+// 32000 211 -> 147 us, 64 rows x 256 x 1024 67 -> 46 us. Beyond, the fp32 logits would not fit a workspace of one row tile.
+constexpr int kNarrowRows = BM / 2;
+
+static int narrow_impl(bool with_target, const void* H_t, const void* H_d, const void* W, int N, long long d, long long V,
+                       int K, const float* grad_loss, const int* idx_in, const float* q_in, float* loss, int* idx_out,
+                       float* q_out, float* lse_t, float* lse_d, void* dH_d, int dH_dtype, uint8_t* ws, const Layout& L,
+                       const PartRoom& part, int sms, cudaStream_t st, float top_p, int* topk_n, const Combined* cmb = nullptr) {
+    const int CT = ceil_div(V, BN), DT = ceil_div(d, BN);
+    unsigned int* status = reinterpret_cast<unsigned int*>(ws + L.status);
+    float* z = reinterpret_cast<float*>(ws + L.scratch);
+    // (1) target and draft rows in one sweep: statistics, candidates, the draft's logits
+    GemmParams p;
+    std::memset(&p, 0, sizeof(p));
+    p.row_tiles = with_target ? 2 : 1;
+    int rc = plan_launch(p.row_tiles, CT, sms, L.slot_cap, &p.sched);
+    if (rc != HASS_OK) return rc;
+    log_schedule("narrow sweep", p.sched);
+    rc = make_tmap(&p.tmA1, H_d, N, d, d, BK, BM);
+    if (rc == HASS_OK) rc = make_tmap(&p.tmA0, with_target ? H_t : H_d, N, d, d, BK, BM);
+    if (rc == HASS_OK) rc = make_tmap(&p.tmB, W, V, d, d, BK, BN / p.sched.pair);
+    if (rc != HASS_OK) return rc;
+    p.row_tiles0 = 1;
+    p.topk_row_tiles = with_target ? 1 : 0;
+    p.spill_begin = INT_MAX;
+    p.z_begin = cmb ? 0 : p.row_tiles - 1;
+    p.z_rows = N;
+    p.z_out = z;
+    p.zt_out = cmb ? reinterpret_cast<float*>(cmb->Pt) : nullptr;
+    p.z_pitch = L.p_pitch;
+    p.rows_valid = N;
+    p.n_cols = static_cast<int>(V);
+    p.col_tiles = CT;
+    p.k_blocks = ceil_div(d, BK);
+    p.K = K;
+    p.cap = topk_cap(K);
+    p.part_m = reinterpret_cast<float*>(ws + L.part_m);
+    p.part_s = reinterpret_cast<float*>(ws + L.part_s);
+    p.cand = reinterpret_cast<uint2*>(ws + L.cand_v);
+    p.cand_n = reinterpret_cast<int*>(ws + L.cand_i);
+    p.thr_share = reinterpret_cast<unsigned int*>(ws + L.thr_share);
+    p.status = status;
+    rc = clear_status(ws, L, with_target ? p.sched.total_slots : 0, st);
+    if (rc != HASS_OK) return rc;
+    rc = launch_gemm<MODE_STATS>(p, st, with_target ? KIND_STATS : KIND_STATS_DRAFT);
+    if (rc != HASS_OK) return rc;
+    // (2) Omega_hat
+    if (with_target) {
+        SelectParams sp = select_params(p, 0, 0, N, idx_out, q_out, K, lse_t);
+        sp.n_out = topk_n;
+        sp.top_p = top_p;
+        rc = launch_select(sp, sms, st);
+        if (rc != HASS_OK) return rc;
+    }
+    // (3) lse_d, loss, dz_d
+    DzParams z_params;
+    std::memset(&z_params, 0, sizeof(z_params));
+    z_params.sched = p.sched;
+    z_params.first_tile = p.row_tiles - 1;
+    z_params.K = K;
+    z_params.V = static_cast<int>(V);
+    z_params.part_m = p.part_m;
+    z_params.part_s = p.part_s;
+    z_params.idx = with_target ? idx_out : idx_in;
+    z_params.q = with_target ? q_out : q_in;
+    z_params.grad_loss = grad_loss;
+    z_params.loss = loss;
+    z_params.lse_d = lse_d;
+    z_params.z = z;
+    z_params.pitch = L.p_pitch;
+    z_params.make_dz = dH_d != nullptr ? 1 : 0;
+    if (cmb) {
+        z_params.zt = p.zt_out;
+        z_params.lse_t = lse_t;
+        z_params.w = cmb->w;
+        z_params.loss_ce = cmb->loss_ce;
+    }
+    {
+        KernelTimer timer(KIND_FINALIZE, st);
+        if (cmb)
+            dz_kernel<true><<<N, DZ_THREADS, 0, st>>>(z_params);
+        else
+            dz_kernel<false><<<N, DZ_THREADS, 0, st>>>(z_params);
+    }
+    g_launches.fetch_add(1);
+    if (cudaGetLastError() != cudaSuccess) return HASS_ERR_CUDA;
+    if (dH_d == nullptr) return HASS_OK;      // the forward alone
+    // (4) dH_d = dz_d W
+    GemmParams o;
+    std::memset(&o, 0, sizeof(o));
+    rc = make_tmap(&o.tmA0, z, N, V, 2 * L.p_pitch, BK, BM);
+    if (rc == HASS_OK) rc = make_tmap(&o.tmB, W, V, d, d, 64, BK);
+    if (rc != HASS_OK) return rc;
+    o.tmA1 = o.tmA0;
+    o.row_tiles = 1;
+    o.row_tiles0 = 1;
+    o.spill_begin = INT_MAX;
+    o.rows_valid = N;
+    o.n_cols = static_cast<int>(d);
+    o.col_tiles = DT;
+    o.k_blocks = ceil_div(V, BK);
+    o.K = K;
+    o.out = dH_d;
+    o.out_fp32 = dH_dtype == HASS_FP32 ? 1 : 0;
+    o.out_align32 = ((reinterpret_cast<uintptr_t>(dH_d) | static_cast<uintptr_t>(d * (dH_dtype == HASS_FP32 ? 4 : 2))) & 31u) == 0 ? 1 : 0;
+    o.out_pitch = d;
+    o.status = status;
+    return launch_out(o, part, sms, st);
+}
+
 static int fused_impl(bool with_target, const void* H_t, const void* H_d, const void* W, long long N, long long d,
                       long long V, int K, const float* grad_loss, const int* idx_in, const float* q_in, float* loss,
                       int* idx_out, float* q_out, float* lse_t, float* lse_d, void* dH_d, int dH_dtype,
@@ -793,6 +905,9 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
     __nv_bfloat16* P = reinterpret_cast<__nv_bfloat16*>(ws + L.scratch);
     unsigned int* status = reinterpret_cast<unsigned int*>(ws + L.status);
     int* idx_d = reinterpret_cast<int*>(ws + L.sidx);
+    if (cmb && with_target && N <= kNarrowRows)
+        return narrow_impl(true, H_t, H_d, W, static_cast<int>(N), d, V, K, grad_loss, nullptr, nullptr, loss, idx_out, q_out, lse_t,
+                           lse_d, dH_d, dH_dtype, ws, L, part, di.sms, st, 0.f, nullptr, cmb);
     CUtensorMap tmHt, tmHd, tmWn, tmP;
     rc = make_tmap(&tmHd, H_d, N, d, d, BK, BM);
     if (rc == HASS_OK) rc = with_target ? make_tmap(&tmHt, H_t, N, d, d, BK, BM) : make_tmap(&tmHt, H_d, N, d, d, BK, BM);
@@ -1030,106 +1145,6 @@ static int pipe_out(ChunkPipe* pipe, const void* dH_d, size_t row, size_t rows, 
         return HASS_ERR_CUDA;
     }
     return HASS_OK;
-}
-
-// Rows of one call up to which the draft logits go through the workspace in fp32 (narrow_impl): two rows of 128-row bf16
-// scratch hold one of them. Up to here a call is bound by reading W, which this route does twice (both sweeps in one
-// launch, then the second GEMM) instead of three times, with no range condition and so no second pass: 61 rows x 4096 x
-// 32000 211 -> 147 us, 64 rows x 256 x 1024 67 -> 46 us. Beyond, the fp32 logits would not fit a workspace of one row tile.
-constexpr int kNarrowRows = BM / 2;
-
-static int narrow_impl(bool with_target, const void* H_t, const void* H_d, const void* W, int N, long long d, long long V,
-                       int K, const float* grad_loss, const int* idx_in, const float* q_in, float* loss, int* idx_out,
-                       float* q_out, float* lse_t, float* lse_d, void* dH_d, int dH_dtype, uint8_t* ws, const Layout& L,
-                       const PartRoom& part, int sms, cudaStream_t st, float top_p, int* topk_n) {
-    const int CT = ceil_div(V, BN), DT = ceil_div(d, BN);
-    unsigned int* status = reinterpret_cast<unsigned int*>(ws + L.status);
-    float* z = reinterpret_cast<float*>(ws + L.scratch);
-    // (1) target and draft rows in one sweep: statistics, candidates, the draft's logits
-    GemmParams p;
-    std::memset(&p, 0, sizeof(p));
-    p.row_tiles = with_target ? 2 : 1;
-    int rc = plan_launch(p.row_tiles, CT, sms, L.slot_cap, &p.sched);
-    if (rc != HASS_OK) return rc;
-    log_schedule("narrow sweep", p.sched);
-    rc = make_tmap(&p.tmA1, H_d, N, d, d, BK, BM);
-    if (rc == HASS_OK) rc = make_tmap(&p.tmA0, with_target ? H_t : H_d, N, d, d, BK, BM);
-    if (rc == HASS_OK) rc = make_tmap(&p.tmB, W, V, d, d, BK, BN / p.sched.pair);
-    if (rc != HASS_OK) return rc;
-    p.row_tiles0 = 1;
-    p.topk_row_tiles = with_target ? 1 : 0;
-    p.spill_begin = INT_MAX;
-    p.z_begin = p.row_tiles - 1;
-    p.z_rows = N;
-    p.z_out = z;
-    p.z_pitch = L.p_pitch;
-    p.rows_valid = N;
-    p.n_cols = static_cast<int>(V);
-    p.col_tiles = CT;
-    p.k_blocks = ceil_div(d, BK);
-    p.K = K;
-    p.cap = topk_cap(K);
-    p.part_m = reinterpret_cast<float*>(ws + L.part_m);
-    p.part_s = reinterpret_cast<float*>(ws + L.part_s);
-    p.cand = reinterpret_cast<uint2*>(ws + L.cand_v);
-    p.cand_n = reinterpret_cast<int*>(ws + L.cand_i);
-    p.thr_share = reinterpret_cast<unsigned int*>(ws + L.thr_share);
-    p.status = status;
-    rc = clear_status(ws, L, with_target ? p.sched.total_slots : 0, st);
-    if (rc != HASS_OK) return rc;
-    rc = launch_gemm<MODE_STATS>(p, st, with_target ? KIND_STATS : KIND_STATS_DRAFT);
-    if (rc != HASS_OK) return rc;
-    // (2) Omega_hat
-    if (with_target) {
-        SelectParams sp = select_params(p, 0, 0, N, idx_out, q_out, K, lse_t);
-        sp.n_out = topk_n;
-        sp.top_p = top_p;
-        rc = launch_select(sp, sms, st);
-        if (rc != HASS_OK) return rc;
-    }
-    // (3) lse_d, loss, dz_d
-    DzParams z_params;
-    std::memset(&z_params, 0, sizeof(z_params));
-    z_params.sched = p.sched;
-    z_params.first_tile = p.z_begin;
-    z_params.K = K;
-    z_params.V = static_cast<int>(V);
-    z_params.part_m = p.part_m;
-    z_params.part_s = p.part_s;
-    z_params.idx = with_target ? idx_out : idx_in;
-    z_params.q = with_target ? q_out : q_in;
-    z_params.grad_loss = grad_loss;
-    z_params.loss = loss;
-    z_params.lse_d = lse_d;
-    z_params.z = z;
-    z_params.pitch = L.p_pitch;
-    {
-        KernelTimer timer(KIND_FINALIZE, st);
-        dz_kernel<<<N, DZ_THREADS, 0, st>>>(z_params);
-    }
-    g_launches.fetch_add(1);
-    if (cudaGetLastError() != cudaSuccess) return HASS_ERR_CUDA;
-    // (4) dH_d = dz_d W
-    GemmParams o;
-    std::memset(&o, 0, sizeof(o));
-    rc = make_tmap(&o.tmA0, z, N, V, 2 * L.p_pitch, BK, BM);
-    if (rc == HASS_OK) rc = make_tmap(&o.tmB, W, V, d, d, 64, BK);
-    if (rc != HASS_OK) return rc;
-    o.tmA1 = o.tmA0;
-    o.row_tiles = 1;
-    o.row_tiles0 = 1;
-    o.spill_begin = INT_MAX;
-    o.rows_valid = N;
-    o.n_cols = static_cast<int>(d);
-    o.col_tiles = DT;
-    o.k_blocks = ceil_div(V, BK);
-    o.K = K;
-    o.out = dH_d;
-    o.out_fp32 = dH_dtype == HASS_FP32 ? 1 : 0;
-    o.out_align32 = ((reinterpret_cast<uintptr_t>(dH_d) | static_cast<uintptr_t>(d * (dH_dtype == HASS_FP32 ? 4 : 2))) & 31u) == 0 ? 1 : 0;
-    o.out_pitch = d;
-    o.status = status;
-    return launch_out(o, part, sms, st);
 }
 
 static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const void* W, long long N, long long d,
@@ -1373,6 +1388,9 @@ static int forward2_impl(bool with_target, const void* H_t, const void* H_d, con
                             workspace, workspace_bytes, st);
     const int RT = ceil_div(N, BM), CT = ceil_div(V, BN);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
+    if (N <= kNarrowRows && workspace_bytes >= L.fixed_end + L.scratch_row_tile_bytes)
+        return narrow_impl(with_target, H_t, H_d, W, static_cast<int>(N), d, V, K, nullptr, idx_in, q_in, loss, idx_out, q_out,
+                           lse_t, lse_d, nullptr, HASS_BF16, ws, L, PartRoom(), di.sms, st, 0.f, nullptr);
     GemmParams p;
     std::memset(&p, 0, sizeof(p));
     rc = plan_launch(RT, CT, di.sms, L.slot_cap, &p.sched);

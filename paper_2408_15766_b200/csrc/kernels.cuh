@@ -113,10 +113,11 @@ struct GemmParams {
     __nv_bfloat16* P;      // [chunk rows, p_pitch]
     __nv_bfloat16* Pt;     // [chunk rows, p_pitch] spill of the target tiles, or nullptr
     long long p_pitch;
-    // MODE_STATS: row tiles from z_begin on write their logits in fp32 to z_out [rows of these tiles, z_pitch]; the last
-    // z_rows of them are valid (INT_MAX: none)
+    // MODE_STATS: row tiles from z_begin on write the logits of their first z_rows rows in fp32 (INT_MAX: none): to z_out
+    // [z_rows, z_pitch], those of row tiles < row_tiles0 to zt_out
     int z_begin, z_rows;
     float* z_out;
+    float* zt_out;
     long long z_pitch;
     // MODE_OUT. With sparse != nullptr the epilogue computes coef[row] * acc - sparse[local row, :] (row scale
     // and the Omega_hat term of dz_d W, precomputed by finalize); with coef alone coef[row] * acc; with neither
@@ -641,8 +642,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                 nxt = si[0];
             }
             float* zrow = nullptr;
-            if (HAS_TOPK && tile_ok && rt >= p.z_begin && (rt - p.z_begin) * BM + r_local < p.z_rows)
-                zrow = p.z_out + static_cast<long long>((rt - p.z_begin) * BM + r_local) * p.z_pitch;
+            if (HAS_TOPK && tile_ok && rt >= p.z_begin && r_local < p.z_rows)      // (one row tile of either kind)
+                zrow = (rt < p.row_tiles0 && p.zt_out != nullptr ? p.zt_out : p.z_out) + static_cast<long long>(r_local) * p.z_pitch;
             const int t0 = first_tile(rt, ln);
             const int nt = (p.col_tiles - ln + S - 1) / S;
             for (int t = t0; t < nt; ++t) {
@@ -1852,9 +1853,11 @@ __global__ void __launch_bounds__(256) loss_patch_kernel(const __grid_constant__
 
 // ---------------------------------------------------------------------------------------------
 // dz_kernel: one block per row, after a sweep that left the draft logits of few rows in fp32. Merges the draft's partial
-// statistics into lse_d, evaluates Eq. 1 from the logits at Omega_hat, and turns the row into
+// statistics into lse_d, evaluates Eq. 1 from the logits at Omega_hat, and (make_dz) turns the row into
 // dz_d(v) = g (S_q p(v) - q(v) [v in Omega_hat]) in bf16, in place: the bf16 row begins where the fp32 row did. Every step
 // reads a piece twice as long as the one it writes, and a piece is written after all threads have read theirs.
+// With the target's logits (COMBINED) it is the combined objective's
+// dz_d(v) = g ((1 + w S_q) p(v) - q(v) - w q(v) [v in Omega_hat]), and the cross-entropy sum_v q(v) (lse_d - z_d(v)).
 // Bound by the latency of one pass over a row of 4 V bytes: DZ_THREADS threads with DZ_LOADS 16-byte loads each in flight.
 constexpr int DZ_THREADS = 1024;
 constexpr int DZ_LOADS = 4;
@@ -1872,9 +1875,17 @@ struct DzParams {
     float* lse_d;
     float* z;              // [N, pitch] in: logits (columns up to the pitch readable); out: bf16 [N, 2 pitch]
     long long pitch;       // a multiple of 256
+    int make_dz;
+    // COMBINED
+    const float* zt;       // [N, pitch] target logits
+    const float* lse_t;
+    float w;
+    float* loss_ce;
 };
 
+template <bool COMBINED>
 __global__ void __launch_bounds__(DZ_THREADS) dz_kernel(const __grid_constant__ DzParams p) {
+    __shared__ float sh_ce[DZ_THREADS / 32];
     __shared__ int sh_tok[K_CAP];
     __shared__ float sh_q[K_CAP];
     __shared__ float sh_z[K_CAP];
@@ -1918,7 +1929,11 @@ __global__ void __launch_bounds__(DZ_THREADS) dz_kernel(const __grid_constant__ 
         }
     }
     __syncthreads();
-    const float S_q = sh_sum[1], c = g * S_q, shift = -lse_d * LOG2E;
+    if (!p.make_dz) return;
+    const float S_q = sh_sum[1], c = COMBINED ? g * (1.f + p.w * S_q) : g * S_q, shift = -lse_d * LOG2E;
+    const float* trow = COMBINED ? p.zt + static_cast<long long>(row) * p.pitch : nullptr;
+    const float shift_t = COMBINED ? -p.lse_t[row] * LOG2E : 0.f;
+    float ce = 0.f;
     for (long long c0 = 0; c0 < p.pitch; c0 += DZ_LOADS * DZ_THREADS * 4) {
         float4 v[DZ_LOADS];
 #pragma unroll
@@ -1926,19 +1941,56 @@ __global__ void __launch_bounds__(DZ_THREADS) dz_kernel(const __grid_constant__ 
             const long long at = c0 + (u * DZ_THREADS + tid) * 4;
             if (at < p.pitch) v[u] = *reinterpret_cast<const float4*>(zrow + at);
         }
+        float4 t[COMBINED ? DZ_LOADS : 1];
+        if (COMBINED) {
+#pragma unroll
+            for (int u = 0; u < DZ_LOADS; ++u) {
+                const long long at = c0 + (u * DZ_THREADS + tid) * 4;
+                if (at < p.pitch) t[COMBINED ? u : 0] = *reinterpret_cast<const float4*>(trow + at);
+            }
+        }
         __syncthreads();
 #pragma unroll
         for (int u = 0; u < DZ_LOADS; ++u) {
             const long long at = c0 + (u * DZ_THREADS + tid) * 4;
-            if (at < p.pitch)
-                *reinterpret_cast<uint2*>(drow + at) =
-                    make_uint2(pack_bf16x2(c * ex2(fmaf(v[u].x, LOG2E, shift)), c * ex2(fmaf(v[u].y, LOG2E, shift))),
-                               pack_bf16x2(c * ex2(fmaf(v[u].z, LOG2E, shift)), c * ex2(fmaf(v[u].w, LOG2E, shift))));
+            if (at < p.pitch) {
+                float z[4] = {v[u].x, v[u].y, v[u].z, v[u].w}, o[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) o[j] = c * ex2(fmaf(z[j], LOG2E, shift));
+                if (COMBINED) {
+                    const float4& tu = t[COMBINED ? u : 0];
+                    const float zt[4] = {tu.x, tu.y, tu.z, tu.w};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float q = ex2(fmaf(zt[j], LOG2E, shift_t));
+                        o[j] = fmaf(-g, q, o[j]);
+                        if (at + j < p.V) ce = fmaf(q, lse_d - z[j], ce);      // (-inf beyond the vocabulary)
+                    }
+                }
+                *reinterpret_cast<uint2*>(drow + at) = make_uint2(pack_bf16x2(o[0], o[1]), pack_bf16x2(o[2], o[3]));
+            }
         }
     }
+    if (COMBINED) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ce += __shfl_xor_sync(0xffffffffu, ce, o);
+        if (lane == 0) sh_ce[warp] = ce;
+    }
     __syncthreads();
-    if (tid < K && sh_tok[tid] >= 0)
-        drow[sh_tok[tid]] = __float2bfloat16_rn(c * ex2(fmaf(sh_z[tid], LOG2E, shift)) - g * sh_q[tid]);
+    if (tid < K && sh_tok[tid] >= 0) {
+        float o = c * ex2(fmaf(sh_z[tid], LOG2E, shift));
+        if (COMBINED)
+            o -= g * ex2(fmaf(trow[sh_tok[tid]], LOG2E, shift_t)) + g * p.w * sh_q[tid];
+        else
+            o -= g * sh_q[tid];
+        drow[sh_tok[tid]] = __float2bfloat16_rn(o);
+    }
+    if (COMBINED && warp == 0) {
+        float v = sh_ce[lane];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) p.loss_ce[row] = v;
+    }
 }
 
 // ---------------------------------------------------------------------------------------------
