@@ -206,8 +206,9 @@ __global__ void __launch_bounds__(256, 2) hca_bwd_rows_kernel(const __grid_const
 }
 
 // dQ = the fp32 accumulator as bf16; 8 values per thread.
-__global__ void __launch_bounds__(256) hca_dq_convert_kernel(const float* __restrict__ acc, __nv_bfloat16* __restrict__ dQ,
+__global__ void __launch_bounds__(256) hca_dq_convert_kernel(const float* acc, __nv_bfloat16* dQ,
                                                              long long n8) {
+    wait_previous_kernel();
     const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= n8) return;
     float v[8];
@@ -327,6 +328,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_bwd_fused_kernel(const __g
         tmem_alloc(smem_u32(tmem_ptr_smem), F_TMEM_COLS);
         tmem_relinquish();
     }
+    wait_previous_kernel();
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -411,7 +413,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_bwd_fused_kernel(const __g
                 for (int u = 0; u < 2; ++u) {
                     const int t = jq * QE + lane + 32 * u;
                     nl[u] = t < p.T ? -__ldg(p.lse + rowbase + t) * 1.4426950408889634f : -INFINITY;
-                    nd[u] = t < p.T ? -__ldg(p.D + rowbase + t) * p.scale : 0.f;
+                    nd[u] = t < p.T ? -__ldcg(p.D + rowbase + t) * p.scale : 0.f;
                 }
                 if (lane == 0) ok = wait_barrier(qd_empty(s), ((gq / F_STAGES) & 1u) ^ 1u, abort_flag, p.status, 3);
                 ok = __shfl_sync(0xffffffffu, ok, 0);

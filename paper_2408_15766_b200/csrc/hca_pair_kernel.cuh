@@ -170,6 +170,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
         tmem_alloc(smem_u32(tmem_ptr_smem), TMEM_COLS);
         tmem_relinquish();
     }
+    wait_previous_kernel();
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();

@@ -374,7 +374,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
     constexpr bool B_MN_MAJOR = (MODE == MODE_OUT);
     // conditional launch (the second pass that follows every spilling call): nothing to do unless the first reported a
     // row beyond its exponent range
-    if (p.gate != nullptr && *p.gate == 0u) return;
+    if (p.gate != nullptr) {
+        wait_previous_kernel();
+        if (*p.gate == 0u) return;
+    }
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t smemA = smem_base;
@@ -424,6 +427,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
             tmem_relinquish();
         }
     }
+    if (p.gate == nullptr) wait_previous_kernel();
     tc_fence_before_sync();
     __syncthreads();
     if (CG == 2) cluster_sync();      // the partner's barriers are initialised, its tensor memory is allocated
@@ -1111,6 +1115,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
 // out_reduce_kernel: adds up the partial tiles of MODE_OUT in the order of the contraction and finishes them as its
 // epilogue does. One thread per four columns; memory-bound (reads cuts x, writes 1 x the rest tiles).
 __global__ void __launch_bounds__(256) out_reduce_kernel(const __grid_constant__ GemmParams p) {
+    wait_previous_kernel();
     if (p.gate != nullptr && *p.gate == 0u) return;
     const OutPlan& o = p.plan;
     const long long i = static_cast<long long>(blockIdx.x) * 256 + threadIdx.x;
@@ -1229,6 +1234,7 @@ __device__ __forceinline__ void unpack8(const uint4& v, float (&f)[8]) {
 // in select_kernel; 1024 rows, 10 tokens: 144 -> 55 us): bound by the latency of the gathered rows of W, so that a row's columns are spread over FIN_WARPS
 // warps (8 columns per thread and step) and FIN_GRP rows of W are in flight per thread.
 __global__ void __launch_bounds__(FIN_WARPS * 32) finalize_kernel(const __grid_constant__ FinalizeParams p) {
+    wait_previous_kernel();
     if (p.gate != nullptr && *p.gate == 0u) return;
     __shared__ int sh_tok[K_CAP];         // Omega_hat of the row (the bi-directional set needs 2K <= K_CAP)
     __shared__ float sh_q[K_CAP];
@@ -1566,6 +1572,7 @@ __global__ void __launch_bounds__(sel_block_warps(WARPS) * 32) select_kernel(con
     const int rib = warp / WARPS, w = warp % WARPS;           // row in the block, warp of the row
     const int tid = w * 32 + lane;                            // thread of the row
     const int local = blockIdx.x * ROWS + rib;
+    wait_previous_kernel();
     if (local >= p.rows || (p.gate != nullptr && *p.gate == 0u)) return;      // (WARPS > 1: the whole block)
     auto sync_row = [&]() {
         if (WARPS > 1)
@@ -1809,6 +1816,7 @@ struct LossPatchParams {
 };
 
 __global__ void __launch_bounds__(256) loss_patch_kernel(const __grid_constant__ LossPatchParams p) {
+    wait_previous_kernel();
     if (p.gate != nullptr && *p.gate == 0u) return;
     const int lane = threadIdx.x & 31;
     const int local = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -1893,6 +1901,7 @@ __global__ void __launch_bounds__(DZ_THREADS) dz_kernel(const __grid_constant__ 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int row = blockIdx.x;
     const int K = p.K;
+    wait_previous_kernel();
     float* zrow = p.z + static_cast<long long>(row) * p.pitch;
     __nv_bfloat16* drow = reinterpret_cast<__nv_bfloat16*>(zrow);
     if (tid < K) {
@@ -1997,11 +2006,12 @@ __global__ void __launch_bounds__(DZ_THREADS) dz_kernel(const __grid_constant__ 
 // ce_kernel (combined objective): one warp per row of a chunk. T[local, :] = q W of the row (from the second
 // GEMM over the target spill). Full-vocabulary cross-entropy -sum_v q log p = lse_d - <H_d[row], q W>, and the
 // (with the fp32 correction of the Omega_hat terms from finalize) the q W row joins the row's Omega_hat term so that dH_d = coef (draft spill x W) - sparse.
-__global__ void __launch_bounds__(256) ce_kernel(int rows, int row_begin, int d, const __nv_bfloat16* __restrict__ H_d,
-                                                 const float* __restrict__ T, const float* __restrict__ lse_d,
-                                                 const float* __restrict__ grad_loss, const float* __restrict__ ce_corr,
-                                                 float* __restrict__ loss_ce, float* __restrict__ sparse,
-                                                 const unsigned int* __restrict__ gate) {
+__global__ void __launch_bounds__(256) ce_kernel(int rows, int row_begin, int d, const __nv_bfloat16* H_d,
+                                                 const float* T, const float* lse_d,
+                                                 const float* grad_loss, const float* ce_corr,
+                                                 float* loss_ce, float* sparse,
+                                                 const unsigned int* gate) {
+    wait_previous_kernel();
     if (gate != nullptr && *gate == 0u) return;
     const int lane = threadIdx.x & 31;
     const int local = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -2063,12 +2073,13 @@ __global__ void wait_expiry_selftest_kernel(unsigned int* status, unsigned long 
 // increasing order; entries cut by Top-P carry id -1 and come first) by ranking every entry against the
 // others, and precomputes g * q, g * S_q and lse_d * log2(e).
 constexpr int PREP_WARPS = 4;
-__global__ void __launch_bounds__(PREP_WARPS * 32) bwd_prep_kernel(int N, int K, const int* __restrict__ idx,
-                                                                    const float* __restrict__ q,
-                                                                    const float* __restrict__ lse_d,
-                                                                    const float* __restrict__ grad_loss,
-                                                                    int* __restrict__ sidx, float* __restrict__ sgq,
-                                                                    float* __restrict__ coef, float* __restrict__ lse2) {
+__global__ void __launch_bounds__(PREP_WARPS * 32) bwd_prep_kernel(int N, int K, const int* idx,
+                                                                    const float* q,
+                                                                    const float* lse_d,
+                                                                    const float* grad_loss,
+                                                                    int* sidx, float* sgq,
+                                                                    float* coef, float* lse2) {
+    wait_previous_kernel();
     __shared__ int s_tok[PREP_WARPS][K_CAP];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int row = blockIdx.x * PREP_WARPS + wib;

@@ -70,6 +70,16 @@ __device__ __forceinline__ bool wait_barrier(uint32_t bar, uint32_t parity, vola
     }
 }
 
+// ---- programmatic dependent launch ------------------------------------------------------------
+// Every kernel of the library is launched as a dependent of the one before it in the stream: its blocks may start, and set
+// up barriers and tensor memory, while that one drains. wait_previous_kernel returns when that one has completed and its
+// writes are visible; nothing it wrote is read, and nothing it reads is written, before. (A kernel that waits here at its
+// start orders all earlier ones too.) Data that the previous kernel wrote is not read with ld.global.nc, which the
+// compiler may move.
+__device__ __forceinline__ void wait_previous_kernel() {
+    asm volatile("griddepcontrol.wait;\ngriddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---- TMA ------------------------------------------------------------------------------------
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* tm) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tm)) : "memory");
