@@ -154,7 +154,7 @@ int hass_topk_distill_bwd(const void* H_d, const void* W, int64_t N, int64_t d, 
  * the Top-P variant work the same way, and so do hass_combined_distill_fwd_bwd and the Bi-directional
  * variant, whose exponent comes from the row's largest logit among the first 256 tokens and whose
  * second pass repeats the whole sequence.
- * Calls of at most 64 rows sweep both feature sets in one launch and keep the draft logits in fp32 between
+ * Calls of at most 128 rows sweep both feature sets in one launch and keep the draft logits in fp32 between
  * the sweep and the second GEMM; they have no range condition and no second pass.
  * (HASS_ERR_RANGE is kept for callers that name it; no entry point of this version returns it.)
  */

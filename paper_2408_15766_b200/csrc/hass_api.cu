@@ -49,6 +49,8 @@ struct KernelTimer {
 // duration of a pair's step (256 x 256 outputs) over that of two single CTAs (128 x 256 outputs each); measured 0.89-0.92
 constexpr double kPairStepTime = 0.90;
 
+constexpr int MAX_CLUSTER = 8;
+
 typedef void (*GemmFn)(GemmParams);
 
 // Launches `fn` as a programmatic dependent of the stream's previous kernel (see wait_previous_kernel), in clusters of
@@ -82,6 +84,7 @@ static int launch(void (*fn)(P...), long long grid, int block, size_t smem, cuda
 struct DeviceInfo {
     int ok = 0;   // 0 unknown, 1 usable, <0 hass_status
     int sms = 148;
+    int clusters[MAX_CLUSTER + 1] = {};   // clusters of this many CTAs of the second GEMM that are resident at once
 };
 static DeviceInfo g_dev[64];
 
@@ -115,6 +118,23 @@ static int device_info(DeviceInfo* out) {
             if (e3 == cudaSuccess) e3 = cudaFuncSetAttribute(select_kernel<16, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * 1024 * 8);
             cudaError_t e4 = cudaFuncSetAttribute(hca2::hca_attention_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hca2::SMEM_BYTES);
             if (e4 == cudaSuccess) e4 = cudaFuncSetAttribute(hca_bwd::hca_bwd_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hca_bwd::F_SMEM_BYTES);
+            for (int c = 2; c <= MAX_CLUSTER; ++c) {
+                cudaLaunchConfig_t cfg = {};
+                cfg.gridDim = dim3(c);
+                cfg.blockDim = dim3(NUM_THREADS);
+                cfg.dynamicSmemBytes = SMEM_BYTES;
+                cudaLaunchAttribute at;
+                at.id = cudaLaunchAttributeClusterDimension;
+                at.val.clusterDim.x = c;
+                at.val.clusterDim.y = 1;
+                at.val.clusterDim.z = 1;
+                cfg.attrs = &at;
+                cfg.numAttrs = 1;
+                if (cudaOccupancyMaxActiveClusters(&di.clusters[c], gemm_kernel<MODE_OUT, TOPK_BUF, 1>, &cfg) != cudaSuccess) {
+                    cudaGetLastError();
+                    di.clusters[c] = 0;
+                }
+            }
             if (e3 != cudaSuccess || e4 != cudaSuccess) {
                 cudaGetLastError();
                 return HASS_ERR_CUDA;
@@ -219,7 +239,10 @@ constexpr int kPartTilesMax = 296;      // partial tiles of one CTA each, at mos
 // the partial tiles' way to memory and back (4 TB/s) and one fill and drain of the pipeline (6 steps) per piece.
 // Measured (second GEMM alone): 61 rows x 4096 x 32000 179 -> 56 us (16 tiles in 16 x 8 pieces on 128 of the SMs), 517
 // rows x 4096 x 128256 822 -> 657 us, the 28-row-tile chunk of 8192 rows 4 rounds of 74 pairs -> 3 and a cut rest.
-static OutPlan plan_out(int rows, int CT, int kb, int sms, size_t part_bytes) {
+// A tile per cluster needs no partial tiles and no second kernel; it costs the exchange (6 steps) and fits while all
+// clusters are resident at once (clusters[]: how many are; nullptr: not considered).
+// 250 rows x 4096 x 32000, whose partial tiles do not fit the workspace: call 318 -> 235 us.
+static OutPlan plan_out(int rows, int CT, int kb, int sms, size_t part_bytes, const int* clusters) {
     const int RT = (rows + BM - 1) / BM;
     const int part_rows = RT == 1 ? rows : BM;      // rows kept of a partial tile
     const size_t tile_bytes = static_cast<size_t>(part_rows) * BN * 4;
@@ -244,6 +267,7 @@ static OutPlan plan_out(int rows, int CT, int kb, int sms, size_t part_bytes) {
                 best_cost = cost;
                 best.pair = pair;
                 best.part_rows = part_rows;
+                best.cluster = 1;
                 best.row_units = units;
                 best.whole = cuts == 1 ? static_cast<int>(tiles) : whole;
                 best.rest = cuts == 1 ? 0 : rest;
@@ -253,6 +277,20 @@ static OutPlan plan_out(int rows, int CT, int kb, int sms, size_t part_bytes) {
                                                                                                             : groups);
             }
         }
+    }
+    for (int c = 2; clusters && c <= MAX_CLUSTER; ++c) {
+        const long long tiles = static_cast<long long>(RT) * CT;
+        const double cost = (kb + c - 1) / c + 6. + 6.;
+        if (tiles > clusters[c] || kb < 2 * c || cost >= best_cost) continue;
+        best_cost = cost;
+        best = OutPlan{};
+        best.pair = 1;
+        best.row_units = RT;
+        best.whole = static_cast<int>(tiles);
+        best.cuts = 1;
+        best.groups = static_cast<int>(tiles) * c;
+        best.part_rows = part_rows;
+        best.cluster = c;
     }
     return best;
 }
@@ -398,8 +436,15 @@ static int make_layout(long long N, long long d, long long V, int K, int sms, La
     for (long long rows : chunks) {
         if (rows < 1) continue;
         const size_t need = part_bytes_of(plan_out(static_cast<int>(rows), ceil_div(d, BN), ceil_div(V, BK), sms,
-                                                   L->scratch_row_tile_bytes - 256));
+                                                   L->scratch_row_tile_bytes - 256, nullptr));
         if (need > L->part_bytes) L->part_bytes = need;
+    }
+    if (N > BM / 2 && N <= BM) {
+        // the fp32 logits of such a call (narrow_room), from `sparse` on
+        const size_t z_end = L->sparse + static_cast<size_t>(N) * L->p_pitch * 4;
+        const size_t most = L->scratch_row_tile_bytes - 256;
+        const size_t need = z_end > L->total_pref ? align256(z_end - L->total_pref) : 0;
+        if (need <= most && need > L->part_bytes) L->part_bytes = need;
     }
     return HASS_OK;
 }
@@ -439,7 +484,7 @@ static int launch_gemm(const GemmParams& p, cudaStream_t st, int kind = -1) {
         fn = pair ? gemm_kernel<MODE_STATS, TOPK_REG, 2> : gemm_kernel<MODE_STATS, TOPK_REG, 1>;
     else
         fn = pair ? gemm_kernel<MODE, TOPK_BUF, 2> : gemm_kernel<MODE, TOPK_BUF, 1>;
-    return launch(fn, p.sched.max_ctas, NUM_THREADS, SMEM_BYTES, st, pair ? 2 : 1, p);
+    return launch(fn, p.sched.max_ctas, NUM_THREADS, SMEM_BYTES, st, MODE == MODE_OUT && p.plan.cluster > 1 ? p.plan.cluster : pair ? 2 : 1, p);
 }
 
 // Clears the status block (only_thresholds: not) and the published thresholds of `slots` slots.
@@ -527,16 +572,16 @@ static PartRoom part_room(uint8_t* ws, size_t workspace_bytes, const Layout& L, 
 }
 
 // The second GEMM (MODE_OUT) over p.row_tiles row tiles: plan, tiles, and the sum of the partial tiles.
-static int launch_out(GemmParams& p, const PartRoom& room, int sms, cudaStream_t st) {
+static int launch_out(GemmParams& p, const PartRoom& room, const DeviceInfo& di, cudaStream_t st) {
     const long long left = p.rows_valid - p.row_global_offset;
     const int rows = static_cast<int>(left < static_cast<long long>(p.row_tiles) * BM ? left : p.row_tiles * BM);
-    p.plan = plan_out(rows, p.col_tiles, p.k_blocks, sms, room.bytes);
+    p.plan = plan_out(rows, p.col_tiles, p.k_blocks, di.sms, room.bytes, di.clusters);
     p.part = room.at;
     p.sched.pair = p.plan.pair;
     p.sched.max_ctas = p.plan.groups * p.plan.pair;
     if (kLog)
-        std::fprintf(stderr, "[hass] out: pair %d, grid %d, %d whole tiles, %d rest tiles x %d cuts\n", p.plan.pair, p.sched.max_ctas,
-                     p.plan.whole, p.plan.rest, p.plan.cuts);
+        std::fprintf(stderr, "[hass] out: pair %d, cluster %d, grid %d, %d whole tiles, %d rest tiles x %d cuts\n", p.plan.pair,
+                     p.plan.cluster, p.sched.max_ctas, p.plan.whole, p.plan.rest, p.plan.cuts);
     const int rc = launch_gemm<MODE_OUT>(p, st);
     if (rc != HASS_OK || p.plan.rest == 0) return rc;
     KernelTimer timer(p.gate ? KIND_CONDITIONAL : KIND_OUT, st);
@@ -731,7 +776,7 @@ static int backward_impl(const void* H_d, const void* W, long long N, long long 
         o.out_align32 = ((reinterpret_cast<uintptr_t>(dH_d) | static_cast<uintptr_t>(d * (dH_dtype == HASS_FP32 ? 4 : 2))) & 31u) == 0 ? 1 : 0;
         o.out_pitch = d;
         o.status = p.status;
-        rc = launch_out(o, part, di.sms, st);
+        rc = launch_out(o, part, di, st);
         if (rc != HASS_OK) return rc;
     }
     return HASS_OK;
@@ -753,24 +798,41 @@ struct Combined {
     __nv_bfloat16* Pt;     // [chunk rows, p_pitch] scratch: spill of the target tiles
 };
 
-// Rows of one call up to which the draft logits go through the workspace in fp32 (narrow_impl): two rows of 128-row bf16
-// scratch hold one of them. Up to here a call is bound by reading W, which this route does twice (both sweeps in one
-// launch, then the second GEMM) instead of three times, with no range condition and so no second pass: 61 rows x 4096 x
-// 32000 211 -> 147 us, 64 rows x 256 x 1024 67 -> 46 us. Beyond, the fp32 logits would not fit a workspace of one row tile.
-constexpr int kNarrowRows = BM / 2;
+// Calls of one row tile, where the draft logits go through the workspace in fp32 (narrow_impl). Such a call is bound by
+// reading W, which this route does twice (both sweeps in one launch, then the second GEMM) instead of three times, with no
+// range condition and so no second pass: 61 rows x 4096 x 32000 211 -> 147 us, 64 rows x 256 x 1024 67 -> 46 us, 100 rows
+// x 4096 x 32000 215 -> 147 us. Up to 64 rows they fit the scratch of one row tile; beyond, the fp32 rows kept for the
+// Omega_hat term and the room for partial tiles serve too, and a workspace that ends before them takes the other route.
+struct NarrowRoom {
+    float* z = nullptr;      // [N, p_pitch], or nullptr: no room
+    PartRoom part;           // what is left for partial tiles
+};
+static NarrowRoom narrow_room(long long N, uint8_t* ws, size_t workspace_bytes, const Layout& L, const PartRoom& part) {
+    NarrowRoom r;
+    const size_t need = static_cast<size_t>(N) * L.p_pitch * 4;
+    if (N <= BM / 2 && workspace_bytes >= L.scratch + need) {
+        r.z = reinterpret_cast<float*>(ws + L.scratch);
+        r.part = part;
+    } else if (N <= BM && workspace_bytes >= L.sparse + need) {
+        r.z = reinterpret_cast<float*>(ws + L.sparse);
+    }
+    return r;
+}
 
 static int narrow_impl(bool with_target, const void* H_t, const void* H_d, const void* W, int N, long long d, long long V,
                        int K, const float* grad_loss, const int* idx_in, const float* q_in, float* loss, int* idx_out,
                        float* q_out, float* lse_t, float* lse_d, void* dH_d, int dH_dtype, uint8_t* ws, const Layout& L,
-                       const PartRoom& part, int sms, cudaStream_t st, float top_p, int* topk_n, const Combined* cmb = nullptr) {
+                       const NarrowRoom& room, const DeviceInfo& di, cudaStream_t st, float top_p, int* topk_n,
+                       const Combined* cmb = nullptr) {
     const int CT = ceil_div(V, BN), DT = ceil_div(d, BN);
     unsigned int* status = reinterpret_cast<unsigned int*>(ws + L.status);
-    float* z = reinterpret_cast<float*>(ws + L.scratch);
+    float* z = room.z;
+    const PartRoom& part = room.part;
     // (1) target and draft rows in one sweep: statistics, candidates, the draft's logits
     GemmParams p;
     std::memset(&p, 0, sizeof(p));
     p.row_tiles = with_target ? 2 : 1;
-    int rc = plan_launch(p.row_tiles, CT, sms, L.slot_cap, &p.sched);
+    int rc = plan_launch(p.row_tiles, CT, di.sms, L.slot_cap, &p.sched);
     if (rc != HASS_OK) return rc;
     log_schedule("narrow sweep", p.sched);
     rc = make_tmap(&p.tmA1, H_d, N, d, d, BK, BM);
@@ -806,7 +868,7 @@ static int narrow_impl(bool with_target, const void* H_t, const void* H_d, const
         SelectParams sp = select_params(p, 0, 0, N, idx_out, q_out, K, lse_t);
         sp.n_out = topk_n;
         sp.top_p = top_p;
-        rc = launch_select(sp, sms, st);
+        rc = launch_select(sp, di.sms, st);
         if (rc != HASS_OK) return rc;
     }
     // (3) lse_d, loss, dz_d
@@ -858,7 +920,7 @@ static int narrow_impl(bool with_target, const void* H_t, const void* H_d, const
     o.out_align32 = ((reinterpret_cast<uintptr_t>(dH_d) | static_cast<uintptr_t>(d * (dH_dtype == HASS_FP32 ? 4 : 2))) & 31u) == 0 ? 1 : 0;
     o.out_pitch = d;
     o.status = status;
-    return launch_out(o, part, sms, st);
+    return launch_out(o, part, di, st);
 }
 
 static int fused_impl(bool with_target, const void* H_t, const void* H_d, const void* W, long long N, long long d,
@@ -895,9 +957,9 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
     __nv_bfloat16* P = reinterpret_cast<__nv_bfloat16*>(ws + L.scratch);
     unsigned int* status = reinterpret_cast<unsigned int*>(ws + L.status);
     int* idx_d = reinterpret_cast<int*>(ws + L.sidx);
-    if (cmb && with_target && N <= kNarrowRows)
+    if (cmb && with_target && N <= BM / 2)      // (the target's fp32 logits take the place of its spill: one row tile of scratch)
         return narrow_impl(true, H_t, H_d, W, static_cast<int>(N), d, V, K, grad_loss, nullptr, nullptr, loss, idx_out, q_out, lse_t,
-                           lse_d, dH_d, dH_dtype, ws, L, part, di.sms, st, 0.f, nullptr, cmb);
+                           lse_d, dH_d, dH_dtype, ws, L, narrow_room(N, ws, workspace_bytes, L, part), di, st, 0.f, nullptr, cmb);
     CUtensorMap tmHt, tmHd, tmWn, tmP;
     rc = make_tmap(&tmHd, H_d, N, d, d, BK, BM);
     if (rc == HASS_OK) rc = with_target ? make_tmap(&tmHt, H_t, N, d, d, BK, BM) : make_tmap(&tmHt, H_d, N, d, d, BK, BM);
@@ -1031,7 +1093,7 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
             t.out_pitch = d;
             t.status = status;
             t.gate = gate;
-            rc = launch_out(t, part, di.sms, st);
+            rc = launch_out(t, part, di, st);
             if (rc != HASS_OK) return rc;
             {
                 KernelTimer timer(retry ? KIND_CONDITIONAL : KIND_FINALIZE, st);
@@ -1062,7 +1124,7 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
         o.out_pitch = d;
         o.status = status;
         o.gate = gate;
-        rc = launch_out(o, part, di.sms, st);
+        rc = launch_out(o, part, di, st);
         if (rc != HASS_OK) return rc;
     }
     return HASS_OK;
@@ -1140,7 +1202,7 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
                        long long V, int K, const float* grad_loss, const int* idx_in, const float* q_in, float* loss,
                        int* idx_out, float* q_out, float* lse_t, float* lse_d, void* dH_d, int dH_dtype,
                        void* workspace, size_t workspace_bytes, cudaStream_t st, float top_p = 0.f,
-                       int* topk_n = nullptr, ChunkPipe* pipe = nullptr, const PartRoom* room = nullptr) {
+                       int* topk_n = nullptr, ChunkPipe* pipe = nullptr) {
     int rc = check_sizes(N, d, V, K);
     if (rc != HASS_OK) return rc;
     if (!H_d || !W || !loss || !lse_d || !dH_d || !aligned16(H_d) || !aligned16(W) || !aligned16(dH_d))
@@ -1163,19 +1225,20 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
     int chunk_tiles = L.pref_chunk_tiles;
     if (fit < chunk_tiles) chunk_tiles = even_chunk(static_cast<int>(fit), RT);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
-    const PartRoom part = part_room(ws, workspace_bytes, L, chunk_tiles, room, true);
+    const PartRoom part = part_room(ws, workspace_bytes, L, chunk_tiles, nullptr, true);
     int* sidx = reinterpret_cast<int*>(ws + L.sidx);
     float* sq = reinterpret_cast<float*>(ws + L.sgq);
     float* coef = reinterpret_cast<float*>(ws + L.coef);
     float* capz = reinterpret_cast<float*>(ws + L.capz);
     float* ref2 = reinterpret_cast<float*>(ws + L.lse2);
-    if (N <= kNarrowRows) {
+    const NarrowRoom narrow = narrow_room(N, ws, workspace_bytes, L, part);
+    if (narrow.z) {
         if (pipe) {
             rc = pipe_in(pipe, H_t, H_d, 0, static_cast<size_t>(N), st);
             if (rc != HASS_OK) return rc;
         }
         rc = narrow_impl(with_target, H_t, H_d, W, static_cast<int>(N), d, V, K, grad_loss, idx_in, q_in, loss, idx_out, q_out,
-                         lse_t, lse_d, dH_d, dH_dtype, ws, L, part, di.sms, st, top_p, topk_n);
+                         lse_t, lse_d, dH_d, dH_dtype, ws, L, narrow, di, st, top_p, topk_n);
         if (rc != HASS_OK || !pipe) return rc;
         return pipe_out(pipe, dH_d, 0, static_cast<size_t>(N), st);
     }
@@ -1333,7 +1396,7 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
             o.out_pitch = d;
             o.status = status;
             o.gate = gate;
-            rc = launch_out(o, part, di.sms, st);
+            rc = launch_out(o, part, di, st);
             if (rc != HASS_OK) return rc;
             if (pipe && !retry) {
                 rc = pipe_out(pipe, dH_d, static_cast<size_t>(t0) * BM, static_cast<size_t>(rows), st);
@@ -1376,9 +1439,10 @@ static int forward2_impl(bool with_target, const void* H_t, const void* H_d, con
                             workspace, workspace_bytes, st);
     const int RT = ceil_div(N, BM), CT = ceil_div(V, BN);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
-    if (N <= kNarrowRows && workspace_bytes >= L.fixed_end + L.scratch_row_tile_bytes)
+    const NarrowRoom narrow = narrow_room(N, ws, workspace_bytes, L, PartRoom());
+    if (narrow.z)
         return narrow_impl(with_target, H_t, H_d, W, static_cast<int>(N), d, V, K, nullptr, idx_in, q_in, loss, idx_out, q_out,
-                           lse_t, lse_d, nullptr, HASS_BF16, ws, L, PartRoom(), di.sms, st, 0.f, nullptr);
+                           lse_t, lse_d, nullptr, HASS_BF16, ws, L, narrow, di, st, 0.f, nullptr);
     GemmParams p;
     std::memset(&p, 0, sizeof(p));
     rc = plan_launch(RT, CT, di.sms, L.slot_cap, &p.sched);
@@ -1728,16 +1792,16 @@ int hass_combined_distill_fwd_bwd(const void* H_t, const void* H_d, const void* 
                       lse_d, dH_d, dH_dtype, workspace, c.base, static_cast<cudaStream_t>(cuda_stream), &cmb, nullptr, false, &room);
 }
 
-// Device staging appended to the normal workspace by the *_host entry.
+// Device staging appended to the normal workspace (base bytes; with_part: as hass_topk_distill_workspace_bytes gives
+// it, else without the room that calls can do without) by the *_host entry.
 struct HostStage {
-    size_t base, H_t, H_d, grad, loss, idx, q, lse_t, lse_d, dH, total, part_bytes;   // base, part_bytes: as in CombinedStage
+    size_t base, H_t, H_d, grad, loss, idx, q, lse_t, lse_d, dH, total;
 };
-static int host_stage(int64_t N, int64_t d, int64_t V, int32_t K, int dH_dtype, HostStage* s) {
+static int host_stage(int64_t N, int64_t d, int64_t V, int32_t K, int dH_dtype, bool with_part, HostStage* s) {
     Layout L;
     const int rc = make_layout(N, d, V, K, sm_count_or_default(), &L);
     if (rc != HASS_OK) return rc;
-    s->base = L.total_pref;
-    s->part_bytes = L.part_bytes;
+    s->base = L.total_pref + (with_part ? L.part_bytes : 0);
     size_t off = align256(s->base);
     s->H_t = off;
     off = align256(off + static_cast<size_t>(N) * d * 2);
@@ -1766,9 +1830,9 @@ int hass_topk_distill_host_workspace_bytes(int64_t N, int64_t d, int64_t V, int3
     int rc = check_sizes(N, d, V, K);
     if (rc != HASS_OK) return rc;
     HostStage s;
-    rc = host_stage(N, d, V, K, dH_dtype, &s);
+    rc = host_stage(N, d, V, K, dH_dtype, true, &s);
     if (rc != HASS_OK) return rc;
-    *bytes = s.total + s.part_bytes;
+    *bytes = s.total;
     return HASS_OK;
 }
 
@@ -1811,14 +1875,12 @@ int hass_topk_distill_fwd_bwd_host(const void* H_t_host, const void* H_d_host, c
     if (dH_dtype != HASS_BF16 && dH_dtype != HASS_FP32) return HASS_ERR_INVALID_ARG;
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u)) return HASS_ERR_WORKSPACE;
     HostStage s;
-    rc = host_stage(N, d, V, K, dH_dtype, &s);
+    rc = host_stage(N, d, V, K, dH_dtype, true, &s);
+    if (rc == HASS_OK && workspace_bytes < s.total) rc = host_stage(N, d, V, K, dH_dtype, false, &s);
     if (rc != HASS_OK) return rc;
     if (workspace_bytes < s.total) return HASS_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
-    PartRoom room;
-    room.at = reinterpret_cast<float*>(ws + s.total);
-    room.bytes = workspace_bytes - s.total;
     HostPipeResources* res = nullptr;
     rc = host_pipe_resources(&res);
     if (rc != HASS_OK) return rc;
@@ -1853,7 +1915,7 @@ int hass_topk_distill_fwd_bwd_host(const void* H_t_host, const void* H_d_host, c
     rc = fused2_impl(true, ws + s.H_t, ws + s.H_d, W, N, d, V, K, grad_dev, nullptr, nullptr,
                      reinterpret_cast<float*>(ws + s.loss), reinterpret_cast<int32_t*>(ws + s.idx),
                      reinterpret_cast<float*>(ws + s.q), reinterpret_cast<float*>(ws + s.lse_t),
-                     reinterpret_cast<float*>(ws + s.lse_d), ws + s.dH, dH_dtype, workspace, s.base, st, 0.f, nullptr, &pipe, &room);
+                     reinterpret_cast<float*>(ws + s.lse_d), ws + s.dH, dH_dtype, workspace, s.base, st, 0.f, nullptr, &pipe);
     if (rc == HASS_ERR_UNSUPPORTED) {
         // more row chunks than events (a very small workspace): one copy in, the call, one copy out
         const size_t hbytes = static_cast<size_t>(N) * d * 2;
@@ -1867,7 +1929,7 @@ int hass_topk_distill_fwd_bwd_host(const void* H_t_host, const void* H_d_host, c
         rc = fused2_impl(true, ws + s.H_t, ws + s.H_d, W, N, d, V, K, grad_dev, nullptr, nullptr,
                          reinterpret_cast<float*>(ws + s.loss), reinterpret_cast<int32_t*>(ws + s.idx),
                          reinterpret_cast<float*>(ws + s.q), reinterpret_cast<float*>(ws + s.lse_t),
-                         reinterpret_cast<float*>(ws + s.lse_d), ws + s.dH, dH_dtype, workspace, s.base, st, 0.f, nullptr, nullptr, &room);
+                         reinterpret_cast<float*>(ws + s.lse_d), ws + s.dH, dH_dtype, workspace, s.base, st);
         if (rc == HASS_OK && cudaMemcpyAsync(dH_d_host, ws + s.dH, static_cast<size_t>(N) * pipe.out_row_bytes,
                                              cudaMemcpyDeviceToHost, st) != cudaSuccess) {
             cudaGetLastError();

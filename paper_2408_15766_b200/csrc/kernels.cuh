@@ -72,9 +72,12 @@ struct Schedule {
 // tiles, which would leave most of a round idle, are cut into `cuts` equal pieces of the contraction that are dealt
 // out the same way (piece v = piece index v / rest of tile whole + v % rest: pieces at the same depth run together), stored as
 // fp32 partial tiles and added up by out_reduce_kernel. cuts = 1: whole = all tiles, rest = 0.
+// cluster > 1 (then pair = 1): every tile is one cluster's, whose CTAs take equal pieces of the contraction, hand their
+// accumulators to one another through distributed shared memory by rows, and add up and finish 128 / cluster rows each.
 struct OutPlan {
     int pair, groups, row_units, whole, rest, cuts;
     int part_rows;         // rows kept of a partial tile: BM, or all there are in a single row tile
+    int cluster;
 };
 
 struct GemmParams {
@@ -363,6 +366,21 @@ __device__ __forceinline__ int hist_top(uint32_t hist, int K) {
 enum { TOPK_REG = 0, TOPK_BUF = 1, TOPK_NONE = 2 };
 constexpr int K_REG = 16;
 
+// Four columns of a finished accumulator of MODE_OUT: row scale, Omega_hat term, store.
+__device__ __forceinline__ void finish_out4(const GemmParams& p, float4 a, int local_row, int row, int col) {
+    if (p.coef != nullptr) {
+        const float coef = p.coef[row];
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (p.sparse != nullptr) s = *reinterpret_cast<const float4*>(p.sparse + static_cast<long long>(local_row) * p.out_pitch + col);
+        a.x = fmaf(coef, a.x, -s.x); a.y = fmaf(coef, a.y, -s.y); a.z = fmaf(coef, a.z, -s.z); a.w = fmaf(coef, a.w, -s.w);
+    }
+    const long long at = static_cast<long long>(row) * p.out_pitch + col;
+    if (p.out_fp32)
+        *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + at) = a;
+    else
+        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + at) = make_uint2(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w));
+}
+
 // CG: CTAs per product. The kernel is bound by the tensor pipe and, in calls of many milliseconds, by the power cap. A pair
 // (tcgen05 cta_group::2, 256 x 256 tile) fetches 32 KB per CTA and k block instead of 48 (10 instead of 15 TB/s out of
 // L2) and reads half as much of B from shared memory; with the stages smaller there are six instead of four. A step of
@@ -435,10 +453,17 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
     const uint32_t tmem_base = *tmem_ptr_smem;
 
     // Calls f(row_tile, lane, S, slot, first k block, end of k blocks) for every item of this CTA; f returns false to
-    // stop. MODE_OUT: one column tile (= lane; S = all of them), slot = the partial tile it goes to or -1.
+    // stop. MODE_OUT: one column tile (= lane; S = all of them), slot = the partial tile it goes to, -1, or SHARED_TILE.
+    constexpr int SHARED_TILE = -2;
     auto for_each_item = [&](auto&& f) {
         if constexpr (MODE == MODE_OUT) {
             const OutPlan& o = p.plan;
+            if (CG == 1 && o.cluster > 1) {
+                const int u = cta / o.cluster, z = cta - u * o.cluster;
+                f(u % o.row_units, u / o.row_units, p.col_tiles, SHARED_TILE, static_cast<int>(static_cast<long long>(p.k_blocks) * z / o.cluster),
+                  static_cast<int>(static_cast<long long>(p.k_blocks) * (z + 1) / o.cluster));
+                return;
+            }
             for (int u = cta; u < o.whole; u += o.groups)
                 if (!f(u % o.row_units * CG + static_cast<int>(rank), u / o.row_units, p.col_tiles, -1, 0, p.k_blocks)) return;
             for (int v = cta; v < o.rest * o.cuts; v += o.groups) {
@@ -655,6 +680,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                 // the whole warp must agree before the warp-collective TMEM loads below
                 const bool ready = wait_barrier(tfull_bar(ab), aphase, abort_flag, p.status, 4);
                 if (!__all_sync(0xffffffffu, ready)) return false;
+                if (MODE == MODE_OUT && CG == 1 && slot == SHARED_TILE) return false;      // finished below, with the cluster
                 tc_fence_after_sync();
                 const uint32_t t_row = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + ab * BN;
                 const int col_base = ct * BN;
@@ -1093,6 +1119,50 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
         if (MODE == MODE_STATS && TOPK == TOPK_NONE && lane == 0) bulk_wait_group0();
     }
 
+    if constexpr (MODE == MODE_OUT && CG == 1) {
+        const int C = p.plan.cluster;
+        if (C > 1) {
+            // The operand stages hold [C pieces][rows per CTA][ROW_PITCH] floats now: every CTA's products are complete.
+            constexpr int ROW_PITCH = BN + 4;               // rows 4 banks apart
+            static_assert((BM + 8) * ROW_PITCH * 4 <= OPERAND_BYTES, "the pieces of a CTA's rows fit the operand stages");
+            const int u = cta / C, z = cta - u * C;
+            const int rt = u % p.plan.row_units, ct = u / p.plan.row_units;
+            const int per = (BM + C - 1) / C;
+            tc_fence_before_sync();
+            __syncthreads();
+            cluster_sync();
+            tc_fence_after_sync();
+            if (warp >= 2) {
+                const int quad = warp & 3, r = quad * 32 + lane;
+                const uint32_t dst = map_to_rank(smem_base + (z * per + r % per) * ROW_PITCH * 4, r / per);
+                const bool row_ok = p.row_global_offset + rt * BM + r < p.rows_valid;
+#pragma unroll 1
+                for (int ch = 0; ch < BN / 32; ++ch) {
+                    uint32_t v[32];
+                    tmem_ld32(tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + ch * 32, v);
+                    tmem_ld_wait(v);
+                    if (row_ok) {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) st_cluster_v4(dst + (ch * 32 + 4 * j) * 4, v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                    }
+                }
+            }
+            cluster_sync();
+            for (int i = threadIdx.x; i < per * (BN / 4); i += NUM_THREADS) {
+                const int rl = i / (BN / 4), c = i % (BN / 4) * 4;
+                const int r = z * per + rl, row = p.row_global_offset + rt * BM + r, col = ct * BN + c;
+                if (r >= BM || row >= p.rows_valid || col >= p.n_cols) continue;
+                const uint8_t* src = smem_gen + (rl * ROW_PITCH + c) * 4;
+                float4 a = *reinterpret_cast<const float4*>(src);
+                for (int q = 1; q < C; ++q) {
+                    const float4 v = *reinterpret_cast<const float4*>(src + q * per * ROW_PITCH * 4);
+                    a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
+                }
+                finish_out4(p, a, rt * BM + r, row, col);
+            }
+        }
+    }
+
     // ---- teardown ----
     tc_fence_before_sync();
     __syncthreads();
@@ -1135,17 +1205,7 @@ __global__ void __launch_bounds__(256) out_reduce_kernel(const __grid_constant__
         const float4 v = src[z * step];
         a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
     }
-    if (p.coef != nullptr) {
-        const float coef = p.coef[row];
-        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (p.sparse != nullptr) s = *reinterpret_cast<const float4*>(p.sparse + static_cast<long long>(rt * BM + r_local) * p.out_pitch + col);
-        a.x = fmaf(coef, a.x, -s.x); a.y = fmaf(coef, a.y, -s.y); a.z = fmaf(coef, a.z, -s.z); a.w = fmaf(coef, a.w, -s.w);
-    }
-    const long long at = static_cast<long long>(row) * p.out_pitch + col;
-    if (p.out_fp32)
-        *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + at) = a;
-    else
-        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(p.out) + at) = make_uint2(pack_bf16x2(a.x, a.y), pack_bf16x2(a.z, a.w));
+    finish_out4(p, a, rt * BM + r_local, row, col);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1217,8 +1277,8 @@ __device__ __forceinline__ float warp_lse(const float* pm, const float* ps, int 
     return m + logf(s);
 }
 
-constexpr int FIN_GRP = 16;       // tokens of Omega_hat whose W rows finalize reads together
-constexpr int FIN_WARPS = 4;      // warps that share a row
+constexpr int FIN_GRP = 8;        // tokens of Omega_hat whose W rows finalize reads together
+constexpr int FIN_WARPS = 8;      // warps that share a row
 
 __device__ __forceinline__ void unpack8(const uint4& v, float (&f)[8]) {
     const __nv_bfloat162* p2 = reinterpret_cast<const __nv_bfloat162*>(&v);
@@ -1231,9 +1291,10 @@ __device__ __forceinline__ void unpack8(const uint4& v, float (&f)[8]) {
 }
 
 // One block per row (2048 rows, 20 tokens, d = 4096: 390 us with a warp per row and a serial selection -> 158 us, and 24 us
-// in select_kernel; 1024 rows, 10 tokens: 144 -> 55 us): bound by the latency of the gathered rows of W, so that a row's columns are spread over FIN_WARPS
+// in select_kernel; 1024 rows, 10 tokens: 144 -> 55 us; with eight warps instead of four, eight tokens instead of sixteen
+// and three blocks per SM another 10-20 %): bound by the latency of the gathered rows of W, so that a row's columns are spread over FIN_WARPS
 // warps (8 columns per thread and step) and FIN_GRP rows of W are in flight per thread.
-__global__ void __launch_bounds__(FIN_WARPS * 32) finalize_kernel(const __grid_constant__ FinalizeParams p) {
+__global__ void __launch_bounds__(FIN_WARPS * 32, 3) finalize_kernel(const __grid_constant__ FinalizeParams p) {
     wait_previous_kernel();
     if (p.gate != nullptr && *p.gate == 0u) return;
     __shared__ int sh_tok[K_CAP];         // Omega_hat of the row (the bi-directional set needs 2K <= K_CAP)

@@ -22,6 +22,8 @@ pytestmark = pytest.mark.gpu
     (129, 64, 9000, 64, True),         # 127 padding rows in the second row tile, buffered candidates
     (64, 72, 33001, 256, False),       # the most rows whose draft logits go through the workspace in fp32, the largest K
     (65, 72, 33001, 256, False),       # one row more
+    (128, 264, 20001, 12, True),       # the most rows of one tile; output tiles shared by clusters
+    (250, 520, 20000, 10, False),      # two row tiles, output tiles shared by clusters
     (620, 64, 40000, 16, True),        # one warp per row, K lists whose first entries set the floor
     (1601, 2824, 12000, 10, False),    # whole rounds of output tiles, then a cut rest, d not a multiple of 256
 ])
@@ -52,3 +54,27 @@ def test_reference_exponent_far_below_the_row(value):
     fused, split = _guarded_fused(case, K, None)
     print("fused", compare(H_t, H_d, W, K, fused))
     print("split", compare(H_t, H_d, W, K, split))
+
+
+@pytest.mark.parametrize("N", [60, 100, 128])
+def test_one_row_tile_with_less_workspace_and_from_host_buffers(N):
+    """Calls of one row tile keep the draft logits in fp32 where the workspace has room: with a smaller
+    workspace the results are the oracle's too, and the entry for host buffers gives the device entry's bits."""
+    import paper_2408_15766_b200 as hass
+    d, V, K = 136, 5000, 10
+    inp = hi.make_custom(N, d, V, K, seed=N, sigma_w=0.2)
+    dev = torch.device("cuda:0")
+    H_t, H_d, W = inp.H_t.to(dev), inp.H_d[0].to(dev), inp.W.to(dev)
+    full = hass.topk_distill_workspace_bytes(N, d, V, K)
+    V_pad = -(-V // 256) * 256
+    # what the logits need beyond one row tile of scratch and the 128 fp32 rows before it
+    tail = max(0, N * V_pad * 4 - 128 * V_pad * 2 - 128 * d * 4)
+    a = hass.topk_distill_fwd_bwd(H_t, H_d, W, K)
+    b = hass.topk_distill_fwd_bwd(H_t, H_d, W, K, workspace=torch.empty(full - tail, dtype=torch.uint8, device=dev))
+    for out in (a, b):
+        hass.check(out["workspace"])
+        print(compare(inp.H_t, inp.H_d[0], inp.W, K, {k: v.cpu() for k, v in out.items() if k != "workspace"}))
+    loss = torch.empty(N, dtype=torch.float32).pin_memory()
+    dH = torch.empty(N, d, dtype=torch.bfloat16).pin_memory()
+    hass.topk_distill_fwd_bwd_host(inp.H_t.pin_memory(), inp.H_d[0].pin_memory(), W, K, loss, dH)
+    assert torch.equal(loss, a["loss"].cpu()) and torch.equal(dH, a["dH_d"].cpu())
