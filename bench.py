@@ -616,7 +616,7 @@ def main():
                 "frac_of_sustained": achieved / float(peaks["bf16_tflops_sustained"]),
                 "flops_per_launch": flops_per_launch, "avg_launch_ms": dom_ms / dom_cnt}
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    chunk_rows = min(max(sms // 4, 1) * 128, (N + 127) // 128 * 128)     # the library's chunk: #SM / 4 row tiles
+    chunk_rows = min(max(sms // 8 * 2, 1) * 128, (N + 127) // 128 * 128)     # the library's chunk: #SM / 4 row tiles, an even number
     V_pad = (V + 255) // 256 * 256
     step_tflops = flops_credit / (ms_step * 1e-3) / 1e12
     executed = sum(f for k, f in kinds.items() if prof[k][1] > 0)
