@@ -54,7 +54,7 @@ constexpr int MAX_CLUSTER = 8;
 typedef void (*GemmFn)(GemmParams);
 
 // Launches `fn` as a programmatic dependent of the stream's previous kernel (see wait_previous_kernel), in clusters of
-// `cluster` blocks; cluster = 0: an ordinary launch, for a kernel that does not wait. 64 rows x 256 x 1024, five kernels: 47 -> 39 us per call; HCA forward + backward of 2 x 333
+// `cluster` blocks. 64 rows x 256 x 1024, five kernels: 47 -> 39 us per call; HCA forward + backward of 2 x 333
 // positions, four kernels: 75 -> 73 us.
 template <typename... P, typename... A>
 static int launch(void (*fn)(P...), long long grid, int block, size_t smem, cudaStream_t st, int cluster, A&&... args) {
@@ -71,7 +71,7 @@ static int launch(void (*fn)(P...), long long grid, int block, size_t smem, cuda
     at[1].val.clusterDim.y = 1;
     at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = cluster > 1 ? 2 : cluster;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     g_launches.fetch_add(1);
     if (cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...) != cudaSuccess) {
         cudaGetLastError();
@@ -487,15 +487,17 @@ static int launch_gemm(const GemmParams& p, cudaStream_t st, int kind = -1) {
     return launch(fn, p.sched.max_ctas, NUM_THREADS, SMEM_BYTES, st, MODE == MODE_OUT && p.plan.cluster > 1 ? p.plan.cluster : pair ? 2 : 1, p);
 }
 
+// Clears a 256-byte aligned piece of the workspace (a multiple of 16 bytes).
+static int clear_bytes(void* at, size_t bytes, cudaStream_t st) {
+    const int n = static_cast<int>(bytes / 16);
+    return launch(clear_kernel, n <= 256 * 16 ? ceil_div(n, 256) : 16, 256, 0, st, 1, static_cast<uint4*>(at), n);
+}
+
 // Clears the status block (only_thresholds: not) and the published thresholds of `slots` slots.
 static int clear_status(uint8_t* ws, const Layout& L, int slots, cudaStream_t st, bool only_thresholds = false) {
     const size_t from = only_thresholds ? L.thr_share : L.status;
     if (only_thresholds && slots == 0) return HASS_OK;
-    if (cudaMemsetAsync(ws + from, 0, L.thr_share + static_cast<size_t>(slots) * BM * 4 - from, st) != cudaSuccess) {
-        cudaGetLastError();
-        return HASS_ERR_CUDA;
-    }
-    return HASS_OK;
+    return clear_bytes(ws + from, L.thr_share + static_cast<size_t>(slots) * BM * 4 - from, st);
 }
 
 template <int WARPS, int WIN>
@@ -708,10 +710,8 @@ static int backward_impl(const void* H_d, const void* W, long long N, long long 
     float* coef = reinterpret_cast<float*>(ws + L.coef);
     float* lse2 = reinterpret_cast<float*>(ws + L.lse2);
     __nv_bfloat16* P = reinterpret_cast<__nv_bfloat16*>(ws + L.scratch);
-    if (cudaMemsetAsync(ws + L.status, 0, 256, st) != cudaSuccess) {
-        cudaGetLastError();
-        return HASS_ERR_CUDA;
-    }
+    rc = clear_bytes(ws + L.status, 256, st);
+    if (rc != HASS_OK) return rc;
 
     {
         KernelTimer timer(KIND_PREP, st);
@@ -831,18 +831,21 @@ static int narrow_impl(bool with_target, const void* H_t, const void* H_d, const
     // (1) target and draft rows in one sweep: statistics, candidates, the draft's logits
     GemmParams p;
     std::memset(&p, 0, sizeof(p));
-    p.row_tiles = with_target ? 2 : 1;
+    // up to 64 rows each share one row tile (61 rows x 4096 x 32000: 65 us as two row tiles of a CTA pair, 61 as one)
+    p.half_tiles = with_target && N <= BM / 2 ? 1 : 0;
+    p.row_tiles = with_target && !p.half_tiles ? 2 : 1;
     int rc = plan_launch(p.row_tiles, CT, di.sms, L.slot_cap, &p.sched);
     if (rc != HASS_OK) return rc;
     log_schedule("narrow sweep", p.sched);
-    rc = make_tmap(&p.tmA1, H_d, N, d, d, BK, BM);
-    if (rc == HASS_OK) rc = make_tmap(&p.tmA0, with_target ? H_t : H_d, N, d, d, BK, BM);
+    const int box_rows = p.half_tiles ? BM / 2 : BM;
+    rc = make_tmap(&p.tmA1, H_d, N, d, d, BK, box_rows);
+    if (rc == HASS_OK) rc = make_tmap(&p.tmA0, with_target ? H_t : H_d, N, d, d, BK, box_rows);
     if (rc == HASS_OK) rc = make_tmap(&p.tmB, W, V, d, d, BK, BN / p.sched.pair);
     if (rc != HASS_OK) return rc;
     p.row_tiles0 = 1;
     p.topk_row_tiles = with_target ? 1 : 0;
     p.spill_begin = INT_MAX;
-    p.z_begin = cmb ? 0 : p.row_tiles - 1;
+    p.z_begin = 0;
     p.z_rows = N;
     p.z_out = z;
     p.zt_out = cmb ? reinterpret_cast<float*>(cmb->Pt) : nullptr;
@@ -876,6 +879,7 @@ static int narrow_impl(bool with_target, const void* H_t, const void* H_d, const
     std::memset(&z_params, 0, sizeof(z_params));
     z_params.sched = p.sched;
     z_params.first_tile = p.row_tiles - 1;
+    z_params.first_row = p.half_tiles ? BM / 2 : 0;
     z_params.K = K;
     z_params.V = static_cast<int>(V);
     z_params.part_m = p.part_m;
@@ -973,10 +977,8 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
     // (reference from column tile 0), the same sequence runs a second time as conditional launches with each row's
     // reference taken from that record, which no logit of the row can exceed.
     unsigned int* zmax = reinterpret_cast<unsigned int*>(ws + L.zmax);
-    if (cudaMemsetAsync(zmax, 0, static_cast<size_t>(2 * RT) * BM * 4, st) != cudaSuccess) {
-        cudaGetLastError();
-        return HASS_ERR_CUDA;
-    }
+    rc = clear_bytes(zmax, static_cast<size_t>(2 * RT) * BM * 4, st);
+    if (rc != HASS_OK) return rc;
     auto run = [&](bool retry) -> int {
     const unsigned int* gate = retry ? status + 1 : nullptr;
     for (int t0 = 0; t0 < RT; t0 += chunk_tiles) {
@@ -2073,10 +2075,8 @@ int hass_hca_attention_fwd(const void* Q, const void* K_t, const void* V_t, cons
     if (rc != HASS_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
 
-    if (cudaMemsetAsync(workspace, 0, 256, st) != cudaSuccess) {
-        cudaGetLastError();
-        return HASS_ERR_CUDA;
-    }
+    rc = clear_bytes(workspace, 256, st);
+    if (rc != HASS_OK) return rc;
     {
         hca2::Params p;
         std::memset(&p, 0, sizeof(p));
@@ -2158,10 +2158,6 @@ int hass_hca_attention_bwd(const void* Q, const void* K_t, const void* V_t, cons
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     float* Dv = reinterpret_cast<float*>(ws + L.D);
     float* dQacc = reinterpret_cast<float*>(ws + L.dQacc);
-    if (cudaMemsetAsync(workspace, 0, 256, st) != cudaSuccess) {
-        cudaGetLastError();
-        return HASS_ERR_CUDA;
-    }
     const int iB = static_cast<int>(B), iT = static_cast<int>(T), iH = static_cast<int>(H), iHkv = static_cast<int>(Hkv);
     const float c2 = scale * 1.4426950408889634f;
 
@@ -2201,9 +2197,10 @@ int hass_hca_attention_bwd(const void* Q, const void* K_t, const void* V_t, cons
         r.m = m; r.B = iB; r.T = iT; r.H = iH; r.Hkv = iHkv;
         r.c2 = c2;
         r.scale = scale;
+        r.status = static_cast<unsigned int*>(workspace);
         KernelTimer kt(KIND_HCA_BWD_ROWS, st);
         const long long halves = static_cast<long long>(B) * T * Hkv;
-        rc = launch(hca_bwd::hca_bwd_rows_kernel, (halves * 16 + 255) / 256, 256, 0, st, 0, r);
+        rc = launch(hca_bwd::hca_bwd_rows_kernel, (halves * 16 + 255) / 256, 256, 0, st, 1, r);
     }
     if (rc != HASS_OK) return rc;
 

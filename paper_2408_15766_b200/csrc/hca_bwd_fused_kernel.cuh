@@ -90,9 +90,12 @@ struct RowsParams {
     float* dQacc;                  // [B, T, H, 128] fp32
     int m, B, T, H, Hkv;
     float c2, scale;
+    unsigned int* status;          // status block of 64 words, cleared here
 };
 
 __global__ void __launch_bounds__(256, 2) hca_bwd_rows_kernel(const __grid_constant__ RowsParams p) {
+    wait_previous_kernel();
+    if (blockIdx.x == 0 && threadIdx.x < 64) p.status[threadIdx.x] = 0u;
     const long long w = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 4;   // (b, t, g)
     const int sub = threadIdx.x & 15;
     // no thread leaves early: the shuffles below name all 32 lanes, so a half-warp past the end runs on clamped

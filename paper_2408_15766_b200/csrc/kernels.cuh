@@ -86,6 +86,8 @@ struct GemmParams {
                            // boxes of 64 columns x 32 rows, 128-byte swizzle, for TMA stores
     Schedule sched;
     int row_tiles;         // row tiles of this launch; a pair's second tile may lie beyond
+    int half_tiles;        // MODE_STATS, single CTAs: the one row tile is 64 rows of A0 (Top-K) and 64 of A1 (no Top-K), boxes
+                           // of 64 rows; a sweep of both that reads every tile of B once per call
     int row_tiles0;        // row tiles [0, row_tiles0) read A0, the others A1 (tile index - row_tiles0)
     int topk_row_tiles;    // leading row tiles whose rows collect Top-K candidates (MODE_STATS)
     int a_row_offset;      // added to A0's row coordinate (chunked backward)
@@ -519,7 +521,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                                 tma_load_2d(dst, tm, bar, x, y);
                         };
                         const int col0 = ct * BN + static_cast<int>(rank) * (BN / CG);
-                        load(smemA + stage * A_STAGE_BYTES, tmA, kb * BK, row0);
+                        if (MODE == MODE_STATS && CG == 1 && p.half_tiles) {
+                            load(smemA + stage * A_STAGE_BYTES, &p.tmA0, kb * BK, 0);
+                            load(smemA + stage * A_STAGE_BYTES + A_STAGE_BYTES / 2, &p.tmA1, kb * BK, 0);
+                        } else {
+                            load(smemA + stage * A_STAGE_BYTES, tmA, kb * BK, row0);
+                        }
                         if (!B_MN_MAJOR) {
                             load(smemB + stage * B_STAGE_BYTES, &p.tmB, kb * BK, col0);
                         } else {
@@ -624,6 +631,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
             const int g_row = p.row_global_offset + rt * BM + r_local;
             const bool tile_ok = CG == 1 || rt < p.row_tiles;     // false: the partner of the last row tile, nothing to write
             const bool row_ok = tile_ok && g_row < p.rows_valid;
+            const bool second_half = MODE == MODE_STATS && CG == 1 && p.half_tiles && quad >= 2;
+            const int r_own = MODE == MODE_STATS && CG == 1 && p.half_tiles ? r_local % (BM / 2) : r_local;   // row in its own matrix
             // ---- per-item state ----
             float m = -INFINITY, s = 0.f, thr = -INFINITY;        // MODE_STATS; thr = admission threshold in force
             float thr_own = -INFINITY;                            // K-th (K_REG-th) largest logit of this lane's own list
@@ -638,10 +647,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
             const float* sg = nullptr;
             int cur = 0, nxt = INT_MAX;
             if (MODE == MODE_STATS) {
-                want_topk = HAS_TOPK && tile_ok && rt < p.topk_row_tiles;
+                want_topk = HAS_TOPK && tile_ok && rt < p.topk_row_tiles && !second_half;
                 if (HAS_TOPK) cbuf = p.cand + (static_cast<long long>(slot) * BM + r_local) * p.cap;
                 cnt = 0;
-                if (HAS_TOPK && p.row_global_offset + (rt < p.row_tiles0 ? rt : rt - p.row_tiles0) * BM + r_local >= p.rows_valid) {
+                if (HAS_TOPK && p.row_global_offset + (rt < p.row_tiles0 ? rt : rt - p.row_tiles0) * BM + r_own >= p.rows_valid) {
                     // A padding row collects nothing: its logits are all equal (zero), and 256 of them filled its buffer and
                     // made the warp compact row after row (sweep of 64 rows x 256 x 1024, K = 64: 195 -> 30 us).
                     thr_own = INFINITY;
@@ -671,8 +680,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                 nxt = si[0];
             }
             float* zrow = nullptr;
-            if (HAS_TOPK && tile_ok && rt >= p.z_begin && r_local < p.z_rows)      // (one row tile of either kind)
-                zrow = (rt < p.row_tiles0 && p.zt_out != nullptr ? p.zt_out : p.z_out) + static_cast<long long>(r_local) * p.z_pitch;
+            if (HAS_TOPK && tile_ok && rt >= p.z_begin && r_own < p.z_rows) {      // (one row tile of either kind)
+                const bool target = p.half_tiles ? !second_half : rt < p.row_tiles0 && p.row_tiles > 1;
+                float* z = target ? p.zt_out : p.z_out;
+                if (z != nullptr) zrow = z + static_cast<long long>(r_own) * p.z_pitch;
+            }
             const int t0 = first_tile(rt, ln);
             const int nt = (p.col_tiles - ln + S - 1) / S;
             for (int t = t0; t < nt; ++t) {
@@ -767,7 +779,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                             float x = fmaxf(__uint_as_float(r[16 * h]), __uint_as_float(r[16 * h + 1]));
 #pragma unroll
                             for (int j = 2; j < 16; j += 2) x = fmax3(x, __uint_as_float(r[16 * h + j]), __uint_as_float(r[16 * h + j + 1]));
-                            gm[2 * ch + h] = x;
+                            gm[2 * ch + h] = fmaxf(x, -INFINITY);      // (a group of NaN counts for nothing)
                         }
                     }
                     sort16_descending(gm);
@@ -1934,6 +1946,7 @@ constexpr int DZ_LOADS = 4;
 struct DzParams {
     Schedule sched;        // schedule of the sweep
     int first_tile;        // its row tile of the draft rows
+    int first_row;         // of the draft rows in that tile
     int K, V;
     const float* part_m;
     const float* part_s;
@@ -1974,7 +1987,7 @@ __global__ void __launch_bounds__(DZ_THREADS) dz_kernel(const __grid_constant__ 
     if (warp == DZ_THREADS / 32 - 1) {
         int slot0, S;
         find_slots(p.sched, p.first_tile, slot0, S);
-        const float lse = warp_lse(p.part_m, p.part_s, slot0, S, row, lane);
+        const float lse = warp_lse(p.part_m, p.part_s, slot0, S, p.first_row + row, lane);
         if (lane == 0) sh_sum[0] = lse;
     }
     __syncthreads();
@@ -2101,6 +2114,13 @@ __global__ void __launch_bounds__(256) ce_kernel(int rows, int row_begin, int d,
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
     if (lane == 0) loss_ce[row] = lse_d[row] - dot - ce_corr[row];
+}
+
+// Clears n 16-byte words: the status block and what lies behind it. (A memset node would stand between two dependent
+// launches and make both wait: 5 us per call.)
+__global__ void __launch_bounds__(256) clear_kernel(uint4* at, int n) {
+    wait_previous_kernel();
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) at[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 // Self-test of the bounded waits (hass_selftest_wait_expiry): one CTA, no TMA, no tensor memory. Every thread

@@ -78,3 +78,19 @@ def test_one_row_tile_with_less_workspace_and_from_host_buffers(N):
     dH = torch.empty(N, d, dtype=torch.bfloat16).pin_memory()
     hass.topk_distill_fwd_bwd_host(inp.H_t.pin_memory(), inp.H_d[0].pin_memory(), W, K, loss, dH)
     assert torch.equal(loss, a["loss"].cpu()) and torch.equal(dH, a["dH_d"].cpu())
+
+
+@pytest.mark.parametrize("K", [10, 40])
+def test_nan_logits_hide_no_candidate(K):
+    """Tokens whose rows of W are NaN make a row's sums NaN, but the first tile's admission bound must not count them."""
+    import paper_2408_15766_b200 as hass
+    inp = hi.make_custom(64, 64, 1024, K, seed=4, sigma_w=0.3)
+    W = inp.W.clone()
+    W[16:48] = float("nan")
+    W[200:230] = float("nan")
+    dev = torch.device("cuda:0")
+    out = hass.topk_distill_fwd(inp.H_t.to(dev), inp.H_d[0].to(dev), W.to(dev), K)
+    hass.check(out["workspace"])
+    z = (inp.H_t.double() @ W.double().T).nan_to_num(nan=-np.inf)
+    want = z.topk(K, dim=1).indices.sort(dim=1).values
+    assert torch.equal(out["topk_idx"].cpu().long().sort(dim=1).values, want)
