@@ -19,7 +19,11 @@
 // The substituted entries (t, t - i), i < m, ride the same pipeline as extra products: before the key tiles
 // S = Q K_d[i]^T with the K_d[i] tile fetched i rows early, so that the wanted scores sit on the diagonal and
 // each row's thread keeps its own; the m scores join the row's maximum and sum at the last key tile; after
-// the key tiles O += diag(p_i) V_d[i] with V_d[i] fetched i rows early. No thread reads global memory.
+// the key tiles O += diag(p_i) V_d[i] with V_d[i] fetched i rows early. The weights of a pass take 8 columns beside the
+// last tile's P: a step over 16 keys writes only the 16 lanes whose weights those keys belong to (the instruction's
+// lane mask), so that all steps can share the columns, and the threads hand them over together with the last P instead of
+// in rounds of two passes after it (m = 2 .. 5: one to three round trips of about 1.3 k cycles per item).
+// No thread reads global memory.
 // The running reference moves only when a tile's maximum exceeds it by more than 2^8 (the accumulator is then
 // rescaled in place by the row's thread), so P stays within bf16 range and almost every tile skips the rescale.
 // Warps: 0 = TMA producer, 1 = MMA issuer and TMEM owner (2, 3 idle), 4-7 = softmax + epilogue of slot 0,
@@ -40,6 +44,7 @@ using hca::pack_bf16;
 using hca::tma_load_3d;
 using hca::tmem_st32;
 using hca::tmem_st_wait;
+static_assert(64 + 8 * hca::MAX_DRAFTS <= 128, "the weights of all passes fit the score buffer");
 
 constexpr int QT = 128;            // query rows per item
 constexpr int KT = 128;            // keys per tile
@@ -63,6 +68,7 @@ constexpr int NUM_BARS = 4 + 2 * K_STAGES + 2 * KV_STAGES + 6 + 2 * SCHED_DEPTH;
 constexpr int SMEM_BYTES = SMEM_BAR + 256;           // 229632
 static_assert(8 * NUM_BARS + 4 * (2 + SCHED_DEPTH) <= 256 && SMEM_BYTES <= 232448, "shared-memory window");
 constexpr int TMEM_COLS = 512;     // S of slot s at 128 s (P overwrites its first 64 columns), O of slot s at 256 + 128 s
+constexpr int DRAFT_P = 64;        // the draft passes' weights: 8 columns each behind P in the score buffer
 constexpr float RESCALE_LOG2 = 8.f;
 
 struct Params {
@@ -193,9 +199,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
     //   m draft score products   S = Q K_d[i]^T with the K_d[i] tile fetched i rows early, so that the wanted
     //                            scores <Q[t], K_d[i][t - i]> sit on the tile's diagonal; the row's thread keeps its own
     //   n key tiles              S = Q K_t^T -> softmax -> O += P V_t
-    //   m draft value products   O += diag(p_i) V_d[i] (V_d[i] fetched i rows early; P holds the row's weight on
-    //                            the diagonal and zeros elsewhere), two passes per arrival of the softmax warps
-    // Every product of a slot but the first S follows an arrival of the slot's softmax warps on p_full.
+    //   m draft value products   O += diag(p_i) V_d[i] (V_d[i] fetched i rows early; the weights came with the last P)
+    // Every product of a slot but the first S and the draft value products follows an arrival of the slot's softmax warps
+    // on p_full.
     // The K ring carries the draft key tiles, then the key tiles; the V ring the value tiles, then the draft
     // value tiles. A tile both slots use (always, when the pair is two heads of one group; the key/value
     // tiles otherwise) is one ring entry, released after the second slot's product.
@@ -300,6 +306,22 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
             if (leader && commit) umma_commit(pv_done(s));
             __syncwarp();
         };
+        // O of slot s += diag(p_i) V_d[i], V_d[i] in V stage st: the weights of the 16 rows that step k concerns sit in the
+        // same 8 columns as those of the other rows, whose lanes the step leaves alone.
+        auto issue_draft_pv = [&](int s, int st, int i, bool commit) {
+            tc_fence_after_sync();
+#pragma unroll
+            for (int k = 0; k < KT / 16; ++k) {
+                const uint64_t b_desc = make_smem_desc_sw128(base + SMEM_V + st * KV_BYTES + k * 16 * 128, KV_HALF, 1024);
+                const uint32_t off = k & 1 ? 0x0000ffffu : 0xffff0000u;
+                if (leader)
+                    umma_bf16_ta_lanes(tmem_base + 256 + s * HD, tmem_base + s * KT + DRAFT_P + 8 * i, b_desc, idesc_o,
+                                       k >> 1 == 0 ? off : 0xffffffffu, k >> 1 == 1 ? off : 0xffffffffu, k >> 1 == 2 ? off : 0xffffffffu,
+                                       k >> 1 == 3 ? off : 0xffffffffu);
+            }
+            if (leader && commit) umma_commit(pv_done(s));
+            __syncwarp();
+        };
         auto k_acquire = [&](int& st) {
             st = gk % K_STAGES;
             return wait_all(k_full(st), (gk / K_STAGES) & 1u, 4);
@@ -391,7 +413,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
                 bool k_ready = false;
                 if (j < n0) {
                     if (!p_wait(0)) { ok = false; break; }
-                    issue_pv(0, vst, 0, 0, 8, j == 0, true);
+                    issue_pv(0, vst, 0, 0, 8, j == 0, m == 0 || j + 1 < n0);
                     if (j + 1 < n0) {
                         if (!k_acquire(st)) { ok = false; break; }
                         k_ready = true;
@@ -399,7 +421,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
                     }
                 }
                 if (!p_wait(1)) { ok = false; break; }
-                issue_pv(1, vst, 0, 0, 8, j == 0, true);
+                issue_pv(1, vst, 0, 0, 8, j == 0, m == 0 || j + 1 < n1);
                 v_release(vst);
                 if (j + 1 < n1) {
                     if (!k_ready && !k_acquire(st)) { ok = false; break; }
@@ -407,39 +429,18 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
                     k_release(st);
                 }
             }
-            // ---- draft value rounds: two passes per arrival (their weights sit in the two halves of the S buffer) ----
-            for (int i0 = 0; i0 < m && ok; i0 += 2) {
-                const bool two = i0 + 1 < m;
-                bool waited0 = false, waited1 = false;
-                for (int e = 0; e < (two ? 2 : 1) && ok; ++e) {
-                    const bool fin = (e == 1) || !two;          // the slot's last product of the round
-                    int vst;
-                    if (shared) {
-                        if (!v_acquire(vst)) { ok = false; break; }
-                        if (a_on) {
-                            if (!waited0 && !p_wait(0)) { ok = false; break; }
-                            waited0 = true;
-                            issue_pv(0, vst, 64 * e, 0, 8, false, fin);
-                        }
-                        if (!waited1 && !p_wait(1)) { ok = false; break; }
-                        waited1 = true;
-                        issue_pv(1, vst, 64 * e, 0, 8, false, fin);
-                        v_release(vst);
-                    } else {
-                        if (a_on) {
-                            if (!v_acquire(vst)) { ok = false; break; }
-                            if (!waited0 && !p_wait(0)) { ok = false; break; }
-                            waited0 = true;
-                            issue_pv(0, vst, 64 * e, 0, 8, false, fin);
-                            v_release(vst);
-                        }
-                        if (!v_acquire(vst)) { ok = false; break; }
-                        if (!waited1 && !p_wait(1)) { ok = false; break; }
-                        waited1 = true;
-                        issue_pv(1, vst, 64 * e, 0, 8, false, fin);
-                        v_release(vst);
-                    }
+            // ---- draft value products: the weights are there, each slot's last one completes its item ----
+            for (int i = 0; i < m && ok; ++i) {
+                int vst;
+                if (!shared && a_on) {
+                    if (!v_acquire(vst)) { ok = false; break; }
+                    issue_draft_pv(0, vst, i, i + 1 == m);
+                    v_release(vst);
                 }
+                if (!v_acquire(vst)) { ok = false; break; }
+                if (shared && a_on) issue_draft_pv(0, vst, i, i + 1 == m);
+                issue_draft_pv(1, vst, i, i + 1 == m);
+                v_release(vst);
             }
         }
     }
@@ -566,40 +567,18 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
                 }
                 l += (ls[0] + ls[1]) + (ls[2] + ls[3]);
                 if (last) {
+                    // the substituted entries' weights: pass i in 8 columns beside P, this row's in the word of its key
 #pragma unroll
-                    for (int i = 0; i < MAX_DRAFTS; ++i)
-                        if (i < m && t - i >= 0) l += ex2(fmaf(sd[i], p.c2, nref));
-                }
-                tmem_st_wait();
-                tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(p_full(slot));
-                ++gpv;
-            }
-            if (!ok) break;
-            // ---- draft value rounds: two passes at a time; P holds only the weight 2^(sd c2 - ref) of each row, on the
-            //      diagonal: pass i0 in the first 64 columns of the S buffer, pass i0 + 1 in the last 64 ----
-            const float nref_f = mref == -INFINITY ? 0.f : -mref;
-#pragma unroll 1
-            for (int i0 = 0; i0 < m; i0 += 2) {
-                // the products that last read these columns must be complete before they are overwritten
-                if (!wait_barrier(pv_done(slot), (gpv - 1u) & 1u, abort_flag, p.status, 14)) { ok = false; break; }
-                tc_fence_after_sync();
-#pragma unroll 1
-                for (int e = 0; e < 2 && i0 + e < m; ++e) {
-                    const int i = i0 + e;
-                    float sdi = 0.f;
+                    for (int i = 0; i < MAX_DRAFTS; ++i) {
+                        if (i < m) {
+                            const float pi = t - i >= 0 ? ex2(fmaf(sd[i], p.c2, nref)) : 0.f;
+                            l += pi;
+                            const uint32_t bits = pack_bf16(pi, 0.f) << ((r & 1) * 16);
+                            uint32_t pk[8];
 #pragma unroll
-                    for (int ii = 0; ii < MAX_DRAFTS; ++ii)
-                        if (ii == i) sdi = sd[ii];
-                    const float pi = (t - i >= 0) ? ex2(fmaf(sdi, p.c2, nref_f)) : 0.f;
-                    const uint32_t bits = pack_bf16(pi, 0.f) << ((r & 1) * 16);        // key r sits in word r / 2
-#pragma unroll
-                    for (int hw = 0; hw < 2; ++hw) {
-                        uint32_t pk[32];
-#pragma unroll
-                        for (int w = 0; w < 32; ++w) pk[w] = (32 * hw + w == (r >> 1)) ? bits : 0u;
-                        tmem_st32(tmem_s + 64 * e + 32 * hw, pk);
+                            for (int w = 0; w < 8; ++w) pk[w] = w == ((r & 15) >> 1) ? bits : 0u;
+                            hca::tmem_st8(tmem_s + DRAFT_P + 8 * i, pk);
+                        }
                     }
                 }
                 tmem_st_wait();
