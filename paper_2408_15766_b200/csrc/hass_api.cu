@@ -2075,8 +2075,6 @@ int hass_hca_attention_fwd(const void* Q, const void* K_t, const void* V_t, cons
     if (rc != HASS_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
 
-    rc = clear_bytes(workspace, 256, st);
-    if (rc != HASS_OK) return rc;
     {
         hca2::Params p;
         std::memset(&p, 0, sizeof(p));
@@ -2102,6 +2100,11 @@ int hass_hca_attention_fwd(const void* Q, const void* K_t, const void* V_t, cons
         p.c2 = scale * 1.4426950408889634f;
         p.status = static_cast<unsigned int*>(workspace);
         const int grid = p.pairs < di.sms ? p.pairs : di.sms;
+        p.one_round = p.pairs == grid ? 1 : 0;
+        if (!p.one_round) {
+            rc = clear_bytes(workspace, 256, st);
+            if (rc != HASS_OK) return rc;
+        }
         KernelTimer kt(KIND_HCA, st);
         return launch(hca2::hca_attention_pair_kernel, grid, hca2::NUM_THREADS, hca2::SMEM_BYTES, st, 1, p);
     }

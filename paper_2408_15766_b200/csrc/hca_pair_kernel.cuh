@@ -83,6 +83,7 @@ struct Params {
     int pairs;                     // work units
     int head_pairing;              // 1: a pair = heads 2u, 2u + 1 at one query tile; 0: one head, query tiles qt - 1, qt
     float c2;                      // scale * log2(e)
+    int one_round;                 // every CTA takes one pair: no counter, and the status block is cleared here
     unsigned int* status;
 };
 
@@ -177,12 +178,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
         tmem_relinquish();
     }
     wait_previous_kernel();
+    if (p.one_round && blockIdx.x == 0 && threadIdx.x < 64) p.status[threadIdx.x] = 0u;
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_ptr_smem;
 
-    // Pairs are sorted longest first and handed out dynamically: the producer takes the next index from a counter in
+    // With no more pairs than CTAs each takes its own (one launch instead of two: 22 us forward calls are bound by the host).
+    // Otherwise pairs are sorted longest first and handed out dynamically: the producer takes the next index from a counter in
     // the workspace (word 1, zeroed by the host before the launch) and publishes it to the other roles through a
     // small queue in shared memory, so a CTA that falls behind simply takes fewer pairs. An index >= pairs ends a role.
     // next_pair(k): the k-th index this CTA works on (every consumer warp calls it once per k).
@@ -231,7 +234,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
                 return true;
             };
             for (;; ++it) {
-                const int idx = static_cast<int>(atomicAdd(p.status + 1, 1u));
+                const int idx = !p.one_round ? static_cast<int>(atomicAdd(p.status + 1, 1u)) : it == 0 ? static_cast<int>(blockIdx.x) : INT_MAX;
                 {
                     const int e = it % SCHED_DEPTH;
                     if (!wait_barrier(sched_empty(e), ((it / SCHED_DEPTH) & 1u) ^ 1u, abort_flag, p.status, 15)) break;
