@@ -77,6 +77,9 @@ __device__ __forceinline__ float sum16(float v) {
 // Position s of pass i meets exactly one query per head (t = s + i), so each output row has one writer; the
 // last i rows of pass i meet none and are zeroed by the half-warp of the same index. Passes are taken two at
 // a time; the rows of the next head are requested before the current head is worked on.
+// Its inputs are read with ordinary loads: in a backward that directly follows its forward, the kernel that writes O and lse
+// may still be running when this one starts, so that they are not read-only for this kernel's lifetime and their loads
+// must stay behind the wait.
 struct RowsParams {
     const __nv_bfloat16* Q;        // [B, T, H, 128]
     const __nv_bfloat16* O;
@@ -123,16 +126,16 @@ __global__ void __launch_bounds__(256, 2) hca_bwd_rows_kernel(const __grid_const
             kraw[j] = vraw[j] = make_uint4(0u, 0u, 0u, 0u);
             if (use[j]) {
                 const size_t row = ((static_cast<size_t>(b) * p.T + (t - i)) * p.Hkv + g) * HD;
-                kraw[j] = __ldg(reinterpret_cast<const uint4*>(p.Kd[i] + row) + sub);
-                vraw[j] = __ldg(reinterpret_cast<const uint4*>(p.Vd[i] + row) + sub);
+                kraw[j] = *(reinterpret_cast<const uint4*>(p.Kd[i] + row) + sub);
+                vraw[j] = *(reinterpret_cast<const uint4*>(p.Vd[i] + row) + sub);
             }
 #pragma unroll
             for (int c = 0; c < 8; ++c) kacc[j][c] = vacc[j][c] = 0.f;
         }
-        uint4 qn = __ldg(reinterpret_cast<const uint4*>(p.Q + row0) + sub);
-        uint4 dn = __ldg(reinterpret_cast<const uint4*>(p.dO + row0) + sub);
-        uint4 on = i0 == 0 ? __ldg(reinterpret_cast<const uint4*>(p.O + row0) + sub) : make_uint4(0u, 0u, 0u, 0u);
-        float ln = __ldg(p.lse + ri0);
+        uint4 qn = *(reinterpret_cast<const uint4*>(p.Q + row0) + sub);
+        uint4 dn = *(reinterpret_cast<const uint4*>(p.dO + row0) + sub);
+        uint4 on = i0 == 0 ? *(reinterpret_cast<const uint4*>(p.O + row0) + sub) : make_uint4(0u, 0u, 0u, 0u);
+        float ln = p.lse[ri0];
         for (int hh = 0; hh < rep; ++hh) {
             const size_t row = row0 + static_cast<size_t>(hh) * HD;
             const size_t ri = ri0 + static_cast<size_t>(hh) * p.T;
@@ -142,10 +145,10 @@ __global__ void __launch_bounds__(256, 2) hca_bwd_rows_kernel(const __grid_const
             const uint4 oc = on;
             const float nlse2 = -ln * 1.4426950408889634f;
             if (hh + 1 < rep) {
-                qn = __ldg(reinterpret_cast<const uint4*>(p.Q + row + HD) + sub);
-                dn = __ldg(reinterpret_cast<const uint4*>(p.dO + row + HD) + sub);
-                if (i0 == 0) on = __ldg(reinterpret_cast<const uint4*>(p.O + row + HD) + sub);
-                ln = __ldg(p.lse + ri + p.T);
+                qn = *(reinterpret_cast<const uint4*>(p.Q + row + HD) + sub);
+                dn = *(reinterpret_cast<const uint4*>(p.dO + row + HD) + sub);
+                if (i0 == 0) on = *(reinterpret_cast<const uint4*>(p.O + row + HD) + sub);
+                ln = p.lse[ri + p.T];
             }
             float Dt;
             if (i0 == 0) {
@@ -415,8 +418,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_bwd_fused_kernel(const __g
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
                     const int t = jq * QE + lane + 32 * u;
-                    nl[u] = t < p.T ? -__ldg(p.lse + rowbase + t) * 1.4426950408889634f : -INFINITY;
-                    nd[u] = t < p.T ? -__ldcg(p.D + rowbase + t) * p.scale : 0.f;
+                    nl[u] = t < p.T ? -p.lse[rowbase + t] * 1.4426950408889634f : -INFINITY;
+                    nd[u] = t < p.T ? -p.D[rowbase + t] * p.scale : 0.f;
                 }
                 if (lane == 0) ok = wait_barrier(qd_empty(s), ((gq / F_STAGES) & 1u) ^ 1u, abort_flag, p.status, 3);
                 ok = __shfl_sync(0xffffffffu, ok, 0);

@@ -110,3 +110,14 @@ def test_hca_attention_arguments_rejected_before_the_device(hass):
     g = hass.lib.hass_hca_attention_bwd
     assert g(al, al, al, arr, arr, 1, 1, 16, 2, 1, 128, sc, al, None, al, al, al, al, arr, arr, al, 1 << 20, None) == -1
     assert g(al, al, al, arr, arr, 1, 1, 16, 2, 1, 128, sc, al, al, al, al, al, al, arr, arr, al, 16, None) == -3
+
+
+def test_kernels_read_through_no_non_coherent_load():
+    """Every kernel is a programmatic dependent of the one before it in the stream and may start while that one still
+    writes. A load through the non-coherent path is defined only for data that nothing writes during the kernel's whole
+    life, and the compiler may move it across the wait: no kernel uses one, by name, in PTX or by const __restrict__."""
+    src = os.path.join(ROOT, "paper_2408_15766_b200", "csrc")
+    for name in sorted(os.listdir(src)):
+        text = re.sub(r"//[^\n]*|/\*.*?\*/", "", open(os.path.join(src, name)).read(), flags=re.S)
+        for word in ("__ldg", "ld.global.nc", "__restrict__"):
+            assert word not in text, f"{name}: {word}"

@@ -148,8 +148,10 @@ def _run_bwd(inp, scale=None, pairs=None, whole_tensor=False):
     dO = torch.randn(inp.Q.shape, generator=g).to(torch.bfloat16)
     d = lambda x: x.to(dev)
     Kd, Vd = [d(x) for x in inp.K_d], [d(x) for x in inp.V_d]
-    fw = hass.hca_attention_fwd(d(inp.Q), d(inp.K_t), d(inp.V_t), Kd, Vd, scale=scale)
-    bw = hass.hca_attention_bwd(d(inp.Q), d(inp.K_t), d(inp.V_t), Kd, Vd, fw["O"], fw["lse"], d(dO), scale=scale)
+    # everything is on the device before the forward, so that the backward's kernels are queued right behind it
+    Q, K, V, dOd = d(inp.Q), d(inp.K_t), d(inp.V_t), d(dO)
+    fw = hass.hca_attention_fwd(Q, K, V, Kd, Vd, scale=scale)
+    bw = hass.hca_attention_bwd(Q, K, V, Kd, Vd, fw["O"], fw["lse"], dOd, scale=scale)
     hass.check(bw["workspace"])
     got = dict(dQ=bw["dQ"].cpu(), dK_t=bw["dK_t"].cpu(), dV_t=bw["dV_t"].cpu(),
                dK_d=[x.cpu() for x in bw["dK_d"]], dV_d=[x.cpu() for x in bw["dV_d"]])
@@ -233,6 +235,46 @@ def test_backward_twice_gives_the_same_gradients():
     step = torch.maximum(qa.abs(), qb.abs()) * 2.0 ** -7        # one bf16 step is at most 2^-7 of the value
     assert bool(((qa - qb).abs() <= step).all())
     assert float((qa != qb).float().mean()) < 0.05
+
+
+@pytest.mark.parametrize("B,T,H,Hkv,m", [
+    (2, 1500, 8, 2, 3),       # a pair per CTA: the forward is one launch
+    (2, 700, 16, 4, 2),       # more pairs than SMs
+    (1, 2100, 4, 4, 5),       # three rounds of passes in the row kernel
+])
+def test_backward_directly_behind_its_forward(B, T, H, Hkv, m):
+    # The backward's first kernel starts while the forward still runs and must not read O or lse before it is complete.
+    # Two sets of inputs take turns on the same output memory, with nothing but the two calls in the stream: a value read
+    # early is the other set's. All but dQ (whose fp32 sum has no fixed order) must equal, bit for bit, what the same
+    # calls give with the stream drained in between.
+    hass = _hass()
+    dev = torch.device("cuda:0")
+    sets = []
+    for seed in (1, 2):
+        inp = hi.make_hca_inputs(hi.HcaWorkload("behind", B=B, T=T, H=H, Hkv=Hkv, m=m, seed=seed))
+        dO = torch.randn(inp.Q.shape, generator=torch.Generator().manual_seed(seed)).to(torch.bfloat16).to(dev)
+        sets.append(([x.to(dev) for x in (inp.Q, inp.K_t, inp.V_t)], [x.to(dev) for x in inp.K_d], [x.to(dev) for x in inp.V_d], dO))
+    ws = torch.empty(256, dtype=torch.uint8, device=dev)
+    wsb = torch.empty(hass.hca_attention_bwd_workspace_bytes(B, T, H, m), dtype=torch.uint8, device=dev)
+
+    def step(k, drain):
+        qkv, Kd, Vd, dO = sets[k]
+        fw = hass.hca_attention_fwd(*qkv, Kd, Vd, workspace=ws)
+        if drain:
+            torch.cuda.synchronize()
+        bw = hass.hca_attention_bwd(*qkv, Kd, Vd, fw["O"], fw["lse"], dO, workspace=wsb)
+        return fw["O"], fw["lse"], bw["dK_t"], bw["dV_t"], *bw["dK_d"], *bw["dV_d"]
+
+    want = []
+    for k in (0, 1):
+        want.append([x.clone() for x in step(k, True)])
+        torch.cuda.synchronize()
+    for k in (0, 1, 0, 1):
+        got = step(k, False)       # (into the memory that the previous step's outputs left)
+        for a, b in zip(got, want[k]):
+            assert torch.equal(a, b)
+        del got
+    hass.check(wsb)
 
 
 def test_draft_passes_equal_to_target_change_nothing_on_the_gpu():
