@@ -146,7 +146,7 @@ int hass_topk_distill_bwd(const void* H_d, const void* W, int64_t N, int64_t d, 
  * Precision: every entry of dz_d, the Omega_hat entries included, reaches the tensor cores in bf16
  * (2^-9 relative); the loss uses fp32 logits throughout.
  * Range condition: the fixed exponent holds as long as no draft logit of a row exceeds the one it
- * was taken from by more than about 130 (natural-log units; a probability ratio of e^130). The sweep
+ * was taken from by more than about 90 (natural-log units; a probability ratio of e^90). The sweep
  * detects a violation and records every row's largest logit; the call therefore also enqueues the
  * steps from the draft sweep on a second time, as conditional launches that return at once unless a
  * violation was detected, in which case they redo the call with each row's exponent taken from that

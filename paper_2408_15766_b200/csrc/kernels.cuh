@@ -45,6 +45,11 @@ constexpr int SPILL_STAGES = 2;               // per epilogue warp
 constexpr int SMEM_BYTES = OPERAND_BYTES + 4 * SPILL_STAGES * SPILL_STAGE_BYTES +
                            1024 /*alignment slack*/ + 256 /*barriers*/;
 constexpr float LOG2E = 1.4426950408889634f;
+// A lane's sum of a spilling row's values 2^(z log2e - ref2), ref2 = z_ref log2e + 64, from which on the call is done again
+// with the row's largest logit as z_ref: a logit 90 above z_ref (natural units). The sum leaves fp32 only at 131, but what
+// depends on it does so earlier: the row scale g S_q / sum of the spill is denormal from g S_q < 1e-38 sum on, and q sum /
+// (g S_q) overflows likewise. With 1e20 both hold for g S_q down to 1e-18.
+constexpr float SPILL_SUM_LIMIT = 1e20f;
 
 enum { MODE_STATS = 0, MODE_PROBS = 1, MODE_OUT = 2 };
 
@@ -721,7 +726,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                         }
                     }
                     // spilled values are 2^(z log2e - ref2) <= about 2^-64 for typical rows, which leaves
-                    // 2^191 of headroom above the reference before bf16 / fp32 overflow
+                    // 2^130 of headroom above the reference before SPILL_SUM_LIMIT
                     ref2 = fmaf(mx, LOG2E, 64.f);
                     m = ref2 * (1.0f / LOG2E);
                 }
@@ -1112,9 +1117,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                 const long long so = static_cast<long long>(slot) * BM + r_local;
                 p.part_m[so] = m;
                 p.part_s[so] = s;
-                // a spilled value reached the top of the fp32 range: the row's logits spread too far
-                // above its reference for the fixed-exponent spill
-                if (spill && !(s < 1e38f)) atomicExch(p.status + 1, 1u);
+                // the row's logits spread too far above its reference for the fixed-exponent spill
+                if (spill && !(s < SPILL_SUM_LIMIT)) atomicExch(p.status + 1, 1u);
                 if (track_zmax && !p.use_row_zmax) atomicMax(p.row_zmax + rt * BM + r_local, ordered_key(__float_as_uint(zmax)));
                 if (USE_REG && want_topk) {
                     // the register list goes out as a full buffer of K_REG entries (unused ones carry id -1)
@@ -1923,11 +1927,11 @@ __global__ void __launch_bounds__(256) loss_patch_kernel(const __grid_constant__
         if (p.coef_out) p.coef_out[row] = g * scale;
     }
     if (p.P != nullptr && g != 0.f && scale > 0.f && scale < INFINITY) {      // P == nullptr: forward only, nothing to patch
-        const float inv = 1.f / scale;
+        const float sum = expf(lse_d - m_spill);         // q / scale = q / S_q x sum: neither factor can overflow
         __nv_bfloat16* prow = p.P + static_cast<long long>(local) * p.p_pitch;
         for (int j = lane; j < K; j += 32) {
             const int tok = p.sidx[ro + j];
-            if (tok != INT_MAX) prow[tok] = __float2bfloat16_rn(__bfloat162float(prow[tok]) - p.sq[ro + j] * inv);
+            if (tok != INT_MAX) prow[tok] = __float2bfloat16_rn(__bfloat162float(prow[tok]) - p.sq[ro + j] / S_q * sum);
         }
     }
 }
