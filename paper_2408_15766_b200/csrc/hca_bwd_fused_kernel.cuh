@@ -97,7 +97,7 @@ struct RowsParams {
 };
 
 __global__ void __launch_bounds__(256, 2) hca_bwd_rows_kernel(const __grid_constant__ RowsParams p) {
-    wait_previous_kernel();
+    wait_previous_kernel(false);
     if (blockIdx.x == 0 && threadIdx.x < 64) p.status[threadIdx.x] = 0u;
     const long long w = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 4;   // (b, t, g)
     const int sub = threadIdx.x & 15;
@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(256, 2) hca_bwd_rows_kernel(const __grid_const
 // dQ = the fp32 accumulator as bf16; 8 values per thread.
 __global__ void __launch_bounds__(256) hca_dq_convert_kernel(const float* acc, __nv_bfloat16* dQ,
                                                              long long n8) {
-    wait_previous_kernel();
+    wait_previous_kernel(false);
     const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= n8) return;
     float v[8];
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_bwd_fused_kernel(const __g
         tmem_alloc(smem_u32(tmem_ptr_smem), F_TMEM_COLS);
         tmem_relinquish();
     }
-    wait_previous_kernel();
+    wait_previous_kernel(false);
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();

@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
         tmem_alloc(smem_u32(tmem_ptr_smem), TMEM_COLS);
         tmem_relinquish();
     }
-    wait_previous_kernel();
+    wait_previous_kernel(false);
     if (p.one_round && blockIdx.x == 0 && threadIdx.x < 64) p.status[threadIdx.x] = 0u;
     tc_fence_before_sync();
     __syncthreads();
