@@ -141,16 +141,16 @@ int hass_topk_distill_bwd(const void* H_d, const void* W, int64_t N, int64_t d, 
  * 2^(z_d log2(e) - ref2), ref2 a per-row exponent fixed from the row's draft logit at the most
  * probable token of Omega_hat. With coef = g S_q 2^ref2 / sum_v e^{z_d},
  *     dz_d(v) = coef ( spill(v) - [v in Omega_hat] g q(v) / coef ),
- * so the K entries of a row at its Omega_hat tokens are lowered in place (in bf16) and
+ * so the K entries of a row at its Omega_hat tokens are replaced by that difference, formed in fp32, and
  * dH_d = coef (spill W) is formed by the second GEMM, whose epilogue applies the row scale.
- * Precision: every entry of dz_d, the Omega_hat entries included, reaches the tensor cores in bf16
- * (2^-9 relative); the loss uses fp32 logits throughout.
+ * Precision: every entry of dz_d, the Omega_hat entries included, is rounded to bf16 once (2^-9 relative) on
+ * its way to the tensor cores; the loss uses fp32 logits throughout.
  * Range condition: the fixed exponent holds as long as no draft logit of a row exceeds the one it
  * was taken from by more than about 90 (natural-log units; a probability ratio of e^90). The sweep
  * detects a violation and records every row's largest logit; the call therefore also enqueues the
  * steps from the draft sweep on a second time, as conditional launches that return at once unless a
  * violation was detected, in which case they redo the call with each row's exponent taken from that
- * record (no logit of the row can exceed it). The result is correct either way. The _draft form and
+ * record (no logit of the row can exceed it). The precision is the same either way. The _draft form and
  * the Top-P variant work the same way, and so do hass_combined_distill_fwd_bwd and the Bi-directional
  * variant, whose exponent comes from the row's largest logit among the first 256 tokens and whose
  * second pass repeats the whole sequence.

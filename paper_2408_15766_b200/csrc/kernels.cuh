@@ -1871,9 +1871,11 @@ __global__ void __launch_bounds__(sel_block_warps(WARPS) * 32) select_kernel(con
 // loss_patch_kernel: one warp per row, after the sweep of the draft rows of the fused call. Merges the draft's
 // partial statistics into lse_d, evaluates Eq. 1 from the captured draft logits, writes the per-row scale of the
 // spilled tiles, and puts the Omega_hat term of dz_d into the spill itself: with the spilled value
-// P~(v) = 2^(z_d(v) log2e - ref2), dz_d(v) = coef (P~(v) - [v in Omega_hat] q(v) / (S_q e^(m_spill - lse_d))),
-// so the K entries of the row at its Omega_hat tokens are lowered in place (bf16) and the second GEMM needs
-// nothing but the row scale in its epilogue.
+// P~(v) = e^(z_d(v) - m_spill), dz_d(v) = coef (P~(v) - [v in Omega_hat] q(v) / (S_q e^(m_spill - lse_d))),
+// so the K entries of the row at its Omega_hat tokens are replaced by that difference and the second GEMM needs
+// nothing but the row scale in its epilogue. The difference is formed in fp32 from the captured logit and rounded to
+// bf16 once: taken off the spilled bf16 value, q would leave the rounding of p (2^-9 p), which is most of the
+// difference where the draft is close to its target (p within 1 % of q: 8e-2 of the largest gradient entry).
 struct LossPatchParams {
     Schedule sched;        // schedule of the draft sweep
     int K;
@@ -1931,7 +1933,7 @@ __global__ void __launch_bounds__(256) loss_patch_kernel(const __grid_constant__
         __nv_bfloat16* prow = p.P + static_cast<long long>(local) * p.p_pitch;
         for (int j = lane; j < K; j += 32) {
             const int tok = p.sidx[ro + j];
-            if (tok != INT_MAX) prow[tok] = __float2bfloat16_rn(__bfloat162float(prow[tok]) - p.sq[ro + j] / S_q * sum);
+            if (tok != INT_MAX) prow[tok] = __float2bfloat16_rn(expf(p.cap_z[ro + j] - m_spill) - p.sq[ro + j] / S_q * sum);
         }
     }
 }
