@@ -166,37 +166,54 @@ def test_split_calls_match_fused_call_and_draft_only_forward():
     print("step 2 fused", compare(inp.H_t, inp.H_d[1], inp.W, wl.K, gpu, grad_loss=g.cpu().numpy()))
 
 
-def test_rows_beyond_the_exponent_range_of_the_spill_are_redone_exactly():
+def _second_pass(ws):
+    """Word 1 of the status block: the sweep asked for the second pass."""
+    return int(ws[4:8].view(torch.int32)[0]) != 0
+
+
+def _chunk_rows():
+    """Rows of a full chunk: a quarter of the SM count in row tiles, an even number of them."""
+    return torch.cuda.get_device_properties(0).multi_processor_count // 8 * 2 * 128
+
+
+@pytest.mark.parametrize("N", [40, 200])
+def test_rows_beyond_the_exponent_range_of_the_spill_are_redone(N):
+    # Of 40 rows only the Bi-directional call spills (the others keep the draft logits in fp32), of 200 rows all five do.
     hass = _hass()
-    N, d, V, K = 40, 64, 700, 3
+    d, V, K = 64, 700, 3
     inp = hi.make_custom(N, d, V, K, seed=3, sigma_w=0.1)
     H_d = torch.ones(N, d, dtype=torch.bfloat16)
     W = inp.W.clone()
     W[:256] = -2.0                    # draft logits of the first 256 tokens: -128
     W[300] = 2.0                      # one later token at +128: 256 above the row reference
     dev = torch.device("cuda:0")
-    # the plain fused call notices and falls back to its exact route on the device
+    # the plain fused call notices and sweeps the draft rows a second time, every row's reference taken from the row's
+    # largest logit, which the first sweep recorded
     out = hass.topk_distill_fwd_bwd(inp.H_t.to(dev), H_d.to(dev), W.to(dev), K, dH_dtype=hass.HASS_FP32)
     hass.check(out["workspace"])
+    assert _second_pass(out["workspace"]) == (N > 128)
     print(compare(inp.H_t, H_d, W, K, _to_cpu(out)))
     d2 = hass.topk_distill_fwd_bwd_draft(H_d.to(dev), W.to(dev), out["topk_idx"], out["topk_q"],
                                          dH_dtype=hass.HASS_FP32, workspace=out["workspace"])
     hass.check(out["workspace"])
+    assert _second_pass(out["workspace"]) == (N > 128)
     assert torch.allclose(d2["loss"], out["loss"], rtol=1e-5) and torch.allclose(d2["dH_d"], out["dH_d"], atol=1e-6)
-    # the Top-P variant has the same second route ...
+    # the Top-P variant does the same ...
     import oracle
     v = hass.variant_distill_fwd_bwd(inp.H_t.to(dev), H_d.to(dev), W.to(dev), K, hass.LOSS_TOP_P, 0.004,
                                      dH_dtype=hass.HASS_FP32)
     hass.check(v["workspace"])
-    print("top-p, exact route", compare_variant(inp.H_t, H_d, W, K, oracle.VARIANT_TOP_P, 0.004, _to_cpu(v)))
-    # ... and the Bi-directional variant and the combined objective sweep a second time with every row's reference
-    # taken from the row's largest logit, which the first sweep recorded
+    assert _second_pass(v["workspace"]) == (N > 128)
+    print("top-p, second pass", compare_variant(inp.H_t, H_d, W, K, oracle.VARIANT_TOP_P, 0.004, _to_cpu(v)))
+    # ... and the Bi-directional variant and the combined objective repeat their whole sequence
     v = hass.variant_distill_fwd_bwd(inp.H_t.to(dev), H_d.to(dev), W.to(dev), K, hass.LOSS_BIDIR_TOPK, 0.0,
                                      dH_dtype=hass.HASS_FP32)
     hass.check(v["workspace"])
+    assert _second_pass(v["workspace"])
     print("bidir, second sweep", compare_variant(inp.H_t, H_d, W, K, oracle.VARIANT_BIDIR, 0.0, _to_cpu(v)))
     c = hass.combined_distill_fwd_bwd(inp.H_t.to(dev), H_d.to(dev), W.to(dev), K, w_topk=0.5, dH_dtype=hass.HASS_FP32)
     hass.check(c["workspace"])
+    assert _second_pass(c["workspace"]) == (N > 128)
     cpu = _to_cpu(c)
     print("combined, second sweep", compare(inp.H_t, H_d, W, K, cpu, check_dH=False))
     ref = oracle.objective_from_features(hi.bf16_bits(inp.H_t), hi.bf16_bits(H_d), hi.bf16_bits(W), K, 1.0, 0.5,
@@ -209,10 +226,10 @@ def test_rows_beyond_the_exponent_range_of_the_spill_are_redone_exactly():
     assert hass.status_string(-7) == "HASS_ERR_RANGE"
 
 
-def test_exact_route_with_two_row_chunks_when_only_some_rows_exceed_the_range():
-    """N = 4800 is two row chunks (4736 + 64 rows), K = 17 runs the buffered Top-K sweep. A handful of rows in
-    both chunks have one draft logit more than 200 above everything among the first 256 tokens; the fused call
-    must notice and redo every row exactly."""
+def test_second_pass_with_two_row_chunks_when_only_some_rows_exceed_the_range():
+    """N = 4800 is two row chunks (4608 + 192 rows on a 148-SM device), K = 17 runs the buffered Top-K sweep. A handful of
+    rows, the last of the first chunk and the first of the second among them, have one draft logit more than 200 above
+    everything among the first 256 tokens; the fused call must notice and redo every row."""
     hass = _hass()
     N, d, V, K = 4800, 64, 700, 17
     inp = hi.make_custom(N, d, V, K, seed=31, sigma_w=0.1)
@@ -220,20 +237,24 @@ def test_exact_route_with_two_row_chunks_when_only_some_rows_exceed_the_range():
     W = inp.W.clone()
     W[300] = (0.125 * u).to(torch.bfloat16)          # an ordinary row's logit of token 300 stays of order 1
     H_d = inp.H_d[0].clone()
-    hot = [5, 130, 4735, 4736, 4790]
+    edge = _chunk_rows()
+    assert 130 < edge < 4790
+    hot = [5, 130, edge - 1, edge, 4790]
     H_d[hot] = (37.5 * u).to(torch.bfloat16)         # z_d[300] = 64 * 0.125 * 37.5 = 300 on these rows, |z_d| < 100 elsewhere
     dev = torch.device("cuda:0")
     grad = np.random.default_rng(4).uniform(0.5, 1.5, size=N)
     out = hass.topk_distill_fwd_bwd(inp.H_t.to(dev), H_d.to(dev), W.to(dev), K, dH_dtype=hass.HASS_FP32,
                                     grad_loss=torch.tensor(grad, dtype=torch.float32, device=dev))
     hass.check(out["workspace"])
-    rows = np.unique(np.concatenate([np.array(hot), hi.sample_rows(N, 400, seed=2)]))
+    assert _second_pass(out["workspace"])
+    rows = np.unique(np.concatenate([np.array(hot), [edge - 2, edge + 1], hi.sample_rows(N, 400, seed=2)]))
     print(compare(inp.H_t, H_d, W, K, _to_cpu(out), rows=rows, grad_loss=grad))
     # the same inputs with the hot rows removed stay on the fused route and agree on the other rows
     calm = inp.H_d[0].to(dev)
     ref = hass.topk_distill_fwd_bwd(inp.H_t.to(dev), calm, W.to(dev), K, dH_dtype=hass.HASS_FP32,
                                     grad_loss=torch.tensor(grad, dtype=torch.float32, device=dev))
     hass.check(ref["workspace"])
+    assert not _second_pass(ref["workspace"])
     keep = np.setdiff1d(np.arange(N), hot)
     assert torch.equal(out["topk_idx"].cpu()[keep], ref["topk_idx"].cpu()[keep])
     assert torch.allclose(out["loss"].cpu()[keep], ref["loss"].cpu()[keep], rtol=1e-3, atol=1e-7)
@@ -242,6 +263,7 @@ def test_exact_route_with_two_row_chunks_when_only_some_rows_exceed_the_range():
     v = hass.variant_distill_fwd_bwd(inp.H_t.to(dev), H_d.to(dev), W.to(dev), K, hass.LOSS_BIDIR_TOPK, 0.0,
                                      dH_dtype=hass.HASS_FP32)
     hass.check(v["workspace"])
+    assert _second_pass(v["workspace"])
     print("bidir, two chunks, second pass",
           compare_variant(inp.H_t, H_d, W, K, oracle.VARIANT_BIDIR, 0.0, _to_cpu(v), rows=rows))
 
@@ -306,10 +328,10 @@ def test_host_buffer_entry_matches_device_entry():
     assert torch.equal(idx_h, ref["topk_idx"].cpu())
 
 
-def test_host_buffer_entry_with_several_row_chunks_and_the_exact_route():
+def test_host_buffer_entry_with_several_row_chunks_and_the_second_pass():
     """N = 4800 is two row chunks: the second chunk's rows travel to the device while the first computes and
     the first chunk's dH_d rows travel back meanwhile; results equal the device entry's bit for bit. With a row
-    beyond the spill's exponent range the exact route redoes the call after the chunks' dH_d rows have left,
+    beyond the spill's exponent range the second pass redoes the call after the chunks' dH_d rows have left,
     and the entry must fetch them again."""
     hass = _hass()
     N, d, V, K = 4800, 64, 700, 5
@@ -325,6 +347,7 @@ def test_host_buffer_entry_with_several_row_chunks_and_the_exact_route():
         grad = torch.rand(N, generator=torch.Generator().manual_seed(2)) + 0.5
         ref = hass.topk_distill_fwd_bwd(inp.H_t.to(dev), H_d.to(dev), Wd, K, grad_loss=grad.to(dev))
         hass.check(ref["workspace"])
+        assert _second_pass(ref["workspace"]) == hot
         loss_h = torch.empty(N, dtype=torch.float32).pin_memory()
         dH_h = torch.full((N, d), float("nan"), dtype=torch.bfloat16).pin_memory()
         q_h = torch.empty(N, K, dtype=torch.float32).pin_memory()
@@ -336,11 +359,11 @@ def test_host_buffer_entry_with_several_row_chunks_and_the_exact_route():
         if hot:
             print(compare(inp.H_t, H_d, W, K, dict(loss=loss_h, topk_idx=ref["topk_idx"].cpu(), topk_q=q_h,
                                                    lse_t=ref["lse_t"].cpu(), lse_d=ref["lse_d"].cpu(), dH_d=dH_h),
-                          rows=np.array([0, 7, 100, 4735, 4736, 4790, 4799]), grad_loss=grad.numpy().astype(np.float64)))
+                          rows=np.array([0, 7, 100, _chunk_rows() - 1, _chunk_rows(), 4790, 4799]), grad_loss=grad.numpy().astype(np.float64)))
 
 
 def test_host_buffer_entry_with_more_row_chunks_than_it_has_events():
-    """409600 rows are 87 row chunks on a 148-SM device, more than the entry's event pool covers: it falls back to
+    """409600 rows are 89 row chunks on a 148-SM device, more than the entry's event pool covers: it falls back to
     one copy in, the call, one copy out, and the results still equal the device entry's."""
     hass = _hass()
     N, d, V, K = 3200 * 128, 8, 64, 2
