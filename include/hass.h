@@ -6,8 +6,8 @@
  * with respect to H_d. No N x V logit matrix is ever held in memory: logits exist tile by tile in
  * tensor memory. What does pass through the workspace, between the forward sweep and the
  * back-projection of the fused call, is a bounded chunk of un-normalised bf16 draft probabilities
- * (chunk rows x V, chunk rows = 128 x a quarter of the SM count, 4736 on a 148-SM device whatever
- * N is: 1.2 GB for V = 128256); see hass_topk_distill_fwd_bwd.
+ * (chunk rows x V, chunk rows = 128 x the even part of a quarter of the SM count, 4608 on a 148-SM device
+ * whatever N is: 1.2 GB for V = 128256); see hass_topk_distill_fwd_bwd.
  *
  * Notation follows the paper (Section 3.1): q = softmax(H_t W^T) is the target LLM's
  * next-token distribution, p = softmax(H_d W^T) the draft model's, Omega the vocabulary
@@ -391,7 +391,7 @@ int hass_topk_distill_fwd_static(const void* H_t, const void* H_d, const void* W
  * milliseconds and launch counts per kernel kind into arrays of at least HASS_PROFILE_KINDS
  * entries, and clears the records. Kinds: 0 logits+statistics GEMM (forward), 1 dz_d GEMM
  * (backward, recompute), 2 dH_d GEMM (backward), 3 finalize, 4 backward preparation, 5 the conditional
- * launches of the exact route behind a fused call (they return at once unless it is needed),
+ * launches of the second pass behind a fused call (they return at once unless a row left the range of its spill),
  * 6 HCA attention forward, 7 / 8 / 9 HCA attention backward: conversion of dQ to bf16, the tensor-core kernel,
  * the row kernel (row sums, substituted entries, the draft passes' gradients), 10 the sweep of the draft rows in hass_topk_distill_fwd_bwd, its
  * _draft form and the Top-P variant (kind 0 is then the sweep of the target rows alone).

@@ -414,6 +414,7 @@ def selftest_wait_expiry(workspace: torch.Tensor, limit_ns: int = 2_000_000, str
         "hass_selftest_wait_expiry")
 
 
+# (exact_route_conditional: the conditional launches of the second pass behind a fused call)
 PROFILE_KINDS = ("stats_gemm", "dz_gemm", "dH_gemm", "finalize", "bwd_prep", "exact_route_conditional",
                  "hca_attention", "hca_bwd_dq_convert", "hca_bwd_fused", "hca_bwd_rows", "stats_gemm_draft")
 
