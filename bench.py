@@ -32,13 +32,13 @@ import hass_inputs as hi  # noqa: E402
 
 METRIC = "tokens/sec fused top-K distill fwd+bwd"
 UNIT = "tokens/s"
-# dram__bytes_read + dram__bytes_write per launch of the three GEMM kernels of the fused call, from the ncu
-# captures summarised in profiles/gemm_kernels_l2-7b_ncu_full.md (l2-7b shape, K = 10; mean of the two row-chunk
-# launches of one step). Valid for the library version they were taken with; for the l3-8b shape the figures
-# are scaled by the vocabulary ratio (W, the spill and its re-reads all grow with V; the 2 x 39 MB of H rows
-# and the dH_d rows that do not are 6 % of the total).
-TRAFFIC_CAPTURE = {"version": 10410, "workload": "l2-7b", "V": 32000, "K": 10,
-                   "bytes_per_launch": {"stats_gemm": 495.0e6, "stats_gemm_draft": 759.1e6, "dH_gemm": 1212.1e6}}
+# dram__bytes_read + dram__bytes_write per launch of the two sweeps of the fused call, from the ncu captures summarised
+# in profiles/gemm_kernels_l2-7b_ncu_full.md (l2-7b shape, K = 10; mean of the two row-chunk launches of one step). Valid
+# for the library version they were taken with; for the l3-8b shape the figures are scaled by the vocabulary ratio (W and
+# the spill grow with V; the 2 x 34 MB of H rows that do not are 6-11 % of the total). The launches counted under the
+# dH_d GEMM include the sum of its partial tiles, so that it has no figure per launch here.
+TRAFFIC_CAPTURE = {"version": 10500, "workload": "l2-7b", "V": 32000, "K": 10,
+                   "bytes_per_launch": {"stats_gemm": 302.1e6, "stats_gemm_draft": 578.0e6}}
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 
 

@@ -389,11 +389,12 @@ __device__ __forceinline__ void finish_out4(const GemmParams& p, float4 a, int l
 }
 
 // CG: CTAs per product. The kernel is bound by the tensor pipe and, in calls of many milliseconds, by the power cap. A pair
-// (tcgen05 cta_group::2, 256 x 256 tile) fetches 32 KB per CTA and k block instead of 48 (10 instead of 15 TB/s out of
-// L2) and reads half as much of B from shared memory; with the stages smaller there are six instead of four. A step of
-// a pair takes 0.89-0.91 of the time of the two single steps it replaces (sweep of 8192 rows x 4096 x 32000: 1.77 -> 1.45 ms
-// = 1480 TFLOP/s in short runs; 1.24 -> 1.30 PFLOP/s where the power cap holds). Single CTAs stay for one row tile, where
-// a partner would have nothing to do, and where an odd number of row tiles makes pairs slower (plan_launch, plan_out).
+// (tcgen05 cta_group::2, 256 x 256 tile) fetches 32 KB per CTA and k block instead of 48 (sweep of 4608 rows x 4096 x
+// 32000: 9.4 GB out of L2 at 12.6 TB/s, by its counter; single CTAs half as much again) and reads half as much of B from
+// shared memory; with the stages smaller there are six instead of four. A step of a pair takes 0.89-0.91 of the time of
+// the two single steps it replaces (sweep of 8192 rows x 4096 x 32000: 1.77 -> 1.45 ms = 1480 TFLOP/s in short runs;
+// 1.24 -> 1.30 PFLOP/s where the power cap holds). Single CTAs stay for one row tile, where a partner would have nothing
+// to do, and where an odd number of row tiles makes pairs slower (plan_launch, plan_out).
 template <int MODE, int TOPK, int CG>
 __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_constant__ GemmParams p) {
     constexpr bool B_MN_MAJOR = (MODE == MODE_OUT);
