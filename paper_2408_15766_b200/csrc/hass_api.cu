@@ -3,6 +3,7 @@
 // hass_check and the *_host entry.
 #include <atomic>
 #include <climits>
+#include <cstdint>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -110,7 +111,8 @@ static int device_info(DeviceInfo* out) {
                                     gemm_kernel<MODE_STATS, TOPK_BUF, 1>,  gemm_kernel<MODE_STATS, TOPK_BUF, 2>,
                                     gemm_kernel<MODE_STATS, TOPK_NONE, 1>, gemm_kernel<MODE_STATS, TOPK_NONE, 2>,
                                     gemm_kernel<MODE_PROBS, TOPK_BUF, 1>,  gemm_kernel<MODE_PROBS, TOPK_BUF, 2>,
-                                    gemm_kernel<MODE_OUT, TOPK_BUF, 1>,    gemm_kernel<MODE_OUT, TOPK_BUF, 2>};
+                                    gemm_kernel<MODE_OUT, TOPK_BUF, 1>,    gemm_kernel<MODE_OUT, TOPK_BUF, 2>,
+                                    gemm_kernel<MODE_LOGITS, TOPK_BUF, 1>, gemm_kernel<MODE_LOGITS, TOPK_BUF, 2>};
             cudaError_t e3 = cudaSuccess;
             for (GemmFn f : gemms)
                 if (e3 == cudaSuccess) e3 = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
@@ -439,12 +441,12 @@ static int make_layout(long long N, long long d, long long V, int K, int sms, La
                                                    L->scratch_row_tile_bytes - 256, nullptr));
         if (need > L->part_bytes) L->part_bytes = need;
     }
-    if (N > BM / 2 && N <= BM) {
-        // the fp32 logits of such a call (narrow_room), from `sparse` on
-        const size_t z_end = L->sparse + static_cast<size_t>(N) * L->p_pitch * 4;
-        const size_t most = L->scratch_row_tile_bytes - 256;
-        const size_t need = z_end > L->total_pref ? align256(z_end - L->total_pref) : 0;
-        if (need <= most && need > L->part_bytes) L->part_bytes = need;
+    if (N <= BM) {
+        // the fp32 logits of such a call (narrow_room), from the scratch on, and its partial tiles; one chunk in any case
+        const size_t z = align256(static_cast<size_t>(N) * L->p_pitch * 4);
+        const size_t parts = align256(part_bytes_of(plan_out(static_cast<int>(N), ceil_div(d, BN), ceil_div(V, BK), sms, SIZE_MAX, nullptr)));
+        const size_t end = L->scratch + z + (parts > z ? parts : z);
+        if (end > L->total_pref && end - L->total_pref > L->part_bytes) L->part_bytes = end - L->total_pref;
     }
     return HASS_OK;
 }
@@ -634,7 +636,6 @@ static int forward_impl(bool with_target, const void* H_t, const void* H_d, cons
     if (rc != HASS_OK) return rc;
     log_schedule(with_target ? "fwd stats" : "fwd stats (draft)", p.sched);
     p.spill_begin = INT_MAX;
-    p.z_begin = INT_MAX;
     p.a_row_offset = 0;
     p.row_global_offset = 0;
     p.rows_valid = static_cast<int>(N);
@@ -796,118 +797,125 @@ struct Combined {
     float* coef_t;         // [N] scratch: scale of the target spill
     float* T;              // [chunk rows, d] scratch: q W of the chunk's rows
     __nv_bfloat16* Pt;     // [chunk rows, p_pitch] scratch: spill of the target tiles
+    size_t end;            // bytes of the caller's workspace
 };
 
-// Calls of one row tile, where the draft logits go through the workspace in fp32 (narrow_impl). Such a call is bound by
+// Calls of one row tile, where the logits go through the workspace in fp32 (narrow_impl). Such a call is bound by
 // reading W, which this route does twice (both sweeps in one launch, then the second GEMM) instead of three times, with no
 // range condition and so no second pass: 61 rows x 4096 x 32000 211 -> 147 us, 64 rows x 256 x 1024 67 -> 46 us, 100 rows
-// x 4096 x 32000 215 -> 147 us. Up to 64 rows they fit the scratch of one row tile; beyond, the fp32 rows kept for the
-// Omega_hat term and the room for partial tiles serve too, and a workspace that ends before them takes the other route.
+// x 4096 x 32000 215 -> 147 us. The sweep does nothing but store its accumulators, and one kernel does the rest of a row: with
+// candidate lists and statistics in the sweep's epilogue, a kernel that selects and one that forms dz_d, the last tile's epilogue, on its
+// own at the end, took 12 us and the two kernels 25 (61 rows x 4096 x 32000: 135 -> 112 us on the device, 64 rows x 256 x 1024 39 -> 26,
+// 76 rows x 4096 x 128256 with K = 44 508 -> 478). The logits take the scratch and what follows; the partial
+// tiles of the second GEMM take the target's, which are read no more by then. A workspace that ends before them takes the
+// other route.
+// Bi-directional calls take it from this size of W on (40 rows x 256 x 1024 68 -> 35 us, 35 rows x 4096 x 32000 186 -> 123 us). No head in
+// use is smaller; there the spill and its second pass, which a draft of 256 logits above its reference needs, stay in use
+// at few rows too.
+constexpr long long kNarrowBidirBytes = 128 << 10;
 struct NarrowRoom {
     float* z = nullptr;      // [N, p_pitch], or nullptr: no room
-    PartRoom part;           // what is left for partial tiles
+    float* zt = nullptr;     // [N, p_pitch]
+    PartRoom part;
 };
-static NarrowRoom narrow_room(long long N, uint8_t* ws, size_t workspace_bytes, const Layout& L, const PartRoom& part) {
+static NarrowRoom narrow_room(long long N, uint8_t* ws, size_t workspace_bytes, const Layout& L) {
     NarrowRoom r;
-    const size_t need = static_cast<size_t>(N) * L.p_pitch * 4;
-    if (N <= BM / 2 && workspace_bytes >= L.scratch + need) {
+    const size_t z = align256(static_cast<size_t>(N) * L.p_pitch * 4);
+    if (N <= BM && workspace_bytes >= L.scratch + 2 * z) {
         r.z = reinterpret_cast<float*>(ws + L.scratch);
-        r.part = part;
-    } else if (N <= BM && workspace_bytes >= L.sparse + need) {
-        r.z = reinterpret_cast<float*>(ws + L.sparse);
+        r.zt = reinterpret_cast<float*>(ws + L.scratch + z);
+        r.part.at = r.zt;
+        r.part.bytes = workspace_bytes - L.scratch - z;
     }
     return r;
 }
 
-static int narrow_impl(bool with_target, const void* H_t, const void* H_d, const void* W, int N, long long d, long long V,
-                       int K, const float* grad_loss, const int* idx_in, const float* q_in, float* loss, int* idx_out,
-                       float* q_out, float* lse_t, float* lse_d, void* dH_d, int dH_dtype, uint8_t* ws, const Layout& L,
-                       const NarrowRoom& room, const DeviceInfo& di, cudaStream_t st, float top_p, int* topk_n,
-                       const Combined* cmb = nullptr) {
-    const int CT = ceil_div(V, BN), DT = ceil_div(d, BN);
-    unsigned int* status = reinterpret_cast<unsigned int*>(ws + L.status);
-    float* z = room.z;
-    const PartRoom& part = room.part;
-    // (1) target and draft rows in one sweep: statistics, candidates, the draft's logits
+// The logits of N <= BM rows of H0 and (nullable) of H1 -> z0, z1 [N, p_pitch]; clears the status block.
+static int narrow_sweep(const void* H0, const void* H1, const void* W, int N, long long d, long long V, float* z0, float* z1,
+                        uint8_t* ws, const Layout& L, const DeviceInfo& di, cudaStream_t st) {
     GemmParams p;
     std::memset(&p, 0, sizeof(p));
     // up to 64 rows each share one row tile (61 rows x 4096 x 32000: 65 us as two row tiles of a CTA pair, 61 as one)
-    p.half_tiles = with_target && N <= BM / 2 ? 1 : 0;
-    p.row_tiles = with_target && !p.half_tiles ? 2 : 1;
-    int rc = plan_launch(p.row_tiles, CT, di.sms, L.slot_cap, &p.sched);
+    p.half_tiles = H1 && N <= BM / 2 ? 1 : 0;
+    p.row_tiles = H1 && !p.half_tiles ? 2 : 1;
+    int rc = plan_launch(p.row_tiles, ceil_div(V, BN), di.sms, L.slot_cap, &p.sched);
     if (rc != HASS_OK) return rc;
     log_schedule("narrow sweep", p.sched);
     const int box_rows = p.half_tiles ? BM / 2 : BM;
-    rc = make_tmap(&p.tmA1, H_d, N, d, d, BK, box_rows);
-    if (rc == HASS_OK) rc = make_tmap(&p.tmA0, with_target ? H_t : H_d, N, d, d, BK, box_rows);
+    rc = make_tmap(&p.tmA0, H0, N, d, d, BK, box_rows);
+    if (rc == HASS_OK) rc = make_tmap(&p.tmA1, H1 ? H1 : H0, N, d, d, BK, box_rows);
     if (rc == HASS_OK) rc = make_tmap(&p.tmB, W, V, d, d, BK, BN / p.sched.pair);
     if (rc != HASS_OK) return rc;
     p.row_tiles0 = 1;
-    p.topk_row_tiles = with_target ? 1 : 0;
     p.spill_begin = INT_MAX;
-    p.z_begin = 0;
     p.z_rows = N;
-    p.z_out = z;
-    p.zt_out = cmb ? reinterpret_cast<float*>(cmb->Pt) : nullptr;
+    p.zt_out = z0;
+    p.z_out = z1;
     p.z_pitch = L.p_pitch;
     p.rows_valid = N;
     p.n_cols = static_cast<int>(V);
-    p.col_tiles = CT;
+    p.col_tiles = ceil_div(V, BN);
     p.k_blocks = ceil_div(d, BK);
-    p.K = K;
-    p.cap = topk_cap(K);
-    p.part_m = reinterpret_cast<float*>(ws + L.part_m);
-    p.part_s = reinterpret_cast<float*>(ws + L.part_s);
-    p.cand = reinterpret_cast<uint2*>(ws + L.cand_v);
-    p.cand_n = reinterpret_cast<int*>(ws + L.cand_i);
-    p.thr_share = reinterpret_cast<unsigned int*>(ws + L.thr_share);
-    p.status = status;
-    rc = clear_status(ws, L, with_target ? p.sched.total_slots : 0, st);
+    p.status = reinterpret_cast<unsigned int*>(ws + L.status);
+    p.clear_status = 1;
+    return launch_gemm<MODE_LOGITS>(p, st, H1 ? KIND_STATS : KIND_STATS_DRAFT);
+}
+
+static RowParams row_params(int V, int K, const Layout& L) {
+    RowParams r;
+    std::memset(&r, 0, sizeof(r));
+    r.K = K;
+    r.V = V;
+    r.pitch = L.p_pitch;
+    r.idx_pitch = K;
+    return r;
+}
+static int launch_rows(int objective, const RowParams& r, int N, cudaStream_t st) {
+    KernelTimer timer(KIND_FINALIZE, st);
+    return launch(objective == ROW_COMBINED ? row_kernel<ROW_COMBINED> : objective == ROW_BIDIR ? row_kernel<ROW_BIDIR> : row_kernel<ROW_TOPK>,
+                  N, ROW_THREADS, 0, st, 1, r);
+}
+
+static int narrow_impl(int objective, bool with_target, const void* H_t, const void* H_d, const void* W, int N, long long d,
+                       long long V, int K, const float* grad_loss, const int* idx_in, const float* q_in, float* loss,
+                       int* idx_out, float* q_out, float* lse_t, float* lse_d, void* dH_d, int dH_dtype, uint8_t* ws,
+                       const Layout& L, const NarrowRoom& room, const DeviceInfo& di, cudaStream_t st, float top_p, int* topk_n,
+                       const Combined* cmb = nullptr) {
+    // (1) the logits of the target and draft rows
+    int rc = with_target ? narrow_sweep(H_t, H_d, W, N, d, V, room.zt, room.z, ws, L, di, st)
+                         : narrow_sweep(H_d, nullptr, W, N, d, V, room.z, nullptr, ws, L, di, st);
     if (rc != HASS_OK) return rc;
-    rc = launch_gemm<MODE_STATS>(p, st, with_target ? KIND_STATS : KIND_STATS_DRAFT);
-    if (rc != HASS_OK) return rc;
-    // (2) Omega_hat
-    if (with_target) {
-        SelectParams sp = select_params(p, 0, 0, N, idx_out, q_out, K, lse_t);
-        sp.n_out = topk_n;
-        sp.top_p = top_p;
-        rc = launch_select(sp, di.sms, st);
-        if (rc != HASS_OK) return rc;
-    }
-    // (3) lse_d, loss, dz_d
-    DzParams z_params;
-    std::memset(&z_params, 0, sizeof(z_params));
-    z_params.sched = p.sched;
-    z_params.first_tile = p.row_tiles - 1;
-    z_params.first_row = p.half_tiles ? BM / 2 : 0;
-    z_params.K = K;
-    z_params.V = static_cast<int>(V);
-    z_params.part_m = p.part_m;
-    z_params.part_s = p.part_s;
-    z_params.idx = with_target ? idx_out : idx_in;
-    z_params.q = with_target ? q_out : q_in;
-    z_params.grad_loss = grad_loss;
-    z_params.loss = loss;
-    z_params.lse_d = lse_d;
-    z_params.z = z;
-    z_params.pitch = L.p_pitch;
-    z_params.make_dz = dH_d != nullptr ? 1 : 0;
+    // (2) statistics, Omega_hat, loss, dz_d
+    RowParams r = row_params(static_cast<int>(V), K, L);
+    r.z = room.z;
+    r.zt = with_target ? room.zt : nullptr;
+    r.idx = with_target ? idx_out : const_cast<int*>(idx_in);
+    r.q = with_target ? q_out : const_cast<float*>(q_in);
+    if (objective == ROW_BIDIR) r.idx_pitch = 2 * K;
+    r.top_p = top_p;
+    r.n_out = topk_n;
+    r.grad_loss = grad_loss;
+    r.lse_t = lse_t;
+    r.lse_d = lse_d;
+    r.loss = loss;
+    r.make_dz = dH_d != nullptr ? 1 : 0;
     if (cmb) {
-        z_params.zt = p.zt_out;
-        z_params.lse_t = lse_t;
-        z_params.w = cmb->w;
-        z_params.loss_ce = cmb->loss_ce;
+        r.w = cmb->w;
+        r.loss_ce = cmb->loss_ce;
     }
-    {
-        KernelTimer timer(KIND_FINALIZE, st);
-        rc = launch(cmb ? dz_kernel<true> : dz_kernel<false>, N, DZ_THREADS, 0, st, 1, z_params);
+    if (objective == ROW_BIDIR) {
+        r.W = static_cast<const __nv_bfloat16*>(W);
+        r.d = static_cast<int>(d);
+        r.coef_out = reinterpret_cast<float*>(ws + L.coef);
+        r.sparse_out = reinterpret_cast<float*>(ws + L.sparse);
     }
+    rc = launch_rows(objective, r, N, st);
     if (rc != HASS_OK) return rc;
     if (dH_d == nullptr) return HASS_OK;      // the forward alone
-    // (4) dH_d = dz_d W
+    // (3) dH_d = dz_d W
     GemmParams o;
     std::memset(&o, 0, sizeof(o));
-    rc = make_tmap(&o.tmA0, z, N, V, 2 * L.p_pitch, BK, BM);
+    rc = make_tmap(&o.tmA0, room.z, N, V, 2 * L.p_pitch, BK, BM);
     if (rc == HASS_OK) rc = make_tmap(&o.tmB, W, V, d, d, 64, BK);
     if (rc != HASS_OK) return rc;
     o.tmA1 = o.tmA0;
@@ -916,15 +924,17 @@ static int narrow_impl(bool with_target, const void* H_t, const void* H_d, const
     o.spill_begin = INT_MAX;
     o.rows_valid = N;
     o.n_cols = static_cast<int>(d);
-    o.col_tiles = DT;
+    o.col_tiles = ceil_div(d, BN);
     o.k_blocks = ceil_div(V, BK);
     o.K = K;
     o.out = dH_d;
     o.out_fp32 = dH_dtype == HASS_FP32 ? 1 : 0;
     o.out_align32 = ((reinterpret_cast<uintptr_t>(dH_d) | static_cast<uintptr_t>(d * (dH_dtype == HASS_FP32 ? 4 : 2))) & 31u) == 0 ? 1 : 0;
     o.out_pitch = d;
-    o.status = status;
-    return launch_out(o, part, di, st);
+    o.coef = r.coef_out;
+    o.sparse = r.sparse_out;
+    o.status = reinterpret_cast<unsigned int*>(ws + L.status);
+    return launch_out(o, room.part, di, st);
 }
 
 static int fused_impl(bool with_target, const void* H_t, const void* H_d, const void* W, long long N, long long d,
@@ -961,9 +971,12 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
     __nv_bfloat16* P = reinterpret_cast<__nv_bfloat16*>(ws + L.scratch);
     unsigned int* status = reinterpret_cast<unsigned int*>(ws + L.status);
     int* idx_d = reinterpret_cast<int*>(ws + L.sidx);
-    if (cmb && with_target && N <= BM / 2)      // (the target's fp32 logits take the place of its spill: one row tile of scratch)
-        return narrow_impl(true, H_t, H_d, W, static_cast<int>(N), d, V, K, grad_loss, nullptr, nullptr, loss, idx_out, q_out, lse_t,
-                           lse_d, dH_d, dH_dtype, ws, L, narrow_room(N, ws, workspace_bytes, L, part), di, st, 0.f, nullptr, cmb);
+    if (with_target && !(cmb && N > BM / 2) && !(bidir && V * d * 2 < kNarrowBidirBytes)) {
+        const NarrowRoom narrow = narrow_room(N, ws, cmb ? cmb->end : workspace_bytes, L);
+        if (narrow.z)
+            return narrow_impl(cmb ? ROW_COMBINED : bidir ? ROW_BIDIR : ROW_TOPK, true, H_t, H_d, W, static_cast<int>(N), d, V, K, grad_loss,
+                               nullptr, nullptr, loss, idx_out, q_out, lse_t, lse_d, dH_d, dH_dtype, ws, L, narrow, di, st, 0.f, topk_n, cmb);
+    }
     CUtensorMap tmHt, tmHd, tmWn, tmP;
     rc = make_tmap(&tmHd, H_d, N, d, d, BK, BM);
     if (rc == HASS_OK) rc = with_target ? make_tmap(&tmHt, H_t, N, d, d, BK, BM) : make_tmap(&tmHt, H_d, N, d, d, BK, BM);
@@ -1000,7 +1013,6 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
         p.row_tiles0 = tiles;
         p.topk_row_tiles = with_target ? (bidir ? 2 * tiles : tiles) : 0;
         p.spill_begin = with_target ? tiles : 0;
-        p.z_begin = INT_MAX;
         p.a_row_offset = t0 * BM;
         p.row_global_offset = t0 * BM;
         p.rows_valid = static_cast<int>(N);
@@ -1233,13 +1245,13 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
     float* coef = reinterpret_cast<float*>(ws + L.coef);
     float* capz = reinterpret_cast<float*>(ws + L.capz);
     float* ref2 = reinterpret_cast<float*>(ws + L.lse2);
-    const NarrowRoom narrow = narrow_room(N, ws, workspace_bytes, L, part);
+    const NarrowRoom narrow = narrow_room(N, ws, workspace_bytes, L);
     if (narrow.z) {
         if (pipe) {
             rc = pipe_in(pipe, H_t, H_d, 0, static_cast<size_t>(N), st);
             if (rc != HASS_OK) return rc;
         }
-        rc = narrow_impl(with_target, H_t, H_d, W, static_cast<int>(N), d, V, K, grad_loss, idx_in, q_in, loss, idx_out, q_out,
+        rc = narrow_impl(ROW_TOPK, with_target, H_t, H_d, W, static_cast<int>(N), d, V, K, grad_loss, idx_in, q_in, loss, idx_out, q_out,
                          lse_t, lse_d, dH_d, dH_dtype, ws, L, narrow, di, st, top_p, topk_n);
         if (rc != HASS_OK || !pipe) return rc;
         return pipe_out(pipe, dH_d, 0, static_cast<size_t>(N), st);
@@ -1308,7 +1320,6 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
                     t.tmA1 = tmHt;
                     t.topk_row_tiles = tiles;
                     t.spill_begin = INT_MAX;
-                    t.z_begin = INT_MAX;
                     rc = launch_gemm<MODE_STATS>(t, st);
                     if (rc != HASS_OK) return rc;
                 }
@@ -1441,9 +1452,9 @@ static int forward2_impl(bool with_target, const void* H_t, const void* H_d, con
                             workspace, workspace_bytes, st);
     const int RT = ceil_div(N, BM), CT = ceil_div(V, BN);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
-    const NarrowRoom narrow = narrow_room(N, ws, workspace_bytes, L, PartRoom());
+    const NarrowRoom narrow = narrow_room(N, ws, workspace_bytes, L);
     if (narrow.z)
-        return narrow_impl(with_target, H_t, H_d, W, static_cast<int>(N), d, V, K, nullptr, idx_in, q_in, loss, idx_out, q_out,
+        return narrow_impl(ROW_TOPK, with_target, H_t, H_d, W, static_cast<int>(N), d, V, K, nullptr, idx_in, q_in, loss, idx_out, q_out,
                            lse_t, lse_d, nullptr, HASS_BF16, ws, L, narrow, di, st, 0.f, nullptr);
     GemmParams p;
     std::memset(&p, 0, sizeof(p));
@@ -1455,7 +1466,6 @@ static int forward2_impl(bool with_target, const void* H_t, const void* H_d, con
     p.row_tiles = RT;
     p.row_tiles0 = RT;
     p.spill_begin = INT_MAX;
-    p.z_begin = INT_MAX;
     p.rows_valid = static_cast<int>(N);
     p.n_cols = static_cast<int>(V);
     p.col_tiles = CT;
@@ -1544,38 +1554,51 @@ static int normed_impl(const void* H_t, const void* H_d, const void* W, long lon
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     GemmParams p;
     std::memset(&p, 0, sizeof(p));
-    rc = plan_launch(RT, CT, di.sms, L.slot_cap, &p.sched);
-    if (rc != HASS_OK) return rc;
-    log_schedule("normed stats (target)", p.sched);
-    rc = make_tmap(&p.tmA0, H_t, N, d, d, BK, BM);
-    if (rc == HASS_OK) rc = make_tmap(&p.tmA1, H_t, N, d, d, BK, BM);
-    if (rc == HASS_OK) rc = make_tmap(&p.tmB, W, V, d, d, BK, BN / p.sched.pair);
-    if (rc != HASS_OK) return rc;
-    p.row_tiles = RT;
-    p.row_tiles0 = RT;
-    p.topk_row_tiles = RT;
-    p.spill_begin = INT_MAX;
-    p.z_begin = INT_MAX;
-    p.rows_valid = static_cast<int>(N);
-    p.n_cols = static_cast<int>(V);
-    p.col_tiles = CT;
-    p.k_blocks = ceil_div(d, BK);
-    p.K = K;
-    p.cap = topk_cap(K);
-    p.part_m = reinterpret_cast<float*>(ws + L.part_m);
-    p.part_s = reinterpret_cast<float*>(ws + L.part_s);
-    p.cand = reinterpret_cast<uint2*>(ws + L.cand_v);
-    p.cand_n = reinterpret_cast<int*>(ws + L.cand_i);
-    p.status = reinterpret_cast<unsigned int*>(ws + L.status);
-    p.thr_share = reinterpret_cast<unsigned int*>(ws + L.thr_share);
-    rc = clear_status(ws, L, p.sched.total_slots, st);
-    if (rc != HASS_OK) return rc;
-    rc = launch_gemm<MODE_STATS>(p, st);
-    if (rc != HASS_OK) return rc;
-    SelectParams sp = select_params(p, 0, 0, static_cast<int>(N), idx_out, q_out, K, lse_t);
-    sp.n_out = topk_n;
-    rc = launch_select(sp, di.sms, st);
-    if (rc != HASS_OK) return rc;
+    const NarrowRoom narrow = narrow_room(N, ws, workspace_bytes, L);
+    if (narrow.z) {
+        rc = narrow_sweep(H_t, nullptr, W, static_cast<int>(N), d, V, narrow.z, nullptr, ws, L, di, st);
+        if (rc != HASS_OK) return rc;
+        RowParams r = row_params(static_cast<int>(V), K, L);
+        r.zt = narrow.z;
+        r.idx = idx_out;
+        r.q = q_out;
+        r.n_out = topk_n;
+        r.lse_t = lse_t;
+        rc = launch_rows(ROW_TOPK, r, static_cast<int>(N), st);
+        if (rc != HASS_OK) return rc;
+    } else {
+        rc = plan_launch(RT, CT, di.sms, L.slot_cap, &p.sched);
+        if (rc != HASS_OK) return rc;
+        log_schedule("normed stats (target)", p.sched);
+        rc = make_tmap(&p.tmA0, H_t, N, d, d, BK, BM);
+        if (rc == HASS_OK) rc = make_tmap(&p.tmA1, H_t, N, d, d, BK, BM);
+        if (rc == HASS_OK) rc = make_tmap(&p.tmB, W, V, d, d, BK, BN / p.sched.pair);
+        if (rc != HASS_OK) return rc;
+        p.row_tiles = RT;
+        p.row_tiles0 = RT;
+        p.topk_row_tiles = RT;
+        p.spill_begin = INT_MAX;
+        p.rows_valid = static_cast<int>(N);
+        p.n_cols = static_cast<int>(V);
+        p.col_tiles = CT;
+        p.k_blocks = ceil_div(d, BK);
+        p.K = K;
+        p.cap = topk_cap(K);
+        p.part_m = reinterpret_cast<float*>(ws + L.part_m);
+        p.part_s = reinterpret_cast<float*>(ws + L.part_s);
+        p.cand = reinterpret_cast<uint2*>(ws + L.cand_v);
+        p.cand_n = reinterpret_cast<int*>(ws + L.cand_i);
+        p.status = reinterpret_cast<unsigned int*>(ws + L.status);
+        p.thr_share = reinterpret_cast<unsigned int*>(ws + L.thr_share);
+        rc = clear_status(ws, L, p.sched.total_slots, st);
+        if (rc != HASS_OK) return rc;
+        rc = launch_gemm<MODE_STATS>(p, st);
+        if (rc != HASS_OK) return rc;
+        SelectParams sp = select_params(p, 0, 0, static_cast<int>(N), idx_out, q_out, K, lse_t);
+        sp.n_out = topk_n;
+        rc = launch_select(sp, di.sms, st);
+        if (rc != HASS_OK) return rc;
+    }
     FinalizeParams f;
     std::memset(&f, 0, sizeof(f));
     f.sched = p.sched;
@@ -1790,6 +1813,7 @@ int hass_combined_distill_fwd_bwd(const void* H_t, const void* H_d, const void* 
     cmb.coef_t = reinterpret_cast<float*>(ws + c.coef_t);
     cmb.T = reinterpret_cast<float*>(ws + c.T);
     cmb.Pt = reinterpret_cast<__nv_bfloat16*>(ws + c.Pt);
+    cmb.end = workspace_bytes;
     return fused_impl(true, H_t, H_d, W, N, d, V, K, grad_loss, nullptr, nullptr, loss_topk, topk_idx, topk_q, lse_t,
                       lse_d, dH_d, dH_dtype, workspace, c.base, static_cast<cudaStream_t>(cuda_stream), &cmb, nullptr, false, &room);
 }

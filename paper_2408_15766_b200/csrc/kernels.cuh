@@ -1,7 +1,7 @@
 // Device code of the fused LM-head + Top-K distillation path (sm_100a).
 //
 // One warp-specialised, persistent GEMM kernel (TMA -> shared memory -> tcgen05.mma -> TMEM ->
-// epilogue warps) is instantiated with three epilogues:
+// epilogue warps) is instantiated with four epilogues:
 //   MODE_STATS  logits tile -> per-row softmax statistics, Top-K candidates (two variants: a sorted register
 //               list for K <= 16, append buffers with warp-cooperative compaction otherwise) and, in the fused
 //               forward+backward, a bf16 spill of 2^(z log2e - ref) that the second GEMM consumes
@@ -9,11 +9,13 @@
 //               (the separate, recomputing backward)
 //   MODE_OUT    dH_d tile: coef * acc - Omega_hat row (fused), coef * acc (q W of the combined objective)
 //               or the accumulator as is (separate backward)
+//   MODE_LOGITS logits tile in fp32, as it is (calls of few rows)
 // plus small kernels: out_reduce (partial tiles of MODE_OUT), select (after a sweep with Top-K candidates: lse,
 // Omega_hat, the set sorted by token id, the reference exponent of the draft rows' spill), loss_patch (after the draft
 // sweep: lse_d, Eq. 1, row scale, the Omega_hat term into the spill), finalize (routes without a draft sweep that
 // knows Omega_hat: gathered draft logits, Eq. 1 and its variants, the Omega_hat term of dH_d), ce_kernel (cross-entropy
-// of the combined objective) and bwd_prep (index-sorted Top-K lists for MODE_PROBS).
+// of the combined objective) and bwd_prep (index-sorted Top-K lists for MODE_PROBS). row
+// (after MODE_LOGITS: all that is done with a row's logits).
 // Beside the operand stages the kernel's shared memory holds 32 KB that the epilogue warps use: staging
 // buffers for the TMA stores of the spill (draft sweep) or the logits waiting for admission to the register
 // Top-K lists (target sweep).
@@ -51,7 +53,7 @@ constexpr float LOG2E = 1.4426950408889634f;
 // (g S_q) overflows likewise. With 1e20 both hold for g S_q down to 1e-18.
 constexpr float SPILL_SUM_LIMIT = 1e20f;
 
-enum { MODE_STATS = 0, MODE_PROBS = 1, MODE_OUT = 2 };
+enum { MODE_STATS = 0, MODE_PROBS = 1, MODE_OUT = 2, MODE_LOGITS = 3 };
 
 // A phase gives G consecutive row tiles S "lanes" each; lane l of a row tile sweeps the column
 // tiles l, l + S, l + 2S, ... CTA b < G * S works on row tile row_tile_begin + b / S, lane b % S, and
@@ -91,8 +93,8 @@ struct GemmParams {
                            // boxes of 64 columns x 32 rows, 128-byte swizzle, for TMA stores
     Schedule sched;
     int row_tiles;         // row tiles of this launch; a pair's second tile may lie beyond
-    int half_tiles;        // MODE_STATS, single CTAs: the one row tile is 64 rows of A0 (Top-K) and 64 of A1 (no Top-K), boxes
-                           // of 64 rows; a sweep of both that reads every tile of B once per call
+    int half_tiles;        // MODE_LOGITS, single CTAs: the one row tile is 64 rows of A0 and 64 of A1, boxes of 64 rows; a
+                           // sweep of both that reads every tile of B once per call
     int row_tiles0;        // row tiles [0, row_tiles0) read A0, the others A1 (tile index - row_tiles0)
     int topk_row_tiles;    // leading row tiles whose rows collect Top-K candidates (MODE_STATS)
     int a_row_offset;      // added to A0's row coordinate (chunked backward)
@@ -123,12 +125,13 @@ struct GemmParams {
     __nv_bfloat16* P;      // [chunk rows, p_pitch]
     __nv_bfloat16* Pt;     // [chunk rows, p_pitch] spill of the target tiles, or nullptr
     long long p_pitch;
-    // MODE_STATS: row tiles from z_begin on write the logits of their first z_rows rows in fp32 (INT_MAX: none): to z_out
-    // [z_rows, z_pitch], those of row tiles < row_tiles0 to zt_out
-    int z_begin, z_rows;
+    // MODE_LOGITS: the logits of the first z_rows rows of A0 (zt_out) and of A1 (z_out) in fp32, [z_rows, z_pitch], -inf
+    // beyond n_cols. One row tile of either matrix at most; with a single row tile that is not halved its matrix is A0
+    int z_rows;
     float* z_out;
     float* zt_out;
     long long z_pitch;
+    int clear_status;      // the first CTA zeroes the status block (no kernel of the call has run before this one)
     // MODE_OUT. With sparse != nullptr the epilogue computes coef[row] * acc - sparse[local row, :] (row scale
     // and the Omega_hat term of dz_d W, precomputed by finalize); with coef alone coef[row] * acc; with neither
     // it stores the accumulator.
@@ -442,7 +445,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
         fence_proxy_async_smem();
         prefetch_tensormap(&p.tmA0);
         prefetch_tensormap(&p.tmB);
-        if (MODE == MODE_STATS) prefetch_tensormap(&p.tmA1);
+        if (MODE == MODE_STATS || MODE == MODE_LOGITS) prefetch_tensormap(&p.tmA1);
     }
     if (warp == 1) {
         if (CG == 2) {
@@ -454,6 +457,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
         }
     }
     if (p.gate == nullptr) wait_previous_kernel();
+    // (A wait of another CTA that ran out would be recorded two seconds later.)
+    if (MODE == MODE_LOGITS && p.clear_status && blockIdx.x == 0 && threadIdx.x < 64) p.status[threadIdx.x] = 0u;
     tc_fence_before_sync();
     __syncthreads();
     if (CG == 2) cluster_sync();      // the partner's barriers are initialised, its tensor memory is allocated
@@ -508,7 +513,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
             int stage = 0;
             uint32_t phase = 0;
             for_each_item([&](int rt, int ln, int S, int, int kb0, int kb1) {
-                const bool second = (MODE == MODE_STATS) && rt >= p.row_tiles0;
+                const bool second = (MODE == MODE_STATS || MODE == MODE_LOGITS) && rt >= p.row_tiles0;
                 const CUtensorMap* tmA = second ? &p.tmA1 : &p.tmA0;
                 const int row0 = p.a_row_offset + (second ? rt - p.row_tiles0 : rt) * BM;
                 const int t0 = first_tile(rt, ln);
@@ -527,7 +532,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                                 tma_load_2d(dst, tm, bar, x, y);
                         };
                         const int col0 = ct * BN + static_cast<int>(rank) * (BN / CG);
-                        if (MODE == MODE_STATS && CG == 1 && p.half_tiles) {
+                        if (MODE == MODE_LOGITS && CG == 1 && p.half_tiles) {
                             load(smemA + stage * A_STAGE_BYTES, &p.tmA0, kb * BK, 0);
                             load(smemA + stage * A_STAGE_BYTES + A_STAGE_BYTES / 2, &p.tmA1, kb * BK, 0);
                         } else {
@@ -637,8 +642,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
             const int g_row = p.row_global_offset + rt * BM + r_local;
             const bool tile_ok = CG == 1 || rt < p.row_tiles;     // false: the partner of the last row tile, nothing to write
             const bool row_ok = tile_ok && g_row < p.rows_valid;
-            const bool second_half = MODE == MODE_STATS && CG == 1 && p.half_tiles && quad >= 2;
-            const int r_own = MODE == MODE_STATS && CG == 1 && p.half_tiles ? r_local % (BM / 2) : r_local;   // row in its own matrix
             // ---- per-item state ----
             float m = -INFINITY, s = 0.f, thr = -INFINITY;        // MODE_STATS; thr = admission threshold in force
             float thr_own = -INFINITY;                            // K-th (K_REG-th) largest logit of this lane's own list
@@ -653,10 +656,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
             const float* sg = nullptr;
             int cur = 0, nxt = INT_MAX;
             if (MODE == MODE_STATS) {
-                want_topk = HAS_TOPK && tile_ok && rt < p.topk_row_tiles && !second_half;
+                want_topk = HAS_TOPK && tile_ok && rt < p.topk_row_tiles;
                 if (HAS_TOPK) cbuf = p.cand + (static_cast<long long>(slot) * BM + r_local) * p.cap;
                 cnt = 0;
-                if (HAS_TOPK && p.row_global_offset + (rt < p.row_tiles0 ? rt : rt - p.row_tiles0) * BM + r_own >= p.rows_valid) {
+                if (HAS_TOPK && p.row_global_offset + (rt < p.row_tiles0 ? rt : rt - p.row_tiles0) * BM + r_local >= p.rows_valid) {
                     // A padding row collects nothing: its logits are all equal (zero), and 256 of them filled its buffer and
                     // made the warp compact row after row (sweep of 64 rows x 256 x 1024, K = 64: 195 -> 30 us).
                     thr_own = INFINITY;
@@ -686,10 +689,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                 nxt = si[0];
             }
             float* zrow = nullptr;
-            if (HAS_TOPK && tile_ok && rt >= p.z_begin && r_own < p.z_rows) {      // (one row tile of either kind)
-                const bool target = p.half_tiles ? !second_half : rt < p.row_tiles0 && p.row_tiles > 1;
-                float* z = target ? p.zt_out : p.z_out;
-                if (z != nullptr) zrow = z + static_cast<long long>(r_own) * p.z_pitch;
+            if (MODE == MODE_LOGITS && tile_ok) {
+                const bool halved = CG == 1 && p.half_tiles;
+                const int r_own = halved ? r_local % (BM / 2) : r_local;      // row in its own matrix
+                float* z = (halved ? quad >= 2 : rt >= p.row_tiles0) ? p.z_out : p.zt_out;
+                if (r_own < p.z_rows) zrow = z + static_cast<long long>(r_own) * p.z_pitch;
             }
             const int t0 = first_tile(rt, ln);
             const int nt = (p.col_tiles - ln + S - 1) / S;
@@ -822,18 +826,21 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                     tmem_ld32(t_row + ch * 32, r);
                     tmem_ld_wait(r);
                     const int col0 = col_base + ch * 32;
-                    if (MODE == MODE_STATS) {
+                    if (MODE == MODE_STATS || MODE == MODE_LOGITS) {
                         if (col0 + 32 > p.n_cols) {
 #pragma unroll
                             for (int j = 0; j < 32; ++j)
                                 if (col0 + j >= p.n_cols) r[j] = __float_as_uint(-INFINITY);
                         }
-                        if (HAS_TOPK && zrow != nullptr) {
+                    }
+                    if (MODE == MODE_LOGITS) {
+                        if (zrow != nullptr) {
 #pragma unroll
                             for (int g8 = 0; g8 < 4; ++g8)
                                 st_global_v8(zrow + col0 + 8 * g8, r[8 * g8], r[8 * g8 + 1], r[8 * g8 + 2], r[8 * g8 + 3],
                                              r[8 * g8 + 4], r[8 * g8 + 5], r[8 * g8 + 6], r[8 * g8 + 7]);
                         }
+                    } else if (MODE == MODE_STATS) {
                         if (CAPTURE) {
                             // draft logits at the row's Omega_hat, straight from the fp32 accumulator
                             while (nxt < col0 + 32) {
@@ -1940,72 +1947,316 @@ __global__ void __launch_bounds__(256) loss_patch_kernel(const __grid_constant__
 }
 
 // ---------------------------------------------------------------------------------------------
-// dz_kernel: one block per row, after a sweep that left the draft logits of few rows in fp32. Merges the draft's partial
-// statistics into lse_d, evaluates Eq. 1 from the logits at Omega_hat, and (make_dz) turns the row into
+// row_kernel: one block per row, after a MODE_LOGITS sweep that left the logits of few rows in fp32 (-inf beyond the
+// vocabulary). Per row: lse of the target and of the draft, Omega_hat from the target's logits (or given), Eq. 1 from the
+// draft's logits at Omega_hat, and (make_dz) the draft's row turned into
 // dz_d(v) = g (S_q p(v) - q(v) [v in Omega_hat]) in bf16, in place: the bf16 row begins where the fp32 row did. Every step
 // reads a piece twice as long as the one it writes, and a piece is written after all threads have read theirs.
-// With the target's logits (COMBINED) it is the combined objective's
-// dz_d(v) = g ((1 + w S_q) p(v) - q(v) - w q(v) [v in Omega_hat]), and the cross-entropy sum_v q(v) (lse_d - z_d(v)).
-// Bound by the latency of one pass over a row of 4 V bytes: DZ_THREADS threads with DZ_LOADS 16-byte loads each in flight.
-constexpr int DZ_THREADS = 1024;
-constexpr int DZ_LOADS = 4;
+// ROW_COMBINED: dz_d(v) = g ((1 + w S_q) p(v) - q(v) - w q(v) [v in Omega_hat]), and the cross-entropy
+// sum_v q(v) (lse_d - z_d(v)). ROW_BIDIR: the draft's K most probable tokens join Omega_hat; the row becomes p(v) alone, and
+// g S_q and the row sum_x g q(x) W[x, :] over Omega_hat are left in fp32 for the epilogue of the second GEMM.
+//
+// The K largest of a row: a thread's largest logit is at hand after the pass for lse, and the K-th largest of these 1024
+// maxima bounds the row's K-th largest from below. Little more than K logits reach it; the threads that hold them read their
+// share again and put them into a pool in shared memory, where each counts those above it.
+// Bound by the latency of two passes over rows of 4 V bytes in L2: ROW_THREADS threads with ROW_LOADS 16-byte loads each in
+// flight.
+constexpr int ROW_THREADS = 1024;
+constexpr int ROW_WARPS = ROW_THREADS / 32;
+constexpr int ROW_LOADS = 4;
+constexpr int ROW_STEP = ROW_LOADS * ROW_THREADS * 4;      // logits per step of a pass
+constexpr int ROW_POOL = 1024;
+constexpr int ROW_SLACK = 32;      // maxima beyond K at which the search of the bound ends
+static_assert(ROW_POOL >= K_CAP && ROW_THREADS >= K_CAP, "room for Omega_hat, a thread for each of its tokens");
+enum { ROW_TOPK = 0, ROW_COMBINED = 1, ROW_BIDIR = 2 };
 
-struct DzParams {
-    Schedule sched;        // schedule of the sweep
-    int first_tile;        // its row tile of the draft rows
-    int first_row;         // of the draft rows in that tile
+struct RowParams {
     int K, V;
-    const float* part_m;
-    const float* part_s;
-    const int* idx;        // [N, K] Omega_hat; entries < 0 carry q = 0
-    const float* q;
+    long long pitch;       // of z and zt, a multiple of 256
+    float* z;              // [N, pitch] in: draft logits; out: bf16 [N, 2 pitch]. nullptr: selection only
+    const float* zt;       // [N, pitch] target logits, or nullptr: Omega_hat is given
+    int* idx;              // [N, idx_pitch] Omega_hat in descending q: out with zt, else in (entries < 0 carry q = 0)
+    float* q;
+    int idx_pitch;
+    float top_p;           // > 0: Omega_hat is cut to the shortest sorted prefix with cumulative q > top_p
+    int* n_out;            // [N] |Omega_hat|, negative where K tokens do not reach top_p (nullable)
     const float* grad_loss;
-    float* loss;
+    float* lse_t;
     float* lse_d;
-    float* z;              // [N, pitch] in: logits (columns up to the pitch readable); out: bf16 [N, 2 pitch]
-    long long pitch;       // a multiple of 256
+    float* loss;
     int make_dz;
-    // COMBINED
-    const float* zt;       // [N, pitch] target logits
-    const float* lse_t;
-    float w;
+    float w;               // ROW_COMBINED
     float* loss_ce;
+    const __nv_bfloat16* W;      // ROW_BIDIR: [V, d]
+    int d;
+    float* coef_out;       // [N] g S_q
+    float* sparse_out;     // [N, d]
 };
 
-template <bool COMBINED>
-__global__ void __launch_bounds__(DZ_THREADS) dz_kernel(const __grid_constant__ DzParams p) {
-    __shared__ float sh_ce[DZ_THREADS / 32];
-    __shared__ int sh_tok[K_CAP];
-    __shared__ float sh_q[K_CAP];
-    __shared__ float sh_z[K_CAP];
-    __shared__ float sh_sum[2];           // lse_d, S_q
+struct RowShared {
+    unsigned long long pool[ROW_POOL];
+    float red[4][ROW_WARPS];
+    uint32_t key_min[ROW_WARPS];
+    int tok[K_CAP];        // Omega_hat
+    float q[K_CAP], z[K_CAP];
+    int tok_d[K_CAP];      // the draft's own K largest (ROW_BIDIR)
+    float z_d[K_CAP];
+    float sum;
+    int n, count;
+};
+
+// One logit as a number: larger = larger logit, lower token id first among equal ones (-0 and +0 are equal).
+__device__ __forceinline__ unsigned long long logit_rank(float z, uint32_t id) {
+    return cand_rank(ordered_key(__float_as_uint(z + 0.f)), id);
+}
+
+// f(first column, its four logits) for every piece of the row that this thread owns
+template <typename F>
+__device__ __forceinline__ void for_own_logits(const float* row, long long pitch, F&& f) {
+    for (long long c0 = threadIdx.x * 4; c0 < pitch; c0 += ROW_STEP) {
+        float4 v[ROW_LOADS];
+#pragma unroll
+        for (int u = 0; u < ROW_LOADS; ++u) {
+            const long long at = c0 + u * (ROW_THREADS * 4);
+            if (at < pitch) v[u] = *reinterpret_cast<const float4*>(row + at);
+        }
+#pragma unroll
+        for (int u = 0; u < ROW_LOADS; ++u) {
+            const long long at = c0 + u * (ROW_THREADS * 4);
+            if (at < pitch) f(at, v[u]);
+        }
+    }
+}
+
+// This thread's largest logit m and sum of 2^((z - m) log2e)
+__device__ __forceinline__ void own_stats(const float* row, long long pitch, float& m, float& s) {
+    m = -INFINITY;
+    s = 0.f;
+    for_own_logits(row, pitch, [&](long long, const float4& v) {
+        const float cm = fmaxf(fmax3(v.x, v.y, v.z), v.w);
+        if (cm > m) {
+            s *= ex2((m - cm) * LOG2E);
+            m = cm;
+        }
+        const float mneg = m == -INFINITY ? 0.f : -m * LOG2E;      // (nothing but -inf so far: each adds zero)
+        s += ex2(fmaf(v.x, LOG2E, mneg)) + ex2(fmaf(v.y, LOG2E, mneg)) + ex2(fmaf(v.z, LOG2E, mneg)) + ex2(fmaf(v.w, LOG2E, mneg));
+    });
+}
+
+// The block's log-sum-exp of the threads' (m, s); `red`: 2 x ROW_WARPS floats. Two barriers.
+__device__ __forceinline__ float block_lse(float m, float s, float (*red)[ROW_WARPS]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float mx = m;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    const float base = mx == -INFINITY ? 0.f : mx;
+    s *= ex2((m - base) * LOG2E);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) {
+        red[0][warp] = mx;
+        red[1][warp] = s;
+    }
+    __syncthreads();
+    m = red[0][lane];
+    s = red[1][lane];
+    mx = m;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    const float top = mx == -INFINITY ? 0.f : mx;
+    s *= ex2(((m == -INFINITY ? top : m) - top) * LOG2E);      // (a warp without a logit: its sum is zero)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return top + logf(s);
+}
+
+// Block-collective: the K largest logits of the row, in descending order (lower token id first among equal ones), into
+// tok / val; m = this thread's largest logit. Fewer than K logits above -inf: the rest is token 0 at -inf.
+__device__ __forceinline__ void select_largest(const float* row, long long pitch, int V, int K, float m, RowShared& sh, int* tok, float* val) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t key = m > -INFINITY ? ordered_key(__float_as_uint(m + 0.f)) : 0u;
+    const uint32_t key_hi = __reduce_max_sync(0xffffffffu, key), key_lo = __reduce_min_sync(0xffffffffu, key == 0u ? 0xffffffffu : key);
+    if (lane == 0) {
+        sh.red[0][warp] = __uint_as_float(key_hi);
+        sh.key_min[warp] = key_lo;
+    }
+    if (tid == 0) sh.n = 0;
+    const int groups = __syncthreads_count(key != 0u);
+    uint32_t T = 1u;
+    if (groups >= K) {
+        // the K-th largest maximum, or a value below it that at most K + ROW_SLACK maxima reach, from the highest bit in which
+        // the maxima differ on
+        const uint32_t hi = __reduce_max_sync(0xffffffffu, __float_as_uint(sh.red[0][lane]));
+        const uint32_t lo = __reduce_min_sync(0xffffffffu, sh.key_min[lane]);
+        int bit = 32 - __clz(hi ^ lo);
+        T = bit < 32 ? hi >> bit << bit : 0u;
+        for (--bit; bit >= 0; --bit) {
+            const uint32_t T1 = T | (1u << bit);
+            const int c = __syncthreads_count(key >= T1);
+            if (c >= K) {
+                T = T1;
+                if (c <= K + ROW_SLACK) break;
+            }
+        }
+        T = max(T, 1u);
+    }
+    auto collect = [&](bool mine, unsigned long long bound) {
+        if (mine)
+            for_own_logits(row, pitch, [&](long long at, const float4& v) {
+                const float z[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const unsigned long long r = logit_rank(z[j], static_cast<uint32_t>(at + j));
+                    if (z[j] > -INFINITY && at + j < V && r >= bound) {
+                        const int pos = atomicAdd(&sh.n, 1);
+                        if (pos < ROW_POOL) sh.pool[pos] = r;
+                    }
+                }
+            });
+        __syncthreads();
+    };
+    collect(key >= T, static_cast<unsigned long long>(T) << 32);
+    if (sh.n > ROW_POOL) {
+        // Many equal logits: the bound is searched over logits and token ids, one bit per pass over the row, until the pool
+        // holds what reaches it.
+        unsigned long long T64 = 0ull;
+        for (int bit = 63; bit >= 0; --bit) {
+            const unsigned long long T1 = T64 | (1ull << bit);
+            __syncthreads();
+            if (tid == 0) sh.count = 0;
+            __syncthreads();
+            int c = 0;
+            for_own_logits(row, pitch, [&](long long at, const float4& v) {
+                const float z[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) c += z[j] > -INFINITY && at + j < V && logit_rank(z[j], static_cast<uint32_t>(at + j)) >= T1 ? 1 : 0;
+            });
+            c = __reduce_add_sync(0xffffffffu, c);
+            if (lane == 0) atomicAdd(&sh.count, c);
+            __syncthreads();
+            if (sh.count >= K) {
+                T64 = T1;
+                if (sh.count <= ROW_POOL) break;
+            }
+        }
+        __syncthreads();
+        if (tid == 0) sh.n = 0;
+        __syncthreads();
+        collect(true, T64);
+    }
+    const int n = sh.n;
+    for (int j = n + tid; j < K; j += ROW_THREADS) {
+        tok[j] = 0;
+        val[j] = -INFINITY;
+    }
+    for (int e = warp; e < n; e += ROW_WARPS) {
+        const unsigned long long v = sh.pool[e];
+        int rank = 0;
+        for (int i = lane; i < n; i += 32) rank += sh.pool[i] > v ? 1 : 0;
+        rank = __reduce_add_sync(0xffffffffu, rank);
+        if (lane == 0 && rank < K) {
+            tok[rank] = static_cast<int>(~static_cast<uint32_t>(v));
+            val[rank] = __uint_as_float(key_bits(static_cast<uint32_t>(v >> 32)));
+        }
+    }
+    __syncthreads();
+}
+
+template <int OBJ>
+__global__ void __launch_bounds__(ROW_THREADS) row_kernel(const __grid_constant__ RowParams p) {
+    __shared__ RowShared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int row = blockIdx.x;
     const int K = p.K;
     wait_previous_kernel();
-    float* zrow = p.z + static_cast<long long>(row) * p.pitch;
-    __nv_bfloat16* drow = reinterpret_cast<__nv_bfloat16*>(zrow);
-    if (tid < K) {
-        const int tok = p.idx[static_cast<long long>(row) * K + tid];
-        sh_tok[tid] = tok < p.V ? tok : -1;
-        sh_q[tid] = p.q[static_cast<long long>(row) * K + tid];
-        sh_z[tid] = tok >= 0 && tok < p.V ? zrow[tok] : 0.f;
-    }
-    if (warp == DZ_THREADS / 32 - 1) {
-        int slot0, S;
-        find_slots(p.sched, p.first_tile, slot0, S);
-        const float lse = warp_lse(p.part_m, p.part_s, slot0, S, p.first_row + row, lane);
-        if (lane == 0) sh_sum[0] = lse;
-    }
+    float* zrow = p.z != nullptr ? p.z + static_cast<long long>(row) * p.pitch : nullptr;
+    const float* trow = p.zt != nullptr ? p.zt + static_cast<long long>(row) * p.pitch : nullptr;
+    int* idx = p.idx + static_cast<long long>(row) * p.idx_pitch;
+    float* q = p.q + static_cast<long long>(row) * p.idx_pitch;
+
+    float m_t = -INFINITY, s_t = 0.f, m_d = -INFINITY, s_d = 0.f, lse_t = 0.f, lse_d = 0.f;
+    if (trow) own_stats(trow, p.pitch, m_t, s_t);
+    if (zrow) own_stats(zrow, p.pitch, m_d, s_d);
+    if (trow) lse_t = block_lse(m_t, s_t, sh.red);
+    if (zrow) lse_d = block_lse(m_d, s_d, sh.red + 2);
     __syncthreads();
-    const float g = p.grad_loss ? p.grad_loss[row] : 1.f;
-    const float lse_d = sh_sum[0];
+
+    int n_tok = K;                        // entries of Omega_hat's list (2K at most for the bi-directional set)
+    if (trow) {
+        select_largest(trow, p.pitch, p.V, K, m_t, sh, sh.tok, sh.q);
+        if (tid < K) sh.q[tid] = expf(sh.q[tid] - lse_t);
+        __syncthreads();
+        int taken = K;
+        if (p.top_p > 0.f) {
+            // Top-P: a token belongs to Omega_hat while the probability of those before it is <= P
+            if (tid == 0) {
+                taken = 0;
+                float cum = 0.f;
+                for (int j = 0; j < K; ++j) {
+                    if (cum > p.top_p) {
+                        sh.tok[j] = -1;
+                        sh.q[j] = 0.f;
+                    } else {
+                        ++taken;
+                    }
+                    cum += sh.q[j];
+                }
+                if (!(cum > p.top_p)) taken = -taken;      // all K tokens taken and P still not exceeded: the cap cut the prefix
+            }
+            __syncthreads();
+        }
+        if (OBJ == ROW_BIDIR) {
+            // the draft's own K most probable tokens that are not in the target's set join Omega_hat, in their order
+            select_largest(zrow, p.pitch, p.V, K, m_d, sh, sh.tok_d, sh.z_d);
+            if (warp == 0) {
+                int n = K;
+                for (int j0 = 0; j0 < K; j0 += 32) {
+                    const int j = j0 + lane;
+                    const int t = j < K ? sh.tok_d[j] : -1;
+                    bool joins = j < K;
+                    for (int i = 0; i < K; ++i) joins = joins && sh.tok[i] != t;
+                    const uint32_t bm = __ballot_sync(0xffffffffu, joins);
+                    const int at = n + __popc(bm & ((1u << lane) - 1u));
+                    if (joins) {
+                        sh.tok[at] = t;
+                        sh.q[at] = expf(trow[t] - lse_t);
+                    }
+                    n += __popc(bm);
+                }
+                for (int j = n + lane; j < 2 * K; j += 32) {
+                    sh.tok[j] = -1;
+                    sh.q[j] = 0.f;
+                }
+                if (lane == 0) sh.count = n;
+            }
+            __syncthreads();
+            taken = sh.count;
+            n_tok = 2 * K;
+        }
+        if (tid < n_tok) {
+            idx[tid] = sh.tok[tid];
+            q[tid] = sh.q[tid];
+        }
+        if (tid == 0) {
+            p.lse_t[row] = lse_t;
+            if (p.n_out) p.n_out[row] = taken;
+        }
+    } else {
+        if (tid < K) {
+            const int t = idx[tid];
+            sh.tok[tid] = t < p.V ? t : -1;
+            sh.q[tid] = q[tid];
+        }
+    }
+    if (!zrow) return;
+    if (tid < n_tok) sh.z[tid] = sh.tok[tid] >= 0 ? zrow[sh.tok[tid]] : 0.f;      // (each entry by the thread that wrote it, or behind a barrier)
+    __syncthreads();
     if (warp == 0) {
         float S_q = 0.f, loss = 0.f;
-        for (int j = lane; j < K; j += 32) {
-            if (sh_tok[j] < 0) continue;
-            S_q += sh_q[j];
-            loss += sh_q[j] * (lse_d - sh_z[j]);      // -q log p,  log p = z_d - lse_d
+        for (int j = lane; j < n_tok; j += 32) {
+            if (sh.tok[j] < 0) continue;
+            S_q += sh.q[j];
+            loss += sh.q[j] * (lse_d - sh.z[j]);      // -q log p,  log p = z_d - lse_d
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -2013,70 +2264,89 @@ __global__ void __launch_bounds__(DZ_THREADS) dz_kernel(const __grid_constant__ 
             loss += __shfl_xor_sync(0xffffffffu, loss, o);
         }
         if (lane == 0) {
-            sh_sum[1] = S_q;
+            sh.sum = S_q;
             p.loss[row] = loss;
             p.lse_d[row] = lse_d;
         }
     }
     __syncthreads();
     if (!p.make_dz) return;
-    const float S_q = sh_sum[1], c = COMBINED ? g * (1.f + p.w * S_q) : g * S_q, shift = -lse_d * LOG2E;
-    const float* trow = COMBINED ? p.zt + static_cast<long long>(row) * p.pitch : nullptr;
-    const float shift_t = COMBINED ? -p.lse_t[row] * LOG2E : 0.f;
+    __nv_bfloat16* drow = reinterpret_cast<__nv_bfloat16*>(zrow);
+    const float g = p.grad_loss ? p.grad_loss[row] : 1.f;
+    const float S_q = sh.sum, c = OBJ == ROW_COMBINED ? g * (1.f + p.w * S_q) : OBJ == ROW_BIDIR ? 1.f : g * S_q, shift = -lse_d * LOG2E, shift_t = -lse_t * LOG2E;
     float ce = 0.f;
-    for (long long c0 = 0; c0 < p.pitch; c0 += DZ_LOADS * DZ_THREADS * 4) {
-        float4 v[DZ_LOADS];
+    for (long long c0 = 0; c0 < p.pitch; c0 += ROW_STEP) {
+        float4 v[ROW_LOADS];
 #pragma unroll
-        for (int u = 0; u < DZ_LOADS; ++u) {
-            const long long at = c0 + (u * DZ_THREADS + tid) * 4;
+        for (int u = 0; u < ROW_LOADS; ++u) {
+            const long long at = c0 + (u * ROW_THREADS + tid) * 4;
             if (at < p.pitch) v[u] = *reinterpret_cast<const float4*>(zrow + at);
         }
-        float4 t[COMBINED ? DZ_LOADS : 1];
-        if (COMBINED) {
+        float4 t[OBJ == ROW_COMBINED ? ROW_LOADS : 1];
+        if (OBJ == ROW_COMBINED) {
 #pragma unroll
-            for (int u = 0; u < DZ_LOADS; ++u) {
-                const long long at = c0 + (u * DZ_THREADS + tid) * 4;
-                if (at < p.pitch) t[COMBINED ? u : 0] = *reinterpret_cast<const float4*>(trow + at);
+            for (int u = 0; u < ROW_LOADS; ++u) {
+                const long long at = c0 + (u * ROW_THREADS + tid) * 4;
+                if (at < p.pitch) t[OBJ == ROW_COMBINED ? u : 0] = *reinterpret_cast<const float4*>(trow + at);
             }
         }
         __syncthreads();
 #pragma unroll
-        for (int u = 0; u < DZ_LOADS; ++u) {
-            const long long at = c0 + (u * DZ_THREADS + tid) * 4;
+        for (int u = 0; u < ROW_LOADS; ++u) {
+            const long long at = c0 + (u * ROW_THREADS + tid) * 4;
             if (at < p.pitch) {
                 float z[4] = {v[u].x, v[u].y, v[u].z, v[u].w}, o[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) o[j] = c * ex2(fmaf(z[j], LOG2E, shift));
-                if (COMBINED) {
-                    const float4& tu = t[COMBINED ? u : 0];
+                if (OBJ == ROW_COMBINED) {
+                    const float4& tu = t[OBJ == ROW_COMBINED ? u : 0];
                     const float zt[4] = {tu.x, tu.y, tu.z, tu.w};
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const float q = ex2(fmaf(zt[j], LOG2E, shift_t));
-                        o[j] = fmaf(-g, q, o[j]);
-                        if (at + j < p.V) ce = fmaf(q, lse_d - z[j], ce);      // (-inf beyond the vocabulary)
+                        const float qv = ex2(fmaf(zt[j], LOG2E, shift_t));
+                        o[j] = fmaf(-g, qv, o[j]);
+                        if (at + j < p.V) ce = fmaf(qv, lse_d - z[j], ce);      // (-inf beyond the vocabulary)
                     }
                 }
                 *reinterpret_cast<uint2*>(drow + at) = make_uint2(pack_bf16x2(o[0], o[1]), pack_bf16x2(o[2], o[3]));
             }
         }
     }
-    if (COMBINED) {
+    if (OBJ == ROW_COMBINED) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) ce += __shfl_xor_sync(0xffffffffu, ce, o);
-        if (lane == 0) sh_ce[warp] = ce;
+        if (lane == 0) sh.red[0][warp] = ce;
+    }
+    if (OBJ == ROW_BIDIR) {
+        if (tid == 0) p.coef_out[row] = g * S_q;
+        const int n = sh.count;
+        for (int k0 = tid * 8; k0 < p.d; k0 += ROW_THREADS * 8) {
+            float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+            for (int j = 0; j < n; ++j) {
+                const float gq = g * sh.q[j];
+                float wf[8];
+                unpack8(*reinterpret_cast<const uint4*>(p.W + static_cast<long long>(sh.tok[j]) * p.d + k0), wf);
+#pragma unroll
+                for (int t = 0; t < 8; ++t) a[t] = fmaf(gq, wf[t], a[t]);
+            }
+            float* so = p.sparse_out + static_cast<long long>(row) * p.d + k0;
+            *reinterpret_cast<float4*>(so) = make_float4(a[0], a[1], a[2], a[3]);
+            *reinterpret_cast<float4*>(so + 4) = make_float4(a[4], a[5], a[6], a[7]);
+        }
+        return;
     }
     __syncthreads();
-    if (tid < K && sh_tok[tid] >= 0) {
-        float o = c * ex2(fmaf(sh_z[tid], LOG2E, shift));
-        if (COMBINED)
-            o -= g * ex2(fmaf(trow[sh_tok[tid]], LOG2E, shift_t)) + g * p.w * sh_q[tid];
+    if (tid < n_tok && sh.tok[tid] >= 0) {
+        float o = c * ex2(fmaf(sh.z[tid], LOG2E, shift));
+        if (OBJ == ROW_COMBINED)
+            o -= g * ex2(fmaf(trow[sh.tok[tid]], LOG2E, shift_t)) + g * p.w * sh.q[tid];
         else
-            o -= g * sh_q[tid];
-        drow[sh_tok[tid]] = __float2bfloat16_rn(o);
+            o -= g * sh.q[tid];
+        drow[sh.tok[tid]] = __float2bfloat16_rn(o);
     }
-    if (COMBINED && warp == 0) {
-        float v = sh_ce[lane];
+    if (OBJ == ROW_COMBINED && warp == 0) {
+        float v = sh.red[0][lane];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if (lane == 0) p.loss_ce[row] = v;
