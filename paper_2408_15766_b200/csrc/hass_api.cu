@@ -401,7 +401,7 @@ static int make_layout(long long N, long long d, long long V, int K, int sms, La
     off += 256;
     const size_t slots = static_cast<size_t>(slot_cap);
     L->thr_share = off;                     // admission thresholds the lanes of a row tile publish to each other; behind the
-    off = align256(off + slots * BM * 4);   // status block, so that one memset clears both
+    off = align256(off + slots * BM * 8);   // status block, so that one memset clears both
     L->part_m = off;
     off = align256(off + slots * BM * 4);
     L->part_s = off;
@@ -499,7 +499,7 @@ static int clear_bytes(void* at, size_t bytes, cudaStream_t st) {
 static int clear_status(uint8_t* ws, const Layout& L, int slots, cudaStream_t st, bool only_thresholds = false) {
     const size_t from = only_thresholds ? L.thr_share : L.status;
     if (only_thresholds && slots == 0) return HASS_OK;
-    return clear_bytes(ws + from, L.thr_share + static_cast<size_t>(slots) * BM * 4 - from, st);
+    return clear_bytes(ws + from, L.thr_share + static_cast<size_t>(slots) * BM * 8 - from, st);
 }
 
 template <int WARPS, int WIN>
@@ -649,7 +649,7 @@ static int forward_impl(bool with_target, const void* H_t, const void* H_d, cons
     p.cand = reinterpret_cast<uint2*>(ws + L.cand_v);
     p.cand_n = reinterpret_cast<int*>(ws + L.cand_i);
     p.status = reinterpret_cast<unsigned int*>(ws + L.status);
-    p.thr_share = reinterpret_cast<unsigned int*>(ws + L.thr_share);
+    p.thr_share = reinterpret_cast<uint2*>(ws + L.thr_share);
     rc = clear_status(ws, L, p.sched.total_slots, st);
     if (rc != HASS_OK) return rc;
     rc = launch_gemm<MODE_STATS>(p, st);
@@ -1029,7 +1029,7 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
         p.Pt = cmb ? cmb->Pt : nullptr;
         p.p_pitch = L.p_pitch;
         p.status = status;
-        p.thr_share = reinterpret_cast<unsigned int*>(ws + L.thr_share);
+        p.thr_share = reinterpret_cast<uint2*>(ws + L.thr_share);
         p.row_zmax = zmax + static_cast<size_t>(with_target ? 2 : 1) * t0 * BM;
         p.use_row_zmax = retry ? 1 : 0;
         p.gate = gate;
@@ -1301,7 +1301,7 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
             p.part_s = reinterpret_cast<float*>(ws + L.part_s);
             p.cand = reinterpret_cast<uint2*>(ws + L.cand_v);
             p.cand_n = reinterpret_cast<int*>(ws + L.cand_i);
-            p.thr_share = reinterpret_cast<unsigned int*>(ws + L.thr_share);
+            p.thr_share = reinterpret_cast<uint2*>(ws + L.thr_share);
             p.p_pitch = L.p_pitch;
             p.status = status;
             p.gate = gate;
@@ -1480,7 +1480,7 @@ static int forward2_impl(bool with_target, const void* H_t, const void* H_d, con
     int* sidx = reinterpret_cast<int*>(ws + L.sidx);
     float* sq = reinterpret_cast<float*>(ws + L.sgq);
     float* capz = reinterpret_cast<float*>(ws + L.capz);
-    p.thr_share = reinterpret_cast<unsigned int*>(ws + L.thr_share);
+    p.thr_share = reinterpret_cast<uint2*>(ws + L.thr_share);
     rc = clear_status(ws, L, with_target ? p.sched.total_slots : 0, st);
     if (rc != HASS_OK) return rc;
     if (with_target) {
@@ -1589,7 +1589,7 @@ static int normed_impl(const void* H_t, const void* H_d, const void* W, long lon
         p.cand = reinterpret_cast<uint2*>(ws + L.cand_v);
         p.cand_n = reinterpret_cast<int*>(ws + L.cand_i);
         p.status = reinterpret_cast<unsigned int*>(ws + L.status);
-        p.thr_share = reinterpret_cast<unsigned int*>(ws + L.thr_share);
+        p.thr_share = reinterpret_cast<uint2*>(ws + L.thr_share);
         rc = clear_status(ws, L, p.sched.total_slots, st);
         if (rc != HASS_OK) return rc;
         rc = launch_gemm<MODE_STATS>(p, st);

@@ -113,8 +113,8 @@ struct GemmParams {
     float* part_s;
     uint2* cand;           // [slot, row, cap] (logit bits, token id)
     int* cand_n;           // [slot, row] entries in use
-    unsigned int* thr_share;   // [slot, row] ordered key of each lane's current threshold, read by the other lanes of its row
-                           // tile (zeroed before the sweep: nothing published)
+    uint2* thr_share;      // [slot, row] what a lane publishes to the others of its row tile, as ordered keys (zeroed before the
+                           // sweep: nothing yet): x = a bound that K of its logits reach, y = one that lane_share(K, S) of them reach
     // MODE_PROBS
     const float* lse2;     // [N] lse_d * log2(e)
     const float* coef;     // [N] g * S_q
@@ -346,9 +346,13 @@ __device__ __forceinline__ void sort16_descending(float (&v)[16]) {
             }
 }
 
+// Where S lanes share a row and each has this many logits above a bound, K of the row's logits lie above it.
+__host__ __device__ constexpr int lane_share(int K, int S) { return (K + S - 1) / S; }
+
 // Histogram of a thread's row in shared memory: bucket b of thread T at word b * 128 + T of `hist` (the thread's own
 // column, no conflicts, no synchronisation). The bucket of x is a non-decreasing function of x.
-constexpr int HIST_BUCKETS = 32;
+constexpr int HIST_BUCKETS = 64;
+static_assert(HIST_BUCKETS * 128 * 4 <= 4 * SPILL_STAGES * SPILL_STAGE_BYTES, "the histograms take the room of the spill's staging buffers");
 __device__ __forceinline__ int hist_bucket(float x, float lo, float inv) {
     return min(max(__float2int_rz((x - lo) * inv), 0), HIST_BUCKETS - 1);
 }
@@ -356,16 +360,20 @@ __device__ __forceinline__ void hist_clear(uint32_t hist) {
 #pragma unroll
     for (int b = 0; b < HIST_BUCKETS; ++b) st_shared_b32(hist + b * 512, 0u);
 }
-// the highest bucket that together with those above it holds at least K entries; 0 if there is none
-__device__ __forceinline__ int hist_top(uint32_t hist, int K) {
-    int acc = 0, top = 0;
+__device__ __forceinline__ void hist_count(uint32_t hist, float x, float lo, float inv) {
+    const uint32_t at = hist + hist_bucket(x, lo, inv) * 512;
+    st_shared_b32(at, ld_shared_b32(at) + 1u);
+}
+// the highest buckets that together with those above them hold at least K and k <= K entries; 0 if there are none
+__device__ __forceinline__ void hist_top(uint32_t hist, int K, int k, int& top_K, int& top_k) {
+    int acc = 0;
+    top_K = top_k = 0;
 #pragma unroll
     for (int b = HIST_BUCKETS - 1; b > 0; --b) {
-        const int before = acc;
         acc += static_cast<int>(ld_shared_b32(hist + b * 512));
-        if (before < K && acc >= K) top = b;
+        if (top_k == 0 && acc >= k) top_k = b;
+        if (top_K == 0 && acc >= K) top_K = b;
     }
-    return top;
 }
 
 // TOPK selects how MODE_STATS keeps a row's Top-K candidates: TOPK_REG (K <= K_REG) a sorted list in
@@ -645,7 +653,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
             // ---- per-item state ----
             float m = -INFINITY, s = 0.f, thr = -INFINITY;        // MODE_STATS; thr = admission threshold in force
             float thr_own = -INFINITY;                            // K-th (K_REG-th) largest logit of this lane's own list
-            float thr_sh = -INFINITY;                             // just below the best threshold published by the other lanes
+            float thr_sh = -INFINITY;                             // just below the best bound that what the lanes published gives
+            // TOPK_BUF: the histogram of this lane's logits between hist_lo and the first tile's largest (a quarter of its range
+            // higher); a logit at or below the threshold of its time is missing. hist_inv = 0: none
+            float hist_lo = 0.f, hist_inv = 0.f;
+            int counted = 0;                                      // entries of the buffer that are in it
+            const int share = HAS_TOPK && !USE_REG ? lane_share(p.K, S) : 0;
             bool want_topk = false;
             const bool spill = MODE == MODE_STATS && tile_ok && spills(p, rt);
             const bool track_zmax = MODE == MODE_STATS && spill && p.row_zmax != nullptr;
@@ -737,8 +750,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                 }
                 if (MODE == MODE_STATS && HAS_TOPK && !USE_REG && want_topk && t == 0 && p.n_cols - col_base >= BN) {
                     // First tile of the sweep, buffer empty, no threshold yet: admitting all 256 logits would fill the buffer
-                    // at once. Each thread takes a histogram of its row's 256 logits between the least and the largest and
-                    // starts from half a bucket below the bucket above which at least K of them lie: a valid lower bound of
+                    // at once. Each thread takes a histogram of its row's 256 logits between the least and a little above the
+                    // largest and starts from half a bucket below the bucket above which at least K of them lie: a valid lower bound of
                     // the row's K-th largest logit that admits little more than K of the tile's.
                     float lo = INFINITY, hi = -INFINITY;
 #pragma unroll 1
@@ -752,7 +765,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                             hi = fmaxf(hi, __uint_as_float(r[j]));
                         }
                     }
-                    const float inv = HIST_BUCKETS / (hi - lo);
+                    hist_lo = lo;
+                    hist_inv = HIST_BUCKETS / (1.25f * (hi - lo));
                     hist_clear(pend_v);
 #pragma unroll 1
                     for (int ch = 0; ch < BN / 32; ++ch) {
@@ -760,16 +774,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                         tmem_ld32(t_row + ch * 32, r);
                         tmem_ld_wait(r);
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            const uint32_t at = pend_v + hist_bucket(__uint_as_float(r[j]), lo, inv) * 512;
-                            st_shared_b32(at, ld_shared_b32(at) + 1u);
-                        }
+                        for (int j = 0; j < 32; ++j) hist_count(pend_v, __uint_as_float(r[j]), lo, hist_inv);
                     }
-                    const int top = hist_top(pend_v, p.K);
-                    const float bound = lo + (static_cast<float>(top) - 0.5f) / inv;
                     // (half a bucket must exceed the rounding of these few operations; also false for infinities and NaN)
-                    if (top > 0 && 0.5f / inv > 1e-6f * fmaxf(fabsf(lo), fabsf(hi))) {
-                        thr_own = fmaxf(thr_own, bound);
+                    if (!(0.5f / hist_inv > 1e-6f * fmaxf(fabsf(lo), fabsf(hi)))) hist_inv = 0.f;
+                    int top, top_share;
+                    hist_top(pend_v, p.K, share, top, top_share);
+                    if (top > 0 && hist_inv > 0.f) {
+                        thr_own = fmaxf(thr_own, lo + (static_cast<float>(top) - 0.5f) / hist_inv);
                         thr = fmaxf(thr_own, thr_sh);
                     }
                 }
@@ -820,6 +832,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                             else
                                 compact_rows<CAND_REGS>(full, cbuf, cnt, thr_own, p.K, p.cap, lane);
                             thr = fmaxf(thr_own, thr_sh);
+                            counted = min(counted, cnt);      // (entries that were dropped before they were counted stay uncounted)
                         }
                     }
                     uint32_t r[32];
@@ -1105,20 +1118,54 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                 }
                 ab ^= 1;
                 if (ab == 0) aphase ^= 1u;
-                if (MODE == MODE_STATS && want_topk && S > 1) {
-                    // The K-th largest logit of ANY lane's part of the row is a lower bound of the row's K-th
-                    // largest, so a lane may adopt the other lanes' thresholds: publish ours, read up to three
-                    // neighbours. A logit equal to a foreign threshold must still be admitted (ties are settled
-                    // by token id when the lists are merged), hence the step just below it. Stale or missing
-                    // (zero) values only leave the threshold lower than it could be.
-                    volatile unsigned int* sh = p.thr_share + static_cast<long long>(slot - ln) * BM + r_local;
-                    sh[static_cast<long long>(ln) * BM] = ordered_key(__float_as_uint(thr_own));      // (the first tile's bound is in thr_sh)
-                    const int nn = S - 1 < 3 ? S - 1 : 3;
-                    for (int q = 1; q <= nn; ++q) {
-                        const unsigned int v = sh[static_cast<long long>((ln + q) % S) * BM];
-                        if (v != 0u) thr_sh = fmaxf(thr_sh, nextafterf(__uint_as_float(key_bits(v)), -INFINITY));
+                if (MODE == MODE_STATS && want_topk && (S > 1 || !USE_REG)) {
+                    // Bounds of the row's K-th largest logit, from what this lane and the others have met so far: the K-th
+                    // largest of ANY lane's part of the row, and (TOPK_BUF) the least of ALL lanes' share-th largest, share =
+                    // ceil(K / S): S lanes with so many logits above a bound are K logits. The second is the tighter one: after the
+                    // first tile it leaves about K / S of a tile's logits to a lane instead of K, the buffers hardly fill any more and the
+                    // warp compacts next to nothing. 2047 rows x 4096 x 32000, sweep with K = 100 and nine lanes 497 -> 395 us, call 1815 -> 1705;
+                    // 4096 rows, K = 64, four lanes: call 2670 -> 2510. (The register lists of K <= 16 admit too little for it to show.)
+                    // A logit equal to a foreign bound must still be admitted (ties are settled by token id when the lists
+                    // are merged), hence the step just below it. Stale or missing (zero) values only leave the threshold
+                    // lower than it could be.
+                    float part = thr_own;
+                    if (!USE_REG && hist_inv > 0.f && t >= 0) {
+                        // the first tile's logits are all in the histogram; of a later one's, those admitted follow here
+                        if (t == 0) counted = cnt;
+                        while (counted < cnt) {
+                            uint2 e[8];
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                if (counted + i < cnt) e[i] = __ldcg(cbuf + counted + i);
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                if (counted + i < cnt) hist_count(pend_v, __uint_as_float(e[i].x), hist_lo, hist_inv);
+                            counted += 8;
+                        }
+                        counted = cnt;
+                        int top, top_share;
+                        hist_top(pend_v, p.K, share, top, top_share);
+                        if (top > 0) thr_own = fmaxf(thr_own, hist_lo + (static_cast<float>(top) - 0.5f) / hist_inv);
+                        if (top_share > 0) part = hist_lo + (static_cast<float>(top_share) - 0.5f) / hist_inv;
+                        part = fmaxf(part, thr_own);
                     }
-                    thr = fmaxf(thr, thr_sh);
+                    if (S > 1) {
+                        volatile unsigned int* sh = reinterpret_cast<volatile unsigned int*>(p.thr_share + static_cast<long long>(slot - ln) * BM + r_local);
+                        sh[static_cast<long long>(ln) * (2 * BM)] = ordered_key(__float_as_uint(thr_own));      // (the first tile's bound is in thr_sh)
+                        unsigned int best = 0u;
+                        const int nn = S - 1 < 3 ? S - 1 : 3;
+                        for (int q = 1; q <= nn; ++q) best = max(best, sh[static_cast<long long>((ln + q) % S) * (2 * BM)]);
+                        if (!USE_REG) {
+                            unsigned int least = ordered_key(__float_as_uint(part));
+                            sh[static_cast<long long>(ln) * (2 * BM) + 1] = least;
+#pragma unroll 8
+                            for (int q = 0; q < S; ++q)
+                                if (q != ln) least = min(least, sh[static_cast<long long>(q) * (2 * BM) + 1]);
+                            best = max(best, least);
+                        }
+                        if (best != 0u) thr_sh = fmaxf(thr_sh, nextafterf(__uint_as_float(key_bits(best)), -INFINITY));
+                    }
+                    thr = fmaxf(thr_own, fmaxf(thr, thr_sh));
                 }
             }
             if (MODE == MODE_STATS && tile_ok) {
@@ -1544,7 +1591,7 @@ struct SelectParams {
     const float* part_s;
     const uint2* cand;
     const int* cand_n;
-    const unsigned int* thr_share;    // [slot, row] key of the K-th largest logit of a lane's buffer at its last compaction, or 0
+    const uint2* thr_share;    // as the sweep left it (GemmParams)
     const int* idx_in;     // [N, K]
     const float* q_in;
     int* idx_out;          // [N, K] (from_sweep)
@@ -1678,7 +1725,7 @@ __global__ void __launch_bounds__(sel_block_warps(WARPS) * 32) select_kernel(con
         // lse_t, and a floor below which no candidate can be among the K best: the best K-th largest logit of any list,
         // or the K-th largest of the lists' first entries
         float m = -INFINITY, sum = 0.f;
-        uint32_t floor_key = 0u;
+        uint32_t floor_key = 0u, least_key = 0xffffffffu;
         uint32_t first[SEL_FIRST];
 #pragma unroll
         for (int q = 0; q < SEL_FIRST; ++q) first[q] = 0u;
@@ -1695,7 +1742,11 @@ __global__ void __launch_bounds__(sel_block_warps(WARPS) * 32) select_kernel(con
         for (int j = lane; j < S; j += 32) {
             const long long so = static_cast<long long>(slot0 + j) * BM + r;
             const float pm = p.part_m[so], ps = p.part_s[so];
-            if (!lists) floor_key = max(floor_key, p.thr_share[so]);
+            if (!lists) {
+                const uint2 bounds = p.thr_share[so];
+                floor_key = max(floor_key, bounds.x);
+                least_key = min(least_key, bounds.y);
+            }
             if (pm > m) {
                 sum *= exp2f((m - pm) * LOG2E);
                 m = pm;
@@ -1709,6 +1760,7 @@ __global__ void __launch_bounds__(sel_block_warps(WARPS) * 32) select_kernel(con
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
         floor_key = __reduce_max_sync(0xffffffffu, floor_key);
+        if (!lists) floor_key = max(floor_key, __reduce_min_sync(0xffffffffu, least_key));
         if (lists && S >= K) {
             uint32_t T = 0u;
 #pragma unroll 1

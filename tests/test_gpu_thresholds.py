@@ -1,0 +1,42 @@
+"""Top-K sets of more than 16 tokens: what the lanes of a row tile tell one another about the row, on vocabularies whose large
+logits are spread evenly, lie in one lane's column tiles, come late, come early, or are all alike."""
+import pytest
+import torch
+
+import hass_inputs as hi
+from parity import compare
+
+pytestmark = pytest.mark.gpu
+
+
+# three row tiles over 24 column tiles, two chunks' worth of lanes with one tile each, a ragged last tile, every row tile its own lane
+@pytest.mark.parametrize("N,V", [(300, 6000), (300, 12800), (2100, 1500)])
+@pytest.mark.parametrize("K", [17, 100, 256])
+@pytest.mark.parametrize("layout", ["even", "one tile", "rising", "falling", "alike"])
+def test_sets_of_large_k(N, V, K, layout):
+    import paper_2408_15766_b200 as hass
+    d = 64
+    inp = hi.make_custom(N, d, V, K, seed=V + K, sigma_w=0.3)
+    H_t, W = inp.H_t.clone(), inp.W.clone()
+    H_t[:, 0] = 4.0
+    at = torch.arange(V, dtype=torch.float32) / V
+    if layout == "one tile":
+        W[256:512, 0] = 2.0
+    elif layout == "rising":
+        W[:, 0] = (2.0 * at).to(torch.bfloat16)
+    elif layout == "falling":
+        W[:, 0] = (-2.0 * at).to(torch.bfloat16)
+    elif layout == "alike":
+        H_t[:, 1:] = 0.0
+        W[:, 0] = (torch.arange(V) % 3).to(torch.bfloat16)      # three values: a third of the vocabulary ties at the top
+    dev = torch.device("cuda:0")
+    out = hass.topk_distill_fwd(H_t.to(dev), inp.H_d[0].to(dev), W.to(dev), K)
+    hass.check(out["workspace"])
+    cpu = {k: v.cpu() for k, v in out.items() if k != "workspace"}
+    if layout == "alike":
+        assert torch.equal(cpu["topk_idx"].long(), (2 + 3 * torch.arange(K)).expand(N, K))
+    else:
+        want = (H_t.double() @ W.double().T).topk(K, dim=1).values
+        z = (H_t.double() @ W.double().T).gather(1, cpu["topk_idx"].long())
+        assert (z - want).abs().max() <= 1e-4      # fp32 sums of 64 products of up to 8 in another order: 64 x 2^-24 x 16
+        print(compare(H_t, inp.H_d[0], W, K, cpu, check_dH=False, rows=range(0, N, 37)))
