@@ -131,6 +131,8 @@ struct GemmParams {
     float* z_out;
     float* zt_out;
     long long z_pitch;
+    int keep_from;         // k block from which on this sweep asks the L2 to keep its tiles of B ...
+    int kept;              // MODE_OUT: ... whose second reading this is
     int clear_status;      // the first CTA zeroes the status block (no kernel of the call has run before this one)
     // MODE_OUT. With sparse != nullptr the epilogue computes coef[row] * acc - sparse[local row, :] (row scale
     // and the Omega_hat term of dz_d W, precomputed by finalize); with coef alone coef[row] * acc; with neither
@@ -520,6 +522,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
         if (lane == 0) {
             int stage = 0;
             uint32_t phase = 0;
+            const uint64_t keep = l2_evict_last(), drop = l2_evict_first();
             for_each_item([&](int rt, int ln, int S, int, int kb0, int kb1) {
                 const bool second = (MODE == MODE_STATS || MODE == MODE_LOGITS) && rt >= p.row_tiles0;
                 const CUtensorMap* tmA = second ? &p.tmA1 : &p.tmA0;
@@ -539,6 +542,17 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                             else
                                 tma_load_2d(dst, tm, bar, x, y);
                         };
+                        auto load_b = [&](uint32_t dst, int x, int y) {
+                            if (MODE == MODE_LOGITS || (MODE == MODE_OUT && p.kept)) {
+                                const uint64_t policy = MODE == MODE_LOGITS && kb >= p.keep_from ? keep : drop;
+                                if (CG == 2)
+                                    tma_load_2d_pair_hint(dst, &p.tmB, bar, x, y, policy);
+                                else
+                                    tma_load_2d_hint(dst, &p.tmB, bar, x, y, policy);
+                            } else {
+                                load(dst, &p.tmB, x, y);
+                            }
+                        };
                         const int col0 = ct * BN + static_cast<int>(rank) * (BN / CG);
                         if (MODE == MODE_LOGITS && CG == 1 && p.half_tiles) {
                             load(smemA + stage * A_STAGE_BYTES, &p.tmA0, kb * BK, 0);
@@ -547,13 +561,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                             load(smemA + stage * A_STAGE_BYTES, tmA, kb * BK, row0);
                         }
                         if (!B_MN_MAJOR) {
-                            load(smemB + stage * B_STAGE_BYTES, &p.tmB, kb * BK, col0);
+                            load_b(smemB + stage * B_STAGE_BYTES, kb * BK, col0);
                         } else {
                             // B tile = BK contraction rows x BN / CG contiguous columns, fetched as boxes
                             // of 64 columns (one 128-byte swizzle row) x BK rows
 #pragma unroll
                             for (int j = 0; j < BN / CG / 64; ++j)
-                                load(smemB + stage * B_STAGE_BYTES + j * (BK * 128), &p.tmB, col0 + j * 64, kb * BK);
+                                load_b(smemB + stage * B_STAGE_BYTES + j * (BK * 128), col0 + j * 64, kb * BK);
                         }
                         if (++stage == STAGES) {
                             stage = 0;
