@@ -5,6 +5,7 @@
 // key/value head, so every 128-key tile is fetched once and used by both:
 //   - grouped heads with an even group size: two query heads of one group, same query tile;
 //   - otherwise: two consecutive query tiles of one head (the lower one stops one key tile earlier).
+// Where every item can have a CTA of its own, one slot of a CTA stays empty: the items of a pair wait for one another's turns.
 // Each item owns a "slot": its Q tile in shared memory, a 128-column score buffer and a 128-column output
 // accumulator in tensor memory, and four softmax warps. Per key tile and slot:
 //   S = Q K_t^T            tcgen05.mma, 128 x 128 x 128, fp32 in TMEM
@@ -82,6 +83,7 @@ struct Params {
     int q_tiles;                   // ceil(T / 128)
     int pairs;                     // work units
     int head_pairing;              // 1: a pair = heads 2u, 2u + 1 at one query tile; 0: one head, query tiles qt - 1, qt
+    int single;                    // 1 (head_pairing = 0): a "pair" is one item, in slot 1
     float c2;                      // scale * log2(e)
     int one_round;                 // every CTA takes one pair: no counter, and the status block is cleared here
     unsigned int* status;
@@ -110,9 +112,9 @@ __device__ __forceinline__ Pair decode_pair(const Params& p, int idx) {
         const int u = idx / per, rem = idx - u * per;
         r.b = rem / p.H;
         r.h[0] = r.h[1] = rem - r.b * p.H;
-        r.qt[1] = p.q_tiles - 1 - 2 * u;
+        r.qt[1] = p.q_tiles - 1 - (p.single ? u : 2 * u);
         r.qt[0] = r.qt[1] - 1;
-        r.act0 = r.qt[0] >= 0;
+        r.act0 = !p.single && r.qt[0] >= 0;
     }
     r.kv_col = (r.h[1] / rep) * HD;
     return r;
