@@ -120,7 +120,8 @@ static int device_info(DeviceInfo* out) {
             if (e3 == cudaSuccess) e3 = cudaFuncSetAttribute(select_kernel<16, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * 512 * 8);
             if (e3 == cudaSuccess) e3 = cudaFuncSetAttribute(select_kernel<16, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * 1024 * 8);
             cudaError_t e4 = cudaFuncSetAttribute(hca2::hca_attention_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hca2::SMEM_BYTES);
-            if (e4 == cudaSuccess) e4 = cudaFuncSetAttribute(hca_bwd::hca_bwd_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hca_bwd::F_SMEM_BYTES);
+            if (e4 == cudaSuccess) e4 = cudaFuncSetAttribute(hca_bwd::hca_bwd_fused_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, hca_bwd::F_SMEM_BYTES);
+            if (e4 == cudaSuccess) e4 = cudaFuncSetAttribute(hca_bwd::hca_bwd_fused_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, hca_bwd::F_SMEM_BYTES);
             for (int c = 2; c <= MAX_CLUSTER; ++c) {
                 cudaLaunchConfig_t cfg = {};
                 cfg.gridDim = dim3(c);
@@ -2146,9 +2147,11 @@ int hass_hca_attention_fwd(const void* Q, const void* K_t, const void* V_t, cons
     }
 }
 
-// workspace of the HCA backward: status word, D [B, H, T], and the fp32 dQ accumulator [B, T, H, 128]
+// workspace of the HCA backward: status word, D [B, H, T], the fp32 dQ accumulator [B, T, H, 128], and where
+// key tiles may be split the fp32 dV and dK (not needed: a workspace that ends before them is used without splitting)
+constexpr int64_t kSplitTiles = 2 * 148;      // key tiles up to which splitting them is considered
 struct HcaBwdLayout {
-    size_t D, dQacc, total;
+    size_t D, dQacc, total, dKVacc;
 };
 static HcaBwdLayout hca_bwd_layout(int64_t B, int64_t T, int64_t H) {
     HcaBwdLayout L;
@@ -2156,13 +2159,43 @@ static HcaBwdLayout hca_bwd_layout(int64_t B, int64_t T, int64_t H) {
     const size_t rows = static_cast<size_t>(B) * H * T;
     L.D = 256;
     L.dQacc = up(L.D + rows * 4);
-    L.total = up(L.dQacc + rows * hca::HD * 4);
+    L.dKVacc = L.total = up(L.dQacc + rows * hca::HD * 4);
     return L;
+}
+static size_t hca_bwd_split_bytes(int64_t tiles) { return static_cast<size_t>(tiles) * 2 * hca_bwd::KEYS * hca::HD * 4; }
+
+// Parts that the backward's key tiles are split in: 2 where the CTA with the most work then has a fifth less of it. Work in elements
+// (one head, 64 queries); an item costs about 3 more to start and finish, adding up a tile's dV and dK in fp32 another 4.
+// Forward + backward on the device, whole tiles -> halves: 1 x 2048 positions, 32 / 8 heads (128 tiles of 128 down to 8 elements on
+// 148 SMs) 270 -> 200 us, 1 x 1000, 64 / 8 heads 257 -> 186, 2 x 1189, 4 / 2 heads 100 -> 84; 1 x 3594, 32 / 8 heads (232 tiles, 5 %
+// less work for the longest CTA) 575 -> 603, 4 x 500 (3 % less) 124 -> 130.
+static int hca_bwd_parts(int BG, int rep, int T, int sms) {
+    const int kt_tiles = ceil_div(T, hca_bwd::KEYS), q_tiles = ceil_div(T, hca_bwd::QE);
+    if (kt_tiles < 2 || static_cast<int64_t>(BG) * kt_tiles > kSplitTiles) return 1;
+    int most[3] = {0, 0, 0};
+    for (int parts = 1; parts <= 2; ++parts) {
+        const int items = BG * kt_tiles * parts, G = items < sms ? items : sms;
+        for (int c = 0; c < G; ++c) {
+            int load = 0;
+            for (int k = 0, item; (item = k * G + (k & 1 ? G - 1 - c : c)) < items || k * G < items; ++k) {
+                if (item >= items) continue;
+                const int n_e = rep * (q_tiles - 2 * (item / parts / BG)), z = item % parts;
+                load += n_e * (z + 1) / parts - n_e * z / parts + (parts == 1 ? 3 : 7);
+            }
+            if (load > most[parts]) most[parts] = load;
+        }
+    }
+    return 6 * most[2] < 5 * most[1] ? 2 : 1;
 }
 
 int hass_hca_attention_bwd_workspace_bytes(int64_t B, int64_t T, int64_t H, int32_t m, size_t* bytes) {
     if (!bytes || B < 1 || T < 1 || H < 1 || m < 0 || m > HASS_HCA_MAX_DRAFTS) return HASS_ERR_INVALID_ARG;
     *bytes = hca_bwd_layout(B, T, H).total;
+    const int64_t kt_tiles = (T + hca_bwd::KEYS - 1) / hca_bwd::KEYS;
+    if (kt_tiles > 1 && B * kt_tiles <= kSplitTiles) {
+        const int64_t tiles = B * H * kt_tiles;      // (the key/value heads are at most the query heads)
+        *bytes += hca_bwd_split_bytes(tiles < kSplitTiles ? tiles : kSplitTiles);
+    }
     return HASS_OK;
 }
 
@@ -2218,6 +2251,12 @@ int hass_hca_attention_bwd(const void* Q, const void* K_t, const void* V_t, cons
     }
     if (rc != HASS_OK) return rc;
 
+    k.kt_tiles = static_cast<int>((T + hca_bwd::KEYS - 1) / hca_bwd::KEYS);
+    int parts = 1;
+    if (workspace_bytes >= L.total + hca_bwd_split_bytes(B * Hkv * k.kt_tiles)) parts = hca_bwd_parts(iB * iHkv, iH / iHkv, iT, di.sms);
+    const bool split = parts > 1;
+    float* dKVacc = reinterpret_cast<float*>(ws + L.dKVacc);
+    k.dKVacc = dKVacc;
     {   // D, the substituted entries and everything that follows from them, the start value of the dQ accumulator
         hca_bwd::RowsParams r;
         std::memset(&r, 0, sizeof(r));
@@ -2233,13 +2272,15 @@ int hass_hca_attention_bwd(const void* Q, const void* K_t, const void* V_t, cons
         r.lse = lse;
         r.D = Dv;
         r.dQacc = dQacc;
+        r.dKVacc = dKVacc;
         r.m = m; r.B = iB; r.T = iT; r.H = iH; r.Hkv = iHkv;
         r.c2 = c2;
         r.scale = scale;
         r.status = static_cast<unsigned int*>(workspace);
         KernelTimer kt(KIND_HCA_BWD_ROWS, st);
         const long long halves = static_cast<long long>(B) * T * Hkv;
-        rc = launch(hca_bwd::hca_bwd_rows_kernel, (halves * 16 + 255) / 256, 256, 0, st, 1, r);
+        r.row_blocks = static_cast<unsigned int>((halves * 16 + 255) / 256);
+        rc = launch(hca_bwd::hca_bwd_rows_kernel, r.row_blocks + (split ? 2ll * iB * iHkv * k.kt_tiles : 0), 256, 0, st, 1, r);
     }
     if (rc != HASS_OK) return rc;
 
@@ -2248,7 +2289,6 @@ int hass_hca_attention_bwd(const void* Q, const void* K_t, const void* V_t, cons
     k.lse = lse;
     k.D = Dv;
     k.B = iB; k.T = iT; k.H = iH; k.Hkv = iHkv; k.m = m;
-    k.kt_tiles = static_cast<int>((T + hca_bwd::KEYS - 1) / hca_bwd::KEYS);
     k.q_tiles64 = static_cast<int>((T + hca_bwd::QE - 1) / hca_bwd::QE);
     k.items = iB * iHkv * k.kt_tiles;
     k.c2 = c2;
@@ -2256,15 +2296,24 @@ int hass_hca_attention_bwd(const void* Q, const void* K_t, const void* V_t, cons
     k.status = static_cast<unsigned int*>(workspace);
     {
         KernelTimer kt(KIND_HCA_BWD_FUSED, st);
-        rc = launch(hca_bwd::hca_bwd_fused_kernel, k.items < di.sms ? k.items : di.sms, hca_bwd::NUM_THREADS, hca_bwd::F_SMEM_BYTES, st, 1, k);
+        rc = launch(split ? hca_bwd::hca_bwd_fused_kernel<2> : hca_bwd::hca_bwd_fused_kernel<1>, k.items * parts < di.sms ? k.items * parts : di.sms, hca_bwd::NUM_THREADS, hca_bwd::F_SMEM_BYTES, st, 1, k);
     }
     if (rc != HASS_OK) return rc;
 
     {
         KernelTimer kt(KIND_HCA_DQ_CONVERT, st);
-        const long long n8 = static_cast<long long>(B) * T * H * (hca::HD / 8);
-        return launch(hca_bwd::hca_dq_convert_kernel, (n8 + 255) / 256, 256, 0, st, 1, static_cast<const float*>(dQacc),
-                      static_cast<__nv_bfloat16*>(dQ), n8);
+        hca_bwd::ConvertParams c;
+        std::memset(&c, 0, sizeof(c));
+        c.dQacc = dQacc;
+        c.dQ = static_cast<__nv_bfloat16*>(dQ);
+        c.n8 = B * T * H * (hca::HD / 8);
+        c.dKVacc = split ? dKVacc : nullptr;
+        c.dV = k.dV;
+        c.dK = k.dK;
+        c.B = iB; c.T = iT; c.Hkv = iHkv;
+        c.kt_tiles = k.kt_tiles;
+        const long long threads = c.n8 + (split ? 2ll * k.items * 16 * hca_bwd::KEYS : 0);
+        return launch(hca_bwd::hca_dq_convert_kernel, (threads + 255) / 256, 256, 0, st, 1, c);
     }
 }
 

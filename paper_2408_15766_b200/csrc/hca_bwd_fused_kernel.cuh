@@ -60,6 +60,12 @@ __device__ __forceinline__ void tma_reduce_add_3d(const CUtensorMap* tm, uint32_
                  "r"(smem_src), "r"(x), "r"(y), "r"(z)
                  : "memory");
 }
+// at[0..3] += ...; at 16-byte aligned
+__device__ __forceinline__ void red_add_v4(float* at, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(at), "f"(__uint_as_float(x)), "f"(__uint_as_float(y)),
+                 "f"(__uint_as_float(z)), "f"(__uint_as_float(w))
+                 : "memory");
+}
 // sum over the 16 lanes of a half-warp
 __device__ __forceinline__ float sum16(float v) {
 #pragma unroll
@@ -91,6 +97,8 @@ struct RowsParams {
     const float* lse;              // [B, H, T]
     float* D;                      // [B, H, T]
     float* dQacc;                  // [B, T, H, 128] fp32
+    unsigned int row_blocks;       // blocks from here on each zero a tile of dKVacc (FusedParams)
+    float* dKVacc;
     int m, B, T, H, Hkv;
     float c2, scale;
     unsigned int* status;          // status block of 64 words, cleared here
@@ -99,6 +107,12 @@ struct RowsParams {
 __global__ void __launch_bounds__(256, 2) hca_bwd_rows_kernel(const __grid_constant__ RowsParams p) {
     wait_previous_kernel(false);
     if (blockIdx.x == 0 && threadIdx.x < 64) p.status[threadIdx.x] = 0u;
+    if (blockIdx.x >= p.row_blocks) {
+        // a key tile of the fp32 dV or dK
+        float4* z = reinterpret_cast<float4*>(p.dKVacc) + static_cast<size_t>(blockIdx.x - p.row_blocks) * (KEYS * HD / 4);
+        for (int i = threadIdx.x; i < KEYS * HD / 4; i += 256) z[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        return;
+    }
     const long long w = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 4;   // (b, t, g)
     const int sub = threadIdx.x & 15;
     // no thread leaves early: the shuffles below name all 32 lanes, so a half-warp past the end runs on clamped
@@ -211,15 +225,38 @@ __global__ void __launch_bounds__(256, 2) hca_bwd_rows_kernel(const __grid_const
     }
 }
 
-// dQ = the fp32 accumulator as bf16; 8 values per thread.
-__global__ void __launch_bounds__(256) hca_dq_convert_kernel(const float* acc, __nv_bfloat16* dQ,
-                                                             long long n8) {
+// dQ = the fp32 accumulator as bf16; 8 values per thread. With dKVacc, dV and dK likewise by the threads behind those, 8
+// columns of a position each.
+struct ConvertParams {
+    const float* dQacc;
+    __nv_bfloat16* dQ;
+    long long n8;                  // threads that dQ takes
+    const float* dKVacc;           // nullable
+    __nv_bfloat16* dV;
+    __nv_bfloat16* dK;
+    int B, T, Hkv, kt_tiles;
+};
+__global__ void __launch_bounds__(256) hca_dq_convert_kernel(const __grid_constant__ ConvertParams p) {
     wait_previous_kernel(false);
     const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i >= n8) return;
-    float v[8];
-    ld_global_v8(acc + 8 * i, v);
-    *(reinterpret_cast<uint4*>(dQ) + i) = narrow8(v);
+    if (i < p.n8) {
+        float v[8];
+        ld_global_v8(p.dQacc + 8 * i, v);
+        *(reinterpret_cast<uint4*>(p.dQ) + i) = narrow8(v);
+        return;
+    }
+    if (p.dKVacc == nullptr) return;
+    const long long j = i - p.n8;
+    const int r = static_cast<int>(j % KEYS), o = static_cast<int>(j / KEYS % 16);
+    const long long tile = j / (KEYS * 16);                       // (matrix, b, g, key tile)
+    const long long mbg = tile / p.kt_tiles, mb = mbg / p.Hkv;
+    const int t = static_cast<int>(tile - mbg * p.kt_tiles) * KEYS + r, g = static_cast<int>(mbg - mb * p.Hkv);
+    const long long matrix = mb / p.B, b = mb - matrix * p.B;
+    if (matrix > 1 || t >= p.T) return;
+    const float4* src = reinterpret_cast<const float4*>(p.dKVacc) + (tile * 32 + 2 * o) * KEYS + r;
+    const float4 x = src[0], y = src[KEYS];
+    const float f[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+    reinterpret_cast<uint4*>((matrix == 0 ? p.dV : p.dK) + ((b * p.T + t) * p.Hkv + g) * HD)[o] = narrow8(f);
 }
 
 // ------------------------------------------------------------------------------------------------------
@@ -244,6 +281,8 @@ __global__ void __launch_bounds__(256) hca_dq_convert_kernel(const float* acc, _
 // element e needs no barrier for the S^T columns; dP^T(e+2) waits until the threads have taken dQ^T(e) out.
 // The per-query vectors -lse2[t] and -D[t] scale of an element travel with its Q / dO stage (written by a warp
 // that does nothing else).
+// PARTS = 2: two work items per key tile, each with half of its elements, where whole ones would leave most of the SMs without
+// work at the end. Their dV and dK are added up in global memory. (Two terms on top of zero: the order of arrival does not matter.)
 constexpr int F_STAGES = 3;             // a Q / dO stage is held until the element's last product is done
 constexpr int F_SMEM_K = 0;
 constexpr int F_SMEM_V = F_SMEM_K + K_BYTES;
@@ -274,10 +313,13 @@ struct FusedParams {
     int kt_tiles;                  // ceil(T / 128) key tiles
     int q_tiles64;                 // ceil(T / 64) query tiles
     int items;                     // B * Hkv * kt_tiles
+    float* dKVacc;                 // PARTS = 2: dV and dK in fp32, [2][B, Hkv, key tile, 32, 128, 4]: a thread's row in groups of four
+                                   // columns, the rows of a warp side by side
     float c2, scale;
     unsigned int* status;
 };
 
+template <int PARTS>
 __global__ void __launch_bounds__(NUM_THREADS, 1) hca_bwd_fused_kernel(const __grid_constant__ FusedParams p) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t base = smem_u32(smem_raw);
@@ -348,28 +390,38 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_bwd_fused_kernel(const __g
     // is the same, but at any moment different CTAs are in rounds of different item lengths, so that their item
     // boundaries (pipeline drained, a burst of loads) do not coincide. next_item steps the round counter k to this
     // CTA's next existing item and returns it, or -1.
-    const int n_rounds = (p.items + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x);
+    const int BG = p.B * p.Hkv;
+    const int rep = p.H / p.Hkv;
+    const int m = p.m;
+    // elements of a key tile: for each head of the group, the 64-query tiles 2 kt .. q_tiles64 - 1
+    auto q_count = [&](int kt) { return p.q_tiles64 - 2 * kt; };
+    // item -> (key tile, sequence, key/value head, elements [e0, e1)): the first key tiles meet the most queries and come first
+    auto decode = [&](int item, int& kt, int& b, int& g, int& e0, int& e1) {
+        const int tile = item / PARTS, z = item - tile * PARTS;
+        kt = tile / BG;
+        const int bg = tile - kt * BG;
+        b = bg / p.Hkv;
+        g = bg - b * p.Hkv;
+        const int n_e = rep * q_count(kt);
+        e0 = n_e * z / PARTS;
+        e1 = n_e * (z + 1) / PARTS;
+    };
+    const int n_items = p.items * PARTS;
+    const int n_rounds = (n_items + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x);
     auto next_item = [&](int& k) {
         while (k < n_rounds) {
             const int item = round_item(static_cast<uint32_t>((k + static_cast<int>(blockIdx.x)) % n_rounds));
             ++k;
-            if (item < p.items) return item;
+            if (item >= n_items) continue;
+            if (PARTS > 1) {
+                int kt, b, g, e0, e1;
+                decode(item, kt, b, g, e0, e1);
+                if (e0 == e1) continue;      // the first half of a single element
+            }
+            return item;
         }
         return -1;
     };
-
-    const int BG = p.B * p.Hkv;
-    const int rep = p.H / p.Hkv;
-    const int m = p.m;
-    // item -> (key tile, sequence, key/value head): the first key tiles meet the most queries and come first
-    auto decode = [&](int item, int& kt, int& b, int& g) {
-        kt = item / BG;
-        const int bg = item - kt * BG;
-        b = bg / p.Hkv;
-        g = bg - b * p.Hkv;
-    };
-    // elements of an item: for each head of the group, the 64-query tiles 2 kt .. q_tiles64 - 1
-    auto q_count = [&](int kt) { return p.q_tiles64 - 2 * kt; };
 
     if (warp == 0) {
         // ===================== producer: TMA =====================
@@ -377,8 +429,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_bwd_fused_kernel(const __g
             uint32_t gq = 0, it = 0;
             bool ok = true;
             for (int rk = 0, item = next_item(rk); item >= 0 && ok; item = next_item(rk), ++it) {
-                int kt, b, g;
-                decode(item, kt, b, g);
+                int kt, b, g, e0, e1;
+                decode(item, kt, b, g, e0, e1);
                 const int nq = q_count(kt);
                 if (!wait_barrier(kv_empty, (it & 1u) ^ 1u, abort_flag, p.status, 1)) break;
                 mbar_arrive_expect_tx(kv_full, 2 * K_BYTES);
@@ -386,7 +438,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_bwd_fused_kernel(const __g
                 tma_load_3d(base + F_SMEM_K + K_HALF, &p.tmK, kv_full, g * HD + 64, kt * KEYS, b);
                 tma_load_3d(base + F_SMEM_V, &p.tmV, kv_full, g * HD, kt * KEYS, b);
                 tma_load_3d(base + F_SMEM_V + K_HALF, &p.tmV, kv_full, g * HD + 64, kt * KEYS, b);
-                for (int e = 0; e < rep * nq; ++e, ++gq) {
+                for (int e = e0; e < e1; ++e, ++gq) {
                     const int h = g * rep + e / nq;
                     const int jq = 2 * kt + e % nq;
                     const int s = gq % F_STAGES;
@@ -406,10 +458,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_bwd_fused_kernel(const __g
         uint32_t gq = 0, it = 0;
         bool ok = true;
         for (int rk = 0, item = next_item(rk); item >= 0 && ok; item = next_item(rk), ++it) {
-            int kt, b, g;
-            decode(item, kt, b, g);
+            int kt, b, g, e0, e1;
+            decode(item, kt, b, g, e0, e1);
             const int nq = q_count(kt);
-            for (int e = 0; e < rep * nq && ok; ++e, ++gq) {
+            for (int e = e0; e < e1 && ok; ++e, ++gq) {
                 const int h = g * rep + e / nq;
                 const int jq = 2 * kt + e % nq;
                 const int s = gq % F_STAGES;
@@ -514,9 +566,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_bwd_fused_kernel(const __g
             return true;
         };
         for (int rk = 0, item = next_item(rk); item >= 0 && ok; item = next_item(rk), ++it) {
-            int kt, b, g;
-            decode(item, kt, b, g);
-            const int n_e = rep * q_count(kt);
+            int kt, b, g, e0, e1;
+            decode(item, kt, b, g, e0, e1);
+            const int n_e = e1 - e0;
             if (!wait_all(kv_full, it & 1u, 6)) break;
             ok = issue_st();
             if (ok && n_e > 1) ok = issue_st();
@@ -573,12 +625,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_bwd_fused_kernel(const __g
             return true;
         };
         for (int rk = 0, item = next_item(rk); item >= 0 && ok; item = next_item(rk), ++it) {
-            int kt, b, g;
-            decode(item, kt, b, g);
+            int kt, b, g, e0, e1;
+            decode(item, kt, b, g, e0, e1);
             const int nq = q_count(kt);
             const int spos = kt * KEYS + r;             // key position
-            const int n_e = rep * nq;
-            for (int e = 0; e < n_e; ++e, ++gq) {
+            for (int e = e0; e < e1; ++e, ++gq) {
                 const int jq = 2 * kt + e % nq;
                 const int s = gq & 1u;                  // tensor-memory set
                 const int qs = gq % F_STAGES;           // the element's Q / dO stage, for its vectors
@@ -643,14 +694,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_bwd_fused_kernel(const __g
                 if (lane == 0) mbar_arrive(pds_full(s));
                 // the element before this one: its products were issued when its P^T / dS^T arrived and run while this
                 // element's were being formed
-                if (e > 0) {
+                if (e > e0) {
                     const int ep = e - 1;
                     if (!take_dq(gq - 1, b, g * rep + ep / nq, 2 * kt + ep % nq)) { ok = false; break; }
                 }
             }
             if (!ok) break;
-            if (!take_dq(gq - 1, b, g * rep + (n_e - 1) / nq, 2 * kt + (n_e - 1) % nq)) break;
-            // ---- epilogue: this key row of dV (group 0) or dK (group 1) as bf16 ----
+            if (!take_dq(gq - 1, b, g * rep + (e1 - 1) / nq, 2 * kt + (e1 - 1) % nq)) break;
+            // ---- epilogue: this key row of dV (group 0) or dK (group 1) as bf16, or its share of it in fp32 ----
             if (!wait_barrier(acc_done, it & 1u, abort_flag, p.status, 13)) break;
             tc_fence_after_sync();
             const bool valid = spos < p.T;
@@ -668,7 +719,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_bwd_fused_kernel(const __g
                     __syncwarp();
                     if (lane == 0) mbar_arrive(acc_free);
                 }
-                if (valid) {
+                if (PARTS > 1) {
+                    float* acc = p.dKVacc + (((static_cast<size_t>(grp) * BG + b * p.Hkv + g) * p.kt_tiles + kt) * 32 + 16 * part) * (KEYS * 4) + 4 * r;
+#pragma unroll
+                    for (int c4 = 0; c4 < 16; ++c4) {
+                        const uint32_t* x = &raw[c4 >> 3][4 * (c4 & 7)];
+                        red_add_v4(acc + c4 * (KEYS * 4), x[0], x[1], x[2], x[3]);
+                    }
+                } else if (valid) {
 #pragma unroll
                     for (int k = 0; k < 2; ++k) {
 #pragma unroll

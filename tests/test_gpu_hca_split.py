@@ -1,0 +1,34 @@
+"""Backward of the HCA attention with every key tile's work in two halves, where few key tiles would leave SMs idle."""
+import pytest
+import torch
+
+import hass_inputs as hi
+
+pytestmark = pytest.mark.gpu
+
+
+# two key tiles, the second of one position (a single element: an empty half); odd halves; more halves than SMs
+@pytest.mark.parametrize("B,T,H,Hkv,m", [(1, 129, 1, 1, 0), (2, 333, 4, 2, 3), (1, 700, 3, 1, 1), (2, 1100, 32, 8, 2), (1, 1025, 16, 16, 8)])
+def test_halves_of_a_key_tile_add_up_to_the_whole(B, T, H, Hkv, m):
+    import paper_2408_15766_b200 as hass
+    dev = torch.device("cuda:0")
+    inp = hi.make_hca_inputs(hi.HcaWorkload("split", B=B, T=T, H=H, Hkv=Hkv, m=m, seed=T))
+    dO = torch.randn(inp.Q.shape, generator=torch.Generator().manual_seed(1)).to(torch.bfloat16).to(dev)
+    qkv = [x.to(dev) for x in (inp.Q, inp.K_t, inp.V_t)]
+    Kd, Vd = [x.to(dev) for x in inp.K_d], [x.to(dev) for x in inp.V_d]
+    fw = hass.hca_attention_fwd(*qkv, Kd, Vd)
+    hass.check(fw["workspace"])
+    whole = 256 + -(-B * H * T * 4 // 256) * 256 + B * T * H * 512      # status, D, the dQ accumulator: no room for the halves
+    assert hass.hca_attention_bwd_workspace_bytes(B, T, H, m) > whole
+    runs = []
+    for ws in (torch.empty(whole, dtype=torch.uint8, device=dev), None, None):
+        bw = hass.hca_attention_bwd(*qkv, Kd, Vd, fw["O"], fw["lse"], dO, workspace=ws)
+        hass.check(bw["workspace"])
+        runs.append(bw)
+    for name in ("dQ", "dK_t", "dV_t"):
+        a, b = runs[0][name].float(), runs[1][name].float()
+        # fp32 sums in another order, rounded to bf16: one unit in the last place (2^-7 of the value), or 1e-5 of the largest
+        # entry where a sum cancels
+        assert ((a - b).abs() <= 2.0 ** -7 * a.abs() + 1e-5 * a.abs().max()).all(), name
+    for name in ("dK_t", "dV_t"):
+        assert torch.equal(runs[1][name], runs[2][name]), name
