@@ -2280,7 +2280,7 @@ int hass_hca_attention_bwd(const void* Q, const void* K_t, const void* V_t, cons
         KernelTimer kt(KIND_HCA_BWD_ROWS, st);
         const long long halves = static_cast<long long>(B) * T * Hkv;
         r.row_blocks = static_cast<unsigned int>((halves * 16 + 255) / 256);
-        rc = launch(hca_bwd::hca_bwd_rows_kernel, r.row_blocks + (split ? 2ll * iB * iHkv * k.kt_tiles : 0), 256, 0, st, 1, r);
+        rc = launch(H == Hkv ? hca_bwd::hca_bwd_rows_mha_kernel : hca_bwd::hca_bwd_rows_kernel, r.row_blocks + (split ? 2ll * iB * iHkv * k.kt_tiles : 0), 256, 0, st, 1, r);
     }
     if (rc != HASS_OK) return rc;
 

@@ -104,13 +104,17 @@ struct RowsParams {
     unsigned int* status;          // status block of 64 words, cleared here
 };
 
+// a block's key tile of the fp32 dV or dK
+__device__ __forceinline__ void zero_tile(const RowsParams& p) {
+    float4* z = reinterpret_cast<float4*>(p.dKVacc) + static_cast<size_t>(blockIdx.x - p.row_blocks) * (KEYS * HD / 4);
+    for (int i = threadIdx.x; i < KEYS * HD / 4; i += 256) z[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
 __global__ void __launch_bounds__(256, 2) hca_bwd_rows_kernel(const __grid_constant__ RowsParams p) {
     wait_previous_kernel(false);
     if (blockIdx.x == 0 && threadIdx.x < 64) p.status[threadIdx.x] = 0u;
     if (blockIdx.x >= p.row_blocks) {
-        // a key tile of the fp32 dV or dK
-        float4* z = reinterpret_cast<float4*>(p.dKVacc) + static_cast<size_t>(blockIdx.x - p.row_blocks) * (KEYS * HD / 4);
-        for (int i = threadIdx.x; i < KEYS * HD / 4; i += 256) z[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        zero_tile(p);
         return;
     }
     const long long w = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 4;   // (b, t, g)
@@ -223,6 +227,91 @@ __global__ void __launch_bounds__(256, 2) hca_bwd_rows_kernel(const __grid_const
             }
         }
     }
+}
+
+// The same where every query head has a key/value head of its own (Hkv = H): an output row of dK_d, dV_d has one term, so that
+// nothing is carried from head to head, the passes can follow one another with dQ's share in registers, and Q, dO and the accumulator are
+// touched once however many passes there are. The rows of ROW_PASSES passes are requested together. Bound by memory: 2 x 759
+// positions, 40 heads, m = 5: 91 -> 67 us (390 MB: 5.8 TB/s), forward + backward 246 -> 219 us; 4 x 2048, 32 heads, m = 0 861 -> 810 us,
+// 1 x 3318, 40 heads, m = 5 767 -> 711. (Grouped heads a half-warp each, their sums by shuffles and shared memory, were no faster than the kernel
+// above: 4 x 2048, 32 / 8 heads, m = 2 741 -> 797 us, m = 5 933 -> 946.)
+constexpr int ROW_PASSES = 4;
+__global__ void __launch_bounds__(256, 3) hca_bwd_rows_mha_kernel(const __grid_constant__ RowsParams p) {
+    wait_previous_kernel(false);
+    if (blockIdx.x == 0 && threadIdx.x < 64) p.status[threadIdx.x] = 0u;
+    if (blockIdx.x >= p.row_blocks) {
+        zero_tile(p);
+        return;
+    }
+    const long long w = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 4;   // (b, t, h)
+    const int sub = threadIdx.x & 15;
+    // (as above: a half-warp past the end runs on clamped indices with its stores switched off)
+    const long long total = static_cast<long long>(p.B) * p.T * p.H;
+    const bool live = w < total;
+    const long long wc = live ? w : total - 1;
+    const long long bt = wc / p.H;
+    const int h = static_cast<int>(wc - bt * p.H);
+    const long long b = bt / p.T;
+    const int t = static_cast<int>(bt - b * p.T);
+    const long long at = wc * (HD / 8) + sub;                     // this lane's 8 columns, in 16-byte words
+    const long long back = static_cast<long long>(p.H) * (HD / 8);   // one position earlier
+    const uint4 qr = reinterpret_cast<const uint4*>(p.Q)[at];
+    const uint4 dr = reinterpret_cast<const uint4*>(p.dO)[at];
+    const uint4 orow = reinterpret_cast<const uint4*>(p.O)[at];
+    const long long ri = (b * p.H + h) * p.T + t;
+    const float nlse2 = -p.lse[ri] * 1.4426950408889634f;
+    float qf[8], df[8], dq[8], Dt = 0.f;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) dq[c] = 0.f;
+    for (int i0 = 0; i0 == 0 || i0 < p.m; i0 += ROW_PASSES) {
+        uint4 kraw[ROW_PASSES], vraw[ROW_PASSES];
+#pragma unroll
+        for (int j = 0; j < ROW_PASSES; ++j) {
+            kraw[j] = vraw[j] = make_uint4(0u, 0u, 0u, 0u);
+            if (i0 + j < p.m && t - (i0 + j) >= 0) {
+                kraw[j] = reinterpret_cast<const uint4*>(p.Kd[i0 + j])[at - (i0 + j) * back];
+                vraw[j] = reinterpret_cast<const uint4*>(p.Vd[i0 + j])[at - (i0 + j) * back];
+            }
+        }
+        if (i0 == 0) {
+            float of[8];
+            widen8(qr, qf);
+            widen8(dr, df);
+            widen8(orow, of);
+            Dt = sum16(dot8(df, of));
+            if (live && sub == 0) p.D[ri] = Dt;
+        }
+#pragma unroll
+        for (int j = 0; j < ROW_PASSES; ++j) {
+            const int i = i0 + j;
+            if (i < p.m) {
+                float kf[8], vf[8], x[8];
+                widen8(kraw[j], kf);
+                widen8(vraw[j], vf);
+                const float sv = sum16(dot8(qf, kf));
+                const float dv = sum16(dot8(df, vf));
+                const bool use = t - i >= 0;
+                const float pw = use ? ex2(fmaf(sv, p.c2, nlse2)) : 0.f;
+                const float ds = pw * (dv - Dt) * p.scale;
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    dq[c] = fmaf(ds, kf[c], dq[c]);
+                    kf[c] = ds * qf[c];
+                    x[c] = pw * df[c];
+                }
+                uint4* dk = reinterpret_cast<uint4*>(p.dKd[i]);
+                uint4* dvp = reinterpret_cast<uint4*>(p.dVd[i]);
+                if (live && use) {
+                    dk[at - i * back] = narrow8(kf);
+                    dvp[at - i * back] = narrow8(x);
+                }
+                if (live && t + i >= p.T) dk[at] = dvp[at] = make_uint4(0u, 0u, 0u, 0u);
+            }
+        }
+    }
+    if (live)
+        st_global_v8(p.dQacc + at * 8, __float_as_uint(dq[0]), __float_as_uint(dq[1]), __float_as_uint(dq[2]), __float_as_uint(dq[3]),
+                     __float_as_uint(dq[4]), __float_as_uint(dq[5]), __float_as_uint(dq[6]), __float_as_uint(dq[7]));
 }
 
 // dQ = the fp32 accumulator as bf16; 8 values per thread. With dKVacc, dV and dK likewise by the threads behind those, 8
