@@ -101,13 +101,13 @@ def _ok(status: int, where: str) -> None:
         raise HassError(status, where)
 
 
-def _p(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+def _p(t: Optional[torch.Tensor]) -> Optional[int]:
+    return None if t is None else t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+def _stream(stream) -> int:
+    # (the current stream's handle alone: building a torch.cuda.Stream object takes 3 us)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) if stream is None else stream.cuda_stream
 
 
 def _dims(H: torch.Tensor, W: torch.Tensor):
@@ -130,9 +130,10 @@ def topk_distill_host_workspace_bytes(N: int, d: int, V: int, K: int, dH_dtype: 
     return int(out.value)
 
 
-def _workspace(ws: Optional[torch.Tensor], nbytes: int, device) -> torch.Tensor:
+def _workspace(ws: Optional[torch.Tensor], device, nbytes, *sizes) -> torch.Tensor:
+    """The caller's workspace, or a new one of nbytes(*sizes) bytes."""
     if ws is None:
-        ws = torch.empty(nbytes, dtype=torch.uint8, device=device)
+        ws = torch.empty(nbytes(*sizes), dtype=torch.uint8, device=device)
     assert ws.dtype == torch.uint8 and ws.is_cuda and ws.is_contiguous()
     return ws
 
@@ -145,7 +146,7 @@ def topk_distill_fwd(H_t, H_d, W, K: int, workspace=None, stream=None) -> dict:
     N, d, V = _dims(H_t, W)
     assert H_d.shape == H_t.shape and H_d.dtype == torch.bfloat16 and H_d.is_contiguous()
     dev = H_t.device
-    ws = _workspace(workspace, topk_distill_workspace_bytes(N, d, V, K), dev)
+    ws = _workspace(workspace, dev, topk_distill_workspace_bytes, N, d, V, K)
     out = dict(loss=torch.empty(N, dtype=torch.float32, device=dev),
                topk_idx=torch.empty(N, K, dtype=torch.int32, device=dev),
                topk_q=torch.empty(N, K, dtype=torch.float32, device=dev),
@@ -196,7 +197,7 @@ def topk_distill_fwd_draft(H_d, W, topk_idx, topk_q, workspace=None, stream=None
     assert topk_idx.dtype == torch.int32 and topk_q.dtype == torch.float32
     assert topk_idx.is_contiguous() and topk_q.is_contiguous() and topk_idx.shape == topk_q.shape == (N, K)
     dev = H_d.device
-    ws = _workspace(workspace, topk_distill_workspace_bytes(N, d, V, K), dev)
+    ws = _workspace(workspace, dev, topk_distill_workspace_bytes, N, d, V, K)
     out = dict(loss=torch.empty(N, dtype=torch.float32, device=dev),
                lse_d=torch.empty(N, dtype=torch.float32, device=dev), workspace=ws)
     _ok(lib.hass_topk_distill_fwd_draft(_p(H_d), _p(W), N, d, V, K, _p(topk_idx), _p(topk_q), _p(out["loss"]),
@@ -213,7 +214,7 @@ def topk_distill_bwd(H_d, W, topk_idx, topk_q, lse_d, grad_loss=None, dH_dtype: 
     assert topk_idx.is_contiguous() and topk_q.is_contiguous() and lse_d.is_contiguous()
     assert grad_loss is None or (grad_loss.dtype == torch.float32 and grad_loss.shape == (N,))
     dev = H_d.device
-    ws = _workspace(workspace, topk_distill_workspace_bytes(N, d, V, K), dev)
+    ws = _workspace(workspace, dev, topk_distill_workspace_bytes, N, d, V, K)
     dH = torch.empty(N, d, dtype=_dh_dtype(dH_dtype), device=dev) if out is None else out
     _ok(lib.hass_topk_distill_bwd(_p(H_d), _p(W), N, d, V, K, _p(topk_idx), _p(topk_q), _p(lse_d), _p(grad_loss),
                                   _p(dH), dH_dtype, _p(ws), ws.numel(), _stream(stream)), "hass_topk_distill_bwd")
@@ -226,7 +227,7 @@ def topk_distill_fwd_bwd(H_t, H_d, W, K: int, grad_loss=None, dH_dtype: int = HA
     assert H_d.shape == H_t.shape and H_d.dtype == torch.bfloat16 and H_d.is_contiguous()
     assert grad_loss is None or (grad_loss.dtype == torch.float32 and grad_loss.shape == (N,))
     dev = H_t.device
-    ws = _workspace(workspace, topk_distill_workspace_bytes(N, d, V, K), dev)
+    ws = _workspace(workspace, dev, topk_distill_workspace_bytes, N, d, V, K)
     if out is None:
         out = dict(loss=torch.empty(N, dtype=torch.float32, device=dev),
                    topk_idx=torch.empty(N, K, dtype=torch.int32, device=dev),
@@ -250,7 +251,7 @@ def topk_distill_fwd_bwd_draft(H_d, W, topk_idx, topk_q, grad_loss=None, dH_dtyp
     assert topk_idx.is_contiguous() and topk_q.is_contiguous() and topk_idx.shape == topk_q.shape == (N, K)
     assert grad_loss is None or (grad_loss.dtype == torch.float32 and grad_loss.shape == (N,))
     dev = H_d.device
-    ws = _workspace(workspace, topk_distill_workspace_bytes(N, d, V, K), dev)
+    ws = _workspace(workspace, dev, topk_distill_workspace_bytes, N, d, V, K)
     if out is None:
         out = dict(loss=torch.empty(N, dtype=torch.float32, device=dev),
                    lse_d=torch.empty(N, dtype=torch.float32, device=dev),
@@ -275,7 +276,7 @@ def combined_distill_fwd_bwd(H_t, H_d, W, K: int, w_topk: float = 1.0, grad_loss
     assert H_d.shape == H_t.shape and H_d.dtype == torch.bfloat16 and H_d.is_contiguous()
     assert grad_loss is None or (grad_loss.dtype == torch.float32 and grad_loss.shape == (N,))
     dev = H_t.device
-    ws = _workspace(workspace, combined_distill_workspace_bytes(N, d, V, K), dev)
+    ws = _workspace(workspace, dev, combined_distill_workspace_bytes, N, d, V, K)
     if out is None:
         out = dict(loss_ce=torch.empty(N, dtype=torch.float32, device=dev),
                    loss=torch.empty(N, dtype=torch.float32, device=dev),
@@ -302,7 +303,7 @@ def variant_distill_fwd_bwd(H_t, H_d, W, K: int, variant: int, param: float = 0.
     assert H_d.shape == H_t.shape and H_d.dtype == torch.bfloat16 and H_d.is_contiguous()
     assert grad_loss is None or (grad_loss.dtype == torch.float32 and grad_loss.shape == (N,))
     dev = H_t.device
-    ws = _workspace(workspace, topk_distill_workspace_bytes(N, d, V, K), dev)
+    ws = _workspace(workspace, dev, topk_distill_workspace_bytes, N, d, V, K)
     kk = 2 * K if variant == LOSS_BIDIR_TOPK else K      # the bi-directional set holds up to 2K tokens
     out = dict(loss=torch.empty(N, dtype=torch.float32, device=dev),
                topk_idx=torch.empty(N, kk, dtype=torch.int32, device=dev),
@@ -328,7 +329,7 @@ def topk_distill_fwd_bwd_host(H_t_host, H_d_host, W, K: int, loss_host, dH_d_hos
     assert H_d_host.shape == H_t_host.shape and H_d_host.dtype == torch.bfloat16 and H_d_host.is_contiguous()
     assert loss_host.dtype == torch.float32 and loss_host.shape == (N,) and not loss_host.is_cuda
     assert dH_d_host.dtype == _dh_dtype(dH_dtype) and dH_d_host.shape == (N, d) and dH_d_host.is_contiguous()
-    ws = _workspace(workspace, topk_distill_host_workspace_bytes(N, d, V, K, dH_dtype), W.device)
+    ws = _workspace(workspace, W.device, topk_distill_host_workspace_bytes, N, d, V, K, dH_dtype)
     _ok(lib.hass_topk_distill_fwd_bwd_host(_p(H_t_host), _p(H_d_host), _p(W), N, d, V, K, _p(grad_loss_host),
                                            _p(loss_host), _p(topk_idx_host), _p(topk_q_host), _p(dH_d_host),
                                            dH_dtype, _p(ws), ws.numel(), _stream(stream)),
@@ -352,13 +353,14 @@ def hca_attention_fwd(Q, K_t, V_t, K_d=(), V_d=(), scale: Optional[float] = None
     Hkv = K_t.shape[2]
     m = len(K_d)
     assert len(V_d) == m
+    kv = K_t.shape
+    assert kv == (B, T, Hkv, D)
+    for x in (V_t, *K_d, *V_d):
+        assert x.shape == kv
     for x in (Q, K_t, V_t, *K_d, *V_d):
         assert x.is_cuda and x.dtype == torch.bfloat16 and x.is_contiguous()
-    for x in (V_t, *K_d, *V_d):
-        assert x.shape == K_t.shape
-    assert K_t.shape == (B, T, Hkv, D)
     dev = Q.device
-    ws = _workspace(workspace, hca_attention_workspace_bytes(), dev)
+    ws = _workspace(workspace, dev, hca_attention_workspace_bytes)
     out = dict(O=torch.empty_like(Q), lse=torch.empty(B, H, T, dtype=torch.float32, device=dev) if want_lse else None,
                workspace=ws)
     kd = (ctypes.c_void_p * max(m, 1))(*[x.data_ptr() for x in K_d])
@@ -385,10 +387,11 @@ def hca_attention_bwd(Q, K_t, V_t, K_d, V_d, O, lse, dO, scale: Optional[float] 
     assert len(V_d) == m
     for x in (Q, K_t, V_t, O, dO, *K_d, *V_d):
         assert x.is_cuda and x.dtype == torch.bfloat16 and x.is_contiguous()
-    assert O.shape == Q.shape and dO.shape == Q.shape and V_t.shape == K_t.shape == (B, T, Hkv, D)
+    kv = K_t.shape
+    assert O.shape == Q.shape and dO.shape == Q.shape and V_t.shape == kv == (B, T, Hkv, D)
     assert lse.dtype == torch.float32 and lse.shape == (B, H, T) and lse.is_contiguous()
     dev = Q.device
-    ws = _workspace(workspace, hca_attention_bwd_workspace_bytes(B, T, H, m), dev)
+    ws = _workspace(workspace, dev, hca_attention_bwd_workspace_bytes, B, T, H, m)
     out = dict(dQ=torch.empty_like(Q), dK_t=torch.empty_like(K_t), dV_t=torch.empty_like(V_t),
                dK_d=[torch.empty_like(K_t) for _ in range(m)], dV_d=[torch.empty_like(K_t) for _ in range(m)],
                workspace=ws)
