@@ -70,7 +70,8 @@ int hass_version(void);
  * bounded scratch areas for one chunk of rows (a fixed number of 128-row tiles that does not grow
  * with N): the bf16 un-normalised draft probabilities (fused call) or dz_d (split backward),
  * chunk_rows x V, and the fp32 Omega_hat term of dH_d, chunk_rows x d; and, behind them, fp32 partial
- * tiles of dH_d (less than one 128-row tile of scratch). A smaller workspace is accepted down to room
+ * tiles of dH_d (less than one 128-row tile of scratch). Calls of at most 128 rows keep their logits in fp32 instead, two
+ * matrices of N x V. A smaller workspace is accepted down to room
  * for one 128-row tile of scratch; the calls then work in smaller chunks, and may do without partial tiles.
  * Needs no GPU (assumes 148 SMs if none is present).
  */
@@ -308,11 +309,13 @@ int hass_hca_attention_fwd(const void* Q, const void* K_t, const void* V_t, cons
  *   dQ [B, T, H, D], dK_t, dV_t [B, T, Hkv, D] bf16      out (32-byte aligned)
  *   dK_d, dV_d   HOST arrays of m DEVICE pointers, each [B, T, Hkv, D] bf16, out
  *   workspace    hass_hca_attention_bwd_workspace_bytes(B, T, H, m) bytes, 256-byte aligned: the status
- *                word, Dt, and dQ in fp32 (4 B T H D bytes)
+ *                word, Dt, and dQ in fp32 (4 B T H D bytes), which it must hold; and, for up to 296 key tiles of 128
+ *                positions, dK_t and dV_t in fp32, with which two work items may share a key tile
  * Three kernels are enqueued on cuda_stream: a row kernel (Dt, the substituted entries with the draft passes'
  * gradients and their share of dQ), one tensor-core kernel for dK_t, dV_t and the key tiles' shares of dQ, which
  * it adds into the fp32 copy with atomic reductions (their order is not fixed, so dQ may differ between two
- * runs in the last bits of that fp32 sum), and the conversion of dQ to bf16. Errors as for the forward.
+ * runs in the last bits of that fp32 sum), and the conversion of dQ (and of dK_t, dV_t where items shared tiles) to bf16.
+ * Errors as for the forward.
  */
 int hass_hca_attention_bwd_workspace_bytes(int64_t B, int64_t T, int64_t H, int32_t m, size_t* bytes);
 int hass_hca_attention_bwd(const void* Q, const void* K_t, const void* V_t, const void* const* K_d,

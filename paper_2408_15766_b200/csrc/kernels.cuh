@@ -724,6 +724,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
             }
             const int t0 = first_tile(rt, ln);
             const int nt = (p.col_tiles - ln + S - 1) / S;
+            // lanes of three tiles and more share their bounds (see below)
+            const bool joint = HAS_TOPK && !USE_REG && p.col_tiles > 2 * S;
             for (int t = t0; t < nt; ++t) {
                 const int ct = t < 0 ? 0 : ln + t * S;
                 // the whole warp must agree before the warp-collective TMEM loads below
@@ -1139,11 +1141,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                     // first tile it leaves about K / S of a tile's logits to a lane instead of K, the buffers hardly fill any more and the
                     // warp compacts next to nothing. 2047 rows x 4096 x 32000, sweep with K = 100 and nine lanes 497 -> 395 us, call 1815 -> 1705;
                     // 4096 rows, K = 64, four lanes: call 2670 -> 2510. (The register lists of K <= 16 admit too little for it to show.)
+                    // It pays from a third tile on: with 74 lanes of one or two tiles the work behind a tile costs as much as it
+                    // saves (130 rows, K = 20: 218.6 us without, 230 with it; 200 rows, K = 100 294 and 318; 242 rows, K = 36 277 and 268).
                     // A logit equal to a foreign bound must still be admitted (ties are settled by token id when the lists
                     // are merged), hence the step just below it. Stale or missing (zero) values only leave the threshold
                     // lower than it could be.
                     float part = thr_own;
-                    if (!USE_REG && hist_inv > 0.f && t >= 0) {
+                    if constexpr (!USE_REG) if (joint && hist_inv > 0.f && t >= 0) {
                         // the first tile's logits are all in the histogram; of a later one's, those admitted follow here
                         if (t == 0) counted = cnt;
                         while (counted < cnt) {
@@ -1164,20 +1168,31 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                         part = fmaxf(part, thr_own);
                     }
                     if (S > 1) {
-                        volatile unsigned int* sh = reinterpret_cast<volatile unsigned int*>(p.thr_share + static_cast<long long>(slot - ln) * BM + r_local);
-                        sh[static_cast<long long>(ln) * (2 * BM)] = ordered_key(__float_as_uint(thr_own));      // (the first tile's bound is in thr_sh)
-                        unsigned int best = 0u;
-                        const int nn = S - 1 < 3 ? S - 1 : 3;
-                        for (int q = 1; q <= nn; ++q) best = max(best, sh[static_cast<long long>((ln + q) % S) * (2 * BM)]);
-                        if (!USE_REG) {
-                            unsigned int least = ordered_key(__float_as_uint(part));
-                            sh[static_cast<long long>(ln) * (2 * BM) + 1] = least;
-#pragma unroll 8
-                            for (int q = 0; q < S; ++q)
-                                if (q != ln) least = min(least, sh[static_cast<long long>(q) * (2 * BM) + 1]);
-                            best = max(best, least);
+                        uint2* sh = p.thr_share + static_cast<long long>(slot - ln) * BM + r_local;
+                        const uint2 own = make_uint2(ordered_key(__float_as_uint(thr_own)), ordered_key(__float_as_uint(part)));      // (the first tile's bound is in thr_sh)
+                        st_relaxed_v2(sh + static_cast<long long>(ln) * BM, own);
+                        if (t + 1 < nt) {
+                            unsigned int best = 0u;
+                            if (!joint) {
+                                const int nn = S - 1 < 3 ? S - 1 : 3;
+                                for (int q = 1; q <= nn; ++q) best = max(best, ld_relaxed_v2(sh + static_cast<long long>((ln + q) % S) * BM).x);
+                            } else {
+                                // eight loads in flight (one by one they take as long as the tile's candidates)
+                                unsigned int least = own.y;
+                                for (int q0 = 0; q0 < S; q0 += 8) {
+                                    uint2 v[8];
+#pragma unroll
+                                    for (int i = 0; i < 8; ++i) v[i] = ld_relaxed_v2(sh + static_cast<long long>(q0 + i < S ? q0 + i : ln) * BM);
+#pragma unroll
+                                    for (int i = 0; i < 8; ++i) {
+                                        best = max(best, v[i].x);
+                                        least = min(least, v[i].y);
+                                    }
+                                }
+                                best = max(best, least);
+                            }
+                            if (best != 0u) thr_sh = fmaxf(thr_sh, nextafterf(__uint_as_float(key_bits(best)), -INFINITY));
                         }
-                        if (best != 0u) thr_sh = fmaxf(thr_sh, nextafterf(__uint_as_float(key_bits(best)), -INFINITY));
                     }
                     thr = fmaxf(thr_own, fmaxf(thr, thr_sh));
                 }

@@ -314,6 +314,15 @@ __device__ __forceinline__ void st_shared_b32_if(uint32_t addr, uint32_t v, bool
                  "r"(static_cast<uint32_t>(on))
                  : "memory");
 }
+// words that other CTAs read and write meanwhile, each pair as one
+__device__ __forceinline__ uint2 ld_relaxed_v2(const uint2* at) {
+    uint2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(at) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_relaxed_v2(uint2* at, uint2 v) {
+    asm volatile("st.relaxed.gpu.global.v2.u32 [%0], {%1, %2};" ::"l"(at), "r"(v.x), "r"(v.y) : "memory");
+}
 // *at++ = (x, id) where x > bound
 __device__ __forceinline__ void append_if_above(uint2*& at, float x, uint32_t id, float bound) {
     unsigned long long p = reinterpret_cast<unsigned long long>(at);
