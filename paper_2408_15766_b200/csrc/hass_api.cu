@@ -880,7 +880,14 @@ static RowParams row_params(int V, int K, const Layout& L) {
 }
 static int launch_rows(int objective, const RowParams& r, int N, cudaStream_t st) {
     KernelTimer timer(KIND_FINALIZE, st);
-    return launch(objective == ROW_COMBINED ? row_kernel<ROW_COMBINED> : objective == ROW_BIDIR ? row_kernel<ROW_BIDIR> : row_kernel<ROW_TOPK>,
+    if (r.V <= ROW_SMALL && r.K <= ROW_SMALL_K)
+        return launch(objective == ROW_COMBINED ? row_kernel<ROW_COMBINED, ROW_THREADS_SMALL>
+                      : objective == ROW_BIDIR  ? row_kernel<ROW_BIDIR, ROW_THREADS_SMALL>
+                                                : row_kernel<ROW_TOPK, ROW_THREADS_SMALL>,
+                      N, ROW_THREADS_SMALL, 0, st, 1, r);
+    return launch(objective == ROW_COMBINED ? row_kernel<ROW_COMBINED, ROW_THREADS>
+                  : objective == ROW_BIDIR  ? row_kernel<ROW_BIDIR, ROW_THREADS>
+                                            : row_kernel<ROW_TOPK, ROW_THREADS>,
                   N, ROW_THREADS, 0, st, 1, r);
 }
 

@@ -2040,15 +2040,16 @@ __global__ void __launch_bounds__(256) loss_patch_kernel(const __grid_constant__
 // The K largest of a row: a thread's largest logit is at hand after the pass for lse, and the K-th largest of these 1024
 // maxima bounds the row's K-th largest from below. Little more than K logits reach it; the threads that hold them read their
 // share again and put them into a pool in shared memory, where each counts those above it.
-// Bound by the latency of two passes over rows of 4 V bytes in L2: ROW_THREADS threads with ROW_LOADS 16-byte loads each in
-// flight.
-constexpr int ROW_THREADS = 1024;
-constexpr int ROW_WARPS = ROW_THREADS / 32;
+// Bound by the latency of two passes over rows of 4 V bytes in L2: 1024 threads with ROW_LOADS 16-byte loads each in flight.
+// Rows of up to ROW_SMALL logits, one load each for 256 threads, are bound by the barriers instead and take 256: 64 rows x 256 x
+// 1024 25.9 -> 25.0 us per call, 104 rows 26.8 -> 25.6. (Of 2000 logits, K = 30 22.2 -> 22.5, 4096, K = 64 34.1 -> 36.2. K is a
+// quarter of the maxima at most: the bound of a larger set admits much of the row.)
+constexpr int ROW_THREADS = 1024, ROW_THREADS_SMALL = 256;
+constexpr int ROW_SMALL = 1024, ROW_SMALL_K = 64;
 constexpr int ROW_LOADS = 4;
-constexpr int ROW_STEP = ROW_LOADS * ROW_THREADS * 4;      // logits per step of a pass
 constexpr int ROW_POOL = 1024;
 constexpr int ROW_SLACK = 32;      // maxima beyond K at which the search of the bound ends
-static_assert(ROW_POOL >= K_CAP && ROW_THREADS >= K_CAP, "room for Omega_hat, a thread for each of its tokens");
+static_assert(ROW_POOL >= K_CAP && ROW_THREADS_SMALL >= K_CAP, "room for Omega_hat, a thread for each of its tokens");
 enum { ROW_TOPK = 0, ROW_COMBINED = 1, ROW_BIDIR = 2 };
 
 struct RowParams {
@@ -2076,8 +2077,8 @@ struct RowParams {
 
 struct RowShared {
     unsigned long long pool[ROW_POOL];
-    float red[4][ROW_WARPS];
-    uint32_t key_min[ROW_WARPS];
+    float red[4][32];
+    uint32_t key_min[32];
     int tok[K_CAP];        // Omega_hat
     float q[K_CAP], z[K_CAP];
     int tok_d[K_CAP];      // the draft's own K largest (ROW_BIDIR)
@@ -2092,28 +2093,29 @@ __device__ __forceinline__ unsigned long long logit_rank(float z, uint32_t id) {
 }
 
 // f(first column, its four logits) for every piece of the row that this thread owns
-template <typename F>
+template <int THREADS, typename F>
 __device__ __forceinline__ void for_own_logits(const float* row, long long pitch, F&& f) {
-    for (long long c0 = threadIdx.x * 4; c0 < pitch; c0 += ROW_STEP) {
+    for (long long c0 = threadIdx.x * 4; c0 < pitch; c0 += ROW_LOADS * THREADS * 4) {
         float4 v[ROW_LOADS];
 #pragma unroll
         for (int u = 0; u < ROW_LOADS; ++u) {
-            const long long at = c0 + u * (ROW_THREADS * 4);
+            const long long at = c0 + u * (THREADS * 4);
             if (at < pitch) v[u] = *reinterpret_cast<const float4*>(row + at);
         }
 #pragma unroll
         for (int u = 0; u < ROW_LOADS; ++u) {
-            const long long at = c0 + u * (ROW_THREADS * 4);
+            const long long at = c0 + u * (THREADS * 4);
             if (at < pitch) f(at, v[u]);
         }
     }
 }
 
 // This thread's largest logit m and sum of 2^((z - m) log2e)
+template <int THREADS>
 __device__ __forceinline__ void own_stats(const float* row, long long pitch, float& m, float& s) {
     m = -INFINITY;
     s = 0.f;
-    for_own_logits(row, pitch, [&](long long, const float4& v) {
+    for_own_logits<THREADS>(row, pitch, [&](long long, const float4& v) {
         const float cm = fmaxf(fmax3(v.x, v.y, v.z), v.w);
         if (cm > m) {
             s *= ex2((m - cm) * LOG2E);
@@ -2124,8 +2126,9 @@ __device__ __forceinline__ void own_stats(const float* row, long long pitch, flo
     });
 }
 
-// The block's log-sum-exp of the threads' (m, s); `red`: 2 x ROW_WARPS floats. Two barriers.
-__device__ __forceinline__ float block_lse(float m, float s, float (*red)[ROW_WARPS]) {
+// The block's log-sum-exp of the threads' (m, s); `red`: 2 x 32 floats. Two barriers.
+template <int THREADS>
+__device__ __forceinline__ float block_lse(float m, float s, float (*red)[32]) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float mx = m;
 #pragma unroll
@@ -2139,8 +2142,8 @@ __device__ __forceinline__ float block_lse(float m, float s, float (*red)[ROW_WA
         red[1][warp] = s;
     }
     __syncthreads();
-    m = red[0][lane];
-    s = red[1][lane];
+    m = lane < THREADS / 32 ? red[0][lane] : -INFINITY;
+    s = lane < THREADS / 32 ? red[1][lane] : 0.f;
     mx = m;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -2153,6 +2156,7 @@ __device__ __forceinline__ float block_lse(float m, float s, float (*red)[ROW_WA
 
 // Block-collective: the K largest logits of the row, in descending order (lower token id first among equal ones), into
 // tok / val; m = this thread's largest logit. Fewer than K logits above -inf: the rest is token 0 at -inf.
+template <int THREADS>
 __device__ __forceinline__ void select_largest(const float* row, long long pitch, int V, int K, float m, RowShared& sh, int* tok, float* val) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t key = m > -INFINITY ? ordered_key(__float_as_uint(m + 0.f)) : 0u;
@@ -2167,8 +2171,8 @@ __device__ __forceinline__ void select_largest(const float* row, long long pitch
     if (groups >= K) {
         // the K-th largest maximum, or a value below it that at most K + ROW_SLACK maxima reach, from the highest bit in which
         // the maxima differ on
-        const uint32_t hi = __reduce_max_sync(0xffffffffu, __float_as_uint(sh.red[0][lane]));
-        const uint32_t lo = __reduce_min_sync(0xffffffffu, sh.key_min[lane]);
+        const uint32_t hi = __reduce_max_sync(0xffffffffu, lane < THREADS / 32 ? __float_as_uint(sh.red[0][lane]) : 0u);
+        const uint32_t lo = __reduce_min_sync(0xffffffffu, lane < THREADS / 32 ? sh.key_min[lane] : 0xffffffffu);
         int bit = 32 - __clz(hi ^ lo);
         T = bit < 32 ? hi >> bit << bit : 0u;
         for (--bit; bit >= 0; --bit) {
@@ -2183,7 +2187,7 @@ __device__ __forceinline__ void select_largest(const float* row, long long pitch
     }
     auto collect = [&](bool mine, unsigned long long bound) {
         if (mine)
-            for_own_logits(row, pitch, [&](long long at, const float4& v) {
+            for_own_logits<THREADS>(row, pitch, [&](long long at, const float4& v) {
                 const float z[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -2207,7 +2211,7 @@ __device__ __forceinline__ void select_largest(const float* row, long long pitch
             if (tid == 0) sh.count = 0;
             __syncthreads();
             int c = 0;
-            for_own_logits(row, pitch, [&](long long at, const float4& v) {
+            for_own_logits<THREADS>(row, pitch, [&](long long at, const float4& v) {
                 const float z[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
                 for (int j = 0; j < 4; ++j) c += z[j] > -INFINITY && at + j < V && logit_rank(z[j], static_cast<uint32_t>(at + j)) >= T1 ? 1 : 0;
@@ -2226,11 +2230,11 @@ __device__ __forceinline__ void select_largest(const float* row, long long pitch
         collect(true, T64);
     }
     const int n = sh.n;
-    for (int j = n + tid; j < K; j += ROW_THREADS) {
+    for (int j = n + tid; j < K; j += THREADS) {
         tok[j] = 0;
         val[j] = -INFINITY;
     }
-    for (int e = warp; e < n; e += ROW_WARPS) {
+    for (int e = warp; e < n; e += THREADS / 32) {
         const unsigned long long v = sh.pool[e];
         int rank = 0;
         for (int i = lane; i < n; i += 32) rank += sh.pool[i] > v ? 1 : 0;
@@ -2243,8 +2247,8 @@ __device__ __forceinline__ void select_largest(const float* row, long long pitch
     __syncthreads();
 }
 
-template <int OBJ>
-__global__ void __launch_bounds__(ROW_THREADS) row_kernel(const __grid_constant__ RowParams p) {
+template <int OBJ, int THREADS>
+__global__ void __launch_bounds__(THREADS) row_kernel(const __grid_constant__ RowParams p) {
     __shared__ RowShared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int row = blockIdx.x;
@@ -2256,15 +2260,15 @@ __global__ void __launch_bounds__(ROW_THREADS) row_kernel(const __grid_constant_
     float* q = p.q + static_cast<long long>(row) * p.idx_pitch;
 
     float m_t = -INFINITY, s_t = 0.f, m_d = -INFINITY, s_d = 0.f, lse_t = 0.f, lse_d = 0.f;
-    if (trow) own_stats(trow, p.pitch, m_t, s_t);
-    if (zrow) own_stats(zrow, p.pitch, m_d, s_d);
-    if (trow) lse_t = block_lse(m_t, s_t, sh.red);
-    if (zrow) lse_d = block_lse(m_d, s_d, sh.red + 2);
+    if (trow) own_stats<THREADS>(trow, p.pitch, m_t, s_t);
+    if (zrow) own_stats<THREADS>(zrow, p.pitch, m_d, s_d);
+    if (trow) lse_t = block_lse<THREADS>(m_t, s_t, sh.red);
+    if (zrow) lse_d = block_lse<THREADS>(m_d, s_d, sh.red + 2);
     __syncthreads();
 
     int n_tok = K;                        // entries of Omega_hat's list (2K at most for the bi-directional set)
     if (trow) {
-        select_largest(trow, p.pitch, p.V, K, m_t, sh, sh.tok, sh.q);
+        select_largest<THREADS>(trow, p.pitch, p.V, K, m_t, sh, sh.tok, sh.q);
         if (tid < K) sh.q[tid] = expf(sh.q[tid] - lse_t);
         __syncthreads();
         int taken = K;
@@ -2288,7 +2292,7 @@ __global__ void __launch_bounds__(ROW_THREADS) row_kernel(const __grid_constant_
         }
         if (OBJ == ROW_BIDIR) {
             // the draft's own K most probable tokens that are not in the target's set join Omega_hat, in their order
-            select_largest(zrow, p.pitch, p.V, K, m_d, sh, sh.tok_d, sh.z_d);
+            select_largest<THREADS>(zrow, p.pitch, p.V, K, m_d, sh, sh.tok_d, sh.z_d);
             if (warp == 0) {
                 int n = K;
                 for (int j0 = 0; j0 < K; j0 += 32) {
@@ -2356,25 +2360,25 @@ __global__ void __launch_bounds__(ROW_THREADS) row_kernel(const __grid_constant_
     const float g = p.grad_loss ? p.grad_loss[row] : 1.f;
     const float S_q = sh.sum, c = OBJ == ROW_COMBINED ? g * (1.f + p.w * S_q) : OBJ == ROW_BIDIR ? 1.f : g * S_q, shift = -lse_d * LOG2E, shift_t = -lse_t * LOG2E;
     float ce = 0.f;
-    for (long long c0 = 0; c0 < p.pitch; c0 += ROW_STEP) {
+    for (long long c0 = 0; c0 < p.pitch; c0 += ROW_LOADS * THREADS * 4) {
         float4 v[ROW_LOADS];
 #pragma unroll
         for (int u = 0; u < ROW_LOADS; ++u) {
-            const long long at = c0 + (u * ROW_THREADS + tid) * 4;
+            const long long at = c0 + (u * THREADS + tid) * 4;
             if (at < p.pitch) v[u] = *reinterpret_cast<const float4*>(zrow + at);
         }
         float4 t[OBJ == ROW_COMBINED ? ROW_LOADS : 1];
         if (OBJ == ROW_COMBINED) {
 #pragma unroll
             for (int u = 0; u < ROW_LOADS; ++u) {
-                const long long at = c0 + (u * ROW_THREADS + tid) * 4;
+                const long long at = c0 + (u * THREADS + tid) * 4;
                 if (at < p.pitch) t[OBJ == ROW_COMBINED ? u : 0] = *reinterpret_cast<const float4*>(trow + at);
             }
         }
         __syncthreads();
 #pragma unroll
         for (int u = 0; u < ROW_LOADS; ++u) {
-            const long long at = c0 + (u * ROW_THREADS + tid) * 4;
+            const long long at = c0 + (u * THREADS + tid) * 4;
             if (at < p.pitch) {
                 float z[4] = {v[u].x, v[u].y, v[u].z, v[u].w}, o[4];
 #pragma unroll
@@ -2401,7 +2405,7 @@ __global__ void __launch_bounds__(ROW_THREADS) row_kernel(const __grid_constant_
     if (OBJ == ROW_BIDIR) {
         if (tid == 0) p.coef_out[row] = g * S_q;
         const int n = sh.count;
-        for (int k0 = tid * 8; k0 < p.d; k0 += ROW_THREADS * 8) {
+        for (int k0 = tid * 8; k0 < p.d; k0 += THREADS * 8) {
             float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll 4
             for (int j = 0; j < n; ++j) {
@@ -2427,7 +2431,7 @@ __global__ void __launch_bounds__(ROW_THREADS) row_kernel(const __grid_constant_
         drow[sh.tok[tid]] = __float2bfloat16_rn(o);
     }
     if (OBJ == ROW_COMBINED && warp == 0) {
-        float v = sh.red[0][lane];
+        float v = lane < THREADS / 32 ? sh.red[0][lane] : 0.f;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if (lane == 0) p.loss_ce[row] = v;

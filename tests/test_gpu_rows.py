@@ -21,7 +21,7 @@ def _cpu(out):
 
 # fewer logits than threads, a thread's first piece and one logit more, a step of the pass and one logit more, all K tokens
 @pytest.mark.parametrize("N,d,V,K", [(1, 64, 1024, 256), (3, 64, 300, 256), (5, 8, 9, 5), (7, 16, 4097, 128),
-                                     (64, 64, 16384, 17), (65, 72, 16385, 100), (128, 64, 33000, 1)])
+                                     (64, 64, 16384, 17), (65, 72, 16385, 100), (128, 64, 33000, 1), (33, 72, 1024, 64), (20, 64, 1024, 65)])
 def test_rows_against_the_oracle(N, d, V, K):
     hass = _hass()
     dev = torch.device("cuda:0")
