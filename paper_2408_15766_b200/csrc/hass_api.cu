@@ -820,6 +820,10 @@ constexpr long long kNarrowBidirBytes = 128 << 10;
 // sweep asks the L2 to keep this much of W, its last k blocks, and to let the rest go first: 61 rows x 4096 x 32000
 // (262 MB) 112 -> 104 us; with 48 and 80 MB the same.
 constexpr long long kKeepBytes = 64ll << 20;
+// From this size of W on the kernels of such a call let the next one's blocks in when they end: blocks that wait beside a
+// kernel bound by reading W cost it time (61 rows x 4096 x 32000 103.6 -> 101.3 us, 99 draft rows 114.3 -> 109.7, 100 rows 142.9 -> 138.4);
+// with a head of 0.5 MB their early start is worth more (64 rows x 256 x 1024 24.4 us early, 24.8 late).
+constexpr long long kLateBytes = 16ll << 20;
 struct NarrowRoom {
     float* z = nullptr;      // [N, p_pitch], or nullptr: no room
     float* zt = nullptr;     // [N, p_pitch]
@@ -866,6 +870,7 @@ static int narrow_sweep(const void* H0, const void* H1, const void* W, int N, lo
     p.keep_from = p.k_blocks - static_cast<int>(p.k_blocks * std::min(1., static_cast<double>(kKeepBytes) / (2. * static_cast<double>(V) * static_cast<double>(d))));
     p.status = reinterpret_cast<unsigned int*>(ws + L.status);
     p.clear_status = 1;
+    p.release_late = V * d * 2 >= kLateBytes ? 1 : 0;
     return launch_gemm<MODE_LOGITS>(p, st, H1 ? KIND_STATS : KIND_STATS_DRAFT);
 }
 
@@ -914,6 +919,7 @@ static int narrow_impl(int objective, bool with_target, const void* H_t, const v
     r.lse_d = lse_d;
     r.loss = loss;
     r.make_dz = dH_d != nullptr ? 1 : 0;
+    r.release_late = V * d * 2 >= kLateBytes ? 1 : 0;
     if (cmb) {
         r.w = cmb->w;
         r.loss_ce = cmb->loss_ce;
@@ -947,6 +953,7 @@ static int narrow_impl(int objective, bool with_target, const void* H_t, const v
     o.out_align32 = ((reinterpret_cast<uintptr_t>(dH_d) | static_cast<uintptr_t>(d * (dH_dtype == HASS_FP32 ? 4 : 2))) & 31u) == 0 ? 1 : 0;
     o.out_pitch = d;
     o.kept = 1;
+    o.release_late = r.release_late;
     o.coef = r.coef_out;
     o.sparse = r.sparse_out;
     o.status = reinterpret_cast<unsigned int*>(ws + L.status);

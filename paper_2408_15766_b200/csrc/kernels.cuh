@@ -133,6 +133,7 @@ struct GemmParams {
     long long z_pitch;
     int keep_from;         // k block from which on this sweep asks the L2 to keep its tiles of B ...
     int kept;              // MODE_OUT: ... whose second reading this is
+    int release_late;      // the next kernel's blocks may start when this one's have ended, not before
     int clear_status;      // the first CTA zeroes the status block (no kernel of the call has run before this one)
     // MODE_OUT. With sparse != nullptr the epilogue computes coef[row] * acc - sparse[local row, :] (row scale
     // and the Omega_hat term of dz_d W, precomputed by finalize); with coef alone coef[row] * acc; with neither
@@ -466,7 +467,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
             tmem_relinquish();
         }
     }
-    if (p.gate == nullptr) wait_previous_kernel();
+    if (p.gate == nullptr) {
+        if (MODE == MODE_LOGITS || MODE == MODE_OUT)
+            wait_previous_kernel(!p.release_late);
+        else
+            wait_previous_kernel();
+    }
     // (A wait of another CTA that ran out would be recorded two seconds later.)
     if (MODE == MODE_LOGITS && p.clear_status && blockIdx.x == 0 && threadIdx.x < 64) p.status[threadIdx.x] = 0u;
     tc_fence_before_sync();
@@ -2067,6 +2073,7 @@ struct RowParams {
     float* lse_d;
     float* loss;
     int make_dz;
+    int release_late;      // as in GemmParams
     float w;               // ROW_COMBINED
     float* loss_ce;
     const __nv_bfloat16* W;      // ROW_BIDIR: [V, d]
@@ -2253,7 +2260,7 @@ __global__ void __launch_bounds__(THREADS) row_kernel(const __grid_constant__ Ro
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int row = blockIdx.x;
     const int K = p.K;
-    wait_previous_kernel();
+    wait_previous_kernel(!p.release_late);
     float* zrow = p.z != nullptr ? p.z + static_cast<long long>(row) * p.pitch : nullptr;
     const float* trow = p.zt != nullptr ? p.zt + static_cast<long long>(row) * p.pitch : nullptr;
     int* idx = p.idx + static_cast<long long>(row) * p.idx_pitch;
