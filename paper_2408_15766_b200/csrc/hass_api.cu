@@ -113,6 +113,7 @@ static int device_info(DeviceInfo* out) {
                                     gemm_kernel<MODE_STATS, TOPK_NONE, 1>, gemm_kernel<MODE_STATS, TOPK_NONE, 2>,
                                     gemm_kernel<MODE_PROBS, TOPK_BUF, 1>,  gemm_kernel<MODE_PROBS, TOPK_BUF, 2>,
                                     gemm_kernel<MODE_OUT, TOPK_BUF, 1>,    gemm_kernel<MODE_OUT, TOPK_BUF, 2>,
+                                    gemm_kernel<MODE_OUT, TOPK_NONE, 1>,   gemm_kernel<MODE_OUT, TOPK_NONE, 2>,
                                     gemm_kernel<MODE_LOGITS, TOPK_BUF, 1>, gemm_kernel<MODE_LOGITS, TOPK_BUF, 2>};
             cudaError_t e3 = cudaSuccess;
             for (GemmFn f : gemms)
@@ -486,6 +487,8 @@ static int launch_gemm(const GemmParams& p, cudaStream_t st, int kind = -1) {
         fn = pair ? gemm_kernel<MODE_STATS, TOPK_NONE, 2> : gemm_kernel<MODE_STATS, TOPK_NONE, 1>;
     else if (MODE == MODE_STATS && p.K <= K_REG)
         fn = pair ? gemm_kernel<MODE_STATS, TOPK_REG, 2> : gemm_kernel<MODE_STATS, TOPK_REG, 1>;
+    else if (MODE == MODE_OUT && p.kept)
+        fn = pair ? gemm_kernel<MODE_OUT, TOPK_NONE, 2> : gemm_kernel<MODE_OUT, TOPK_NONE, 1>;
     else
         fn = pair ? gemm_kernel<MODE, TOPK_BUF, 2> : gemm_kernel<MODE, TOPK_BUF, 1>;
     return launch(fn, p.sched.max_ctas, NUM_THREADS, SMEM_BYTES, st, MODE == MODE_OUT && p.plan.cluster > 1 ? p.plan.cluster : pair ? 2 : 1, p);

@@ -132,7 +132,7 @@ struct GemmParams {
     float* zt_out;
     long long z_pitch;
     int keep_from;         // k block from which on this sweep asks the L2 to keep its tiles of B ...
-    int kept;              // MODE_OUT: ... whose second reading this is
+    int kept;              // MODE_OUT: ... whose second reading this is (host: selects the instantiation)
     int release_late;      // the next kernel's blocks may start when this one's have ended, not before
     int clear_status;      // the first CTA zeroes the status block (no kernel of the call has run before this one)
     // MODE_OUT. With sparse != nullptr the epilogue computes coef[row] * acc - sparse[local row, :] (row scale
@@ -412,6 +412,9 @@ __device__ __forceinline__ void finish_out4(const GemmParams& p, float4 a, int l
 template <int MODE, int TOPK, int CG>
 __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_constant__ GemmParams p) {
     constexpr bool B_MN_MAJOR = (MODE == MODE_OUT);
+    // MODE_OUT after a MODE_LOGITS sweep of the same B, as an instantiation of its own (as a condition in the producer's loop it
+    // cost the other calls 3-6 % of this kernel: 517 rows x 4096 x 128256 560 -> 576-595 us)
+    constexpr bool KEPT = MODE == MODE_OUT && TOPK == TOPK_NONE;
     // conditional launch (the second pass that follows every spilling call): nothing to do unless the first reported a
     // row beyond its exponent range
     if (p.gate != nullptr) {
@@ -468,7 +471,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
         }
     }
     if (p.gate == nullptr) {
-        if (MODE == MODE_LOGITS || MODE == MODE_OUT)
+        if (MODE == MODE_LOGITS || KEPT)
             wait_previous_kernel(!p.release_late);
         else
             wait_previous_kernel();
@@ -528,7 +531,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
         if (lane == 0) {
             int stage = 0;
             uint32_t phase = 0;
-            const uint64_t keep = l2_evict_last(), drop = l2_evict_first();
+            const uint64_t keep = MODE == MODE_LOGITS ? l2_evict_last() : 0ull, drop = MODE == MODE_LOGITS || KEPT ? l2_evict_first() : 0ull;
             for_each_item([&](int rt, int ln, int S, int, int kb0, int kb1) {
                 const bool second = (MODE == MODE_STATS || MODE == MODE_LOGITS) && rt >= p.row_tiles0;
                 const CUtensorMap* tmA = second ? &p.tmA1 : &p.tmA0;
@@ -549,7 +552,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                                 tma_load_2d(dst, tm, bar, x, y);
                         };
                         auto load_b = [&](uint32_t dst, int x, int y) {
-                            if (MODE == MODE_LOGITS || (MODE == MODE_OUT && p.kept)) {
+                            if (MODE == MODE_LOGITS || KEPT) {
                                 const uint64_t policy = MODE == MODE_LOGITS && kb >= p.keep_from ? keep : drop;
                                 if (CG == 2)
                                     tma_load_2d_pair_hint(dst, &p.tmB, bar, x, y, policy);
