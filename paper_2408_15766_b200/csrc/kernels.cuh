@@ -2009,8 +2009,8 @@ __global__ void __launch_bounds__(256) loss_patch_kernel(const __grid_constant__
     const long long ro = static_cast<long long>(row) * K;
     float S_q = 0.f, loss = 0.f;
     for (int j = lane; j < K; j += 32) {
-        if (p.sidx[ro + j] != INT_MAX) {
-            const float qv = p.sq[ro + j];
+        const float qv = p.sq[ro + j];
+        if (p.sidx[ro + j] != INT_MAX && qv != 0.f) {      // (0 log p = 0, where z_d = -inf too)
             S_q += qv;
             loss += qv * (lse_d - p.cap_z[ro + j]);     // -q log p,  log p = z_d - lse_d
         }
@@ -2031,7 +2031,9 @@ __global__ void __launch_bounds__(256) loss_patch_kernel(const __grid_constant__
         __nv_bfloat16* prow = p.P + static_cast<long long>(local) * p.p_pitch;
         for (int j = lane; j < K; j += 32) {
             const int tok = p.sidx[ro + j];
-            if (tok != INT_MAX) prow[tok] = __float2bfloat16_rn(expf(p.cap_z[ro + j] - m_spill) - p.sq[ro + j] / S_q * sum);
+            const float qv = p.sq[ro + j];
+            // (q = 0: the spilled value stays; a set filled up with token 0 may name it twice, and an entry has one writer)
+            if (tok != INT_MAX && qv != 0.f) prow[tok] = __float2bfloat16_rn(expf(p.cap_z[ro + j] - m_spill) - qv / S_q * sum);
         }
     }
 }
@@ -2279,7 +2281,7 @@ __global__ void __launch_bounds__(THREADS) row_kernel(const __grid_constant__ Ro
     int n_tok = K;                        // entries of Omega_hat's list (2K at most for the bi-directional set)
     if (trow) {
         select_largest<THREADS>(trow, p.pitch, p.V, K, m_t, sh, sh.tok, sh.q);
-        if (tid < K) sh.q[tid] = expf(sh.q[tid] - lse_t);
+        if (tid < K) sh.q[tid] = sh.q[tid] > -INFINITY ? expf(sh.q[tid] - lse_t) : 0.f;      // (-inf: filled up)
         __syncthreads();
         int taken = K;
         if (p.top_p > 0.f) {
@@ -2349,7 +2351,7 @@ __global__ void __launch_bounds__(THREADS) row_kernel(const __grid_constant__ Ro
     if (warp == 0) {
         float S_q = 0.f, loss = 0.f;
         for (int j = lane; j < n_tok; j += 32) {
-            if (sh.tok[j] < 0) continue;
+            if (sh.tok[j] < 0 || sh.q[j] == 0.f) continue;      // (0 log p = 0, where z_d = -inf too)
             S_q += sh.q[j];
             loss += sh.q[j] * (lse_d - sh.z[j]);      // -q log p,  log p = z_d - lse_d
         }
@@ -2432,7 +2434,9 @@ __global__ void __launch_bounds__(THREADS) row_kernel(const __grid_constant__ Ro
         return;
     }
     __syncthreads();
-    if (tid < n_tok && sh.tok[tid] >= 0) {
+    // Tokens of q = 0 keep the dense value: the one that fills up a set of fewer than K logits above -inf (token 0) may be in it
+    // already, and an entry has one writer.
+    if (tid < n_tok && sh.tok[tid] >= 0 && sh.q[tid] != 0.f) {
         float o = c * ex2(fmaf(sh.z[tid], LOG2E, shift));
         if (OBJ == ROW_COMBINED)
             o -= g * ex2(fmaf(trow[sh.tok[tid]], LOG2E, shift_t)) + g * p.w * sh.q[tid];

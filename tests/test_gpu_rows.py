@@ -70,3 +70,40 @@ def test_variants_of_few_rows_against_the_oracle(N, d, V, K):
         out = hass.variant_distill_fwd_bwd(*args, variant, param, dH_dtype=hass.HASS_FP32)
         hass.check(out["workspace"])
         print(which, compare_variant(inp.H_t, inp.H_d[0], inp.W, K, which, param, _cpu(out)))
+
+
+# 40 rows: the row kernel; 200: the spill and its patch. A vocabulary masked by a bias column of -inf, so that fewer than K tokens
+# are left: token 0 with q = 0 fills the set up, whether it is one of those left or not.
+@pytest.mark.parametrize("N,V", [(40, 700), (200, 30)])
+@pytest.mark.parametrize("K", [10, 20])
+@pytest.mark.parametrize("left", [(0, 3, 7, 11, 12, 29), (5, 6, 17, 28)])
+def test_fewer_than_k_tokens_above_minus_infinity(N, V, K, left):
+    hass = _hass()
+    d = 64
+    inp = hi.make_custom(N, d, V, K, seed=N + K, sigma_w=0.5)
+    H_t, H_d, W = inp.H_t.clone(), inp.H_d[0].clone(), inp.W.clone()
+    H_t[:, 0] = H_d[:, 0] = 1.0
+    masked = torch.ones(V, dtype=torch.bool)
+    masked[list(left)] = False
+    W[masked, 0] = -float("inf")
+    z_t, z_d = ((H[:, 1:].double() @ W[:, 1:].double().T + (H[:, :1].double() @ W[:, :1].double().T)).masked_fill(masked, -np.inf) for H in (H_t, H_d))
+    q, idx = z_t.softmax(1).topk(len(left), dim=1)
+    log_p = z_d.log_softmax(1)
+    dz = q.sum(1, keepdim=True) * log_p.exp()
+    dz.scatter_add_(1, idx, -q)
+    want = {"loss": -(q * log_p.gather(1, idx)).sum(1), "lse_t": z_t.logsumexp(1), "lse_d": z_d.logsumexp(1), "dH_d": dz @ W[:, 1:].double()}
+    dev = torch.device("cuda:0")
+    args = H_t.to(dev), H_d.to(dev), W.to(dev), K
+    out = hass.topk_distill_fwd_bwd(*args, dH_dtype=hass.HASS_FP32)
+    hass.check(out["workspace"])
+    draft = hass.topk_distill_fwd_bwd_draft(args[1], args[2], out["topk_idx"], out["topk_q"], dH_dtype=hass.HASS_FP32)
+    hass.check(draft["workspace"])
+    assert torch.equal(out["topk_idx"].cpu()[:, :len(left)].long(), idx)
+    assert (out["topk_idx"].cpu()[:, len(left):] == 0).all() and (out["topk_q"].cpu()[:, len(left):] == 0).all()
+    for got in (_cpu(out), _cpu(draft)):
+        for k in ("loss", "lse_t", "lse_d"):
+            # fp32 sums of 64 products of up to 8, as in the parity tests
+            assert k not in got or (got[k].double() - want[k]).abs().max() <= 1e-4, k
+        # (column 0: the weights of the masked tokens are zero times -inf) dz_d in bf16, 2^-9 of its largest entry or so
+        err = (got["dH_d"][:, 1:].double() - want["dH_d"]).abs().max()
+        assert err <= 1e-2 * want["dH_d"].abs().max()
