@@ -2050,7 +2050,7 @@ __global__ void __launch_bounds__(256) loss_patch_kernel(const __grid_constant__
 //
 // The K largest of a row: a thread's largest logit is at hand after the pass for lse, and the K-th largest of these 1024
 // maxima bounds the row's K-th largest from below. Little more than K logits reach it; the threads that hold them read their
-// share again and put them into a pool in shared memory, where each counts those above it.
+// share again and put them into a pool in shared memory, where each counts those above it (more than it takes: collect_from_many).
 // Bound by the latency of two passes over rows of 4 V bytes in L2: 1024 threads with ROW_LOADS 16-byte loads each in flight.
 // Rows of up to ROW_SMALL logits, one load each for 256 threads, are bound by the barriers instead and take 256: 64 rows x 256 x
 // 1024 25.9 -> 25.0 us per call, 104 rows 26.8 -> 25.6. (Of 2000 logits, K = 30 22.2 -> 22.5, 4096, K = 64 34.1 -> 36.2. K is a
@@ -2097,6 +2097,7 @@ struct RowShared {
     float z_d[K_CAP];
     float sum;
     int n, count;
+    int reach[3], equal[32];
 };
 
 // One logit as a number: larger = larger logit, lower token id first among equal ones (-0 and +0 are equal).
@@ -2104,10 +2105,15 @@ __device__ __forceinline__ unsigned long long logit_rank(float z, uint32_t id) {
     return cand_rank(ordered_key(__float_as_uint(z + 0.f)), id);
 }
 
-// f(first column, its four logits) for every piece of the row that this thread owns
-template <int THREADS, typename F>
-__device__ __forceinline__ void for_own_logits(const float* row, long long pitch, F&& f) {
-    for (long long c0 = threadIdx.x * 4; c0 < pitch; c0 += ROW_LOADS * THREADS * 4) {
+// Whether column `at` of a row, with logit z, is a token whose logit reaches the ordered key `bound` (> 0)
+__device__ __forceinline__ bool reaches(float z, long long at, int V, uint32_t bound) {
+    return z > -INFINITY && at < V && ordered_key(__float_as_uint(z + 0.f)) >= bound;
+}
+
+// f(first column, its four logits) for every piece of the row that this thread owns, ROW_LOADS at a time while go()
+template <int THREADS, typename F, typename G>
+__device__ __forceinline__ void for_own_logits_while(const float* row, long long pitch, F&& f, G&& go) {
+    for (long long c0 = threadIdx.x * 4; c0 < pitch && go(); c0 += ROW_LOADS * THREADS * 4) {
         float4 v[ROW_LOADS];
 #pragma unroll
         for (int u = 0; u < ROW_LOADS; ++u) {
@@ -2120,6 +2126,10 @@ __device__ __forceinline__ void for_own_logits(const float* row, long long pitch
             if (at < pitch) f(at, v[u]);
         }
     }
+}
+template <int THREADS, typename F>
+__device__ __forceinline__ void for_own_logits(const float* row, long long pitch, F&& f) {
+    for_own_logits_while<THREADS>(row, pitch, f, [] { return true; });
 }
 
 // This thread's largest logit m and sum of 2^((z - m) log2e)
@@ -2166,6 +2176,129 @@ __device__ __forceinline__ float block_lse(float m, float s, float (*red)[32]) {
     return top + logf(s);
 }
 
+// Logits that are ranked one against all others: those of K + ROW_SLACK pieces of four. (1024 equal ones of a row of zeros fit the
+// pool; ranking them took 55 us.)
+__device__ __forceinline__ int pool_room(int K) { return min(4 * (K + ROW_SLACK), ROW_POOL); }
+
+// Block-collective: the logits that reach `bound` into the pool, by the threads whose maximum `key` does; given up when they are
+// more than `room` (then sh.n > room).
+template <int THREADS>
+__device__ __forceinline__ void collect(const float* row, long long pitch, int V, uint32_t key, uint32_t bound, int room, RowShared& sh) {
+    auto full = [&] { return *static_cast<volatile int*>(&sh.n) > room; };
+    if (key >= bound)
+        for_own_logits_while<THREADS>(row, pitch, [&](long long at, const float4& v) {
+            const float z[4] = {v.x, v.y, v.z, v.w};
+            if (!reaches(fmaxf(fmax3(z[0], z[1], z[2]), z[3]), at, V, bound)) return;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (reaches(z[j], at + j, V, bound)) {
+                    const int pos = atomicAdd(&sh.n, 1);
+                    if (pos < room) sh.pool[pos] = logit_rank(z[j], static_cast<uint32_t>(at + j));
+                }
+        }, [&] { return !full(); });
+    __syncthreads();
+}
+
+// Block-collective: more logits reach T, a bound of the K-th largest, than the pool takes (hi: the largest). As a rule they are equal
+// (a row of zeros has nothing else), and T is the K-th largest logit itself: known without a look where it is also the largest,
+// else from one count. Otherwise its bits are searched two per pass over the row, until it is found or the pool holds what
+// reaches it. Of logits equal to the K-th the first in token order are taken, and no more of the row is read than that takes.
+// Half of 61 rows x 4096 x 32000 zeros: 346 -> 117 us per call, as without zeros (116), of 8 rows x 128256 1140 -> 370, of 64 rows x 256 x
+// 1024 83 -> 30 (a search of token ids bit by bit, a pass over the row for each, and 1024 equal logits ranked).
+// Returns the entries left in the pool. (A function of its own: in line it costs row_kernel registers that it does not have.)
+template <int THREADS>
+__device__ __noinline__ int collect_from_many(const float* row, long long pitch, int V, int K, uint32_t key, uint32_t T, uint32_t hi, RowShared& sh) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    auto count = [&](uint32_t t1, uint32_t t2, uint32_t t3) {
+        __syncthreads();
+        if (tid < 3) sh.reach[tid] = 0;
+        __syncthreads();
+        int c1 = 0, c2 = 0, c3 = 0;
+        for_own_logits<THREADS>(row, pitch, [&](long long at, const float4& v) {
+            const float z[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                c1 += reaches(z[j], at + j, V, t1) ? 1 : 0;
+                c2 += reaches(z[j], at + j, V, t2) ? 1 : 0;
+                c3 += reaches(z[j], at + j, V, t3) ? 1 : 0;
+            }
+        });
+        c1 = __reduce_add_sync(0xffffffffu, c1);
+        c2 = __reduce_add_sync(0xffffffffu, c2);
+        c3 = __reduce_add_sync(0xffffffffu, c3);
+        if (lane == 0) {
+            atomicAdd(&sh.reach[0], c1);
+            atomicAdd(&sh.reach[1], c2);
+            atomicAdd(&sh.reach[2], c3);
+        }
+        __syncthreads();
+    };
+    bool exact = T == hi;
+    if (!exact) {
+        count(T + 1u, T + 1u, T + 1u);
+        exact = sh.reach[0] < K;
+    }
+    if (!exact) {
+        int bit = 32 - __clz(hi ^ T);
+        bit += bit & 1;
+        T = bit < 32 ? hi >> bit << bit : 0u;
+        exact = true;
+        for (bit -= 2; bit >= 0; bit -= 2) {
+            const uint32_t t1 = T | (1u << bit), t2 = T | (2u << bit), t3 = T | (3u << bit);
+            count(t1, t2, t3);
+            const int c1 = sh.reach[0], c2 = sh.reach[1], c3 = sh.reach[2];
+            const int c = c3 >= K ? c3 : c2 >= K ? c2 : c1 >= K ? c1 : INT_MAX;
+            T = c3 >= K ? t3 : c2 >= K ? t2 : c1 >= K ? t1 : T;
+            if (c <= pool_room(K)) {
+                exact = false;
+                break;
+            }
+        }
+    }
+    __syncthreads();
+    if (tid == 0) sh.n = 0;
+    __syncthreads();
+    collect<THREADS>(row, pitch, V, key, exact ? T + 1u : T, pool_room(K), sh);
+    int n = sh.n;
+    if (exact) {
+        // fewer than K lie above it; of those equal to it the first in token order
+        int taken = n;
+        for (long long c0 = 0; c0 < pitch && taken < K; c0 += THREADS * 4) {
+            const long long at = c0 + tid * 4;
+            const float4 v = at < pitch ? *reinterpret_cast<const float4*>(row + at) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+            const float z[4] = {v.x, v.y, v.z, v.w};
+            bool in[4];
+            int c = 0;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                in[j] = reaches(z[j], at + j, V, T) && !reaches(z[j], at + j, V, T + 1u);
+                c += in[j] ? 1 : 0;
+            }
+            int pos = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int before = __shfl_up_sync(0xffffffffu, pos, o);
+                if (lane >= o) pos += before;
+            }
+            __syncthreads();
+            if (lane == 31) sh.equal[warp] = pos;
+            __syncthreads();
+            const int of_warp = lane < THREADS / 32 ? sh.equal[lane] : 0;
+            pos += taken - c + __reduce_add_sync(0xffffffffu, lane < warp ? of_warp : 0);
+            taken += __reduce_add_sync(0xffffffffu, of_warp);
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (in[j]) {
+                    if (pos < K) sh.pool[pos] = logit_rank(z[j], static_cast<uint32_t>(at + j));
+                    ++pos;
+                }
+        }
+        n = taken < K ? taken : K;
+        __syncthreads();
+    }
+    return n;
+}
+
 // Block-collective: the K largest logits of the row, in descending order (lower token id first among equal ones), into
 // tok / val; m = this thread's largest logit. Fewer than K logits above -inf: the rest is token 0 at -inf.
 template <int THREADS>
@@ -2179,11 +2312,11 @@ __device__ __forceinline__ void select_largest(const float* row, long long pitch
     }
     if (tid == 0) sh.n = 0;
     const int groups = __syncthreads_count(key != 0u);
+    const uint32_t hi = __reduce_max_sync(0xffffffffu, lane < THREADS / 32 ? __float_as_uint(sh.red[0][lane]) : 0u);
     uint32_t T = 1u;
     if (groups >= K) {
         // the K-th largest maximum, or a value below it that at most K + ROW_SLACK maxima reach, from the highest bit in which
         // the maxima differ on
-        const uint32_t hi = __reduce_max_sync(0xffffffffu, lane < THREADS / 32 ? __float_as_uint(sh.red[0][lane]) : 0u);
         const uint32_t lo = __reduce_min_sync(0xffffffffu, lane < THREADS / 32 ? sh.key_min[lane] : 0xffffffffu);
         int bit = 32 - __clz(hi ^ lo);
         T = bit < 32 ? hi >> bit << bit : 0u;
@@ -2197,51 +2330,9 @@ __device__ __forceinline__ void select_largest(const float* row, long long pitch
         }
         T = max(T, 1u);
     }
-    auto collect = [&](bool mine, unsigned long long bound) {
-        if (mine)
-            for_own_logits<THREADS>(row, pitch, [&](long long at, const float4& v) {
-                const float z[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const unsigned long long r = logit_rank(z[j], static_cast<uint32_t>(at + j));
-                    if (z[j] > -INFINITY && at + j < V && r >= bound) {
-                        const int pos = atomicAdd(&sh.n, 1);
-                        if (pos < ROW_POOL) sh.pool[pos] = r;
-                    }
-                }
-            });
-        __syncthreads();
-    };
-    collect(key >= T, static_cast<unsigned long long>(T) << 32);
-    if (sh.n > ROW_POOL) {
-        // Many equal logits: the bound is searched over logits and token ids, one bit per pass over the row, until the pool
-        // holds what reaches it.
-        unsigned long long T64 = 0ull;
-        for (int bit = 63; bit >= 0; --bit) {
-            const unsigned long long T1 = T64 | (1ull << bit);
-            __syncthreads();
-            if (tid == 0) sh.count = 0;
-            __syncthreads();
-            int c = 0;
-            for_own_logits<THREADS>(row, pitch, [&](long long at, const float4& v) {
-                const float z[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j) c += z[j] > -INFINITY && at + j < V && logit_rank(z[j], static_cast<uint32_t>(at + j)) >= T1 ? 1 : 0;
-            });
-            c = __reduce_add_sync(0xffffffffu, c);
-            if (lane == 0) atomicAdd(&sh.count, c);
-            __syncthreads();
-            if (sh.count >= K) {
-                T64 = T1;
-                if (sh.count <= ROW_POOL) break;
-            }
-        }
-        __syncthreads();
-        if (tid == 0) sh.n = 0;
-        __syncthreads();
-        collect(true, T64);
-    }
-    const int n = sh.n;
+    collect<THREADS>(row, pitch, V, key, T, pool_room(K), sh);
+    int n = sh.n;
+    if (n > pool_room(K)) n = collect_from_many<THREADS>(row, pitch, V, K, key, T, hi, sh);
     for (int j = n + tid; j < K; j += THREADS) {
         tok[j] = 0;
         val[j] = -INFINITY;

@@ -107,3 +107,70 @@ def test_fewer_than_k_tokens_above_minus_infinity(N, V, K, left):
         # (column 0: the weights of the masked tokens are zero times -inf) dz_d in bf16, 2^-9 of its largest entry or so
         err = (got["dH_d"][:, 1:].double() - want["dH_d"]).abs().max()
         assert err <= 1e-2 * want["dH_d"].abs().max()
+
+
+def _levels(V, pattern):
+    """Logits of a vocabulary at which the bound from the threads' maxima (thread (v // 4) % 1024 owns token v) admits more than the
+    pool holds: three digits of up to eight bits each, so that every sum below is exact."""
+    v = torch.arange(V)
+    owner = v // 4 % 1024
+    if pattern == "few above":            # 41 distinct logits above a level that all others share
+        hi = torch.where(v % 977 == 5, 2.0, 1.0)
+        return hi, torch.where(v % 977 == 5, (v // 977) / 64.0, torch.zeros(V))
+    if pattern == "by thread":            # what a thread owns lies close together, the threads apart; nearly no ties
+        return (owner // 16).float(), owner % 16 / 16.0 + v % 4 / 128.0 + (v // 4096) / 1024.0 % 0.0078125
+    if pattern == "two levels":           # the largest logit five times in all, then every second token alike
+        return torch.where(v % 8000 == 4001, 3.0, 1.0), (v % 2) / 2.0
+    hi = torch.where(owner % 10 == 3, 1.0, -float("inf"))      # "masked": a tenth of the threads has all there is
+    return hi, v % 61 / 64.0
+
+
+@pytest.mark.parametrize("K", [1, 64, 256])
+@pytest.mark.parametrize("pattern", ["few above", "by thread", "two levels", "masked"])
+def test_more_logits_at_the_bound_than_the_pool_holds(pattern, K):
+    hass = _hass()
+    dev = torch.device("cuda:0")
+    V, d = 40001, 64
+    W = torch.zeros(V, d, dtype=torch.bfloat16)
+    hi, lo = _levels(V, pattern)
+    W[:, 0] = hi.to(torch.bfloat16)
+    W[:, 1] = lo.to(torch.bfloat16)
+    W[:, 2] = (lo - lo.to(torch.bfloat16).float()).to(torch.bfloat16)
+    H = torch.zeros(2, d, dtype=torch.bfloat16)
+    H[:, :3] = 1.0
+    H[1, 1:] = 0.0                        # the second row has the first digit alone: ties everywhere
+    z = H[:, 1:].double() @ W[:, 1:].double().T + W[:, 0].double()
+    want = z.sort(dim=1, descending=True, stable=True).indices[:, :K]
+    out = hass.topk_distill_fwd(H.to(dev), H.to(dev), W.to(dev), K)
+    hass.check(out["workspace"])
+    assert torch.equal(out["topk_idx"].cpu().long(), want)
+
+
+@pytest.mark.parametrize("d,V,K", [(256, 128256, 10), (256, 128256, 64), (256, 1024, 10)])
+def test_rows_of_zeros_take_no_longer(d, V, K):
+    """Feature rows of zeros (padding) have V equal logits. Where token ids are searched bit by bit, they take a call of 128256 tokens
+    from 114 to 878 us, and ranking 1024 equal logits one of 1024 from 30 to 83; with one look at the first tokens neither changes."""
+    hass = _hass()
+    dev = torch.device("cuda:0")
+    inp = hi.make_custom(8, d, V, K, seed=1, sigma_w=0.05)
+    H_t, H_d, W = inp.H_t.to(dev), inp.H_d[0].to(dev), inp.W.to(dev)
+    ws = torch.empty(hass.topk_distill_workspace_bytes(8, d, V, K), dtype=torch.uint8, device=dev)
+
+    def median_us():
+        times = []
+        for _ in range(40):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            hass.topk_distill_fwd_bwd(H_t, H_d, W, K, workspace=ws)
+            b.record()
+            b.synchronize()
+            times.append(a.elapsed_time(b) * 1e3)
+        return sorted(times[10:])[15]
+
+    plain = median_us()
+    H_t[4:] = 0
+    H_d[4:] = 0
+    zeros = median_us()
+    hass.check(ws)
+    print(plain, zeros)
+    assert zeros <= 1.25 * plain + 20.0
