@@ -820,8 +820,9 @@ struct Combined {
 constexpr long long kNarrowBidirBytes = 128 << 10;
 // The second GEMM of such a call reads W again. The L2 (126 MB) would hold the end of the first reading, but that is the last
 // k blocks of all columns, and the second reading, which walks the other way, evicts them before it comes to them. So the
-// sweep asks the L2 to keep this much of W, its last k blocks, and to let the rest go first: 61 rows x 4096 x 32000
-// (262 MB) 112 -> 104 us; with 48 and 80 MB the same.
+// sweep lets this much of W, its last k blocks, into the L2 like any other data and asks that the rest go first: 61 rows x 4096 x 32000
+// (262 MB) from a cold L2 129 -> 116 us, 100 rows 137 -> 125. Asking the L2 to hold those blocks longest (evict_last) gave the same, 117
+// and 127, but they stayed when the call was over: a pass over 80 MB of the caller's took 26.6 us after a call instead of 21.5.
 constexpr long long kKeepBytes = 64ll << 20;
 // From this size of W on the kernels of such a call let the next one's blocks in when they end: blocks that wait beside a
 // kernel bound by reading W cost it time (61 rows x 4096 x 32000 103.6 -> 101.3 us, 99 draft rows 114.3 -> 109.7, 100 rows 142.9 -> 138.4);

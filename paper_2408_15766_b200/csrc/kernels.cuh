@@ -131,8 +131,8 @@ struct GemmParams {
     float* z_out;
     float* zt_out;
     long long z_pitch;
-    int keep_from;         // k block from which on this sweep asks the L2 to keep its tiles of B ...
-    int kept;              // MODE_OUT: ... whose second reading this is (host: selects the instantiation)
+    int keep_from;         // k block from which on the L2 holds this sweep's tiles of B like any other's; those before it go first ...
+    int kept;              // MODE_OUT: ... as all do in the second reading of B, which this is (host: selects the instantiation)
     int release_late;      // the next kernel's blocks may start when this one's have ended, not before
     int clear_status;      // the first CTA zeroes the status block (no kernel of the call has run before this one)
     // MODE_OUT. With sparse != nullptr the epilogue computes coef[row] * acc - sparse[local row, :] (row scale
@@ -531,7 +531,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
         if (lane == 0) {
             int stage = 0;
             uint32_t phase = 0;
-            const uint64_t keep = MODE == MODE_LOGITS ? l2_evict_last() : 0ull, drop = MODE == MODE_LOGITS || KEPT ? l2_evict_first() : 0ull;
+            const uint64_t keep = MODE == MODE_LOGITS ? l2_evict_normal() : 0ull, drop = MODE == MODE_LOGITS || KEPT ? l2_evict_first() : 0ull;
             for_each_item([&](int rt, int ln, int S, int, int kb0, int kb1) {
                 const bool second = (MODE == MODE_STATS || MODE == MODE_LOGITS) && rt >= p.row_tiles0;
                 const CUtensorMap* tmA = second ? &p.tmA1 : &p.tmA0;

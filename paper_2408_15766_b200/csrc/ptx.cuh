@@ -98,10 +98,10 @@ __device__ __forceinline__ void tma_load_2d(uint32_t smem_dst, const CUtensorMap
         ::"r"(smem_dst), "l"(reinterpret_cast<uint64_t>(tm)), "r"(bar), "r"(x), "r"(y)
         : "memory");
 }
-// L2 policies of a load: what it brings stays longest, or goes first
-__device__ __forceinline__ uint64_t l2_evict_last() {
+// L2 policies of a load: what it brings is as good as what anyone else has there, or goes first
+__device__ __forceinline__ uint64_t l2_evict_normal() {
     uint64_t p;
-    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
+    asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
     return p;
 }
 __device__ __forceinline__ uint64_t l2_evict_first() {
