@@ -404,7 +404,7 @@ static int make_layout(long long N, long long d, long long V, int K, int sms, La
     off += 256;
     const size_t slots = static_cast<size_t>(slot_cap);
     L->thr_share = off;                     // admission thresholds the lanes of a row tile publish to each other; behind the
-    off = align256(off + slots * BM * 8);   // status block, so that one memset clears both
+    off = align256(off + slots * BM * 4);   // status block, so that one memset clears both
     L->part_m = off;
     off = align256(off + slots * BM * 4);
     L->part_s = off;
@@ -494,17 +494,25 @@ static int launch_gemm(const GemmParams& p, cudaStream_t st, int kind = -1) {
     return launch(fn, p.sched.max_ctas, NUM_THREADS, SMEM_BYTES, st, MODE == MODE_OUT && p.plan.cluster > 1 ? p.plan.cluster : pair ? 2 : 1, p);
 }
 
-// Clears a 256-byte aligned piece of the workspace (a multiple of 16 bytes).
-static int clear_bytes(void* at, size_t bytes, cudaStream_t st) {
-    const int n = static_cast<int>(bytes / 16);
-    return launch(clear_kernel, n <= 256 * 16 ? ceil_div(n, 256) : 16, 256, 0, st, 1, static_cast<uint4*>(at), n);
+// Clears a 256-byte aligned piece of the workspace (a multiple of 16 bytes), and a second one.
+static int clear_bytes(void* at, size_t bytes, cudaStream_t st, void* at2 = nullptr, size_t bytes2 = 0) {
+    const int n = static_cast<int>(bytes / 16), n2 = static_cast<int>(bytes2 / 16);
+    return launch(clear_kernel, n + n2 <= 256 * 16 ? ceil_div(n + n2, 256) : 16, 256, 0, st, 1, static_cast<uint4*>(at), n, static_cast<uint4*>(at2), n2);
 }
 
-// Clears the status block (only_thresholds: not) and the published thresholds of `slots` slots.
-static int clear_status(uint8_t* ws, const Layout& L, int slots, cudaStream_t st, bool only_thresholds = false) {
+// Clears the status block (only_thresholds: not) and the published thresholds of `slots` slots, with their shared bounds.
+static int clear_status(uint8_t* ws, const Layout& L, int slots, cudaStream_t st, bool only_thresholds = false, uint2* bounds = nullptr) {
     const size_t from = only_thresholds ? L.thr_share : L.status;
     if (only_thresholds && slots == 0) return HASS_OK;
-    return clear_bytes(ws + from, L.thr_share + static_cast<size_t>(slots) * BM * 8 - from, st);
+    return clear_bytes(ws + from, L.thr_share + static_cast<size_t>(slots) * BM * 4 - from, st, bounds,
+                       bounds ? static_cast<size_t>(slots) * BM * 8 : 0);
+}
+
+// Bytes [from, to) of the workspace, which nothing else uses between the clearing and the selection after a sweep of this
+// schedule, as the room in which its lanes share their bounds (GemmParams::bounds); nullptr where they do not fit or K needs none. With
+// a place of their own in the layout they would take from calls at the least workspace and from the built-in scratch.
+static uint2* bounds_room(uint8_t* ws, size_t from, size_t to, const Schedule& s, int K) {
+    return K > K_REG && to >= from + static_cast<size_t>(s.total_slots) * BM * 8 ? reinterpret_cast<uint2*>(ws + from) : nullptr;
 }
 
 template <int WARPS, int WIN>
@@ -545,6 +553,8 @@ static SelectParams select_params(const GemmParams& p, int first_tile, int row_b
     sp.cand = p.cand;
     sp.cand_n = p.cand_n;
     sp.thr_share = p.thr_share;
+    sp.bounds = p.bounds;
+    sp.col_tiles = p.col_tiles;
     sp.idx_out = idx_out;
     sp.q_out = q_out;
     sp.out_pitch = out_pitch;
@@ -654,8 +664,9 @@ static int forward_impl(bool with_target, const void* H_t, const void* H_d, cons
     p.cand = reinterpret_cast<uint2*>(ws + L.cand_v);
     p.cand_n = reinterpret_cast<int*>(ws + L.cand_i);
     p.status = reinterpret_cast<unsigned int*>(ws + L.status);
-    p.thr_share = reinterpret_cast<uint2*>(ws + L.thr_share);
-    rc = clear_status(ws, L, p.sched.total_slots, st);
+    p.thr_share = reinterpret_cast<unsigned int*>(ws + L.thr_share);
+    if (with_target) p.bounds = bounds_room(ws, L.fwd_end, workspace_bytes, p.sched, K);
+    rc = clear_status(ws, L, p.sched.total_slots, st, false, p.bounds);
     if (rc != HASS_OK) return rc;
     rc = launch_gemm<MODE_STATS>(p, st);
     if (rc != HASS_OK) return rc;
@@ -1056,12 +1067,14 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
         p.Pt = cmb ? cmb->Pt : nullptr;
         p.p_pitch = L.p_pitch;
         p.status = status;
-        p.thr_share = reinterpret_cast<uint2*>(ws + L.thr_share);
+        p.thr_share = reinterpret_cast<unsigned int*>(ws + L.thr_share);
         p.row_zmax = zmax + static_cast<size_t>(with_target ? 2 : 1) * t0 * BM;
         p.use_row_zmax = retry ? 1 : 0;
         p.gate = gate;
+        // (finalize's rows take the place of the bounds, so the second pass of a single chunk, which clears nothing, has none)
+        if (!retry && with_target) p.bounds = bounds_room(ws, L.sparse, L.scratch, p.sched, K);
         if (!retry || RT > chunk_tiles) {      // (a single chunk's thresholds hold for its second pass too)
-            rc = clear_status(ws, L, p.sched.total_slots, st, retry || t0 > 0);
+            rc = clear_status(ws, L, p.sched.total_slots, st, retry || t0 > 0, p.bounds);
             if (rc != HASS_OK) return rc;
         }
         rc = launch_gemm<MODE_STATS>(p, st);
@@ -1328,7 +1341,7 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
             p.part_s = reinterpret_cast<float*>(ws + L.part_s);
             p.cand = reinterpret_cast<uint2*>(ws + L.cand_v);
             p.cand_n = reinterpret_cast<int*>(ws + L.cand_i);
-            p.thr_share = reinterpret_cast<uint2*>(ws + L.thr_share);
+            p.thr_share = reinterpret_cast<unsigned int*>(ws + L.thr_share);
             p.p_pitch = L.p_pitch;
             p.status = status;
             p.gate = gate;
@@ -1338,7 +1351,8 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
                     rc = pipe_in(pipe, H_t, H_d, static_cast<size_t>(t0) * BM, static_cast<size_t>(rows), st, &ev_d);
                     if (rc != HASS_OK) return rc;
                 }
-                rc = clear_status(ws, L, with_target ? p.sched.total_slots : 0, st, t0 > 0);
+                if (with_target) p.bounds = bounds_room(ws, L.sparse, L.scratch, p.sched, K);
+                rc = clear_status(ws, L, with_target ? p.sched.total_slots : 0, st, t0 > 0, p.bounds);
                 if (rc != HASS_OK) return rc;
                 if (with_target) {
                     // (1) target rows: statistics + candidates
@@ -1507,8 +1521,9 @@ static int forward2_impl(bool with_target, const void* H_t, const void* H_d, con
     int* sidx = reinterpret_cast<int*>(ws + L.sidx);
     float* sq = reinterpret_cast<float*>(ws + L.sgq);
     float* capz = reinterpret_cast<float*>(ws + L.capz);
-    p.thr_share = reinterpret_cast<uint2*>(ws + L.thr_share);
-    rc = clear_status(ws, L, with_target ? p.sched.total_slots : 0, st);
+    p.thr_share = reinterpret_cast<unsigned int*>(ws + L.thr_share);
+    if (with_target) p.bounds = bounds_room(ws, L.sparse, workspace_bytes, p.sched, K);
+    rc = clear_status(ws, L, with_target ? p.sched.total_slots : 0, st, false, p.bounds);
     if (rc != HASS_OK) return rc;
     if (with_target) {
         GemmParams t = p;
@@ -1616,8 +1631,9 @@ static int normed_impl(const void* H_t, const void* H_d, const void* W, long lon
         p.cand = reinterpret_cast<uint2*>(ws + L.cand_v);
         p.cand_n = reinterpret_cast<int*>(ws + L.cand_i);
         p.status = reinterpret_cast<unsigned int*>(ws + L.status);
-        p.thr_share = reinterpret_cast<uint2*>(ws + L.thr_share);
-        rc = clear_status(ws, L, p.sched.total_slots, st);
+        p.thr_share = reinterpret_cast<unsigned int*>(ws + L.thr_share);
+        p.bounds = bounds_room(ws, L.fwd_end, workspace_bytes, p.sched, K);
+        rc = clear_status(ws, L, p.sched.total_slots, st, false, p.bounds);
         if (rc != HASS_OK) return rc;
         rc = launch_gemm<MODE_STATS>(p, st);
         if (rc != HASS_OK) return rc;

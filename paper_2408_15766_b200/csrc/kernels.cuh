@@ -113,8 +113,10 @@ struct GemmParams {
     float* part_s;
     uint2* cand;           // [slot, row, cap] (logit bits, token id)
     int* cand_n;           // [slot, row] entries in use
-    uint2* thr_share;      // [slot, row] what a lane publishes to the others of its row tile, as ordered keys (zeroed before the
-                           // sweep: nothing yet): x = a bound that K of its logits reach, y = one that lane_share(K, S) of them reach
+    unsigned int* thr_share;   // [slot, row] what a lane publishes to the others of its row tile, as an ordered key (zeroed before the
+                           // sweep: nothing yet): a bound that K of its logits reach
+    uint2* bounds;         // TOPK_BUF, nullable: [slot, row] the same with room for two (zeroed likewise): x = that bound, y = one that
+                           // lane_share(K, S) of its logits reach. Without it lanes do not share their bounds
     // MODE_PROBS
     const float* lse2;     // [N] lse_d * log2(e)
     const float* coef;     // [N] g * S_q
@@ -734,7 +736,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
             const int t0 = first_tile(rt, ln);
             const int nt = (p.col_tiles - ln + S - 1) / S;
             // lanes of three tiles and more share their bounds (see below)
-            const bool joint = HAS_TOPK && !USE_REG && p.col_tiles > 2 * S;
+            const bool joint = HAS_TOPK && !USE_REG && p.bounds != nullptr && p.col_tiles > 2 * S;
             for (int t = t0; t < nt; ++t) {
                 const int ct = t < 0 ? 0 : ln + t * S;
                 // the whole warp must agree before the warp-collective TMEM loads below
@@ -1177,15 +1179,18 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                         part = fmaxf(part, thr_own);
                     }
                     if (S > 1) {
-                        uint2* sh = p.thr_share + static_cast<long long>(slot - ln) * BM + r_local;
+                        const long long at = static_cast<long long>(slot - ln) * BM + r_local;
                         const uint2 own = make_uint2(ordered_key(__float_as_uint(thr_own)), ordered_key(__float_as_uint(part)));      // (the first tile's bound is in thr_sh)
-                        st_relaxed_v2(sh + static_cast<long long>(ln) * BM, own);
-                        if (t + 1 < nt) {
-                            unsigned int best = 0u;
-                            if (!joint) {
-                                const int nn = S - 1 < 3 ? S - 1 : 3;
-                                for (int q = 1; q <= nn; ++q) best = max(best, ld_relaxed_v2(sh + static_cast<long long>((ln + q) % S) * BM).x);
-                            } else {
+                        unsigned int best = 0u;
+                        if (!joint) {
+                            unsigned int* sh = p.thr_share + at;
+                            st_relaxed(sh + static_cast<long long>(ln) * BM, own.x);
+                            const int nn = t + 1 < nt ? (S - 1 < 3 ? S - 1 : 3) : 0;
+                            for (int q = 1; q <= nn; ++q) best = max(best, ld_relaxed(sh + static_cast<long long>((ln + q) % S) * BM));
+                        } else {
+                            uint2* sh = p.bounds + at;
+                            st_relaxed_v2(sh + static_cast<long long>(ln) * BM, own);
+                            if (t + 1 < nt) {
                                 // eight loads in flight (one by one they take as long as the tile's candidates)
                                 unsigned int least = own.y;
                                 for (int q0 = 0; q0 < S; q0 += 8) {
@@ -1200,8 +1205,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                                 }
                                 best = max(best, least);
                             }
-                            if (best != 0u) thr_sh = fmaxf(thr_sh, nextafterf(__uint_as_float(key_bits(best)), -INFINITY));
                         }
+                        if (best != 0u) thr_sh = fmaxf(thr_sh, nextafterf(__uint_as_float(key_bits(best)), -INFINITY));
                     }
                     thr = fmaxf(thr_own, fmaxf(thr, thr_sh));
                 }
@@ -1629,7 +1634,9 @@ struct SelectParams {
     const float* part_s;
     const uint2* cand;
     const int* cand_n;
-    const uint2* thr_share;    // as the sweep left it (GemmParams)
+    const unsigned int* thr_share;    // as the sweep left them (GemmParams)
+    const uint2* bounds;
+    int col_tiles;
     const int* idx_in;     // [N, K]
     const float* q_in;
     int* idx_out;          // [N, K] (from_sweep)
@@ -1760,6 +1767,7 @@ __global__ void __launch_bounds__(sel_block_warps(WARPS) * 32) select_kernel(con
         int slot0, S;
         find_slots(p.sched, rt, slot0, S);
         const bool lists = p.cap == K_REG;      // sorted register lists of K_REG entries (unused ones: id -1)
+        const bool joint = p.bounds != nullptr && S > 1 && p.col_tiles > 2 * S;      // (as in the sweep)
         // lse_t, and a floor below which no candidate can be among the K best: the best K-th largest logit of any list,
         // or the K-th largest of the lists' first entries
         float m = -INFINITY, sum = 0.f;
@@ -1780,10 +1788,12 @@ __global__ void __launch_bounds__(sel_block_warps(WARPS) * 32) select_kernel(con
         for (int j = lane; j < S; j += 32) {
             const long long so = static_cast<long long>(slot0 + j) * BM + r;
             const float pm = p.part_m[so], ps = p.part_s[so];
-            if (!lists) {
-                const uint2 bounds = p.thr_share[so];
+            if (joint) {
+                const uint2 bounds = p.bounds[so];
                 floor_key = max(floor_key, bounds.x);
                 least_key = min(least_key, bounds.y);
+            } else if (!lists) {
+                floor_key = max(floor_key, p.thr_share[so]);
             }
             if (pm > m) {
                 sum *= exp2f((m - pm) * LOG2E);
@@ -1798,7 +1808,7 @@ __global__ void __launch_bounds__(sel_block_warps(WARPS) * 32) select_kernel(con
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
         floor_key = __reduce_max_sync(0xffffffffu, floor_key);
-        if (!lists) floor_key = max(floor_key, __reduce_min_sync(0xffffffffu, least_key));
+        if (joint) floor_key = max(floor_key, __reduce_min_sync(0xffffffffu, least_key));
         if (lists && S >= K) {
             uint32_t T = 0u;
 #pragma unroll 1
@@ -2585,9 +2595,9 @@ __global__ void __launch_bounds__(256) ce_kernel(int rows, int row_begin, int d,
 
 // Clears n 16-byte words: the status block and what lies behind it. (A memset node would stand between two dependent
 // launches and make both wait: 5 us per call.)
-__global__ void __launch_bounds__(256) clear_kernel(uint4* at, int n) {
+__global__ void __launch_bounds__(256) clear_kernel(uint4* at, int n, uint4* at2, int n2) {
     wait_previous_kernel();
-    for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) at[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < n + n2; i += gridDim.x * 256) *(i < n ? at + i : at2 + (i - n)) = make_uint4(0u, 0u, 0u, 0u);
 }
 
 // Self-test of the bounded waits (hass_selftest_wait_expiry): one CTA, no TMA, no tensor memory. Every thread

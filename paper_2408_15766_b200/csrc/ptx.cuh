@@ -314,7 +314,15 @@ __device__ __forceinline__ void st_shared_b32_if(uint32_t addr, uint32_t v, bool
                  "r"(static_cast<uint32_t>(on))
                  : "memory");
 }
-// words that other CTAs read and write meanwhile, each pair as one
+// words that other CTAs read and write meanwhile; of a pair, either may be older than the other
+__device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* at) {
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(at) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_relaxed(uint32_t* at, uint32_t v) {
+    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(at), "r"(v) : "memory");
+}
 __device__ __forceinline__ uint2 ld_relaxed_v2(const uint2* at) {
     uint2 v;
     asm volatile("ld.relaxed.gpu.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(at) : "memory");

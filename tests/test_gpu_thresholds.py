@@ -40,3 +40,18 @@ def test_sets_of_large_k(N, V, K, layout):
         z = (H_t.double() @ W.double().T).gather(1, cpu["topk_idx"].long())
         assert (z - want).abs().max() <= 1e-4      # fp32 sums of 64 products of up to 8 in another order: 64 x 2^-24 x 16
         print(compare(H_t, inp.H_d[0], W, K, cpu, check_dH=False, rows=range(0, N, 37)))
+
+
+@pytest.mark.parametrize("K", [17, 100])
+def test_the_least_workspace_gives_the_same_sets(K):
+    """Lanes share their bounds in room that the call does not use meanwhile; a workspace that ends before it does without."""
+    import paper_2408_15766_b200 as hass
+    N, d, V = 2100, 64, 12800
+    inp = hi.make_custom(N, d, V, K, seed=K, sigma_w=0.3)
+    dev = torch.device("cuda:0")
+    args = inp.H_t.to(dev), inp.H_d[0].to(dev), inp.W.to(dev), K
+    least = torch.empty(hass.topk_distill_fwd_static_scratch_bytes(N, d, V, K), dtype=torch.uint8, device=dev)
+    a, b = hass.topk_distill_fwd(*args, workspace=least), hass.topk_distill_fwd(*args)
+    hass.check(a["workspace"])
+    hass.check(b["workspace"])
+    assert torch.equal(a["topk_idx"], b["topk_idx"])
