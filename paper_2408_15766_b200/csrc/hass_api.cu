@@ -822,13 +822,9 @@ struct Combined {
 // x 4096 x 32000 215 -> 147 us. The sweep does nothing but store its accumulators, and one kernel does the rest of a row: with
 // candidate lists and statistics in the sweep's epilogue, a kernel that selects and one that forms dz_d, the last tile's epilogue, on its
 // own at the end, took 12 us and the two kernels 25 (61 rows x 4096 x 32000: 135 -> 112 us on the device, 64 rows x 256 x 1024 39 -> 26,
-// 76 rows x 4096 x 128256 with K = 44 508 -> 478). The logits take the scratch and what follows; the partial
+// 76 rows x 4096 x 128256 with K = 44 508 -> 478; Bi-directional 40 rows x 64 x 700 76 -> 39, 35 x 4096 x 32000 186 -> 123). The logits take the scratch and what follows; the partial
 // tiles of the second GEMM take the target's, which are read no more by then. A workspace that ends before them takes the
 // other route.
-// Bi-directional calls take it from this size of W on (40 rows x 256 x 1024 68 -> 35 us, 35 rows x 4096 x 32000 186 -> 123 us). No head in
-// use is smaller; there the spill and its second pass, which a draft of 256 logits above its reference needs, stay in use
-// at few rows too.
-constexpr long long kNarrowBidirBytes = 128 << 10;
 // The second GEMM of such a call reads W again. The L2 (126 MB) would hold the end of the first reading, but that is the last
 // k blocks of all columns, and the second reading, which walks the other way, evicts them before it comes to them. So the
 // sweep lets this much of W, its last k blocks, into the L2 like any other data and asks that the rest go first: 61 rows x 4096 x 32000
@@ -1009,7 +1005,7 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
     __nv_bfloat16* P = reinterpret_cast<__nv_bfloat16*>(ws + L.scratch);
     unsigned int* status = reinterpret_cast<unsigned int*>(ws + L.status);
     int* idx_d = reinterpret_cast<int*>(ws + L.sidx);
-    if (with_target && !(cmb && N > BM / 2) && !(bidir && V * d * 2 < kNarrowBidirBytes)) {
+    if (with_target && !(cmb && N > BM / 2)) {
         const NarrowRoom narrow = narrow_room(N, ws, cmb ? cmb->end : workspace_bytes, L);
         if (narrow.z)
             return narrow_impl(cmb ? ROW_COMBINED : bidir ? ROW_BIDIR : ROW_TOPK, true, H_t, H_d, W, static_cast<int>(N), d, V, K, grad_loss,

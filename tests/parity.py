@@ -23,6 +23,17 @@ LSE_ATOL = 1e-4
 Q_RTOL = 1e-3
 
 
+def least_workspace(N, d, V, K) -> int:
+    """Bytes of the smallest workspace that a call of at most 128 rows with a gradient accepts: the forward's part, the [N, K] lists and
+    [N] vectors behind it, the largest logits, 128 rows of fp32 and one row tile of scratch, each 256-byte aligned. Beyond 32 rows it
+    has no room for two fp32 logit matrices."""
+    import paper_2408_15766_b200 as hass
+    assert N <= 128
+    up = lambda x: -(-x // 256) * 256
+    return (hass.topk_distill_fwd_static_scratch_bytes(N, d, V, K) + 3 * up(N * K * 4) + 2 * up(N * 4) + 2 * 128 * 4 + 128 * d * 4
+            + 128 * up(V) * 2)
+
+
 def compare(H_t, H_d, W, K, gpu: dict, rows=None, grad_loss=None, check_dH=True) -> dict:
     """H_t, H_d, W: bf16 CPU tensors. gpu: dict of CPU tensors/arrays with loss, topk_idx, topk_q,
     lse_t, lse_d and (if check_dH) dH_d, for ALL N rows. rows: subset the oracle evaluates."""

@@ -6,7 +6,7 @@ import pytest
 import torch
 
 import hass_inputs as hi
-from parity import compare, compare_variant
+from parity import compare, compare_variant, least_workspace
 
 pytestmark = pytest.mark.gpu
 
@@ -178,7 +178,7 @@ def _chunk_rows():
 
 @pytest.mark.parametrize("N", [40, 200])
 def test_rows_beyond_the_exponent_range_of_the_spill_are_redone(N):
-    # Of 40 rows only the Bi-directional call spills (the others keep the draft logits in fp32), of 200 rows all five do.
+    # Calls of 40 rows keep the draft logits in fp32 where the workspace has room; of 200 rows all five spill.
     hass = _hass()
     d, V, K = 64, 700, 3
     inp = hi.make_custom(N, d, V, K, seed=3, sigma_w=0.1)
@@ -209,8 +209,20 @@ def test_rows_beyond_the_exponent_range_of_the_spill_are_redone(N):
     v = hass.variant_distill_fwd_bwd(inp.H_t.to(dev), H_d.to(dev), W.to(dev), K, hass.LOSS_BIDIR_TOPK, 0.0,
                                      dH_dtype=hass.HASS_FP32)
     hass.check(v["workspace"])
-    assert _second_pass(v["workspace"])
+    assert _second_pass(v["workspace"]) == (N > 128)
     print("bidir, second sweep", compare_variant(inp.H_t, H_d, W, K, oracle.VARIANT_BIDIR, 0.0, _to_cpu(v)))
+    if N <= 128:
+        # in the least workspace they spill, and are redone, too
+        least = least_workspace(N, d, V, K)
+        with pytest.raises(hass.HassError):
+            hass.variant_distill_fwd_bwd(inp.H_t.to(dev), H_d.to(dev), W.to(dev), K, hass.LOSS_BIDIR_TOPK, 0.0,
+                                         workspace=torch.empty(least - 256, dtype=torch.uint8, device=dev))
+        for which, code, param in ((hass.LOSS_BIDIR_TOPK, oracle.VARIANT_BIDIR, 0.0), (hass.LOSS_TOP_P, oracle.VARIANT_TOP_P, 0.004)):
+            v = hass.variant_distill_fwd_bwd(inp.H_t.to(dev), H_d.to(dev), W.to(dev), K, which, param, dH_dtype=hass.HASS_FP32,
+                                             workspace=torch.empty(least, dtype=torch.uint8, device=dev))
+            hass.check(v["workspace"])
+            assert _second_pass(v["workspace"])
+            print("few rows, second sweep", compare_variant(inp.H_t, H_d, W, K, code, param, _to_cpu(v)))
     c = hass.combined_distill_fwd_bwd(inp.H_t.to(dev), H_d.to(dev), W.to(dev), K, w_topk=0.5, dH_dtype=hass.HASS_FP32)
     hass.check(c["workspace"])
     assert _second_pass(c["workspace"]) == (N > 128)

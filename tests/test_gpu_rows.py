@@ -58,7 +58,7 @@ def test_equal_logits_give_the_lowest_tokens(V, K, first):
 
 @pytest.mark.parametrize("N,d,V,K", [(1, 264, 8200, 20), (64, 512, 4100, 7), (100, 264, 8200, 128), (128, 8, 270000, 3)])
 def test_variants_of_few_rows_against_the_oracle(N, d, V, K):
-    """The Bi-directional variant takes this route for heads of 128 KB and more; its Omega_hat term stays in fp32."""
+    """The Omega_hat term of the Bi-directional variant stays in fp32 on this route too."""
     hass = _hass()
     dev = torch.device("cuda:0")
     inp = hi.make_custom(N, d, V, K, seed=N + V, sigma_w=0.1)
