@@ -1682,7 +1682,7 @@ const char* hass_status_string(int status) {
     }
 }
 
-int hass_version(void) { return 10500; }
+int hass_version(void) { return 10600; }
 
 int64_t hass_kernel_launch_count(void) { return g_launches.load(); }
 
