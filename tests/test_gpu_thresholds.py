@@ -9,11 +9,20 @@ from parity import compare
 pytestmark = pytest.mark.gpu
 
 
-# three row tiles over 24 column tiles, two chunks' worth of lanes with one tile each, a ragged last tile, every row tile its own lane
-@pytest.mark.parametrize("N,V", [(300, 6000), (300, 12800), (2100, 1500)])
+def _shared_bounds(ws, N, V, K):
+    """Whether lanes have shared their bounds in this workspace of the forward: the room behind the largest logits is not zero."""
+    import paper_2408_15766_b200 as hass
+    up = lambda x: -(-x // 256) * 256
+    at = hass.topk_distill_fwd_static_scratch_bytes(N, 64, V, K) + 3 * up(N * K * 4) + 2 * up(N * 4) + 2 * -(-N // 128) * 128 * 4
+    return bool(ws[at:at + 128 * 8].view(torch.int32).any())
+
+
+# On 148 SMs: lanes of one column tile; of one or two; of two or three (125 tiles on 49 lanes), a pair per row tile; of six or seven (50 on
+# 8), the last row tile alone in its pair; of three (24 on 8). From three tiles on lanes share their bounds.
+@pytest.mark.parametrize("N,V,shared", [(300, 6000, False), (300, 12800, False), (300, 32000, True), (2100, 12800, True), (2100, 6000, True)])
 @pytest.mark.parametrize("K", [17, 100, 256])
 @pytest.mark.parametrize("layout", ["even", "one tile", "rising", "falling", "alike"])
-def test_sets_of_large_k(N, V, K, layout):
+def test_sets_of_large_k(N, V, shared, K, layout):
     import paper_2408_15766_b200 as hass
     d = 64
     inp = hi.make_custom(N, d, V, K, seed=V + K, sigma_w=0.3)
@@ -30,8 +39,10 @@ def test_sets_of_large_k(N, V, K, layout):
         H_t[:, 1:] = 0.0
         W[:, 0] = (torch.arange(V) % 3).to(torch.bfloat16)      # three values: a third of the vocabulary ties at the top
     dev = torch.device("cuda:0")
-    out = hass.topk_distill_fwd(H_t.to(dev), inp.H_d[0].to(dev), W.to(dev), K)
-    hass.check(out["workspace"])
+    ws = torch.zeros(hass.topk_distill_workspace_bytes(N, d, V, K), dtype=torch.uint8, device=dev)
+    out = hass.topk_distill_fwd(H_t.to(dev), inp.H_d[0].to(dev), W.to(dev), K, workspace=ws)
+    hass.check(ws)
+    assert _shared_bounds(ws, N, V, K) == shared
     cpu = {k: v.cpu() for k, v in out.items() if k != "workspace"}
     if layout == "alike":
         assert torch.equal(cpu["topk_idx"].long(), (2 + 3 * torch.arange(K)).expand(N, K))
