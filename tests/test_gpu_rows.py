@@ -174,3 +174,18 @@ def test_rows_of_zeros_take_no_longer(d, V, K):
     hass.check(ws)
     print(plain, zeros)
     assert zeros <= 1.25 * plain + 20.0
+
+
+@pytest.mark.parametrize("V,K", [(700, 5), (5000, 40)])
+def test_an_infinite_logit_comes_first(V, K):
+    hass = _hass()
+    dev = torch.device("cuda:0")
+    inp = hi.make_custom(3, 64, V, K, seed=V, sigma_w=0.3)
+    H, W = inp.H_t.clone(), inp.W.clone()
+    H[:, 0] = 1.0
+    W[[V - 3, 17], 0] = float("inf")
+    W[300:400, 0] = -float("inf")
+    out = hass.topk_distill_fwd(H.to(dev), H.to(dev), W.to(dev), K)
+    hass.check(out["workspace"])
+    z = H[:, 1:].double() @ W[:, 1:].double().T + W[:, 0].double()
+    assert torch.equal(out["topk_idx"].cpu().long(), z.sort(dim=1, descending=True, stable=True).indices[:, :K])
