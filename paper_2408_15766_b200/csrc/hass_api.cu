@@ -818,13 +818,12 @@ struct Combined {
 
 // Calls of one row tile, where the logits go through the workspace in fp32 (narrow_impl). Such a call is bound by
 // reading W, which this route does twice (both sweeps in one launch, then the second GEMM) instead of three times, with no
-// range condition and so no second pass: 61 rows x 4096 x 32000 211 -> 147 us, 64 rows x 256 x 1024 67 -> 46 us, 100 rows
-// x 4096 x 32000 215 -> 147 us. The sweep does nothing but store its accumulators, and one kernel does the rest of a row: with
-// candidate lists and statistics in the sweep's epilogue, a kernel that selects and one that forms dz_d, the last tile's epilogue, on its
-// own at the end, took 12 us and the two kernels 25 (61 rows x 4096 x 32000: 135 -> 112 us on the device, 64 rows x 256 x 1024 39 -> 26,
-// 76 rows x 4096 x 128256 with K = 44 508 -> 478; Bi-directional 40 rows x 64 x 700 76 -> 39, 35 x 4096 x 32000 186 -> 123). The logits take the scratch and what follows; the partial
-// tiles of the second GEMM take the target's, which are read no more by then. A workspace that ends before them takes the
-// other route.
+// range condition and so no second pass. The sweep does nothing but store its accumulators, and one kernel does the rest of a row:
+// with candidate lists and statistics in the sweep's epilogue, a kernel that selects and one that forms dz_d, the last tile's epilogue,
+// on its own at the end, took 12 us and the two kernels 25. From a flushed L2 61 rows x 4096 x 32000 take 115 us (154 in that form),
+// 100 rows 125 (160), 64 rows x 256 x 1024 30 (45), and Bi-directional calls, which spilled, 35 rows x 4096 x 32000 125 (203), 40 x 64 x 700
+// 39 (76). The logits take the scratch and what follows; the partial tiles of the second GEMM take the target's, which are read no
+// more by then. A workspace that ends before them takes the other route.
 // The second GEMM of such a call reads W again. The L2 (126 MB) would hold the end of the first reading, but that is the last
 // k blocks of all columns, and the second reading, which walks the other way, evicts them before it comes to them. So the
 // sweep lets this much of W, its last k blocks, into the L2 like any other data and asks that the rest go first: 61 rows x 4096 x 32000
@@ -832,8 +831,8 @@ struct Combined {
 // and 127, but they stayed when the call was over: a pass over 80 MB of the caller's took 26.6 us after a call instead of 21.5.
 constexpr long long kKeepBytes = 64ll << 20;
 // From this size of W on the kernels of such a call let the next one's blocks in when they end: blocks that wait beside a
-// kernel bound by reading W cost it time (61 rows x 4096 x 32000 103.6 -> 101.3 us, 99 draft rows 114.3 -> 109.7, 100 rows 142.9 -> 138.4);
-// with a head of 0.5 MB their early start is worth more (64 rows x 256 x 1024 24.4 us early, 24.8 late).
+// kernel bound by reading W cost it time (from a flushed L2 61 rows x 4096 x 32000 118.8 -> 114.8 us, 99 draft rows 117.5 -> 112.6, 100 rows
+// 129.0 -> 124.9); with a head of 0.5 MB it is the same (64 rows x 256 x 1024 30.3 us early, 30.0 late).
 constexpr long long kLateBytes = 16ll << 20;
 struct NarrowRoom {
     float* z = nullptr;      // [N, p_pitch], or nullptr: no room
@@ -1005,6 +1004,9 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
     __nv_bfloat16* P = reinterpret_cast<__nv_bfloat16*>(ws + L.scratch);
     unsigned int* status = reinterpret_cast<unsigned int*>(ws + L.status);
     int* idx_d = reinterpret_cast<int*>(ws + L.sidx);
+    // The combined objective takes that route up to 64 rows only: the line was drawn where both fp32 matrices fitted the scratch of one
+    // row tile. There is room up to 128 rows now, and the route would be the faster one there as well (65 rows x 4096 x 32000 254 us as it
+    // is, 123 on that route, 128 rows x 4096 x 128256 675 and 472, 100 rows x 256 x 1024 82 and 37).
     if (with_target && !(cmb && N > BM / 2)) {
         const NarrowRoom narrow = narrow_room(N, ws, cmb ? cmb->end : workspace_bytes, L);
         if (narrow.z)

@@ -656,16 +656,15 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
         uint32_t spill_boxes = 0;                  // chunks this warp has staged for TMA stores (two per box)
         // TOPK_REG: the K_REG largest logits so far sorted descending in tv[] (the admission threshold is the
         // K_REG-th largest: a list of exactly K entries with its K-th as threshold measured slower), and the
-        // current chunk's admitted logits waiting in a small local-memory buffer
+        // current chunk's admitted logits waiting in shared memory: entry q of thread T at word q * 128 + T of the values' array and
+        // of the tokens' array (16 KB each, the room the draft sweep uses for its spill boxes; this instantiation stores no boxes). With
+        // 200 KB of shared memory carved out little L1 is left, and a per-thread array in local memory cost about a thousand
+        // cycles per admitted logit here.
         constexpr bool USE_REG = MODE == MODE_STATS && TOPK == TOPK_REG;
         constexpr bool HAS_TOPK = MODE == MODE_STATS && TOPK != TOPK_NONE;
         constexpr bool CAPTURE = MODE == MODE_STATS && TOPK == TOPK_NONE;
         float tv[USE_REG ? K_REG : 1];
         int ti[USE_REG ? K_REG : 1];
-        // ... waiting in shared memory: entry q of thread T at word q * 128 + T of the values' array and of the
-        // tokens' array (16 KB each, the room the draft sweep uses for its spill boxes; this instantiation stores no
-        // boxes). With 200 KB of shared memory carved out little L1 is left, and a per-thread array in local memory
-        // cost about a thousand cycles per admitted logit here.
         static_assert(4 * SPILL_STAGES * SPILL_STAGE_BYTES >= 2 * 32 * 128 * 4, "room for the pending logits");
         const uint32_t pend_v = spill_stage + (threadIdx.x - 64) * 4;
         const uint32_t pend_i = pend_v + 32 * 128 * 4;
@@ -2158,7 +2157,8 @@ __device__ __forceinline__ void own_stats(const float* row, long long pitch, flo
     });
 }
 
-// The block's log-sum-exp of the threads' (m, s); `red`: 2 x 32 floats. Two barriers.
+// The block's log-sum-exp of the threads' (m, s); `red`: 2 x 32 floats, which
+// the caller keeps until all have read them. One barrier.
 template <int THREADS>
 __device__ __forceinline__ float block_lse(float m, float s, float (*red)[32]) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
