@@ -149,29 +149,29 @@ def test_more_logits_at_the_bound_than_the_pool_holds(pattern, K):
 @pytest.mark.parametrize("d,V,K", [(256, 128256, 10), (256, 128256, 64), (256, 1024, 10)])
 def test_rows_of_zeros_take_no_longer(d, V, K):
     """Feature rows of zeros (padding) have V equal logits. Where token ids are searched bit by bit, they take a call of 128256 tokens
-    from 114 to 878 us, and ranking 1024 equal logits one of 1024 from 30 to 83; with one look at the first tokens neither changes."""
+    from 107 to 874 us, and ranking 1024 equal logits one of 1024 from 42 to 97; with one look at the first tokens neither changes."""
     hass = _hass()
     dev = torch.device("cuda:0")
     inp = hi.make_custom(8, d, V, K, seed=1, sigma_w=0.05)
-    H_t, H_d, W = inp.H_t.to(dev), inp.H_d[0].to(dev), inp.W.to(dev)
+    W = inp.W.to(dev)
     ws = torch.empty(hass.topk_distill_workspace_bytes(8, d, V, K), dtype=torch.uint8, device=dev)
-
-    def median_us():
-        times = []
-        for _ in range(40):
-            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-            a.record()
-            hass.topk_distill_fwd_bwd(H_t, H_d, W, K, workspace=ws)
-            b.record()
-            b.synchronize()
-            times.append(a.elapsed_time(b) * 1e3)
-        return sorted(times[10:])[15]
-
-    plain = median_us()
-    H_t[4:] = 0
-    H_d[4:] = 0
-    zeros = median_us()
+    features = []
+    for zero in (False, True):
+        H_t, H_d = inp.H_t.clone(), inp.H_d[0].clone()
+        if zero:
+            H_t[4:] = 0
+            H_d[4:] = 0
+        features.append((H_t.to(dev), H_d.to(dev)))
+    times = [[], []]
+    for i in range(120):      # (in turn, and the least of each: the host is part of these calls' time)
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        hass.topk_distill_fwd_bwd(*features[i % 2], W, K, workspace=ws)
+        b.record()
+        b.synchronize()
+        times[i % 2].append(a.elapsed_time(b) * 1e3)
     hass.check(ws)
+    plain, zeros = (min(t[5:]) for t in times)
     print(plain, zeros)
     assert zeros <= 1.25 * plain + 20.0
 
