@@ -37,8 +37,8 @@ UNIT = "tokens/s"
 # for the library version they were taken with; for the l3-8b shape the figures are scaled by the vocabulary ratio (W and
 # the spill grow with V; the 2 x 34 MB of H rows that do not are 6-11 % of the total). The launches counted under the
 # dH_d GEMM include the sum of its partial tiles, so that it has no figure per launch here.
-TRAFFIC_CAPTURE = {"version": 10500, "workload": "l2-7b", "V": 32000, "K": 10,
-                   "bytes_per_launch": {"stats_gemm": 302.1e6, "stats_gemm_draft": 578.0e6}}
+TRAFFIC_CAPTURE = {"version": 10600, "workload": "l2-7b", "V": 32000, "K": 10,
+                   "bytes_per_launch": {"stats_gemm": 301.8e6, "stats_gemm_draft": 573.3e6}}
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 
 

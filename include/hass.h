@@ -72,7 +72,7 @@ int hass_version(void);
  * chunk_rows x V, and the fp32 Omega_hat term of dH_d, chunk_rows x d; and, behind them, fp32 partial
  * tiles of dH_d (less than one 128-row tile of scratch). Calls of at most 128 rows keep their logits in fp32 instead, two
  * matrices of N x V. A smaller workspace is accepted down to room
- * for one 128-row tile of scratch; the calls then work in smaller chunks, and may do without partial tiles.
+ * for one 128-row tile of scratch; the calls then work in smaller chunks, and may do without partial tiles and fp32 logits.
  * Needs no GPU (assumes 148 SMs if none is present).
  */
 int hass_topk_distill_workspace_bytes(int64_t N, int64_t d, int64_t V, int32_t K, size_t* bytes);
