@@ -90,7 +90,8 @@ struct OutPlan {
 struct GemmParams {
     CUtensorMap tmA0, tmA1, tmB;   // boxes: 128 rows of A; of B the BN / pair columns that one CTA holds
     CUtensorMap tmSpill;   // MODE_STATS without Top-K lists (the draft sweep): the spill P as [chunk rows, p_pitch] bf16 with
-                           // boxes of 64 columns x 32 rows, 128-byte swizzle, for TMA stores
+                           // boxes of 64 columns x 32 rows, 128-byte swizzle, for TMA stores. MODE_LOGITS: B with boxes of the
+                           // lane's last, narrower tile
     Schedule sched;
     int row_tiles;         // row tiles of this launch; a pair's second tile may lie beyond
     int half_tiles;        // MODE_LOGITS, single CTAs: the one row tile is 64 rows of A0 and 64 of A1, boxes of 64 rows; a
@@ -133,6 +134,8 @@ struct GemmParams {
     float* z_out;
     float* zt_out;
     long long z_pitch;
+    int lane_cols;         // lane l sweeps the columns [l lane_cols, (l + 1) lane_cols) below z_pitch, in tiles of BN and a
+                           // narrower last one (a multiple of 32)
     int keep_from;         // k block from which on the L2 holds this sweep's tiles of B like any other's; those before it go first ...
     int kept;              // MODE_OUT: ... as all do in the second reading of B, which this is (host: selects the instantiation)
     int release_late;      // the next kernel's blocks may start when this one's have ended, not before
@@ -520,6 +523,19 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
             }
         }
     };
+    // Column tiles of lane ln, the first column of its tile t, and that tile's columns (BN but for the last one of MODE_LOGITS)
+    auto tiles_of = [&](int ln, int S) {
+        if constexpr (MODE == MODE_LOGITS) return (min(p.lane_cols, static_cast<int>(p.z_pitch) - ln * p.lane_cols) + BN - 1) / BN;
+        return (p.col_tiles - ln + S - 1) / S;
+    };
+    auto tile_col = [&](int ln, int S, int t) {
+        if constexpr (MODE == MODE_LOGITS) return ln * p.lane_cols + t * BN;
+        return (t < 0 ? 0 : ln + t * S) * BN;      // t = -1: column tile 0, for the row references only
+    };
+    auto tile_width = [&](int t) {
+        if constexpr (MODE == MODE_LOGITS) return min(BN, p.lane_cols - t * BN);
+        return BN;
+    };
     // Where rows spill without a given reference exponent, a lane that does not begin with column tile 0 computes it first
     // (t = -1); a pair agrees.
     auto first_tile = [&](int rt, int ln) {
@@ -539,13 +555,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                 const CUtensorMap* tmA = second ? &p.tmA1 : &p.tmA0;
                 const int row0 = p.a_row_offset + (second ? rt - p.row_tiles0 : rt) * BM;
                 const int t0 = first_tile(rt, ln);
-                const int nt = (p.col_tiles - ln + S - 1) / S;
+                const int nt = tiles_of(ln, S);
                 for (int t = t0; t < nt; ++t) {
-                    const int ct = t < 0 ? 0 : ln + t * S;   // t = -1: column tile 0, for the row references only
+                    const int width = tile_width(t);
+                    const CUtensorMap* tmB = MODE == MODE_LOGITS && width < BN ? &p.tmSpill : &p.tmB;
                     for (int kb = kb0; kb < kb1; ++kb) {
                         if (!wait_barrier(empty_bar(stage), phase ^ 1u, abort_flag, p.status, 1)) return false;
                         // a pair's bytes are all counted on the barrier of its first CTA, whose thread issues the products
-                        if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), CG * (A_STAGE_BYTES + B_STAGE_BYTES));
+                        if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), CG * A_STAGE_BYTES + width * (BK * 2));
                         const uint32_t bar = CG == 2 ? map_to_rank(full_bar(stage), 0) : full_bar(stage);
                         auto load = [&](uint32_t dst, const CUtensorMap* tm, int x, int y) {
                             if (CG == 2)
@@ -557,14 +574,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                             if (MODE == MODE_LOGITS || KEPT) {
                                 const uint64_t policy = MODE == MODE_LOGITS && kb >= p.keep_from ? keep : drop;
                                 if (CG == 2)
-                                    tma_load_2d_pair_hint(dst, &p.tmB, bar, x, y, policy);
+                                    tma_load_2d_pair_hint(dst, tmB, bar, x, y, policy);
                                 else
-                                    tma_load_2d_hint(dst, &p.tmB, bar, x, y, policy);
+                                    tma_load_2d_hint(dst, tmB, bar, x, y, policy);
                             } else {
-                                load(dst, &p.tmB, x, y);
+                                load(dst, tmB, x, y);
                             }
                         };
-                        const int col0 = ct * BN + static_cast<int>(rank) * (BN / CG);
+                        const int col0 = tile_col(ln, S, t) + static_cast<int>(rank) * (width / CG);
                         if (MODE == MODE_LOGITS && CG == 1 && p.half_tiles) {
                             load(smemA + stage * A_STAGE_BYTES, &p.tmA0, kb * BK, 0);
                             load(smemA + stage * A_STAGE_BYTES + A_STAGE_BYTES / 2, &p.tmA1, kb * BK, 0);
@@ -592,15 +609,15 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
     } else if (warp == 1) {
         // ===================== MMA issuer =====================
         if (lane == 0 && rank == 0) {
-            constexpr uint32_t idesc = make_idesc_bf16(CG * BM, BN, 0, B_MN_MAJOR ? 1 : 0);
             int stage = 0;
             uint32_t phase = 0;
             int ab = 0;
             uint32_t aphase = 0;
             for_each_item([&](int rt, int ln, int S, int, int kb0, int kb1) {
                 const int t0 = first_tile(rt, ln);
-                const int nt = (p.col_tiles - ln + S - 1) / S;
+                const int nt = tiles_of(ln, S);
                 for (int t = t0; t < nt; ++t) {
+                    const uint32_t idesc = make_idesc_bf16(CG * BM, tile_width(t), 0, B_MN_MAJOR ? 1 : 0);
                     if (!wait_barrier(tempty_bar(ab), aphase ^ 1u, abort_flag, p.status, 2)) return false;
                     tc_fence_after_sync();
                     const uint32_t d_tmem = tmem_base + ab * BN;
@@ -733,18 +750,17 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                 if (r_own < p.z_rows) zrow = z + static_cast<long long>(r_own) * p.z_pitch;
             }
             const int t0 = first_tile(rt, ln);
-            const int nt = (p.col_tiles - ln + S - 1) / S;
+            const int nt = tiles_of(ln, S);
             // lanes of three tiles and more share their bounds (see below)
             const bool joint = HAS_TOPK && !USE_REG && p.bounds != nullptr && p.col_tiles > 2 * S;
             for (int t = t0; t < nt; ++t) {
-                const int ct = t < 0 ? 0 : ln + t * S;
                 // the whole warp must agree before the warp-collective TMEM loads below
                 const bool ready = wait_barrier(tfull_bar(ab), aphase, abort_flag, p.status, 4);
                 if (!__all_sync(0xffffffffu, ready)) return false;
                 if (MODE == MODE_OUT && CG == 1 && slot == SHARED_TILE) return false;      // finished below, with the cluster
                 tc_fence_after_sync();
                 const uint32_t t_row = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + ab * BN;
-                const int col_base = ct * BN;
+                const int col_base = tile_col(ln, S, t);
                 const bool skip_tile = t < 0 || !tile_ok;
                 if (CAPTURE && spill && t == 0) {
                     ref2 = 0.f;
@@ -845,7 +861,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                     }
                 }
 #pragma unroll 1
-                for (int ch = 0; ch < BN / 32 && !skip_tile; ++ch) {
+                for (int ch = 0; ch < tile_width(t) / 32 && !skip_tile; ++ch) {
                     if (MODE == MODE_STATS && !USE_REG && want_topk) {
                         // make room for a whole chunk in every row's buffer (warp-uniform control flow), before the
                         // chunk's logits occupy registers
@@ -873,7 +889,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                         }
                     }
                     if (MODE == MODE_LOGITS) {
-                        if (zrow != nullptr) {
+                        if (zrow != nullptr && col0 < p.z_pitch) {
 #pragma unroll
                             for (int g8 = 0; g8 < 4; ++g8)
                                 st_global_v8(zrow + col0 + 8 * g8, r[8 * g8], r[8 * g8 + 1], r[8 * g8 + 2], r[8 * g8 + 3],
