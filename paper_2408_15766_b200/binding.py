@@ -1,4 +1,7 @@
-"""ctypes binding of libhass_b200.so. See include/hass.h for the contract of every call."""
+"""ctypes binding of libhass_b200.so. See include/hass.h for the contract of every call.
+
+The calls of a training step have a native form of the plain case (csrc/host_calls.cpp: tensors on the GPU, a workspace given,
+outputs made by the call); everything else, and every refusal, is the Python below it."""
 from __future__ import annotations
 
 import ctypes
@@ -84,6 +87,21 @@ def _load() -> ctypes.CDLL:
 lib = _load()
 
 
+def _load_host(L: ctypes.CDLL):
+    path = os.path.join(_HERE, "hass_host.so")
+    if not os.path.exists(path):
+        raise ImportError(f"{path} is missing: build it with `python paper_2408_15766_b200/build.py`. There is no fallback path.")
+    from . import hass_host
+    names = ("hass_topk_distill_fwd", "hass_topk_distill_fwd_draft", "hass_topk_distill_bwd", "hass_topk_distill_fwd_bwd",
+             "hass_topk_distill_fwd_bwd_draft", "hass_combined_distill_fwd_bwd", "hass_variant_distill_fwd_bwd",
+             "hass_hca_attention_fwd", "hass_hca_attention_bwd")
+    hass_host.bind(*(ctypes.cast(getattr(L, n), ctypes.c_void_p).value for n in names))
+    return hass_host
+
+
+_host = _load_host(lib)
+
+
 def status_string(status: int) -> str:
     return lib.hass_status_string(int(status)).decode()
 
@@ -99,6 +117,19 @@ def kernel_launch_count() -> int:
 def _ok(status: int, where: str) -> None:
     if status != 0:
         raise HassError(status, where)
+
+
+def _handle(stream) -> Optional[int]:
+    return None if stream is None else stream.cuda_stream
+
+
+def _native(got, workspace, where: str) -> Optional[dict]:
+    """What a native call returned: its outputs with the workspace, HassError for a status, None for a call that is not its own."""
+    if type(got) is int:
+        raise HassError(got, where)
+    if got is not None:
+        got["workspace"] = workspace
+    return got
 
 
 def _p(t: Optional[torch.Tensor]) -> Optional[int]:
@@ -143,6 +174,9 @@ def _dh_dtype(code: int):
 
 
 def topk_distill_fwd(H_t, H_d, W, K: int, workspace=None, stream=None) -> dict:
+    got = _native(_host.topk_distill_fwd(H_t, H_d, W, K, workspace, _handle(stream)), workspace, "hass_topk_distill_fwd")
+    if got is not None:
+        return got
     N, d, V = _dims(H_t, W)
     assert H_d.shape == H_t.shape and H_d.dtype == torch.bfloat16 and H_d.is_contiguous()
     dev = H_t.device
@@ -192,6 +226,10 @@ def topk_distill_fwd_static(H_t, H_d, W, K: int, stream=None, out: Optional[dict
 
 
 def topk_distill_fwd_draft(H_d, W, topk_idx, topk_q, workspace=None, stream=None) -> dict:
+    got = _native(_host.topk_distill_fwd_draft(H_d, W, topk_idx, topk_q, workspace, _handle(stream)), workspace,
+                  "hass_topk_distill_fwd_draft")
+    if got is not None:
+        return got
     N, d, V = _dims(H_d, W)
     K = topk_idx.shape[1]
     assert topk_idx.dtype == torch.int32 and topk_q.dtype == torch.float32
@@ -208,6 +246,11 @@ def topk_distill_fwd_draft(H_d, W, topk_idx, topk_q, workspace=None, stream=None
 
 def topk_distill_bwd(H_d, W, topk_idx, topk_q, lse_d, grad_loss=None, dH_dtype: int = HASS_BF16, workspace=None,
                      stream=None, out=None) -> torch.Tensor:
+    if out is None:
+        got = _native(_host.topk_distill_bwd(H_d, W, topk_idx, topk_q, lse_d, grad_loss, dH_dtype, workspace, _handle(stream)),
+                      workspace, "hass_topk_distill_bwd")
+        if got is not None:
+            return got["dH_d"]
     N, d, V = _dims(H_d, W)
     K = topk_idx.shape[1]
     assert topk_idx.dtype == torch.int32 and topk_q.dtype == torch.float32 and lse_d.dtype == torch.float32
@@ -223,6 +266,11 @@ def topk_distill_bwd(H_d, W, topk_idx, topk_q, lse_d, grad_loss=None, dH_dtype: 
 
 def topk_distill_fwd_bwd(H_t, H_d, W, K: int, grad_loss=None, dH_dtype: int = HASS_BF16, workspace=None,
                          stream=None, out: Optional[dict] = None) -> dict:
+    if out is None:
+        got = _native(_host.topk_distill_fwd_bwd(H_t, H_d, W, K, grad_loss, dH_dtype, workspace, _handle(stream)), workspace,
+                      "hass_topk_distill_fwd_bwd")
+        if got is not None:
+            return got
     N, d, V = _dims(H_t, W)
     assert H_d.shape == H_t.shape and H_d.dtype == torch.bfloat16 and H_d.is_contiguous()
     assert grad_loss is None or (grad_loss.dtype == torch.float32 and grad_loss.shape == (N,))
@@ -245,6 +293,11 @@ def topk_distill_fwd_bwd(H_t, H_d, W, K: int, grad_loss=None, dH_dtype: int = HA
 
 def topk_distill_fwd_bwd_draft(H_d, W, topk_idx, topk_q, grad_loss=None, dH_dtype: int = HASS_BF16, workspace=None,
                                stream=None, out: Optional[dict] = None) -> dict:
+    if out is None:
+        got = _native(_host.topk_distill_fwd_bwd_draft(H_d, W, topk_idx, topk_q, grad_loss, dH_dtype, workspace, _handle(stream)),
+                      workspace, "hass_topk_distill_fwd_bwd_draft")
+        if got is not None:
+            return got
     N, d, V = _dims(H_d, W)
     K = topk_idx.shape[1]
     assert topk_idx.dtype == torch.int32 and topk_q.dtype == torch.float32
@@ -272,6 +325,11 @@ def combined_distill_workspace_bytes(N: int, d: int, V: int, K: int) -> int:
 def combined_distill_fwd_bwd(H_t, H_d, W, K: int, w_topk: float = 1.0, grad_loss=None, dH_dtype: int = HASS_BF16,
                              workspace=None, stream=None, out: Optional[dict] = None) -> dict:
     """Cross-entropy over the full vocabulary plus w times the Top-K loss, forward and backward."""
+    if out is None:
+        got = _native(_host.combined_distill_fwd_bwd(H_t, H_d, W, K, w_topk, grad_loss, dH_dtype, workspace, _handle(stream)),
+                      workspace, "hass_combined_distill_fwd_bwd")
+        if got is not None:
+            return got
     N, d, V = _dims(H_t, W)
     assert H_d.shape == H_t.shape and H_d.dtype == torch.bfloat16 and H_d.is_contiguous()
     assert grad_loss is None or (grad_loss.dtype == torch.float32 and grad_loss.shape == (N,))
@@ -299,6 +357,10 @@ LOSS_TOPK, LOSS_TOP_P, LOSS_NORMED_TOPK, LOSS_BIDIR_TOPK = 0, 1, 2, 3
 def variant_distill_fwd_bwd(H_t, H_d, W, K: int, variant: int, param: float = 0.0, grad_loss=None,
                             dH_dtype: int = HASS_BF16, workspace=None, stream=None) -> dict:
     """Top-P / Normed Top-K / Top-K loss, forward and backward. See hass_variant_distill_fwd_bwd."""
+    got = _native(_host.variant_distill_fwd_bwd(H_t, H_d, W, K, variant, param, grad_loss, dH_dtype, workspace, _handle(stream)),
+                  workspace, "hass_variant_distill_fwd_bwd")
+    if got is not None:
+        return got
     N, d, V = _dims(H_t, W)
     assert H_d.shape == H_t.shape and H_d.dtype == torch.bfloat16 and H_d.is_contiguous()
     assert grad_loss is None or (grad_loss.dtype == torch.float32 and grad_loss.shape == (N,))
@@ -349,6 +411,10 @@ def hca_attention_fwd(Q, K_t, V_t, K_d=(), V_d=(), scale: Optional[float] = None
                       workspace=None, stream=None) -> dict:
     """HCA attention forward. Q [B, T, H, D]; K_t, V_t and every K_d[i], V_d[i] [B, T, Hkv, D], bf16 CUDA
     tensors; entry i of K_d / V_d replaces the i-th sub-diagonal. See hass_hca_attention_fwd."""
+    got = _native(_host.hca_attention_fwd(Q, K_t, V_t, K_d, V_d, scale, want_lse, workspace, _handle(stream)), workspace,
+                  "hass_hca_attention_fwd")
+    if got is not None:
+        return got
     B, T, H, D = Q.shape
     Hkv = K_t.shape[2]
     m = len(K_d)
@@ -381,6 +447,10 @@ def hca_attention_bwd_workspace_bytes(B: int, T: int, H: int, m: int) -> int:
 def hca_attention_bwd(Q, K_t, V_t, K_d, V_d, O, lse, dO, scale: Optional[float] = None, workspace=None,
                       stream=None) -> dict:
     """HCA attention backward: gradients of every projected input. See hass_hca_attention_bwd."""
+    got = _native(_host.hca_attention_bwd(Q, K_t, V_t, K_d, V_d, O, lse, dO, scale, workspace, _handle(stream)), workspace,
+                  "hass_hca_attention_bwd")
+    if got is not None:
+        return got
     B, T, H, D = Q.shape
     Hkv = K_t.shape[2]
     m = len(K_d)

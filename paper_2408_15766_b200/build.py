@@ -1,9 +1,11 @@
-"""Builds the CUDA library in-tree: paper_2408_15766_b200/libhass_b200.so (sm_100a only)."""
+"""Builds in-tree the CUDA library, paper_2408_15766_b200/libhass_b200.so (sm_100a only), and the binding's native
+calls, paper_2408_15766_b200/hass_host.so (against the installed torch)."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 SRC_DIR = os.path.join(HERE, "csrc")
@@ -11,17 +13,33 @@ LIB = os.path.join(HERE, "libhass_b200.so")
 SOURCES = ["hass_api.cu"]
 # every header under csrc/ and the public header: a change to any of them makes the library stale
 HEADERS = sorted(f for f in os.listdir(SRC_DIR) if f.endswith((".cuh", ".h"))) + [os.path.join("..", "..", "include", "hass.h")]
+HOST = os.path.join(HERE, "hass_host.so")
+HOST_SOURCES = ["host_calls.cpp", os.path.join("..", "..", "include", "hass.h")]
 
 
-def _stale() -> bool:
-    if not os.path.exists(LIB):
+def _stale(out, sources) -> bool:
+    if not os.path.exists(out):
         return True
-    t = os.path.getmtime(LIB)
-    return any(os.path.getmtime(os.path.join(SRC_DIR, f)) > t for f in SOURCES + HEADERS)
+    t = os.path.getmtime(out)
+    return any(os.path.getmtime(os.path.join(SRC_DIR, f)) > t for f in sources)
+
+
+def build_host(force: bool = False) -> str:
+    if not force and not _stale(HOST, HOST_SOURCES):
+        return HOST
+    from torch.utils.cpp_extension import include_paths, library_paths
+    tmp = HOST + f".tmp{os.getpid()}"
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-o", tmp, os.path.join(SRC_DIR, HOST_SOURCES[0])]
+    cmd += ["-I" + p for p in include_paths("cuda") + [sysconfig.get_paths()["include"]]]
+    cmd += ["-L" + p for p in library_paths("cuda")] + ["-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+    subprocess.run(cmd, check=True)
+    os.replace(tmp, HOST)
+    return HOST
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:
-    if not force and not _stale():
+    build_host(force)
+    if not force and not _stale(LIB, SOURCES + HEADERS):
         return LIB
     nvcc = os.environ.get("NVCC", "nvcc")
     tmp = LIB + f".tmp{os.getpid()}"
