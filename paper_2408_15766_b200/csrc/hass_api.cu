@@ -11,7 +11,7 @@
 #include <vector>
 
 #include "../../include/hass.h"
-#include "kernels.cuh"
+#include "row_split_kernel.cuh"
 #include "hca_kernels.cuh"
 #include "hca_pair_kernel.cuh"
 #include "hca_bwd_fused_kernel.cuh"
@@ -565,7 +565,7 @@ static SelectParams select_params(const GemmParams& p, int first_tile, int row_b
 
 static int launch_finalize(const FinalizeParams& f, cudaStream_t st) {
     KernelTimer timer(f.gate ? KIND_CONDITIONAL : KIND_FINALIZE, st);
-    return launch(finalize_kernel, f.rows, FIN_WARPS * 32, 0, st, 1, f);
+    return launch(finalize_kernel, f.rows, FIN_WARPS * 32, gather_smem(f.d), st, 1, f);
 }
 
 // Partial tiles' room of a call: behind the scratch of its row chunks, where the caller says, or (routes without an
@@ -697,6 +697,11 @@ static int forward_impl(bool with_target, const void* H_t, const void* H_d, cons
 }
 
 // ---- backward ---------------------------------------------------------------------------------
+// The backward of at most 128 rows (below); HASS_ERR_UNSUPPORTED: no room for it.
+static int narrow_backward(const void* H_d, const void* W, long long N, long long d, long long V, int K, const int* topk_idx, const float* topk_q,
+                           const float* lse_d, const float* grad_loss, void* dH_d, int dH_dtype, uint8_t* ws, size_t workspace_bytes,
+                           const Layout& L, const DeviceInfo& di, cudaStream_t st);
+
 static int backward_impl(const void* H_d, const void* W, long long N, long long d, long long V, int K,
                          const int* topk_idx, const float* topk_q, const float* lse_d, const float* grad_loss,
                          void* dH_d, int dH_dtype, void* workspace, size_t workspace_bytes, cudaStream_t st) {
@@ -721,6 +726,8 @@ static int backward_impl(const void* H_d, const void* W, long long N, long long 
     int chunk_tiles = L.pref_chunk_tiles;
     if (fit < chunk_tiles) chunk_tiles = even_chunk(static_cast<int>(fit), RT);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
+    rc = narrow_backward(H_d, W, N, d, V, K, topk_idx, topk_q, lse_d, grad_loss, dH_d, dH_dtype, ws, workspace_bytes, L, di, st);
+    if (rc != HASS_ERR_UNSUPPORTED) return rc;
     const PartRoom part = part_room(ws, workspace_bytes, L, chunk_tiles, nullptr, true);
     int* sidx = reinterpret_cast<int*>(ws + L.sidx);
     float* sgq = reinterpret_cast<float*>(ws + L.sgq);
@@ -834,18 +841,42 @@ constexpr long long kKeepBytes = 64ll << 20;
 // kernel bound by reading W cost it time (from a flushed L2 61 rows x 4096 x 32000 118.8 -> 114.8 us, 99 draft rows 117.5 -> 112.6, 100 rows
 // 129.0 -> 124.9); with a head of 0.5 MB it is the same (64 rows x 256 x 1024 30.3 us early, 30.0 late).
 constexpr long long kLateBytes = 16ll << 20;
+// Blocks per row of row_split_kernel and 16-byte pieces of it per thread; blocks = 0: row_kernel, a block per row. As few blocks as
+// leave a thread four pieces (eight of the longest rows), where all of them are resident at once: a block is a chain of about twenty
+// barriers, 7 us and more, so that a second round of them costs as much as row_kernel's longer passes (100 rows x 4096 x 32000 120 us per call
+// on row_kernel, 136 as two rounds; 100 rows x 128256 416 and 474). Per call, from row_kernel: 2 rows x 8192 x 128256 655 -> 635 us, 5 rows x
+// 4096 x 32000, K = 128 99.5 -> 96, 53 rows x 280 x 2179 combined 29.4 -> 26, 2 rows x 1240 x 7791, K = 85 44 -> 39. With four blocks where one
+// or two do, 64 rows x 256 x 1024 22 -> 31; with eight pieces, which 512 threads hold of both rows in 64 registers, 118 rows x 12454
+// Bi-directional 111 -> 123.
+struct RowSplit {
+    int blocks, pieces;
+};
+static RowSplit row_split(long long N, long long pitch, int sms) {
+    for (int c = 1; c <= SPLIT_MAX; c *= 2) {
+        const int e = ceil_div(pitch, static_cast<long long>(c) * SPLIT_STEP);
+        if (e > (c == SPLIT_MAX ? SPLIT_PIECES : SPLIT_PIECES / 2)) continue;
+        if (c * N > sms) break;
+        return RowSplit{c, e > 4 ? SPLIT_PIECES : e > 2 ? 4 : e};
+    }
+    return RowSplit{0, 0};
+}
 struct NarrowRoom {
     float* z = nullptr;      // [N, p_pitch], or nullptr: no room
     float* zt = nullptr;     // [N, p_pitch]
+    float* dz = nullptr;     // the one of the two that dz_d goes over, which lies first
     PartRoom part;
 };
-static NarrowRoom narrow_room(long long N, uint8_t* ws, size_t workspace_bytes, const Layout& L) {
+static NarrowRoom narrow_room(long long N, uint8_t* ws, size_t workspace_bytes, const Layout& L, int sms) {
     NarrowRoom r;
     const size_t z = align256(static_cast<size_t>(N) * L.p_pitch * 4);
     if (N <= BM && workspace_bytes >= L.scratch + 2 * z) {
-        r.z = reinterpret_cast<float*>(ws + L.scratch);
-        r.zt = reinterpret_cast<float*>(ws + L.scratch + z);
-        r.part.at = r.zt;
+        float* const a = reinterpret_cast<float*>(ws + L.scratch);
+        float* const b = reinterpret_cast<float*>(ws + L.scratch + z);
+        const bool split = row_split(N, L.p_pitch, sms).blocks != 0;
+        r.z = split ? b : a;
+        r.zt = split ? a : b;
+        r.dz = a;
+        r.part.at = b;
         r.part.bytes = workspace_bytes - L.scratch - z;
     }
     return r;
@@ -902,24 +933,31 @@ static RowParams row_params(int V, int K, const Layout& L) {
     r.idx_pitch = K;
     return r;
 }
-static int launch_rows(int objective, const RowParams& r, int N, cudaStream_t st) {
+template <int OBJ>
+static int launch_rows_as(RowParams& r, int N, int sms, cudaStream_t st) {
     KernelTimer timer(KIND_FINALIZE, st);
-    if (r.V <= ROW_SMALL && r.K <= ROW_SMALL_K)
-        return launch(objective == ROW_COMBINED ? row_kernel<ROW_COMBINED, ROW_THREADS_SMALL>
-                      : objective == ROW_BIDIR  ? row_kernel<ROW_BIDIR, ROW_THREADS_SMALL>
-                                                : row_kernel<ROW_TOPK, ROW_THREADS_SMALL>,
-                      N, ROW_THREADS_SMALL, 0, st, 1, r);
-    return launch(objective == ROW_COMBINED ? row_kernel<ROW_COMBINED, ROW_THREADS>
-                  : objective == ROW_BIDIR  ? row_kernel<ROW_BIDIR, ROW_THREADS>
-                                            : row_kernel<ROW_TOPK, ROW_THREADS>,
-                  N, ROW_THREADS, 0, st, 1, r);
+    const RowSplit w = row_split(N, r.pitch, sms);
+    if (w.blocks) {
+        r.split = w.blocks;
+        const auto fn = w.pieces == 1   ? row_split_kernel<OBJ, 1>
+                        : w.pieces == 2 ? row_split_kernel<OBJ, 2>
+                        : w.pieces == 4 ? row_split_kernel<OBJ, 4>
+                                        : row_split_kernel<OBJ, SPLIT_PIECES>;
+        return launch(fn, static_cast<long long>(N) * w.blocks, SPLIT_THREADS, 0, st, w.blocks, r);
+    }
+    return launch(row_kernel<OBJ>, N, ROW_THREADS, 0, st, 1, r);
+}
+static int launch_rows(int objective, RowParams& r, int N, int sms, cudaStream_t st) {
+    return objective == ROW_COMBINED ? launch_rows_as<ROW_COMBINED>(r, N, sms, st)
+           : objective == ROW_BIDIR  ? launch_rows_as<ROW_BIDIR>(r, N, sms, st)
+                                     : launch_rows_as<ROW_TOPK>(r, N, sms, st);
 }
 
 static int narrow_impl(int objective, bool with_target, const void* H_t, const void* H_d, const void* W, int N, long long d,
                        long long V, int K, const float* grad_loss, const int* idx_in, const float* q_in, float* loss,
                        int* idx_out, float* q_out, float* lse_t, float* lse_d, void* dH_d, int dH_dtype, uint8_t* ws,
                        const Layout& L, const NarrowRoom& room, const DeviceInfo& di, cudaStream_t st, float top_p, int* topk_n,
-                       const Combined* cmb = nullptr) {
+                       const Combined* cmb = nullptr, const float* lse_in = nullptr) {
     // (1) the logits of the target and draft rows
     int rc = with_target ? narrow_sweep(H_t, H_d, W, N, d, V, room.zt, room.z, ws, L, di, st)
                          : narrow_sweep(H_d, nullptr, W, N, d, V, room.z, nullptr, ws, L, di, st);
@@ -937,6 +975,7 @@ static int narrow_impl(int objective, bool with_target, const void* H_t, const v
     r.lse_t = lse_t;
     r.lse_d = lse_d;
     r.loss = loss;
+    r.lse_in = lse_in;
     r.make_dz = dH_d != nullptr ? 1 : 0;
     r.release_late = V * d * 2 >= kLateBytes ? 1 : 0;
     if (cmb) {
@@ -949,13 +988,14 @@ static int narrow_impl(int objective, bool with_target, const void* H_t, const v
         r.coef_out = reinterpret_cast<float*>(ws + L.coef);
         r.sparse_out = reinterpret_cast<float*>(ws + L.sparse);
     }
-    rc = launch_rows(objective, r, N, st);
+    r.dz = reinterpret_cast<__nv_bfloat16*>(room.dz);
+    rc = launch_rows(objective, r, N, di.sms, st);
     if (rc != HASS_OK) return rc;
     if (dH_d == nullptr) return HASS_OK;      // the forward alone
     // (3) dH_d = dz_d W
     GemmParams o;
     std::memset(&o, 0, sizeof(o));
-    rc = make_tmap(&o.tmA0, room.z, N, V, 2 * L.p_pitch, BK, BM);
+    rc = make_tmap(&o.tmA0, room.dz, N, V, 2 * L.p_pitch, BK, BM);
     if (rc == HASS_OK) rc = make_tmap(&o.tmB, W, V, d, d, 64, BK);
     if (rc != HASS_OK) return rc;
     o.tmA1 = o.tmA0;
@@ -977,6 +1017,18 @@ static int narrow_impl(int objective, bool with_target, const void* H_t, const v
     o.sparse = r.sparse_out;
     o.status = reinterpret_cast<unsigned int*>(ws + L.status);
     return launch_out(o, room.part, di, st);
+}
+
+// lse_d is given: the draft's logits, dz_d and its product with W, as in the fused call. It replaces the sorted sets and the MODE_PROBS
+// sweep, whose epilogue walks them: forward + backward of 11 rows x 3848 x 3306 86 -> 81 us, 61 x 4096 x 32000 163 ->
+// 153, 100 x 256 x 1024 45 -> 32.
+static int narrow_backward(const void* H_d, const void* W, long long N, long long d, long long V, int K, const int* topk_idx, const float* topk_q,
+                           const float* lse_d, const float* grad_loss, void* dH_d, int dH_dtype, uint8_t* ws, size_t workspace_bytes,
+                           const Layout& L, const DeviceInfo& di, cudaStream_t st) {
+    const NarrowRoom room = narrow_room(N, ws, workspace_bytes, L, di.sms);
+    if (!room.z) return HASS_ERR_UNSUPPORTED;
+    return narrow_impl(ROW_TOPK, false, nullptr, H_d, W, static_cast<int>(N), d, V, K, grad_loss, topk_idx, topk_q, nullptr, nullptr, nullptr,
+                       nullptr, nullptr, dH_d, dH_dtype, ws, L, room, di, st, 0.f, nullptr, nullptr, lse_d);
 }
 
 static int fused_impl(bool with_target, const void* H_t, const void* H_d, const void* W, long long N, long long d,
@@ -1013,11 +1065,9 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
     __nv_bfloat16* P = reinterpret_cast<__nv_bfloat16*>(ws + L.scratch);
     unsigned int* status = reinterpret_cast<unsigned int*>(ws + L.status);
     int* idx_d = reinterpret_cast<int*>(ws + L.sidx);
-    // The combined objective takes that route up to 64 rows only: the line was drawn where both fp32 matrices fitted the scratch of one
-    // row tile. There is room up to 128 rows now, and the route would be the faster one there as well (65 rows x 4096 x 32000 254 us as it
-    // is, 123 on that route, 128 rows x 4096 x 128256 675 and 472, 100 rows x 256 x 1024 82 and 37).
-    if (with_target && !(cmb && N > BM / 2)) {
-        const NarrowRoom narrow = narrow_room(N, ws, cmb ? cmb->end : workspace_bytes, L);
+    // (The combined objective too: 65 rows x 4096 x 32000 254 -> 123 us, 128 rows x 4096 x 128256 675 -> 472, 100 x 256 x 1024 82 -> 37.)
+    if (with_target) {
+        const NarrowRoom narrow = narrow_room(N, ws, cmb ? cmb->end : workspace_bytes, L, di.sms);
         if (narrow.z)
             return narrow_impl(cmb ? ROW_COMBINED : bidir ? ROW_BIDIR : ROW_TOPK, true, H_t, H_d, W, static_cast<int>(N), d, V, K, grad_loss,
                                nullptr, nullptr, loss, idx_out, q_out, lse_t, lse_d, dH_d, dH_dtype, ws, L, narrow, di, st, 0.f, topk_n, cmb);
@@ -1292,7 +1342,7 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
     float* coef = reinterpret_cast<float*>(ws + L.coef);
     float* capz = reinterpret_cast<float*>(ws + L.capz);
     float* ref2 = reinterpret_cast<float*>(ws + L.lse2);
-    const NarrowRoom narrow = narrow_room(N, ws, workspace_bytes, L);
+    const NarrowRoom narrow = narrow_room(N, ws, workspace_bytes, L, di.sms);
     if (narrow.z) {
         if (pipe) {
             rc = pipe_in(pipe, H_t, H_d, 0, static_cast<size_t>(N), st);
@@ -1500,7 +1550,7 @@ static int forward2_impl(bool with_target, const void* H_t, const void* H_d, con
                             workspace, workspace_bytes, st);
     const int RT = ceil_div(N, BM), CT = ceil_div(V, BN);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
-    const NarrowRoom narrow = narrow_room(N, ws, workspace_bytes, L);
+    const NarrowRoom narrow = narrow_room(N, ws, workspace_bytes, L, di.sms);
     if (narrow.z)
         return narrow_impl(ROW_TOPK, with_target, H_t, H_d, W, static_cast<int>(N), d, V, K, nullptr, idx_in, q_in, loss, idx_out, q_out,
                            lse_t, lse_d, nullptr, HASS_BF16, ws, L, narrow, di, st, 0.f, nullptr);
@@ -1603,17 +1653,17 @@ static int normed_impl(const void* H_t, const void* H_d, const void* W, long lon
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     GemmParams p;
     std::memset(&p, 0, sizeof(p));
-    const NarrowRoom narrow = narrow_room(N, ws, workspace_bytes, L);
+    const NarrowRoom narrow = narrow_room(N, ws, workspace_bytes, L, di.sms);
     if (narrow.z) {
-        rc = narrow_sweep(H_t, nullptr, W, static_cast<int>(N), d, V, narrow.z, nullptr, ws, L, di, st);
+        rc = narrow_sweep(H_t, nullptr, W, static_cast<int>(N), d, V, narrow.zt, nullptr, ws, L, di, st);
         if (rc != HASS_OK) return rc;
         RowParams r = row_params(static_cast<int>(V), K, L);
-        r.zt = narrow.z;
+        r.zt = narrow.zt;
         r.idx = idx_out;
         r.q = q_out;
         r.n_out = topk_n;
         r.lse_t = lse_t;
-        rc = launch_rows(ROW_TOPK, r, static_cast<int>(N), st);
+        rc = launch_rows(ROW_TOPK, r, static_cast<int>(N), di.sms, st);
         if (rc != HASS_OK) return rc;
     } else {
         rc = plan_launch(RT, CT, di.sms, L.slot_cap, &p.sched);
@@ -1649,28 +1699,22 @@ static int normed_impl(const void* H_t, const void* H_d, const void* W, long lon
         rc = launch_select(sp, di.sms, st);
         if (rc != HASS_OK) return rc;
     }
-    FinalizeParams f;
-    std::memset(&f, 0, sizeof(f));
-    f.sched = p.sched;
+    NormedParams f;
     f.d = static_cast<int>(d);
     f.K = K;
-    f.row_begin = 0;
-    f.rows = static_cast<int>(N);
-    f.row_tiles_t = RT;
-    f.part_m = p.part_m;
-    f.part_s = p.part_s;
     f.H_d = static_cast<const __nv_bfloat16*>(H_d);
     f.W = static_cast<const __nv_bfloat16*>(W);
-    f.loss = loss;
     f.idx = idx_out;
     f.q = q_out;
-    f.idx_pitch = K;
-    f.lse_t = lse_t;
     f.grad_loss = grad_loss;
-    f.normed = 1;
-    f.dH_out = dH_d;
+    f.loss = loss;
+    f.dH = dH_d;
     f.dH_fp32 = dH_dtype == HASS_FP32 ? 1 : 0;
-    return launch_finalize(f, st);
+    // as many blocks per row as are resident at once, of 256 columns at least
+    f.split = 1;
+    while (f.split < NORMED_MAX && 2 * f.split * N <= 3ll * di.sms && d >= 512ll * f.split) f.split *= 2;
+    KernelTimer timer(KIND_FINALIZE, st);
+    return launch(normed_kernel, N * f.split, NORMED_THREADS, gather_smem(ceil_div(d / 8, f.split) * 8), st, f.split, f);
 }
 
 }  // namespace hass

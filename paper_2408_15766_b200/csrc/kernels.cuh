@@ -1352,7 +1352,7 @@ struct FinalizeParams {
     int* idx;              // [N, idx_pitch] Omega_hat in descending q, from select_kernel or the caller
     float* q;              // (bidir: the joining tokens are added behind the K of the target)
     int idx_pitch;
-    const float* lse_t;    // (read by the combined objective, Normed and Bi-directional Top-K)
+    const float* lse_t;    // (read by the combined objective and Bi-directional Top-K)
     float* loss;
     float* lse_d;
     // fused backward (all nullable): per-row scale of the spilled tiles and the Omega_hat term
@@ -1368,10 +1368,6 @@ struct FinalizeParams {
                            // the bf16 spill; its largest terms are put back in fp32
     // loss variants of Section 4.3
     int* n_out;            // [N] |Omega_hat| (bidir, nullable)
-    int normed;            // 1: Normed Top-K - q, p renormalised over Omega_hat; no draft sweep exists, and the
-                           // gradient row sum_x g (pn(x) - qn(x)) W[x,:] goes straight to dH_out
-    void* dH_out;          // [N, d] (normed only)
-    int dH_fp32;
     const int* idx_d;      // bidir: [N, K] the draft's K most probable tokens in descending p; those outside the target's
                            // set join Omega_hat (idx / q have 2K entries per row)
     const __nv_bfloat16* H_t;   // target features (bidir: target logits of the draft's tokens)
@@ -1419,6 +1415,114 @@ __device__ __forceinline__ void unpack8(const uint4& v, float (&f)[8]) {
     }
 }
 
+// Dynamic shared memory of a kernel that gathers parts of `cols` columns: the groups' sums, where there are groups (with wide rows the
+// space is left to the L1)
+__host__ __device__ constexpr int gather_smem(int cols) { return cols <= FIN_WARPS * 32 * 4 ? 8 * FIN_WARPS * 32 * 4 : 0; }
+
+// Eight columns of the rows of W of tokens tok[0 .. n), n <= FIN_GRP: dot[j] += <h, row j>, a += gw q[j] row j (q nullable).
+__device__ __forceinline__ void gather_unit(const __nv_bfloat16* W, long long d, const int* tok, int n, const float (&h)[8], float (&dot)[FIN_GRP],
+                                            const float* q, float gw, float (&a)[8]) {
+    uint4 wv[FIN_GRP];
+#pragma unroll
+    for (int jj = 0; jj < FIN_GRP; ++jj)
+        if (jj < n) wv[jj] = *reinterpret_cast<const uint4*>(W + tok[jj] * d);
+#pragma unroll
+    for (int jj = 0; jj < FIN_GRP; ++jj) {
+        if (jj < n) {
+            float wf[8];
+            unpack8(wv[jj], wf);
+            const float gq = q ? gw * q[jj] : 0.f;
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                dot[jj] = fmaf(h[t], wf[t], dot[jj]);
+                a[t] = fmaf(gq, wf[t], a[t]);
+            }
+        }
+    }
+}
+
+// Block-collective: over the columns 8 u0 .. 8 u1 - 1, the dot products of row `from` with the rows of W of tokens [b0, n) into to[b0 .. n), and
+// with `so` the row sum over [0, n) of gw q[j] W[tok[j], :] into so (then b0 = 0). FIN_GRP rows of W are in flight per thread. Of narrow rows
+// groups of threads take FIN_GRP tokens each, with their columns' sums in registers to the end (one group had a warp of eight at work on 256
+// columns: Bi-directional call of 2795 rows x 256 x 1024, K = 41 223 -> 183 us, combined 1318 x 376 x 38201, K = 65 658 -> 621).
+__device__ __forceinline__ void gather_rows(const __nv_bfloat16* from, const __nv_bfloat16* W, int d, int u0, int u1, const int* tok, int b0, int n,
+                                            float* to, const float* q, float gw, float* so, float (&part)[FIN_WARPS][FIN_GRP], float* cols) {
+    constexpr int THREADS = FIN_WARPS * 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int per = max(32, min((u1 - u0 + 31) / 32 * 32, THREADS)), groups = THREADS / per, g = tid / per;
+    // the sums of a group's dot products over its threads
+    auto finish = [&](float (&dot)[FIN_GRP], int b, int each) {
+        // eight sums over the warp at once: at each step half of the values go to the other half of the lanes
+        static_assert(FIN_GRP == 8, "lane bits 4, 3, 2 say which sum");
+#pragma unroll
+        for (int h = 4; h > 0; h >>= 1) {
+            const bool up = (lane & (4 * h)) != 0;
+#pragma unroll
+            for (int i = 0; i < h; ++i) {
+                const float other = __shfl_xor_sync(0xffffffffu, up ? dot[i] : dot[i + h], 4 * h);
+                dot[i] = (up ? dot[i + h] : dot[i]) + other;
+            }
+        }
+        dot[0] += __shfl_xor_sync(0xffffffffu, dot[0], 2);
+        dot[0] += __shfl_xor_sync(0xffffffffu, dot[0], 1);
+        if ((lane & 3) == 0) part[warp][lane >> 2] = dot[0];
+        __syncthreads();
+        if (tid < groups * each && b + tid < n) {
+            float acc = 0.f;
+            for (int w = 0; w < per / 32; ++w) acc += part[tid / each * (per / 32) + w][tid % each];
+            to[b + tid] = acc;
+        }
+        __syncthreads();
+    };
+    if (groups == 1) {
+        for (int b = b0; b < n; b += FIN_GRP) {
+            float dot[FIN_GRP] = {};
+            for (int at = u0 + tid; at < u1; at += THREADS) {
+                float h[8], a[8] = {};
+                unpack8(*reinterpret_cast<const uint4*>(from + 8 * at), h);
+                float4* s4 = reinterpret_cast<float4*>(so + 8 * at);
+                if (so && b > 0) {
+                    const float4 a0 = s4[0], a1 = s4[1];
+                    a[0] = a0.x; a[1] = a0.y; a[2] = a0.z; a[3] = a0.w;
+                    a[4] = a1.x; a[5] = a1.y; a[6] = a1.z; a[7] = a1.w;
+                }
+                gather_unit(W + 8 * at, d, tok + b, n - b, h, dot, so ? q + b : nullptr, gw, a);
+                if (so) {
+                    s4[0] = make_float4(a[0], a[1], a[2], a[3]);
+                    s4[1] = make_float4(a[4], a[5], a[6], a[7]);
+                }
+            }
+            finish(dot, b, FIN_GRP);
+        }
+        return;
+    }
+    const int u = u0 + tid - g * per;
+    const bool mine = g < groups && u < u1;
+    float h[8] = {}, a[8] = {};
+    if (mine) unpack8(*reinterpret_cast<const uint4*>(from + 8 * u), h);
+    for (int b = b0; b < n; b += groups * FIN_GRP) {
+        const int each = min((n - b + groups - 1) / groups, FIN_GRP), bg = b + g * each;      // a group's tokens, this group's first
+        float dot[FIN_GRP] = {};
+        if (mine) gather_unit(W + 8 * u, d, tok + bg, min(n - bg, each), h, dot, so ? q + bg : nullptr, gw, a);
+        finish(dot, b, each);
+    }
+    if (so) {
+        // the groups' sums in order
+#pragma unroll
+        for (int t = 0; t < 8; ++t) cols[t * THREADS + tid] = a[t];
+        __syncthreads();
+        if (g == 0 && mine) {
+            for (int o = 1; o < groups; ++o)
+#pragma unroll
+                for (int t = 0; t < 8; ++t) a[t] += cols[t * THREADS + tid + o * per];
+            float4* s4 = reinterpret_cast<float4*>(so + 8 * u);
+            s4[0] = make_float4(a[0], a[1], a[2], a[3]);
+            s4[1] = make_float4(a[4], a[5], a[6], a[7]);
+        }
+        __syncthreads();
+    }
+}
+
 // One block per row (2048 rows, 20 tokens, d = 4096: 390 us with a warp per row and a serial selection -> 158 us, and 24 us
 // in select_kernel; 1024 rows, 10 tokens: 144 -> 55 us; with eight warps instead of four, eight tokens instead of sixteen
 // and three blocks per SM another 10-20 %): bound by the latency of the gathered rows of W, so that a row's columns are spread over FIN_WARPS
@@ -1430,6 +1534,7 @@ __global__ void __launch_bounds__(FIN_WARPS * 32, 3) finalize_kernel(const __gri
     __shared__ float sh_q[K_CAP];
     __shared__ float sh_dot[K_CAP];       // z_d at Omega_hat
     __shared__ float sh_part[FIN_WARPS][FIN_GRP];
+    extern __shared__ float sh_cols[];
     __shared__ int sh_n;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int local = blockIdx.x;
@@ -1442,14 +1547,11 @@ __global__ void __launch_bounds__(FIN_WARPS * 32, 3) finalize_kernel(const __gri
         return v;
     };
 
-    // draft statistics (the Normed Top-K variant has none: it needs the draft logits on Omega_hat only)
-    float lse_d = 0.f, m_spill = 0.f;
+    // draft statistics
     int slot0, S;
-    if (!p.normed) {
-        find_slots(p.sched, p.row_tiles_t + rt, slot0, S);
-        lse_d = warp_lse(p.part_m, p.part_s, slot0, S, r, lane);
-        m_spill = p.part_m[static_cast<long long>(slot0) * BM + r];
-    }
+    find_slots(p.sched, p.row_tiles_t + rt, slot0, S);
+    const float lse_d = warp_lse(p.part_m, p.part_s, slot0, S, r, lane);
+    const float m_spill = p.part_m[static_cast<long long>(slot0) * BM + r];
     const float g = p.grad_loss ? p.grad_loss[row] : 1.f;
     const bool combined = p.coef_t_out != nullptr;
     float coef_t = 0.f;
@@ -1467,59 +1569,6 @@ __global__ void __launch_bounds__(FIN_WARPS * 32, 3) finalize_kernel(const __gri
         sh_q[j] = p.q[io + j];
     }
     __syncthreads();
-
-    // The dot products of `from`'s row with the W rows of tokens [b, b + n), n <= FIN_GRP, summed over the block into
-    // `to`; with `so` also the row sum of gw q(x) W[x, :], added to what is there when b > 0.
-    auto gather = [&](const __nv_bfloat16* from, int b, int n, float* to, float* so) {
-        float dot[FIN_GRP];
-#pragma unroll
-        for (int jj = 0; jj < FIN_GRP; ++jj) dot[jj] = 0.f;
-        for (int k0 = tid * 8; k0 < p.d; k0 += FIN_WARPS * 256) {
-            float h[8];
-            unpack8(*reinterpret_cast<const uint4*>(from + k0), h);
-            float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            if (so && b > 0) {
-                const float4 a0 = *reinterpret_cast<const float4*>(so + k0);
-                const float4 a1 = *reinterpret_cast<const float4*>(so + k0 + 4);
-                a[0] = a0.x; a[1] = a0.y; a[2] = a0.z; a[3] = a0.w;
-                a[4] = a1.x; a[5] = a1.y; a[6] = a1.z; a[7] = a1.w;
-            }
-            uint4 wv[FIN_GRP];
-#pragma unroll
-            for (int jj = 0; jj < FIN_GRP; ++jj)
-                if (jj < n) wv[jj] = *reinterpret_cast<const uint4*>(p.W + static_cast<long long>(sh_tok[b + jj]) * p.d + k0);
-#pragma unroll
-            for (int jj = 0; jj < FIN_GRP; ++jj) {
-                if (jj < n) {
-                    float wf[8];
-                    unpack8(wv[jj], wf);
-                    const float gq = so ? gw * sh_q[b + jj] : 0.f;
-#pragma unroll
-                    for (int t = 0; t < 8; ++t) {
-                        dot[jj] = fmaf(h[t], wf[t], dot[jj]);
-                        a[t] = fmaf(gq, wf[t], a[t]);
-                    }
-                }
-            }
-            if (so) {
-                *reinterpret_cast<float4*>(so + k0) = make_float4(a[0], a[1], a[2], a[3]);
-                *reinterpret_cast<float4*>(so + k0 + 4) = make_float4(a[4], a[5], a[6], a[7]);
-            }
-        }
-#pragma unroll
-        for (int jj = 0; jj < FIN_GRP; ++jj) {
-            const float acc = warp_sum(dot[jj]);
-            if (lane == 0) sh_part[warp][jj] = acc;
-        }
-        __syncthreads();
-        if (tid < n) {
-            float acc = 0.f;
-#pragma unroll
-            for (int w = 0; w < FIN_WARPS; ++w) acc += sh_part[w][tid];
-            to[b + tid] = acc;
-        }
-        __syncthreads();
-    };
 
     int Ku = K;                                       // |Omega_hat| (2K at most for the bi-directional set)
     if (p.idx_d != nullptr) {
@@ -1541,8 +1590,7 @@ __global__ void __launch_bounds__(FIN_WARPS * 32, 3) finalize_kernel(const __gri
         Ku = sh_n;
         // their target probabilities: q = exp(<H_t[row], W[tok]> - lse_t)
         const float lse_t = p.lse_t[row];
-        for (int b = K; b < Ku; b += FIN_GRP)
-            gather(p.H_t + static_cast<long long>(row) * p.d, b, Ku - b < FIN_GRP ? Ku - b : FIN_GRP, sh_q, nullptr);
+        gather_rows(p.H_t + static_cast<long long>(row) * p.d, p.W, p.d, 0, p.d / 8, sh_tok, K, Ku, sh_q, nullptr, 0.f, nullptr, sh_part, sh_cols);
         for (int j = K + tid; j < 2 * K; j += FIN_WARPS * 32) {
             const float qv = j < Ku ? expf(sh_q[j] - lse_t) : 0.f;
             if (j < Ku) sh_q[j] = qv;
@@ -1553,54 +1601,12 @@ __global__ void __launch_bounds__(FIN_WARPS * 32, 3) finalize_kernel(const __gri
         __syncthreads();
     }
     // draft logits at Omega_hat and, for the fused backward, the row sum_{x in Omega_hat} g q(x) W[x, :]
-    float* so = (p.sparse_out && !p.normed) ? p.sparse_out + static_cast<long long>(local) * p.d : nullptr;
-    for (int b = 0; b < Ku; b += FIN_GRP) gather(hrow, b, Ku - b < FIN_GRP ? Ku - b : FIN_GRP, sh_dot, so);
+    float* so = p.sparse_out ? p.sparse_out + static_cast<long long>(local) * p.d : nullptr;
+    gather_rows(hrow, p.W, p.d, 0, p.d / 8, sh_tok, 0, Ku, sh_dot, sh_q, gw, so, sh_part, sh_cols);
 
     float S_q = 0.f;
     for (int j = lane; j < Ku; j += 32) S_q += sh_q[j];
     S_q = warp_sum(S_q);
-    if (p.normed) {
-        // Normed Top-K: qn = q / S_q, pn = softmax of the draft logits restricted to Omega_hat
-        float mx = -INFINITY;
-        for (int j = lane; j < K; j += 32) mx = fmaxf(mx, sh_dot[j]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        float se = 0.f;
-        for (int j = lane; j < K; j += 32) se += expf(sh_dot[j] - mx);
-        const float lse_k = mx + logf(warp_sum(se));
-        float ln = 0.f;
-        for (int j = lane; j < K; j += 32) ln += sh_q[j] / S_q * (lse_k - sh_dot[j]);
-        ln = warp_sum(ln);
-        __syncthreads();
-        for (int j = tid; j < K; j += FIN_WARPS * 32)
-            sh_dot[j] = g * (expf(sh_dot[j] - lse_k) - sh_q[j] / S_q);      // dL/dz_d on Omega_hat
-        __syncthreads();
-        for (int k0 = tid * 8; k0 < p.d; k0 += FIN_WARPS * 256) {
-            float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll 8
-            for (int j = 0; j < K; ++j) {
-                const float c = sh_dot[j];
-                float wf[8];
-                unpack8(*reinterpret_cast<const uint4*>(p.W + static_cast<long long>(sh_tok[j]) * p.d + k0), wf);
-#pragma unroll
-                for (int t = 0; t < 8; ++t) a[t] = fmaf(c, wf[t], a[t]);
-            }
-            if (p.dH_fp32) {
-                float* o = reinterpret_cast<float*>(p.dH_out) + static_cast<long long>(row) * p.d + k0;
-                *reinterpret_cast<float4*>(o) = make_float4(a[0], a[1], a[2], a[3]);
-                *reinterpret_cast<float4*>(o + 4) = make_float4(a[4], a[5], a[6], a[7]);
-            } else {
-                uint4 w;
-                w.x = pack_bf16x2(a[0], a[1]);
-                w.y = pack_bf16x2(a[2], a[3]);
-                w.z = pack_bf16x2(a[4], a[5]);
-                w.w = pack_bf16x2(a[6], a[7]);
-                *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.dH_out) + static_cast<long long>(row) * p.d + k0) = w;
-            }
-        }
-        if (tid == 0) p.loss[row] = ln;
-        return;
-    }
     if (warp == 0) {
         float loss = 0.f, ce_corr = 0.f;
         for (int j = lane; j < Ku; j += 32) {
@@ -2077,15 +2083,12 @@ __global__ void __launch_bounds__(256) loss_patch_kernel(const __grid_constant__
 // maxima bounds the row's K-th largest from below. Little more than K logits reach it; the threads that hold them read their
 // share again and put them into a pool in shared memory, where each counts those above it (more than it takes: collect_from_many).
 // Bound by the latency of two passes over rows of 4 V bytes in L2: 1024 threads with ROW_LOADS 16-byte loads each in flight.
-// Rows of up to ROW_SMALL logits, one load each for 256 threads, are bound by the barriers instead and take 256: 64 rows x 256 x
-// 1024 25.9 -> 25.0 us per call, 104 rows 26.8 -> 25.6. (Of 2000 logits, K = 30 22.2 -> 22.5, 4096, K = 64 34.1 -> 36.2. K is a
-// quarter of the maxima at most: the bound of a larger set admits much of the row.)
-constexpr int ROW_THREADS = 1024, ROW_THREADS_SMALL = 256;
-constexpr int ROW_SMALL = 1024, ROW_SMALL_K = 64;
+// It takes the rows that row_split_kernel does not (row_split in the host code): those of more than 8192 logits, when they are many.
+constexpr int ROW_THREADS = 1024;
 constexpr int ROW_LOADS = 4;
 constexpr int ROW_POOL = 1024;
 constexpr int ROW_SLACK = 32;      // maxima beyond K at which the search of the bound ends
-static_assert(ROW_POOL >= K_CAP && ROW_THREADS_SMALL >= K_CAP, "room for Omega_hat, a thread for each of its tokens");
+static_assert(ROW_POOL >= K_CAP && ROW_THREADS >= K_CAP, "room for Omega_hat, a thread for each of its tokens");
 enum { ROW_TOPK = 0, ROW_COMBINED = 1, ROW_BIDIR = 2 };
 
 struct RowParams {
@@ -2102,8 +2105,11 @@ struct RowParams {
     float* lse_t;
     float* lse_d;
     float* loss;
+    const float* lse_in;   // nullable: [N] lse_d, given (the separate backward: dz_d alone, neither loss nor lse_d is written)
     int make_dz;
     int release_late;      // as in GemmParams
+    int split;             // row_split_kernel: blocks per row
+    __nv_bfloat16* dz;     // row_split_kernel: [N, 2 pitch] dz_d; may be the target's logits, not the draft's
     float w;               // ROW_COMBINED
     float* loss_ce;
     const __nv_bfloat16* W;      // ROW_BIDIR: [V, d]
@@ -2112,17 +2118,32 @@ struct RowParams {
     float* sparse_out;     // [N, d]
 };
 
-struct RowShared {
+// The separate backward's set is the caller's and may name a token more than once: what its first entry takes off for all of them,
+// and 0 for the others (n entries; q of entry j).
+__device__ __forceinline__ float repeated_q(const int* tok, const float* q, int n, int j) {
+    float sum = 0.f;
+    for (int i = 0; i < n; ++i) {
+        if (tok[i] != tok[j]) continue;
+        if (i < j && q[i] != 0.f) return 0.f;
+        sum += q[i];
+    }
+    return sum;
+}
+
+struct RowPool {           // of a block that looks for the K largest logits of a row, or of its piece of one
     unsigned long long pool[ROW_POOL];
     float red[4][32];
     uint32_t key_min[32];
+    int n;
+    int reach[3], equal[32];
+};
+struct RowShared : RowPool {
     int tok[K_CAP];        // Omega_hat
     float q[K_CAP], z[K_CAP];
     int tok_d[K_CAP];      // the draft's own K largest (ROW_BIDIR)
     float z_d[K_CAP];
     float sum;
-    int n, count;
-    int reach[3], equal[32];
+    int count;
 };
 
 // One logit as a number: larger = larger logit, lower token id first among equal ones (-0 and +0 are equal).
@@ -2207,9 +2228,9 @@ __device__ __forceinline__ float block_lse(float m, float s, float (*red)[32]) {
 __device__ __forceinline__ int pool_room(int K) { return min(4 * (K + ROW_SLACK), ROW_POOL); }
 
 // Block-collective: the logits that reach `bound` into the pool, by the threads whose maximum `key` does; given up when they are
-// more than `room` (then sh.n > room).
+// more than `room` (then sh.n > room). (row, pitch, V): a row, or the piece of it that begins with token `first`.
 template <int THREADS>
-__device__ __forceinline__ void collect(const float* row, long long pitch, int V, uint32_t key, uint32_t bound, int room, RowShared& sh) {
+__device__ __forceinline__ void collect(const float* row, long long pitch, int V, int first, uint32_t key, uint32_t bound, int room, RowPool& sh) {
     auto full = [&] { return *static_cast<volatile int*>(&sh.n) > room; };
     if (key >= bound)
         for_own_logits_while<THREADS>(row, pitch, [&](long long at, const float4& v) {
@@ -2219,7 +2240,7 @@ __device__ __forceinline__ void collect(const float* row, long long pitch, int V
             for (int j = 0; j < 4; ++j)
                 if (reaches(z[j], at + j, V, bound)) {
                     const int pos = atomicAdd(&sh.n, 1);
-                    if (pos < room) sh.pool[pos] = logit_rank(z[j], static_cast<uint32_t>(at + j));
+                    if (pos < room) sh.pool[pos] = logit_rank(z[j], static_cast<uint32_t>(first + at + j));
                 }
         }, [&] { return !full(); });
     __syncthreads();
@@ -2233,7 +2254,7 @@ __device__ __forceinline__ void collect(const float* row, long long pitch, int V
 // 1024 83 -> 30 (a search of token ids bit by bit, a pass over the row for each, and 1024 equal logits ranked).
 // Returns the entries left in the pool. (A function of its own: in line it costs row_kernel registers that it does not have.)
 template <int THREADS>
-__device__ __noinline__ int collect_from_many(const float* row, long long pitch, int V, int K, uint32_t key, uint32_t T, uint32_t hi, RowShared& sh) {
+__device__ __noinline__ int collect_from_many(const float* row, long long pitch, int V, int first, int K, uint32_t key, uint32_t T, uint32_t hi, RowPool& sh) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     auto count = [&](uint32_t t1, uint32_t t2, uint32_t t3) {
         __syncthreads();
@@ -2284,7 +2305,7 @@ __device__ __noinline__ int collect_from_many(const float* row, long long pitch,
     __syncthreads();
     if (tid == 0) sh.n = 0;
     __syncthreads();
-    collect<THREADS>(row, pitch, V, key, exact ? T + 1u : T, pool_room(K), sh);
+    collect<THREADS>(row, pitch, V, first, key, exact ? T + 1u : T, pool_room(K), sh);
     int n = sh.n;
     if (exact) {
         // fewer than K lie above it; of those equal to it the first in token order
@@ -2315,7 +2336,7 @@ __device__ __noinline__ int collect_from_many(const float* row, long long pitch,
 #pragma unroll
             for (int j = 0; j < 4; ++j)
                 if (in[j]) {
-                    if (pos < K) sh.pool[pos] = logit_rank(z[j], static_cast<uint32_t>(at + j));
+                    if (pos < K) sh.pool[pos] = logit_rank(z[j], static_cast<uint32_t>(first + at + j));
                     ++pos;
                 }
         }
@@ -2325,40 +2346,47 @@ __device__ __noinline__ int collect_from_many(const float* row, long long pitch,
     return n;
 }
 
-// Block-collective: the K largest logits of the row, in descending order (lower token id first among equal ones), into
-// tok / val; m = this thread's largest logit. Fewer than K logits above -inf: the rest is token 0 at -inf.
+// Block-collective: a bound that K of the threads' largest logits reach (m = this thread's), as an ordered key, or 1 where fewer
+// threads have one above -inf; key = this thread's, hi = the largest. Leaves the pool empty.
 template <int THREADS>
-__device__ __forceinline__ void select_largest(const float* row, long long pitch, int V, int K, float m, RowShared& sh, int* tok, float* val) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t key = m > -INFINITY ? ordered_key(__float_as_uint(m + 0.f)) : 0u;
+__device__ __forceinline__ uint32_t bound_from_maxima(int K, float m, RowPool& sh, uint32_t& key, uint32_t& hi) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    key = m > -INFINITY ? ordered_key(__float_as_uint(m + 0.f)) : 0u;
     const uint32_t key_hi = __reduce_max_sync(0xffffffffu, key), key_lo = __reduce_min_sync(0xffffffffu, key == 0u ? 0xffffffffu : key);
     if (lane == 0) {
         sh.red[0][warp] = __uint_as_float(key_hi);
         sh.key_min[warp] = key_lo;
     }
-    if (tid == 0) sh.n = 0;
+    if (threadIdx.x == 0) sh.n = 0;
     const int groups = __syncthreads_count(key != 0u);
-    const uint32_t hi = __reduce_max_sync(0xffffffffu, lane < THREADS / 32 ? __float_as_uint(sh.red[0][lane]) : 0u);
-    uint32_t T = 1u;
-    if (groups >= K) {
-        // the K-th largest maximum, or a value below it that at most K + ROW_SLACK maxima reach, from the highest bit in which
-        // the maxima differ on
-        const uint32_t lo = __reduce_min_sync(0xffffffffu, lane < THREADS / 32 ? sh.key_min[lane] : 0xffffffffu);
-        int bit = 32 - __clz(hi ^ lo);
-        T = bit < 32 ? hi >> bit << bit : 0u;
-        for (--bit; bit >= 0; --bit) {
-            const uint32_t T1 = T | (1u << bit);
-            const int c = __syncthreads_count(key >= T1);
-            if (c >= K) {
-                T = T1;
-                if (c <= K + ROW_SLACK) break;
-            }
+    hi = __reduce_max_sync(0xffffffffu, lane < THREADS / 32 ? __float_as_uint(sh.red[0][lane]) : 0u);
+    if (groups < K) return 1u;
+    // the K-th largest maximum, or a value below it that at most K + ROW_SLACK maxima reach, from the highest bit in which
+    // the maxima differ on
+    const uint32_t lo = __reduce_min_sync(0xffffffffu, lane < THREADS / 32 ? sh.key_min[lane] : 0xffffffffu);
+    int bit = 32 - __clz(hi ^ lo);
+    uint32_t T = bit < 32 ? hi >> bit << bit : 0u;
+    for (--bit; bit >= 0; --bit) {
+        const uint32_t T1 = T | (1u << bit);
+        const int c = __syncthreads_count(key >= T1);
+        if (c >= K) {
+            T = T1;
+            if (c <= K + ROW_SLACK) break;
         }
-        T = max(T, 1u);
     }
-    collect<THREADS>(row, pitch, V, key, T, pool_room(K), sh);
+    return max(T, 1u);
+}
+
+// Block-collective: the K largest logits of the row, in descending order (lower token id first among equal ones), into
+// tok / val; m = this thread's largest logit. Fewer than K logits above -inf: the rest is token 0 at -inf.
+template <int THREADS>
+__device__ __forceinline__ void select_largest(const float* row, long long pitch, int V, int K, float m, RowPool& sh, int* tok, float* val) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t key, hi;
+    const uint32_t T = bound_from_maxima<THREADS>(K, m, sh, key, hi);
+    collect<THREADS>(row, pitch, V, 0, key, T, pool_room(K), sh);
     int n = sh.n;
-    if (n > pool_room(K)) n = collect_from_many<THREADS>(row, pitch, V, K, key, T, hi, sh);
+    if (n > pool_room(K)) n = collect_from_many<THREADS>(row, pitch, V, 0, K, key, T, hi, sh);
     for (int j = n + tid; j < K; j += THREADS) {
         tok[j] = 0;
         val[j] = -INFINITY;
@@ -2376,8 +2404,9 @@ __device__ __forceinline__ void select_largest(const float* row, long long pitch
     __syncthreads();
 }
 
-template <int OBJ, int THREADS>
-__global__ void __launch_bounds__(THREADS) row_kernel(const __grid_constant__ RowParams p) {
+template <int OBJ>
+__global__ void __launch_bounds__(ROW_THREADS) row_kernel(const __grid_constant__ RowParams p) {
+    constexpr int THREADS = ROW_THREADS;
     __shared__ RowShared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int row = blockIdx.x;
@@ -2390,9 +2419,9 @@ __global__ void __launch_bounds__(THREADS) row_kernel(const __grid_constant__ Ro
 
     float m_t = -INFINITY, s_t = 0.f, m_d = -INFINITY, s_d = 0.f, lse_t = 0.f, lse_d = 0.f;
     if (trow) own_stats<THREADS>(trow, p.pitch, m_t, s_t);
-    if (zrow) own_stats<THREADS>(zrow, p.pitch, m_d, s_d);
+    if (zrow && p.lse_in == nullptr) own_stats<THREADS>(zrow, p.pitch, m_d, s_d);
     if (trow) lse_t = block_lse<THREADS>(m_t, s_t, sh.red);
-    if (zrow) lse_d = block_lse<THREADS>(m_d, s_d, sh.red + 2);
+    if (zrow) lse_d = p.lse_in != nullptr ? p.lse_in[row] : block_lse<THREADS>(m_d, s_d, sh.red + 2);
     __syncthreads();
 
     int n_tok = K;                        // entries of Omega_hat's list (2K at most for the bi-directional set)
@@ -2479,8 +2508,10 @@ __global__ void __launch_bounds__(THREADS) row_kernel(const __grid_constant__ Ro
         }
         if (lane == 0) {
             sh.sum = S_q;
-            p.loss[row] = loss;
-            p.lse_d[row] = lse_d;
+            if (p.lse_in == nullptr) {
+                p.loss[row] = loss;
+                p.lse_d[row] = lse_d;
+            }
         }
     }
     __syncthreads();
@@ -2553,12 +2584,13 @@ __global__ void __launch_bounds__(THREADS) row_kernel(const __grid_constant__ Ro
     __syncthreads();
     // Tokens of q = 0 keep the dense value: the one that fills up a set of fewer than K logits above -inf (token 0) may be in it
     // already, and an entry has one writer.
-    if (tid < n_tok && sh.tok[tid] >= 0 && sh.q[tid] != 0.f) {
+    const float q_own = tid < n_tok && sh.tok[tid] >= 0 ? (p.lse_in != nullptr ? repeated_q(sh.tok, sh.q, n_tok, tid) : sh.q[tid]) : 0.f;
+    if (q_own != 0.f) {
         float o = c * ex2(fmaf(sh.z[tid], LOG2E, shift));
         if (OBJ == ROW_COMBINED)
-            o -= g * ex2(fmaf(trow[sh.tok[tid]], LOG2E, shift_t)) + g * p.w * sh.q[tid];
+            o -= g * ex2(fmaf(trow[sh.tok[tid]], LOG2E, shift_t)) + g * p.w * q_own;
         else
-            o -= g * sh.q[tid];
+            o -= g * q_own;
         drow[sh.tok[tid]] = __float2bfloat16_rn(o);
     }
     if (OBJ == ROW_COMBINED && warp == 0) {

@@ -72,6 +72,26 @@ def test_variants_of_few_rows_against_the_oracle(N, d, V, K):
         print(which, compare_variant(inp.H_t, inp.H_d[0], inp.W, K, which, param, _cpu(out)))
 
 
+# One, two, four and eight blocks per row and one logit more, as many rows as their blocks are resident for and one more (a block
+# per row), a last block with a piece of one logit, with none, and rows longer than eight blocks take
+@pytest.mark.parametrize("N,d,V,K", [(1, 64, 8192, 256), (74, 16, 8193, 100), (75, 16, 8193, 100), (37, 64, 16385, 10), (2, 64, 24577, 33),
+                                     (18, 8, 32769, 64), (19, 8, 65537, 64), (2, 16, 131072, 128), (2, 16, 131073, 10)])
+def test_rows_split_over_blocks_against_the_oracle(N, d, V, K):
+    hass = _hass()
+    dev = torch.device("cuda:0")
+    inp = hi.make_custom(N, d, V, K, seed=N + V, sigma_w=0.3)
+    args = inp.H_t.to(dev), inp.H_d[0].to(dev), inp.W.to(dev), K
+    out = hass.topk_distill_fwd_bwd(*args, dH_dtype=hass.HASS_FP32)
+    hass.check(out["workspace"])
+    print("fused", compare(inp.H_t, inp.H_d[0], inp.W, K, _cpu(out)))
+    for variant, which in ((hass.LOSS_NORMED_TOPK, oracle.VARIANT_NORMED), (hass.LOSS_BIDIR_TOPK, oracle.VARIANT_BIDIR)):
+        if which == oracle.VARIANT_BIDIR and K > 128:
+            continue
+        out = hass.variant_distill_fwd_bwd(*args, variant, dH_dtype=hass.HASS_FP32)
+        hass.check(out["workspace"])
+        print(which, compare_variant(inp.H_t, inp.H_d[0], inp.W, K, which, 0.0, _cpu(out)))
+
+
 # 40 rows: the row kernel; 200: the spill and its patch. A vocabulary masked by a bias column of -inf, so that fewer than K tokens
 # are left: token 0 with q = 0 fills the set up, whether it is one of those left or not.
 @pytest.mark.parametrize("N,V", [(40, 700), (200, 30)])
