@@ -111,6 +111,8 @@ static int device_info(DeviceInfo* out) {
             GemmFn const gemms[] = {gemm_kernel<MODE_STATS, TOPK_REG, 1>,  gemm_kernel<MODE_STATS, TOPK_REG, 2>,
                                     gemm_kernel<MODE_STATS, TOPK_BUF, 1>,  gemm_kernel<MODE_STATS, TOPK_BUF, 2>,
                                     gemm_kernel<MODE_STATS, TOPK_NONE, 1>, gemm_kernel<MODE_STATS, TOPK_NONE, 2>,
+                                    gemm_kernel<MODE_STATS, TOPK_REG, 1, 8>, gemm_kernel<MODE_STATS, TOPK_REG, 2, 8>,
+                                    gemm_kernel<MODE_STATS, TOPK_NONE, 1, 8>, gemm_kernel<MODE_STATS, TOPK_NONE, 2, 8>,
                                     gemm_kernel<MODE_PROBS, TOPK_BUF, 1>,  gemm_kernel<MODE_PROBS, TOPK_BUF, 2>,
                                     gemm_kernel<MODE_OUT, TOPK_BUF, 1>,    gemm_kernel<MODE_OUT, TOPK_BUF, 2>,
                                     gemm_kernel<MODE_OUT, TOPK_NONE, 1>,   gemm_kernel<MODE_OUT, TOPK_NONE, 2>,
@@ -483,7 +485,21 @@ static int launch_gemm(const GemmParams& p, cudaStream_t st, int kind = -1) {
     KernelTimer timer(p.gate ? KIND_CONDITIONAL : (kind >= 0 ? kind : MODE), st);
     const bool pair = p.sched.pair == 2;
     GemmFn fn;
-    if (MODE == MODE_STATS && p.topk_row_tiles == 0 && p.cap_z != nullptr)
+    // Eight epilogue warps where the products of a tile are short, up to 1024 columns of features, and a lane has three tiles or more, behind which
+    // their meeting disappears. Calls of 2048 rows x d x 32000, K = 10, on four and on eight: d = 256 288 -> 250 us, 512 309 -> 277, 1024 375 -> 360, K =
+    // 64 366 -> 336, 387 -> 357, 453 -> 435; from 2048 on the stage that they cost shows (2048 584 -> 587, 600 x 2048 285 -> 330), and so does the
+    // meeting where a lane has one tile (383 x 256 x 1024 59 -> 61).
+    constexpr int kWideBlocks = 16;
+    const bool none = MODE == MODE_STATS && p.topk_row_tiles == 0 && p.cap_z != nullptr;
+    if (MODE == MODE_STATS && p.k_blocks <= kWideBlocks && p.col_tiles > 2 * p.sched.ph[0].S &&
+        (none || (p.K <= K_REG && p.spill_begin == INT_MAX && p.Pt == nullptr))) {
+        if (none)
+            fn = pair ? gemm_kernel<MODE_STATS, TOPK_NONE, 2, 8> : gemm_kernel<MODE_STATS, TOPK_NONE, 1, 8>;
+        else
+            fn = pair ? gemm_kernel<MODE_STATS, TOPK_REG, 2, 8> : gemm_kernel<MODE_STATS, TOPK_REG, 1, 8>;
+        return launch(fn, p.sched.max_ctas, gemm_threads(8), gemm_smem(pair ? 2 : 1, 8), st, pair ? 2 : 1, p);
+    }
+    if (none)
         fn = pair ? gemm_kernel<MODE_STATS, TOPK_NONE, 2> : gemm_kernel<MODE_STATS, TOPK_NONE, 1>;
     else if (MODE == MODE_STATS && p.K <= K_REG)
         fn = pair ? gemm_kernel<MODE_STATS, TOPK_REG, 2> : gemm_kernel<MODE_STATS, TOPK_REG, 1>;

@@ -34,11 +34,13 @@ constexpr int BK = 64;         // contraction elements per pipeline stage (128 B
 constexpr int UMMA_K = 16;     // contraction elements per tcgen05.mma (bf16)
 constexpr int A_STAGE_BYTES = BM * BK * 2;
 // CG = CTAs that work on one product (1, or a pair): each holds its own BM rows of A and BN / CG of the tile's columns
-__host__ __device__ constexpr int stages(int CG) { return CG == 2 ? 6 : 4; }
+// EW = epilogue warps (4 or 8); eight take a stage's room for their staging buffers
+__host__ __device__ constexpr int stages(int CG, int EW = 4) { return (CG == 2 ? 6 : 4) - (EW == 8 ? 1 : 0); }
 __host__ __device__ constexpr int b_stage_bytes(int CG) { return BN / CG * BK * 2; }
 constexpr int OPERAND_BYTES = stages(1) * (A_STAGE_BYTES + b_stage_bytes(1));
 static_assert(OPERAND_BYTES == stages(2) * (A_STAGE_BYTES + b_stage_bytes(2)), "both forms use the same shared memory");
 constexpr int NUM_THREADS = 192;   // warp 0: TMA, warp 1: MMA + TMEM owner, warps 2-5: epilogue
+__host__ __device__ constexpr int gemm_threads(int EW) { return 64 + 32 * EW; }
 constexpr int TMEM_COLS = 512;     // two accumulator buffers of BN fp32 columns
 constexpr int MAX_PHASES = 48;
 constexpr int K_CAP = 256;         // == HASS_K_MAX
@@ -46,6 +48,9 @@ constexpr int SPILL_STAGE_BYTES = 32 * 128;   // 32 rows x 64 bf16 of a spilled 
 constexpr int SPILL_STAGES = 2;               // per epilogue warp
 constexpr int SMEM_BYTES = OPERAND_BYTES + 4 * SPILL_STAGES * SPILL_STAGE_BYTES +
                            1024 /*alignment slack*/ + 256 /*barriers*/;
+__host__ __device__ constexpr int operand_bytes(int CG, int EW) { return stages(CG, EW) * (A_STAGE_BYTES + b_stage_bytes(CG)); }
+__host__ __device__ constexpr int gemm_smem(int CG, int EW) { return operand_bytes(CG, EW) + EW * SPILL_STAGES * SPILL_STAGE_BYTES + 1024 + 256; }
+static_assert(gemm_smem(1, 4) == SMEM_BYTES && gemm_smem(2, 4) == SMEM_BYTES && gemm_smem(2, 8) <= SMEM_BYTES && gemm_smem(1, 8) <= SMEM_BYTES, "shared memory of a CTA");
 constexpr float LOG2E = 1.4426950408889634f;
 // A lane's sum of a spilling row's values 2^(z log2e - ref2), ref2 = z_ref log2e + 64, from which on the call is done again
 // with the row's largest logit as z_ref: a logit 90 above z_ref (natural units). The sum leaves fp32 only at 131, but what
@@ -414,8 +419,12 @@ __device__ __forceinline__ void finish_out4(const GemmParams& p, float4 a, int l
 // the two single steps it replaces (sweep of 8192 rows x 4096 x 32000: 1.77 -> 1.45 ms = 1480 TFLOP/s in short runs;
 // 1.24 -> 1.30 PFLOP/s where the power cap holds). Single CTAs stay for one row tile, where a partner would have nothing
 // to do, and where an odd number of row tiles makes pairs slower (plan_launch, plan_out).
-template <int MODE, int TOPK, int CG>
-__global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_constant__ GemmParams p) {
+// EW: epilogue warps. With eight, two threads share a row, 128 columns of every tile each, and meet at an item's end, where the second
+// hands its statistics and list to the first. A tile's epilogue is bound by the instructions of its warps, 11 k cycles and more, the products
+// take 512 per k block: narrow features leave the tensor core waiting (launch_gemm has the line and what it gives). It exists for the sweeps that
+// keep a row's state in registers: statistics alone, and lists of K <= 16 without a spill.
+template <int MODE, int TOPK, int CG, int EW = 4>
+__global__ void __launch_bounds__(gemm_threads(EW), 1) gemm_kernel(const __grid_constant__ GemmParams p) {
     constexpr bool B_MN_MAJOR = (MODE == MODE_OUT);
     // MODE_OUT after a MODE_LOGITS sweep of the same B, as an instantiation of its own (as a condition in the producer's loop it
     // cost the other calls 3-6 % of this kernel: 517 rows x 4096 x 128256 560 -> 576-595 us)
@@ -429,20 +438,22 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t smemA = smem_base;
-    constexpr int STAGES = stages(CG);
+    static_assert(EW == 4 || (MODE == MODE_STATS && TOPK != TOPK_BUF), "eight epilogue warps");
+    constexpr int STAGES = stages(CG, EW);
+    constexpr int OPERANDS = operand_bytes(CG, EW), STAGING = EW * SPILL_STAGES * SPILL_STAGE_BYTES;
     constexpr int B_STAGE_BYTES = b_stage_bytes(CG);
     const uint32_t smemB = smem_base + STAGES * A_STAGE_BYTES;
-    const uint32_t spill_stage = smem_base + OPERAND_BYTES;      // [epilogue warp][SPILL_STAGES] x SPILL_STAGE_BYTES
-    const uint32_t bar_base = spill_stage + 4 * SPILL_STAGES * SPILL_STAGE_BYTES;
-    // barriers: full[STAGES], empty[STAGES], tmem_full[2], tmem_empty[2]; then tmem pointer, abort flag
+    const uint32_t spill_stage = smem_base + OPERANDS;      // [epilogue warp][SPILL_STAGES] x SPILL_STAGE_BYTES
+    const uint32_t bar_base = spill_stage + STAGING;
+    // barriers: full[STAGES], empty[STAGES], tmem_full[2], tmem_empty[2], meet[2]; then tmem pointer, abort flag
     auto full_bar = [&](int s) { return bar_base + 8u * s; };
     auto empty_bar = [&](int s) { return bar_base + 8u * (STAGES + s); };
     auto tfull_bar = [&](int b) { return bar_base + 8u * (2 * STAGES + b); };
     auto tempty_bar = [&](int b) { return bar_base + 8u * (2 * STAGES + 2 + b); };
+    auto meet_bar = [&](int b) { return bar_base + 8u * (2 * STAGES + 4 + b); };      // EW = 8: the second threads' results are there / taken
     uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
     uint32_t* tmem_ptr_smem =
-        reinterpret_cast<uint32_t*>(smem_gen + OPERAND_BYTES + 4 * SPILL_STAGES * SPILL_STAGE_BYTES +
-                                    8 * (2 * STAGES + 4));
+        reinterpret_cast<uint32_t*>(smem_gen + OPERANDS + STAGING + 8 * (2 * STAGES + 6));
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_ptr_smem + 1);
 
     const int warp = threadIdx.x >> 5;
@@ -457,7 +468,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(tfull_bar(b), 1);
-            mbar_init(tempty_bar(b), 4 * CG);
+            mbar_init(tempty_bar(b), EW * CG);
+            if (EW == 8) mbar_init(meet_bar(b), 4);
         }
         *abort_flag = 0;
         fence_barrier_init();
@@ -665,6 +677,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
         // ===================== epilogue warps =====================
         const int quad = warp & 3;                 // TMEM lane quadrant this warp may read
         const int r_local = quad * 32 + lane;      // row inside the tile
+        const int half = EW == 8 ? (warp - 2) >> 2 : 0;      // EW = 8: which columns of a tile
+        constexpr int SHARE = BN * 4 / EW;         // columns of a tile that a thread takes: [half SHARE, (half + 1) SHARE)
+        uint32_t meet_phase = 0;
         int ab = 0;
         uint32_t aphase = 0;
         // Top-K candidates of this thread's row (MODE_STATS): buffer in the workspace, entries in use
@@ -682,9 +697,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
         constexpr bool CAPTURE = MODE == MODE_STATS && TOPK == TOPK_NONE;
         float tv[USE_REG ? K_REG : 1];
         int ti[USE_REG ? K_REG : 1];
-        static_assert(4 * SPILL_STAGES * SPILL_STAGE_BYTES >= 2 * 32 * 128 * 4, "room for the pending logits");
+        constexpr int PEND = EW * 32 * 4;          // bytes from one entry to the next
+        static_assert(STAGING >= 2 * 32 * PEND, "room for the pending logits");
         const uint32_t pend_v = spill_stage + (threadIdx.x - 64) * 4;
-        const uint32_t pend_i = pend_v + 32 * 128 * 4;
+        const uint32_t pend_i = pend_v + 32 * PEND;
         constexpr int lo = 0;
 
         for_each_item([&](int rt, int ln, int S, int slot, int, int) {
@@ -833,17 +849,18 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                     // row inserts its first 32 logits and some 70 more one by one, the warp as often as its slowest row
                     // (64 rows x 256 x 1024, four tiles on four CTAs: 28.0 -> 17.5 us).
                     float gm[16];
+                    constexpr int GROUP = SHARE / 16;
 #pragma unroll
-                    for (int ch = 0; ch < BN / 32; ++ch) {
+                    for (int ch = 0; ch < SHARE / 32; ++ch) {
                         uint32_t r[32];
-                        tmem_ld32(t_row + ch * 32, r);
+                        tmem_ld32(t_row + half * SHARE + ch * 32, r);
                         tmem_ld_wait(r);
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            float x = fmaxf(__uint_as_float(r[16 * h]), __uint_as_float(r[16 * h + 1]));
+                        for (int h = 0; h < 32 / GROUP; ++h) {
+                            float x = fmaxf(__uint_as_float(r[GROUP * h]), __uint_as_float(r[GROUP * h + 1]));
 #pragma unroll
-                            for (int j = 2; j < 16; j += 2) x = fmax3(x, __uint_as_float(r[16 * h + j]), __uint_as_float(r[16 * h + j + 1]));
-                            gm[2 * ch + h] = fmaxf(x, -INFINITY);      // (a group of NaN counts for nothing)
+                            for (int j = 2; j < GROUP; j += 2) x = fmax3(x, __uint_as_float(r[GROUP * h + j]), __uint_as_float(r[GROUP * h + j + 1]));
+                            gm[32 / GROUP * ch + h] = fmaxf(x, -INFINITY);      // (a group of NaN counts for nothing)
                         }
                     }
                     sort16_descending(gm);
@@ -855,13 +872,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                     thr = fmaxf(thr, thr_sh);
                 }
                 if (CAPTURE && !skip_tile) {
-                    while (nxt < col_base) {
+                    while (nxt < col_base + half * SHARE) {
                         ++cur;
                         nxt = cur < p.K ? si[cur] : INT_MAX;
                     }
                 }
 #pragma unroll 1
-                for (int ch = 0; ch < tile_width(t) / 32 && !skip_tile; ++ch) {
+                for (int ch = half * (SHARE / 32); ch < (EW == 8 ? (half + 1) * (SHARE / 32) : tile_width(t) / 32) && !skip_tile; ++ch) {
                     if (MODE == MODE_STATS && !USE_REG && want_topk) {
                         // make room for a whole chunk in every row's buffer (warp-uniform control flow), before the
                         // chunk's logits occupy registers
@@ -921,7 +938,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                                 s *= ex2((m - cm) * LOG2E);
                                 m = cm;
                             }
-                            const float mneg = -m * LOG2E;
+                            // (EW = 8: of a lane's last tile the second thread may meet columns beyond the vocabulary alone)
+                            const float mneg = EW == 8 && m == -INFINITY ? 0.f : -m * LOG2E;
                             float acc0 = 0.f, acc1 = 0.f;
 #pragma unroll
                             for (int j = 0; j < 32; j += 2) {
@@ -950,7 +968,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                                 // staging buffer (128-byte rows, swizzled), and after every second chunk one lane
                                 // requests the store of the 32 x 64 box. That is one request per 4 KB from this warp
                                 // instead of 64 store instructions that each touch 32 rows.
-                                const uint32_t buf = spill_stage + (quad * SPILL_STAGES + ((spill_boxes >> 1) & 1)) * SPILL_STAGE_BYTES;
+                                const uint32_t buf = spill_stage + ((4 * half + quad) * SPILL_STAGES + ((spill_boxes >> 1) & 1)) * SPILL_STAGE_BYTES;
                                 if ((ch & 1) == 0) {
                                     // the store that read this buffer two boxes ago must have finished reading it
                                     if (lane == 0) bulk_wait_group_read<SPILL_STAGES - 1>();
@@ -1002,13 +1020,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                             for (int j = 0; j < 32; ++j) {
                                 const float x = __uint_as_float(r[j]);
                                 const bool in = x > thr;       // predicated stores, no branches
-                                st_shared_b32_if(pend_v + np * 512, __float_as_uint(x), in);
-                                st_shared_b32_if(pend_i + np * 512, static_cast<uint32_t>(col0 + j), in);
+                                st_shared_b32_if(pend_v + np * PEND, __float_as_uint(x), in);
+                                st_shared_b32_if(pend_i + np * PEND, static_cast<uint32_t>(col0 + j), in);
                                 np += in ? 1 : 0;
                             }
                             for (int q = 0; q < np; ++q) {
-                                const float x = __uint_as_float(ld_shared_b32(pend_v + q * 512));
-                                const int id = static_cast<int>(ld_shared_b32(pend_i + q * 512));
+                                const float x = __uint_as_float(ld_shared_b32(pend_v + q * PEND));
+                                const int id = static_cast<int>(ld_shared_b32(pend_i + q * PEND));
                                 if (!(x > thr)) continue;
                                 // sorted insertion; equal logits stay behind earlier (lower) token ids
 #pragma unroll
@@ -1225,6 +1243,73 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) gemm_kernel(const __grid_const
                     }
                     thr = fmaxf(thr_own, fmaxf(thr, thr_sh));
                 }
+            }
+            if constexpr (EW == 8) {
+                // The second thread of a row hands over m, s and its list through the staging area; the first adds them to its own.
+                const uint32_t at = spill_stage + ((threadIdx.x - 64) & 127) * 4;      // word e of the row at + e PEND: the first thread's columns of the room
+                if (half == 1) {
+                    if (TOPK == TOPK_NONE && lane == 0) bulk_wait_group_read<0>();      // (its own staging buffers have been read)
+                    __syncwarp();
+                    // the first threads' staging buffers and pending logits lie there too: they say when the room is free
+                    if (!__all_sync(0xffffffffu, wait_barrier(meet_bar(1), meet_phase, abort_flag, p.status, 5))) return false;
+                    st_shared_b32(at, __float_as_uint(m));
+                    st_shared_b32(at + PEND, __float_as_uint(s));
+                    if (USE_REG) {
+#pragma unroll
+                        for (int k = 0; k < (USE_REG ? K_REG : 1); ++k) {
+                            st_shared_b32(at + PEND * (2 + 2 * k), __float_as_uint(tv[k]));
+                            st_shared_b32(at + PEND * (3 + 2 * k), static_cast<uint32_t>(ti[k]));
+                        }
+                    }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(meet_bar(0));
+                    if (!__all_sync(0xffffffffu, wait_barrier(meet_bar(1), meet_phase ^ 1u, abort_flag, p.status, 6))) return false;
+                    if (spill && track_zmax && !p.use_row_zmax) atomicMax(p.row_zmax + rt * BM + r_local, ordered_key(__float_as_uint(zmax)));
+                    return true;
+                }
+                if (TOPK == TOPK_NONE && lane == 0) bulk_wait_group_read<0>();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(meet_bar(1));
+                if (!__all_sync(0xffffffffu, wait_barrier(meet_bar(0), meet_phase, abort_flag, p.status, 5))) return false;
+                meet_phase ^= 1u;
+                const float m2 = __uint_as_float(ld_shared_b32(at)), s2 = __uint_as_float(ld_shared_b32(at + PEND));
+                if (spill) {
+                    s += s2;      // (of the same reference)
+                } else {
+                    const float top = fmaxf(m, m2), base = top == -INFINITY ? 0.f : top;
+                    s = s * ex2((m - base) * LOG2E) + s2 * ex2((m2 - base) * LOG2E);
+                    m = top;
+                }
+                if (USE_REG) {
+                    // the 16 best of both lists, which are sorted (larger logit first, of equal ones the lower token): best of k and 15 - k,
+                    // then the last steps of a sorting network
+                    auto before = [](float xv, int xi, float yv, int yi) { return xv > yv || (xv == yv && static_cast<uint32_t>(xi) < static_cast<uint32_t>(yi)); };
+#pragma unroll
+                    for (int k = 0; k < (USE_REG ? K_REG : 1); ++k) {
+                        const float ov = __uint_as_float(ld_shared_b32(at + PEND * (2 + 2 * (K_REG - 1 - k))));
+                        const int oi = static_cast<int>(ld_shared_b32(at + PEND * (3 + 2 * (K_REG - 1 - k))));
+                        const bool mine = before(tv[k], ti[k], ov, oi);
+                        tv[k] = mine ? tv[k] : ov;
+                        ti[k] = mine ? ti[k] : oi;
+                    }
+#pragma unroll
+                    for (int j = K_REG / 2; j > 0; j /= 2)
+#pragma unroll
+                        for (int k = 0; k < (USE_REG ? K_REG : 1); ++k) {
+                            const int l = k ^ j;
+                            if (l > k && l < (USE_REG ? K_REG : 1)) {
+                                const bool keep = before(tv[k], ti[k], tv[l], ti[l]);
+                                const float hv = keep ? tv[k] : tv[l], lv = keep ? tv[l] : tv[k];
+                                const int hi_ = keep ? ti[k] : ti[l], li = keep ? ti[l] : ti[k];
+                                tv[k] = hv;
+                                ti[k] = hi_;
+                                tv[l] = lv;
+                                ti[l] = li;
+                            }
+                        }
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(meet_bar(1));
             }
             if (MODE == MODE_STATS && tile_ok) {
                 const long long so = static_cast<long long>(slot) * BM + r_local;
