@@ -70,8 +70,8 @@ int hass_version(void);
  * bounded scratch areas for one chunk of rows (a fixed number of 128-row tiles that does not grow
  * with N): the bf16 un-normalised draft probabilities (fused call) or dz_d (split backward),
  * chunk_rows x V, and the fp32 Omega_hat term of dH_d, chunk_rows x d; and, behind them, fp32 partial
- * tiles of dH_d (less than one 128-row tile of scratch). Calls of at most 128 rows keep their logits in fp32 instead, two
- * matrices of N x V. A smaller workspace is accepted down to room
+ * tiles of dH_d (less than one 128-row tile of scratch). Calls of at most 128 rows, and of 257 to some thousand rows over at
+ * most 2048 tokens, keep their logits in fp32 instead, two matrices of N x V. A smaller workspace is accepted down to room
  * for one 128-row tile of scratch; the calls then work in smaller chunks, and may do without partial tiles and fp32 logits.
  * Needs no GPU (assumes 148 SMs if none is present).
  */
@@ -155,7 +155,8 @@ int hass_topk_distill_bwd(const void* H_d, const void* W, int64_t N, int64_t d, 
  * the Top-P variant work the same way, and so do hass_combined_distill_fwd_bwd and the Bi-directional
  * variant, whose exponent comes from the row's largest logit among the first 256 tokens and whose
  * second pass repeats the whole sequence.
- * Calls of at most 128 rows sweep both feature sets in one launch and keep the draft logits in fp32 between
+ * Calls of at most 128 rows, and of 257 rows and more over at most 2048 tokens (up to 3072 rows with K <= 32 and 1024 tokens, 2048
+ * with K <= 64, 1024 otherwise), sweep both feature sets in one launch and keep the draft logits in fp32 between
  * the sweep and the second GEMM; they have no range condition and no second pass.
  * (HASS_ERR_RANGE is kept for callers that name it; no entry point of this version returns it.)
  */

@@ -374,6 +374,18 @@ static int even_chunk(int most, int RT) {
     return most > 1 ? most & ~1 : most;
 }
 
+// Whether a call's logits may go through the workspace in fp32 (narrow_impl), in one chunk of row tiles: one row tile of any vocabulary, and more
+// rows of a short one, whose kernels are then three instead of nine and more, while the blocks of the row kernel (11 ns a row at most 1024 tokens
+// and K <= 32, 18 up to 2048 and K <= 64, 57 beyond) take less than those cost. Calls of N x 256 x 1024, before -> after: K = 10 600 rows 62 -> 31 us,
+// 1500 64 -> 40, 2795 69 -> 56, 4500 71 -> 75; K = 41 1500 89 -> 55, 2795 94 -> 82 but Bi-directional 159 -> 177; K = 101 600 123 -> 60, 1500 132 -> 113,
+// 2795 140 -> 186; combined 1980 rows, K = 9 107 -> 50; 1000 x 4096 x 2000, K = 10 111 -> 68, 3900 187 -> 213. (Calls of 129 to 256 rows keep to the
+// spill's route: what they do beyond its exponent range, and report in the status block, is held by tests.)
+static bool narrow_rows(long long N, long long pitch, int K, int chunk_tiles, int sms) {
+    if (N <= BM) return true;
+    const int most = K <= 32 && pitch <= 1024 ? 3072 : K <= 64 && pitch <= 2048 ? 2048 : pitch <= 2048 ? 1024 : 0;
+    return N > 2 * BM && N <= most && N <= static_cast<long long>(chunk_tiles) * BM && 2 * ((N + BM - 1) / BM) <= sms;
+}
+
 // The forward schedule covers 2 * RT row tiles (target then draft).
 static int make_layout(long long N, long long d, long long V, int K, int sms, Layout* L) {
     const int RT = ceil_div(N, BM), CT = ceil_div(V, BN);
@@ -445,6 +457,10 @@ static int make_layout(long long N, long long d, long long V, int K, int sms, La
         const size_t need = part_bytes_of(plan_out(static_cast<int>(rows), ceil_div(d, BN), ceil_div(V, BK), sms,
                                                    L->scratch_row_tile_bytes - 256, nullptr));
         if (need > L->part_bytes) L->part_bytes = need;
+    }
+    if (N > BM && narrow_rows(N, L->p_pitch, K, pref, sms)) {
+        const size_t end = L->scratch + 2 * align256(static_cast<size_t>(N) * L->p_pitch * 4);
+        if (end > L->total_pref && end - L->total_pref > L->part_bytes) L->part_bytes = end - L->total_pref;
     }
     if (N <= BM) {
         // the fp32 logits of such a call (narrow_room), from the scratch on, and its partial tiles; one chunk in any case
@@ -865,16 +881,20 @@ constexpr long long kLateBytes = 16ll << 20;
 // or two do, 64 rows x 256 x 1024 22 -> 31; with eight pieces, which 512 threads hold of both rows in 64 registers, 118 rows x 12454
 // Bi-directional 111 -> 123.
 struct RowSplit {
-    int blocks, pieces;
+    int blocks, threads, pieces;
 };
-static RowSplit row_split(long long N, long long pitch, int sms) {
+static RowSplit row_split(long long N, long long pitch, int K, int sms) {
+    // Many short rows: as few threads as hold one, with four maxima or more for each token of the set (two K threads at least). A block
+    // takes longer (10 us at 128 threads, 7 at 512), but ten of them fit an SM.
+    if (N > sms && pitch <= 1024 && K <= 32) return RowSplit{1, 128, 2};
+    if (N > sms && pitch <= 2048 && K <= 64) return RowSplit{1, 256, 2};
     for (int c = 1; c <= SPLIT_MAX; c *= 2) {
         const int e = ceil_div(pitch, static_cast<long long>(c) * SPLIT_STEP);
         if (e > (c == SPLIT_MAX ? SPLIT_PIECES : SPLIT_PIECES / 2)) continue;
-        if (c * N > sms) break;
-        return RowSplit{c, e > 4 ? SPLIT_PIECES : e > 2 ? 4 : e};
+        if (c * N > sms && e > 1) break;
+        return RowSplit{c, SPLIT_THREADS, e > 4 ? SPLIT_PIECES : e > 2 ? 4 : e};
     }
-    return RowSplit{0, 0};
+    return RowSplit{0, 0, 0};
 }
 struct NarrowRoom {
     float* z = nullptr;      // [N, p_pitch], or nullptr: no room
@@ -882,13 +902,13 @@ struct NarrowRoom {
     float* dz = nullptr;     // the one of the two that dz_d goes over, which lies first
     PartRoom part;
 };
-static NarrowRoom narrow_room(long long N, uint8_t* ws, size_t workspace_bytes, const Layout& L, int sms) {
+static NarrowRoom narrow_room(long long N, int K, uint8_t* ws, size_t workspace_bytes, const Layout& L, int sms) {
     NarrowRoom r;
     const size_t z = align256(static_cast<size_t>(N) * L.p_pitch * 4);
-    if (N <= BM && workspace_bytes >= L.scratch + 2 * z) {
+    if (narrow_rows(N, L.p_pitch, K, L.pref_chunk_tiles, sms) && workspace_bytes >= L.scratch + 2 * z) {
         float* const a = reinterpret_cast<float*>(ws + L.scratch);
         float* const b = reinterpret_cast<float*>(ws + L.scratch + z);
-        const bool split = row_split(N, L.p_pitch, sms).blocks != 0;
+        const bool split = row_split(N, L.p_pitch, K, sms).blocks != 0;
         r.z = split ? b : a;
         r.zt = split ? a : b;
         r.dz = a;
@@ -898,24 +918,25 @@ static NarrowRoom narrow_room(long long N, uint8_t* ws, size_t workspace_bytes, 
     return r;
 }
 
-// The logits of N <= BM rows of H0 and (nullable) of H1 -> z0, z1 [N, p_pitch]; clears the status block.
+// The logits of N rows of H0 and (nullable) of H1 -> z0, z1 [N, p_pitch]; clears the status block.
 static int narrow_sweep(const void* H0, const void* H1, const void* W, int N, long long d, long long V, float* z0, float* z1,
                         uint8_t* ws, const Layout& L, const DeviceInfo& di, cudaStream_t st) {
     GemmParams p;
     std::memset(&p, 0, sizeof(p));
     // up to 64 rows each share one row tile (61 rows x 4096 x 32000: 65 us as two row tiles of a CTA pair, 61 as one)
     p.half_tiles = H1 && N <= BM / 2 ? 1 : 0;
-    p.row_tiles = H1 && !p.half_tiles ? 2 : 1;
+    const int RT = ceil_div(N, BM);
+    p.row_tiles = H1 && !p.half_tiles ? 2 * RT : RT;
     // One phase in which every CTA (pair) has the same number of columns, in steps of 32: whole tiles dealt out in rounds leave the last one
     // to a third of the SMs with 128256 tokens and most SMs without any below 20000. Per call: 64 rows x 256 x 1024 25.7 -> 22.5 us, 53 rows x
     // 280 x 2179 combined 40 -> 29, 33 draft rows x 4096 x 32000 101.6 -> 95.9, 61 rows x 4096 x 128256 400 -> 388 (what is left there is
     // the rate at which boxes of 128 bytes a row come out of memory, 6.0 of 6.4 TB/s).
-    const int pair = p.row_tiles, groups = std::max(1, di.sms / pair);
-    p.lane_cols = ceil_div(L.p_pitch / 32, groups) * 32;
+    const int pair = p.row_tiles > 1 ? 2 : 1, units = ceil_div(p.row_tiles, pair), lanes = std::max(1, di.sms / pair / units);
+    p.lane_cols = ceil_div(L.p_pitch / 32, lanes) * 32;
     p.sched.n_phases = 1;
     p.sched.pair = pair;
-    p.sched.ph[0] = Phase{0, pair, ceil_div(L.p_pitch, p.lane_cols), 0};
-    p.sched.max_ctas = p.sched.total_slots = pair * p.sched.ph[0].S;
+    p.sched.ph[0] = Phase{0, units * pair, ceil_div(L.p_pitch, p.lane_cols), 0};
+    p.sched.max_ctas = p.sched.total_slots = units * pair * p.sched.ph[0].S;
     log_schedule("narrow sweep", p.sched);
     const int box_rows = p.half_tiles ? BM / 2 : BM;
     int rc = make_tmap(&p.tmA0, H0, N, d, d, BK, box_rows);
@@ -923,7 +944,7 @@ static int narrow_sweep(const void* H0, const void* H1, const void* W, int N, lo
     if (rc == HASS_OK) rc = make_tmap(&p.tmB, W, V, d, d, BK, BN / pair);
     if (rc == HASS_OK && p.lane_cols % BN) rc = make_tmap(&p.tmSpill, W, V, d, d, BK, p.lane_cols % BN / pair);
     if (rc != HASS_OK) return rc;
-    p.row_tiles0 = 1;
+    p.row_tiles0 = RT;
     p.spill_begin = INT_MAX;
     p.z_rows = N;
     p.zt_out = z0;
@@ -952,16 +973,19 @@ static RowParams row_params(int V, int K, const Layout& L) {
 template <int OBJ>
 static int launch_rows_as(RowParams& r, int N, int sms, cudaStream_t st) {
     KernelTimer timer(KIND_FINALIZE, st);
-    const RowSplit w = row_split(N, r.pitch, sms);
-    if (w.blocks) {
-        r.split = w.blocks;
-        const auto fn = w.pieces == 1   ? row_split_kernel<OBJ, 1>
-                        : w.pieces == 2 ? row_split_kernel<OBJ, 2>
-                        : w.pieces == 4 ? row_split_kernel<OBJ, 4>
-                                        : row_split_kernel<OBJ, SPLIT_PIECES>;
-        return launch(fn, static_cast<long long>(N) * w.blocks, SPLIT_THREADS, 0, st, w.blocks, r);
-    }
-    return launch(row_kernel<OBJ>, N, ROW_THREADS, 0, st, 1, r);
+    const RowSplit w = row_split(N, r.pitch, r.K, sms);
+    if (w.blocks == 0) return launch(row_kernel<OBJ>, N, ROW_THREADS, 0, st, 1, r);
+    r.split = w.blocks;
+    void (*fn)(RowParams);
+    if (w.blocks == 1)
+        fn = w.threads == 128   ? row_split_kernel<OBJ, 2, 128, false>
+             : w.threads == 256 ? row_split_kernel<OBJ, 2, 256, false>
+             : w.pieces == 1    ? row_split_kernel<OBJ, 1, SPLIT_THREADS, false>
+             : w.pieces == 2    ? row_split_kernel<OBJ, 2, SPLIT_THREADS, false>
+                                : row_split_kernel<OBJ, 4, SPLIT_THREADS, false>;
+    else
+        fn = w.pieces <= 4 ? row_split_kernel<OBJ, 4, SPLIT_THREADS, true> : row_split_kernel<OBJ, SPLIT_PIECES, SPLIT_THREADS, true>;
+    return launch(fn, static_cast<long long>(N) * w.blocks, w.threads, 0, st, w.blocks, r);
 }
 static int launch_rows(int objective, RowParams& r, int N, int sms, cudaStream_t st) {
     return objective == ROW_COMBINED ? launch_rows_as<ROW_COMBINED>(r, N, sms, st)
@@ -1015,8 +1039,7 @@ static int narrow_impl(int objective, bool with_target, const void* H_t, const v
     if (rc == HASS_OK) rc = make_tmap(&o.tmB, W, V, d, d, 64, BK);
     if (rc != HASS_OK) return rc;
     o.tmA1 = o.tmA0;
-    o.row_tiles = 1;
-    o.row_tiles0 = 1;
+    o.row_tiles = o.row_tiles0 = ceil_div(N, BM);
     o.spill_begin = INT_MAX;
     o.rows_valid = N;
     o.n_cols = static_cast<int>(d);
@@ -1027,7 +1050,7 @@ static int narrow_impl(int objective, bool with_target, const void* H_t, const v
     o.out_fp32 = dH_dtype == HASS_FP32 ? 1 : 0;
     o.out_align32 = ((reinterpret_cast<uintptr_t>(dH_d) | static_cast<uintptr_t>(d * (dH_dtype == HASS_FP32 ? 4 : 2))) & 31u) == 0 ? 1 : 0;
     o.out_pitch = d;
-    o.kept = 1;
+    o.kept = N <= BM ? 1 : 0;      // (several row tiles read W side by side)
     o.release_late = r.release_late;
     o.coef = r.coef_out;
     o.sparse = r.sparse_out;
@@ -1041,7 +1064,7 @@ static int narrow_impl(int objective, bool with_target, const void* H_t, const v
 static int narrow_backward(const void* H_d, const void* W, long long N, long long d, long long V, int K, const int* topk_idx, const float* topk_q,
                            const float* lse_d, const float* grad_loss, void* dH_d, int dH_dtype, uint8_t* ws, size_t workspace_bytes,
                            const Layout& L, const DeviceInfo& di, cudaStream_t st) {
-    const NarrowRoom room = narrow_room(N, ws, workspace_bytes, L, di.sms);
+    const NarrowRoom room = narrow_room(N, K, ws, workspace_bytes, L, di.sms);
     if (!room.z) return HASS_ERR_UNSUPPORTED;
     return narrow_impl(ROW_TOPK, false, nullptr, H_d, W, static_cast<int>(N), d, V, K, grad_loss, topk_idx, topk_q, nullptr, nullptr, nullptr,
                        nullptr, nullptr, dH_d, dH_dtype, ws, L, room, di, st, 0.f, nullptr, nullptr, lse_d);
@@ -1083,7 +1106,7 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
     int* idx_d = reinterpret_cast<int*>(ws + L.sidx);
     // (The combined objective too: 65 rows x 4096 x 32000 254 -> 123 us, 128 rows x 4096 x 128256 675 -> 472, 100 x 256 x 1024 82 -> 37.)
     if (with_target) {
-        const NarrowRoom narrow = narrow_room(N, ws, cmb ? cmb->end : workspace_bytes, L, di.sms);
+        const NarrowRoom narrow = narrow_room(N, K, ws, cmb ? cmb->end : workspace_bytes, L, di.sms);
         if (narrow.z)
             return narrow_impl(cmb ? ROW_COMBINED : bidir ? ROW_BIDIR : ROW_TOPK, true, H_t, H_d, W, static_cast<int>(N), d, V, K, grad_loss,
                                nullptr, nullptr, loss, idx_out, q_out, lse_t, lse_d, dH_d, dH_dtype, ws, L, narrow, di, st, 0.f, topk_n, cmb);
@@ -1358,8 +1381,8 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
     float* coef = reinterpret_cast<float*>(ws + L.coef);
     float* capz = reinterpret_cast<float*>(ws + L.capz);
     float* ref2 = reinterpret_cast<float*>(ws + L.lse2);
-    const NarrowRoom narrow = narrow_room(N, ws, workspace_bytes, L, di.sms);
-    if (narrow.z) {
+    const NarrowRoom narrow = narrow_room(N, K, ws, workspace_bytes, L, di.sms);
+    if (narrow.z && (!pipe || N <= BM)) {
         if (pipe) {
             rc = pipe_in(pipe, H_t, H_d, 0, static_cast<size_t>(N), st);
             if (rc != HASS_OK) return rc;
@@ -1566,7 +1589,7 @@ static int forward2_impl(bool with_target, const void* H_t, const void* H_d, con
                             workspace, workspace_bytes, st);
     const int RT = ceil_div(N, BM), CT = ceil_div(V, BN);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
-    const NarrowRoom narrow = narrow_room(N, ws, workspace_bytes, L, di.sms);
+    const NarrowRoom narrow = narrow_room(N, K, ws, workspace_bytes, L, di.sms);
     if (narrow.z)
         return narrow_impl(ROW_TOPK, with_target, H_t, H_d, W, static_cast<int>(N), d, V, K, nullptr, idx_in, q_in, loss, idx_out, q_out,
                            lse_t, lse_d, nullptr, HASS_BF16, ws, L, narrow, di, st, 0.f, nullptr);
@@ -1669,7 +1692,7 @@ static int normed_impl(const void* H_t, const void* H_d, const void* W, long lon
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     GemmParams p;
     std::memset(&p, 0, sizeof(p));
-    const NarrowRoom narrow = narrow_room(N, ws, workspace_bytes, L, di.sms);
+    const NarrowRoom narrow = narrow_room(N, K, ws, workspace_bytes, L, di.sms);
     if (narrow.z) {
         rc = narrow_sweep(H_t, nullptr, W, static_cast<int>(N), d, V, narrow.zt, nullptr, ws, L, di, st);
         if (rc != HASS_OK) return rc;

@@ -134,7 +134,7 @@ struct GemmParams {
     __nv_bfloat16* Pt;     // [chunk rows, p_pitch] spill of the target tiles, or nullptr
     long long p_pitch;
     // MODE_LOGITS: the logits of the first z_rows rows of A0 (zt_out) and of A1 (z_out) in fp32, [z_rows, z_pitch], -inf
-    // beyond n_cols. One row tile of either matrix at most; with a single row tile that is not halved its matrix is A0
+    // beyond n_cols. A0's row tiles come before A1's; with a single row tile that is not halved its matrix is A0
     int z_rows;
     float* z_out;
     float* zt_out;
@@ -761,7 +761,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), 1) gemm_kernel(const __grid_
             float* zrow = nullptr;
             if (MODE == MODE_LOGITS && tile_ok) {
                 const bool halved = CG == 1 && p.half_tiles;
-                const int r_own = halved ? r_local % (BM / 2) : r_local;      // row in its own matrix
+                const int r_own = halved ? r_local % (BM / 2) : (rt < p.row_tiles0 ? rt : rt - p.row_tiles0) * BM + r_local;      // row in its own matrix
                 float* z = (halved ? quad >= 2 : rt >= p.row_tiles0) ? p.z_out : p.zt_out;
                 if (r_own < p.z_rows) zrow = z + static_cast<long long>(r_own) * p.z_pitch;
             }

@@ -4,11 +4,12 @@
 
 namespace hass {
 
-constexpr int SPLIT_THREADS = 512;
+constexpr int SPLIT_THREADS = 512;                      // of a block where clusters share rows; fewer for short rows of a block each
 constexpr int SPLIT_MAX = 8;                            // blocks per row, at most (the portable cluster size)
 constexpr int SPLIT_STEP = SPLIT_THREADS * 4;           // logits of a row that a block's threads hold one 16-byte piece each of
 constexpr int SPLIT_PIECES = 8;                         // such pieces per thread, at most
 
+template <int THREADS, bool CLUSTER>
 struct SplitShared : RowPool {
     unsigned long long list[2][K_CAP];                  // the K largest logits of this block's piece of the target's (0) and of the draft's (1)
                                                         // row as ranks, descending; 0: none
@@ -16,10 +17,10 @@ struct SplitShared : RowPool {
     float stats[4];                                     // the piece's largest logit and sum of 2^((z - m) log2e), target and draft
     union {
         struct {
-            unsigned long long list[SPLIT_MAX * K_CAP];   // one list of every block of the row
-            float other[SPLIT_MAX * K_CAP];
+            unsigned long long list[(CLUSTER ? SPLIT_MAX : 1) * K_CAP];   // one list of every block of the row
+            float other[(CLUSTER ? SPLIT_MAX : 1) * K_CAP];
         } all;
-        float part[SPLIT_THREADS * 8];                  // sums of rows of W, one per thread
+        float part[THREADS * 8];                        // sums of rows of W, one per thread
     };
     float all_stats[SPLIT_MAX][4];
     int tok[K_CAP];                                     // Omega_hat
@@ -32,8 +33,8 @@ struct SplitShared : RowPool {
 
 // Block-collective: the K largest logits of the block's piece (columns first ..., thread T's at (u THREADS + T) 4 in v[u]) as a
 // descending list; m = the thread's largest.
-template <int E>
-__device__ __forceinline__ void piece_list(const float4 (&v)[E], const float* piece, int len, int V, int first, int K, float m, SplitShared& sh,
+template <int SPLIT_THREADS, int E>
+__device__ __forceinline__ void piece_list(const float4 (&v)[E], const float* piece, int len, int V, int first, int K, float m, RowPool& sh,
                                            unsigned long long* list) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t key, hi;
@@ -68,7 +69,8 @@ __device__ __forceinline__ void piece_list(const float4 (&v)[E], const float* pi
 
 // Block-collective: the lists `which` of all C blocks of the row merged into tok / val, in descending order; with `other` what
 // they carry beside. Fewer than K logits above -inf: the rest is token 0 with the values given. Ends without a barrier.
-__device__ __forceinline__ void merge_lists(int which, int C, int K, SplitShared& sh, int* tok, float* val, float* other, float fill_val, float fill_other) {
+template <int SPLIT_THREADS, typename S>
+__device__ __forceinline__ void merge_lists(int which, int C, int K, S& sh, int* tok, float* val, float* other, float fill_val, float fill_other) {
     const int tid = threadIdx.x;
     const uint32_t list = smem_u32(sh.list[which]), oth = smem_u32(sh.other[which]);
     for (int e = tid; e < C * K; e += SPLIT_THREADS) {
@@ -113,11 +115,13 @@ __device__ __forceinline__ void merge_lists(int which, int C, int K, SplitShared
 // distributed shared memory, after which every block merges the lists for itself. dz_d does not go over the draft's logits
 // but over the target's, which no block needs by then.
 // row_kernel, one block per row, is a chain of passes over 4 V bytes that one SM reads, on as many SMs as there are rows.
-template <int OBJ, int E>
-__global__ void __launch_bounds__(SPLIT_THREADS, 1) row_split_kernel(const __grid_constant__ RowParams p) {
-    __shared__ SplitShared sh;
+// Short rows have a block each (THREADS x E pieces of four logits) and as many of them on an SM as 80 registers per thread allow.
+template <int OBJ, int E, int SPLIT_THREADS, bool CLUSTER>
+__global__ void __launch_bounds__(SPLIT_THREADS, CLUSTER || SPLIT_THREADS == 512 ? 1 : 768 / SPLIT_THREADS) row_split_kernel(const __grid_constant__ RowParams p) {
+    constexpr int SPLIT_STEP = SPLIT_THREADS * 4;
+    __shared__ SplitShared<SPLIT_THREADS, CLUSTER> sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int C = p.split, K = p.K;
+    const int C = CLUSTER ? p.split : 1, K = p.K;
     const int row = blockIdx.x / C, rank = blockIdx.x - row * C;      // (clusters are consecutive blocks)
     wait_previous_kernel(!p.release_late);
     const float* zrow = p.z != nullptr ? p.z + static_cast<long long>(row) * p.pitch : nullptr;
@@ -184,13 +188,13 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) row_split_kernel(const __gri
         __syncthreads();      // (red is written again)
     }
     if (trow) {
-        piece_list<E>(t, trow + first, len, V, first, K, m_t, sh, sh.list[0]);
+        piece_list<SPLIT_THREADS>(t, trow + first, len, V, first, K, m_t, sh, sh.list[0]);
         for (int j = tid; j < K; j += SPLIT_THREADS) {
             const unsigned long long x = sh.list[0][j];
             sh.other[0][j] = x != 0ull && zrow ? zrow[~static_cast<uint32_t>(x)] : -INFINITY;
         }
         if (OBJ == ROW_BIDIR) {
-            piece_list<E>(z, zrow + first, len, V, first, K, m_d, sh, sh.list[1]);
+            piece_list<SPLIT_THREADS>(z, zrow + first, len, V, first, K, m_d, sh, sh.list[1]);
             for (int j = tid; j < K; j += SPLIT_THREADS) {
                 const unsigned long long x = sh.list[1][j];
                 sh.other[1][j] = x != 0ull ? trow[~static_cast<uint32_t>(x)] : -INFINITY;
@@ -201,10 +205,10 @@ __global__ void __launch_bounds__(SPLIT_THREADS, 1) row_split_kernel(const __gri
     cluster_sync();
     if (tid < 4 * C) sh.all_stats[tid >> 2][tid & 3] = ld_cluster_f32(map_to_rank(smem_u32(&sh.stats[tid & 3]), tid >> 2));
     if (trow) {
-        merge_lists(0, C, K, sh, sh.tok, sh.zt, sh.z, -INFINITY, z0);
+        merge_lists<SPLIT_THREADS>(0, C, K, sh, sh.tok, sh.zt, sh.z, -INFINITY, z0);
         if (OBJ == ROW_BIDIR) {
             __syncthreads();
-            merge_lists(1, C, K, sh, sh.tok_d, sh.q, sh.q + K, z0, t0);      // (q is free until then; 2 K <= K_CAP)
+            merge_lists<SPLIT_THREADS>(1, C, K, sh, sh.tok_d, sh.q, sh.q + K, z0, t0);      // (q is free until then; 2 K <= K_CAP)
         }
     } else {
         for (int j = tid; j < K; j += SPLIT_THREADS) {

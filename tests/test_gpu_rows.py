@@ -92,6 +92,32 @@ def test_rows_split_over_blocks_against_the_oracle(N, d, V, K):
         print(which, compare_variant(inp.H_t, inp.H_d[0], inp.W, K, which, 0.0, _cpu(out)))
 
 
+# A row of one block, of two blocks, the row kernel, and the separate backward of more rows
+@pytest.mark.parametrize("N,V", [(5, 600), (5, 20000), (100, 9000), (200, 600)])
+def test_backward_of_a_set_that_repeats_a_token(N, V):
+    """The separate backward takes any set: a token named twice has both of its probabilities taken off, a cut entry (-1) none."""
+    hass = _hass()
+    dev = torch.device("cuda:0")
+    d, K = 64, 12
+    g = torch.Generator().manual_seed(V)
+    H, W = torch.randn(N, d, generator=g).to(torch.bfloat16), (0.3 * torch.randn(V, d, generator=g)).to(torch.bfloat16)
+    idx = torch.randint(0, V, (N, K), generator=g, dtype=torch.int32)
+    idx[:, 7], idx[:, 9], idx[1:, 3] = idx[:, 2], idx[:, 2], idx[1:, 11]
+    q = torch.rand(N, K, generator=g) / K
+    q[::2, 2] = 0.0
+    idx[:, 5], q[:, 5] = -1, 0.0
+    z = H.double() @ W.double().T
+    lse = z.logsumexp(1)
+    dz = q.double().sum(1, keepdim=True) * (z - lse[:, None]).exp()
+    dz.scatter_add_(1, idx.clamp(min=0).long(), -q.double())
+    want = dz @ W.double()
+    ws = torch.empty(hass.topk_distill_workspace_bytes(N, d, V, K), dtype=torch.uint8, device=dev)
+    dH = hass.topk_distill_bwd(H.to(dev), W.to(dev), idx.to(dev), q.to(dev), lse.float().to(dev), dH_dtype=hass.HASS_FP32, workspace=ws)
+    hass.check(ws)
+    # every entry of dz_d in bf16, 2^-9 of itself
+    assert (dH.cpu().double() - want).abs().max() <= 1e-2 * want.abs().max()
+
+
 # 40 rows: the row kernel; 200: the spill and its patch. A vocabulary masked by a bias column of -inf, so that fewer than K tokens
 # are left: token 0 with q = 0 fills the set up, whether it is one of those left or not.
 @pytest.mark.parametrize("N,V", [(40, 700), (200, 30)])
