@@ -164,6 +164,8 @@ static int sm_count_or_default() {
     return device_info(&di) == HASS_OK ? di.sms : 148;
 }
 
+static int ceil_div(long long a, long long b) { return static_cast<int>((a + b - 1) / b); }
+
 // ---- tile schedule ----------------------------------------------------------------------------
 // Splits RT row tiles into phases (G row tiles x S lanes, G * S <= sms) minimising the summed phase
 // durations ceil(CT / S), by dynamic programming over the number of row tiles already covered. pair = 2: the
@@ -239,6 +241,7 @@ static int plan_launch(int RT, int CT, int sms, int max_slots, Schedule* out) {
 }
 
 // ---- division of the output tiles of MODE_OUT -----------------------------------------------------
+constexpr long long kKeepBytes = 64ll << 20;      // of W that the first of two readings leaves in the L2 (narrow_sweep)
 constexpr int kPartTilesMax = 296;      // partial tiles of one CTA each, at most (38.8 MB): two rounds of the grid
 
 // Over `rows` rows, CT column tiles and a contraction of `kb` blocks, with room for part_bytes of partial tiles. Expected
@@ -249,7 +252,12 @@ constexpr int kPartTilesMax = 296;      // partial tiles of one CTA each, at mos
 // A tile per cluster needs no partial tiles and no second kernel; it costs the exchange (6 steps) and fits while all
 // clusters are resident at once (clusters[]: how many are; nullptr: not considered).
 // 250 rows x 4096 x 32000, whose partial tiles do not fit the workspace: call 318 -> 235 us.
-static OutPlan plan_out(int rows, int CT, int kb, int sms, size_t part_bytes, const int* clusters) {
+// l2_cols > 0: B, of so many columns, is small enough to be in the L2 from the sweep before, and the contraction short. Few tiles of it are a chain of latencies, and narrower
+// ones leave a cluster less to exchange and every CTA less to load: 64 rows x 256 x 1024 22.0 -> 17.5 us per call, 53 x 280 x 2179 combined
+// 28.7 -> 20.5, 12 x 2784 x 4695 Bi-directional 47 -> 43. (Out of memory B comes faster in cut pieces of wide tiles, on
+// more of the SMs: 2 rows x 8192 x 128256 636 us per call, 699 with clusters of two on 128 columns; 128 x 4096 x 32000 122 and 135. Long contractions are better cut, too: 2048 x 256 x 32000 242 and 247.)
+constexpr int kShortBlocks = 256;
+static OutPlan plan_out(int rows, int CT, int kb, int sms, size_t part_bytes, const int* clusters, int l2_cols = 0) {
     const int RT = (rows + BM - 1) / BM;
     const int part_rows = RT == 1 ? rows : BM;      // rows kept of a partial tile
     const size_t tile_bytes = static_cast<size_t>(part_rows) * BN * 4;
@@ -275,6 +283,7 @@ static OutPlan plan_out(int rows, int CT, int kb, int sms, size_t part_bytes, co
                 best.pair = pair;
                 best.part_rows = part_rows;
                 best.cluster = 1;
+                best.width = BN;
                 best.row_units = units;
                 best.whole = cuts == 1 ? static_cast<int>(tiles) : whole;
                 best.rest = cuts == 1 ? 0 : rest;
@@ -285,9 +294,11 @@ static OutPlan plan_out(int rows, int CT, int kb, int sms, size_t part_bytes, co
             }
         }
     }
-    for (int c = 2; clusters && c <= MAX_CLUSTER; ++c) {
-        const long long tiles = static_cast<long long>(RT) * CT;
-        const double cost = (kb + c - 1) / c + 6. + 6.;
+    for (int cand = 0; clusters && cand < (l2_cols ? 3 : 1) * (MAX_CLUSTER - 1); ++cand) {
+        const int width = BN >> cand / (MAX_CLUSTER - 1), c = 2 + cand % (MAX_CLUSTER - 1);
+        const long long tiles = static_cast<long long>(RT) * (l2_cols ? ceil_div(l2_cols, width) : CT);
+        // a step fetches 16 KB of A and up to 32 of B; the exchange: 2 steps and up to 4
+        const double cost = (kb + c - 1) / c * (1. + 2. * width / BN) / 3. + 6. + 2. + 4. * width / BN;
         if (tiles > clusters[c] || kb < 2 * c || cost >= best_cost) continue;
         best_cost = cost;
         best = OutPlan{};
@@ -298,6 +309,7 @@ static OutPlan plan_out(int rows, int CT, int kb, int sms, size_t part_bytes, co
         best.groups = static_cast<int>(tiles) * c;
         best.part_rows = part_rows;
         best.cluster = c;
+        best.width = width;
     }
     return best;
 }
@@ -366,7 +378,6 @@ struct Layout {
     size_t part_bytes;               // partial tiles of the second GEMM, behind the scratch; without them it is not cut
 };
 
-static int ceil_div(long long a, long long b) { return static_cast<int>((a + b - 1) / b); }
 
 // Row tiles per chunk when at most `most` fit: all RT, or an even number of them (pairs of CTAs work on two).
 static int even_chunk(int most, int RT) {
@@ -626,7 +637,10 @@ static PartRoom part_room(uint8_t* ws, size_t workspace_bytes, const Layout& L, 
 static int launch_out(GemmParams& p, const PartRoom& room, const DeviceInfo& di, cudaStream_t st) {
     const long long left = p.rows_valid - p.row_global_offset;
     const int rows = static_cast<int>(left < static_cast<long long>(p.row_tiles) * BM ? left : p.row_tiles * BM);
-    p.plan = plan_out(rows, p.col_tiles, p.k_blocks, di.sms, room.bytes, di.clusters);
+    const long long w_bytes = 128ll * p.k_blocks * p.n_cols;
+    p.plan = plan_out(rows, p.col_tiles, p.k_blocks, di.sms, room.bytes, di.clusters, w_bytes <= kKeepBytes && p.k_blocks <= kShortBlocks ? p.n_cols : 0);
+    p.col_tiles = ceil_div(p.n_cols, p.plan.width);
+    if (p.plan.width < BN) p.kept = 1;      // (the instantiation that has such tiles)
     p.part = room.at;
     p.sched.pair = p.plan.pair;
     p.sched.max_ctas = p.plan.groups * p.plan.pair;
@@ -868,7 +882,6 @@ struct Combined {
 // sweep lets this much of W, its last k blocks, into the L2 like any other data and asks that the rest go first: 61 rows x 4096 x 32000
 // (262 MB) from a cold L2 129 -> 116 us, 100 rows 137 -> 125. Asking the L2 to hold those blocks longest (evict_last) gave the same, 117
 // and 127, but they stayed when the call was over: a pass over 80 MB of the caller's took 26.6 us after a call instead of 21.5.
-constexpr long long kKeepBytes = 64ll << 20;
 // From this size of W on the kernels of such a call let the next one's blocks in when they end: blocks that wait beside a
 // kernel bound by reading W cost it time (from a flushed L2 61 rows x 4096 x 32000 118.8 -> 114.8 us, 99 draft rows 117.5 -> 112.6, 100 rows
 // 129.0 -> 124.9); with a head of 0.5 MB it is the same (64 rows x 256 x 1024 30.3 us early, 30.0 late).
@@ -932,7 +945,9 @@ static int narrow_sweep(const void* H0, const void* H1, const void* W, int N, lo
     // 280 x 2179 combined 40 -> 29, 33 draft rows x 4096 x 32000 101.6 -> 95.9, 61 rows x 4096 x 128256 400 -> 388 (what is left there is
     // the rate at which boxes of 128 bytes a row come out of memory, 6.0 of 6.4 TB/s).
     const int pair = p.row_tiles > 1 ? 2 : 1, units = ceil_div(p.row_tiles, pair), lanes = std::max(1, di.sms / pair / units);
-    p.lane_cols = ceil_div(L.p_pitch / 32, lanes) * 32;
+    // (192 columns at least where W comes out of memory: the stages of a CTA hold too little of a narrower tile. 3 rows x 3136 x 21829 50 us per call in
+    // tiles of 256 on 86 CTAs, 56 in tiles of 160 on 138; from the L2 100 rows x 512 x 5000 33 -> 25)
+    p.lane_cols = std::max(ceil_div(L.p_pitch / 32, lanes) * 32, V * d * 2 > kKeepBytes ? 192 : 32);
     p.sched.n_phases = 1;
     p.sched.pair = pair;
     p.sched.ph[0] = Phase{0, units * pair, ceil_div(L.p_pitch, p.lane_cols), 0};
@@ -1749,9 +1764,9 @@ static int normed_impl(const void* H_t, const void* H_d, const void* W, long lon
     f.loss = loss;
     f.dH = dH_d;
     f.dH_fp32 = dH_dtype == HASS_FP32 ? 1 : 0;
-    // as many blocks per row as are resident at once, of 256 columns at least
+    // as many blocks per row as are resident at once, of 256 columns at least, 2048 where there is one group of tokens to gather
     f.split = 1;
-    while (f.split < NORMED_MAX && 2 * f.split * N <= 3ll * di.sms && d >= 512ll * f.split) f.split *= 2;
+    while (f.split < NORMED_MAX && 2 * f.split * N <= 3ll * di.sms && d >= (K > FIN_GRP ? 512ll : 4096ll) * f.split) f.split *= 2;
     KernelTimer timer(KIND_FINALIZE, st);
     return launch(normed_kernel, N * f.split, NORMED_THREADS, gather_smem(ceil_div(d / 8, f.split) * 8), st, f.split, f);
 }

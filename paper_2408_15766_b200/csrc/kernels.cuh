@@ -90,6 +90,7 @@ struct OutPlan {
     int pair, groups, row_units, whole, rest, cuts;
     int part_rows;         // rows kept of a partial tile: BM, or all there are in a single row tile
     int cluster;
+    int width;             // columns of a tile: BN, or 128 or 64 of a cluster's (then GemmParams::kept)
 };
 
 struct GemmParams {
@@ -142,7 +143,8 @@ struct GemmParams {
     int lane_cols;         // lane l sweeps the columns [l lane_cols, (l + 1) lane_cols) below z_pitch, in tiles of BN and a
                            // narrower last one (a multiple of 32)
     int keep_from;         // k block from which on the L2 holds this sweep's tiles of B like any other's; those before it go first ...
-    int kept;              // MODE_OUT: ... as all do in the second reading of B, which this is (host: selects the instantiation)
+    int kept;              // MODE_OUT: ... as all do in the second reading of B, which this is (host: selects the instantiation, which also has
+                           // narrower tiles)
     int release_late;      // the next kernel's blocks may start when this one's have ended, not before
     int clear_status;      // the first CTA zeroes the status block (no kernel of the call has run before this one)
     // MODE_OUT. With sparse != nullptr the epilogue computes coef[row] * acc - sparse[local row, :] (row scale
@@ -542,10 +544,11 @@ __global__ void __launch_bounds__(gemm_threads(EW), 1) gemm_kernel(const __grid_
     };
     auto tile_col = [&](int ln, int S, int t) {
         if constexpr (MODE == MODE_LOGITS) return ln * p.lane_cols + t * BN;
-        return (t < 0 ? 0 : ln + t * S) * BN;      // t = -1: column tile 0, for the row references only
+        return (t < 0 ? 0 : ln + t * S) * (KEPT && CG == 1 ? p.plan.width : BN);      // t = -1: column tile 0, for the row references only
     };
     auto tile_width = [&](int t) {
         if constexpr (MODE == MODE_LOGITS) return min(BN, p.lane_cols - t * BN);
+        if constexpr (KEPT && CG == 1) return p.plan.width;
         return BN;
     };
     // Where rows spill without a given reference exponent, a lane that does not begin with column tile 0 computes it first
@@ -603,10 +606,10 @@ __global__ void __launch_bounds__(gemm_threads(EW), 1) gemm_kernel(const __grid_
                         if (!B_MN_MAJOR) {
                             load_b(smemB + stage * B_STAGE_BYTES, kb * BK, col0);
                         } else {
-                            // B tile = BK contraction rows x BN / CG contiguous columns, fetched as boxes
+                            // B tile = BK contraction rows x width / CG contiguous columns, fetched as boxes
                             // of 64 columns (one 128-byte swizzle row) x BK rows
 #pragma unroll
-                            for (int j = 0; j < BN / CG / 64; ++j)
+                            for (int j = 0; j < width / CG / 64; ++j)
                                 load_b(smemB + stage * B_STAGE_BYTES + j * (BK * 128), col0 + j * 64, kb * BK);
                         }
                         if (++stage == STAGES) {
@@ -1337,11 +1340,11 @@ __global__ void __launch_bounds__(gemm_threads(EW), 1) gemm_kernel(const __grid_
         const int C = p.plan.cluster;
         if (C > 1) {
             // The operand stages hold [C pieces][rows per CTA][ROW_PITCH] floats now: every CTA's products are complete.
-            constexpr int ROW_PITCH = BN + 4;               // rows 4 banks apart
-            static_assert((BM + 8) * ROW_PITCH * 4 <= OPERAND_BYTES, "the pieces of a CTA's rows fit the operand stages");
+            const int width = tile_width(0), ROW_PITCH = width + 4;               // rows 4 banks apart
+            static_assert((BM + 8) * (BN + 4) * 4 <= OPERAND_BYTES, "the pieces of a CTA's rows fit the operand stages");
             const int u = cta / C, z = cta - u * C;
             const int rt = u % p.plan.row_units, ct = u / p.plan.row_units;
-            const int per = (BM + C - 1) / C;
+            const int per = (min(BM, p.rows_valid - p.row_global_offset - rt * BM) + C - 1) / C;      // (rows that exist are dealt out)
             tc_fence_before_sync();
             __syncthreads();
             cluster_sync();
@@ -1351,7 +1354,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), 1) gemm_kernel(const __grid_
                 const uint32_t dst = map_to_rank(smem_base + (z * per + r % per) * ROW_PITCH * 4, r / per);
                 const bool row_ok = p.row_global_offset + rt * BM + r < p.rows_valid;
 #pragma unroll 1
-                for (int ch = 0; ch < BN / 32; ++ch) {
+                for (int ch = 0; ch < width / 32; ++ch) {
                     uint32_t v[32];
                     tmem_ld32(tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + ch * 32, v);
                     tmem_ld_wait(v);
@@ -1362,9 +1365,9 @@ __global__ void __launch_bounds__(gemm_threads(EW), 1) gemm_kernel(const __grid_
                 }
             }
             cluster_sync();
-            for (int i = threadIdx.x; i < per * (BN / 4); i += NUM_THREADS) {
-                const int rl = i / (BN / 4), c = i % (BN / 4) * 4;
-                const int r = z * per + rl, row = p.row_global_offset + rt * BM + r, col = ct * BN + c;
+            for (int i = threadIdx.x; i < per * (width / 4); i += NUM_THREADS) {
+                const int rl = i / (width / 4), c = i % (width / 4) * 4;
+                const int r = z * per + rl, row = p.row_global_offset + rt * BM + r, col = ct * width + c;
                 if (r >= BM || row >= p.rows_valid || col >= p.n_cols) continue;
                 const uint8_t* src = smem_gen + (rl * ROW_PITCH + c) * 4;
                 float4 a = *reinterpret_cast<const float4*>(src);
