@@ -87,6 +87,8 @@ struct DeviceInfo {
     int ok = 0;   // 0 unknown, 1 usable, <0 hass_status
     int sms = 148;
     int clusters[MAX_CLUSTER + 1] = {};   // clusters of this many CTAs of the second GEMM that are resident at once
+    int hca_clusters[MAX_CLUSTER + 1] = {};   // ... of the attention's backward
+    int hca_fwd_clusters[MAX_CLUSTER + 1] = {};   // ... and forward
 };
 static DeviceInfo g_dev[64];
 
@@ -122,9 +124,11 @@ static int device_info(DeviceInfo* out) {
                 if (e3 == cudaSuccess) e3 = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
             if (e3 == cudaSuccess) e3 = cudaFuncSetAttribute(select_kernel<16, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * 512 * 8);
             if (e3 == cudaSuccess) e3 = cudaFuncSetAttribute(select_kernel<16, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * 1024 * 8);
-            cudaError_t e4 = cudaFuncSetAttribute(hca2::hca_attention_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, hca2::SMEM_BYTES);
+            cudaError_t e4 = cudaFuncSetAttribute(hca2::hca_attention_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, hca2::SMEM_BYTES);
+            if (e4 == cudaSuccess) e4 = cudaFuncSetAttribute(hca2::hca_attention_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, hca2::SMEM_BYTES);
             if (e4 == cudaSuccess) e4 = cudaFuncSetAttribute(hca_bwd::hca_bwd_fused_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, hca_bwd::F_SMEM_BYTES);
             if (e4 == cudaSuccess) e4 = cudaFuncSetAttribute(hca_bwd::hca_bwd_fused_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, hca_bwd::F_SMEM_BYTES);
+            if (e4 == cudaSuccess) e4 = cudaFuncSetAttribute(hca_bwd::hca_bwd_fused_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, hca_bwd::F_SMEM_BYTES);
             for (int c = 2; c <= MAX_CLUSTER; ++c) {
                 cudaLaunchConfig_t cfg = {};
                 cfg.gridDim = dim3(c);
@@ -140,6 +144,18 @@ static int device_info(DeviceInfo* out) {
                 if (cudaOccupancyMaxActiveClusters(&di.clusters[c], gemm_kernel<MODE_OUT, TOPK_BUF, 1>, &cfg) != cudaSuccess) {
                     cudaGetLastError();
                     di.clusters[c] = 0;
+                }
+                cfg.blockDim = dim3(hca_bwd::NUM_THREADS);
+                cfg.dynamicSmemBytes = hca_bwd::F_SMEM_BYTES;
+                if (cudaOccupancyMaxActiveClusters(&di.hca_clusters[c], hca_bwd::hca_bwd_fused_kernel<1, true>, &cfg) != cudaSuccess) {
+                    cudaGetLastError();
+                    di.hca_clusters[c] = 0;
+                }
+                cfg.blockDim = dim3(hca2::NUM_THREADS);
+                cfg.dynamicSmemBytes = hca2::SMEM_BYTES;
+                if (cudaOccupancyMaxActiveClusters(&di.hca_fwd_clusters[c], hca2::hca_attention_pair_kernel<true>, &cfg) != cudaSuccess) {
+                    cudaGetLastError();
+                    di.hca_fwd_clusters[c] = 0;
                 }
             }
             if (e3 != cudaSuccess || e4 != cudaSuccess) {
@@ -2222,6 +2238,26 @@ int hass_hca_attention_workspace_bytes(size_t* bytes) {
     return HASS_OK;
 }
 
+// CTAs per item of the forward, a cluster, where every item has a CTA of its own: as many as are worth their exchange while all clusters are resident
+// at once; 1: no clusters. In half key tiles (0.9 us each): a draft pass counts one, the exchange five. 1 x 1000 positions, 4 / 2 heads, m = 0 18.6 ->
+// 14.2 us, 1 x 1829, m = 3 33.0 -> 25.8, 1 x 2435, 2 / 1 heads 40.6 -> 28.3, 1 x 3749 55.2 -> 36.1; 2 x 333, 4 / 2 heads, m = 3 13.2 alone, 14.5 in
+// pairs, 5 x 48 8.5 and 12.8.
+static int hca_fwd_cluster(int items, int q_tiles, int m, const int* clusters) {
+    int best = 1, cost = 2 * q_tiles + m;
+    for (int c = 2; c <= MAX_CLUSTER; c *= 2) {
+        int with = 0;
+        for (int z = 0; z < c; ++z) {
+            int j0, j1;
+            hca2::tile_share(q_tiles, m, z, c, j0, j1);
+            with = std::max(with, 2 * (j1 - j0) + (z + 1 == c ? m : 0));
+        }
+        if (items > clusters[c] || with + 5 >= cost) continue;
+        best = c;
+        cost = with + 5;
+    }
+    return best;
+}
+
 int hass_hca_attention_fwd(const void* Q, const void* K_t, const void* V_t, const void* const* K_d,
                            const void* const* V_d, int32_t m, int64_t B, int64_t T, int64_t H, int64_t Hkv, int64_t D,
                            float scale, void* O, float* lse, void* workspace, size_t workspace_bytes,
@@ -2275,14 +2311,15 @@ int hass_hca_attention_fwd(const void* Q, const void* K_t, const void* V_t, cons
         p.pairs = p.single ? static_cast<int>(B * H) * p.q_tiles : p.head_pairing ? static_cast<int>(B * (H / 2)) * p.q_tiles : static_cast<int>(B * H) * ((p.q_tiles + 1) / 2);
         p.c2 = scale * 1.4426950408889634f;
         p.status = static_cast<unsigned int*>(workspace);
-        const int grid = p.pairs < di.sms ? p.pairs : di.sms;
-        p.one_round = p.pairs == grid ? 1 : 0;
+        p.cluster = p.single ? hca_fwd_cluster(p.pairs, p.q_tiles, m, di.hca_fwd_clusters) : 1;
+        const int grid = p.cluster > 1 ? p.pairs * p.cluster : p.pairs < di.sms ? p.pairs : di.sms;
+        p.one_round = p.cluster > 1 || p.pairs == grid ? 1 : 0;
         if (!p.one_round) {
             rc = clear_bytes(workspace, 256, st);
             if (rc != HASS_OK) return rc;
         }
         KernelTimer kt(KIND_HCA, st);
-        return launch(hca2::hca_attention_pair_kernel, grid, hca2::NUM_THREADS, hca2::SMEM_BYTES, st, 1, p);
+        return launch(p.cluster > 1 ? hca2::hca_attention_pair_kernel<true> : hca2::hca_attention_pair_kernel<false>, grid, hca2::NUM_THREADS, hca2::SMEM_BYTES, st, p.cluster, p);
     }
 }
 
@@ -2325,6 +2362,23 @@ static int hca_bwd_parts(int BG, int rep, int T, int sms) {
         }
     }
     return 6 * most[2] < 5 * most[1] ? 2 : 1;
+}
+
+// CTAs per key tile of the backward, a cluster: as many as are worth their exchange where all clusters are resident at once; 1: no clusters. In
+// elements (1.35 us each): the exchange costs about four. Forward + backward: 3 x 124 positions, 64 / 8 heads (24 tiles of 16 elements in
+// fours) 50.7 -> 42.9 us, 2 x 333, 4 / 2 heads (12 tiles of up to 12, in eights) 42.8 -> 38.5; 4 x 60, 32 / 8 heads (4 elements) 27.8 alone, 31.5 in
+// pairs, 8 x 100, 2 / 1 heads 33.1 and 36.3.
+static int hca_bwd_cluster(int BG, int rep, int T, const int* clusters) {
+    const int kt_tiles = ceil_div(T, hca_bwd::KEYS), most = rep * ceil_div(T, hca_bwd::QE);      // elements of the longest tile
+    int best = 1;
+    double cost = most;
+    for (int c = 2; c <= MAX_CLUSTER; c *= 2) {
+        const double with = ceil_div(most, c) + 4.;
+        if (static_cast<int64_t>(BG) * kt_tiles > clusters[c] || with >= 0.9 * cost) continue;
+        best = c;
+        cost = with;
+    }
+    return best;
 }
 
 int hass_hca_attention_bwd_workspace_bytes(int64_t B, int64_t T, int64_t H, int32_t m, size_t* bytes) {
@@ -2394,6 +2448,7 @@ int hass_hca_attention_bwd(const void* Q, const void* K_t, const void* V_t, cons
     int parts = 1;
     if (workspace_bytes >= L.total + hca_bwd_split_bytes(B * Hkv * k.kt_tiles)) parts = hca_bwd_parts(iB * iHkv, iH / iHkv, iT, di.sms);
     const bool split = parts > 1;
+    k.cluster = split ? 1 : hca_bwd_cluster(iB * iHkv, iH / iHkv, iT, di.hca_clusters);
     float* dKVacc = reinterpret_cast<float*>(ws + L.dKVacc);
     k.dKVacc = dKVacc;
     {   // D, the substituted entries and everything that follows from them, the start value of the dQ accumulator
@@ -2435,7 +2490,10 @@ int hass_hca_attention_bwd(const void* Q, const void* K_t, const void* V_t, cons
     k.status = static_cast<unsigned int*>(workspace);
     {
         KernelTimer kt(KIND_HCA_BWD_FUSED, st);
-        rc = launch(split ? hca_bwd::hca_bwd_fused_kernel<2> : hca_bwd::hca_bwd_fused_kernel<1>, k.items * parts < di.sms ? k.items * parts : di.sms, hca_bwd::NUM_THREADS, hca_bwd::F_SMEM_BYTES, st, 1, k);
+        if (k.cluster > 1)
+            rc = launch(hca_bwd::hca_bwd_fused_kernel<1, true>, k.items * k.cluster, hca_bwd::NUM_THREADS, hca_bwd::F_SMEM_BYTES, st, k.cluster, k);
+        else
+            rc = launch(split ? hca_bwd::hca_bwd_fused_kernel<2> : hca_bwd::hca_bwd_fused_kernel<1>, k.items * parts < di.sms ? k.items * parts : di.sms, hca_bwd::NUM_THREADS, hca_bwd::F_SMEM_BYTES, st, 1, k);
     }
     if (rc != HASS_OK) return rc;
 

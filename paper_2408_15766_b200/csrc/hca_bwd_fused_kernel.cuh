@@ -372,6 +372,9 @@ __global__ void __launch_bounds__(256) hca_dq_convert_kernel(const __grid_consta
 // that does nothing else).
 // PARTS = 2: two work items per key tile, each with half of its elements, where whole ones would leave most of the SMs without
 // work at the end. Their dV and dK are added up in global memory. (Two terms on top of zero: the order of arrival does not matter.)
+// CLUSTER: a cluster of p.cluster CTAs per key tile, each with its part of the tile's elements, one tile per CTA, where the tiles are so few that all
+// clusters are resident at once. In the end the CTAs hand one another their dV and dK by rows through distributed shared memory, in
+// the room of the operands, and each adds up and stores 128 / p.cluster rows, in the order of the parts (hca_bwd_cluster has the line).
 constexpr int F_STAGES = 3;             // a Q / dO stage is held until the element's last product is done
 constexpr int F_SMEM_K = 0;
 constexpr int F_SMEM_V = F_SMEM_K + K_BYTES;
@@ -405,10 +408,13 @@ struct FusedParams {
     float* dKVacc;                 // PARTS = 2: dV and dK in fp32, [2][B, Hkv, key tile, 32, 128, 4]: a thread's row in groups of four
                                    // columns, the rows of a warp side by side
     float c2, scale;
+    int cluster;                   // CLUSTER: CTAs per key tile: 2, 4 or 8
     unsigned int* status;
 };
+constexpr int F_ROW_PITCH = HD + 4;     // floats of a handed-over row: rows 4 banks apart
+static_assert(2 * KEYS * F_ROW_PITCH * 4 <= F_SMEM_DS, "the parts of a CTA's rows fit the operands");
 
-template <int PARTS>
+template <int PARTS, bool CLUSTER = false>
 __global__ void __launch_bounds__(NUM_THREADS, 1) hca_bwd_fused_kernel(const __grid_constant__ FusedParams p) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t base = smem_u32(smem_raw);
@@ -485,27 +491,28 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_bwd_fused_kernel(const __g
     // elements of a key tile: for each head of the group, the 64-query tiles 2 kt .. q_tiles64 - 1
     auto q_count = [&](int kt) { return p.q_tiles64 - 2 * kt; };
     // item -> (key tile, sequence, key/value head, elements [e0, e1)): the first key tiles meet the most queries and come first
+    const int parts = CLUSTER ? p.cluster : PARTS;
     auto decode = [&](int item, int& kt, int& b, int& g, int& e0, int& e1) {
-        const int tile = item / PARTS, z = item - tile * PARTS;
+        const int tile = item / parts, z = item - tile * parts;
         kt = tile / BG;
         const int bg = tile - kt * BG;
         b = bg / p.Hkv;
         g = bg - b * p.Hkv;
         const int n_e = rep * q_count(kt);
-        e0 = n_e * z / PARTS;
-        e1 = n_e * (z + 1) / PARTS;
+        e0 = n_e * z / parts;
+        e1 = n_e * (z + 1) / parts;
     };
-    const int n_items = p.items * PARTS;
+    const int n_items = p.items * parts;      // (CLUSTER: as many as CTAs; a cluster's are consecutive)
     const int n_rounds = (n_items + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x);
     auto next_item = [&](int& k) {
         while (k < n_rounds) {
             const int item = round_item(static_cast<uint32_t>((k + static_cast<int>(blockIdx.x)) % n_rounds));
             ++k;
             if (item >= n_items) continue;
-            if (PARTS > 1) {
+            if (PARTS > 1 || CLUSTER) {
                 int kt, b, g, e0, e1;
                 decode(item, kt, b, g, e0, e1);
-                if (e0 == e1) continue;      // the first half of a single element
+                if (e0 == e1) continue;      // fewer elements than parts
             }
             return item;
         }
@@ -792,6 +799,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_bwd_fused_kernel(const __g
             if (!take_dq(gq - 1, b, g * rep + (e1 - 1) / nq, 2 * kt + (e1 - 1) % nq)) break;
             // ---- epilogue: this key row of dV (group 0) or dK (group 1) as bf16, or its share of it in fp32 ----
             if (!wait_barrier(acc_done, it & 1u, abort_flag, p.status, 13)) break;
+            if (CLUSTER) break;
             tc_fence_after_sync();
             const bool valid = spos < p.T;
             const size_t orow = ((static_cast<size_t>(b) * p.T + (valid ? spos : 0)) * p.Hkv + g) * HD;
@@ -835,6 +843,46 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_bwd_fused_kernel(const __g
             }
         }
         if (issuer) bulk_wait_group0();     // shared memory must outlive the reductions that read it
+    }
+
+    if constexpr (CLUSTER) {
+        // every CTA's products are complete, its operands' room is free
+        const int C = p.cluster, z = static_cast<int>(blockIdx.x) % C, rows = KEYS / C;
+        int kt, b, g, e0, e1;
+        decode(static_cast<int>(blockIdx.x), kt, b, g, e0, e1);
+        tc_fence_before_sync();
+        __syncthreads();
+        cluster_sync();
+        tc_fence_after_sync();
+        if (warp >= 2 && warp < VEC_WARP) {
+            const int grp = (warp - 2) >> 2, quad = warp & 3, r = quad * 32 + lane;
+            const uint32_t dst = map_to_rank(base + ((z * 2 + grp) * rows + r % rows) * (F_ROW_PITCH * 4), r / rows);
+#pragma unroll 1
+            for (int c0 = 0; c0 < HD; c0 += 32) {
+                uint32_t v[32];
+                tmem_ld32(tmem_base + 256 + 128 * grp + (static_cast<uint32_t>(quad * 32) << 16) + c0, v);
+                tmem_ld_wait(v);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    if (e0 == e1) v[4 * j] = v[4 * j + 1] = v[4 * j + 2] = v[4 * j + 3] = 0u;      // no element: no accumulator
+                    st_cluster_v4(dst + (c0 + 4 * j) * 4, v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                }
+            }
+        }
+        cluster_sync();
+        for (int i = threadIdx.x; i < 2 * rows * (HD / 8); i += NUM_THREADS) {
+            const int c8 = i % (HD / 8), rl = i / (HD / 8) % rows, grp = i / (HD / 8) / rows;
+            const int spos = kt * KEYS + z * rows + rl;
+            if (spos >= p.T) continue;
+            float f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            for (int q = 0; q < C; ++q) {
+                const float4* src = reinterpret_cast<const float4*>(smem_raw + ((q * 2 + grp) * rows + rl) * (F_ROW_PITCH * 4) + c8 * 32);
+                const float4 x = src[0], y = src[1];
+                f[0] += x.x; f[1] += x.y; f[2] += x.z; f[3] += x.w;
+                f[4] += y.x; f[5] += y.y; f[6] += y.z; f[7] += y.w;
+            }
+            reinterpret_cast<uint4*>((grp == 0 ? p.dV : p.dK) + ((static_cast<size_t>(b) * p.T + spos) * p.Hkv + g) * HD)[c8] = narrow8(f);
+        }
     }
 
     tc_fence_before_sync();

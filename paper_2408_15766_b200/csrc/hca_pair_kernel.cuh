@@ -27,6 +27,9 @@
 // No thread reads global memory.
 // The running reference moves only when a tile's maximum exceeds it by more than 2^8 (the accumulator is then
 // rescaled in place by the row's thread), so P stays within bf16 range and almost every tile skips the rescale.
+// CLUSTER: a cluster of p.cluster CTAs per item, each with a part of its key tiles (the last one, which ends with the diagonal's, has the draft
+// passes as well), where items are so few that all clusters are resident at once. In the end the CTAs hand one another their accumulators,
+// references and sums by rows through distributed shared memory, and each finishes 128 / p.cluster rows (hca_fwd_cluster has the line).
 // Warps: 0 = TMA producer, 1 = MMA issuer and TMEM owner (2, 3 idle), 4-7 = softmax + epilogue of slot 0,
 // 8-11 = of slot 1 (TMEM lane quadrant = warp % 4). The first warpgroup gives registers up (setmaxnreg) and the
 // two softmax warpgroups take them: a row's 128 scores stay in registers. Every wait is bounded (wait_barrier); a wait that gives up sets the status
@@ -85,6 +88,7 @@ struct Params {
     int head_pairing;              // 1: a pair = heads 2u, 2u + 1 at one query tile; 0: one head, query tiles qt - 1, qt
     int single;                    // 1 (head_pairing = 0): a "pair" is one item, in slot 1
     float c2;                      // scale * log2(e)
+    int cluster;                   // CLUSTER: CTAs per item: 2, 4 or 8 (single = 1, one_round = 1)
     int one_round;                 // every CTA takes one pair: no counter, and the status block is cleared here
     unsigned int* status;
 };
@@ -120,6 +124,18 @@ __device__ __forceinline__ Pair decode_pair(const Params& p, int idx) {
     return r;
 }
 
+constexpr int ROW_PITCH = HD + 4;  // floats of a handed-over row (the accumulator, its reference, its sum): rows 4 banks apart
+static_assert(QT * ROW_PITCH * 4 <= SMEM_V, "the parts of a CTA's rows fit the room of queries and keys");
+
+// The part [j0, j1) of n key tiles that is CTA z's of C: even shares, a draft pass counting as half a tile of the last CTA's, which has one tile at least
+__host__ __device__ __forceinline__ void tile_share(int n, int m, int z, int C, int& j0, int& j1) {
+    const int total = 2 * n + m;
+    const int from = total * z / (2 * C), to = total * (z + 1) / (2 * C);
+    j0 = from < n - 1 ? from : n - 1;
+    j1 = z + 1 == C ? n : to < n - 1 ? to : n - 1;
+}
+
+template <bool CLUSTER>
 __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(const __grid_constant__ Params p) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t base = smem_u32(smem_raw);
@@ -147,6 +163,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
+    // this CTA's index among its cluster's, and the key tiles and draft passes it takes of slot 1's item
+    const int z = CLUSTER ? static_cast<int>(blockIdx.x) % p.cluster : 0;
+    auto own_share = [&](const Pair& pr, int& j0, int& j1) {
+        j0 = 0;
+        j1 = pr.qt[1] + 1;
+        if (CLUSTER) tile_share(j1, p.m, z, p.cluster, j0, j1);
+    };
+    const int md = CLUSTER && z + 1 < p.cluster ? 0 : p.m;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2; ++s) {
@@ -236,7 +260,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
                 return true;
             };
             for (;; ++it) {
-                const int idx = !p.one_round ? static_cast<int>(atomicAdd(p.status + 1, 1u)) : it == 0 ? static_cast<int>(blockIdx.x) : INT_MAX;
+                const int idx = !p.one_round ? static_cast<int>(atomicAdd(p.status + 1, 1u)) : it == 0 ? static_cast<int>(blockIdx.x) / (CLUSTER ? p.cluster : 1) : INT_MAX;
                 {
                     const int e = it % SCHED_DEPTH;
                     if (!wait_barrier(sched_empty(e), ((it / SCHED_DEPTH) & 1u) ^ 1u, abort_flag, p.status, 15)) break;
@@ -245,6 +269,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
                 }
                 if (idx >= p.pairs || !ok) break;
                 const Pair pr = decode_pair(p, idx);
+                int j0, n;
+                own_share(pr, j0, n);
+                if (CLUSTER && j0 == n) continue;
 #pragma unroll
                 for (int s = 0; s < 2; ++s) {
                     if (s == 0 && !pr.act0) continue;
@@ -254,17 +281,16 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
                     tma_load_3d(base + SMEM_Q + s * Q_BYTES + Q_HALF, &p.tmQ, q_full(s), pr.h[s] * HD + 64, pr.qt[s] * QT, pr.b);
                     ++gq[s];
                 }
-                const int n = pr.qt[1] + 1;
                 // draft keys start i rows early: row c of the tile is position qt * 128 + c - i (zeros before the sequence)
-                for (int i = 0; i < p.m && ok; ++i) {
+                for (int i = 0; i < md && ok; ++i) {
                     if (!p.head_pairing && pr.act0) ok = load_k(&p.tmKd[i], pr.kv_col, pr.qt[0] * QT - i, pr.b);
                     if (ok) ok = load_k(&p.tmKd[i], pr.kv_col, pr.qt[1] * QT - i, pr.b);
                 }
-                for (int j = 0; j < n && ok; ++j) {
+                for (int j = j0; j < n && ok; ++j) {
                     ok = load_k(&p.tmK, pr.kv_col, j * KT, pr.b);
                     if (ok) ok = load_v(&p.tmV, pr.kv_col, j * KT, pr.b);
                 }
-                for (int i = 0; i < p.m && ok; ++i) {
+                for (int i = 0; i < md && ok; ++i) {
                     if (!p.head_pairing && pr.act0) ok = load_v(&p.tmVd[i], pr.kv_col, pr.qt[0] * QT - i, pr.b);
                     if (ok) ok = load_v(&p.tmVd[i], pr.kv_col, pr.qt[1] * QT - i, pr.b);
                 }
@@ -353,8 +379,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
 
         for (int idx = next_pair(0, 16); idx < p.pairs && ok; idx = next_pair(++it, 16)) {
             const Pair pr = decode_pair(p, idx);
-            const int m = p.m;
-            const int n1 = pr.qt[1] + 1;
+            const int m = md;
+            int j0, n1;
+            own_share(pr, j0, n1);
+            n1 -= j0;                                        // key tiles of slot 1
+            if (CLUSTER && n1 == 0) continue;
             const int n0 = pr.act0 ? pr.qt[0] + 1 : 0;
             const bool a_on = pr.act0;
             const bool shared = p.head_pairing != 0;         // the draft tiles serve both slots
@@ -459,13 +488,17 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
         const uint32_t tmem_s = tmem_base + slot * KT + lane_addr;
         const uint32_t tmem_o = tmem_base + 256 + slot * HD + lane_addr;
         const int m = p.m;
+        float own_ref = -INFINITY, own_sum = 0.f;             // CLUSTER: of the row's part
+        bool own_rows = false;
         uint32_t gs = 0, gpv = 0, it = 0;                     // S-type products seen, PV-type products requested
         bool ok = true;
         for (int idx = next_pair(0, 17); idx < p.pairs && ok; idx = next_pair(++it, 17)) {
             const Pair pr = decode_pair(p, idx);
             if (slot == 0 && !pr.act0) continue;
             const int qt = pr.qt[slot], h = pr.h[slot], b = pr.b;
-            const int n = qt + 1;
+            int j0 = 0, n = qt + 1;
+            if (CLUSTER) own_share(pr, j0, n);
+            if (CLUSTER && j0 == n) continue;
             const int t = qt * QT + r;                        // position in the sequence
             const bool valid = t < p.T;
             // ---- draft score steps: keep the diagonal element of each S (raw, unscaled) ----
@@ -473,7 +506,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
 #pragma unroll
             for (int i = 0; i < MAX_DRAFTS; ++i) sd[i] = 0.f;
 #pragma unroll 1
-            for (int i = 0; i < m; ++i, ++gs) {
+            for (int i = 0; i < md; ++i, ++gs) {
                 if (!wait_barrier(s_full(slot), gs & 1u, abort_flag, p.status, 10)) { ok = false; break; }
                 tc_fence_after_sync();
                 uint32_t blk[32];
@@ -493,7 +526,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
             if (!ok) break;
             float mref = -INFINITY, l = 0.f;
 #pragma unroll 1
-            for (int j = 0; j < n; ++j, ++gs) {
+            for (int j = j0; j < n; ++j, ++gs) {
                 if (!wait_barrier(s_full(slot), gs & 1u, abort_flag, p.status, 10)) { ok = false; break; }
                 tc_fence_after_sync();
                 const bool last = (j == n - 1);
@@ -525,10 +558,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
                 if (last) {
 #pragma unroll
                     for (int i = 0; i < MAX_DRAFTS; ++i)
-                        if (i < m && t - i >= 0) mxa = fmaxf(mxa, sd[i]);
+                        if (i < md && t - i >= 0) mxa = fmaxf(mxa, sd[i]);
                 }
                 const float cand = mxa * p.c2;
-                if (j == 0) {
+                if (j == j0) {
                     mref = cand;
                 } else {
                     const bool grow = cand > mref + RESCALE_LOG2;      // also true when every earlier column of the row was hidden
@@ -575,7 +608,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
                     // the substituted entries' weights: pass i in 8 columns beside P, this row's in the word of its key
 #pragma unroll
                     for (int i = 0; i < MAX_DRAFTS; ++i) {
-                        if (i < m) {
+                        if (i < md) {
                             const float pi = t - i >= 0 ? ex2(fmaf(sd[i], p.c2, nref)) : 0.f;
                             l += pi;
                             const uint32_t bits = pack_bf16(pi, 0.f) << ((r & 1) * 16);
@@ -596,6 +629,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
             // ---- epilogue: O / l as bf16, each thread stores its own 256-byte row ----
             if (!wait_barrier(pv_done(slot), (gpv - 1u) & 1u, abort_flag, p.status, 13)) break;
             tc_fence_after_sync();
+            if (CLUSTER) {
+                own_ref = mref;
+                own_sum = l;
+                own_rows = true;
+                break;
+            }
             const float inv = 1.f / l;
             if (valid && p.lse != nullptr)
                 p.lse[(static_cast<size_t>(b) * p.H + h) * p.T + t] = (mref + log2f(l)) * 0.6931471805599453f;
@@ -628,6 +667,58 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) hca_attention_pair_kernel(cons
             // the accumulator and the score buffer go back to the tensor core with the next item's first step
             tc_fence_before_sync();
         }
+        if constexpr (CLUSTER) {
+            const int C = p.cluster, rows = QT / C;
+            const Pair pr = decode_pair(p, static_cast<int>(blockIdx.x) / C);
+            tc_fence_before_sync();
+            __syncthreads();
+            cluster_sync();                                   // every CTA's products are complete, its queries' and keys' room is free
+            tc_fence_after_sync();
+            if (slot == 1) {
+                const uint32_t dst = map_to_rank(base + (z * rows + r % rows) * (ROW_PITCH * 4), r / rows);
+#pragma unroll 1
+                for (int c0 = 0; c0 < HD; c0 += 32) {
+                    uint32_t v[32];
+                    tmem_ld32(tmem_o + c0, v);
+                    tmem_ld_wait(v);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        if (!own_rows) v[4 * j] = v[4 * j + 1] = v[4 * j + 2] = v[4 * j + 3] = 0u;      // no tile: no accumulator
+                        st_cluster_v4(dst + (c0 + 4 * j) * 4, v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                    }
+                }
+                st_cluster_v4(dst + HD * 4, __float_as_uint(own_ref), __float_as_uint(own_sum), 0u, 0u);
+            }
+            cluster_sync();
+            for (int i = static_cast<int>(threadIdx.x) - 128; i < rows * (HD / 8); i += 256) {
+                const int c8 = i % (HD / 8), rl = i / (HD / 8), t = pr.qt[1] * QT + z * rows + rl;
+                if (t >= p.T) continue;
+                const float* src = reinterpret_cast<const float*>(smem_raw) + rl * ROW_PITCH;
+                float ref = -INFINITY, sum = 0.f, f[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                for (int q = 0; q < C; ++q) ref = fmaxf(ref, src[q * rows * ROW_PITCH + HD]);
+                for (int q = 0; q < C; ++q) {
+                    const float* part = src + q * rows * ROW_PITCH;
+                    const float w = ex2(part[HD] - ref);      // (a part without a visible key: 2^-inf)
+                    sum = fmaf(w, part[HD + 1], sum);
+                    const float4 x = *reinterpret_cast<const float4*>(part + 8 * c8), y = *reinterpret_cast<const float4*>(part + 8 * c8 + 4);
+                    f[0] = fmaf(w, x.x, f[0]); f[1] = fmaf(w, x.y, f[1]); f[2] = fmaf(w, x.z, f[2]); f[3] = fmaf(w, x.w, f[3]);
+                    f[4] = fmaf(w, y.x, f[4]); f[5] = fmaf(w, y.y, f[5]); f[6] = fmaf(w, y.z, f[6]); f[7] = fmaf(w, y.w, f[7]);
+                }
+                const float inv = 1.f / sum;
+                if (c8 == 0 && p.lse != nullptr)
+                    p.lse[(static_cast<size_t>(pr.b) * p.H + pr.h[1]) * p.T + t] = (ref + log2f(sum)) * 0.6931471805599453f;
+                reinterpret_cast<uint4*>(p.O + ((static_cast<size_t>(pr.b) * p.T + t) * p.H + pr.h[1]) * HD)[c8] =
+                    make_uint4(pack_bf16(f[0] * inv, f[1] * inv), pack_bf16(f[2] * inv, f[3] * inv), pack_bf16(f[4] * inv, f[5] * inv), pack_bf16(f[6] * inv, f[7] * inv));
+            }
+        }
+    }
+    if (CLUSTER && warp < 4) {
+        // (apart from the softmax warps' side: these warps have given their registers up)
+        __syncwarp();
+        tc_fence_before_sync();
+        __syncthreads();
+        cluster_sync();
+        cluster_sync();
     }
 
     // ---- teardown ----
