@@ -152,7 +152,7 @@ int hass_topk_distill_bwd(const void* H_d, const void* W, int64_t N, int64_t d, 
  * steps from the draft sweep on a second time, as conditional launches that return at once unless a
  * violation was detected, in which case they redo the call with each row's exponent taken from that
  * record (no logit of the row can exceed it). The precision is the same either way. The _draft form and
- * the Top-P variant work the same way, and so do hass_combined_distill_fwd_bwd and the Bi-directional
+ * the Top-P variant work the same way, and so do hass_combined_distill_fwd_bwd, where it spills, and the Bi-directional
  * variant, whose exponent comes from the row's largest logit among the first 256 tokens and whose
  * second pass repeats the whole sequence.
  * Calls of at most 128 rows, and of 257 rows and more over at most 2048 tokens (up to 3072 rows with K <= 32 and 1024 tokens, 2048
@@ -187,13 +187,15 @@ int hass_topk_distill_fwd_bwd_draft(const void* H_d, const void* W, int64_t N, i
  *   dH_d         = dz_d W
  *
  * i.e. the gradient of sum_i grad_loss[i] (loss_ce[i] + w loss_topk[i]) with respect to H_d. The
- * sweep spills the target tiles as well, a second GEMM forms q W per row, from which both the
- * cross-entropy, lse_d - <H_d[i], (q W)[i]>, and its gradient term follow; 8 N d V tensor FLOPs
- * are executed. Range condition as for hass_topk_distill_fwd_bwd, for target and draft logits
- * alike; a violation is repaired by a second pass of the same sequence (see there). The other
- * outputs are those of hass_topk_distill_fwd.
- * Workspace: hass_combined_distill_workspace_bytes (the normal workspace plus the target spill and
- * a q W buffer for one chunk of rows).
+ * logits of both feature sets go through the workspace in fp32, in chunks of rows; one kernel forms
+ * the losses and dz_d, rounded to bf16 once, and one product gives dH_d (6 N d V tensor FLOPs). No
+ * range condition and no second pass. Calls of 129 to 256 rows, and those with a smaller workspace,
+ * spill the target tiles as well as the draft's, and a second GEMM forms q W per row, from which both
+ * the cross-entropy, lse_d - <H_d[i], (q W)[i]>, and its gradient term follow (8 N d V); these have the
+ * range condition of hass_topk_distill_fwd_bwd, for target and draft logits alike, and its second pass.
+ * The other outputs are those of hass_topk_distill_fwd.
+ * Workspace: hass_combined_distill_workspace_bytes (the normal workspace, the target spill and a q W
+ * buffer for one chunk of rows, or the fp32 logits of one, at most 1.6 GB, where they are more).
  */
 int hass_combined_distill_workspace_bytes(int64_t N, int64_t d, int64_t V, int32_t K, size_t* bytes);
 int hass_combined_distill_fwd_bwd(const void* H_t, const void* H_d, const void* W, int64_t N, int64_t d,

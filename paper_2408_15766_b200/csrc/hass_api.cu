@@ -413,6 +413,25 @@ static bool narrow_rows(long long N, long long pitch, int K, int chunk_tiles, in
     return N > 2 * BM && N <= most && N <= static_cast<long long>(chunk_tiles) * BM && 2 * ((N + BM - 1) / BM) <= sms;
 }
 
+// Rows per chunk of a combined call whose logits go through the workspace in fp32; 0: it spills. The spilled probabilities of target and draft
+// have references of their own, known before the sums are, so that the gradient takes a product with W for each; from fp32 logits the row
+// kernel forms their difference (rounded once instead of twice) and one product is enough. The sweep stores twice the bytes, which its products
+// hide, and the row kernel reads them twice. Per call: 1024 rows x 4096 x 128256 2980 -> 2610 us, 517 rows 2140 -> 1620, 2048 x 4096 x 32000
+// 1600 -> 1290, 8192 rows 6240 -> 5300, 300 rows 500 -> 285, 1318 x 376 x 38201, K = 65 560 -> 460, 8000 x 704 x 3000, K = 128 1190 -> 590,
+// 640 x 512 x 8000 130 -> 72. Chunks of an eighth of the SM count in row tiles (every CTA pair has its part of the columns), or of a quarter
+// where their logits stay in the L2 (8000 x 256 x 1024 216 -> 184), of 1.6 GB at most: 8192 x 4096 x 32000 takes 5300 us in chunks of 18 or of 37
+// tiles, 1024 x 4096 x 128256 2690 in two of 4 and 2610 in one. (Calls of 129 to 256 rows keep to the spill, as narrow_rows has it.)
+constexpr long long kCombinedBytes = 1600ll << 20, kCombinedL2Bytes = 128ll << 20;
+static int combined_rows(long long N, long long V, int sms) {
+    if (N <= 2 * BM) return 0;
+    const int RT = ceil_div(N, BM);
+    const long long tile = static_cast<long long>(BM) * ceil_div(V, BN) * BN * 8;
+    const long long most = std::max(1, sms / 4) * tile <= kCombinedL2Bytes ? sms / 4 : std::min<long long>(sms / 8, kCombinedBytes / tile);
+    if (most < 4) return 0;
+    const int chunks = ceil_div(RT, most);
+    return ceil_div(RT, chunks) * BM;
+}
+
 // The forward schedule covers 2 * RT row tiles (target then draft).
 static int make_layout(long long N, long long d, long long V, int K, int sms, Layout* L) {
     const int RT = ceil_div(N, BM), CT = ceil_div(V, BN);
@@ -931,10 +950,11 @@ struct NarrowRoom {
     float* dz = nullptr;     // the one of the two that dz_d goes over, which lies first
     PartRoom part;
 };
-static NarrowRoom narrow_room(long long N, int K, uint8_t* ws, size_t workspace_bytes, const Layout& L, int sms) {
+// chunked: N rows of a combined call (combined_rows)
+static NarrowRoom narrow_room(long long N, int K, uint8_t* ws, size_t workspace_bytes, const Layout& L, int sms, bool chunked = false) {
     NarrowRoom r;
     const size_t z = align256(static_cast<size_t>(N) * L.p_pitch * 4);
-    if (narrow_rows(N, L.p_pitch, K, L.pref_chunk_tiles, sms) && workspace_bytes >= L.scratch + 2 * z) {
+    if ((chunked || narrow_rows(N, L.p_pitch, K, L.pref_chunk_tiles, sms)) && workspace_bytes >= L.scratch + 2 * z) {
         float* const a = reinterpret_cast<float*>(ws + L.scratch);
         float* const b = reinterpret_cast<float*>(ws + L.scratch + z);
         const bool split = row_split(N, L.p_pitch, K, sms).blocks != 0;
@@ -947,9 +967,9 @@ static NarrowRoom narrow_room(long long N, int K, uint8_t* ws, size_t workspace_
     return r;
 }
 
-// The logits of N rows of H0 and (nullable) of H1 -> z0, z1 [N, p_pitch]; clears the status block.
+// The logits of N rows of H0 and (nullable) of H1 -> z0, z1 [N, p_pitch]; clears the status block (the first chunk of a call).
 static int narrow_sweep(const void* H0, const void* H1, const void* W, int N, long long d, long long V, float* z0, float* z1,
-                        uint8_t* ws, const Layout& L, const DeviceInfo& di, cudaStream_t st) {
+                        uint8_t* ws, const Layout& L, const DeviceInfo& di, cudaStream_t st, bool first = true) {
     GemmParams p;
     std::memset(&p, 0, sizeof(p));
     // up to 64 rows each share one row tile (61 rows x 4096 x 32000: 65 us as two row tiles of a CTA pair, 61 as one)
@@ -987,7 +1007,7 @@ static int narrow_sweep(const void* H0, const void* H1, const void* W, int N, lo
     p.k_blocks = ceil_div(d, BK);
     p.keep_from = p.k_blocks - static_cast<int>(p.k_blocks * std::min(1., static_cast<double>(kKeepBytes) / (2. * static_cast<double>(V) * static_cast<double>(d))));
     p.status = reinterpret_cast<unsigned int*>(ws + L.status);
-    p.clear_status = 1;
+    p.clear_status = first ? 1 : 0;
     p.release_late = V * d * 2 >= kLateBytes ? 1 : 0;
     return launch_gemm<MODE_LOGITS>(p, st, H1 ? KIND_STATS : KIND_STATS_DRAFT);
 }
@@ -1005,7 +1025,8 @@ template <int OBJ>
 static int launch_rows_as(RowParams& r, int N, int sms, cudaStream_t st) {
     KernelTimer timer(KIND_FINALIZE, st);
     const RowSplit w = row_split(N, r.pitch, r.K, sms);
-    if (w.blocks == 0) return launch(row_kernel<OBJ>, N, ROW_THREADS, 0, st, 1, r);
+    if (w.blocks == 0 && N > sms) return launch(row_kernel<OBJ, ROW_THREADS / 2>, N, ROW_THREADS / 2, 0, st, 1, r);
+    if (w.blocks == 0) return launch(row_kernel<OBJ, ROW_THREADS>, N, ROW_THREADS, 0, st, 1, r);
     r.split = w.blocks;
     void (*fn)(RowParams);
     if (w.blocks == 1)
@@ -1028,10 +1049,10 @@ static int narrow_impl(int objective, bool with_target, const void* H_t, const v
                        long long V, int K, const float* grad_loss, const int* idx_in, const float* q_in, float* loss,
                        int* idx_out, float* q_out, float* lse_t, float* lse_d, void* dH_d, int dH_dtype, uint8_t* ws,
                        const Layout& L, const NarrowRoom& room, const DeviceInfo& di, cudaStream_t st, float top_p, int* topk_n,
-                       const Combined* cmb = nullptr, const float* lse_in = nullptr) {
+                       const Combined* cmb = nullptr, const float* lse_in = nullptr, bool first = true) {
     // (1) the logits of the target and draft rows
-    int rc = with_target ? narrow_sweep(H_t, H_d, W, N, d, V, room.zt, room.z, ws, L, di, st)
-                         : narrow_sweep(H_d, nullptr, W, N, d, V, room.z, nullptr, ws, L, di, st);
+    int rc = with_target ? narrow_sweep(H_t, H_d, W, N, d, V, room.zt, room.z, ws, L, di, st, first)
+                         : narrow_sweep(H_d, nullptr, W, N, d, V, room.z, nullptr, ws, L, di, st, first);
     if (rc != HASS_OK) return rc;
     // (2) statistics, Omega_hat, loss, dz_d
     RowParams r = row_params(static_cast<int>(V), K, L);
@@ -1135,6 +1156,21 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
     __nv_bfloat16* P = reinterpret_cast<__nv_bfloat16*>(ws + L.scratch);
     unsigned int* status = reinterpret_cast<unsigned int*>(ws + L.status);
     int* idx_d = reinterpret_cast<int*>(ws + L.sidx);
+    const long long most = cmb ? std::min<long long>(N, combined_rows(N, V, di.sms)) : 0;
+    if (most > 0 && narrow_room(most, K, ws, cmb->end, L, di.sms, true).z) {
+        const size_t dH_row = static_cast<size_t>(d) * (dH_dtype == HASS_FP32 ? 4 : 2);
+        for (long long r0 = 0; r0 < N; r0 += most) {
+            const int rows = static_cast<int>(std::min(most, N - r0));
+            const NarrowRoom narrow = narrow_room(rows, K, ws, cmb->end, L, di.sms, true);
+            Combined c = *cmb;
+            c.loss_ce += r0;
+            rc = narrow_impl(ROW_COMBINED, true, static_cast<const __nv_bfloat16*>(H_t) + r0 * d, static_cast<const __nv_bfloat16*>(H_d) + r0 * d, W, rows, d, V, K,
+                             grad_loss ? grad_loss + r0 : nullptr, nullptr, nullptr, loss + r0, idx_out + r0 * K, q_out + r0 * K, lse_t + r0, lse_d + r0,
+                             static_cast<uint8_t*>(dH_d) + r0 * dH_row, dH_dtype, ws, L, narrow, di, st, 0.f, nullptr, &c, nullptr, r0 == 0);
+            if (rc != HASS_OK) return rc;
+        }
+        return HASS_OK;
+    }
     // (The combined objective too: 65 rows x 4096 x 32000 254 -> 123 us, 128 rows x 4096 x 128256 675 -> 472, 100 x 256 x 1024 82 -> 37.)
     if (with_target) {
         const NarrowRoom narrow = narrow_room(N, K, ws, cmb ? cmb->end : workspace_bytes, L, di.sms);
@@ -1941,6 +1977,10 @@ static int combined_stage(int64_t N, int64_t d, int64_t V, int32_t K, CombinedSt
     c->Pt = off;
     off = align256(off + L.scratch_row_tile_bytes * L.pref_chunk_tiles);
     c->total = off;
+    // (the fp32 logits of a chunk lie from the scratch on, over all of these)
+    const long long rows = std::min<long long>(N, combined_rows(N, V, sm_count_or_default()));
+    const size_t end = L.scratch + 2 * align256(static_cast<size_t>(rows) * L.p_pitch * 4);
+    if (end > c->total + c->part_bytes) c->part_bytes = end - c->total;
     return HASS_OK;
 }
 

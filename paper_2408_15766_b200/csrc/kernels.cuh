@@ -2172,11 +2172,14 @@ __global__ void __launch_bounds__(256) loss_patch_kernel(const __grid_constant__
 // share again and put them into a pool in shared memory, where each counts those above it (more than it takes: collect_from_many).
 // Bound by the latency of two passes over rows of 4 V bytes in L2: 1024 threads with ROW_LOADS 16-byte loads each in flight.
 // It takes the rows that row_split_kernel does not (row_split in the host code): those of more than 8192 logits, when they are many.
+// Where there are more rows than SMs two blocks of 512 threads share one, so that one row's barriers fall into the other's loads:
+// combined calls of 2048 rows x 32000 260 -> 215 us, 640 x 8000 54 -> 35, 8000 x 3000, K = 128 620 -> 400; 1024 x 128256, where the rows come
+// out of memory and go back (2.4 GB: two readings of both matrices and dz_d, 5.0 TB/s), 474 either way. Four blocks of 256: 257, 33, 455.
 constexpr int ROW_THREADS = 1024;
 constexpr int ROW_LOADS = 4;
 constexpr int ROW_POOL = 1024;
 constexpr int ROW_SLACK = 32;      // maxima beyond K at which the search of the bound ends
-static_assert(ROW_POOL >= K_CAP && ROW_THREADS >= K_CAP, "room for Omega_hat, a thread for each of its tokens");
+static_assert(ROW_POOL >= K_CAP && ROW_THREADS / 2 >= K_CAP, "room for Omega_hat, a thread for each of its tokens");
 enum { ROW_TOPK = 0, ROW_COMBINED = 1, ROW_BIDIR = 2 };
 
 struct RowParams {
@@ -2492,9 +2495,8 @@ __device__ __forceinline__ void select_largest(const float* row, long long pitch
     __syncthreads();
 }
 
-template <int OBJ>
-__global__ void __launch_bounds__(ROW_THREADS) row_kernel(const __grid_constant__ RowParams p) {
-    constexpr int THREADS = ROW_THREADS;
+template <int OBJ, int THREADS>      // THREADS: ROW_THREADS, or half of them
+__global__ void __launch_bounds__(THREADS, ROW_THREADS / THREADS) row_kernel(const __grid_constant__ RowParams p) {
     __shared__ RowShared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int row = blockIdx.x;
