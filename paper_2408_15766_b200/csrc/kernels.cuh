@@ -1534,13 +1534,12 @@ __device__ __forceinline__ void gather_unit(const __nv_bfloat16* W, long long d,
 // groups of threads take FIN_GRP tokens each, with their columns' sums in registers to the end (one group had a warp of eight at work on 256
 // columns: Bi-directional call of 2795 rows x 256 x 1024, K = 41 223 -> 183 us, combined 1318 x 376 x 38201, K = 65 658 -> 621).
 __device__ __forceinline__ void gather_rows(const __nv_bfloat16* from, const __nv_bfloat16* W, int d, int u0, int u1, const int* tok, int b0, int n,
-                                            float* to, const float* q, float gw, float* so, float (&part)[FIN_WARPS][FIN_GRP], float* cols) {
+                                            float* to, const float* q, float gw, float* so, float (&part)[FIN_WARPS][K_CAP], float* cols) {
     constexpr int THREADS = FIN_WARPS * 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int per = max(32, min((u1 - u0 + 31) / 32 * 32, THREADS)), groups = THREADS / per, g = tid / per;
-    // the sums of a group's dot products over its threads
-    auto finish = [&](float (&dot)[FIN_GRP], int b, int each) {
-        // eight sums over the warp at once: at each step half of the values go to the other half of the lanes
+    // eight sums over the warp at once, sum (lane >> 2) in the end: at each step half of the values go to the other half of the lanes
+    auto warp_sums = [&](float (&dot)[FIN_GRP]) {
         static_assert(FIN_GRP == 8, "lane bits 4, 3, 2 say which sum");
 #pragma unroll
         for (int h = 4; h > 0; h >>= 1) {
@@ -1553,6 +1552,45 @@ __device__ __forceinline__ void gather_rows(const __nv_bfloat16* from, const __n
         }
         dot[0] += __shfl_xor_sync(0xffffffffu, dot[0], 2);
         dot[0] += __shfl_xor_sync(0xffffffffu, dot[0], 1);
+    };
+    if (groups == 1 && n - b0 > FIN_GRP) {
+        // a thread's columns in turn, all tokens for each, so that their sum stays in registers; a warp adds its dot products up in its own part of
+        // `part`, and the block meets once. With the tokens in turn and the columns' sum in memory in between, finalize and the selections of
+        // 2048 Bi-directional rows x 4096, K = 10 took 139 us, now 133; 300 x 8192, K = 41 215 -> 205, 2795 x 1040, K = 41 250 -> 226. (The rows of W
+        // come at 4.7 TB/s, from the L2 and from memory; up to FIN_GRP tokens one turn is all there is, below: 1000 x 5120, K = 3 73 us this way, 59 that.)
+        for (int a0 = u0; a0 < u1; a0 += THREADS) {
+            const int at = a0 + tid;
+            const bool mine = at < u1;
+            float h[8] = {}, a[8] = {};
+            if (mine) unpack8(*reinterpret_cast<const uint4*>(from + 8 * at), h);
+            for (int b = b0; b < n; b += FIN_GRP) {
+                float dot[FIN_GRP] = {};
+                if (mine) gather_unit(W + 8 * at, d, tok + b, n - b, h, dot, so ? q + b : nullptr, gw, a);
+                warp_sums(dot);
+                if ((lane & 3) == 0 && b + (lane >> 2) < n) {
+                    float* const sum = &part[warp][b + (lane >> 2)];
+                    *sum = a0 == u0 ? dot[0] : *sum + dot[0];
+                }
+            }
+            if (so && mine) {
+                float4* s4 = reinterpret_cast<float4*>(so + 8 * at);
+                s4[0] = make_float4(a[0], a[1], a[2], a[3]);
+                s4[1] = make_float4(a[4], a[5], a[6], a[7]);
+            }
+        }
+        __syncthreads();
+        for (int j = b0 + tid; j < n; j += THREADS) {
+            float acc = 0.f;
+#pragma unroll
+            for (int w = 0; w < FIN_WARPS; ++w) acc += part[w][j];
+            to[j] = acc;
+        }
+        __syncthreads();
+        return;
+    }
+    // the sums of a group's dot products over its threads
+    auto finish = [&](float (&dot)[FIN_GRP], int b, int each) {
+        warp_sums(dot);
         if ((lane & 3) == 0) part[warp][lane >> 2] = dot[0];
         __syncthreads();
         if (tid < groups * each && b + tid < n) {
@@ -1563,25 +1601,18 @@ __device__ __forceinline__ void gather_rows(const __nv_bfloat16* from, const __n
         __syncthreads();
     };
     if (groups == 1) {
-        for (int b = b0; b < n; b += FIN_GRP) {
-            float dot[FIN_GRP] = {};
-            for (int at = u0 + tid; at < u1; at += THREADS) {
-                float h[8], a[8] = {};
-                unpack8(*reinterpret_cast<const uint4*>(from + 8 * at), h);
+        float dot[FIN_GRP] = {};
+        for (int at = u0 + tid; at < u1; at += THREADS) {
+            float h[8], a[8] = {};
+            unpack8(*reinterpret_cast<const uint4*>(from + 8 * at), h);
+            gather_unit(W + 8 * at, d, tok + b0, n - b0, h, dot, so ? q + b0 : nullptr, gw, a);
+            if (so) {
                 float4* s4 = reinterpret_cast<float4*>(so + 8 * at);
-                if (so && b > 0) {
-                    const float4 a0 = s4[0], a1 = s4[1];
-                    a[0] = a0.x; a[1] = a0.y; a[2] = a0.z; a[3] = a0.w;
-                    a[4] = a1.x; a[5] = a1.y; a[6] = a1.z; a[7] = a1.w;
-                }
-                gather_unit(W + 8 * at, d, tok + b, n - b, h, dot, so ? q + b : nullptr, gw, a);
-                if (so) {
-                    s4[0] = make_float4(a[0], a[1], a[2], a[3]);
-                    s4[1] = make_float4(a[4], a[5], a[6], a[7]);
-                }
+                s4[0] = make_float4(a[0], a[1], a[2], a[3]);
+                s4[1] = make_float4(a[4], a[5], a[6], a[7]);
             }
-            finish(dot, b, FIN_GRP);
         }
+        finish(dot, b0, FIN_GRP);
         return;
     }
     const int u = u0 + tid - g * per;
@@ -1621,7 +1652,7 @@ __global__ void __launch_bounds__(FIN_WARPS * 32, 3) finalize_kernel(const __gri
     __shared__ int sh_tok[K_CAP];         // Omega_hat of the row (the bi-directional set needs 2K <= K_CAP)
     __shared__ float sh_q[K_CAP];
     __shared__ float sh_dot[K_CAP];       // z_d at Omega_hat
-    __shared__ float sh_part[FIN_WARPS][FIN_GRP];
+    __shared__ float sh_part[FIN_WARPS][K_CAP];
     extern __shared__ float sh_cols[];
     __shared__ int sh_n;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;

@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(NORMED_THREADS, 3) normed_kernel(const __grid_
     __shared__ int tok[K_CAP];
     __shared__ float q[K_CAP], z[K_CAP], w[K_CAP];
     __shared__ float parts[NORMED_MAX][K_CAP];      // the blocks' parts of the dot products
-    __shared__ float part[FIN_WARPS][FIN_GRP];
+    __shared__ float part[FIN_WARPS][K_CAP];
     extern __shared__ float sh_cols[];
     wait_previous_kernel();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
