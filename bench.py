@@ -425,7 +425,7 @@ def main():
     ap.add_argument("--K", type=int, default=None)
     ap.add_argument("--objective", default="topk", choices=["topk", "combined", "top_p", "normed", "bidir"],
                     help="topk: Eq. 1 alone (the headline metric); combined: cross-entropy over the vocabulary "
-                         "+ w * Top-K in one call (8 N d V tensor FLOPs); top_p (P = 0.5, at most K tokens) and "
+                         "+ w * Top-K in one call (6 N d V tensor FLOPs; 8 at 129 to 256 rows); top_p (P = 0.5, at most K tokens) and "
                          "normed (Normed Top-K: only the target product, 2 N d V) and bidir (Bi-directional "
                          "Top-K) are the loss variants of Section 4.3")
     ap.add_argument("--route", default="fused", choices=["fused", "split"],
@@ -571,9 +571,10 @@ def main():
         return
 
     # ---- roofline of the dominant kernel (tensor-core bound) ----
-    # three d x V products per token (z_t, z_d, dH_d); the combined objective needs a fourth (q W)
+    # three d x V products per token (z_t, z_d, dH_d); the combined objective spills at 129 to 256 rows and needs a fourth (q W) there
+    fourth = combined and 128 < N <= 256
     normed = args.objective == "normed"
-    flops_credit = (8.0 if combined else 2.0 if normed else 6.0) * N * d * V
+    flops_credit = (8.0 if fourth else 2.0 if normed else 6.0) * N * d * V
     # executed tensor work per step, averaged over the timed steps (a draft-only step skips the target product)
     # the Top-K and Top-P calls sweep the target rows and the draft rows in separate launches (timed as
     # stats_gemm and stats_gemm_draft); the combined and Bi-directional calls sweep both in one launch
@@ -582,7 +583,7 @@ def main():
     kinds = {"stats_gemm": (2.0 * n_full if (normed or two_sweeps) else 4.0 * n_full) / args.steps * N * d * V,
              "stats_gemm_draft": 2.0 * (n_full + n_draft) / args.steps * N * d * V if two_sweeps else 0.0,
              "dz_gemm": 2.0 * N * d * V if split else 0.0,
-             "dH_gemm": (4.0 if combined else 2.0) * N * d * V}
+             "dH_gemm": (4.0 if fourth else 2.0) * N * d * V}
     total_ms = sum(v[0] for v in prof.values())
     kernel_rows = {}
     for k, (ms, cnt) in prof.items():

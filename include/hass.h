@@ -7,7 +7,8 @@
  * tensor memory. What does pass through the workspace, between the forward sweep and the
  * back-projection of the fused call, is a bounded chunk of un-normalised bf16 draft probabilities
  * (chunk rows x V, chunk rows = 128 x the even part of a quarter of the SM count, 4608 on a 148-SM device
- * whatever N is: 1.2 GB for V = 128256); see hass_topk_distill_fwd_bwd.
+ * whatever N is: 1.2 GB for V = 128256); see hass_topk_distill_fwd_bwd. (Calls of few rows, or of a short
+ * vocabulary, and the combined objective pass fp32 logits through it instead, in chunks of 1.6 GB at most.)
  *
  * Notation follows the paper (Section 3.1): q = softmax(H_t W^T) is the target LLM's
  * next-token distribution, p = softmax(H_d W^T) the draft model's, Omega the vocabulary
@@ -70,8 +71,8 @@ int hass_version(void);
  * bounded scratch areas for one chunk of rows (a fixed number of 128-row tiles that does not grow
  * with N): the bf16 un-normalised draft probabilities (fused call) or dz_d (split backward),
  * chunk_rows x V, and the fp32 Omega_hat term of dH_d, chunk_rows x d; and, behind them, fp32 partial
- * tiles of dH_d (less than one 128-row tile of scratch). Calls of at most 128 rows, and of 257 to some thousand rows over at
- * most 2048 tokens, keep their logits in fp32 instead, two matrices of N x V. A smaller workspace is accepted down to room
+ * tiles of dH_d (less than one 128-row tile of scratch). Calls of at most 128 rows, and of 257 rows and more where
+ * hass_topk_distill_fwd_bwd says so, keep their logits in fp32 instead, two matrices of N x V. A smaller workspace is accepted down to room
  * for one 128-row tile of scratch; the calls then work in smaller chunks, and may do without partial tiles and fp32 logits.
  * Needs no GPU (assumes 148 SMs if none is present).
  */
