@@ -2198,14 +2198,14 @@ __global__ void __launch_bounds__(256) loss_patch_kernel(const __grid_constant__
 // sum_v q(v) (lse_d - z_d(v)). ROW_BIDIR: the draft's K most probable tokens join Omega_hat; the row becomes p(v) alone, and
 // g S_q and the row sum_x g q(x) W[x, :] over Omega_hat are left in fp32 for the epilogue of the second GEMM.
 //
-// The K largest of a row: a thread's largest logit is at hand after the pass for lse, and the K-th largest of these 1024
-// maxima bounds the row's K-th largest from below. Little more than K logits reach it; the threads that hold them read their
-// share again and put them into a pool in shared memory, where each counts those above it (more than it takes: collect_from_many).
+// The K largest of a row: a thread's largest logit is at hand after the pass for lse, and the K-th largest of these
+// maxima bounds the row's K-th largest from below. Little more than K logits reach it; warps read the shares of the threads that hold
+// them again and put them into a pool in shared memory, where each counts those above it (more than it takes: collect_from_many).
 // Bound by the latency of two passes over rows of 4 V bytes in L2: 1024 threads with ROW_LOADS 16-byte loads each in flight.
 // It takes the rows that row_split_kernel does not (row_split in the host code): those of more than 8192 logits, when they are many.
 // Where there are more rows than SMs two blocks of 512 threads share one, so that one row's barriers fall into the other's loads:
 // combined calls of 2048 rows x 32000 260 -> 215 us, 640 x 8000 54 -> 35, 8000 x 3000, K = 128 620 -> 400; 1024 x 128256, where the rows come
-// out of memory and go back (2.4 GB: two readings of both matrices and dz_d, 5.0 TB/s), 474 either way. Four blocks of 256: 257, 33, 455.
+// out of memory and go back (2.4 GB: two readings of both matrices and dz_d, 5.4 TB/s in the 437 us it takes now), 474 either way then. Four blocks of 256: 257, 33, 455.
 constexpr int ROW_THREADS = 1024;
 constexpr int ROW_LOADS = 4;
 constexpr int ROW_POOL = 1024;
@@ -2256,10 +2256,11 @@ struct RowPool {           // of a block that looks for the K largest logits of 
     unsigned long long pool[ROW_POOL];
     float red[4][32];
     uint32_t key_min[32];
-    int n;
+    int n, holders;
     int reach[3], equal[32];
 };
 struct RowShared : RowPool {
+    unsigned short holder[ROW_THREADS];      // threads whose largest logit reaches the bound
     int tok[K_CAP];        // Omega_hat
     float q[K_CAP], z[K_CAP];
     int tok_d[K_CAP];      // the draft's own K largest (ROW_BIDIR)
@@ -2365,6 +2366,34 @@ __device__ __forceinline__ void collect(const float* row, long long pitch, int V
                     if (pos < room) sh.pool[pos] = logit_rank(z[j], static_cast<uint32_t>(first + at + j));
                 }
         }, [&] { return !full(); });
+    __syncthreads();
+}
+
+// The same, where few threads hold such logits as a rule: a warp reads the share of one of them at a time, a piece per lane. (Read by their own
+// threads, hardly a warp was without one, and went over the row once more with a lane or two at work: the row kernel of 1024 x 128256, combined, 479 ->
+// 437 us, 517 rows 246 -> 226, 100 x 128256, K = 20 51 -> 45.6, 61 x 32000 18.9 -> 18.2.)
+template <int THREADS>
+__device__ __forceinline__ void collect_from_holders(const float* row, long long pitch, int V, uint32_t key, uint32_t bound, int room, RowPool& sh,
+                                                     unsigned short* holder) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (key >= bound) holder[atomicAdd(&sh.holders, 1)] = static_cast<unsigned short>(threadIdx.x);
+    __syncthreads();
+    const int n = sh.holders, pieces = static_cast<int>((pitch + THREADS * 4 - 1) / (THREADS * 4));
+    for (int h = warp; h < n && *static_cast<volatile int*>(&sh.n) <= room; h += THREADS / 32) {
+        const int own = holder[h] * 4;
+        for (int u = lane; u < pieces; u += 32) {
+            const long long at = static_cast<long long>(u) * (THREADS * 4) + own;
+            if (at >= pitch) continue;
+            const float4 v = *reinterpret_cast<const float4*>(row + at);
+            const float z[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (reaches(z[j], at + j, V, bound)) {
+                    const int pos = atomicAdd(&sh.n, 1);
+                    if (pos < room) sh.pool[pos] = logit_rank(z[j], static_cast<uint32_t>(at + j));
+                }
+        }
+    }
     __syncthreads();
 }
 
@@ -2479,7 +2508,7 @@ __device__ __forceinline__ uint32_t bound_from_maxima(int K, float m, RowPool& s
         sh.red[0][warp] = __uint_as_float(key_hi);
         sh.key_min[warp] = key_lo;
     }
-    if (threadIdx.x == 0) sh.n = 0;
+    if (threadIdx.x == 0) sh.n = sh.holders = 0;
     const int groups = __syncthreads_count(key != 0u);
     hi = __reduce_max_sync(0xffffffffu, lane < THREADS / 32 ? __float_as_uint(sh.red[0][lane]) : 0u);
     if (groups < K) return 1u;
@@ -2502,11 +2531,11 @@ __device__ __forceinline__ uint32_t bound_from_maxima(int K, float m, RowPool& s
 // Block-collective: the K largest logits of the row, in descending order (lower token id first among equal ones), into
 // tok / val; m = this thread's largest logit. Fewer than K logits above -inf: the rest is token 0 at -inf.
 template <int THREADS>
-__device__ __forceinline__ void select_largest(const float* row, long long pitch, int V, int K, float m, RowPool& sh, int* tok, float* val) {
+__device__ __forceinline__ void select_largest(const float* row, long long pitch, int V, int K, float m, RowShared& sh, int* tok, float* val) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint32_t key, hi;
     const uint32_t T = bound_from_maxima<THREADS>(K, m, sh, key, hi);
-    collect<THREADS>(row, pitch, V, 0, key, T, pool_room(K), sh);
+    collect_from_holders<THREADS>(row, pitch, V, key, T, pool_room(K), sh, sh.holder);
     int n = sh.n;
     if (n > pool_room(K)) n = collect_from_many<THREADS>(row, pitch, V, 0, K, key, T, hi, sh);
     for (int j = n + tid; j < K; j += THREADS) {
@@ -2667,11 +2696,12 @@ __global__ void __launch_bounds__(THREADS, ROW_THREADS / THREADS) row_kernel(con
                 if (OBJ == ROW_COMBINED) {
                     const float4& tu = t[OBJ == ROW_COMBINED ? u : 0];
                     const float zt[4] = {tu.x, tu.y, tu.z, tu.w};
+                    const bool whole = at + 4 <= p.V;
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         const float qv = ex2(fmaf(zt[j], LOG2E, shift_t));
                         o[j] = fmaf(-g, qv, o[j]);
-                        if (at + j < p.V) ce = fmaf(qv, lse_d - z[j], ce);      // (-inf beyond the vocabulary)
+                        if (whole || at + j < p.V) ce = fmaf(qv, lse_d - z[j], ce);      // (-inf beyond the vocabulary)
                     }
                 }
                 *reinterpret_cast<uint2*>(drow + at) = make_uint2(pack_bf16x2(o[0], o[1]), pack_bf16x2(o[2], o[3]));

@@ -11,9 +11,10 @@ pytestmark = pytest.mark.gpu
 
 
 # The first row of the route; one chunk, and one row more (two of ten and nine tiles, one row in the last); the largest vocabulary whose chunks
-# stay in the L2 (4736 rows on 148 SMs) and one chunk of it and a row; rows of a block's first step and of one logit more; all tokens; K = 256
+# stay in the L2 (4736 rows on 148 SMs) and one chunk of it and a row; rows of a block's first step and of one logit more; all tokens; K = 256; rows of
+# which a thread of the row kernel has more pieces than a warp has lanes (512 and 1024 threads)
 @pytest.mark.parametrize("N,d,V,K", [(257, 64, 9000, 10), (2304, 16, 4097, 3), (2305, 16, 4097, 3), (4737, 8, 3300, 2), (300, 72, 8192, 100),
-                                     (300, 64, 8193, 256), (333, 64, 200, 200)])
+                                     (300, 64, 8193, 256), (333, 64, 200, 200), (300, 8, 66000, 5), (3, 8, 140000, 7)])
 def test_combined_chunks_against_the_oracle(N, d, V, K):
     import paper_2408_15766_b200 as hass
     dev = torch.device("cuda:0")
@@ -33,7 +34,7 @@ def test_combined_chunks_against_the_oracle(N, d, V, K):
     # every entry of dz_d is rounded to bf16 once (2^-9 of it), of which the product keeps the size at most
     scale = np.abs(ref["dH_d"]).max()
     assert np.abs(cpu["dH_d"].numpy().astype(np.float64) - ref["dH_d"]).max() <= 2.0 ** -8 * scale
-    if N > 1000:
+    if N > 1000 or N < 128:
         return
     # a workspace without that room takes the spill, whose entries are rounded once for q and once for p
     small = torch.empty(hass.combined_distill_workspace_bytes(N, d, V, K) - 256, dtype=torch.uint8, device=dev)
