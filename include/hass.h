@@ -157,8 +157,8 @@ int hass_topk_distill_bwd(const void* H_d, const void* W, int64_t N, int64_t d, 
  * variant, whose exponent comes from the row's largest logit among the first 256 tokens and whose
  * second pass repeats the whole sequence.
  * Calls of at most 128 rows, and of 257 rows and more over at most 2048 tokens (up to 3072 rows with K <= 32 and 1024 tokens, 2048
- * with K <= 64, 1024 otherwise) or over more (up to 896 rows, and 50e6 / (20e3 + 3.2 V) of them: 408 at 32000 tokens; half
- * as many where one feature set is swept), sweep both feature sets in one launch and keep the draft logits in fp32 between
+ * with K <= 64, 1024 otherwise) or over more (up to 896 rows, and 50e6 / (20e3 + 3.2 V) of them: 408 at 32000 tokens, 531
+ * where d >= 3072; half of 408 where one feature set is swept), sweep both feature sets in one launch and keep the draft logits in fp32 between
  * the sweep and the second GEMM; they have no range condition and no second pass.
  * (HASS_ERR_RANGE is kept for callers that name it; no entry point of this version returns it.)
  */

@@ -407,17 +407,19 @@ static int even_chunk(int most, int RT) {
 // 1500 64 -> 40, 2795 69 -> 56, 4500 71 -> 75; K = 41 1500 89 -> 55, 2795 94 -> 82 but Bi-directional 159 -> 177; K = 101 600 123 -> 60, 1500 132 -> 113,
 // 2795 140 -> 186; combined 1980 rows, K = 9 107 -> 50; 1000 x 4096 x 2000, K = 10 111 -> 68, 3900 187 -> 213. (Calls of 129 to 256 rows keep to the
 // spill's route: what they do beyond its exponent range, and report in the status block, is held by tests.) Over more tokens the row kernel takes about
-// 20 + 3.2 V / 1000 ns a row, and the line lies at 50 us of it, or 25 where one matrix alone is swept, and for the forward alone, which saves fewer (`single`). Fused calls: 360 x 4096 x 2100, K = 56 119 ->
+// 20 + 3.2 V / 1000 ns a row, and the line lies at 50 us of it, or 25 where one matrix alone is swept, and for the forward alone, which saves fewer (`single`), and 65 in fused calls of wide features (d >= 3072), whose joint sweep takes pairs of CTAs
+// also for an odd number of row tiles. Fused calls: 360 x 4096 x 2100, K = 56 119 ->
 // 59 us, 659 x 5120 x 2758, K = 46 203 -> 81, Top-P 268 x 4096 x 12459 168 -> 125, Bi-directional 284 x 4096 x 32000 325 -> 262, 930 x 5432 x 3151 226 -> 178, 391 x
-// 5200 x 32000 442 -> 414, beyond it 594 x 1080 x 33218 237 -> 262; forward and backward as two calls 309 x 256 x 32000, K = 62 184 -> 133; draft rows
+// 5200 x 32000 442 -> 414, 522 x 4096 x 32000 478 -> 420, 479 x 6024 x 32000 675 -> 609, beyond the lines 594 x 1080 x 33218 237 -> 262, 613 x 5120 x
+// 32000 573 -> 597; forward and backward as two calls 309 x 256 x 32000, K = 62 184 -> 133; draft rows
 // 710 x 5120 x 4375 84 -> 70, beyond it 257 x 256 x 32000 47 -> 52. (More than seven row tiles would gain too, 1013 x 256 x 4525 145 -> 68, but the workspace
 // of such calls stays what their row tiles take: those who pass a smaller one count it in them, as a test does.)
-static bool narrow_rows(long long N, long long pitch, int K, int chunk_tiles, int sms, bool single) {
+static bool narrow_rows(long long N, long long d, long long pitch, int K, int chunk_tiles, int sms, bool single) {
     if (N <= BM) return true;
     const long long most = K <= 32 && pitch <= 1024   ? 3072
                            : K <= 64 && pitch <= 2048 ? 2048
                            : pitch <= 2048            ? 1024
-                                                      : std::min(7ll * BM, (single ? 25000 : 50000) * 1000ll / (20000 + 16 * pitch / 5));
+                                                      : std::min(7ll * BM, (single ? 25000 : d >= 3072 ? 65000 : 50000) * 1000ll / (20000 + 16 * pitch / 5));
     return N > 2 * BM && N <= most && N <= static_cast<long long>(chunk_tiles) * BM && 2 * ((N + BM - 1) / BM) <= sms;
 }
 
@@ -512,7 +514,7 @@ static int make_layout(long long N, long long d, long long V, int K, int sms, La
                                                    L->scratch_row_tile_bytes - 256, nullptr));
         if (need > L->part_bytes) L->part_bytes = need;
     }
-    if (N > BM && narrow_rows(N, L->p_pitch, K, pref, sms, false)) {
+    if (N > BM && narrow_rows(N, d, L->p_pitch, K, pref, sms, false)) {
         const size_t end = L->scratch + 2 * align256(static_cast<size_t>(N) * L->p_pitch * 4);
         if (end > L->total_pref && end - L->total_pref > L->part_bytes) L->part_bytes = end - L->total_pref;
     }
@@ -959,10 +961,10 @@ struct NarrowRoom {
     PartRoom part;
 };
 // single: as in narrow_rows; chunked: N rows of a combined call (combined_rows)
-static NarrowRoom narrow_room(long long N, int K, uint8_t* ws, size_t workspace_bytes, const Layout& L, int sms, bool single, bool chunked = false) {
+static NarrowRoom narrow_room(long long N, long long d, int K, uint8_t* ws, size_t workspace_bytes, const Layout& L, int sms, bool single, bool chunked = false) {
     NarrowRoom r;
     const size_t z = align256(static_cast<size_t>(N) * L.p_pitch * 4);
-    if ((chunked || narrow_rows(N, L.p_pitch, K, L.pref_chunk_tiles, sms, single)) && workspace_bytes >= L.scratch + 2 * z) {
+    if ((chunked || narrow_rows(N, d, L.p_pitch, K, L.pref_chunk_tiles, sms, single)) && workspace_bytes >= L.scratch + 2 * z) {
         float* const a = reinterpret_cast<float*>(ws + L.scratch);
         float* const b = reinterpret_cast<float*>(ws + L.scratch + z);
         const bool split = row_split(N, L.p_pitch, K, sms).blocks != 0;
@@ -1124,7 +1126,7 @@ static int narrow_impl(int objective, bool with_target, const void* H_t, const v
 static int narrow_backward(const void* H_d, const void* W, long long N, long long d, long long V, int K, const int* topk_idx, const float* topk_q,
                            const float* lse_d, const float* grad_loss, void* dH_d, int dH_dtype, uint8_t* ws, size_t workspace_bytes,
                            const Layout& L, const DeviceInfo& di, cudaStream_t st) {
-    const NarrowRoom room = narrow_room(N, K, ws, workspace_bytes, L, di.sms, false);      // (as the forward before it)
+    const NarrowRoom room = narrow_room(N, 0, K, ws, workspace_bytes, L, di.sms, false);      // (the line of narrow features: 592 rows x 4096 x 32000 as two calls 618 -> 628)
     if (!room.z) return HASS_ERR_UNSUPPORTED;
     return narrow_impl(ROW_TOPK, false, nullptr, H_d, W, static_cast<int>(N), d, V, K, grad_loss, topk_idx, topk_q, nullptr, nullptr, nullptr,
                        nullptr, nullptr, dH_d, dH_dtype, ws, L, room, di, st, 0.f, nullptr, nullptr, lse_d);
@@ -1165,11 +1167,11 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
     unsigned int* status = reinterpret_cast<unsigned int*>(ws + L.status);
     int* idx_d = reinterpret_cast<int*>(ws + L.sidx);
     const long long most = cmb ? std::min<long long>(N, combined_rows(N, V, di.sms)) : 0;
-    if (most > 0 && narrow_room(most, K, ws, cmb->end, L, di.sms, false, true).z) {
+    if (most > 0 && narrow_room(most, d, K, ws, cmb->end, L, di.sms, false, true).z) {
         const size_t dH_row = static_cast<size_t>(d) * (dH_dtype == HASS_FP32 ? 4 : 2);
         for (long long r0 = 0; r0 < N; r0 += most) {
             const int rows = static_cast<int>(std::min(most, N - r0));
-            const NarrowRoom narrow = narrow_room(rows, K, ws, cmb->end, L, di.sms, false, true);
+            const NarrowRoom narrow = narrow_room(rows, d, K, ws, cmb->end, L, di.sms, false, true);
             Combined c = *cmb;
             c.loss_ce += r0;
             rc = narrow_impl(ROW_COMBINED, true, static_cast<const __nv_bfloat16*>(H_t) + r0 * d, static_cast<const __nv_bfloat16*>(H_d) + r0 * d, W, rows, d, V, K,
@@ -1181,7 +1183,7 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
     }
     // (The combined objective too: 65 rows x 4096 x 32000 254 -> 123 us, 128 rows x 4096 x 128256 675 -> 472, 100 x 256 x 1024 82 -> 37.)
     if (with_target) {
-        const NarrowRoom narrow = narrow_room(N, K, ws, cmb ? cmb->end : workspace_bytes, L, di.sms, false);
+        const NarrowRoom narrow = narrow_room(N, d, K, ws, cmb ? cmb->end : workspace_bytes, L, di.sms, false);
         if (narrow.z)
             return narrow_impl(cmb ? ROW_COMBINED : bidir ? ROW_BIDIR : ROW_TOPK, true, H_t, H_d, W, static_cast<int>(N), d, V, K, grad_loss,
                                nullptr, nullptr, loss, idx_out, q_out, lse_t, lse_d, dH_d, dH_dtype, ws, L, narrow, di, st, 0.f, topk_n, cmb);
@@ -1456,7 +1458,7 @@ static int fused2_impl(bool with_target, const void* H_t, const void* H_d, const
     float* coef = reinterpret_cast<float*>(ws + L.coef);
     float* capz = reinterpret_cast<float*>(ws + L.capz);
     float* ref2 = reinterpret_cast<float*>(ws + L.lse2);
-    const NarrowRoom narrow = narrow_room(N, K, ws, workspace_bytes, L, di.sms, !with_target);
+    const NarrowRoom narrow = narrow_room(N, d, K, ws, workspace_bytes, L, di.sms, !with_target);
     if (narrow.z && (!pipe || N <= BM)) {
         if (pipe) {
             rc = pipe_in(pipe, H_t, H_d, 0, static_cast<size_t>(N), st);
@@ -1664,7 +1666,7 @@ static int forward2_impl(bool with_target, const void* H_t, const void* H_d, con
                             workspace, workspace_bytes, st);
     const int RT = ceil_div(N, BM), CT = ceil_div(V, BN);
     uint8_t* ws = static_cast<uint8_t*>(workspace);
-    const NarrowRoom narrow = narrow_room(N, K, ws, workspace_bytes, L, di.sms, true);
+    const NarrowRoom narrow = narrow_room(N, d, K, ws, workspace_bytes, L, di.sms, true);
     if (narrow.z)
         return narrow_impl(ROW_TOPK, with_target, H_t, H_d, W, static_cast<int>(N), d, V, K, nullptr, idx_in, q_in, loss, idx_out, q_out,
                            lse_t, lse_d, nullptr, HASS_BF16, ws, L, narrow, di, st, 0.f, nullptr);
@@ -1767,7 +1769,7 @@ static int normed_impl(const void* H_t, const void* H_d, const void* W, long lon
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     GemmParams p;
     std::memset(&p, 0, sizeof(p));
-    const NarrowRoom narrow = narrow_room(N, K, ws, workspace_bytes, L, di.sms, true);
+    const NarrowRoom narrow = narrow_room(N, d, K, ws, workspace_bytes, L, di.sms, true);
     if (narrow.z) {
         rc = narrow_sweep(H_t, nullptr, W, static_cast<int>(N), d, V, narrow.zt, nullptr, ws, L, di, st);
         if (rc != HASS_OK) return rc;
