@@ -72,6 +72,7 @@ __global__ void __launch_bounds__(NORMED_THREADS, 3) normed_kernel(const __grid_
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int C = p.split, K = p.K;
     const int row = blockIdx.x / C, rank = blockIdx.x - row * C;      // (clusters are consecutive blocks)
+    if (C > 1) cluster_arrive();
     for (int j = tid; j < K; j += NORMED_THREADS) {
         const int t = p.idx[static_cast<long long>(row) * K + j];
         tok[j] = t < 0 ? 0 : t;
@@ -86,6 +87,7 @@ __global__ void __launch_bounds__(NORMED_THREADS, 3) normed_kernel(const __grid_
     const int units = p.d / 8;
     gather_rows(p.H_d + static_cast<long long>(row) * p.d, p.W, p.d, units * rank / C, units * (rank + 1) / C, tok, 0, K, z, nullptr, 0.f, nullptr, part, sh_cols);
     if (C > 1) {
+        cluster_wait();      // all blocks of the row run: their shared memory may be written
         for (int e = tid; e < C * K; e += NORMED_THREADS) {
             const int c = e / K, j = e - c * K;
             st_cluster_f32(map_to_rank(smem_u32(&parts[rank][j]), c), z[j]);
