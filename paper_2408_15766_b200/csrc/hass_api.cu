@@ -653,7 +653,7 @@ static SelectParams select_params(const GemmParams& p, int first_tile, int row_b
 
 static int launch_finalize(const FinalizeParams& f, cudaStream_t st) {
     KernelTimer timer(f.gate ? KIND_CONDITIONAL : KIND_FINALIZE, st);
-    return launch(finalize_kernel, f.rows, FIN_WARPS * 32, gather_smem(f.d), st, 1, f);
+    return launch(finalize_kernel, f.rows, FIN_WARPS * 32, gather_smem(f.d / 8), st, 1, f);
 }
 
 // Partial tiles' room of a call: behind the scratch of its row chunks, where the caller says, or (routes without an
@@ -1826,11 +1826,9 @@ static int normed_impl(const void* H_t, const void* H_d, const void* W, long lon
     f.loss = loss;
     f.dH = dH_d;
     f.dH_fp32 = dH_dtype == HASS_FP32 ? 1 : 0;
-    // as many blocks per row as are resident at once, of 256 columns at least, 2048 where there is one group of tokens to gather
-    f.split = 1;
-    while (f.split < NORMED_MAX && 2 * f.split * N <= 3ll * di.sms && d >= (K > FIN_GRP ? 512ll : 4096ll) * f.split) f.split *= 2;
+    f.split = normed_split(N, d, K, di.sms);
     KernelTimer timer(KIND_FINALIZE, st);
-    return launch(normed_kernel, N * f.split, NORMED_THREADS, gather_smem(ceil_div(d / 8, f.split) * 8), st, f.split, f);
+    return launch(normed_kernel, N * f.split, NORMED_THREADS, normed_smem(d, f.split), st, f.split, f);
 }
 
 }  // namespace hass

@@ -1503,9 +1503,16 @@ __device__ __forceinline__ void unpack8(const uint4& v, float (&f)[8]) {
     }
 }
 
-// Dynamic shared memory of a kernel that gathers parts of `cols` columns: the groups' sums, where there are groups (with wide rows the
-// space is left to the L1)
-__host__ __device__ constexpr int gather_smem(int cols) { return cols <= FIN_WARPS * 32 * 4 ? 8 * FIN_WARPS * 32 * 4 : 0; }
+// Groups of a block's threads that take tokens of their own in a gather, where its part of the columns is `units` units of eight: as many as have a
+// warp or more per eight columns; 1: all threads share the columns
+__host__ __device__ constexpr int gather_groups(int units, int threads) {
+    const int warps = (units + 31) / 32;
+    return threads / 32 / (warps < 1 ? 1 : warps > threads / 32 ? threads / 32 : warps);
+}
+
+// Dynamic shared memory of a kernel whose blocks gather `units` units of eight columns each, or more: the groups' sums, where any block has
+// groups (with wide rows the space is left to the L1)
+__host__ __device__ constexpr int gather_smem(int units) { return gather_groups(units, FIN_WARPS * 32) > 1 ? 8 * FIN_WARPS * 32 * 4 : 0; }
 
 // Eight columns of the rows of W of tokens tok[0 .. n), n <= FIN_GRP: dot[j] += <h, row j>, a += gw q[j] row j (q nullable).
 __device__ __forceinline__ void gather_unit(const __nv_bfloat16* W, long long d, const int* tok, int n, const float (&h)[8], float (&dot)[FIN_GRP],
@@ -1537,7 +1544,7 @@ __device__ __forceinline__ void gather_rows(const __nv_bfloat16* from, const __n
                                             float* to, const float* q, float gw, float* so, float (&part)[FIN_WARPS][K_CAP], float* cols) {
     constexpr int THREADS = FIN_WARPS * 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int per = max(32, min((u1 - u0 + 31) / 32 * 32, THREADS)), groups = THREADS / per, g = tid / per;
+    const int per = max(32, min((u1 - u0 + 31) / 32 * 32, THREADS)), groups = gather_groups(u1 - u0, THREADS), g = tid / per;
     // eight sums over the warp at once, sum (lane >> 2) in the end: at each step half of the values go to the other half of the lanes
     auto warp_sums = [&](float (&dot)[FIN_GRP]) {
         static_assert(FIN_GRP == 8, "lane bits 4, 3, 2 say which sum");

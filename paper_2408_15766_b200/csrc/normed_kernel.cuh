@@ -5,14 +5,17 @@
 
 namespace hass {
 
+// The first of `units` units that is the rank-th of C blocks', which share them: a block has units / C of them, or one more
+__host__ __device__ constexpr int part_begin(int units, int rank, int C) { return static_cast<int>(static_cast<long long>(units) * rank / C); }
+
 // Block-collective: this block's part of the columns of sum_j w[j] W[tok[j], :], j < n, handed to out(first column, eight sums), where C
 // blocks share the columns and this is the rank-th. Where the part is narrow, groups of threads take every so many-th token each, and their
 // sums are added up in order (part: 8 THREADS floats of shared memory).
 template <int THREADS, typename F>
 __device__ __forceinline__ void sum_rows(const __nv_bfloat16* W, int d, const int* tok, const float* w, int n, int rank, int C, float* part, F&& out) {
     const int tid = threadIdx.x, units = d / 8;
-    const int u0 = static_cast<int>(static_cast<long long>(units) * rank / C), u1 = static_cast<int>(static_cast<long long>(units) * (rank + 1) / C);
-    const int per = max(32, min((u1 - u0 + 31) / 32 * 32, THREADS)), groups = THREADS / per, g = tid / per;
+    const int u0 = part_begin(units, rank, C), u1 = part_begin(units, rank + 1, C);
+    const int per = max(32, min((u1 - u0 + 31) / 32 * 32, THREADS)), groups = gather_groups(u1 - u0, THREADS), g = tid / per;
     for (int b = u0; b < u1; b += THREADS) {
         const int u = b + tid - g * per;
         float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -42,6 +45,16 @@ __device__ __forceinline__ void sum_rows(const __nv_bfloat16* W, int d, const in
 
 constexpr int NORMED_THREADS = FIN_WARPS * 32;
 constexpr int NORMED_MAX = 8;      // blocks per row, at most (the portable cluster size)
+
+// Blocks per row: as many as are resident at once, of 256 columns at least, 2048 where there is one group of tokens to gather
+inline int normed_split(long long N, long long d, int K, int sms) {
+    int split = 1;
+    while (split < NORMED_MAX && 2 * split * N <= 3ll * sms && d >= (K > FIN_GRP ? 512ll : 4096ll) * split) split *= 2;
+    return split;
+}
+// Their dynamic shared memory, the same for all: what the narrowest part needs (of 257 units in two parts the one of 128 has groups, the one of 129
+// has none)
+inline int normed_smem(long long d, int split) { return gather_smem(static_cast<int>(d / 8 / split)); }
 
 struct NormedParams {
     int d, K;
@@ -85,7 +98,7 @@ __global__ void __launch_bounds__(NORMED_THREADS, 3) normed_kernel(const __grid_
         return v;
     };
     const int units = p.d / 8;
-    gather_rows(p.H_d + static_cast<long long>(row) * p.d, p.W, p.d, units * rank / C, units * (rank + 1) / C, tok, 0, K, z, nullptr, 0.f, nullptr, part, sh_cols);
+    gather_rows(p.H_d + static_cast<long long>(row) * p.d, p.W, p.d, part_begin(units, rank, C), part_begin(units, rank + 1, C), tok, 0, K, z, nullptr, 0.f, nullptr, part, sh_cols);
     if (C > 1) {
         cluster_wait();      // all blocks of the row run: their shared memory may be written
         for (int e = tid; e < C * K; e += NORMED_THREADS) {

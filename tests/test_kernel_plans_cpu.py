@@ -1,0 +1,46 @@
+"""Host-side rules that kernels rely on, from the headers that hold them: compiled into a small host program."""
+import os
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2408_15766_b200", "csrc")
+
+
+def run_host_program(tmp_path, header: str, body: str) -> str:
+    src = tmp_path / "plan.cu"
+    src.write_text(f'#include "{os.path.join(CSRC, header)}"\n#include <cstdio>\nusing namespace hass;\n{body}')
+    exe = str(tmp_path / "plan")
+    subprocess.run([os.environ.get("NVCC", "nvcc"), "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-o", exe, str(src)],
+                   check=True)
+    return subprocess.run([exe], capture_output=True, text=True).stdout
+
+
+def test_blocks_that_add_up_groups_have_the_room_for_it(tmp_path):
+    """A Normed Top-K block whose part of the columns leaves threads for several groups of tokens adds the groups' sums up in dynamic shared
+    memory: for every part of every split the launch must have allocated it."""
+    out = run_host_program(tmp_path, "normed_kernel.cuh", r"""
+int main() {
+    long long groups = 0, none = 0;
+    for (int sms : {132, 148, 160})
+        for (int d = 8; d <= 16384; d += 8)
+            for (int K : {FIN_GRP, FIN_GRP + 1})
+                for (int N = 1; N <= 260; ++N) {
+                    const int split = normed_split(N, d, K, sms), bytes = normed_smem(d, split);
+                    for (int rank = 0; rank < split; ++rank) {
+                        const int units = part_begin(d / 8, rank + 1, split) - part_begin(d / 8, rank, split);
+                        // as the kernel deals its threads out: `per` of them to a group
+                        const int want = (units + 31) / 32 * 32, per = want < 32 ? 32 : want > NORMED_THREADS ? NORMED_THREADS : want;
+                        if (NORMED_THREADS / per != gather_groups(units, NORMED_THREADS)) return std::printf("groups %d\n", units), 1;
+                        if (NORMED_THREADS / per > 1) {
+                            ++groups;
+                            if (bytes < 8 * NORMED_THREADS * 4) return std::printf("room N %d d %d K %d split %d rank %d\n", N, d, K, split, rank), 1;
+                        } else {
+                            ++none;
+                        }
+                    }
+                }
+    std::printf("ok %d\n", groups > 0 && none > 0);
+}
+""")
+    assert out == "ok 1\n", out
