@@ -51,6 +51,17 @@ constexpr int SMEM_BYTES = OPERAND_BYTES + 4 * SPILL_STAGES * SPILL_STAGE_BYTES 
 __host__ __device__ constexpr int operand_bytes(int CG, int EW) { return stages(CG, EW) * (A_STAGE_BYTES + b_stage_bytes(CG)); }
 __host__ __device__ constexpr int gemm_smem(int CG, int EW) { return operand_bytes(CG, EW) + EW * SPILL_STAGES * SPILL_STAGE_BYTES + 1024 + 256; }
 static_assert(gemm_smem(1, 4) == SMEM_BYTES && gemm_smem(2, 4) == SMEM_BYTES && gemm_smem(2, 8) <= SMEM_BYTES && gemm_smem(1, 8) <= SMEM_BYTES, "shared memory of a CTA");
+// Staging buffers of an epilogue warp (half: of eight warps, which columns of a tile it takes; quad: which rows) and a thread's column of the pending
+// logits, in bytes of the staging area
+__host__ __device__ constexpr int stage_at(int half, int quad) { return (4 * half + quad) * SPILL_STAGES * SPILL_STAGE_BYTES; }
+__host__ __device__ constexpr int pending_at(int thread) { return (thread - 64) * 4; }
+// Eight epilogue warps: where the second thread of a row (128 threads behind the first) leaves word e of its statistics and its list for the first.
+// With a register list (`list`) that is the first thread's column of the pending logits; without one (two words) the first staging buffer of the
+// first thread's warp. Either way the next tile's values go there from the threads that read the words, not from another warp's.
+__host__ __device__ constexpr int meet_word(bool list, int thread, int e) {
+    const int first = 64 + (thread - 64) % 128;
+    return list ? pending_at(first) + e * 256 * 4 : stage_at(0, first / 32 % 4) + e * 128 + first % 32 * 4;
+}
 constexpr float LOG2E = 1.4426950408889634f;
 // A lane's sum of a spilling row's values 2^(z log2e - ref2), ref2 = z_ref log2e + 64, from which on the call is done again
 // with the row's largest logit as z_ref: a logit 90 above z_ref (natural units). The sum leaves fp32 only at 131, but what
@@ -702,7 +713,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), 1) gemm_kernel(const __grid_
         int ti[USE_REG ? K_REG : 1];
         constexpr int PEND = EW * 32 * 4;          // bytes from one entry to the next
         static_assert(STAGING >= 2 * 32 * PEND, "room for the pending logits");
-        const uint32_t pend_v = spill_stage + (threadIdx.x - 64) * 4;
+        const uint32_t pend_v = spill_stage + pending_at(threadIdx.x);
         const uint32_t pend_i = pend_v + 32 * PEND;
         constexpr int lo = 0;
 
@@ -971,7 +982,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), 1) gemm_kernel(const __grid_
                                 // staging buffer (128-byte rows, swizzled), and after every second chunk one lane
                                 // requests the store of the 32 x 64 box. That is one request per 4 KB from this warp
                                 // instead of 64 store instructions that each touch 32 rows.
-                                const uint32_t buf = spill_stage + ((4 * half + quad) * SPILL_STAGES + ((spill_boxes >> 1) & 1)) * SPILL_STAGE_BYTES;
+                                const uint32_t buf = spill_stage + stage_at(half, quad) + ((spill_boxes >> 1) & 1) * SPILL_STAGE_BYTES;
                                 if ((ch & 1) == 0) {
                                     // the store that read this buffer two boxes ago must have finished reading it
                                     if (lane == 0) bulk_wait_group_read<SPILL_STAGES - 1>();
@@ -1249,19 +1260,20 @@ __global__ void __launch_bounds__(gemm_threads(EW), 1) gemm_kernel(const __grid_
             }
             if constexpr (EW == 8) {
                 // The second thread of a row hands over m, s and its list through the staging area; the first adds them to its own.
-                const uint32_t at = spill_stage + ((threadIdx.x - 64) & 127) * 4;      // word e of the row at + e PEND: the first thread's columns of the room
+                static_assert(PEND == 256 * 4, "meet_word's columns");
+                auto word = [&](int e) { return spill_stage + meet_word(USE_REG, threadIdx.x, e); };
                 if (half == 1) {
                     if (TOPK == TOPK_NONE && lane == 0) bulk_wait_group_read<0>();      // (its own staging buffers have been read)
                     __syncwarp();
                     // the first threads' staging buffers and pending logits lie there too: they say when the room is free
                     if (!__all_sync(0xffffffffu, wait_barrier(meet_bar(1), meet_phase, abort_flag, p.status, 5))) return false;
-                    st_shared_b32(at, __float_as_uint(m));
-                    st_shared_b32(at + PEND, __float_as_uint(s));
+                    st_shared_b32(word(0), __float_as_uint(m));
+                    st_shared_b32(word(1), __float_as_uint(s));
                     if (USE_REG) {
 #pragma unroll
                         for (int k = 0; k < (USE_REG ? K_REG : 1); ++k) {
-                            st_shared_b32(at + PEND * (2 + 2 * k), __float_as_uint(tv[k]));
-                            st_shared_b32(at + PEND * (3 + 2 * k), static_cast<uint32_t>(ti[k]));
+                            st_shared_b32(word(2 + 2 * k), __float_as_uint(tv[k]));
+                            st_shared_b32(word(3 + 2 * k), static_cast<uint32_t>(ti[k]));
                         }
                     }
                     __syncwarp();
@@ -1275,7 +1287,7 @@ __global__ void __launch_bounds__(gemm_threads(EW), 1) gemm_kernel(const __grid_
                 if (lane == 0) mbar_arrive(meet_bar(1));
                 if (!__all_sync(0xffffffffu, wait_barrier(meet_bar(0), meet_phase, abort_flag, p.status, 5))) return false;
                 meet_phase ^= 1u;
-                const float m2 = __uint_as_float(ld_shared_b32(at)), s2 = __uint_as_float(ld_shared_b32(at + PEND));
+                const float m2 = __uint_as_float(ld_shared_b32(word(0))), s2 = __uint_as_float(ld_shared_b32(word(1)));
                 if (spill) {
                     s += s2;      // (of the same reference)
                 } else {
@@ -1289,8 +1301,8 @@ __global__ void __launch_bounds__(gemm_threads(EW), 1) gemm_kernel(const __grid_
                     auto before = [](float xv, int xi, float yv, int yi) { return xv > yv || (xv == yv && static_cast<uint32_t>(xi) < static_cast<uint32_t>(yi)); };
 #pragma unroll
                     for (int k = 0; k < (USE_REG ? K_REG : 1); ++k) {
-                        const float ov = __uint_as_float(ld_shared_b32(at + PEND * (2 + 2 * (K_REG - 1 - k))));
-                        const int oi = static_cast<int>(ld_shared_b32(at + PEND * (3 + 2 * (K_REG - 1 - k))));
+                        const float ov = __uint_as_float(ld_shared_b32(word(2 + 2 * (K_REG - 1 - k))));
+                        const int oi = static_cast<int>(ld_shared_b32(word(3 + 2 * (K_REG - 1 - k))));
                         const bool mine = before(tv[k], ti[k], ov, oi);
                         tv[k] = mine ? tv[k] : ov;
                         ti[k] = mine ? ti[k] : oi;

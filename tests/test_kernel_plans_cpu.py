@@ -44,3 +44,31 @@ int main() {
 }
 """)
     assert out == "ok 1\n", out
+
+
+def test_handed_over_words_lie_where_their_reader_writes_next(tmp_path):
+    """Eight epilogue warps: the first thread of a row may go on to its next tile while other rows' words are still being read. So no warp but
+    the reader's own writes there: neither its staging buffers nor its columns of the pending logits hold another row's words."""
+    out = run_host_program(tmp_path, "kernels.cuh", r"""
+int main() {
+    for (int thread = 64; thread < 192; ++thread) {
+        const int quad = thread / 32 % 4;      // as the kernel has it
+        for (int e = 0; e < 2; ++e) {          // a spill: two words
+            const int at = meet_word(false, thread, e);
+            if (at != meet_word(false, thread + 128, e)) return std::printf("two places, thread %d\n", thread), 1;
+            if (at < stage_at(0, quad) || at + 4 > stage_at(0, quad) + SPILL_STAGES * SPILL_STAGE_BYTES)
+                return std::printf("another warp's buffer, thread %d\n", thread), 1;
+            for (int other = 64; other < 192; ++other)
+                for (int e2 = 0; e2 < 2; ++e2)
+                    if ((other != thread || e2 != e) && at == meet_word(false, other, e2)) return std::printf("shared, threads %d %d\n", thread, other), 1;
+        }
+        for (int e = 0; e < 2 + 2 * K_REG; ++e) {      // a list: entry q of the pending logits is 256 words behind entry q - 1
+            const int at = meet_word(true, thread, e);
+            if (at != meet_word(true, thread + 128, e) || at % 1024 != pending_at(thread) || at + 4 > 8 * SPILL_STAGES * SPILL_STAGE_BYTES)
+                return std::printf("column, thread %d\n", thread), 1;
+        }
+    }
+    std::printf("ok\n");
+}
+""")
+    assert out == "ok\n", out
