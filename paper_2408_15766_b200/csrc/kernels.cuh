@@ -104,6 +104,11 @@ struct OutPlan {
     int width;             // columns of a tile: BN, or 128 or 64 of a cluster's (then GemmParams::kept)
 };
 
+// A cluster of C CTAs finishes `rows` rows of a tile, piece_rows(rows, C) each: the CTA that finishes row r. (Rows of the tile that do not exist
+// belong to the last CTA: an address in a CTA beyond the cluster is undefined even where nothing is stored to it.)
+__host__ __device__ constexpr int piece_rows(int rows, int C) { return (rows + C - 1) / C; }
+__host__ __device__ constexpr int piece_rank(int r, int per, int C) { return r / per < C ? r / per : C - 1; }
+
 struct GemmParams {
     CUtensorMap tmA0, tmA1, tmB;   // boxes: 128 rows of A; of B the BN / pair columns that one CTA holds
     CUtensorMap tmSpill;   // MODE_STATS without Top-K lists (the draft sweep): the spill P as [chunk rows, p_pitch] bf16 with
@@ -1356,14 +1361,14 @@ __global__ void __launch_bounds__(gemm_threads(EW), 1) gemm_kernel(const __grid_
             static_assert((BM + 8) * (BN + 4) * 4 <= OPERAND_BYTES, "the pieces of a CTA's rows fit the operand stages");
             const int u = cta / C, z = cta - u * C;
             const int rt = u % p.plan.row_units, ct = u / p.plan.row_units;
-            const int per = (min(BM, p.rows_valid - p.row_global_offset - rt * BM) + C - 1) / C;      // (rows that exist are dealt out)
+            const int per = piece_rows(min(BM, p.rows_valid - p.row_global_offset - rt * BM), C);      // (rows that exist are dealt out)
             tc_fence_before_sync();
             __syncthreads();
             cluster_sync();
             tc_fence_after_sync();
             if (warp >= 2) {
                 const int quad = warp & 3, r = quad * 32 + lane;
-                const uint32_t dst = map_to_rank(smem_base + (z * per + r % per) * ROW_PITCH * 4, r / per);
+                const uint32_t dst = map_to_rank(smem_base + (z * per + r % per) * ROW_PITCH * 4, piece_rank(r, per, C));
                 const bool row_ok = p.row_global_offset + rt * BM + r < p.rows_valid;
 #pragma unroll 1
                 for (int ch = 0; ch < width / 32; ++ch) {

@@ -72,3 +72,21 @@ int main() {
 }
 """)
     assert out == "ok\n", out
+
+
+def test_rows_of_a_shared_tile_go_to_ctas_of_the_cluster(tmp_path):
+    out = run_host_program(tmp_path, "kernels.cuh", r"""
+int main() {
+    for (int C = 2; C <= 8; ++C)
+        for (int rows = 1; rows <= BM; ++rows) {
+            const int per = piece_rows(rows, C);
+            for (int r = 0; r < BM; ++r) {
+                const int rank = piece_rank(r, per, C);
+                if (rank < 0 || rank >= C) return std::printf("no such CTA: row %d of %d, %d CTAs\n", r, rows, C), 1;
+                if (r < rows && (rank * per + r % per != r || r % per >= per)) return std::printf("row %d of %d, %d CTAs\n", r, rows, C), 1;
+            }
+        }
+    std::printf("ok\n");
+}
+""")
+    assert out == "ok\n", out
