@@ -169,6 +169,20 @@ def _workspace(ws: Optional[torch.Tensor], device, nbytes, *sizes) -> torch.Tens
     return ws
 
 
+def _per_row(grad: Optional[torch.Tensor], N: int, stream) -> Optional[torch.Tensor]:
+    """The rows' incoming gradients as the kernels read them: N floats side by side (a loss behind .sum() gets an expanded single one).
+    A copy is made on the call's stream, whose later work alone may reuse its memory."""
+    if grad is None:
+        return None
+    assert grad.dtype == torch.float32 and grad.shape == (N,)
+    if not grad.is_cuda:
+        assert grad.is_pinned() and grad.is_contiguous(), "grad_loss must be on the GPU"
+    if grad.is_contiguous():
+        return grad
+    with torch.cuda.stream(stream):
+        return grad.detach().contiguous()
+
+
 def _dh_dtype(code: int):
     return torch.float32 if code == HASS_FP32 else torch.bfloat16
 
@@ -255,7 +269,7 @@ def topk_distill_bwd(H_d, W, topk_idx, topk_q, lse_d, grad_loss=None, dH_dtype: 
     K = topk_idx.shape[1]
     assert topk_idx.dtype == torch.int32 and topk_q.dtype == torch.float32 and lse_d.dtype == torch.float32
     assert topk_idx.is_contiguous() and topk_q.is_contiguous() and lse_d.is_contiguous()
-    assert grad_loss is None or (grad_loss.dtype == torch.float32 and grad_loss.shape == (N,))
+    grad_loss = _per_row(grad_loss, N, stream)
     dev = H_d.device
     ws = _workspace(workspace, dev, topk_distill_workspace_bytes, N, d, V, K)
     dH = torch.empty(N, d, dtype=_dh_dtype(dH_dtype), device=dev) if out is None else out
@@ -273,7 +287,7 @@ def topk_distill_fwd_bwd(H_t, H_d, W, K: int, grad_loss=None, dH_dtype: int = HA
             return got
     N, d, V = _dims(H_t, W)
     assert H_d.shape == H_t.shape and H_d.dtype == torch.bfloat16 and H_d.is_contiguous()
-    assert grad_loss is None or (grad_loss.dtype == torch.float32 and grad_loss.shape == (N,))
+    grad_loss = _per_row(grad_loss, N, stream)
     dev = H_t.device
     ws = _workspace(workspace, dev, topk_distill_workspace_bytes, N, d, V, K)
     if out is None:
@@ -302,7 +316,7 @@ def topk_distill_fwd_bwd_draft(H_d, W, topk_idx, topk_q, grad_loss=None, dH_dtyp
     K = topk_idx.shape[1]
     assert topk_idx.dtype == torch.int32 and topk_q.dtype == torch.float32
     assert topk_idx.is_contiguous() and topk_q.is_contiguous() and topk_idx.shape == topk_q.shape == (N, K)
-    assert grad_loss is None or (grad_loss.dtype == torch.float32 and grad_loss.shape == (N,))
+    grad_loss = _per_row(grad_loss, N, stream)
     dev = H_d.device
     ws = _workspace(workspace, dev, topk_distill_workspace_bytes, N, d, V, K)
     if out is None:
@@ -332,7 +346,7 @@ def combined_distill_fwd_bwd(H_t, H_d, W, K: int, w_topk: float = 1.0, grad_loss
             return got
     N, d, V = _dims(H_t, W)
     assert H_d.shape == H_t.shape and H_d.dtype == torch.bfloat16 and H_d.is_contiguous()
-    assert grad_loss is None or (grad_loss.dtype == torch.float32 and grad_loss.shape == (N,))
+    grad_loss = _per_row(grad_loss, N, stream)
     dev = H_t.device
     ws = _workspace(workspace, dev, combined_distill_workspace_bytes, N, d, V, K)
     if out is None:
@@ -363,7 +377,7 @@ def variant_distill_fwd_bwd(H_t, H_d, W, K: int, variant: int, param: float = 0.
         return got
     N, d, V = _dims(H_t, W)
     assert H_d.shape == H_t.shape and H_d.dtype == torch.bfloat16 and H_d.is_contiguous()
-    assert grad_loss is None or (grad_loss.dtype == torch.float32 and grad_loss.shape == (N,))
+    grad_loss = _per_row(grad_loss, N, stream)
     dev = H_t.device
     ws = _workspace(workspace, dev, topk_distill_workspace_bytes, N, d, V, K)
     kk = 2 * K if variant == LOSS_BIDIR_TOPK else K      # the bi-directional set holds up to 2K tokens
@@ -391,6 +405,9 @@ def topk_distill_fwd_bwd_host(H_t_host, H_d_host, W, K: int, loss_host, dH_d_hos
     assert H_d_host.shape == H_t_host.shape and H_d_host.dtype == torch.bfloat16 and H_d_host.is_contiguous()
     assert loss_host.dtype == torch.float32 and loss_host.shape == (N,) and not loss_host.is_cuda
     assert dH_d_host.dtype == _dh_dtype(dH_dtype) and dH_d_host.shape == (N, d) and dH_d_host.is_contiguous()
+    if grad_loss_host is not None:
+        assert grad_loss_host.dtype == torch.float32 and grad_loss_host.shape == (N,)
+        grad_loss_host = grad_loss_host.detach().contiguous()
     ws = _workspace(workspace, W.device, topk_distill_host_workspace_bytes, N, d, V, K, dH_dtype)
     _ok(lib.hass_topk_distill_fwd_bwd_host(_p(H_t_host), _p(H_d_host), _p(W), N, d, V, K, _p(grad_loss_host),
                                            _p(loss_host), _p(topk_idx_host), _p(topk_q_host), _p(dH_d_host),

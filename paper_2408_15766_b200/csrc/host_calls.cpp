@@ -114,11 +114,11 @@ struct Head {
         }
         return true;
     }
-    bool rows(PyObject* o, const float*& p) const {      // fp32 [N] or None
+    bool rows(PyObject* o, const float*& p) const {      // fp32 [N] or None (autograd's gradient of a sum is an expanded element: not the plain case)
         p = nullptr;
         if (o == Py_None) return true;
-        const at::Tensor* t = tensor(o);
-        if (!t || t->scalar_type() != at::kFloat || !t->is_cuda() || t->dim() != 1 || t->size(0) != N) return false;
+        const at::Tensor* t = plain(o, at::kFloat);
+        if (!t || t->dim() != 1 || t->size(0) != N) return false;
         p = static_cast<const float*>(t->data_ptr());
         return true;
     }
@@ -197,8 +197,8 @@ ENTRY(topk_distill_bwd, 9) {
     const float *q, *lse = nullptr, *g;
     int code;
     at::ScalarType type;
-    if (!h.take(nullptr, a[0], a[1]) || !h.set(a[2], a[3], idx, q) || a[4] == Py_None || !h.rows(a[4], lse) || !tensor(a[4])->is_contiguous() ||
-        !h.rows(a[5], g) || !type_of(a[6], code, type) || !c.take(a[7], a[8]))
+    if (!h.take(nullptr, a[0], a[1]) || !h.set(a[2], a[3], idx, q) || a[4] == Py_None || !h.rows(a[4], lse) || !h.rows(a[5], g) ||
+        !type_of(a[6], code, type) || !c.take(a[7], a[8]))
         DEFER;
     const at::Tensor dH = make({h.N, h.d}, type, *h.H_d);
     const int rc = c.run(lib.bwd, h.H_d->data_ptr(), h.W->data_ptr(), h.N, h.d, h.V, static_cast<int32_t>(h.K), idx, q, lse, g, dH.data_ptr(), code);

@@ -68,6 +68,50 @@ def test_native_and_python_forms_agree(monkeypatch, grad):
                     assert torch.equal(x, y) if key != "dQ" else torch.allclose(x.float(), y.float(), rtol=2.0 ** -7, atol=1e-3), (name, key)
 
 
+# What autograd hands a per-row loss: behind .sum() one element for all rows, behind an indexed sum every second of a longer buffer. (Both lie in
+# buffers that N floats from their first element on do not leave.)
+@pytest.mark.gpu
+@pytest.mark.parametrize("native", [True, False])
+@pytest.mark.parametrize("layout", ["expanded", "strided"])
+def test_grad_loss_of_any_stride(monkeypatch, native, layout):
+    dev = torch.device("cuda:0")
+    g = torch.Generator(device=dev).manual_seed(4)
+    R = lambda *s: torch.randn(*s, generator=g, device=dev).to(torch.bfloat16)
+    N, d, V, K = 37, 128, 1500, 7
+    H_t, H_d, W = R(N, d), R(N, d), R(V, d)
+    buf = torch.rand(2 * N, generator=g, device=dev)
+    gl = (buf[:1].expand(N) if layout == "expanded" else buf[::2]).requires_grad_()
+    plain = torch.tensor(gl.tolist(), device=dev)
+    ws = torch.empty(hass.combined_distill_workspace_bytes(N, d, V, K), dtype=torch.uint8, device=dev)
+    f = hass.topk_distill_fwd(H_t, H_d, W, K, workspace=ws)
+    host = {k: v.cpu() for k, v in {"H_t": H_t, "H_d": H_d}.items()}
+
+    def from_host(w):
+        loss, dH = torch.empty(N), torch.empty(N, d, dtype=torch.bfloat16)
+        hass.topk_distill_fwd_bwd_host(host["H_t"], host["H_d"], W, K, loss, dH, w.cpu() if w is plain else w.detach().cpu().as_strided((N,), (0,)) if
+                                       layout == "expanded" else buf.cpu()[::2])
+        return dH
+
+    if not native:
+        monkeypatch.setattr(binding, "_host", _Nothing())
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    calls = {
+        "bwd": lambda w: hass.topk_distill_bwd(H_d, W, f["topk_idx"], f["topk_q"], f["lse_d"], w, workspace=ws),
+        "fwd_bwd": lambda w: hass.topk_distill_fwd_bwd(H_t, H_d, W, K, w, workspace=ws)["dH_d"],
+        "fwd_bwd_draft": lambda w: hass.topk_distill_fwd_bwd_draft(H_d, W, f["topk_idx"], f["topk_q"], w, workspace=ws)["dH_d"],
+        "combined": lambda w: hass.combined_distill_fwd_bwd(H_t, H_d, W, K, 0.5, w, workspace=ws)["dH_d"],
+        "normed": lambda w: hass.variant_distill_fwd_bwd(H_t, H_d, W, K, hass.LOSS_NORMED_TOPK, grad_loss=w, workspace=ws)["dH_d"],
+        "bidir": lambda w: hass.variant_distill_fwd_bwd(H_t, H_d, W, K, hass.LOSS_BIDIR_TOPK, grad_loss=w, workspace=ws)["dH_d"],
+        "host": from_host,
+        "side": lambda w: hass.topk_distill_fwd_bwd(H_t, H_d, W, K, w, workspace=ws, stream=side)["dH_d"],
+    }
+    for name, call in calls.items():
+        a, b = call(gl), call(plain)
+        torch.cuda.synchronize()
+        assert torch.equal(a, b) and not a.requires_grad, name
+
+
 @pytest.mark.gpu
 def test_a_status_is_the_same_error_in_both_forms(monkeypatch):
     dev = torch.device("cuda:0")
@@ -95,3 +139,5 @@ def test_what_is_not_the_plain_case_is_left_to_python():
         hass.topk_distill_fwd_bwd(x, x, x.float(), 2)
     with pytest.raises(AssertionError):
         hass.topk_distill_fwd_bwd(x, x, x, 2, workspace=ws)
+    with pytest.raises(AssertionError):
+        hass.topk_distill_fwd_bwd(x, x, x, 2, torch.ones(4))                                    # pageable host memory
