@@ -190,7 +190,8 @@ int hass_topk_distill_fwd_bwd_draft(const void* H_d, const void* W, int64_t N, i
  *
  * i.e. the gradient of sum_i grad_loss[i] (loss_ce[i] + w loss_topk[i]) with respect to H_d. The
  * logits of both feature sets go through the workspace in fp32, in chunks of rows; one kernel forms
- * the losses and dz_d, rounded to bf16 once, and one product gives dH_d (6 N d V tensor FLOPs). No
+ * the losses and dz_d, rounded to bf16 once but for the term -w q, which keeps its fp32 value where it is
+ * what makes the entry large, and one product gives dH_d (6 N d V tensor FLOPs). No
  * range condition and no second pass. Calls of 129 to 256 rows, and those with a smaller workspace,
  * spill the target tiles as well as the draft's, and a second GEMM forms q W per row, from which both
  * the cross-entropy, lse_d - <H_d[i], (q W)[i]>, and its gradient term follow (8 N d V); these have the

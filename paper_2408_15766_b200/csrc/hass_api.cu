@@ -436,7 +436,8 @@ static int combined_rows(long long N, long long V, int sms) {
     if (N <= 2 * BM) return 0;
     const int RT = ceil_div(N, BM);
     const long long tile = static_cast<long long>(BM) * ceil_div(V, BN) * BN * 8;
-    const long long most = std::max(1, sms / 4) * tile <= kCombinedL2Bytes ? sms / 4 : std::min<long long>(sms / 8, kCombinedBytes / tile);
+    const int part = even_chunk(sms / 4, RT);      // row tiles whose fp32 rows of d the workspace holds (make_layout)
+    const long long most = std::max(1, part) * tile <= kCombinedL2Bytes ? part : std::min<long long>(sms / 8, kCombinedBytes / tile);
     if (most < 4) return 0;
     const int chunks = ceil_div(RT, most);
     return ceil_div(RT, chunks) * BM;
@@ -1084,7 +1085,7 @@ static int narrow_impl(int objective, bool with_target, const void* H_t, const v
         r.w = cmb->w;
         r.loss_ce = cmb->loss_ce;
     }
-    if (objective == ROW_BIDIR) {
+    if (objective != ROW_TOPK) {
         r.W = static_cast<const __nv_bfloat16*>(W);
         r.d = static_cast<int>(d);
         r.coef_out = reinterpret_cast<float*>(ws + L.coef);

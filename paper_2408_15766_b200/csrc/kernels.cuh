@@ -2219,7 +2219,10 @@ __global__ void __launch_bounds__(256) loss_patch_kernel(const __grid_constant__
 // dz_d(v) = g (S_q p(v) - q(v) [v in Omega_hat]) in bf16, in place: the bf16 row begins where the fp32 row did. Every step
 // reads a piece twice as long as the one it writes, and a piece is written after all threads have read theirs.
 // ROW_COMBINED: dz_d(v) = g ((1 + w S_q) p(v) - q(v) - w q(v) [v in Omega_hat]), and the cross-entropy
-// sum_v q(v) (lse_d - z_d(v)). ROW_BIDIR: the draft's K most probable tokens join Omega_hat; the row becomes p(v) alone, and
+// sum_v q(v) (lse_d - z_d(v)); what bf16 leaves of the entries at Omega_hat that w q makes large goes, with their rows of W, to the epilogue of the
+// second GEMM in fp32 (left_over; with the whole entry in bf16 dH_d of rows whose target and draft are peaked on different tokens was 1.7e-3 off
+// fp64 in 2-norm at 100 x 4096 x 32000, logits of deviation 4, with a spill of either matrix 1.2e-3, now 1.06e-3; per call 64 x 256 x 1024
+// 18 -> 19 us, 100 x 4096 x 32000, K = 100 117 -> 125, 300 x 4096 x 32000 269 -> 273). ROW_BIDIR: the draft's K most probable tokens join Omega_hat; the row becomes p(v) alone, and
 // g S_q and the row sum_x g q(x) W[x, :] over Omega_hat are left in fp32 for the epilogue of the second GEMM.
 //
 // The K largest of a row: a thread's largest logit is at hand after the pass for lse, and the K-th largest of these
@@ -2258,10 +2261,10 @@ struct RowParams {
     __nv_bfloat16* dz;     // row_split_kernel: [N, 2 pitch] dz_d; may be the target's logits, not the draft's
     float w;               // ROW_COMBINED
     float* loss_ce;
-    const __nv_bfloat16* W;      // ROW_BIDIR: [V, d]
+    const __nv_bfloat16* W;      // ROW_BIDIR, ROW_COMBINED: [V, d]
     int d;
-    float* coef_out;       // [N] g S_q
-    float* sparse_out;     // [N, d]
+    float* coef_out;       // [N] row scale of the second GEMM: g S_q, or 1
+    float* sparse_out;     // [N, d] what its epilogue takes off
 };
 
 // The separate backward's set is the caller's and may name a token more than once: what its first entry takes off for all of them,
@@ -2274,6 +2277,31 @@ __device__ __forceinline__ float repeated_q(const int* tok, const float* q, int 
         sum += q[i];
     }
     return sum;
+}
+
+// Combined objective: what is to be added to an entry of dz_d at a token of Omega_hat, dense - target - w q, that was rounded to bf16 as `b`; 0 where
+// the rounding is at most that of its dense and target terms by themselves, as they have it in a spill (w q(x) as a term of its own stays in fp32
+// there). The row of W goes with it to the fp32 rows of the second GEMM's epilogue.
+__device__ __forceinline__ float left_over(float o, __nv_bfloat16 b, float dense, float target) {
+    return fabsf(o) > fabsf(dense) + fabsf(target) ? __bfloat162float(b) - o : 0.f;
+}
+// One warp: the entries whose weight is not zero go to the front, in their order; returns how many there are.
+__device__ __forceinline__ int keep_weighted(int* tok, float* w, int n) {
+    const int lane = threadIdx.x & 31;
+    int kept = 0;
+    for (int j0 = 0; j0 < n; j0 += 32) {
+        const int j = j0 + lane, t = j < n ? tok[j] : 0;
+        const float x = j < n ? w[j] : 0.f;
+        const uint32_t bm = __ballot_sync(0xffffffffu, x != 0.f);
+        const int at = kept + __popc(bm & ((1u << lane) - 1u));
+        if (x != 0.f) {
+            tok[at] = t;
+            w[at] = x;
+        }
+        kept += __popc(bm);
+        __syncwarp();
+    }
+    return kept;
 }
 
 struct RowPool {           // of a block that looks for the K largest logits of a row, or of its piece of one
@@ -2737,36 +2765,53 @@ __global__ void __launch_bounds__(THREADS, ROW_THREADS / THREADS) row_kernel(con
         for (int o = 16; o > 0; o >>= 1) ce += __shfl_xor_sync(0xffffffffu, ce, o);
         if (lane == 0) sh.red[0][warp] = ce;
     }
-    if (OBJ == ROW_BIDIR) {
-        if (tid == 0) p.coef_out[row] = g * S_q;
-        const int n = sh.count;
+    // sum_j sh.z[j] W[sh.tok[j], :], j < n, in fp32 for the second GEMM's epilogue
+    auto sparse_row = [&](int n) {
         for (int k0 = tid * 8; k0 < p.d; k0 += THREADS * 8) {
             float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll 4
             for (int j = 0; j < n; ++j) {
-                const float gq = g * sh.q[j];
+                const float c = sh.z[j];
                 float wf[8];
                 unpack8(*reinterpret_cast<const uint4*>(p.W + static_cast<long long>(sh.tok[j]) * p.d + k0), wf);
 #pragma unroll
-                for (int t = 0; t < 8; ++t) a[t] = fmaf(gq, wf[t], a[t]);
+                for (int t = 0; t < 8; ++t) a[t] = fmaf(c, wf[t], a[t]);
             }
             float* so = p.sparse_out + static_cast<long long>(row) * p.d + k0;
             *reinterpret_cast<float4*>(so) = make_float4(a[0], a[1], a[2], a[3]);
             *reinterpret_cast<float4*>(so + 4) = make_float4(a[4], a[5], a[6], a[7]);
         }
+    };
+    if (OBJ == ROW_BIDIR) {
+        if (tid == 0) p.coef_out[row] = g * S_q;
+        if (tid < sh.count) sh.z[tid] = g * sh.q[tid];
+        __syncthreads();
+        sparse_row(sh.count);
         return;
     }
     __syncthreads();
     // Tokens of q = 0 keep the dense value: the one that fills up a set of fewer than K logits above -inf (token 0) may be in it
     // already, and an entry has one writer.
     const float q_own = tid < n_tok && sh.tok[tid] >= 0 ? (p.lse_in != nullptr ? repeated_q(sh.tok, sh.q, n_tok, tid) : sh.q[tid]) : 0.f;
+    float left = 0.f;
     if (q_own != 0.f) {
-        float o = c * ex2(fmaf(sh.z[tid], LOG2E, shift));
-        if (OBJ == ROW_COMBINED)
-            o -= g * ex2(fmaf(trow[sh.tok[tid]], LOG2E, shift_t)) + g * p.w * q_own;
-        else
-            o -= g * q_own;
-        drow[sh.tok[tid]] = __float2bfloat16_rn(o);
+        const float dense = c * ex2(fmaf(sh.z[tid], LOG2E, shift)), target = OBJ == ROW_COMBINED ? g * ex2(fmaf(trow[sh.tok[tid]], LOG2E, shift_t)) : 0.f;
+        const float o = dense - (OBJ == ROW_COMBINED ? target + g * p.w * q_own : g * q_own);
+        const __nv_bfloat16 b = __float2bfloat16_rn(o);
+        drow[sh.tok[tid]] = b;
+        if (OBJ == ROW_COMBINED) left = left_over(o, b, dense, target);
+    }
+    if (OBJ == ROW_COMBINED) {
+        if (tid == 0) p.coef_out[row] = 1.f;
+        if (tid < K) sh.z[tid] = left;
+        if (K > 32) __syncthreads();      // (up to 32 tokens are the first warp's own)
+        __syncwarp();
+        if (warp == 0) {
+            const int n = keep_weighted(sh.tok, sh.z, K);
+            if (lane == 0) sh.count = n;
+        }
+        __syncthreads();
+        sparse_row(sh.count);
     }
     if (OBJ == ROW_COMBINED && warp == 0) {
         float v = lane < THREADS / 32 ? sh.red[0][lane] : 0.f;

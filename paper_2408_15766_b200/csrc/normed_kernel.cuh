@@ -15,7 +15,7 @@ template <int THREADS, typename F>
 __device__ __forceinline__ void sum_rows(const __nv_bfloat16* W, int d, const int* tok, const float* w, int n, int rank, int C, float* part, F&& out) {
     const int tid = threadIdx.x, units = d / 8;
     const int u0 = part_begin(units, rank, C), u1 = part_begin(units, rank + 1, C);
-    const int per = max(32, min((u1 - u0 + 31) / 32 * 32, THREADS)), groups = gather_groups(u1 - u0, THREADS), g = tid / per;
+    const int per = max(32, min((u1 - u0 + 31) / 32 * 32, THREADS)), groups = min(gather_groups(u1 - u0, THREADS), max(n, 1)), g = tid / per;
     for (int b = u0; b < u1; b += THREADS) {
         const int u = b + tid - g * per;
         float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};

@@ -344,16 +344,17 @@ __global__ void __launch_bounds__(SPLIT_THREADS, CLUSTER || SPLIT_THREADS == 512
             *reinterpret_cast<uint2*>(drow + at) = make_uint2(pack_bf16x2(o[0], o[1]), pack_bf16x2(o[2], o[3]));
         }
     }
+    auto sparse_out = [&](int k0, const float (&a)[8]) {
+        float* o = p.sparse_out + static_cast<long long>(row) * p.d + k0;
+        *reinterpret_cast<float4*>(o) = make_float4(a[0], a[1], a[2], a[3]);
+        *reinterpret_cast<float4*>(o + 4) = make_float4(a[4], a[5], a[6], a[7]);
+    };
     if (OBJ == ROW_BIDIR) {
         if (rank == 0 && tid == 0) p.coef_out[row] = g * S_q;
         const int n = sh.count;
         if (tid < n) sh.zt[tid] = g * sh.q[tid];
         __syncthreads();
-        sum_rows<SPLIT_THREADS>(p.W, p.d, sh.tok, sh.zt, n, rank, C, sh.part, [&](int k0, const float (&a)[8]) {
-            float* o = p.sparse_out + static_cast<long long>(row) * p.d + k0;
-            *reinterpret_cast<float4*>(o) = make_float4(a[0], a[1], a[2], a[3]);
-            *reinterpret_cast<float4*>(o + 4) = make_float4(a[4], a[5], a[6], a[7]);
-        });
+        sum_rows<SPLIT_THREADS>(p.W, p.d, sh.tok, sh.zt, n, rank, C, sh.part, sparse_out);
         return;
     }
     if (OBJ == ROW_COMBINED) {
@@ -367,15 +368,27 @@ __global__ void __launch_bounds__(SPLIT_THREADS, CLUSTER || SPLIT_THREADS == 512
     if (tid < n_tok) {
         const int at = sh.tok[tid] - first;
         const bool own = sh.tok[tid] >= 0 && at >= 0 && at < E * SPLIT_STEP;
-        const float q_own = !own ? 0.f : p.lse_in != nullptr ? repeated_q(sh.tok, sh.q, n_tok, tid) : sh.q[tid];
+        const float q_own = !own && OBJ != ROW_COMBINED ? 0.f : p.lse_in != nullptr ? repeated_q(sh.tok, sh.q, n_tok, tid) : sh.q[tid];
+        float left = 0.f;
         if (q_own != 0.f) {
-            float o = c * ex2(fmaf(sh.z[tid], LOG2E, shift));
-            if (OBJ == ROW_COMBINED)
-                o -= g * ex2(fmaf(sh.zt[tid], LOG2E, shift_t)) + g * p.w * q_own;
-            else
-                o -= g * q_own;
-            drow[at] = __float2bfloat16_rn(o);
+            const float dense = c * ex2(fmaf(sh.z[tid], LOG2E, shift)), target = OBJ == ROW_COMBINED ? g * ex2(fmaf(sh.zt[tid], LOG2E, shift_t)) : 0.f;
+            const float o = dense - (OBJ == ROW_COMBINED ? target + g * p.w * q_own : g * q_own);
+            const __nv_bfloat16 b = __float2bfloat16_rn(o);
+            if (own) drow[at] = b;
+            if (OBJ == ROW_COMBINED) left = left_over(o, b, dense, target);      // (of all tokens: the blocks share the columns)
         }
+        if (OBJ == ROW_COMBINED) sh.zt[tid] = left;
+    }
+    if (OBJ == ROW_COMBINED) {
+        if (rank == 0 && tid == 0) p.coef_out[row] = 1.f;
+        if (K > 32) __syncthreads();      // (up to 32 tokens are the first warp's own)
+        __syncwarp();
+        if (warp == 0) {
+            const int n = keep_weighted(sh.tok, sh.zt, K);
+            if (lane == 0) sh.count = n;
+        }
+        __syncthreads();
+        sum_rows<SPLIT_THREADS>(p.W, p.d, sh.tok, sh.zt, sh.count, rank, C, sh.part, sparse_out);
     }
     if (OBJ == ROW_COMBINED) {
         if (warp == 0) {
