@@ -1,19 +1,26 @@
 """Builds in-tree the CUDA library, paper_2408_15766_b200/libhass_b200.so (sm_100a only), and the binding's native
-calls, paper_2408_15766_b200/hass_host.so (against the installed torch)."""
+calls, paper_2408_15766_b200/hass_host-<torch><Python>.so (against the installed torch)."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
 import sysconfig
+from importlib.metadata import version
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 SRC_DIR = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libhass_b200.so")
 SOURCES = ["hass_api.cu"]
+
+
 # every header under csrc/ and the public header: a change to any of them makes the library stale
-HEADERS = sorted(f for f in os.listdir(SRC_DIR) if f.endswith((".cuh", ".h"))) + [os.path.join("..", "..", "include", "hass.h")]
-HOST = os.path.join(HERE, "hass_host.so")
+def _headers() -> list:
+    return sorted(f for f in os.listdir(SRC_DIR) if f.endswith((".cuh", ".h"))) + [os.path.join("..", "..", "include", "hass.h")]
+
+
+# named after what its binary interface depends on: under another torch or Python it is not found, and built again, instead of loaded
+HOST = os.path.join(HERE, f"hass_host-{version('torch')}{sysconfig.get_config_var('EXT_SUFFIX')}")
 HOST_SOURCES = ["host_calls.cpp", os.path.join("..", "..", "include", "hass.h")]
 
 
@@ -38,9 +45,13 @@ def build_host(force: bool = False) -> str:
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:
+    if force or _stale(LIB, SOURCES + _headers()):
+        _build_cuda(verbose)
     build_host(force)
-    if not force and not _stale(LIB, SOURCES + HEADERS):
-        return LIB
+    return LIB
+
+
+def _build_cuda(verbose: bool) -> None:
     nvcc = os.environ.get("NVCC", "nvcc")
     tmp = LIB + f".tmp{os.getpid()}"
     cmd = [nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -50,7 +61,6 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
         cmd.insert(2, "-v")
     subprocess.run(cmd, check=True)
     os.replace(tmp, LIB)
-    return LIB
 
 
 if __name__ == "__main__":

@@ -1,4 +1,7 @@
 """The native form of the binding's calls: the same outputs as the Python form, which does everything that is not the plain case."""
+import os
+import sysconfig
+
 import pytest
 import torch
 
@@ -141,3 +144,14 @@ def test_what_is_not_the_plain_case_is_left_to_python():
         hass.topk_distill_fwd_bwd(x, x, x, 2, workspace=ws)
     with pytest.raises(AssertionError):
         hass.topk_distill_fwd_bwd(x, x, x, 2, torch.ones(4))                                    # pageable host memory
+
+
+def test_native_calls_of_another_torch_are_not_loaded(tmp_path):
+    """Their file is named after torch and Python; where it is missing the package loads and every call is left to its Python form."""
+    name = os.path.basename(binding.HOST)
+    assert torch.__version__ in name and name.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+    assert binding._host.__file__ == binding.HOST
+    with pytest.warns(UserWarning, match="is missing"):
+        host = binding._load_host(binding.lib, str(tmp_path / "hass_host-0.0.so"))
+    x = torch.zeros(4, 64, dtype=torch.bfloat16)
+    assert host.topk_distill_fwd(x, x, x, 2, None, None) is None
