@@ -436,10 +436,10 @@ static int combined_rows(long long N, long long V, int sms) {
     if (N <= 2 * BM) return 0;
     const int RT = ceil_div(N, BM);
     const long long tile = static_cast<long long>(BM) * ceil_div(V, BN) * BN * 8;
-    const int part = even_chunk(sms / 4, RT);      // row tiles whose fp32 rows of d the workspace holds (make_layout)
-    const long long most = std::max(1, part) * tile <= kCombinedL2Bytes ? part : std::min<long long>(sms / 8, kCombinedBytes / tile);
+    const bool stays = std::max(1, sms / 4) * tile <= kCombinedL2Bytes;
+    const long long most = stays ? sms / 4 : std::min<long long>(sms / 8, kCombinedBytes / tile);
     if (most < 4) return 0;
-    const int chunks = ceil_div(RT, most);
+    const int chunks = ceil_div(RT, stays ? even_chunk(sms / 4, RT) : most);      // (even_chunk: the workspace holds no more rows of d in fp32)
     return ceil_div(RT, chunks) * BM;
 }
 
