@@ -71,8 +71,8 @@ int hass_version(void);
  * bounded scratch areas for one chunk of rows (a fixed number of 128-row tiles that does not grow
  * with N): the bf16 un-normalised draft probabilities (fused call) or dz_d (split backward),
  * chunk_rows x V, and the fp32 Omega_hat term of dH_d, chunk_rows x d; and, behind them, fp32 partial
- * tiles of dH_d (less than one 128-row tile of scratch). Calls of at most 128 rows, and of 257 rows and more where
- * hass_topk_distill_fwd_bwd says so, keep their logits in fp32 instead, two matrices of N x V. A smaller workspace is accepted down to room
+ * tiles of dH_d (less than one 128-row tile of scratch). Calls of at most 128 rows, and of 257 rows and more up to the
+ * numbers that hass_topk_distill_fwd_bwd lists, keep their logits in fp32 instead, two matrices of N x V. A smaller workspace is accepted down to room
  * for one 128-row tile of scratch; the calls then work in smaller chunks, and may do without partial tiles and fp32 logits.
  * Needs no GPU (assumes 148 SMs if none is present).
  */
@@ -156,10 +156,13 @@ int hass_topk_distill_bwd(const void* H_d, const void* W, int64_t N, int64_t d, 
  * the Top-P variant work the same way, and so do hass_combined_distill_fwd_bwd, where it spills, and the Bi-directional
  * variant, whose exponent comes from the row's largest logit among the first 256 tokens and whose
  * second pass repeats the whole sequence.
- * Calls of at most 128 rows, and of 257 rows and more over at most 2048 tokens (up to 3072 rows with K <= 32 and 1024 tokens, 2048
- * with K <= 64, 1024 otherwise) or over more (up to 896 rows, and 50e6 / (20e3 + 3.2 V) of them: 408 at 32000 tokens, 531
- * where d >= 3072; half of 408 where one feature set is swept), sweep both feature sets in one launch and keep the draft logits in fp32 between
- * the sweep and the second GEMM; they have no range condition and no second pass.
+ * Calls of at most 128 rows, and of 257 rows and more up to the following, keep their logits in fp32 between one sweep of
+ * their feature sets and the second GEMM; they have no range condition and no second pass. With V rounded up to a multiple of 256:
+ *   V <= 1024, K <= 32    3072 rows
+ *   V <= 2048, K <= 64    2048 rows
+ *   V <= 2048             1024 rows
+ *   larger V              t / (20e3 + 3.2 V) rows, 896 at most: t = 50e6 (408 rows at V = 32000), 65e6 (531) where d >= 3072; 25e6 (204: none
+ *                         from 257 on) for the _draft form, the forward alone and Normed Top-K. The separate backward: 50e6 for every d.
  * (HASS_ERR_RANGE is kept for callers that name it; no entry point of this version returns it.)
  */
 int hass_topk_distill_fwd_bwd(const void* H_t, const void* H_d, const void* W, int64_t N, int64_t d,

@@ -401,19 +401,21 @@ static int even_chunk(int most, int RT) {
     return most > 1 ? most & ~1 : most;
 }
 
-// Whether a call's logits may go through the workspace in fp32 (narrow_impl), in one chunk of row tiles: one row tile of any vocabulary, and more
-// rows of a short one, whose kernels are then three instead of nine and more, while the blocks of the row kernel (11 ns a row at most 1024 tokens
-// and K <= 32, 18 up to 2048 and K <= 64, 57 beyond) take less than those cost. Calls of N x 256 x 1024, before -> after: K = 10 600 rows 62 -> 31 us,
-// 1500 64 -> 40, 2795 69 -> 56, 4500 71 -> 75; K = 41 1500 89 -> 55, 2795 94 -> 82 but Bi-directional 159 -> 177; K = 101 600 123 -> 60, 1500 132 -> 113,
-// 2795 140 -> 186; combined 1980 rows, K = 9 107 -> 50; 1000 x 4096 x 2000, K = 10 111 -> 68, 3900 187 -> 213. (Calls of 129 to 256 rows keep to the
-// spill's route: what they do beyond its exponent range, and report in the status block, is held by tests.) Over more tokens the row kernel takes about
-// 20 + 3.2 V / 1000 ns a row, and the line lies at 50 us of it, or 25 where one matrix alone is swept, and for the forward alone, which saves fewer (`single`), and 65 in fused calls of wide features (d >= 3072), whose joint sweep takes pairs of CTAs
-// also for an odd number of row tiles. Fused calls: 360 x 4096 x 2100, K = 56 119 ->
-// 59 us, 659 x 5120 x 2758, K = 46 203 -> 81, Top-P 268 x 4096 x 12459 168 -> 125, Bi-directional 284 x 4096 x 32000 325 -> 262, 930 x 5432 x 3151 226 -> 178, 391 x
-// 5200 x 32000 442 -> 414, 522 x 4096 x 32000 478 -> 420, 479 x 6024 x 32000 675 -> 609, beyond the lines 594 x 1080 x 33218 237 -> 262, 613 x 5120 x
-// 32000 573 -> 597; forward and backward as two calls 309 x 256 x 32000, K = 62 184 -> 133; draft rows
-// 710 x 5120 x 4375 84 -> 70, beyond it 257 x 256 x 32000 47 -> 52. (More than seven row tiles would gain too, 1013 x 256 x 4525 145 -> 68, but the workspace
-// of such calls stays what their row tiles take: those who pass a smaller one count it in them, as a test does.)
+// Whether a call's logits may go through the workspace in fp32 (narrow_impl), in one chunk of row tiles: three kernels instead of nine and more. One
+// row tile: always. From 257 rows on: while the row kernel takes less time than the launches that go. Its blocks take 11 ns a row at pitch <= 1024 and
+// K <= 32, 18 at pitch <= 2048 and K <= 64, 57 at pitch <= 2048 otherwise, and about 20 + 3.2 pitch / 1000 beyond; there the line lies at 50 us of it, at 65
+// where d >= 3072 (the joint sweep takes pairs of CTAs also for an odd number of row tiles), and at 25 (`single`) where one matrix alone is swept
+// and for the forward alone, which save fewer launches. us per call, the other route -> this one:
+//   pitch 1024, K = 10, d = 256     600 rows 62 -> 31, 1500 64 -> 40, 2795 69 -> 56; beyond the line 4500 71 -> 75
+//   pitch 1024, K = 41, d = 256     1500 rows 89 -> 55; beyond 2795 94 -> 82, but Bi-directional 159 -> 177
+//   pitch 1024, K = 101, d = 256    600 rows 123 -> 60; beyond 1500 132 -> 113, 2795 140 -> 186
+//   pitch 2048, K = 10, d = 4096    1000 rows 111 -> 68; beyond 3900 187 -> 213
+//   50 us: 360 x 4096 x 2100, K = 56 119 -> 59, 659 x 5120 x 2758, K = 46 203 -> 81, 268 x 4096 x 12459 171 -> 128, 300 x 4096 x 32000 334 -> 294; beyond 594 x 1080 x 33218 237 -> 262
+//   65 us: 450 x 4096 x 32000 391 -> 380, 512 399 -> 396, 530 514 -> 478; beyond 613 x 5120 x 32000 573 -> 597
+//   25 us: draft rows 710 x 5120 x 4375 84 -> 70; beyond 257 x 256 x 32000 47 -> 52
+// Two limits are no measurement. 129 to 256 rows stay on the spill's route, because tests hold what such calls do beyond its exponent range and
+// report in the status block. Beyond 2048 tokens seven row tiles are the most (1013 x 256 x 4525 145 -> 68 would gain), because a test counts the
+// workspace of larger calls in row tiles.
 static bool narrow_rows(long long N, long long d, long long pitch, int K, int chunk_tiles, int sms, bool single) {
     if (N <= BM) return true;
     const long long most = K <= 32 && pitch <= 1024   ? 3072
@@ -944,7 +946,7 @@ struct RowSplit {
 };
 static RowSplit row_split(long long N, long long pitch, int K, int sms) {
     // Many short rows: as few threads as hold one, with four maxima or more for each token of the set (two K threads at least). A block
-    // takes longer (10 us at 128 threads, 7 at 512), but ten of them fit an SM.
+    // takes longer (10 us at 128 threads, 7 at 512), but six of them are resident on an SM (80 registers a thread), three of 256 threads.
     if (N > sms && pitch <= 1024 && K <= 32) return RowSplit{1, 128, 2};
     if (N > sms && pitch <= 2048 && K <= 64) return RowSplit{1, 256, 2};
     for (int c = 1; c <= SPLIT_MAX; c *= 2) {
