@@ -630,9 +630,12 @@ def main():
                        "dH_dtype": "bf16", "aligning_steps": wl.steps, "objective": args.objective,
                        **({"top_p": TOP_P, "prefix_tokens_mean": float(var_out["topk_n"].abs().float().mean()),
                            "rows_cut_by_the_cap": int((var_out["topk_n"] < 0).sum())} if args.objective == "top_p" else {}),
-                       "spill_scratch": "un-normalised bf16 draft probabilities of one chunk of %d rows x %d tokens "
-                                        "= %.0f MB live at a time (the N x V matrix would be %.0f MB)" % (
-                                            chunk_rows, V_pad, chunk_rows * V_pad * 2 / 1e6, N * V * 2 / 1e6),
+                       "spill_scratch": ("fp32 logits of both feature sets, %.0f MB" % (2 * N * V_pad * 4 / 1e6) if N <= 128 else
+                                         "fp32 logits of both feature sets, in chunks of rows of %.0f MB at most" % (
+                                             min(2 * N * V_pad * 4, 1600 << 20) / 1e6) if combined and N > 256 else
+                                         "un-normalised bf16 draft probabilities of one chunk of %d rows x %d tokens "
+                                         "= %.0f MB live at a time (the N x V matrix would be %.0f MB)" % (
+                                             chunk_rows, V_pad, chunk_rows * V_pad * 2 / 1e6, N * V * 2 / 1e6)),
                        "target_stats": ("recomputed every step" if wl.steps == 1 else
                                         "computed in aligning step 1, reused in steps 2..%d" % wl.steps),
                        "path": {"combined": "hass_combined_distill_fwd_bwd", "top_p": "hass_variant_distill_fwd_bwd (Top-P)",

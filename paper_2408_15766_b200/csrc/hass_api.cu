@@ -428,11 +428,11 @@ static bool narrow_rows(long long N, long long d, long long pitch, int K, int ch
 // Rows per chunk of a combined call whose logits go through the workspace in fp32; 0: it spills. The spilled probabilities of target and draft
 // have references of their own, known before the sums are, so that the gradient takes a product with W for each; from fp32 logits the row
 // kernel forms their difference (rounded once instead of twice) and one product is enough. The sweep stores twice the bytes, which its products
-// hide, and the row kernel reads them twice. Per call: 1024 rows x 4096 x 128256 2980 -> 2610 us, 517 rows 2140 -> 1620, 2048 x 4096 x 32000
-// 1600 -> 1290, 8192 rows 6240 -> 5300, 300 rows 500 -> 285, 1318 x 376 x 38201, K = 65 560 -> 460, 8000 x 704 x 3000, K = 128 1190 -> 590,
-// 640 x 512 x 8000 130 -> 72. Chunks of an eighth of the SM count in row tiles (every CTA pair has its part of the columns), or of a quarter
-// where their logits stay in the L2 (8000 x 256 x 1024 216 -> 184), of 1.6 GB at most: 8192 x 4096 x 32000 takes 5300 us in chunks of 18 or of 37
-// tiles, 1024 x 4096 x 128256 2690 in two of 4 and 2610 in one. (Calls of 129 to 256 rows keep to the spill, as narrow_rows has it.)
+// hide, and the row kernel reads them twice. Per call, in runs of 0.4 s (the power cap): 1024 rows x 4096 x 128256 3670 -> 3350 us, 517 rows 2580 -> 2110,
+// 2048 x 4096 x 32000 1930 -> 1580, 8192 rows 7780 -> 6330, 300 rows 518 -> 326, 1318 x 376 x 38201, K = 65 522 -> 433, 8000 x 704 x 3000, K = 128 1170 -> 676,
+// 640 x 512 x 8000 127 -> 67. Chunks of an eighth of the SM count in row tiles (every CTA pair has its part of the columns), or of a quarter
+// where their logits stay in the L2 (8000 x 256 x 1024 216 -> 184), of 1.6 GB at most: 8192 x 4096 x 32000 takes the same in chunks of 18 and of 37
+// tiles, 1024 x 4096 x 128256 3 % more in two of 4 than in one. (Calls of 129 to 256 rows keep to the spill, as narrow_rows has it.)
 constexpr long long kCombinedBytes = 1600ll << 20, kCombinedL2Bytes = 128ll << 20;
 static int combined_rows(long long N, long long V, int sms) {
     if (N <= 2 * BM) return 0;
@@ -1184,7 +1184,7 @@ static int fused_impl(bool with_target, const void* H_t, const void* H_d, const 
         }
         return HASS_OK;
     }
-    // (The combined objective too: 65 rows x 4096 x 32000 254 -> 123 us, 128 rows x 4096 x 128256 675 -> 472, 100 x 256 x 1024 82 -> 37.)
+    // (The combined objective too: 65 rows x 4096 x 32000 247 -> 123 us, 128 rows x 4096 x 128256 764 -> 551, 100 x 256 x 1024 79 -> 25.)
     if (with_target) {
         const NarrowRoom narrow = narrow_room(N, d, K, ws, cmb ? cmb->end : workspace_bytes, L, di.sms, false);
         if (narrow.z)

@@ -2232,7 +2232,7 @@ __global__ void __launch_bounds__(256) loss_patch_kernel(const __grid_constant__
 // It takes the rows that row_split_kernel does not (row_split in the host code): those of more than 8192 logits, when they are many.
 // Where there are more rows than SMs two blocks of 512 threads share one, so that one row's barriers fall into the other's loads:
 // combined calls of 2048 rows x 32000 260 -> 215 us, 640 x 8000 54 -> 35, 8000 x 3000, K = 128 620 -> 400; 1024 x 128256, where the rows come
-// out of memory and go back (2.4 GB: two readings of both matrices and dz_d, 5.4 TB/s in the 437 us it takes now), 474 either way then. Four blocks of 256: 257, 33, 455.
+// out of memory and go back (2.4 GB: two readings of both matrices and dz_d, 5.4 TB/s in 437 us, up to 480 under the power cap), 474 either way then. Four blocks of 256: 257, 33, 455.
 constexpr int ROW_THREADS = 1024;
 constexpr int ROW_LOADS = 4;
 constexpr int ROW_POOL = 1024;

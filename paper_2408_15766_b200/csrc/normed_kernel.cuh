@@ -73,8 +73,8 @@ struct NormedParams {
 // sum_x g (pn(x) - qn(x)) W[x, :]. There is no sweep of the draft rows: the K draft logits are dot products in fp32. A block takes its part of the
 // columns in the dot products, whose sums the blocks exchange through distributed shared memory, and in the gradient.
 // Bound by the latency of gathered rows of W, so that the rows of a call are spread over all SMs (one block of eight warps per row
-// left 106 SMs idle with 42 rows): call of 42 rows x 8192 x 128256, K = 98 474 -> 405-423 us, 4 x 4096 x 128256, K = 55 249 -> 236, 85 x 4096 x 32000,
-// K = 15 76.5 -> 73.2; 2048 x 4096 x 32000 412 either way.
+// left 106 SMs idle with 42 rows): call of 42 rows x 8192 x 128256, K = 98 486 -> 423 us, 4 x 4096 x 128256, K = 55 253 -> 244, 85 x 4096 x 32000,
+// K = 15 71.0 -> 66.7; 2048 x 4096 x 32000 499 either way.
 __global__ void __launch_bounds__(NORMED_THREADS, 3) normed_kernel(const __grid_constant__ NormedParams p) {
     __shared__ int tok[K_CAP];
     __shared__ float q[K_CAP], z[K_CAP], w[K_CAP];
