@@ -693,8 +693,8 @@ static int launch_out(GemmParams& p, const PartRoom& room, const DeviceInfo& di,
     p.sched.pair = p.plan.pair;
     p.sched.max_ctas = p.plan.groups * p.plan.pair;
     if (kLog)
-        std::fprintf(stderr, "[hass] out: pair %d, cluster %d, grid %d, %d whole tiles, %d rest tiles x %d cuts\n", p.plan.pair,
-                     p.plan.cluster, p.sched.max_ctas, p.plan.whole, p.plan.rest, p.plan.cuts);
+        std::fprintf(stderr, "[hass] out: pair %d, cluster %d, grid %d, %d whole tiles of %d columns, %d rest tiles x %d cuts\n", p.plan.pair,
+                     p.plan.cluster, p.sched.max_ctas, p.plan.whole, p.plan.width, p.plan.rest, p.plan.cuts);
     const int rc = launch_gemm<MODE_OUT>(p, st);
     if (rc != HASS_OK || p.plan.rest == 0) return rc;
     KernelTimer timer(p.gate ? KIND_CONDITIONAL : KIND_OUT, st);
