@@ -183,18 +183,16 @@ def _workspace(ws: Optional[torch.Tensor], device, nbytes, *sizes) -> torch.Tens
     return ws
 
 
-def _per_row(grad: Optional[torch.Tensor], N: int, stream) -> Optional[torch.Tensor]:
-    """The rows' incoming gradients as the kernels read them: N floats side by side (a loss behind .sum() gets an expanded single one).
-    A copy is made on the call's stream, whose later work alone may reuse its memory."""
+def _per_row(grad: Optional[torch.Tensor], N: int, device, stream) -> Optional[torch.Tensor]:
+    """The rows' incoming gradients as the kernels read them: N floats side by side (a loss behind .sum() gets an expanded single one), on the
+    GPU or in page-locked memory. A copy is made on the call's stream, whose later work alone may reuse its memory."""
     if grad is None:
         return None
     assert grad.dtype == torch.float32 and grad.shape == (N,)
-    if not grad.is_cuda:
-        assert grad.is_pinned() and grad.is_contiguous(), "grad_loss must be on the GPU"
-    if grad.is_contiguous():
+    if grad.is_contiguous() and (grad.is_cuda or grad.is_pinned()):
         return grad
     with torch.cuda.stream(stream):
-        return grad.detach().contiguous()
+        return grad.detach().to(device).contiguous()
 
 
 def _dh_dtype(code: int):
@@ -283,7 +281,7 @@ def topk_distill_bwd(H_d, W, topk_idx, topk_q, lse_d, grad_loss=None, dH_dtype: 
     K = topk_idx.shape[1]
     assert topk_idx.dtype == torch.int32 and topk_q.dtype == torch.float32 and lse_d.dtype == torch.float32
     assert topk_idx.is_contiguous() and topk_q.is_contiguous() and lse_d.is_contiguous()
-    grad_loss = _per_row(grad_loss, N, stream)
+    grad_loss = _per_row(grad_loss, N, H_d.device, stream)
     dev = H_d.device
     ws = _workspace(workspace, dev, topk_distill_workspace_bytes, N, d, V, K)
     dH = torch.empty(N, d, dtype=_dh_dtype(dH_dtype), device=dev) if out is None else out
@@ -301,7 +299,7 @@ def topk_distill_fwd_bwd(H_t, H_d, W, K: int, grad_loss=None, dH_dtype: int = HA
             return got
     N, d, V = _dims(H_t, W)
     assert H_d.shape == H_t.shape and H_d.dtype == torch.bfloat16 and H_d.is_contiguous()
-    grad_loss = _per_row(grad_loss, N, stream)
+    grad_loss = _per_row(grad_loss, N, H_t.device, stream)
     dev = H_t.device
     ws = _workspace(workspace, dev, topk_distill_workspace_bytes, N, d, V, K)
     if out is None:
@@ -330,7 +328,7 @@ def topk_distill_fwd_bwd_draft(H_d, W, topk_idx, topk_q, grad_loss=None, dH_dtyp
     K = topk_idx.shape[1]
     assert topk_idx.dtype == torch.int32 and topk_q.dtype == torch.float32
     assert topk_idx.is_contiguous() and topk_q.is_contiguous() and topk_idx.shape == topk_q.shape == (N, K)
-    grad_loss = _per_row(grad_loss, N, stream)
+    grad_loss = _per_row(grad_loss, N, H_d.device, stream)
     dev = H_d.device
     ws = _workspace(workspace, dev, topk_distill_workspace_bytes, N, d, V, K)
     if out is None:
@@ -360,7 +358,7 @@ def combined_distill_fwd_bwd(H_t, H_d, W, K: int, w_topk: float = 1.0, grad_loss
             return got
     N, d, V = _dims(H_t, W)
     assert H_d.shape == H_t.shape and H_d.dtype == torch.bfloat16 and H_d.is_contiguous()
-    grad_loss = _per_row(grad_loss, N, stream)
+    grad_loss = _per_row(grad_loss, N, H_t.device, stream)
     dev = H_t.device
     ws = _workspace(workspace, dev, combined_distill_workspace_bytes, N, d, V, K)
     if out is None:
@@ -391,7 +389,7 @@ def variant_distill_fwd_bwd(H_t, H_d, W, K: int, variant: int, param: float = 0.
         return got
     N, d, V = _dims(H_t, W)
     assert H_d.shape == H_t.shape and H_d.dtype == torch.bfloat16 and H_d.is_contiguous()
-    grad_loss = _per_row(grad_loss, N, stream)
+    grad_loss = _per_row(grad_loss, N, H_t.device, stream)
     dev = H_t.device
     ws = _workspace(workspace, dev, topk_distill_workspace_bytes, N, d, V, K)
     kk = 2 * K if variant == LOSS_BIDIR_TOPK else K      # the bi-directional set holds up to 2K tokens
